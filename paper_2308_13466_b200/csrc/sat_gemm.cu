@@ -5,6 +5,8 @@
 //   TN: C (+)= A^T (B o mask), colsum (+)= 1^T (B o mask), split-K    weight / bias gradient
 #include "sat_internal.h"
 
+#include <algorithm>
+
 #define BM 64
 #define BN 64
 #define BK 16
@@ -242,15 +244,24 @@ k_gemm_tn(int64_t rows, int64_t rows_per_split, int32_t m, int32_t n, const floa
     }
 }
 
-// out[i] (+)= sum_z part[z][i]: eight lanes take the splits round-robin (four independent loads in flight each), their sums
+// out[i] (+)= sum_z part[z][i], and behind it (blocks from `blocks1`) the same for a second, one-row array: eight lanes take the splits round-robin (four independent loads in flight each), their sums
 // are added in lane order (fixed order: reproducible)
 __global__ void __launch_bounds__(256)
 k_splitk_reduce(const float *__restrict__ part, int64_t count, int32_t splits, int accumulate, float *__restrict__ out,
-                int32_t ncols, int64_t ld_out)
+                int32_t ncols, int64_t ld_out, int64_t blocks1, const float *__restrict__ part2, int64_t count2, float *__restrict__ out2)
 {
     __shared__ float red[8][32];
     const int o = threadIdx.x & 31, zl = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 32 + o;
+    int64_t blk = blockIdx.x;
+    if (blk >= blocks1) {
+        blk -= blocks1;
+        part = part2;
+        count = count2;
+        out = out2;
+        ncols = (int32_t)count2;
+        ld_out = count2;
+    }
+    const int64_t i = blk * 32 + o;
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
     if (i < count) {
         int z = zl;
@@ -278,7 +289,8 @@ sat_status sat_splitk_reduce(sat_ctx *ctx, const float *part, int64_t count, int
                              int32_t ld_out)
 {
     if (count == 0) return SAT_OK;
-    k_splitk_reduce<<<(unsigned)cdiv64(count, 32), 256, 0, ctx->stream>>>(part, count, splits, accumulate, out, ncols, ld_out);
+    const int64_t b1 = cdiv64(count, 32);
+    k_splitk_reduce<<<(unsigned)b1, 256, 0, ctx->stream>>>(part, count, splits, accumulate, out, ncols, ld_out, b1, nullptr, 0, nullptr);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
@@ -288,10 +300,13 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
 {
     if (m == 0 || n == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_GEMM_TN, 4.0 * ((double)rows * (m + n) + (double)m * n), 2.0 * (double)rows * m * n);
-    int64_t splits = cdiv64(rows > 0 ? rows : 1, TN_ROWS_PER_SPLIT);
+    // Enough row splits for two blocks per SM (one block walking 2,048 rows alone took 168 us, 32 of 64 rows each take 4), and
+    // at most TN_ROWS_PER_SPLIT rows in each; a split has at least 4 BK rows, below which its partial sums outweigh its products
+    const int64_t r1 = rows > 0 ? rows : 1, tiles = cdiv64(m, BM) * cdiv64(n, BN);
+    int64_t splits = std::max<int64_t>(cdiv64(r1, TN_ROWS_PER_SPLIT), std::min<int64_t>(cdiv64(2 * 148, tiles), cdiv64(r1, 4 * BK)));
     if (splits > 1024) splits = 1024;
-    int64_t rows_per_split = cdiv64(cdiv64(rows > 0 ? rows : 1, splits), BK) * BK;
-    splits = cdiv64(rows > 0 ? rows : 1, rows_per_split);
+    int64_t rows_per_split = cdiv64(cdiv64(r1, splits), BK) * BK;
+    splits = cdiv64(r1, rows_per_split);
     const size_t bytes = (size_t)splits * ((size_t)m * n + n) * sizeof(float);
     SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, bytes));
     float *part_C = (float *)ctx->buf_splitk.p;
@@ -299,8 +314,9 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN), (unsigned)splits);
     k_gemm_tn<<<grid, 256, 0, ctx->stream>>>(rows, rows_per_split, m, n, A, lda, B, ldb, mask, mask_words, part_C, part_cs);
     SAT_LAUNCHED(ctx);
-    SAT_TRY(sat_splitk_reduce(ctx, part_C, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc));
-    if (colsum) SAT_TRY(sat_splitk_reduce(ctx, part_cs, n, (int32_t)splits, accumulate, colsum, n, n));
+    const int64_t b1 = cdiv64((int64_t)m * n, 32), b2 = colsum ? cdiv64(n, 32) : 0;
+    k_splitk_reduce<<<(unsigned)(b1 + b2), 256, 0, ctx->stream>>>(part_C, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, b1, part_cs, n, colsum);
+    SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
 
@@ -509,7 +525,8 @@ extern "C" sat_status sat_dense_tn_static(void *cuda_stream, int64_t rows, int32
     k_gemm_tn<<<grid, 256, 0, st>>>(rows, rows_per_split, m, n, A, lda, B, ldb, nullptr, 0, scratch, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return static_fail(errbuf, errbuf_len, SAT_ECUDA, "sat_dense_tn_static: launch failed (%s)", cudaGetErrorString(e));
-    k_splitk_reduce<<<(unsigned)cdiv64((int64_t)m * n, 32), 256, 0, st>>>(scratch, (int64_t)m * n, (int32_t)splits, 0, C, n, n);
+    const int64_t b1 = cdiv64((int64_t)m * n, 32);
+    k_splitk_reduce<<<(unsigned)b1, 256, 0, st>>>(scratch, (int64_t)m * n, (int32_t)splits, 0, C, n, n, b1, nullptr, 0, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return static_fail(errbuf, errbuf_len, SAT_ECUDA, "sat_dense_tn_static: launch failed (%s)", cudaGetErrorString(e));
     return SAT_OK;
