@@ -95,12 +95,12 @@ extern "C" sat_status sat_create(sat_ctx **out, int device, void *cuda_stream)
     if (!ctx) return SAT_ENOMEM;
     ctx->device = device;
     ctx->stream = (cudaStream_t)cuda_stream;
-    if (cudaMalloc((void **)&ctx->d_flag, 2 * sizeof(int)) != cudaSuccess ||
+    if (cudaMalloc((void **)&ctx->d_flag, 4 * sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void **)&ctx->h_flag, sizeof(int)) != cudaSuccess) {
         delete ctx;
         return SAT_ENOMEM;
     }
-    cudaMemsetAsync(ctx->d_flag, 0, 2 * sizeof(int), ctx->stream);  // [0] validation flags, [1] kernel wait time-outs
+    cudaMemsetAsync(ctx->d_flag, 0, 4 * sizeof(int), ctx->stream);  // [0] validation flags, [1] kernel wait time-outs, [2] ticket of loss_finish
     *out = ctx;
     return SAT_OK;
 }

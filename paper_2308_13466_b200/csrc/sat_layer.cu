@@ -252,7 +252,7 @@ __global__ void k_lstm_cell(const float *__restrict__ gates, int64_t rows, int32
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= rows * h) return;
-    const int64_t r = t / h;
+    const int64_t r = sat_div(t, h);
     const int j = (int)(t - r * h);
     const float *a = gates + r * 4 * (int64_t)h;
     const float gi = 1.f / (1.f + expf(-a[j]));
@@ -280,7 +280,8 @@ __global__ void k_lstm_cell_first(const float *__restrict__ proj, int64_t rows, 
     const float gg = tanh_fast(a.z);
     const float go = sigmoid_fast(a.w);
     const float cn = gi * gg;
-    c[sat_cell_offset(t / h, (int32_t)(t % h), h)] = cn;
+    const int64_t r = sat_div(t, h);
+    c[sat_cell_offset(r, (int32_t)(t - r * h), h)] = cn;
     s[t] = go * tanh_fast(cn);
 }
 
@@ -382,7 +383,7 @@ __global__ void k_gru_cell(const float *__restrict__ gx, const float *__restrict
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= rows * h) return;
-    const int64_t r0 = t / h;
+    const int64_t r0 = sat_div(t, h);
     const int j = (int)(t - r0 * h);
     const float *ax = gx + r0 * 3 * (int64_t)h;
     float hr = 0.f, hz = 0.f, hn = 0.f, sp = 0.f;
@@ -924,77 +925,98 @@ extern "C" sat_status sat_dense_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_
 // =====================================================================================
 // loss seed, parameter step
 // =====================================================================================
-// one warp per row
-// Loss kernels: one warp per row, LOSS_ROWS_PER_BLOCK consecutive rows per block (each warp walks its share in order).
-// The row losses are summed in double per warp, the warps of a block in fixed order, and k_loss_sum adds the block
-// partials in fixed order: the total does not depend on scheduling.
-#define LOSS_ROWS_PER_BLOCK 256
+// Loss kernels.  The rows go round-robin over the lane groups of at most LOSS_MAX_BLOCKS blocks (one resident wave).  Row losses
+// are summed in double per thread, then per warp, the warps of a block in fixed order, and the last block to finish adds the block
+// partials in fixed order: which rows a thread owns depends on the row count alone, so the total does not depend on scheduling.
+#define LOSS_MAX_BLOCKS (148 * 6)
 
-__device__ __forceinline__ void loss_block_partial(double warp_sum, double *__restrict__ block_partial)
+__device__ __forceinline__ void loss_finish(double thread_sum, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
 {
-    __shared__ double red[8];
+    __shared__ double red[256];
+    __shared__ int last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) red[warp] = warp_sum;
+    for (int o = 16; o > 0; o >>= 1) thread_sum += __shfl_xor_sync(0xffffffffu, thread_sum, o);
+    if (lane == 0) red[warp] = thread_sum;
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < 8; ++w) s += red[w];
         block_partial[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double s = 0.0;
+    for (unsigned i = threadIdx.x; i < gridDim.x; i += 256) s += __ldcg(block_partial + i);
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        *ticket = 0;   // the next launch on this stream starts from zero again
+        if (total) *total += red[0];
     }
 }
 
-// softmax cross-entropy: the row (up to 32 CPL classes) is held in registers, one exponential per class
+// Softmax cross-entropy, up to 8 CPL classes: eight lanes hold a row in registers, one exponential per class.  Bound by HBM (z in,
+// g out) and instruction issue; a warp per row spent most of its instructions in the two five-step reductions of a row
+// (612 k rows x 47 classes: 136 us).
 template <int CPL>
 __global__ void __launch_bounds__(256)
 k_loss_ce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const int32_t *__restrict__ y, float scale,
-          float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial)
+          float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r0 = (int64_t)blockIdx.x * LOSS_ROWS_PER_BLOCK;
+    const int lane = threadIdx.x & 7;
     double acc = 0.0;
-    for (int i = warp; i < LOSS_ROWS_PER_BLOCK; i += 8) {
-        const int64_t r = r0 + i;
-        if (r >= rows) break;
-        const float *zr = z + r * ld_z;
+    // whole warps stay together (the shuffles name every lane): a warp walks four rows at a time
+    for (int64_t rw = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5; rw * 4 < rows; rw += (int64_t)gridDim.x * 8) {
+        const int64_t r = rw * 4 + ((threadIdx.x & 31) >> 3);
+        const bool ok = r < rows;
+        const float *zr = z + (ok ? r : rows - 1) * ld_z;
+        const int32_t yr = y[ok ? r : rows - 1];
         float v[CPL];
         float mx = -INFINITY;
 #pragma unroll
         for (int j = 0; j < CPL; ++j) {
-            const int c = lane + 32 * j;
-            v[j] = c < C ? zr[c] : -INFINITY;
+            v[j] = lane + 8 * j < C ? zr[lane + 8 * j] : -INFINITY;
             mx = fmaxf(mx, v[j]);
         }
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const float zy = lane == 0 ? zr[yr] : 0.f;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         float se = 0.f;
 #pragma unroll
         for (int j = 0; j < CPL; ++j) {
-            v[j] = lane + 32 * j < C ? expf(v[j] - mx) : 0.f;
+            v[j] = lane + 8 * j < C ? expf(v[j] - mx) : 0.f;
             se += v[j];
         }
-        for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+        if (!ok) continue;
         const float inv = 1.f / se;
-        const int32_t yr = y[r];
+        float *gr = g + r * ld_g;
 #pragma unroll
         for (int j = 0; j < CPL; ++j) {
-            const int c = lane + 32 * j;
-            if (c < C) g[r * ld_g + c] = scale * (v[j] * inv - (c == yr ? 1.f : 0.f));
+            const int c = lane + 8 * j;
+            if (c < C) gr[c] = scale * (v[j] * inv - (c == yr ? 1.f : 0.f));
         }
-        if (lane == 0) acc += (double)(scale * (mx + logf(se) - zr[yr]));
+        if (lane == 0) acc += (double)(scale * (mx + logf(se) - zy));
     }
-    loss_block_partial(acc, block_partial);
+    loss_finish(acc, block_partial, ticket, total);
 }
 
 // any number of classes: three passes over the row
 __global__ void __launch_bounds__(256)
 k_loss_ce_wide(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const int32_t *__restrict__ y, float scale,
-               float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial)
+               float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r0 = (int64_t)blockIdx.x * LOSS_ROWS_PER_BLOCK;
     double acc = 0.0;
-    for (int i = warp; i < LOSS_ROWS_PER_BLOCK; i += 8) {
-        const int64_t r = r0 + i;
-        if (r >= rows) break;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + warp; r < rows; r += (int64_t)gridDim.x * 8) {
         const float *zr = z + r * ld_z;
         float mx = -INFINITY;
         for (int c = lane; c < C; c += 32) mx = fmaxf(mx, zr[c]);
@@ -1007,46 +1029,46 @@ k_loss_ce_wide(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_
         for (int c = lane; c < C; c += 32) g[r * ld_g + c] = scale * (expf(zr[c] - mx) * inv - (c == yr ? 1.f : 0.f));
         if (lane == 0) acc += (double)(scale * (mx + logf(se) - zr[yr]));
     }
-    loss_block_partial(acc, block_partial);
+    loss_finish(acc, block_partial, ticket, total);
 }
 
+// Sigmoid cross-entropy, element by element (the loss is a plain sum over nodes and labels): V consecutive labels per thread, V = 4
+// where the rows allow 16-byte accesses.  One exponential serves the loss and the gradient: with e = exp(-|x|), softplus(x) = max(x, 0)
+// + log1p(e) and sigmoid(x) = 1 / (1 + e) or e / (1 + e).
+template <int V>
 __global__ void __launch_bounds__(256)
 k_loss_bce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const uint8_t *__restrict__ y, float scale,
-           float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial)
+           float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r0 = (int64_t)blockIdx.x * LOSS_ROWS_PER_BLOCK;
-    const float inv_c = 1.f / (float)C;
+    const float sc = scale / (float)C;
+    const int32_t cv = C / V;
+    const int64_t count = rows * cv;
     double acc = 0.0;
-    for (int i = warp; i < LOSS_ROWS_PER_BLOCK; i += 8) {
-        const int64_t r = r0 + i;
-        if (r >= rows) break;
-        const float *zr = z + r * ld_z;
-        float a = 0.f;
-        for (int c = lane; c < C; c += 32) {
-            const float x = zr[c], yv = (float)y[r * C + c];
-            a += fmaxf(x, 0.f) + log1pf(expf(-fabsf(x))) - yv * x;
-            g[r * ld_g + c] = scale * inv_c * (1.f / (1.f + expf(-x)) - yv);
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < count; i += (int64_t)gridDim.x * 256) {
+        const int64_t r = sat_div(i, cv);
+        const int32_t c = (int32_t)(i - r * cv) * V;
+        float x[V], t[V], gx[V];
+        if (V == 4) {
+            const float4 zv = *reinterpret_cast<const float4 *>(z + r * ld_z + c);
+            const uchar4 yv = *reinterpret_cast<const uchar4 *>(y + r * C + c);
+            x[0] = zv.x; x[1 % V] = zv.y; x[2 % V] = zv.z; x[3 % V] = zv.w;
+            t[0] = yv.x; t[1 % V] = yv.y; t[2 % V] = yv.z; t[3 % V] = yv.w;
+        } else {
+            x[0] = z[r * ld_z + c];
+            t[0] = (float)y[r * C + c];
         }
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) acc += (double)(scale * inv_c * a);
+        float a = 0.f;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            const float e = expf(-fabsf(x[k])), inv = 1.f / (1.f + e);
+            a += fmaxf(x[k], 0.f) + log1pf(e) - t[k] * x[k];
+            gx[k] = sc * ((x[k] >= 0.f ? inv : e * inv) - t[k]);
+        }
+        if (V == 4) *reinterpret_cast<float4 *>(g + r * ld_g + c) = make_float4(gx[0], gx[1 % V], gx[2 % V], gx[3 % V]);
+        else g[r * ld_g + c] = gx[0];
+        acc += (double)(sc * a);
     }
-    loss_block_partial(acc, block_partial);
-}
-
-// single block, fixed order: *total += sum(block_partial)
-__global__ void k_loss_sum(const double *__restrict__ block_partial, int64_t count, double *total)
-{
-    __shared__ double red[256];
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < count; i += 256) s += block_partial[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *total += red[0];
+    loss_finish(acc, block_partial, ticket, total);
 }
 
 extern "C" sat_status sat_loss_grad(sat_ctx *ctx, int32_t part, int kind, int32_t n_classes, const float *z, int32_t ld_z,
@@ -1058,39 +1080,43 @@ extern "C" sat_status sat_loss_grad(sat_ctx *ctx, int32_t part, int kind, int32_
     if (kind != SAT_LOSS_SOFTMAX_CE && kind != SAT_LOSS_SIGMOID_BCE) return sat_fail(ctx, SAT_EINVAL, "sat_loss_grad: unknown loss");
     if (v.n_rows == 0) return SAT_OK;
     if (n_classes <= 0 || !z || !labels || !g || ld_z < n_classes || ld_g < n_classes) return sat_fail(ctx, SAT_EINVAL, "sat_loss_grad: null tensor or bad shape");
-    const unsigned blocks = (unsigned)cdiv64(v.n_rows, LOSS_ROWS_PER_BLOCK);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)blocks * sizeof(double)));
+    const bool vec4 = kind == SAT_LOSS_SIGMOID_BCE && !(n_classes & 3) && !(ld_z & 3) && !(ld_g & 3) && aligned16(z) && aligned16(g) &&
+                      (((uintptr_t)labels) & 3u) == 0;
+    const int64_t groups = kind == SAT_LOSS_SOFTMAX_CE ? cdiv64(v.n_rows, n_classes <= 128 ? 32 : 8)
+                                                       : cdiv64((int64_t)v.n_rows * n_classes, vec4 ? 1024 : 256);
+    const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS ? groups : LOSS_MAX_BLOCKS);
+    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS * sizeof(double)));
     double *block_partial = (double *)ctx->buf_misc.p;
+    int *ticket = ctx->d_flag + 2;
     const float scale = 1.0f / (float)ctx->n;
     ProfScope prof(ctx, SATK_LOSS, 8.0 * (double)v.n_rows * n_classes, 0.0);
+#define ARGS v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial, ticket, loss_sum
     if (kind == SAT_LOSS_SOFTMAX_CE) {
         const int32_t *yl = (const int32_t *)labels;
-        if (n_classes <= 32) k_loss_ce<1><<<blocks, 256, 0, ctx->stream>>>(v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial);
-        else if (n_classes <= 64) k_loss_ce<2><<<blocks, 256, 0, ctx->stream>>>(v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial);
-        else if (n_classes <= 128) k_loss_ce<4><<<blocks, 256, 0, ctx->stream>>>(v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial);
-        else k_loss_ce_wide<<<blocks, 256, 0, ctx->stream>>>(v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial);
+        if (n_classes <= 16) k_loss_ce<2><<<blocks, 256, 0, ctx->stream>>>(ARGS);
+        else if (n_classes <= 32) k_loss_ce<4><<<blocks, 256, 0, ctx->stream>>>(ARGS);
+        else if (n_classes <= 64) k_loss_ce<8><<<blocks, 256, 0, ctx->stream>>>(ARGS);
+        else if (n_classes <= 128) k_loss_ce<16><<<blocks, 256, 0, ctx->stream>>>(ARGS);
+        else k_loss_ce_wide<<<blocks, 256, 0, ctx->stream>>>(ARGS);
     } else {
-        k_loss_bce<<<blocks, 256, 0, ctx->stream>>>(v.n_rows, n_classes, z, ld_z, (const uint8_t *)labels, scale, g, ld_g, block_partial);
+        const uint8_t *yl = (const uint8_t *)labels;
+        if (vec4) k_loss_bce<4><<<blocks, 256, 0, ctx->stream>>>(ARGS);
+        else k_loss_bce<1><<<blocks, 256, 0, ctx->stream>>>(ARGS);
     }
+#undef ARGS
     SAT_LAUNCHED(ctx);
-    if (loss_sum) {
-        k_loss_sum<<<1, 256, 0, ctx->stream>>>(block_partial, (int64_t)blocks, loss_sum);
-        SAT_LAUNCHED(ctx);
-    }
     return SAT_OK;
 }
 
-// staleness diagnostic: one warp per halo row, fp64 accumulation, block partials added in fixed order by k_loss_sum
+// staleness diagnostic: one warp per halo row, fp64 accumulation, block partials added in fixed order (loss_finish)
 __global__ void __launch_bounds__(256)
 k_staleness(const int32_t *__restrict__ halo_gid, const int32_t *__restrict__ pos, int64_t halo0, int64_t n_halo, int32_t d,
-            const float *__restrict__ fresh, int64_t ld, const float *__restrict__ used, int64_t ld_used, double *__restrict__ block_partial)
+            const float *__restrict__ fresh, int64_t ld, const float *__restrict__ used, int64_t ld_used, double *__restrict__ block_partial,
+            int *__restrict__ ticket, double *total)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t j0 = (int64_t)blockIdx.x * LOSS_ROWS_PER_BLOCK;
     double acc = 0.0;
-    for (int i = warp; i < LOSS_ROWS_PER_BLOCK; i += 8) {
-        const int64_t j = j0 + i;
-        if (j >= n_halo) break;
+    for (int64_t j = (int64_t)blockIdx.x * 8 + warp; j < n_halo; j += (int64_t)gridDim.x * 8) {
         const float *a = fresh + (int64_t)pos[halo_gid[halo0 + j]] * ld;
         const float *b = used + j * ld_used;
         double s = 0.0;
@@ -1098,10 +1124,9 @@ k_staleness(const int32_t *__restrict__ halo_gid, const int32_t *__restrict__ po
             const double t = (double)a[c] - (double)b[c];
             s += t * t;
         }
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         acc += s;
     }
-    loss_block_partial(acc, block_partial);
+    loss_finish(acc, block_partial, ticket, total);
 }
 
 extern "C" sat_status sat_staleness(sat_ctx *ctx, int32_t part, int32_t d, const float *h_fresh, int32_t ld, const float *h_used_halo,
@@ -1114,13 +1139,11 @@ extern "C" sat_status sat_staleness(sat_ctx *ctx, int32_t part, int32_t d, const
     SAT_CUDA(ctx, cudaMemsetAsync(sq_sum, 0, sizeof(double), ctx->stream));
     if (v.n_halo == 0) return SAT_OK;
     if (!h_fresh || !h_used_halo || ld < d || ld_halo < d) return sat_fail(ctx, SAT_EINVAL, "sat_staleness: null tensor or bad leading dimension");
-    const unsigned blocks = (unsigned)cdiv64(v.n_halo, LOSS_ROWS_PER_BLOCK);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)blocks * sizeof(double)));
-    double *block_partial = (double *)ctx->buf_misc.p;
-    k_staleness<<<blocks, 256, 0, ctx->stream>>>(ctx->halo_gid, ctx->pos, v.halo0, v.n_halo, d, h_fresh, ld,
-                                                 h_used_halo, ld_halo, block_partial);
-    SAT_LAUNCHED(ctx);
-    k_loss_sum<<<1, 256, 0, ctx->stream>>>(block_partial, (int64_t)blocks, sq_sum);
+    const int64_t groups = cdiv64(v.n_halo, 8);
+    const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS ? groups : LOSS_MAX_BLOCKS);
+    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS * sizeof(double)));
+    k_staleness<<<blocks, 256, 0, ctx->stream>>>(ctx->halo_gid, ctx->pos, v.halo0, v.n_halo, d, h_fresh, ld, h_used_halo, ld_halo,
+                                                 (double *)ctx->buf_misc.p, ctx->d_flag + 2, sq_sum);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
