@@ -192,7 +192,7 @@ __global__ void k_gat_fwd_fixup(const int32_t *__restrict__ mrows, int32_t mrow0
 {
     const int d4 = (d + 3) >> 2;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t i = t / d4;
+    const int64_t i = sat_div(t, d4);
     const int c4 = (int)(t - i * d4);
     if (i >= n_mrows) return;
     const int32_t row = mrows[mrow0 + i];
@@ -227,7 +227,7 @@ __global__ void k_gat_dmask(const float *__restrict__ g, int64_t ld_g, const flo
                             float *__restrict__ D, int64_t ld_d)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t r = t / d;
+    const int64_t r = sat_div(t, d);
     const int c = (int)(t - r * d);
     if (r >= rows) return;
     const float x = g[r * ld_g + c];
@@ -472,7 +472,7 @@ __global__ void k_gat_cols_combine(const int32_t *__restrict__ first_item, int32
 {
     const int d4 = (d + 3) >> 2;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t i = t / d4;
+    const int64_t i = sat_div(t, d4);
     const int c4 = (int)(t - i * d4);
     if (i >= n_rows) return;
     const int32_t u = row0 + (int32_t)i;

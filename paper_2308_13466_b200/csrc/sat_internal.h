@@ -9,15 +9,15 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <deque>
 #include <vector>
 
 #include "../../include/sat_b200.h"
 
 #define SAT_MAX_LAYERS 16
 #define SAT_MAX_PARTS 4096
-#define SAT_SPMM_CHUNK 256 /* edges per SpMM work item */
-#define SAT_HROW_LONG 256  /* halo rows with more entries than this are cut into chunks, a thread block per chunk */
-#define SAT_HROW_CHUNK 2048 /* entries per chunk of a long halo row */
+#define SAT_SPMM_CHUNK 256 /* edges per work item of the attention layer */
+#define SAT_HROW_LONG 256  /* halo rows with more entries than this get a thread block in the attention layer's backward */
 
 // Debug build (-DSAT_DEBUG_BOUNDS, libsat_b200_dbg.so): every index the graph kernels load from an index array (column ids,
 // row lists, cache slots) is checked against the extent of the matrix it addresses; an index outside it raises bit 4 of
@@ -118,22 +118,23 @@ struct ProfRec {
     double bytes, flops;
 };
 
-// Forward SpMM work list in source-block-major order (sat_spmm.cu).  The sources of a partition (its inner rows, then its
-// halo rows) are cut into blocks of at most `block_rows` rows; the entries of every local-CSR row are sorted by source, so a
-// row meets each block in one contiguous run of entries.  An item is such a run (cut further at SAT_SPMM_CHUNK entries);
-// within a partition items are ordered by block, then by row, so that the rows gathered at any one time come from one or
-// two blocks.  Rows with more than one item add their partial sums in item order (k_spmm_sb_fixup).
-struct SrcBlockedItems {
-    int64_t block_rows = 0, fit_rows = 0, min_run = 0, row_run = 0;  // key
-    int mode = 0;              // key: 0 = all entries of a row, 1 = its inner prefix only (one block per partition)
-    int32_t n_items = 0, n_mrows = 0;
-    int64_t n_slots = 0;
+// Which work list of the SpMM kernels (sat_spmm.cu): the kind of rows and, for forward lists with source-blocked partitions, the cut.
+struct ListKey {
+    int mode = 0;
+    int64_t block_rows = 0, fit_rows = 0, min_run = 0, row_run = 0;
+    bool operator==(const ListKey &o) const
+    {
+        return mode == o.mode && block_rows == o.block_rows && fit_rows == o.fit_rows && min_run == o.min_run && row_run == o.row_run;
+    }
+};
+struct SpmmList {
+    ListKey asked, key;        // the key it was first asked for with; the cut it was made with (all zero: no partition is blocked)
     int4 *item = nullptr;      // {row, partial slot or -1, first entry: low 32 bits, first entry: high 16 bits | entries << 16}
-    int32_t *slot0 = nullptr;  // [n] first partial slot of a row with several items
-    int32_t *tot = nullptr;    // [n] items of the row
-    int32_t *mrows = nullptr;  // [n_mrows] rows with several items
-    std::vector<int32_t> h_item_off, h_mrow_off;  // [M+1] per partition
-    std::vector<int64_t> h_slot_off;              // [M+1]
+    int32_t *slot0 = nullptr;  // per row: first partial slot of a row with several runs (one allocation with the three below)
+    int32_t *tot = nullptr;    // per row: runs of the row
+    int32_t *mrows = nullptr;  // rows with a few runs
+    int32_t *hrows = nullptr;  // rows with many runs
+    std::vector<int64_t> off;  // [4 x (M+1)] first item, first partial slot, first entry of mrows and of hrows of every partition
 };
 
 struct sat_ctx {
@@ -172,12 +173,14 @@ struct sat_ctx {
     int32_t *row_slot = nullptr;  // [n] cache slot of every partition-major row, -1 for interior nodes (built on first use)
     int64_t *lrowptr = nullptr;   // [n+1] local CSR, rows partition-major
     int32_t *lenc = nullptr;      // [nnz+n] encoded column: < n: partition-major row of an inner node; >= n: n + halo position
-    int32_t *lenc_gid = nullptr;  // [nnz+n] the same with halo columns as n + global node id (built on first use: SAT_FWD_HALO_GLOBAL)
-    int32_t *lenc_all_gid = nullptr; // [nnz+n] every column as a global node id (built on first use: SAT_FWD_INPUT_GLOBAL)
-    std::vector<SrcBlockedItems> src_blocked;  // source-blocked forward work lists, one per block size (built on first use)
+    int2 *ent = nullptr;          // [nnz+n] {encoded column, weight = dinv of the column}: what the SpMM reads
+    int2 *ent_gid = nullptr;      // [nnz+n] the same with halo columns as n + global node id (built on first use: SAT_FWD_HALO_GLOBAL)
+    int2 *ent_all_gid = nullptr;  // [nnz+n] every column as a global node id (built on first use: SAT_FWD_INPUT_GLOBAL)
+    int2 *hent_pos = nullptr;     // [nnz_cut] entries of the halo-row CSR by partition-major row (built on first use)
+    int2 *hent_slot = nullptr;    // [nnz_cut+nb] ... by cache slot, the self entry in front of every row (built on first use)
+    std::deque<SpmmList> lists;   // SpMM work lists (built on first use)
     int32_t *inner_cnt = nullptr; // [n] number of inner entries (incl. self-loop) at the front of each row
     float *dinv_enc = nullptr;    // [n + nb] dinv of the node behind each encoded column
-    float *lw = nullptr;          // [nnz+n] dinv_enc[lenc[e]] stored per entry (read with the column instead of gathered)
     int64_t *hrow_ptr = nullptr;  // [nb+1] halo-row CSR
     int32_t *hrow_pos = nullptr;  // [nnz_cut] partition-major row of the inner neighbour
     int32_t *hrow_slot = nullptr; // [nnz_cut] its cache slot
@@ -188,13 +191,8 @@ struct sat_ctx {
     int32_t *hlong = nullptr;     // [n_hlong] halo positions of the halo rows longer than SAT_HROW_LONG
     int32_t n_hlong = 0;
     std::vector<int32_t> h_hlong_off;
-    // the long halo rows cut into chunks of SAT_HROW_CHUNK entries (a hub next to most of a partition has tens of thousands)
-    int64_t *hchunk_first = nullptr; // [n_hlong+1] first chunk of every long row
-    int32_t *hchunk_row = nullptr;   // [n_hchunks] index into hlong[] of the row a chunk belongs to
     int32_t *halo_tile_order = nullptr;  // [ceil(n_halo / 128)] tiles of 128 halo rows ordered by the cache slot of their first row (built on first use)
-    int32_t n_hchunks = 0;
-    std::vector<int32_t> h_hchunk_off;  // [M+1] first chunk of every partition
-    // SpMM work items (rows cut into chunks of SAT_SPMM_CHUNK edges)
+    // work items of the attention layer (rows cut into chunks of SAT_SPMM_CHUNK edges)
     int32_t *first_item = nullptr; // [n+1]
     int32_t *item_row = nullptr;   // [n_items]
     int32_t *item_mslot = nullptr; // [n_items] index of the partial-sum row for items of multi-chunk rows, else -1
@@ -215,7 +213,6 @@ struct sat_ctx {
 
     // ---- scratch ----
     DevBuf buf_codec_sizes, buf_codec_off, buf_codec_bytes;  // embedding codec scratch
-    DevBuf buf_hpartial, buf_sbpartial;
     DevBuf buf_partial, buf_gagg, buf_splitk, buf_lstm_c, buf_lstm_s, buf_lstm_w, buf_pred_a, buf_misc, buf_colsum, buf_dmask,
         buf_wsplit, buf_wsplit2, buf_wsplit3, buf_bias, buf_pred_train, buf_ghist_halo, buf_ghist_rows, buf_ghist_out, buf_gat, buf_gat_items;
 };
@@ -325,7 +322,7 @@ struct PartView {
     int32_t mitem0, n_mitems; // partial-sum rows
     int32_t push0, n_push;
     int32_t hlong0, n_hlong;  // long halo rows
-    int32_t hchunk0, n_hchunks; // their chunks
+    int p0, p1;               // partitions [p0, p1)
     int64_t lnnz;             // local non-zeros (entries of A + I) of the selected rows
     int64_t hnnz;             // of which entries with a halo column (= entries of the halo-row CSR)
 };
@@ -333,7 +330,8 @@ sat_status sat_part_view(sat_ctx *ctx, int32_t part, PartView *v);
 
 // SpMM family (sat_spmm.cu)
 //   out[row] = dinv[row] * sum_e dinv[col_e] * src(col_e), over all entries of the row (inner_only = 0)
-//   or over its inner prefix (inner_only = 1), or over its halo suffix (inner_only = 2; in_base is not read).  `in_base` / `halo_base` are the virtual bases of the
+//   or over its inner prefix (inner_only = 1), or over its halo suffix (inner_only = 2; in_base is not read, rows without
+//   halo entries are not written).  `in_base` / `halo_base` are the virtual bases of the
 //   partition-major inner matrix and of the concatenated halo matrix (already offset for a single
 //   partition); `out_base` likewise.
 // omask (or null): bit mask [rows x omask_words] indexed like out_base; output components whose bit is 0 are written as 0
@@ -342,9 +340,10 @@ sat_status sat_part_view(sat_ctx *ctx, int32_t part, PartView *v);
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask = nullptr,
                     int32_t omask_words = 0, bool halo_global = false, bool in_global = false);
-//   halo-row products: out[j] = sum_{e in hrow(j)} dinv[halo j] dinv[inner e] * src[pos_e]   (+ self term if self_src)
-sat_status sat_spmm_hrow(sat_ctx *ctx, const PartView &v, int32_t d, const float *src_base, int32_t ld_src,
-                         int by_slot, const float *self_src, float *out_base, int32_t ld_out);
+//   halo-row products: out[j] = sum_{e in hrow(j)} dinv[halo j] dinv[inner e] * src[pos_e], or with by_slot the rows of src by cache
+//   slot, including the self term
+sat_status sat_spmm_hrow(sat_ctx *ctx, const PartView &v, int32_t d, const float *src_base, int32_t ld_src, int by_slot, float *out_base,
+                         int32_t ld_out);
 // src_rows / dst_rows: valid row indices of the source / destination matrices, used by the debug build's index checks
 // (SAT_ANY_ROW: unknown, not checked)
 static const DbgRange SAT_ANY_ROW = {INT64_MIN, INT64_MAX};

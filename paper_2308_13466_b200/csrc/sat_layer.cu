@@ -597,7 +597,7 @@ extern "C" sat_status sat_predict(sat_ctx *ctx, int32_t layer, int32_t part, con
     SAT_TRY(sat_ensure(ctx, ctx->buf_pred_a, (size_t)v.n_halo * ld_a * sizeof(float)));
     float *a = (float *)ctx->buf_pred_a.p;
     // graph convolution on the LSTM state: a_u = p_uu S_u + sum_{v in N(u) cap V_m} p_uv S_v
-    SAT_TRY(sat_spmm_hrow(ctx, v, h, c->S, h, 1, c->S, a - v.halo0 * ld_a, ld_a));
+    SAT_TRY(sat_spmm_hrow(ctx, v, h, c->S, h, 1, a - v.halo0 * ld_a, ld_a));
     if (sat_use_tc(d, h)) {
         TcWeights Wg;
         TcEpilogueHost eh;
@@ -817,7 +817,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
         if (v.n_halo > 0 && v.n_rows > 0) {
             SAT_TRY(sat_ensure(ctx, ctx->buf_ghist_halo, (size_t)v.n_halo * ld_q * sizeof(float)));
             float *qh = (float *)ctx->buf_ghist_halo.p;
-            SAT_TRY(sat_spmm_hrow(ctx, v, d_out, D - (int64_t)v.row0 * ld_d, ld_d, 0, nullptr, qh - v.halo0 * (int64_t)ld_q, ld_q));
+            SAT_TRY(sat_spmm_hrow(ctx, v, d_out, D - (int64_t)v.row0 * ld_d, ld_d, 0, qh - v.halo0 * (int64_t)ld_q, ld_q));
             float *qw = GH.buf + (size_t)(1 - GH.read_idx) * plane;
             if (part == SAT_ALL_PARTS) {
                 // all copies of every boundary node are in qh: one gather-sum per slot, copies taken in partition order
@@ -868,7 +868,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
                                 mask_in, mask_in_words));
     }
     // G_halo = P_out^T G_AGG over the halo-row CSR
-    if (g_halo) SAT_TRY(sat_spmm_hrow(ctx, v, d_in, ga_base, ld_ga, 0, nullptr, g_halo - v.halo0 * (int64_t)ld_gh, ld_gh));
+    if (g_halo) SAT_TRY(sat_spmm_hrow(ctx, v, d_in, ga_base, ld_ga, 0, g_halo - v.halo0 * (int64_t)ld_gh, ld_gh));
     return SAT_OK;
 }
 

@@ -324,7 +324,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     }
     // ---- graph convolution on the final state, output layer, skip connection ----
     const float *newest = k > 0 ? ring_buf(ctx, c, ring_index(ctx, 0)) : nullptr;
-    if (k > 0) SAT_TRY(sat_spmm_hrow(ctx, v, h, hs + (k - 1) * plane_s, h, 1, hs + (k - 1) * plane_s, a, h));
+    if (k > 0) SAT_TRY(sat_spmm_hrow(ctx, v, h, hs + (k - 1) * plane_s, h, 1, a, h));
     else SAT_CUDA(ctx, cudaMemsetAsync(a, 0, (size_t)nb * h * sizeof(float), ctx->stream));
     if (sat_use_tc(d, h)) {
         TcWeights Wg;
