@@ -69,6 +69,11 @@ enum { SAT_ACT_NONE = 0, SAT_ACT_RELU = 1 };
  * halo list.  For layer 1 the caller then needs neither the partition-major copy of the features nor the halo pull.  Same
  * result, bit for bit, as the call on gathered rows. */
 #define SAT_FWD_INPUT_GLOBAL 0x400
+/* ... and SAT_FWD_HALO_CACHED: h_halo is ignored (may be NULL); the out-of-subgraph rows are the plain historical embeddings, read
+ * from the newest committed snapshot of cached layer `layer` - 1 (width d_in) through the halo nodes' cache slots (zeros while
+ * there is no snapshot: then only the in-subgraph terms are summed).  With a snapshot the result is, bit for bit, that of
+ * sat_predict without parameters followed by the plain call, without the [sum_m b_m x d_in] copy.  Not together with the two flags above (SAT_EINVAL). */
+#define SAT_FWD_HALO_CACHED 0x800
 enum { SAT_LOSS_SOFTMAX_CE = 0, SAT_LOSS_SIGMOID_BCE = 1 };
 enum { SAT_ROWS_INNER = 0, SAT_ROWS_HALO = 1 };          /* sat_gather_rows                      */
 enum { SAT_CACHE_ZERO = 0, SAT_CACHE_COPY = 1 };         /* sat_cache_init                       */

@@ -122,6 +122,7 @@ static void free_partition(sat_ctx *ctx)
     dev_free(&ctx->lenc);
     dev_free(&ctx->ent);
     dev_free(&ctx->ent_gid);
+    dev_free(&ctx->ent_slot);
     dev_free(&ctx->ent_all_gid);
     dev_free(&ctx->hent_pos);
     dev_free(&ctx->hent_slot);

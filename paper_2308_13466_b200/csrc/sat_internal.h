@@ -175,6 +175,7 @@ struct sat_ctx {
     int32_t *lenc = nullptr;      // [nnz+n] encoded column: < n: partition-major row of an inner node; >= n: n + halo position
     int2 *ent = nullptr;          // [nnz+n] {encoded column, weight = dinv of the column}: what the SpMM reads
     int2 *ent_gid = nullptr;      // [nnz+n] the same with halo columns as n + global node id (built on first use: SAT_FWD_HALO_GLOBAL)
+    int2 *ent_slot = nullptr;     // [nnz+n] ... as n + cache slot (built on first use: SAT_FWD_HALO_CACHED)
     int2 *ent_all_gid = nullptr;  // [nnz+n] every column as a global node id (built on first use: SAT_FWD_INPUT_GLOBAL)
     int2 *hent_pos = nullptr;     // [nnz_cut] entries of the halo-row CSR by partition-major row (built on first use)
     int2 *hent_slot = nullptr;    // [nnz_cut+nb] ... by cache slot, the self entry in front of every row (built on first use)
@@ -329,17 +330,18 @@ struct PartView {
 sat_status sat_part_view(sat_ctx *ctx, int32_t part, PartView *v);
 
 // SpMM family (sat_spmm.cu)
+enum class SpmmHalo { by_position, by_gid, by_slot };
 //   out[row] = dinv[row] * sum_e dinv[col_e] * src(col_e), over all entries of the row (inner_only = 0)
 //   or over its inner prefix (inner_only = 1), or over its halo suffix (inner_only = 2; in_base is not read, rows without
 //   halo entries are not written).  `in_base` / `halo_base` are the virtual bases of the
 //   partition-major inner matrix and of the concatenated halo matrix (already offset for a single
 //   partition); `out_base` likewise.
 // omask (or null): bit mask [rows x omask_words] indexed like out_base; output components whose bit is 0 are written as 0
-// halo_global: the halo columns address a matrix over all n nodes in global id order (halo_base = its first row);
-// in_global: inner and halo columns both address such a matrix (in_base = its first row; halo_base is not used)
+// halo_kind: what the halo columns address: the concatenated halo matrix, a matrix over all n nodes in global id order, or one over
+// the cache slots (halo_base = its first row in the last two); in_global: inner and halo columns both address such a matrix (in_base = its first row; halo_base is not used)
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask = nullptr,
-                    int32_t omask_words = 0, bool halo_global = false, bool in_global = false);
+                    int32_t omask_words = 0, SpmmHalo halo_kind = SpmmHalo::by_position, bool in_global = false);
 //   halo-row products: out[j] = sum_{e in hrow(j)} dinv[halo j] dinv[inner e] * src[pos_e], or with by_slot the rows of src by cache
 //   slot, including the self term
 sat_status sat_spmm_hrow(sat_ctx *ctx, const PartView &v, int32_t d, const float *src_base, int32_t ld_src, int by_slot, float *out_base,

@@ -676,7 +676,14 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
     const bool push = (act & SAT_FWD_PUSH) != 0;
     const bool in_global = (act & SAT_FWD_INPUT_GLOBAL) != 0;
     const bool halo_global = in_global || (act & SAT_FWD_HALO_GLOBAL) != 0;
-    act &= ~(SAT_FWD_PUSH | SAT_FWD_HALO_GLOBAL | SAT_FWD_INPUT_GLOBAL);
+    const bool halo_cached = (act & SAT_FWD_HALO_CACHED) != 0;
+    act &= ~(SAT_FWD_PUSH | SAT_FWD_HALO_GLOBAL | SAT_FWD_INPUT_GLOBAL | SAT_FWD_HALO_CACHED);
+    if (halo_cached && halo_global) return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: SAT_FWD_HALO_CACHED excludes the global-matrix flags");
+    CacheLayer *hc = nullptr;
+    if (halo_cached) {
+        SAT_TRY(cache_layer(ctx, layer - 1, &hc, "sat_layer_fwd"));
+        if (hc->width != d_in) return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: cached layer %d has width %d, not %d", layer - 1, hc->width, d_in);
+    }
     if (d_in <= 0 || d_out <= 0 || !W || (act != SAT_ACT_NONE && act != SAT_ACT_RELU)) return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: bad dims / W / act");
     CacheLayer *pc = nullptr;
     if (push) {
@@ -685,7 +692,7 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
     }
     if (v.n_rows > 0 && (!h_in || !h_out || !ok_ld(ld_in, d_in) || !ok_ld(ld_out, d_out) || !aligned16(h_in) || !aligned16(h_out)))
         return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: null / misaligned h_in / h_out or bad leading dimension");
-    if (!in_global && v.n_halo > 0 && (!h_halo || !ok_ld(ld_halo, d_in) || !aligned16(h_halo)))
+    if (!in_global && !halo_cached && v.n_halo > 0 && (!h_halo || !ok_ld(ld_halo, d_in) || !aligned16(h_halo)))
         return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: null / misaligned h_halo or bad ld_halo");
     LayerState &L = ctx->layers[layer];
     const int32_t ld_agg = round_up4(d_in), words = (d_out + 31) / 32;
@@ -704,7 +711,14 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
     // over all nodes; the halo source is the concatenated halo matrix (virtual first row) or a matrix over all nodes
     const float *in_base = in_global ? h_in : h_in - (int64_t)v.row0 * ld_in;
     const float *halo_base = in_global || !h_halo ? nullptr : halo_global ? h_halo : h_halo - v.halo0 * (int64_t)ld_halo;
-    SAT_TRY(sat_spmm(ctx, v, 0, d_in, in_base, ld_in, halo_base, ld_halo, L.agg, ld_agg, nullptr, 0, halo_global, in_global));
+    SpmmHalo halo_kind = halo_global ? SpmmHalo::by_gid : SpmmHalo::by_position;
+    if (halo_cached) {
+        halo_kind = SpmmHalo::by_slot;
+        halo_base = ctx->n_valid > 0 ? ring_buf(ctx, hc, ring_index(ctx, 0)) : nullptr;
+        ld_halo = hc->ld;
+    }
+    // (no snapshot yet: the halo terms are zero, the inner entries of the rows are all there is)
+    SAT_TRY(sat_spmm(ctx, v, halo_cached && !halo_base ? 1 : 0, d_in, in_base, ld_in, halo_base, ld_halo, L.agg, ld_agg, nullptr, 0, halo_kind, in_global));
     uint32_t *mask_out = act == SAT_ACT_RELU ? L.mask + (int64_t)v.row0 * words : nullptr;
     const float *agg = L.agg + (int64_t)v.row0 * ld_agg;
     if (sat_use_tc(d_out, d_in)) {

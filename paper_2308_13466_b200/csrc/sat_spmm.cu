@@ -614,13 +614,13 @@ static sat_status run_list(sat_ctx *ctx, const PartView &v, const SpmmList &l, i
     return SAT_OK;
 }
 
-// entries with halo columns as n + global node id (for a halo source that is a matrix over all nodes)
-__global__ void k_ent_by_gid(const int2 *__restrict__ ent, const int32_t *__restrict__ halo_gid, int64_t count, int32_t n, int2 *__restrict__ out)
+// entries with halo columns as n + global node id or n + cache slot (`halo_id` of the halo position)
+__global__ void k_ent_by_id(const int2 *__restrict__ ent, const int32_t *__restrict__ halo_id, int64_t count, int32_t n, int2 *__restrict__ out)
 {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= count) return;
     const int2 q = ent[e];
-    out[e] = make_int2(q.x < n ? q.x : n + halo_gid[q.x - n], q.y);
+    out[e] = make_int2(q.x < n ? q.x : n + halo_id[q.x - n], q.y);
 }
 
 // entries with every column as a global node id (inner columns through the partition-major order, halo columns through the halo list)
@@ -635,7 +635,7 @@ __global__ void k_ent_all_gid(const int2 *__restrict__ ent, const int32_t *__res
 
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask, int32_t omask_words,
-                    bool halo_global, bool in_global)
+                    SpmmHalo halo_kind, bool in_global)
 {
     if (v.n_rows == 0) return SAT_OK;
     const int32_t d4 = (d + 3) / 4;
@@ -656,18 +656,20 @@ sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, 
         a.ent = ctx->ent_all_gid;
         a.src = DbgRange{0, ctx->n};
         a.halo = DbgRange{0, 0};
-    } else if (halo_global) {
-        if (!ctx->ent_gid) {
-            SAT_CUDA(ctx, cudaMalloc((void **)&ctx->ent_gid, (size_t)lnnz * sizeof(int2)));
-            k_ent_by_gid<<<(unsigned)cdiv64(lnnz, 256), 256, 0, ctx->stream>>>(ctx->ent, ctx->halo_gid, lnnz, ctx->n, ctx->ent_gid);
+    } else if (halo_kind != SpmmHalo::by_position && inner_only == 0) {
+        const bool slot = halo_kind == SpmmHalo::by_slot;
+        int2 *&ent = slot ? ctx->ent_slot : ctx->ent_gid;
+        if (!ent) {
+            SAT_CUDA(ctx, cudaMalloc((void **)&ent, (size_t)lnnz * sizeof(int2)));
+            k_ent_by_id<<<(unsigned)cdiv64(lnnz, 256), 256, 0, ctx->stream>>>(ctx->ent, slot ? ctx->halo_slot : ctx->halo_gid, lnnz, ctx->n, ent);
             SAT_LAUNCHED(ctx);
         }
-        a.ent = ctx->ent_gid;
-        a.halo = DbgRange{0, ctx->n};
+        a.ent = ent;
+        a.halo = DbgRange{0, slot ? ctx->n_slots : ctx->n};
     }
     // algorithmic bytes: column ids + row offsets + dinv, every source row once, every output row once (a halo source over
     // all nodes holds at most n distinct rows)
-    const double n_halo_src = halo_global && v.n_halo > ctx->n ? (double)ctx->n : (double)v.n_halo;
+    const double n_halo_src = halo_kind != SpmmHalo::by_position && v.n_halo > ctx->n ? (double)ctx->n : (double)v.n_halo;
     double n_src = inner_only == 1 ? (double)v.n_rows : inner_only == 2 ? n_halo_src : (double)v.n_rows + n_halo_src;
     if (in_global && n_src > ctx->n) n_src = ctx->n;
     // the backward reads the inner prefix of every row, the transposed predictor convolution the halo suffix

@@ -83,7 +83,8 @@ class SatEpoch:
         return self.X_in
 
     def halo_view(self, l: int, m: int = B.SAT_ALL_PARTS):
-        """Halo rows of the input of GNN layer l + 1 (predicted embeddings of cached layer l), all partitions or one."""
+        """Halo rows of the input of GNN layer l + 1 (predicted embeddings of cached layer l), all partitions or one.  (Plain
+        historical embeddings are read from the ring by the layer and not copied here.)"""
         d = self.dims[l]
         if m == B.SAT_ALL_PARTS:
             return self.halo[:, :d]
@@ -105,9 +106,12 @@ class SatEpoch:
                 # itself (global id order) through the partition's inner and halo lists: no gathered copies, no pull
                 h_in, hv = self.X, None
                 act |= B.SAT_FWD_INPUT_GLOBAL
+            elif pred is None or pred[l - 2] is None:
+                hv = None                            # plain historical embeddings: the layer reads them from the ring itself
+                act |= B.SAT_FWD_HALO_CACHED
             else:
                 hv = self.halo_view(l - 1, m)
-                B.sat_predict(ctx, l - 1, m, pred[l - 2] if pred is not None else None, reuse_state, hv)  # pull predicted
+                B.sat_predict(ctx, l - 1, m, pred[l - 2], reuse_state, hv)  # pull predicted
             h_out = self.rows(self.H[l], m)
             # forward; for the cached layers the push of the boundary rows rides on the transform's epilogue
             B.sat_layer_fwd(ctx, m, l, h_in, hv, W[l - 1], b[l - 1], act, h_out)
