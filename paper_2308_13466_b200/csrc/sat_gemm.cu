@@ -286,11 +286,11 @@ k_splitk_reduce(const float *__restrict__ part, int64_t count, int32_t splits, i
 }
 
 sat_status sat_splitk_reduce(sat_ctx *ctx, const float *part, int64_t count, int32_t splits, int accumulate, float *out, int32_t ncols,
-                             int32_t ld_out)
+                             int32_t ld_out, const float *part2, int64_t count2, float *out2)
 {
     if (count == 0) return SAT_OK;
-    const int64_t b1 = cdiv64(count, 32);
-    k_splitk_reduce<<<(unsigned)b1, 256, 0, ctx->stream>>>(part, count, splits, accumulate, out, ncols, ld_out, b1, nullptr, 0, nullptr);
+    const int64_t b1 = cdiv64(count, 32), b2 = out2 ? cdiv64(count2, 32) : 0;
+    k_splitk_reduce<<<(unsigned)(b1 + b2), 256, 0, ctx->stream>>>(part, count, splits, accumulate, out, ncols, ld_out, b1, part2, count2, out2);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
@@ -314,10 +314,7 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN), (unsigned)splits);
     k_gemm_tn<<<grid, 256, 0, ctx->stream>>>(rows, rows_per_split, m, n, A, lda, B, ldb, mask, mask_words, part_C, part_cs);
     SAT_LAUNCHED(ctx);
-    const int64_t b1 = cdiv64((int64_t)m * n, 32), b2 = colsum ? cdiv64(n, 32) : 0;
-    k_splitk_reduce<<<(unsigned)(b1 + b2), 256, 0, ctx->stream>>>(part_C, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, b1, part_cs, n, colsum);
-    SAT_LAUNCHED(ctx);
-    return SAT_OK;
+    return sat_splitk_reduce(ctx, part_C, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, part_cs, n, colsum);
 }
 
 // =====================================================================================
@@ -342,9 +339,13 @@ __device__ __forceinline__ void tnn_cp16(void *smem_dst, const void *gsrc, bool 
 template <int NT>
 __global__ void __launch_bounds__(128)
 k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, const float *__restrict__ A, int64_t lda,
-                 const float *__restrict__ B, int64_t ldb, float *__restrict__ part)
+                 const float *__restrict__ B, int64_t ldb, float *__restrict__ part, float *__restrict__ part_cs)
 {
     extern __shared__ __align__(16) float tnn_smem[];
+    // column sums of B (the bias gradient), by the blocks with y == 0: thread t takes column t % NT of every (128 / NT)-th staged row
+    constexpr int CS_GROUPS = 128 / NT;
+    const bool want_cs = part_cs != nullptr && blockIdx.y == 0 && threadIdx.x < NT * CS_GROUPS;
+    float cs = 0.f;
     constexpr int STAGE_FLOATS = TNN_STAGE * 256 + TNN_STAGE * NT;
     const int32_t m0 = blockIdx.y * 256;
     const int32_t col0 = m0 + threadIdx.x, col1 = col0 + 128;
@@ -396,7 +397,21 @@ k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, con
                 acc1[j4 / 2 + 1] = __ffma2_rn(a1p, bhi, acc1[j4 / 2 + 1]);
             }
         }
+        if (want_cs) {
+#pragma unroll 4
+            for (int rr = threadIdx.x / NT; rr < TNN_STAGE; rr += CS_GROUPS) cs += Bs[rr * NT + threadIdx.x % NT];
+        }
         __syncthreads();  // the stage is refilled two iterations later
+    }
+    if (part_cs != nullptr && blockIdx.y == 0) {
+        if (want_cs) tnn_smem[threadIdx.x] = cs;
+        __syncthreads();
+        if ((int)threadIdx.x < n) {
+            float t = tnn_smem[threadIdx.x];
+#pragma unroll
+            for (int g = 1; g < CS_GROUPS; ++g) t += tnn_smem[g * NT + threadIdx.x];
+            part_cs[(int64_t)blockIdx.x * n + threadIdx.x] = t;
+        }
     }
     if (col0 < m) {
         float *o = part + ((int64_t)blockIdx.x * m + col0) * n;
@@ -414,7 +429,7 @@ k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, con
 
 template <int NT>
 static sat_status launch_tn_narrow(sat_ctx *ctx, dim3 grid, int64_t rows, int64_t rpb, int32_t m, int32_t n, const float *A, int32_t lda,
-                                   const float *B, int32_t ldb, float *part)
+                                   const float *B, int32_t ldb, float *part, float *part_cs)
 {
     static PerDeviceOnce attr_set;
     const size_t smem = 2 * (size_t)(TNN_STAGE * 256 + TNN_STAGE * NT) * sizeof(float);
@@ -422,14 +437,14 @@ static sat_status launch_tn_narrow(sat_ctx *ctx, dim3 grid, int64_t rows, int64_
         SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tn_narrow<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr_set.mark(ctx->device);
     }
-    k_gemm_tn_narrow<NT><<<grid, 128, smem, ctx->stream>>>(rows, rpb, m, n, A, lda, B, ldb, part);
+    k_gemm_tn_narrow<NT><<<grid, 128, smem, ctx->stream>>>(rows, rpb, m, n, A, lda, B, ldb, part, part_cs);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
 
 // C[m x n] (+)= A^T B over `rows` rows for n <= 64 (B already masked)
 sat_status sat_gemm_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb,
-                              float *C, int32_t ldc, int accumulate)
+                              float *C, int32_t ldc, int accumulate, float *colsum)
 {
     if (m == 0 || n == 0) return SAT_OK;
     if (n > 64 || (lda & 3) || (ldb & 3) || (((uintptr_t)A | (uintptr_t)B) & 15u))
@@ -442,14 +457,15 @@ sat_status sat_gemm_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, 
     int64_t rpb = cdiv64(cdiv64(rows > 0 ? rows : 1, want), TNN_STAGE) * TNN_STAGE;
     if (rpb < 4 * TNN_STAGE) rpb = 4 * TNN_STAGE;
     const int64_t blocks = cdiv64(rows > 0 ? rows : 1, rpb);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)blocks * m * n * sizeof(float)));
+    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)blocks * ((size_t)m * n + n) * sizeof(float)));
     float *part = (float *)ctx->buf_splitk.p;
+    float *part_cs = colsum ? part + (size_t)blocks * m * n : nullptr;
     dim3 grid((unsigned)blocks, (unsigned)cdiv64(m, 256));
-    if (n <= 16) SAT_TRY(launch_tn_narrow<16>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part));
-    else if (n <= 32) SAT_TRY(launch_tn_narrow<32>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part));
-    else if (n <= 48) SAT_TRY(launch_tn_narrow<48>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part));
-    else SAT_TRY(launch_tn_narrow<64>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part));
-    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)blocks, accumulate, C, n, ldc);
+    if (n <= 16) SAT_TRY(launch_tn_narrow<16>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
+    else if (n <= 32) SAT_TRY(launch_tn_narrow<32>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
+    else if (n <= 48) SAT_TRY(launch_tn_narrow<48>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
+    else SAT_TRY(launch_tn_narrow<64>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
+    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)blocks, accumulate, C, n, ldc, part_cs, n, colsum);
 }
 
 // =====================================================================================

@@ -724,11 +724,15 @@ done:
 }
 
 // =====================================================================================
-// MN-major kernel (weight gradient): block (x, y, z) = tile (x, y) of A^T B over rows [z * rps, (z + 1) * rps)
+// MN-major kernel (weight gradient): block (x, y, z) = tile (x, y) of A^T B over rows [z * rps, (z + 1) * rps); the blocks with x == 0
+// also leave the column sums of their rows of B (the bias gradient) in part_cs [z x N] when it is given: the converters hold every
+// value of B in registers anyway, which saves a pass over it (34 us for 169 k x 256).
+// The main loop is bound by shared-memory traffic: per k-block of 16 rows at N = 256 the TMA writes 24 KB, the converters read 24
+// and write 48 KB and the MMAs read 72 KB, 0.7 us at 128 B per clock against 0.4 us of tensor work.
 // =====================================================================================
 __global__ void __launch_bounds__(TC_THREADS, 2)
 k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int32_t Mdim, int32_t N, int64_t rps,
-             int32_t bn, int32_t stages, int32_t tmem_cols, float *part_C, int *status)
+             int32_t bn, int32_t stages, int32_t tmem_cols, float *part_C, float *part_cs, int *status)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -808,6 +812,10 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
         }
     } else {
         const int ctid = threadIdx.x - 64;
+        const bool want_cs = part_cs != nullptr && blockIdx.x == 0;
+        float4 cs[8];   // this thread's share of the column sums: one 16-byte piece of every 32-column block, row ctid / 8 of each k-block
+#pragma unroll
+        for (int bl = 0; bl < 8; ++bl) cs[bl] = make_float4(0.f, 0.f, 0.f, 0.f);
         bool alive = true;
         for (int32_t kb = 0; kb < nkb && alive; ++kb) {
             const int s = kb % stages;
@@ -816,25 +824,65 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
             if (!alive) break;
             uint8_t *st = smem + (size_t)s * stage_bytes;
             split_tile_round(st, st + a_bytes, a_bytes, ctid, TC_CONV_THREADS);
-            split_tile_round(st + 2 * a_bytes, st + 2 * a_bytes + b_bytes, b_bytes, ctid, TC_CONV_THREADS);
+            if (!want_cs) {
+                split_tile_round(st + 2 * a_bytes, st + 2 * a_bytes + b_bytes, b_bytes, ctid, TC_CONV_THREADS);
+            } else {
+                uint8_t *bh = st + 2 * a_bytes + ctid * 16, *bl_ = bh + b_bytes;
+#pragma unroll
+                for (int bl = 0; bl < 8; ++bl) {
+                    if (bl < n_blks_b) {
+                        const float4 x = *reinterpret_cast<const float4 *>(bh + bl * blk_bytes);
+                        float4 h, l;
+                        split4(x, h, l);
+                        *reinterpret_cast<float4 *>(bh + bl * blk_bytes) = h;
+                        *reinterpret_cast<float4 *>(bl_ + bl * blk_bytes) = l;
+                        cs[bl].x += x.x;
+                        cs[bl].y += x.y;
+                        cs[bl].z += x.z;
+                        cs[bl].w += x.w;
+                    }
+                }
+            }
             fence_async_smem();
             mbar_arrive(&sh->conv[s]);
         }
         const int q = warp & 3;
-        const int32_t row = m0 + q * 32 + lane;
-        const bool ok = alive && mbar_wait(&sh->accum, 0, dead, status);
+        const bool ok = alive && mbar_wait(&sh->accum, 0, dead, status);   // every MMA has completed: the stages are free
         tc_fence_after();
         if (ok) {
+            // each warp turns its 32 x 32 block around in shared memory and writes whole row segments: with one row per lane a store
+            // instruction touched 32 lines, and the partial sums of a tile took 35 us
+            float *tb = reinterpret_cast<float *>(smem) + q * (32 * 33);
             float *pc = part_C + (int64_t)blockIdx.z * Mdim * N;
+            const int32_t row0 = m0 + q * 32;
             for (int c0 = 0; c0 < bn; c0 += 32) {
                 uint32_t r[32];
                 tc_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-                if (row >= Mdim) continue;
+                __syncwarp();
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int32_t col = n0 + c0 + j;
-                    if (col < N) pc[(int64_t)row * N + col] = __uint_as_float(r[j]);
+                for (int j = 0; j < 32; ++j) tb[lane * 33 + j] = __uint_as_float(r[j]);
+                __syncwarp();
+                const int32_t col = n0 + c0 + lane;
+                if (col < N) {
+#pragma unroll 8
+                    for (int i = 0; i < 32; ++i)
+                        if (row0 + i < Mdim) pc[(int64_t)(row0 + i) * N + col] = tb[i * 33 + lane];
                 }
+            }
+        }
+        if (want_cs) {
+            // the 16 rows of a k-block lie in 16 groups of eight threads; the 32-byte atoms of a row are exchanged by its low two bits
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            float *cb = reinterpret_cast<float *>(smem);   // [16][n_blks_b * 32]
+            const int rr = ctid >> 3, piece = (ctid & 7) ^ ((rr & 3) << 1), w = n_blks_b * 32;
+#pragma unroll
+            for (int bl = 0; bl < 8; ++bl)
+                if (bl < n_blks_b && ok) *reinterpret_cast<float4 *>(cb + rr * w + bl * 32 + piece * 4) = cs[bl];
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            for (int c = ctid; c < w; c += TC_CONV_THREADS) {
+                float t = cb[c];
+                for (int g = 1; g < 16; ++g) t += cb[g * w + c];
+                if (n0 + c < N && c < bn) part_cs[(int64_t)blockIdx.z * N + n0 + c] = t;
             }
         }
     }
@@ -1161,7 +1209,7 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
 
 // C[m x n] (+)= A^T B over `rows` rows: A fp32 [rows x m] (lda), B fp32 [rows x n] (ldb)
 sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb, float *C,
-                          int32_t ldc, int accumulate)
+                          int32_t ldc, int accumulate, float *colsum)
 {
     if (m == 0 || n == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_GEMM_TN, 4.0 * ((double)rows * (m + n) + (double)m * n), 2.0 * (double)rows * m * n);
@@ -1173,14 +1221,20 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
     if (stages < 2) stages = 2;
     const size_t smem = (size_t)stages * stage_bytes + sizeof(TcShared) + 1024;
     const int64_t tiles = cdiv64(m, TC_BM) * cdiv64(n, bn);
+    // Two CTAs fit on an SM: one wave of 2 x 148 for tall inputs.  Below ~100 k-blocks per CTA of such a wave, half as many splits: the
+    // m x n partial sums of a split cost as much as ~10 of its k-blocks (21 k rows, 256 x 256: 65 us with 148 splits of the old store,
+    // see the epilogue)
+    const int64_t kblocks = cdiv64(rows > 0 ? rows : 1, TC_BK);
     int64_t splits = (2 * 148 + tiles - 1) / tiles;
+    if (kblocks < 40 * splits) splits = (148 + tiles - 1) / tiles;
     const int64_t max_splits = cdiv64(rows > 0 ? rows : 1, 8 * TC_BK);
     if (splits > max_splits) splits = max_splits;
     if (splits < 1) splits = 1;
     const int64_t rps = cdiv64(cdiv64(rows > 0 ? rows : 1, splits), TC_BK) * TC_BK;
     splits = cdiv64(rows > 0 ? rows : 1, rps);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)splits * m * n * sizeof(float)));
+    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)splits * ((size_t)m * n + n) * sizeof(float)));
     float *part = (float *)ctx->buf_splitk.p;
+    float *part_cs = colsum ? part + (size_t)splits * m * n : nullptr;
     CUtensorMap mA, mB;
     SAT_TRY(make_map(ctx, &mA, A, m, rows, lda, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
     SAT_TRY(make_map(ctx, &mB, B, n, rows, ldb, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
@@ -1189,7 +1243,7 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
         g_attr_mn.mark(ctx->device);
     }
     dim3 grid((unsigned)cdiv64(m, TC_BM), (unsigned)cdiv64(n, bn), (unsigned)splits);
-    k_gemm_tc_mn<<<grid, TC_THREADS, smem, ctx->stream>>>(mA, mB, m, n, rps, bn, stages, tmem_cols_for(bn), part, ctx->d_flag + 1);
+    k_gemm_tc_mn<<<grid, TC_THREADS, smem, ctx->stream>>>(mA, mB, m, n, rps, bn, stages, tmem_cols_for(bn), part, part_cs, ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
-    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc);
+    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, part_cs, n, colsum);
 }

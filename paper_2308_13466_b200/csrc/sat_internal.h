@@ -384,11 +384,12 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
                        int32_t ldb, const uint32_t *mask, int32_t mask_words, float *C, int32_t ldc, float *colsum,
                        int accumulate);
 
-// out[r][c] (+)= sum_z part[z][r * ncols + c], z ascending (fixed order: reproducible)
+// C[m x n] (+)= A^T B, colsum[n] (+)= 1^T B if non-null, for n <= 64 (B already masked)
 sat_status sat_gemm_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb,
-                              float *C, int32_t ldc, int accumulate);
+                              float *C, int32_t ldc, int accumulate, float *colsum = nullptr);
+// out[r][c] (+)= sum_z part[z][r * ncols + c] in a fixed order (reproducible); the same launch can take a second, one-row array
 sat_status sat_splitk_reduce(sat_ctx *ctx, const float *part, int64_t count, int32_t splits, int accumulate, float *out, int32_t ncols,
-                             int32_t ld_out);
+                             int32_t ld_out, const float *part2 = nullptr, int64_t count2 = 0, float *out2 = nullptr);
 
 // GEMM family on the tensor cores (sat_gemm_tc.cu): TF32 two-term split, fp32 operands in global memory
 // Cell state of the fused LSTM (internal scratch, never exposed): blocks of [32 rows x 8 units] = 1 KB, block index
@@ -476,6 +477,6 @@ sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeig
 // C[m x n] = [A | A2] B^T (+ epilogue)
 sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32_t lda, int32_t k1, const float *A2, int32_t lda2, int32_t k2,
                        const TcWeights &Bw, const TcEpilogueHost &eh, int family);
-// C[m x n] (+)= A^T B over `rows` rows
+// C[m x n] (+)= A^T B over `rows` rows, colsum[n] (+)= 1^T B if non-null
 sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb, float *C,
-                          int32_t ldc, int accumulate);
+                          int32_t ldc, int accumulate, float *colsum = nullptr);

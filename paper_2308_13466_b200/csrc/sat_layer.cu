@@ -800,19 +800,15 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
     const bool tc_x = want_dx && !g_halo && sat_use_tc(d_in, d_out);
     const float *D = g_out;  // D = g_out o [Z > 0]: materialised once for the tensor-core contractions
     int32_t ld_d = ld_g;
-    if (tc_w || tc_x || (hist && mask)) {
-        float *dm = nullptr;
-        if (mask) {
-            ld_d = round_up4(d_out);
-            SAT_TRY(sat_ensure(ctx, ctx->buf_dmask, (size_t)v.n_rows * ld_d * sizeof(float)));
-            dm = (float *)ctx->buf_dmask.p;
-            D = dm;
-        }
-        SAT_TRY(sat_mask_rows(ctx, g_out, ld_g, v.n_rows, d_out, mask, L.mask_words, dm, ld_d, tc_w ? g_b : nullptr, accumulate));
+    if (mask && (tc_w || tc_x || hist)) {
+        ld_d = round_up4(d_out);
+        SAT_TRY(sat_ensure(ctx, ctx->buf_dmask, (size_t)v.n_rows * ld_d * sizeof(float)));
+        D = (float *)ctx->buf_dmask.p;
+        SAT_TRY(sat_mask_rows(ctx, g_out, ld_g, v.n_rows, d_out, mask, L.mask_words, (float *)ctx->buf_dmask.p, ld_d, nullptr, accumulate));
     }
     // G_W (+)= AGG^T D, G_b (+)= 1^T D
-    if (tc_w && d_out <= 64) SAT_TRY(sat_gemm_tn_narrow(ctx, v.n_rows, d_in, d_out, agg, L.ld_in, D, ld_d, g_W, d_out, accumulate));
-    else if (tc_w) SAT_TRY(sat_gemm_tc_tn(ctx, v.n_rows, d_in, d_out, agg, L.ld_in, D, ld_d, g_W, d_out, accumulate));
+    if (tc_w && d_out <= 64) SAT_TRY(sat_gemm_tn_narrow(ctx, v.n_rows, d_in, d_out, agg, L.ld_in, D, ld_d, g_W, d_out, accumulate, g_b));
+    else if (tc_w) SAT_TRY(sat_gemm_tc_tn(ctx, v.n_rows, d_in, d_out, agg, L.ld_in, D, ld_d, g_W, d_out, accumulate, g_b));
     else SAT_TRY(sat_gemm_tn(ctx, v.n_rows, d_in, d_out, agg, L.ld_in, g_out, ld_g, mask, L.mask_words, g_W, d_out, g_b, accumulate));
     // gradient-side history, this epoch's contribution: Q_write[slot(u)] += (P_out^T D)[u] for the halo nodes u of the
     // selected partitions, one partition after the other (the halo slots of one partition are distinct)

@@ -1,0 +1,206 @@
+"""Kernels and dispatch rules at the sizes where they can go wrong: run lengths around the limits of the SpMM work lists, column
+slices, row splits and tiles of the weight gradient, class counts of the losses.  References are computed in fp64; a sum of k fp32
+terms t_i in any order is within k 2^-24 sum |t_i| of the exact one (u = 2^-24; one rounding per product and per addition), and the
+TF32 contractions add at most 2^-20 of the same sum (two-term split, truncating accumulation)."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+import torch
+
+from tests.gpu_util import dev, dev2d, empty2d
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -24
+
+
+@pytest.fixture(scope="module")
+def B():
+    import paper_2308_13466_b200.binding as binding
+    return binding
+
+
+def _graph(hubs, n):
+    """Node i < len(hubs) is next to hubs[i] others (evenly spread); a ring keeps every node connected."""
+    pairs = {(i, (i + 1) % n) for i in range(n)}
+    for i, deg in enumerate(hubs):
+        pairs |= {(i, int(j)) for j in np.linspace(0, n - 1, deg).astype(int) if j != i}
+    a = np.array([(min(p), max(p)) for p in pairs if p[0] != p[1]])
+    m = sp.coo_matrix((np.ones(len(a)), (a[:, 0], a[:, 1])), shape=(n, n))
+    m = ((m + m.T) > 0).astype(np.float64).tocsr()
+    m.sort_indices()
+    return m
+
+
+def _propagation(A):
+    dinv = 1.0 / np.sqrt(np.asarray(A.sum(1)).ravel() + 1.0)
+    return sp.diags(dinv) @ (A + sp.identity(A.shape[0])) @ sp.diags(dinv)
+
+
+# degrees around the run lengths (32), the block reduction of many runs (16 x 32) and far above
+HUBS = [29, 30, 31, 32, 33, 62, 64, 100, 500, 510, 520, 1000, 2900]
+
+
+@pytest.mark.parametrize("d", [4, 5, 12, 31, 33, 64, 65, 100, 128, 129, 256, 260, 300, 512, 602])
+def test_aggregation_and_its_transpose(B, d):
+    n, M = 3000, 3
+    A = _graph(HUBS, n)
+    P = _propagation(A)
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    part = rng.integers(0, M, n).astype(np.int32)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+        off = np.concatenate([[0], np.cumsum(np.bincount(part, minlength=M))])
+        eye = dev(np.eye(d, 4, dtype=np.float32))            # four output columns on the CUDA cores: the aggregation itself, columns 0-3
+        out = empty2d(n, 4)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(X), None, eye, None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, out)
+        want, mag = P @ X.astype(np.float64), abs(P) @ np.abs(X.astype(np.float64))
+        terms = np.diff(A.indptr).max() + 8
+        err = np.abs(out.cpu().numpy() - want[perm][:, :4])
+        assert (err <= terms * U * mag[perm][:, :4]).all()
+        # every column through the weight gradient with one-hot gradients: G_W = AGG^T D picks rows of AGG
+        rows = rng.choice(n, 3, replace=False)
+        D = np.zeros((n, 3), np.float32)
+        D[rows, np.arange(3)] = 1.0
+        W3 = dev(np.zeros((d, 3), np.float32))
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(X), None, W3, None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, empty2d(n, 3))
+        gW, gb = torch.full((d, 3), float("nan"), device="cuda"), torch.full((3,), float("nan"), device="cuda")
+        B.sat_layer_bwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(D), W3, gW, gb, 0, None, None)
+        assert (np.abs(gW.cpu().numpy().T - want[perm[rows]]) <= terms * U * mag[perm[rows]]).all()
+        assert (gb.cpu().numpy() == 1.0).all()
+        # G_in of a layer with W = first rows of the identity: P_in^T D; all partitions at once = one after the other
+        k = min(d, 4)
+        Wi = dev(np.eye(d, k, dtype=np.float32))
+        G = rng.standard_normal((n, k)).astype(np.float32)
+        h_in = dev2d(X[perm])
+        n_halo = B.sat_part_sizes(ctx, B.SAT_ALL_PARTS)[1]
+        halo = dev2d(np.zeros((n_halo, d), np.float32))
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, h_in, halo, Wi, None, B.SAT_ACT_NONE, empty2d(n, k))
+        gW2, g_in, g_halo = torch.empty((d, k), device="cuda"), empty2d(n, d), empty2d(n_halo, d)
+        B.sat_layer_bwd(ctx, B.SAT_ALL_PARTS, 2, dev2d(G), Wi, gW2, None, 0, g_in, g_halo)
+        same = sp.csr_matrix((P.tocoo().data * (part[P.tocoo().row] == part[P.tocoo().col]), (P.tocoo().row, P.tocoo().col)), shape=P.shape)
+        Gn = np.zeros((n, k))
+        Gn[perm] = G
+        want_in, mag_in = same @ Gn, abs(same) @ np.abs(Gn)
+        assert (np.abs(g_in.cpu().numpy()[:, :k] - want_in[perm]) <= terms * U * mag_in[perm]).all()
+        one = empty2d(n, d)
+        for m in range(M):
+            r = slice(off[m], off[m + 1])
+            B.sat_layer_bwd(ctx, m, 2, dev2d(G[r]), Wi, gW2, None, 0, one[r], None)
+        assert torch.equal(one[:, :k], g_in[:, :k])
+        lists = [B.sat_part_lists(ctx, m) for m in range(M)]
+        gh, h0 = g_halo.cpu().numpy()[:, :k], 0
+        for m in range(M):
+            ids, inner = lists[m]["halo_gid"], perm[off[m]:off[m + 1]]
+            sub = P.tocsr()[ids][:, inner]
+            assert (np.abs(gh[h0:h0 + len(ids)] - sub @ Gn[inner]) <= terms * U * (abs(sub) @ np.abs(Gn[inner]))).all()
+            h0 += len(ids)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("given", [False, True])
+def test_historical_rows_read_from_the_ring(B, given):
+    """SAT_FWD_HALO_CACHED against the pull through sat_predict: same bits once there is a snapshot, and zeros before."""
+    n, M, d, d2 = 1500, 4, 40, 24
+    A = _graph(HUBS[:9], n)
+    rng = np.random.default_rng(2)
+    part = rng.integers(0, M, n).astype(np.int32) if given else None
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN if given else B.SAT_PART_CONTIG_BLOCKS, part)
+        B.sat_cache_init(ctx, [d], 2)
+        sizes = [B.sat_part_sizes(ctx, m) for m in range(M)]
+        H, W = dev2d(rng.standard_normal((n, d)).astype(np.float32)), dev(rng.standard_normal((d, d2)).astype(np.float32))
+        for epoch in range(3):
+            halo = empty2d(sum(s[1] for s in sizes), d)
+            B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, None, 0, halo)
+            a, b, c = empty2d(n, d2), empty2d(n, d2), empty2d(n, d2)
+            B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, H, halo, W, None, B.SAT_ACT_NONE, a)
+            B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, H, None, W, None, B.SAT_ACT_NONE | B.SAT_FWD_HALO_CACHED, b)
+            r0 = 0
+            for m in range(M):
+                r1 = r0 + sizes[m][0]
+                B.sat_layer_fwd(ctx, m, 2, H[r0:r1], None, W, None, B.SAT_ACT_NONE | B.SAT_FWD_HALO_CACHED, c[r0:r1])
+                r0 = r1
+            assert torch.equal(b, c)
+            assert torch.equal(a, b) if epoch else torch.allclose(a, b, rtol=0, atol=float(a.abs().max()) * 600 * U)
+            B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, dev2d(rng.standard_normal((n, d)).astype(np.float32)))
+            B.sat_cache_commit(ctx)
+        for bad in (B.SAT_FWD_HALO_GLOBAL, B.SAT_FWD_INPUT_GLOBAL):
+            with pytest.raises(B.SatError) as ei:
+                B.sat_layer_fwd(ctx, 0, 2, H, H, W, None, B.SAT_ACT_NONE | B.SAT_FWD_HALO_CACHED | bad, empty2d(n, d2))
+            assert ei.value.status == B.SAT_EINVAL
+        with pytest.raises(B.SatError):                       # layer 1 has no cached layer below it
+            B.sat_layer_fwd(ctx, 0, 1, H, None, W, None, B.SAT_ACT_NONE | B.SAT_FWD_HALO_CACHED, empty2d(n, d2))
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("rows", [3, 64, 255, 256, 257, 1000, 5000, 21000])
+@pytest.mark.parametrize("m,n", [(4, 3), (16, 16), (20, 64), (130, 48), (128, 65), (100, 100), (256, 256), (300, 260), (65, 512)])
+def test_weight_and_bias_gradient(B, rows, m, n):
+    """G_W = AGG^T D and G_b = 1^T D of a layer on a ring graph (AGG from three rows each), one partition."""
+    A = _graph([], rows)
+    P = _propagation(A)
+    rng = np.random.default_rng(rows + m + n)
+    X, D = rng.standard_normal((rows, m)).astype(np.float32), rng.standard_normal((rows, n)).astype(np.float32)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, 1, B.SAT_PART_CONTIG_BLOCKS)
+        W = dev(np.zeros((m, n), np.float32))
+        B.sat_layer_fwd(ctx, 0, 1, dev2d(X), None, W, None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, empty2d(rows, n))
+        gW, gb = torch.full((m, n), float("nan"), device="cuda"), torch.full((n,), float("nan"), device="cuda")
+        B.sat_layer_bwd(ctx, 0, 1, dev2d(D), W, gW, gb, 0, None, None)
+        X64, D64 = P @ X.astype(np.float64), D.astype(np.float64)
+        mag = (abs(P) @ np.abs(X.astype(np.float64))).T @ np.abs(D64)       # AGG itself carries 8 roundings of its own terms
+        assert (np.abs(gW.cpu().numpy() - X64.T @ D64) <= ((min(rows, 1500) + 8) * U + 2.0 ** -20) * mag).all()
+        assert (np.abs(gb.cpu().numpy() - D64.sum(0)) <= min(rows, 1500) * U * np.abs(D64).sum(0)).all()
+        B.sat_layer_bwd(ctx, 0, 1, dev2d(D), W, gW, gb, 1, None, None)      # accumulate
+        assert (np.abs(gb.cpu().numpy() - 2 * D64.sum(0)) <= 2 * (min(rows, 1500) + 2) * U * np.abs(D64).sum(0)).all()
+        assert (np.abs(gW.cpu().numpy() - 2 * (X64.T @ D64)) <= 2 * ((min(rows, 1500) + 10) * U + 2.0 ** -20) * mag).all()
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("rows", [3, 31, 33, 1000, 30011])
+@pytest.mark.parametrize("C", [1, 2, 8, 9, 16, 17, 32, 33, 64, 65, 100, 128, 129, 300])
+@pytest.mark.parametrize("kind", ["ce", "bce"])
+def test_losses(B, rows, C, kind):
+    """Loss sum and gradient; expf / logf / log1pf are within 2 units in the last place, the sums of C terms as above."""
+    rng = np.random.default_rng(C)
+    A = _graph([], rows)
+    z = (3 * rng.standard_normal((rows, C))).astype(np.float32)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, 1, B.SAT_PART_CONTIG_BLOCKS)
+        z64 = torch.from_numpy(z).double().requires_grad_()
+        if kind == "ce":
+            y = rng.integers(0, C, rows).astype(np.int32)
+            per = torch.nn.functional.cross_entropy(z64, torch.from_numpy(y).long(), reduction="none")
+        else:
+            y = (rng.random((rows, C)) < 0.3).astype(np.uint8)
+            per = torch.nn.functional.binary_cross_entropy_with_logits(z64, torch.from_numpy(y).double(), reduction="none").mean(1)
+        want = per.sum() / rows
+        want.backward()
+        for view in (dev2d(z), torch.zeros((rows, C + 3), device="cuda")[:, :C]):      # rows of 16 bytes, and any rows
+            view.copy_(torch.from_numpy(z))
+            g, total = torch.full((rows, C + 1), float("nan"), device="cuda")[:, :C], torch.zeros(1, dtype=torch.float64, device="cuda")
+            for _ in range(2):
+                B.sat_loss_grad(ctx, 0, B.SAT_LOSS_SOFTMAX_CE if kind == "ce" else B.SAT_LOSS_SIGMOID_BCE, view, dev(y), total, g)
+            # one term of a row: a few roundings of values up to |z| + log C, about 20
+            assert abs(float(total) / 2 - float(want.detach())) <= (C + 16) * U * max(20.0, float(want.detach()))
+            assert float((g.cpu().double() - z64.grad).abs().max()) <= (C + 16) * U / rows * (1.0 if kind == "ce" else 1.0 / C)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
