@@ -139,10 +139,9 @@ static void free_partition(sat_ctx *ctx)
     dev_free(&ctx->hrow_w);
     dev_free(&ctx->hlong);
     dev_free(&ctx->halo_tile_order);
-    dev_free(&ctx->first_item);
-    dev_free(&ctx->item_row);
-    dev_free(&ctx->item_mslot);
-    dev_free(&ctx->mrows);
+    dev_free(&ctx->gat_rev);
+    dev_free(&ctx->gat_hmap);
+    dev_free(&ctx->gat_long);
     ctx->part_ok = false;
 }
 
@@ -174,6 +173,7 @@ static void free_layers(sat_ctx *ctx)
         sat_free_buf(ctx->gat[i].z_in);
         sat_free_buf(ctx->gat[i].z_halo);
         sat_free_buf(ctx->gat[i].scal);
+        sat_free_buf(ctx->gat[i].ent);
         ctx->gat[i].d_out = 0;
         ctx->gat[i].valid.clear();
     }
@@ -829,45 +829,6 @@ __global__ void k_hlong_fill(const int32_t *__restrict__ flag, const int64_t *__
     if (j < nb && flag[j]) out[off[j]] = (int32_t)j;
 }
 
-__global__ void k_chunks(const int64_t *__restrict__ lrowptr, int32_t n, int32_t *__restrict__ nch)
-{
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) nch[r] = (int32_t)((lrowptr[r + 1] - lrowptr[r] + SAT_SPMM_CHUNK - 1) / SAT_SPMM_CHUNK);
-}
-
-__global__ void k_items(const int64_t *__restrict__ item_off, int32_t n, int32_t *__restrict__ first_item, int32_t *__restrict__ item_row,
-                        int32_t *__restrict__ item_multi)
-{
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r > n) return;
-    first_item[r] = (int32_t)item_off[r];
-    if (r == n) return;
-    int32_t a = (int32_t)item_off[r], b = (int32_t)item_off[r + 1];
-    for (int32_t i = a; i < b; ++i) {
-        item_row[i] = (int32_t)r;
-        item_multi[i] = (b - a) > 1 ? 1 : 0;
-    }
-}
-
-__global__ void k_item_mslot(const int32_t *__restrict__ item_multi, const int64_t *__restrict__ moff, int32_t n_items,
-                             int32_t *__restrict__ item_mslot)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_items) item_mslot[i] = item_multi[i] ? (int32_t)moff[i] : -1;
-}
-
-__global__ void k_mrow_flag(const int32_t *__restrict__ first_item, int32_t n, int32_t *__restrict__ flag)
-{
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) flag[r] = (first_item[r + 1] - first_item[r]) > 1 ? 1 : 0;
-}
-
-__global__ void k_mrow_fill(const int32_t *__restrict__ flag, const int64_t *__restrict__ off, int32_t n, int32_t *__restrict__ mrows)
-{
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n && flag[r]) mrows[off[r]] = (int32_t)r;
-}
-
 // =====================================================================================
 // sat_partition
 // =====================================================================================
@@ -965,14 +926,14 @@ extern "C" sat_status sat_partition(sat_ctx *ctx, int32_t M, int method, const i
     }
 
     // temporaries (freed at the end of this function)
-    int32_t *t_hist = nullptr, *t_cnt = nullptr, *t_flag = nullptr, *t_item_multi = nullptr;
-    int64_t *t_hist_off = nullptr, *t_woff = nullptr, *t_coff = nullptr, *t_off = nullptr, *t_item_off = nullptr, *t_moff = nullptr;
+    int32_t *t_hist = nullptr, *t_cnt = nullptr, *t_flag = nullptr;
+    int64_t *t_hist_off = nullptr, *t_woff = nullptr, *t_coff = nullptr, *t_off = nullptr;
     uint32_t *t_bits = nullptr, *t_cbits = nullptr;
     sat_status rc = SAT_OK;
     auto cleanup = [&]() {
         cudaStreamSynchronize(st);
-        dev_free(&t_hist); dev_free(&t_cnt); dev_free(&t_flag); dev_free(&t_item_multi);
-        dev_free(&t_hist_off); dev_free(&t_woff); dev_free(&t_coff); dev_free(&t_off); dev_free(&t_item_off); dev_free(&t_moff);
+        dev_free(&t_hist); dev_free(&t_cnt); dev_free(&t_flag);
+        dev_free(&t_hist_off); dev_free(&t_woff); dev_free(&t_coff); dev_free(&t_off);
         dev_free(&t_bits); dev_free(&t_cbits);
     };
 #define P_TRY(expr)             \
@@ -1157,56 +1118,6 @@ extern "C" sat_status sat_partition(sat_ctx *ctx, int32_t M, int method, const i
         P_TRY(rc);
     }
 
-    // ---- work items of the attention layer ----
-    P_TRY(dev_alloc(ctx, &t_item_off, (int64_t)n + 2));
-    P_TRY(dev_alloc(ctx, &ctx->first_item, (int64_t)n + 1));
-    k_chunks<<<GRID1(n)>>>(ctx->lrowptr, n, t_flag);
-    P_LAUNCHED();
-    P_TRY(sat_scan_i32(ctx, t_flag, n, t_item_off));
-    int64_t n_items64 = 0;
-    P_TRY(copy_i64(ctx, t_item_off + n, &n_items64));
-    P_CUDA(cudaStreamSynchronize(st));
-    if (n_items64 >= ((int64_t)1 << 31)) P_TRY(sat_fail(ctx, SAT_EINVAL, "sat_partition: too many work items"));
-    ctx->n_items = (int32_t)n_items64;
-    P_TRY(dev_alloc(ctx, &ctx->item_row, ctx->n_items));
-    P_TRY(dev_alloc(ctx, &ctx->item_mslot, ctx->n_items));
-    P_TRY(dev_alloc(ctx, &t_item_multi, (int64_t)ctx->n_items + 1));
-    P_TRY(dev_alloc(ctx, &t_moff, (int64_t)ctx->n_items + 2));
-    k_items<<<GRID1((int64_t)n + 1)>>>(t_item_off, n, ctx->first_item, ctx->item_row, t_item_multi);
-    P_LAUNCHED();
-    P_TRY(sat_scan_i32(ctx, t_item_multi, ctx->n_items, t_moff));
-    k_item_mslot<<<GRID1(ctx->n_items)>>>(t_item_multi, t_moff, ctx->n_items, ctx->item_mslot);
-    P_LAUNCHED();
-    int64_t n_mitems64 = 0;
-    P_TRY(copy_i64(ctx, t_moff + ctx->n_items, &n_mitems64));
-    ctx->h_item_off.assign(M + 1, 0);
-    ctx->h_mitem_off.assign(M + 1, 0);
-    ctx->h_mrow_off.assign(M + 1, 0);
-    std::vector<int64_t> item_off_h((size_t)M + 1), mitem_off_h((size_t)M + 1), mrow_off_h((size_t)M + 1);
-    for (int m = 0; m <= M; ++m) P_TRY(copy_i64(ctx, t_item_off + ctx->h_inner_off[m], &item_off_h[m]));
-    P_CUDA(cudaStreamSynchronize(st));
-    for (int m = 0; m <= M; ++m) {
-        ctx->h_item_off[m] = (int32_t)item_off_h[m];
-        P_TRY(copy_i64(ctx, t_moff + ctx->h_item_off[m], &mitem_off_h[m]));
-    }
-    // multi-chunk rows
-    k_mrow_flag<<<GRID1(n)>>>(ctx->first_item, n, t_flag);
-    P_LAUNCHED();
-    P_TRY(sat_scan_i32(ctx, t_flag, n, t_off));
-    int64_t n_mrows64 = 0;
-    P_TRY(copy_i64(ctx, t_off + n, &n_mrows64));
-    for (int m = 0; m <= M; ++m) P_TRY(copy_i64(ctx, t_off + ctx->h_inner_off[m], &mrow_off_h[m]));
-    P_CUDA(cudaStreamSynchronize(st));
-    ctx->n_mitems = (int32_t)n_mitems64;
-    ctx->n_mrows = (int32_t)n_mrows64;
-    for (int m = 0; m <= M; ++m) {
-        ctx->h_mitem_off[m] = (int32_t)mitem_off_h[m];
-        ctx->h_mrow_off[m] = (int32_t)mrow_off_h[m];
-    }
-    P_TRY(dev_alloc(ctx, &ctx->mrows, ctx->n_mrows));
-    k_mrow_fill<<<GRID1(n)>>>(t_flag, t_off, n, ctx->mrows);
-    P_LAUNCHED();
-
     cleanup();
     if (ctx->cuda_failed) return SAT_ECUDA;
     cudaError_t e = cudaGetLastError();
@@ -1225,12 +1136,6 @@ sat_status sat_part_view(sat_ctx *ctx, int32_t part, PartView *v)
     v->n_rows = ctx->h_inner_off[b] - v->row0;
     v->halo0 = ctx->h_halo_off[a];
     v->n_halo = ctx->h_halo_off[b] - v->halo0;
-    v->item0 = ctx->h_item_off[a];
-    v->n_items = ctx->h_item_off[b] - v->item0;
-    v->mrow0 = ctx->h_mrow_off[a];
-    v->n_mrows = ctx->h_mrow_off[b] - v->mrow0;
-    v->mitem0 = ctx->h_mitem_off[a];
-    v->n_mitems = ctx->h_mitem_off[b] - v->mitem0;
     v->push0 = ctx->h_push_off[a];
     v->n_push = ctx->h_push_off[b] - v->push0;
     v->lnnz = ctx->h_lnnz_off[b] - ctx->h_lnnz_off[a];

@@ -8,11 +8,15 @@
 //     dpre_vu = alpha_vu (dalpha_vu - t_v) LeakyReLU'(pre_vu);  ds_dst[v] = sum_u dpre_vu;  ds_src[u] = sum_v dpre_vu;
 //     dZ_u = sum_v alpha_vu D_v + ds_src[u] a_src (+ ds_dst[u] a_dst for inner u);
 //     G_W = H^T dZ over inner and halo rows;  G_a_src = Z^T ds_src;  G_a_dst = Z_in^T ds_dst;  G_b = 1^T D;  G_in = dZ_in W^T.
-// The sums over v for a fixed u run over the inner prefix of u's own row (the inner block is symmetric) or over the
-// halo-row CSR; alpha_vu is recomputed from the per-row scalars (s_dst[v], log-sum-exp of row v), so no per-edge array
-// is stored.  One warp per work item of the SpMM (a row, or a 256-entry chunk of a long row), per-item partial sums added in
-// item order by small combine kernels: every sum has a single writer and a fixed order.  The halo-node side of the backward
-// still walks a halo row with one warp.
+// Every sum has a single writer and a fixed order.  How it is cut into passes:
+//   forward   k_gat_alpha: softmax of every row, written as {column, alpha} entries; the weighted sums of z rows are then the product
+//             kernel of the GCN layer (sat_spmm_entries) with those entries and a bias / ReLU epilogue.
+//   backward  k_gat_dots: D_v . z_u of every entry, once (a gather of z rows, doubles out); k_gat_rows: t_v, ds_dst and the entry's
+//             alpha and dpre; k_gat_cols brings both to the column side through an index of mirrored entries (gat_prepare) and sums
+//             ds_src; dZ is again the product kernel, with D rows gathered and the a_src / a_dst terms in its epilogue.
+// The first version recomputed alpha and the dot product in each of three gather sweeps and walked every halo row with one warp:
+// 169 k nodes, 2.6 M entries, 256 wide: 763 + 626 + 911 us per layer in its sweeps against 389 (dots) + 65 (rows, cols) + 370 (the two
+// products) now.
 #include "sat_internal.h"
 
 #define GAT_SLOPE 0.2f
@@ -42,16 +46,6 @@ __device__ __forceinline__ float4 ldz(const float *row, int c4, int d)
 }
 __device__ __forceinline__ float dot4(const float4 &a, const float4 &b) { return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w))); }
 __device__ __forceinline__ float lrelu(float x) { return x > 0.f ? x : GAT_SLOPE * x; }
-// D_v . z_u feeds differences (dalpha - t_v) that cancel most of their size: the products are summed in double
-__device__ __forceinline__ double ddot4(const float4 &a, const float4 &b)
-{
-    return (double)a.x * (double)b.x + (double)a.y * (double)b.y + (double)a.z * (double)b.z + (double)a.w * (double)b.w;
-}
-__device__ __forceinline__ double warp_sum_d(double x)
-{
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
 
 // s_src[r] = a_src . z_r, s_dst[r] = a_dst . z_r (when asked for); one warp per row
 __global__ void __launch_bounds__(256)
@@ -62,10 +56,17 @@ k_gat_scores(const float *__restrict__ z, int64_t ld, int64_t rows, int32_t d, c
     const int lane = threadIdx.x & 31;
     if (r >= rows) return;
     float ps = 0.f, pd = 0.f;
-    for (int c = lane; c < d; c += 32) {
-        const float x = z[r * ld + c];
-        ps = fmaf(x, a_src[c], ps);
-        if (a_dst) pd = fmaf(x, a_dst[c], pd);
+    for (int c4 = lane; 4 * c4 < d; c4 += 32) {   // rows are 16-byte aligned and padded with zeros, the vectors end at d
+        const float4 x = __ldg(reinterpret_cast<const float4 *>(z + r * ld) + c4);
+        const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = 4 * c4 + k;
+            if (c < d) {
+                ps = fmaf(xs[k], a_src[c], ps);
+                if (a_dst) pd = fmaf(xs[k], a_dst[c], pd);
+            }
+        }
     }
     ps = warp_sum(ps);
     pd = warp_sum(pd);
@@ -75,494 +76,320 @@ k_gat_scores(const float *__restrict__ z, int64_t ld, int64_t rows, int32_t d, c
     }
 }
 
-// forward over work items: k_gat_lse (a warp per row, lanes over the entries) gives the log-sum-exp of every row; then one warp
-// per item accumulates its chunk of the weighted sum.  Rows of a single item are finished here (bias, ReLU); items of
-// longer rows write their partial sum to `partial` (row index item_mslot) and k_gat_fwd_fixup adds them in item order.
-__global__ void __launch_bounds__(256)
-k_gat_lse(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ lenc, int32_t n, int32_t row0, int32_t n_rows,
-          const float *__restrict__ s_in, const float *__restrict__ s_halo, const float *__restrict__ s_dst, float *__restrict__ lse)
+// A row is worked on by a team of T threads: 16 lanes of a warp for the ordinary rows, a thread block for rows of more than GAT_LONG
+// entries (a hub's ten thousand entries were the whole launch for one warp).
+#define GAT_TEAM 16
+#define GAT_LONG SAT_HROW_LONG
+
+template <int T, typename V, typename F>
+__device__ __forceinline__ V team_reduce(V x, F op, V *sh)
 {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    if (T < 256) {
+        const unsigned mask = ((1u << (T & 31)) - 1u) << (threadIdx.x & 31 & ~(T - 1));
+#pragma unroll
+        for (int o = T / 2; o > 0; o >>= 1) x = op(x, __shfl_xor_sync(mask, x, o));
+        return x;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = op(x, __shfl_xor_sync(0xffffffffu, x, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
+    __syncthreads();
+    x = sh[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) x = op(x, sh[w]);
+    return x;
+}
+struct OpAdd {
+    template <typename V> __device__ V operator()(V a, V b) const { return a + b; }
+};
+struct OpMax {
+    __device__ float operator()(float a, float b) const { return fmaxf(a, b); }
+};
+
+// softmax of one row: ent[e] = {column, alpha}
+template <int T>
+__device__ __forceinline__ void gat_alpha_row(int tid, int64_t e0, int64_t e1, float sd, const int32_t *__restrict__ lenc, int32_t n,
+                                              const float *__restrict__ s_in, const float *__restrict__ s_halo, int2 *__restrict__ ent, float *sh)
+{
+    auto logit = [&](int32_t c) { return lrelu(sd + (c < n ? s_in[c] : s_halo[c - n])); };
+    // the first entry of every thread stays in registers (most rows have no more); the others are fetched again per pass
+    const int64_t ef = e0 + tid;
+    const int32_t c_first = ef < e1 ? lenc[ef] : 0;
+    const float l_first = ef < e1 ? logit(c_first) : -INFINITY;
+    float mx = l_first;
+#pragma unroll 4
+    for (int64_t e = ef + T; e < e1; e += T) mx = fmaxf(mx, logit(lenc[e]));
+    mx = team_reduce<T>(mx, OpMax(), sh);
+    const float x_first = ef < e1 ? expf(l_first - mx) : 0.f;
+    float den = x_first;
+#pragma unroll 4
+    for (int64_t e = ef + T; e < e1; e += T) den += expf(logit(lenc[e]) - mx);
+    den = team_reduce<T>(den, OpAdd(), sh);
+    if (ef < e1) ent[ef] = make_int2(c_first, __float_as_int(x_first / den));
+#pragma unroll 4
+    for (int64_t e = ef + T; e < e1; e += T) {
+        const int32_t c = lenc[e];
+        ent[e] = make_int2(c, __float_as_int(expf(logit(c) - mx) / den));
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_gat_alpha(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ lenc, int32_t n, int32_t row0, int32_t n_rows,
+            const int32_t *__restrict__ long_rows, int32_t n_long, const float *__restrict__ s_in, const float *__restrict__ s_halo,
+            const float *__restrict__ s_dst, int2 *__restrict__ ent)
+{
+    __shared__ float sh[8];
+    if ((int32_t)blockIdx.x < n_long) {
+        const int32_t row = long_rows[blockIdx.x];
+        gat_alpha_row<256>(threadIdx.x, lrowptr[row], lrowptr[row + 1], s_dst[row], lenc, n, s_in, s_halo, ent, sh);
+        return;
+    }
+    const int64_t w = ((int64_t)(blockIdx.x - n_long) * 256 + threadIdx.x) / GAT_TEAM;
     if (w >= n_rows) return;
     const int32_t row = row0 + (int32_t)w;
     const int64_t e0 = lrowptr[row], e1 = lrowptr[row + 1];
-    const float sd = s_dst[row];
-    float mx = -INFINITY;
-    for (int64_t e = e0 + lane; e < e1; e += 32) {
-        const int32_t c = lenc[e];
-        mx = fmaxf(mx, lrelu(sd + (c < n ? s_in[c] : s_halo[c - n])));
-    }
-    mx = warp_max(mx);
-    float den = 0.f;
-    for (int64_t e = e0 + lane; e < e1; e += 32) {
-        const int32_t c = lenc[e];
-        den += expf(lrelu(sd + (c < n ? s_in[c] : s_halo[c - n])) - mx);
-    }
-    den = warp_sum(den);
-    if (lane == 0) lse[row] = mx + logf(den);
+    if (e1 - e0 > GAT_LONG) return;
+    gat_alpha_row<GAT_TEAM>(threadIdx.x & (GAT_TEAM - 1), e0, e1, s_dst[row], lenc, n, s_in, s_halo, ent, sh);
 }
 
-template <int NV>
-__global__ void __launch_bounds__(256)
-k_gat_fwd_items(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ lenc, const int32_t *__restrict__ item_row,
-                const int32_t *__restrict__ first_item, const int32_t *__restrict__ item_mslot, int32_t item0, int32_t n_items, int32_t mitem0,
-                int32_t n, const float *__restrict__ z_in, const float *__restrict__ z_halo, int64_t ld_z, const float *__restrict__ s_in,
-                const float *__restrict__ s_halo, const float *__restrict__ s_dst, const float *__restrict__ lse, int32_t d,
-                const float *__restrict__ bias, int relu, float *__restrict__ out_base, int64_t ld_out, float *__restrict__ partial)
+// dots[e] = D_v . z_u for every entry (v, u): a group of G lanes per work item, D_v in registers, four z rows in flight.  The products
+// are summed in double ((dalpha - t_v) cancels most of their size); the sums of four entries are reduced together, six
+// shuffles for the four.  Bound by the conversions of the gathered values to double (256 per entry at d = 256).
+template <int G, int NV>
+__global__ void __launch_bounds__(256, NV <= 2 ? 3 : NV <= 4 ? 2 : 1)
+k_gat_dots(const int4 *__restrict__ items, int32_t n_items, const int32_t *__restrict__ lenc, int32_t n, int32_t d4, const float *__restrict__ z_in,
+           const float *__restrict__ z_halo, uint32_t ldz4, const float *__restrict__ D, double *__restrict__ dots)
 {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= n_items) return;
-    const int32_t item = item0 + (int32_t)w;
-    const int32_t row = item_row[item];
-    const int64_t re = lrowptr[row + 1];
-    const int64_t e0 = lrowptr[row] + (int64_t)(item - first_item[row]) * SAT_SPMM_CHUNK;
-    const int64_t e1 = e0 + SAT_SPMM_CHUNK < re ? e0 + SAT_SPMM_CHUNK : re;
-    const float sd = s_dst[row], l = lse[row];
-    const int d4 = (d + 3) >> 2;
-    float4 acc[NV];
+    const int lane = threadIdx.x & (G - 1);
+    const int64_t gid = ((int64_t)blockIdx.x * 256 + threadIdx.x) / G;
+    if (gid >= n_items) return;
+    const unsigned mask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+    const int4 it = __ldg(items + gid);
+    const int64_t e0 = (int64_t)(uint32_t)it.z | ((int64_t)(it.w & 0xffff) << 32);
+    const int32_t len = it.w >> 16;
+    const float4 *zi = reinterpret_cast<const float4 *>(z_in) + lane, *zh = reinterpret_cast<const float4 *>(z_halo) + lane - (int64_t)n * ldz4;
+    double dv[NV][4];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t eb = e0; eb < e1; eb += 32) {
-        const int64_t e = eb + lane;
-        int32_t c = 0;
-        float a = 0.f;
-        if (e < e1) {
-            c = lenc[e];
-            a = expf(lrelu(sd + (c < n ? s_in[c] : s_halo[c - n])) - l);
+    for (int v = 0; v < NV; ++v) {
+        const float4 x = lane + v * G < d4 ? __ldg(reinterpret_cast<const float4 *>(D) + (int64_t)it.x * ldz4 + lane + v * G) : make_float4(0.f, 0.f, 0.f, 0.f);
+        dv[v][0] = x.x;
+        dv[v][1] = x.y;
+        dv[v][2] = x.z;
+        dv[v][3] = x.w;
+    }
+    const int32_t *__restrict__ cols = lenc + e0;
+    for (int32_t e = 0; e < len; e += 4) {
+        float4 x[4][NV];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int32_t c = __ldg(cols + (e + u < len ? e + u : len - 1));
+            const float4 *src = (c < n ? zi : zh) + (uint64_t)(uint32_t)c * ldz4;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) x[u][v] = lane + v * G < d4 ? __ldg(src + v * G) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        const int cnt = (e1 - eb) < 32 ? (int)(e1 - eb) : 32;
-#pragma unroll 4
-        for (int j = 0; j < cnt; ++j) {
-            const int32_t cj = __shfl_sync(0xffffffffu, c, j);
-            const float aj = __shfl_sync(0xffffffffu, a, j);
-            const float *src = cj < n ? z_in + (int64_t)cj * ld_z : z_halo + (int64_t)(cj - n) * ld_z;
+        double p[4];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const int c4 = lane + 32 * v;
-                if (c4 < d4) {
-                    const float4 x = *reinterpret_cast<const float4 *>(src + 4 * c4);
-                    acc[v].x = fmaf(aj, x.x, acc[v].x);
-                    acc[v].y = fmaf(aj, x.y, acc[v].y);
-                    acc[v].z = fmaf(aj, x.z, acc[v].z);
-                    acc[v].w = fmaf(aj, x.w, acc[v].w);
-                }
-            }
+        for (int u = 0; u < 4; ++u) {
+            p[u] = 0.0;
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+                p[u] += dv[v][0] * (double)x[u][v].x + dv[v][1] * (double)x[u][v].y + dv[v][2] * (double)x[u][v].z + dv[v][3] * (double)x[u][v].w;
+        }
+        // lanes with bit 1 keep entries 2 and 3, the others 0 and 1; then bit 0 picks one; then the lanes that hold the same entry add up
+        const bool b1 = lane & 2, b0 = lane & 1;
+        double q0 = (b1 ? p[2] : p[0]) + __shfl_xor_sync(mask, b1 ? p[0] : p[2], 2);
+        double q1 = (b1 ? p[3] : p[1]) + __shfl_xor_sync(mask, b1 ? p[1] : p[3], 2);
+        double r = (b0 ? q1 : q0) + __shfl_xor_sync(mask, b0 ? q0 : q1, 1);
+#pragma unroll
+        for (int o = G / 2; o > 2; o >>= 1) r += __shfl_xor_sync(mask, r, o);
+        if (lane < 4 && e + lane < len) dots[e0 + e + lane] = r;
+    }
+}
+
+// per row v: t_v = sum alpha dot / sum alpha and ds_dst[v]; per entry, over the dot product: {alpha, dpre = alpha slope (dot - t_v)}
+// (the sums in double and divided by sum alpha: the fp32 weights sum to 1 + eps, and ds_dst, exactly zero where all slopes agree,
+// would inherit -eps t_v)
+template <int T>
+__device__ __forceinline__ void gat_row(int tid, int64_t e0, int64_t e1, float sd, const int2 *__restrict__ ent, int32_t n,
+                                        const float *__restrict__ s_in, const float *__restrict__ s_halo, double *__restrict__ dots,
+                                        float *__restrict__ ds_dst, double *sh)
+{
+    auto slope = [&](int32_t c) { return sd + (c < n ? s_in[c] : s_halo[c - n]) > 0.f ? 1.f : GAT_SLOPE; };
+    const int64_t ef = e0 + tid;
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, p_first = 0.0;
+    float al_first = 0.f, as_first = 0.f;
+#pragma unroll 4
+    for (int64_t e = ef; e < e1; e += T) {
+        const int2 q = ent[e];
+        const float al = __int_as_float(q.y), sl = slope(q.x);
+        const double p = dots[e], as = (double)al * (double)sl;
+        a0 += (double)al;
+        a1 += (double)al * p;
+        a2 += as * p;
+        a3 += as;
+        if (e == ef) {
+            p_first = p;
+            al_first = al;
+            as_first = al * sl;
         }
     }
-    const int32_t ms = item_mslot[item];
-    if (ms >= 0) {
-        float *o = partial + (int64_t)(ms - mitem0) * ld_z;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int c4 = lane + 32 * v;
-            if (c4 < d4) *reinterpret_cast<float4 *>(o + 4 * c4) = acc[v];
-        }
+    a0 = team_reduce<T>(a0, OpAdd(), sh);
+    a1 = team_reduce<T>(a1, OpAdd(), sh);
+    a2 = team_reduce<T>(a2, OpAdd(), sh);
+    a3 = team_reduce<T>(a3, OpAdd(), sh);
+    const double t = a1 / a0;
+    if (tid == 0) *ds_dst = (float)(a2 / a0 - t * (a3 / a0));
+    float2 *edge = reinterpret_cast<float2 *>(dots);
+    if (ef < e1) edge[ef] = make_float2(al_first, (float)((double)as_first * (p_first - t)));
+#pragma unroll 4
+    for (int64_t e = ef + T; e < e1; e += T) {
+        const int2 q = ent[e];
+        const float al = __int_as_float(q.y);
+        edge[e] = make_float2(al, (float)((double)(al * slope(q.x)) * (dots[e] - t)));
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_gat_rows(const int64_t *__restrict__ lrowptr, const int2 *__restrict__ ent, int32_t n, int32_t row0, int32_t n_rows, const int32_t *__restrict__ long_rows,
+           int32_t n_long, const float *__restrict__ s_in, const float *__restrict__ s_halo, const float *__restrict__ s_dst, double *dots,
+           float *__restrict__ ds_dst)
+{
+    __shared__ double sh[8];
+    if ((int32_t)blockIdx.x < n_long) {
+        const int32_t row = long_rows[blockIdx.x];
+        gat_row<256>(threadIdx.x, lrowptr[row], lrowptr[row + 1], s_dst[row], ent, n, s_in, s_halo, dots, ds_dst + row, sh);
         return;
     }
-    float *o = out_base + (int64_t)row * ld_out;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        if (c4 < d4) {
-            float4 r = acc[v];
-            const int c = 4 * c4;
-            if (bias) {
-                r.x += bias[c];
-                if (c + 1 < d) r.y += bias[c + 1];
-                if (c + 2 < d) r.z += bias[c + 2];
-                if (c + 3 < d) r.w += bias[c + 3];
-            }
-            if (relu) {
-                r.x = fmaxf(r.x, 0.f);
-                r.y = fmaxf(r.y, 0.f);
-                r.z = fmaxf(r.z, 0.f);
-                r.w = fmaxf(r.w, 0.f);
-            }
-            *reinterpret_cast<float4 *>(o + 4 * c4) = r;
-        }
-    }
+    const int64_t w = ((int64_t)(blockIdx.x - n_long) * 256 + threadIdx.x) / GAT_TEAM;
+    if (w >= n_rows) return;
+    const int32_t row = row0 + (int32_t)w;
+    const int64_t e0 = lrowptr[row], e1 = lrowptr[row + 1];
+    if (e1 - e0 > GAT_LONG) return;
+    gat_row<GAT_TEAM>(threadIdx.x & (GAT_TEAM - 1), e0, e1, s_dst[row], ent, n, s_in, s_halo, dots, ds_dst + row, sh);
 }
 
-// rows cut into several items: add the partial sums in item order, then bias and activation
-__global__ void k_gat_fwd_fixup(const int32_t *__restrict__ mrows, int32_t mrow0, int32_t n_mrows, const int32_t *__restrict__ first_item,
-                                const int32_t *__restrict__ item_mslot, int32_t mitem0, int32_t d, const float *__restrict__ partial, int64_t ld_z,
-                                const float *__restrict__ bias, int relu, float *__restrict__ out_base, int64_t ld_out)
+// column side of node u: its entries are the mirror images map[e] of row entries (v, u); ent_out[e] = {v, alpha_vu}, ds_src[u] = sum dpre_vu
+template <int T>
+__device__ __forceinline__ void gat_col(int tid, int64_t e0, int64_t e1, const int32_t *__restrict__ idx, const uint32_t *__restrict__ map,
+                                        const float2 *__restrict__ edge, int2 *__restrict__ ent_out, float *__restrict__ ds_src, double *sh)
 {
-    const int d4 = (d + 3) >> 2;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t i = sat_div(t, d4);
-    const int c4 = (int)(t - i * d4);
-    if (i >= n_mrows) return;
-    const int32_t row = mrows[mrow0 + i];
-    const int32_t it0 = first_item[row], it1 = first_item[row + 1];
-    const int32_t ms0 = item_mslot[it0] - mitem0;
-    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int32_t q = 0; q < it1 - it0; ++q) {
-        const float4 x = *reinterpret_cast<const float4 *>(partial + (int64_t)(ms0 + q) * ld_z + 4 * c4);
-        r.x += x.x;
-        r.y += x.y;
-        r.z += x.z;
-        r.w += x.w;
-    }
-    const int c = 4 * c4;
-    if (bias) {
-        r.x += bias[c];
-        if (c + 1 < d) r.y += bias[c + 1];
-        if (c + 2 < d) r.z += bias[c + 2];
-        if (c + 3 < d) r.w += bias[c + 3];
-    }
-    if (relu) {
-        r.x = fmaxf(r.x, 0.f);
-        r.y = fmaxf(r.y, 0.f);
-        r.z = fmaxf(r.z, 0.f);
-        r.w = fmaxf(r.w, 0.f);
-    }
-    *reinterpret_cast<float4 *>(out_base + (int64_t)row * ld_out + 4 * c4) = r;
-}
-
-// D = g o [h_out > 0] (ReLU layer) or g
-__global__ void k_gat_dmask(const float *__restrict__ g, int64_t ld_g, const float *__restrict__ h_out, int64_t ld_h, int64_t rows, int32_t d,
-                            float *__restrict__ D, int64_t ld_d)
-{
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t r = sat_div(t, d);
-    const int c = (int)(t - r * d);
-    if (r >= rows) return;
-    const float x = g[r * ld_g + c];
-    D[r * ld_d + c] = (!h_out || h_out[r * ld_h + c] > 0.f) ? x : 0.f;
-}
-
-// Column-side walk shared by the three kernels below: entries e_first, e_first + stride, ... (< e_end) of an index list of
-// rows v that hold node u.  The lanes fetch the row scalars of 32 entries at a time — one exponential per entry instead of
-// one per lane and entry — and then walk those entries together, lanes over the columns, four rows in flight.
-//   acc += alpha_vu D_v,   returns sum_v alpha_vu slope_vu (D_v . z_u - t_v), the same on every lane
-// ds_src is linear in the dot products, so every lane keeps its own share and the warp is reduced once at the end (the
-// first version reduced every dot product across the warp: ten dependent shuffles per entry).
-template <int NV>
-__device__ __forceinline__ double gat_cols_walk(const int32_t *__restrict__ idx, int64_t e_first, int64_t e_end, int64_t stride, float su,
-                                                const float *__restrict__ s_dst, const float *__restrict__ lse, const double *__restrict__ t_in,
-                                                const float *__restrict__ D, int64_t ld_d, int32_t d, int d4, int lane, const float4 (&zu)[NV],
-                                                float4 (&acc)[NV])
-{
-    double dss = 0.0, tss = 0.0;
-    for (int64_t eb = e_first; eb < e_end; eb += 32 * stride) {
-        const int64_t e = eb + lane * stride;
-        int32_t v_row = 0;
-        float al = 0.f, as = 0.f;
-        if (e < e_end) {
-            v_row = idx[e];
-            const float pre = s_dst[v_row] + su;
-            al = expf(lrelu(pre) - lse[v_row]);
-            as = al * (pre > 0.f ? 1.f : GAT_SLOPE);
-            tss += (double)as * t_in[v_row];
-        }
-        const int64_t left = (e_end - eb + stride - 1) / stride;
-        const int cnt = left < 32 ? (int)left : 32;
+    double s = 0.0;
 #pragma unroll 4
-        for (int j = 0; j < cnt; ++j) {
-            const int32_t vj = __shfl_sync(0xffffffffu, v_row, j);
-            const float aj = __shfl_sync(0xffffffffu, al, j);
-            const float asj = __shfl_sync(0xffffffffu, as, j);
-            const float *dr = D + (int64_t)vj * ld_d;
-            double p = 0.0;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const int c4 = lane + 32 * v;
-                if (c4 < d4) {
-                    const float4 x = ldz(dr, c4, d);
-                    p += ddot4(x, zu[v]);
-                    acc[v].x = fmaf(aj, x.x, acc[v].x);
-                    acc[v].y = fmaf(aj, x.y, acc[v].y);
-                    acc[v].z = fmaf(aj, x.z, acc[v].z);
-                    acc[v].w = fmaf(aj, x.w, acc[v].w);
-                }
-            }
-            dss += (double)asj * p;
-        }
+    for (int64_t e = e0 + tid; e < e1; e += T) {
+        const float2 x = edge[map[e]];
+        ent_out[e] = make_int2(idx[e], __float_as_int(x.x));
+        s += (double)x.y;
     }
-    return warp_sum_d(dss) - warp_sum_d(tss);
+    s = team_reduce<T>(s, OpAdd(), sh);
+    if (tid == 0) *ds_src = (float)s;
 }
 
-// backward, column side: one warp per node u keeps z_u in registers and walks the rows v that have u as an entry:
-//   HALO = 0: u is inner row `row0 + w`, the v are the inner prefix of its own row (symmetric block, self entry included);
-//   HALO = 1: u is halo position `halo0 + w`, the v are its halo-row CSR entries.
-//   dZ_u = sum_v alpha_vu D_v + ds_src[u] a_src (+ ds_dst[u] a_dst),  ds_src[u] = sum_v alpha_vu (D_v . z_u - t_v) slope_vu
-template <int NV, int HALO>
 __global__ void __launch_bounds__(256)
-k_gat_bwd_cols(const int64_t *__restrict__ ptr, const int32_t *__restrict__ idx, const int32_t *__restrict__ inner_cnt, int64_t u0, int64_t n_u,
-               const float *__restrict__ z_u_base, int64_t ld_z, const float *__restrict__ s_u, const float *__restrict__ s_dst,
-               const float *__restrict__ lse, const double *__restrict__ t_in, const float *__restrict__ ds_dst, int32_t d,
-               const float *__restrict__ D, int64_t ld_d, const float *__restrict__ a_src, const float *__restrict__ a_dst,
-               float *__restrict__ dz_base, float *__restrict__ ds_src)
+k_gat_cols(const int64_t *__restrict__ ptr, const int32_t *__restrict__ cnt, int64_t u0, int64_t n_u, const int32_t *__restrict__ long_u, int32_t n_long,
+           const int32_t *__restrict__ idx, const uint32_t *__restrict__ map, const float2 *__restrict__ edge, int2 *__restrict__ ent_out,
+           float *__restrict__ ds_src)
 {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    __shared__ double sh[8];
+    if ((int32_t)blockIdx.x < n_long) {
+        const int32_t u = long_u[blockIdx.x];
+        gat_col<256>(threadIdx.x, ptr[u], cnt ? ptr[u] + cnt[u] : ptr[u + 1], idx, map, edge, ent_out, ds_src + u, sh);
+        return;
+    }
+    const int64_t w = ((int64_t)(blockIdx.x - n_long) * 256 + threadIdx.x) / GAT_TEAM;
     if (w >= n_u) return;
-    const int64_t u = u0 + w;
-    const int d4 = (d + 3) >> 2;
-    float4 zu[NV], acc[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        zu[v] = c4 < d4 ? ldz(z_u_base + u * ld_z, c4, d) : make_float4(0.f, 0.f, 0.f, 0.f);
-        acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const int64_t e0 = ptr[u], e1 = HALO ? ptr[u + 1] : e0 + inner_cnt[u];
-    if (HALO && e1 - e0 > SAT_HROW_LONG) return;   // long halo rows: k_gat_bwd_cols_long, a thread block each
-    const float su = s_u[u];
-    const double dss = gat_cols_walk<NV>(idx, e0, e1, 1, su, s_dst, lse, t_in, D, ld_d, d, d4, lane, zu, acc);
-    const float dsd = HALO ? 0.f : ds_dst[u];
-    const float dssf = (float)dss;
-    float *o = dz_base + u * ld_z;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        if (c4 < d4) {
-            const int c = 4 * c4;
-            float4 r = acc[v];
-            r.x += dssf * a_src[c] + (HALO ? 0.f : dsd * a_dst[c]);
-            if (c + 1 < d) r.y += dssf * a_src[c + 1] + (HALO ? 0.f : dsd * a_dst[c + 1]);
-            if (c + 2 < d) r.z += dssf * a_src[c + 2] + (HALO ? 0.f : dsd * a_dst[c + 2]);
-            if (c + 3 < d) r.w += dssf * a_src[c + 3] + (HALO ? 0.f : dsd * a_dst[c + 3]);
-            if (c + 1 >= d) r.y = 0.f;
-            if (c + 2 >= d) r.z = 0.f;
-            if (c + 3 >= d) r.w = 0.f;
-            *reinterpret_cast<float4 *>(o + 4 * c4) = r;
-        }
-    }
-    if (lane == 0) ds_src[u] = dssf;
+    const int64_t u = u0 + w, e0 = ptr[u];
+    if (ptr[u + 1] - e0 > GAT_LONG) return;
+    gat_col<GAT_TEAM>(threadIdx.x & (GAT_TEAM - 1), e0, cnt ? e0 + cnt[u] : ptr[u + 1], idx, map, edge, ent_out, ds_src + u, sh);
 }
 
-// -------------------------------------------------------------------------------------
-// The same two sweeps over the SpMM's work items (rows cut into chunks of SAT_SPMM_CHUNK entries), one warp per item, so
-// that a hub row is walked by many warps; the per-item partial sums are added per row in item order by the combine kernels.
-// -------------------------------------------------------------------------------------
-template <int NV>
-__global__ void __launch_bounds__(256)
-k_gat_bwd_rows_items(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ lenc, const int32_t *__restrict__ item_row,
-                     const int32_t *__restrict__ first_item, int32_t item0, int32_t n_items, int32_t n, const float *__restrict__ z_in,
-                     const float *__restrict__ z_halo, int64_t ld_z, const float *__restrict__ s_in, const float *__restrict__ s_halo,
-                     const float *__restrict__ s_dst, const float *__restrict__ lse, int32_t d, const float *__restrict__ D, int64_t ld_d,
-                     double *__restrict__ part4)
+// mirror images: entry e = (r, c) of the inner block is entry rev[e] = (c, r); entry i of halo row j (node u, inner neighbour v) is the
+// entry (v, u) of v's local row.  Columns are ascending inside both parts of a row.
+__device__ __forceinline__ uint32_t gat_find(const int32_t *__restrict__ lenc, int64_t lo, int64_t hi, int32_t key)
 {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (lenc[mid] < key) lo = mid + 1;
+        else hi = mid;
+    }
+    return (uint32_t)lo;
+}
+__global__ void k_gat_rev(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ lenc, const int32_t *__restrict__ inner_cnt, int32_t n,
+                          uint32_t *__restrict__ rev, int32_t *__restrict__ is_long)
+{
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (w >= n_items) return;
-    const int32_t item = item0 + (int32_t)w;
-    const int32_t row = item_row[item];
-    const int d4 = (d + 3) >> 2;
-    float4 dv[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        dv[v] = c4 < d4 ? ldz(D + (int64_t)row * ld_d, c4, d) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r >= n) return;
+    const int64_t e0 = lrowptr[r], e1 = e0 + inner_cnt[r];
+    for (int64_t e = e0 + lane; e < e1; e += 32) {
+        const int32_t c = lenc[e];
+        rev[e] = gat_find(lenc, lrowptr[c], lrowptr[c] + inner_cnt[c], (int32_t)r);
     }
-    const int64_t re = lrowptr[row + 1];
-    const int64_t e0 = lrowptr[row] + (int64_t)(item - first_item[row]) * SAT_SPMM_CHUNK;
-    const int64_t e1 = e0 + SAT_SPMM_CHUNK < re ? e0 + SAT_SPMM_CHUNK : re;
-    const float sd = s_dst[row], l = lse[row];
-    // the lanes fetch the scalars of 32 entries at a time (one exponential per entry), then the warp walks those entries
-    // together; t_v and ds_dst are linear in the dot products D_v . z_u, so the lanes keep their shares and the warp is reduced
-    // once per item
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (int64_t eb = e0; eb < e1; eb += 32) {
-        const int64_t e = eb + lane;
-        int32_t c = 0;
-        float al = 0.f, as = 0.f;
-        if (e < e1) {
-            c = lenc[e];
-            const float pre = sd + (c < n ? s_in[c] : s_halo[c - n]);
-            const float slope = pre > 0.f ? 1.f : GAT_SLOPE;
-            al = expf(lrelu(pre) - l);
-            as = al * slope;
-            a0 += (double)al;
-            a3 += (double)al * (double)slope;
-        }
-        const int cnt = (e1 - eb) < 32 ? (int)(e1 - eb) : 32;
-#pragma unroll 4
-        for (int j = 0; j < cnt; ++j) {
-            const int32_t cj = __shfl_sync(0xffffffffu, c, j);
-            const float aj = __shfl_sync(0xffffffffu, al, j);
-            const float asj = __shfl_sync(0xffffffffu, as, j);
-            const float *src = cj < n ? z_in + (int64_t)cj * ld_z : z_halo + (int64_t)(cj - n) * ld_z;
-            double p = 0.0;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const int c4 = lane + 32 * v;
-                if (c4 < d4) p += ddot4(dv[v], ldz(src, c4, d));
-            }
-            a1 += (double)aj * p;
-            a2 += (double)asj * p;
-        }
-    }
-    a0 = warp_sum_d(a0);
-    a1 = warp_sum_d(a1);
-    a2 = warp_sum_d(a2);
-    a3 = warp_sum_d(a3);
-    if (lane == 0) {
-        double *o = part4 + 4 * w;
-        o[0] = a0;
-        o[1] = a1;
-        o[2] = a2;
-        o[3] = a3;
-    }
+    if (lane == 0) is_long[r] = lrowptr[r + 1] - e0 > GAT_LONG ? 1 : 0;
 }
-
-__global__ void k_gat_rows_combine(const int32_t *__restrict__ first_item, int32_t item0, int32_t row0, int32_t n_rows,
-                                   const double *__restrict__ part4, double *__restrict__ t_out, float *__restrict__ ds_dst)
+__global__ void k_gat_hmap(const int64_t *__restrict__ hrow_ptr, const int32_t *__restrict__ hrow_pos, const int64_t *__restrict__ lrowptr,
+                           const int32_t *__restrict__ lenc, const int32_t *__restrict__ inner_cnt, int32_t n, int64_t nb, uint32_t *__restrict__ hmap)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_rows) return;
-    const int32_t row = row0 + (int32_t)i;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (int32_t it = first_item[row]; it < first_item[row + 1]; ++it) {
-        const double *p = part4 + 4 * (int64_t)(it - item0);
-        a0 += p[0];
-        a1 += p[1];
-        a2 += p[2];
-        a3 += p[3];
-    }
-    t_out[row] = a1 / a0;
-    ds_dst[row] = (float)(a2 / a0 - (a1 / a0) * (a3 / a0));
-}
-
-// column side for the inner nodes: the item's entries that lie in the inner prefix of the row of u
-template <int NV>
-__global__ void __launch_bounds__(256)
-k_gat_bwd_cols_items(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ lenc, const int32_t *__restrict__ inner_cnt,
-                     const int32_t *__restrict__ item_row, const int32_t *__restrict__ first_item, int32_t item0, int32_t n_items,
-                     const float *__restrict__ z_in, int64_t ld_z, const float *__restrict__ s_in, const float *__restrict__ s_dst,
-                     const float *__restrict__ lse, const double *__restrict__ t_in, int32_t d, const float *__restrict__ D, int64_t ld_d,
-                     float *__restrict__ pdz, double *__restrict__ pdss)
-{
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (w >= n_items) return;
-    const int32_t item = item0 + (int32_t)w;
-    const int32_t u = item_row[item];
-    const int d4 = (d + 3) >> 2;
-    float4 zu[NV], acc[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        zu[v] = c4 < d4 ? ldz(z_in + (int64_t)u * ld_z, c4, d) : make_float4(0.f, 0.f, 0.f, 0.f);
-        acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j >= nb) return;
+    for (int64_t i = hrow_ptr[j] + lane; i < hrow_ptr[j + 1]; i += 32) {
+        const int32_t v = hrow_pos[i];
+        hmap[i] = gat_find(lenc, lrowptr[v] + inner_cnt[v], lrowptr[v + 1], (int32_t)(n + j));
     }
-    const int64_t rb = lrowptr[u], re = rb + inner_cnt[u];
-    const int64_t e0 = rb + (int64_t)(item - first_item[u]) * SAT_SPMM_CHUNK;
-    const int64_t e1 = e0 + SAT_SPMM_CHUNK < re ? e0 + SAT_SPMM_CHUNK : re;
-    const float su = s_in[u];
-    const double dss = gat_cols_walk<NV>(lenc, e0, e1, 1, su, s_dst, lse, t_in, D, ld_d, d, d4, lane, zu, acc);
-    float *o = pdz + w * ld_z;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        if (c4 < d4) *reinterpret_cast<float4 *>(o + 4 * c4) = acc[v];
-    }
-    if (lane == 0) pdss[w] = dss;
 }
-
-// dZ_u = sum of the item partials in item order + ds_src[u] a_src + ds_dst[u] a_dst; one thread per (row, float4 column)
-__global__ void k_gat_cols_combine(const int32_t *__restrict__ first_item, int32_t item0, int32_t row0, int32_t n_rows, int32_t d,
-                                   const float *__restrict__ pdz, int64_t ld_z, const double *__restrict__ pdss, const float *__restrict__ ds_dst,
-                                   const float *__restrict__ a_src, const float *__restrict__ a_dst, float *__restrict__ dz_base,
-                                   float *__restrict__ ds_src)
+__global__ void k_gat_long(const int32_t *__restrict__ is_long, const int64_t *__restrict__ off, int32_t n, int32_t *__restrict__ out)
 {
-    const int d4 = (d + 3) >> 2;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t i = sat_div(t, d4);
-    const int c4 = (int)(t - i * d4);
-    if (i >= n_rows) return;
-    const int32_t u = row0 + (int32_t)i;
-    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-    double dss = 0.0;
-    for (int32_t it = first_item[u]; it < first_item[u + 1]; ++it) {
-        const float4 x = *reinterpret_cast<const float4 *>(pdz + (int64_t)(it - item0) * ld_z + 4 * c4);
-        r.x += x.x;
-        r.y += x.y;
-        r.z += x.z;
-        r.w += x.w;
-        dss += pdss[it - item0];
-    }
-    const float s1 = (float)dss, s2 = ds_dst[u];
-    const int c = 4 * c4;
-    r.x += s1 * a_src[c] + s2 * a_dst[c];
-    r.y = c + 1 < d ? r.y + s1 * a_src[c + 1] + s2 * a_dst[c + 1] : 0.f;
-    r.z = c + 2 < d ? r.z + s1 * a_src[c + 2] + s2 * a_dst[c + 2] : 0.f;
-    r.w = c + 3 < d ? r.w + s1 * a_src[c + 3] + s2 * a_dst[c + 3] : 0.f;
-    *reinterpret_cast<float4 *>(dz_base + (int64_t)u * ld_z + 4 * c4) = r;
-    if (c4 == 0) ds_src[u] = s1;
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < n && is_long[r]) out[off[r]] = (int32_t)r;
 }
 
-// column side for the halo rows with more than SAT_HROW_LONG entries (hub nodes seen from another partition): one thread
-// block per row, its 8 warps taking the entries round-robin; the warps' partial sums are added in warp order.
-template <int NV>
-__global__ void __launch_bounds__(256)
-k_gat_bwd_cols_long(const int32_t *__restrict__ hlong, int32_t hlong0, const int64_t *__restrict__ ptr, const int32_t *__restrict__ idx,
-                    const float *__restrict__ z_halo, int64_t ld_z, const float *__restrict__ s_halo, const float *__restrict__ s_dst,
-                    const float *__restrict__ lse, const double *__restrict__ t_in, int32_t d, const float *__restrict__ D, int64_t ld_d,
-                    const float *__restrict__ a_src, float *__restrict__ dz_base, float *__restrict__ ds_src)
-{
-    __shared__ float4 red[8][NV][32];
-    __shared__ double red_s[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t u = hlong[hlong0 + blockIdx.x];
-    const int d4 = (d + 3) >> 2;
-    float4 zu[NV], acc[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        zu[v] = c4 < d4 ? ldz(z_halo + u * ld_z, c4, d) : make_float4(0.f, 0.f, 0.f, 0.f);
-        acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const int64_t e0 = ptr[u], e1 = ptr[u + 1];
-    const float su = s_halo[u];
-    const double dss = gat_cols_walk<NV>(idx, e0 + warp, e1, 8, su, s_dst, lse, t_in, D, ld_d, d, d4, lane, zu, acc);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) red[warp][v][lane] = acc[v];
-    if (lane == 0) red_s[warp] = dss;
-    __syncthreads();
-    if (warp != 0) return;
-    double tot = 0.0;
-    for (int q = 0; q < 8; ++q) tot += red_s[q];
-    const float s1 = (float)tot;
-    float *o = dz_base + u * ld_z;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int c4 = lane + 32 * v;
-        if (c4 < d4) {
-            float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int q = 0; q < 8; ++q) {
-                const float4 x = red[q][v][lane];
-                r.x += x.x;
-                r.y += x.y;
-                r.z += x.z;
-                r.w += x.w;
-            }
-            const int c = 4 * c4;
-            r.x += s1 * a_src[c];
-            r.y = c + 1 < d ? r.y + s1 * a_src[c + 1] : 0.f;
-            r.z = c + 2 < d ? r.z + s1 * a_src[c + 2] : 0.f;
-            r.w = c + 3 < d ? r.w + s1 * a_src[c + 3] : 0.f;
-            *reinterpret_cast<float4 *>(o + 4 * c4) = r;
-        }
-    }
-    if (lane == 0) ds_src[u] = s1;
-}
-
-// part[b][c] = sum over the rows r of block b, in order, of w[r] x[r][c]
+// part1[b][c] = sum over the rows r of block b of w1[r] x[r][c], and part2 with w2 where given: one pass over x for both.  tpr threads
+// (a power of two) walk a row with 128-bit accesses, four rows in flight per thread; the row groups of a block are added in order.
 #define GAT_WSUM_ROWS 256
 __global__ void __launch_bounds__(256)
-k_gat_wcolsum(const float *__restrict__ x, int64_t ld, int64_t rows, int32_t d, const float *__restrict__ wgt, float *__restrict__ part)
+k_gat_wcolsum(const float *__restrict__ x, int64_t ld, int64_t rows, int32_t d, int32_t tpr, const float *__restrict__ w1, const float *__restrict__ w2,
+              float *__restrict__ part1, float *__restrict__ part2)
 {
-    const int64_t r0 = (int64_t)blockIdx.x * GAT_WSUM_ROWS;
-    const int64_t r1 = r0 + GAT_WSUM_ROWS < rows ? r0 + GAT_WSUM_ROWS : rows;
-    for (int c = threadIdx.x; c < d; c += 256) {
-        float s = 0.f;
-        for (int64_t r = r0; r < r1; ++r) s = fmaf(wgt[r], x[r * ld + c], s);
-        part[(int64_t)blockIdx.x * d + c] = s;
+    __shared__ float4 red[2][256];
+    const int c4 = threadIdx.x % tpr, rg = threadIdx.x / tpr, n_rg = 256 / tpr, d4 = (d + 3) >> 2;
+    const int64_t r0 = (int64_t)blockIdx.x * GAT_WSUM_ROWS, r1 = r0 + GAT_WSUM_ROWS < rows ? r0 + GAT_WSUM_ROWS : rows;
+    float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f), s2 = s1;
+    if (c4 < d4) {
+        for (int64_t r = r0 + rg; r < r1; r += 4 * n_rg) {
+            float4 v[4];
+            float a[4], b[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t rr = r + (int64_t)u * n_rg;
+                const bool ok = rr < r1;
+                v[u] = ok ? __ldg(reinterpret_cast<const float4 *>(x + rr * ld) + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                a[u] = ok ? __ldg(w1 + rr) : 0.f;
+                b[u] = ok && w2 ? __ldg(w2 + rr) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                s1.x = fmaf(a[u], v[u].x, s1.x); s1.y = fmaf(a[u], v[u].y, s1.y); s1.z = fmaf(a[u], v[u].z, s1.z); s1.w = fmaf(a[u], v[u].w, s1.w);
+                s2.x = fmaf(b[u], v[u].x, s2.x); s2.y = fmaf(b[u], v[u].y, s2.y); s2.z = fmaf(b[u], v[u].z, s2.z); s2.w = fmaf(b[u], v[u].w, s2.w);
+            }
+        }
+    }
+    red[0][threadIdx.x] = s1;
+    red[1][threadIdx.x] = s2;
+    __syncthreads();
+    if (rg < 2 && rg < n_rg && c4 < d4) {
+        for (int k = rg; k < (w2 ? 2 : 1); k += n_rg < 2 ? 1 : 2) {
+            float4 t = red[k][c4];
+            for (int g = 1; g < n_rg; ++g) {
+                const float4 y = red[k][g * tpr + c4];
+                t.x += y.x; t.y += y.y; t.z += y.z; t.w += y.w;
+            }
+            float *o = (k ? part2 : part1) + (int64_t)blockIdx.x * d + 4 * c4;
+            o[0] = t.x;
+            if (4 * c4 + 1 < d) o[1] = t.y;
+            if (4 * c4 + 2 < d) o[2] = t.z;
+            if (4 * c4 + 3 < d) o[3] = t.w;
+        }
     }
 }
 
@@ -612,27 +439,75 @@ static sat_status gat_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const
     return sat_gemm_tn(ctx, rows, m, n, A, lda, B, ldb, nullptr, 0, C, n, nullptr, accumulate);
 }
 
-// out[c] (+)= sum_r w[r] x[r][c]
-static sat_status gat_wcolsum(sat_ctx *ctx, const float *x, int32_t ld, int64_t rows, int32_t d, const float *w, float *out, int accumulate)
+// out1[c] (+)= sum_r w1[r] x[r][c], and the same with w2 / out2 where given
+static sat_status gat_wcolsum(sat_ctx *ctx, const float *x, int32_t ld, int64_t rows, int32_t d, const float *w1, float *out1, const float *w2,
+                              float *out2, int accumulate)
 {
     if (rows == 0) {
-        if (!accumulate) SAT_CUDA(ctx, cudaMemsetAsync(out, 0, (size_t)d * sizeof(float), ctx->stream));
+        if (!accumulate) {
+            SAT_CUDA(ctx, cudaMemsetAsync(out1, 0, (size_t)d * sizeof(float), ctx->stream));
+            if (out2) SAT_CUDA(ctx, cudaMemsetAsync(out2, 0, (size_t)d * sizeof(float), ctx->stream));
+        }
         return SAT_OK;
     }
     const int64_t blocks = cdiv64(rows, GAT_WSUM_ROWS);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)blocks * d * sizeof(float)));
-    k_gat_wcolsum<<<(unsigned)blocks, 256, 0, ctx->stream>>>(x, ld, rows, d, w, (float *)ctx->buf_colsum.p);
+    SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)2 * blocks * d * sizeof(float)));
+    float *p1 = (float *)ctx->buf_colsum.p, *p2 = w2 ? p1 + (size_t)blocks * d : nullptr;
+    int tpr = 1;
+    while (tpr < (d + 3) / 4) tpr <<= 1;   // d <= 1024: at most 256
+    k_gat_wcolsum<<<(unsigned)blocks, 256, 0, ctx->stream>>>(x, ld, rows, d, tpr, w1, w2, p1, p2);
     SAT_LAUNCHED(ctx);
-    return sat_splitk_reduce(ctx, (const float *)ctx->buf_colsum.p, d, (int32_t)blocks, accumulate, out, d, d);
+    return sat_splitk_reduce(ctx, p1, d, (int32_t)blocks, accumulate, out1, d, d, p2, d, out2);
 }
 
-#define GAT_DISPATCH(NVV, CALL)            \
-    do {                                   \
-        if ((NVV) <= 1) { CALL(1); }       \
-        else if ((NVV) <= 2) { CALL(2); }  \
-        else if ((NVV) <= 4) { CALL(4); }  \
-        else { CALL(8); }                  \
-    } while (0)
+// what the attention layer needs to know about the partitioning: the mirror image of every inner entry and of every halo-row entry, and
+// the rows that get a thread block (built on first use, freed with the partition)
+static sat_status gat_prepare(sat_ctx *ctx)
+{
+    if (ctx->gat_rev) return SAT_OK;
+    const int32_t n = ctx->n, M = ctx->M;
+    const int64_t lnnz = ctx->nnz + n, nb = ctx->nb;
+    if (lnnz >= ((int64_t)1 << 32)) return sat_fail(ctx, SAT_EINVAL, "sat_gat_fwd: more than 2^32 entries");
+    uint32_t *rev = nullptr, *hmap = nullptr;
+    int32_t *flag = nullptr, *rows = nullptr;
+    int64_t *off = nullptr;
+    std::vector<int64_t> h((size_t)M + 1, 0);
+    sat_status rc = SAT_OK;
+    cudaError_t e = cudaMalloc((void **)&rev, (size_t)lnnz * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&hmap, (size_t)(ctx->nnz_cut > 0 ? ctx->nnz_cut : 1) * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&flag, (size_t)n * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&off, ((size_t)n + 1) * sizeof(int64_t));
+    if (e == cudaSuccess) {
+        k_gat_rev<<<(unsigned)cdiv64((int64_t)n * 32, 256), 256, 0, ctx->stream>>>(ctx->lrowptr, ctx->lenc, ctx->inner_cnt, n, rev, flag);
+        if (nb > 0)
+            k_gat_hmap<<<(unsigned)cdiv64(nb * 32, 256), 256, 0, ctx->stream>>>(ctx->hrow_ptr, ctx->hrow_pos, ctx->lrowptr, ctx->lenc, ctx->inner_cnt, n, nb, hmap);
+        ctx->launches += nb > 0 ? 2 : 1;
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) rc = sat_scan_i32(ctx, flag, n, off);
+    for (int m = 0; e == cudaSuccess && rc == SAT_OK && m <= M; ++m)
+        e = cudaMemcpyAsync(&h[m], off + ctx->h_inner_off[m], sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess && rc == SAT_OK) e = cudaStreamSynchronize(ctx->stream);
+    if (e == cudaSuccess && rc == SAT_OK) e = cudaMalloc((void **)&rows, (size_t)(h[M] > 0 ? h[M] : 1) * sizeof(int32_t));
+    if (e == cudaSuccess && rc == SAT_OK) {
+        k_gat_long<<<(unsigned)cdiv64(n, 256), 256, 0, ctx->stream>>>(flag, off, n, rows);
+        ctx->launches++;
+        e = cudaStreamSynchronize(ctx->stream);
+    }
+    cudaFree(flag);
+    cudaFree(off);
+    if (e != cudaSuccess || rc != SAT_OK) {
+        cudaFree(rev);
+        cudaFree(hmap);
+        cudaFree(rows);
+        return rc != SAT_OK ? rc : sat_check_cuda(ctx, e, "mirrored entries of the attention layer");
+    }
+    ctx->gat_rev = rev;
+    ctx->gat_hmap = hmap;
+    ctx->gat_long = rows;
+    ctx->h_gat_long_off = h;
+    return SAT_OK;
+}
 
 extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int32_t d_in, int32_t d_out, const float *h_in, int32_t ld_in,
                                   const float *h_halo, int32_t ld_halo, const float *W, const float *a_src, const float *a_dst,
@@ -655,7 +530,8 @@ extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int
         // columns of the z rows, which no kernel writes, read as zero
         SAT_TRY(sat_ensure(ctx, G.z_in, (size_t)(n > 0 ? n : 1) * ld_z * sizeof(float)));
         SAT_TRY(sat_ensure(ctx, G.z_halo, (size_t)(nb > 0 ? nb : 1) * ld_z * sizeof(float)));
-        SAT_TRY(sat_ensure(ctx, G.scal, (size_t)(3 * (n > 0 ? n : 1) + (nb > 0 ? nb : 1)) * sizeof(float)));
+        SAT_TRY(sat_ensure(ctx, G.scal, (size_t)(2 * (n > 0 ? n : 1) + (nb > 0 ? nb : 1)) * sizeof(float)));
+        SAT_TRY(sat_ensure(ctx, G.ent, (size_t)(ctx->nnz + n) * sizeof(int2)));
         SAT_CUDA(ctx, cudaMemsetAsync(G.z_in.p, 0, G.z_in.bytes, ctx->stream));
         SAT_CUDA(ctx, cudaMemsetAsync(G.z_halo.p, 0, G.z_halo.bytes, ctx->stream));
         G.d_out = d_out;
@@ -663,7 +539,8 @@ extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int
     }
     G.relu = act == SAT_ACT_RELU;
     float *z_in = (float *)G.z_in.p, *z_halo = (float *)G.z_halo.p;
-    float *s_in = (float *)G.scal.p, *s_dst = s_in + n, *lse = s_dst + n, *s_halo = lse + n;
+    float *s_in = (float *)G.scal.p, *s_dst = s_in + n, *s_halo = s_dst + n;
+    SAT_TRY(gat_prepare(ctx));
     SAT_TRY(gat_nn(ctx, v.n_rows, d_out, d_in, h_in, ld_in, W, z_in + (int64_t)v.row0 * ld_z, ld_z));
     SAT_TRY(gat_nn(ctx, v.n_halo, d_out, d_in, h_halo, ld_halo, W, z_halo + v.halo0 * ld_z, ld_z));
     ProfScope prof(ctx, SATK_GAT, 0.0, 0.0);
@@ -678,29 +555,14 @@ extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int
         SAT_LAUNCHED(ctx);
     }
     if (v.n_rows > 0) {
-        const int nv = ((d_out + 3) / 4 + 31) / 32;
-        float *partial = nullptr;
-        if (v.n_mitems > 0) {
-            SAT_TRY(sat_ensure(ctx, ctx->buf_partial, (size_t)v.n_mitems * ld_z * sizeof(float)));
-            partial = (float *)ctx->buf_partial.p;
-        }
-        k_gat_lse<<<(unsigned)cdiv64((int64_t)v.n_rows * 32, 256), 256, 0, ctx->stream>>>(ctx->lrowptr, ctx->lenc, ctx->n, v.row0, v.n_rows, s_in, s_halo,
-                                                                                        s_dst, lse);
+        const int64_t l0 = ctx->h_gat_long_off[v.p0], n_long = ctx->h_gat_long_off[v.p1] - l0;
+        k_gat_alpha<<<(unsigned)(n_long + cdiv64((int64_t)v.n_rows * GAT_TEAM, 256)), 256, 0, ctx->stream>>>(
+            ctx->lrowptr, ctx->lenc, ctx->n, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, s_in, s_halo, s_dst, (int2 *)G.ent.p);
         SAT_LAUNCHED(ctx);
-        const unsigned grid = (unsigned)cdiv64((int64_t)v.n_items * 32, 256);
-        float *out_base = h_out - (int64_t)v.row0 * ld_out;
-#define CALL(NV)                                                                                                                                    \
-    k_gat_fwd_items<NV><<<grid, 256, 0, ctx->stream>>>(ctx->lrowptr, ctx->lenc, ctx->item_row, ctx->first_item, ctx->item_mslot, v.item0, v.n_items,    \
-                                                       v.mitem0, ctx->n, z_in, z_halo, ld_z, s_in, s_halo, s_dst, lse, d_out, bias, G.relu, out_base, \
-                                                       ld_out, partial)
-        GAT_DISPATCH(nv, CALL);
-#undef CALL
-        SAT_LAUNCHED(ctx);
-        if (v.n_mrows > 0) {
-            k_gat_fwd_fixup<<<(unsigned)cdiv64((int64_t)v.n_mrows * ((d_out + 3) / 4), 256), 256, 0, ctx->stream>>>(
-                ctx->mrows, v.mrow0, v.n_mrows, ctx->first_item, ctx->item_mslot, v.mitem0, d_out, partial, ld_z, bias, G.relu, out_base, ld_out);
-            SAT_LAUNCHED(ctx);
-        }
+        SpmmEpilogue ep;
+        ep.bias = bias;
+        ep.relu = G.relu;
+        SAT_TRY(sat_spmm_entries(ctx, v, 0, d_out, (const int2 *)G.ent.p, z_in, ld_z, z_halo, ld_z, h_out - (int64_t)v.row0 * ld_out, ld_out, ep));
     }
     for (int m = (part == SAT_ALL_PARTS ? 0 : part); m < (part == SAT_ALL_PARTS ? ctx->M : part + 1); ++m) G.valid[m] = 1;
     return SAT_OK;
@@ -716,7 +578,7 @@ extern "C" sat_status sat_gat_scores(sat_ctx *ctx, int32_t layer, float *s_src_i
     for (int m = 0; m < ctx->M; ++m)
         if (!G.valid[m]) return sat_fail(ctx, SAT_ESTATE, "sat_gat_scores: sat_gat_fwd has not run for partition %d of layer %d", m, layer);
     const int64_t n = ctx->n, nb = ctx->nb;
-    const float *s_in = (const float *)G.scal.p, *s_dst = s_in + n, *s_halo = s_dst + 2 * n;
+    const float *s_in = (const float *)G.scal.p, *s_dst = s_in + n, *s_halo = s_dst + n;
     if (s_src_inner_host) SAT_CUDA(ctx, cudaMemcpyAsync(s_src_inner_host, s_in, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     if (s_dst_host) SAT_CUDA(ctx, cudaMemcpyAsync(s_dst_host, s_dst, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     if (s_src_halo_host && nb > 0) SAT_CUDA(ctx, cudaMemcpyAsync(s_src_halo_host, s_halo, (size_t)nb * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
@@ -745,83 +607,78 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
         return sat_fail(ctx, SAT_EINVAL, "sat_gat_bwd: null / misaligned g_out / h_in / h_out or bad leading dimension");
     if (v.n_halo > 0 && (!h_halo || !ok_ld(ld_halo, d_in) || !aligned16(h_halo))) return sat_fail(ctx, SAT_EINVAL, "sat_gat_bwd: null / misaligned h_halo");
     if (g_in && v.n_rows > 0 && (!ok_ld(ld_gin, d_in) || !aligned16(g_in))) return sat_fail(ctx, SAT_EINVAL, "sat_gat_bwd: misaligned g_in or bad ld_gin");
-    const int64_t n = ctx->n, nb = ctx->nb;
+    const int64_t n = ctx->n;
     float *z_in = (float *)G.z_in.p, *z_halo = (float *)G.z_halo.p;
-    float *s_in = (float *)G.scal.p, *s_dst = s_in + n, *lse = s_dst + n, *s_halo = lse + n;
-    // scratch of the call: D, dZ (inner rows of the selection, halo rows of the selection), t, ds_dst, ds_src
-    const size_t f_rows = (size_t)(v.n_rows > 0 ? v.n_rows : 1), f_halo = (size_t)(v.n_halo > 0 ? v.n_halo : 1);
-    const size_t t_floats = (2 * f_rows + 3) & ~(size_t)3;                  // the doubles first, then 16-byte aligned rows
-    SAT_TRY(sat_ensure(ctx, ctx->buf_gat, (t_floats + (2 * f_rows + f_halo) * ld_z + 2 * f_rows + f_halo + 64) * sizeof(float)));
-    double *t = (double *)ctx->buf_gat.p;
-    float *D = (float *)ctx->buf_gat.p + t_floats, *dz_in = D + f_rows * ld_z, *dz_halo = dz_in + f_rows * ld_z;
+    float *s_in = (float *)G.scal.p, *s_dst = s_in + n, *s_halo = s_dst + n;
+    // scratch of the call, by row / halo position / entry of the selection: dot products (then alpha and dpre), entries of the inner and
+    // of the halo column side, D, dZ, ds_dst, ds_src
+    const int64_t ent0 = ctx->h_lnnz_off[v.p0], cut0 = ctx->h_hrow_off[v.p0];
+    const size_t f_rows = (size_t)(v.n_rows > 0 ? v.n_rows : 1), f_halo = (size_t)(v.n_halo > 0 ? v.n_halo : 1), f_ent = (size_t)v.lnnz + 2,
+                 f_cut = (size_t)v.hnnz + 2;
+    SAT_TRY(sat_ensure(ctx, ctx->buf_gat_items, (2 * f_ent + f_cut) * sizeof(double) + 32));
+    double *dots = (double *)ctx->buf_gat_items.p;
+    int2 *ent_in = (int2 *)(dots + f_ent), *ent_halo = ent_in + f_ent;
+    SAT_TRY(sat_ensure(ctx, ctx->buf_gat, ((2 * f_rows + f_halo) * ld_z + 2 * f_rows + f_halo + 64) * sizeof(float)));
+    float *D = (float *)ctx->buf_gat.p, *dz_in = D + f_rows * ld_z, *dz_halo = dz_in + f_rows * ld_z;
     float *ds_dst = dz_halo + f_halo * ld_z, *ds_in = ds_dst + f_rows, *ds_halo = ds_in + f_rows;
-    // virtual bases indexed by partition-major row / global halo position
+    // virtual bases indexed by partition-major row / global halo position / entry
     const float *Db = D - (int64_t)v.row0 * ld_z;
     float *dz_in_b = dz_in - (int64_t)v.row0 * ld_z, *dz_halo_b = dz_halo - v.halo0 * ld_z;
-    double *t_b = t - v.row0;
     float *ds_dst_b = ds_dst - v.row0, *ds_in_b = ds_in - v.row0, *ds_halo_b = ds_halo - v.halo0;
-    const int nv = ((d_out + 3) / 4 + 31) / 32;
+    double *dots_b = dots - ent0;
+    int2 *ent_in_b = ent_in - ent0, *ent_halo_b = ent_halo - cut0;
+    const int32_t d4 = (d_out + 3) / 4;
     if (v.n_rows > 0) {
-        SAT_CUDA(ctx, cudaMemsetAsync(D, 0, f_rows * ld_z * sizeof(float), ctx->stream));   // padding columns of D read as zero
-        {
-            ProfScope prof(ctx, SATK_GAT, 0.0, 0.0);
-            k_gat_dmask<<<(unsigned)cdiv64((int64_t)v.n_rows * d_out, 256), 256, 0, ctx->stream>>>(g_out, ld_g, G.relu ? h_out : nullptr, ld_out, v.n_rows, d_out,
-                                                                                                 D, ld_z);
-            SAT_LAUNCHED(ctx);
-        }
-        SAT_TRY(sat_mask_rows(ctx, D, ld_z, v.n_rows, d_out, nullptr, 0, nullptr, 0, g_b, accumulate));
-        // per-item partial sums: 4 doubles for the row side, a dZ row and a double for the column side
-        const size_t n_it = (size_t)v.n_items;
-        SAT_TRY(sat_ensure(ctx, ctx->buf_gat_items, (5 * n_it * 2 + n_it * ld_z + 64) * sizeof(float)));
-        double *part4 = (double *)ctx->buf_gat_items.p, *pdss = part4 + 4 * n_it;
-        float *pdz = (float *)(pdss + n_it + (n_it & 1));   // 16-byte aligned rows after an even number of doubles
+        SAT_TRY(sat_mask_rows(ctx, g_out, ld_g, v.n_rows, d_out, nullptr, 0, D, ld_z, g_b, accumulate, G.relu ? h_out : nullptr, ld_out));
         ProfScope prof(ctx, SATK_GAT, 0.0, 0.0);
-        const unsigned grid = (unsigned)cdiv64((int64_t)v.n_items * 32, 256);
-#define CALL(NV)                                                                                                                                 \
-    k_gat_bwd_rows_items<NV><<<grid, 256, 0, ctx->stream>>>(ctx->lrowptr, ctx->lenc, ctx->item_row, ctx->first_item, v.item0, v.n_items, ctx->n, z_in, \
-                                                            z_halo, ld_z, s_in, s_halo, s_dst, lse, d_out, Db, ld_z, part4)
-        GAT_DISPATCH(nv, CALL);
+        const int4 *items = nullptr;
+        int64_t n_items = 0;
+        SAT_TRY(sat_spmm_items(ctx, v, 0, d_out, &items, &n_items));
+#define CALL(GG, NV)                                                                                                                            \
+    k_gat_dots<GG, NV><<<(unsigned)cdiv64(n_items * GG, 256), 256, 0, ctx->stream>>>(items, (int32_t)n_items, ctx->lenc, ctx->n, d4, z_in, z_halo, \
+                                                                                     (uint32_t)(ld_z / 4), Db, dots_b)
+        if (d4 <= 8) CALL(8, 1);
+        else if (d4 <= 16) CALL(16, 1);
+        else if (d4 <= 32) CALL(32, 1);
+        else if (d4 <= 64) CALL(32, 2);
+        else if (d4 <= 128) CALL(32, 4);
+        else CALL(32, 8);
 #undef CALL
         SAT_LAUNCHED(ctx);
-        k_gat_rows_combine<<<(unsigned)cdiv64(v.n_rows, 256), 256, 0, ctx->stream>>>(ctx->first_item, v.item0, v.row0, v.n_rows, part4, t_b, ds_dst_b);
+        const int64_t l0 = ctx->h_gat_long_off[v.p0], n_long = ctx->h_gat_long_off[v.p1] - l0;
+        const unsigned grid = (unsigned)(n_long + cdiv64((int64_t)v.n_rows * GAT_TEAM, 256));
+        k_gat_rows<<<grid, 256, 0, ctx->stream>>>(ctx->lrowptr, (const int2 *)G.ent.p, ctx->n, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, s_in,
+                                                  s_halo, s_dst, dots_b, ds_dst_b);
         SAT_LAUNCHED(ctx);
-#define CALL(NV)                                                                                                                                  \
-    k_gat_bwd_cols_items<NV><<<grid, 256, 0, ctx->stream>>>(ctx->lrowptr, ctx->lenc, ctx->inner_cnt, ctx->item_row, ctx->first_item, v.item0, v.n_items, \
-                                                            z_in, ld_z, s_in, s_dst, lse, t_b, d_out, Db, ld_z, pdz, pdss)
-        GAT_DISPATCH(nv, CALL);
-#undef CALL
+        k_gat_cols<<<grid, 256, 0, ctx->stream>>>(ctx->lrowptr, ctx->inner_cnt, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, ctx->lenc,
+                                                  ctx->gat_rev, (const float2 *)dots_b, ent_in_b, ds_in_b);
         SAT_LAUNCHED(ctx);
-        k_gat_cols_combine<<<(unsigned)cdiv64((int64_t)v.n_rows * ((d_out + 3) / 4), 256), 256, 0, ctx->stream>>>(
-            ctx->first_item, v.item0, v.row0, v.n_rows, d_out, pdz, ld_z, pdss, ds_dst_b, a_src, a_dst, dz_in_b, ds_in_b);
-        SAT_LAUNCHED(ctx);
+        SpmmEpilogue ep;
+        ep.s1 = ds_in_b;
+        ep.v1 = a_src;
+        ep.s2 = ds_dst_b;
+        ep.v2 = a_dst;
+        SAT_TRY(sat_spmm_entries(ctx, v, 1, d_out, ent_in_b, Db, ld_z, nullptr, 0, dz_in_b, ld_z, ep));
     } else if (!accumulate) {
         SAT_CUDA(ctx, cudaMemsetAsync(g_b, 0, (size_t)d_out * sizeof(float), ctx->stream));
     }
     if (v.n_halo > 0 && v.n_rows > 0) {
         ProfScope prof(ctx, SATK_GAT, 0.0, 0.0);
-        const unsigned grid = (unsigned)cdiv64(v.n_halo * 32, 256);
-#define CALL(NV)                                                                                                                                   \
-    k_gat_bwd_cols<NV, 1><<<grid, 256, 0, ctx->stream>>>(ctx->hrow_ptr, ctx->hrow_pos, nullptr, v.halo0, v.n_halo, z_halo, ld_z, s_halo, s_dst, lse, \
-                                                         t_b, nullptr, d_out, Db, ld_z, a_src, a_dst, dz_halo_b, ds_halo_b)
-        GAT_DISPATCH(nv, CALL);
-#undef CALL
+        k_gat_cols<<<(unsigned)(v.n_hlong + cdiv64(v.n_halo * GAT_TEAM, 256)), 256, 0, ctx->stream>>>(
+            ctx->hrow_ptr, nullptr, v.halo0, v.n_halo, ctx->hlong ? ctx->hlong + v.hlong0 : nullptr, v.n_hlong, ctx->hrow_pos, ctx->gat_hmap,
+            (const float2 *)dots_b, ent_halo_b, ds_halo_b);
         SAT_LAUNCHED(ctx);
-        if (v.n_hlong > 0) {
-#define CALL(NV)                                                                                                                                  \
-    k_gat_bwd_cols_long<NV><<<(unsigned)v.n_hlong, 256, 0, ctx->stream>>>(ctx->hlong, v.hlong0, ctx->hrow_ptr, ctx->hrow_pos, z_halo, ld_z, s_halo, s_dst, \
-                                                                          lse, t_b, d_out, Db, ld_z, a_src, dz_halo_b, ds_halo_b)
-            GAT_DISPATCH(nv, CALL);
-#undef CALL
-            SAT_LAUNCHED(ctx);
-        }
+        SpmmEpilogue ep;
+        ep.s1 = ds_halo_b;
+        ep.v1 = a_src;
+        SAT_TRY(sat_spmm_entries(ctx, v, 3, d_out, ent_halo_b, Db, ld_z, nullptr, 0, dz_halo_b, ld_z, ep));
     }
     const int64_t halo_rows = v.n_rows > 0 ? v.n_halo : 0;
     // parameter gradients
     SAT_TRY(gat_tn(ctx, v.n_rows, d_in, d_out, h_in, ld_in, dz_in, ld_z, g_W, accumulate));
     if (halo_rows > 0) SAT_TRY(gat_tn(ctx, halo_rows, d_in, d_out, h_halo, ld_halo, dz_halo, ld_z, g_W, 1));
-    SAT_TRY(gat_wcolsum(ctx, z_in + (int64_t)v.row0 * ld_z, ld_z, v.n_rows, d_out, ds_in, g_a_src, accumulate));
-    if (halo_rows > 0) SAT_TRY(gat_wcolsum(ctx, z_halo + v.halo0 * ld_z, ld_z, halo_rows, d_out, ds_halo, g_a_src, 1));
-    SAT_TRY(gat_wcolsum(ctx, z_in + (int64_t)v.row0 * ld_z, ld_z, v.n_rows, d_out, ds_dst, g_a_dst, accumulate));
+    SAT_TRY(gat_wcolsum(ctx, z_in + (int64_t)v.row0 * ld_z, ld_z, v.n_rows, d_out, ds_in, g_a_src, ds_dst, g_a_dst, accumulate));
+    if (halo_rows > 0) SAT_TRY(gat_wcolsum(ctx, z_halo + v.halo0 * ld_z, ld_z, halo_rows, d_out, ds_halo, g_a_src, nullptr, nullptr, 1));
     // input gradient of the inner rows
     if (g_in && v.n_rows > 0) SAT_TRY(gat_nt(ctx, v.n_rows, d_in, d_out, dz_in, ld_z, W, g_in, ld_gin));
     return SAT_OK;

@@ -904,7 +904,8 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
 #define MASK_ROWS_PER_BLOCK 256
 __global__ void __launch_bounds__(256)
 k_mask_rows(const float *__restrict__ src, int64_t ld, int64_t rows, int32_t d, int32_t tpr, const uint32_t *__restrict__ mask,
-            int32_t mask_words, float *__restrict__ dst, int64_t ld_dst, float *__restrict__ colsum_part)
+            int32_t mask_words, const float *__restrict__ act, int64_t ld_act, int act_vec, float *__restrict__ dst, int64_t ld_dst,
+            float *__restrict__ colsum_part)
 {
     __shared__ float4 red[256];
     const int c4 = threadIdx.x % tpr, rg = threadIdx.x / tpr, n_rg = 256 / tpr;
@@ -927,6 +928,18 @@ k_mask_rows(const float *__restrict__ src, int64_t ld, int64_t rows, int32_t d, 
                     if (rr < r1) {
                         x[u] = __ldg(reinterpret_cast<const float4 *>(src + rr * ld) + c);
                         if (mask) w[u] = __ldg(mask + rr * mask_words + (c >> 3)) >> ((c & 7) * 4);
+                        if (act) {
+                            const float *ar = act + rr * ld_act + 4 * c;
+                            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (act_vec) a = __ldg(reinterpret_cast<const float4 *>(ar));
+                            else {
+                                a.x = ar[0];
+                                if (4 * c + 1 < d) a.y = ar[1];
+                                if (4 * c + 2 < d) a.z = ar[2];
+                                if (4 * c + 3 < d) a.w = ar[3];
+                            }
+                            w[u] = (a.x > 0.f ? 1u : 0u) | (a.y > 0.f ? 2u : 0u) | (a.z > 0.f ? 4u : 0u) | (a.w > 0.f ? 8u : 0u);
+                        }
                     }
                 }
 #pragma unroll
@@ -1047,7 +1060,7 @@ bool sat_use_tc(int32_t n, int32_t k)
 }
 
 sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t rows, int32_t d, const uint32_t *mask, int32_t mask_words,
-                         float *dst, int32_t ld_dst, float *colsum, int accumulate)
+                         float *dst, int32_t ld_dst, float *colsum, int accumulate, const float *act, int32_t ld_act)
 {
     if (rows == 0 || d == 0) return SAT_OK;
     if (!dst && !colsum) return SAT_OK;
@@ -1060,7 +1073,8 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
     }
     int tpr = 1;
     while (tpr < (d + 3) / 4 && tpr < 256) tpr <<= 1;
-    k_mask_rows<<<(unsigned)blocks, 256, 0, ctx->stream>>>(src, ld, rows, d, tpr, mask, mask_words, dst, ld_dst, part);
+    k_mask_rows<<<(unsigned)blocks, 256, 0, ctx->stream>>>(src, ld, rows, d, tpr, mask, mask_words, act, ld_act, aligned16(act) && !(ld_act & 3),
+                                                            dst, ld_dst, part);
     SAT_LAUNCHED(ctx);
     if (colsum) SAT_TRY(sat_splitk_reduce(ctx, part, d, (int32_t)blocks, accumulate, colsum, d, d));
     return SAT_OK;

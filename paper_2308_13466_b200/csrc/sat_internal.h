@@ -16,8 +16,7 @@
 
 #define SAT_MAX_LAYERS 16
 #define SAT_MAX_PARTS 4096
-#define SAT_SPMM_CHUNK 256 /* edges per work item of the attention layer */
-#define SAT_HROW_LONG 256  /* halo rows with more entries than this get a thread block in the attention layer's backward */
+#define SAT_HROW_LONG 256  /* rows and halo rows with more entries than this get a thread block in the attention layer */
 
 // Debug build (-DSAT_DEBUG_BOUNDS, libsat_b200_dbg.so): every index the graph kernels load from an index array (column ids,
 // row lists, cache slots) is checked against the extent of the matrix it addresses; an index outside it raises bit 4 of
@@ -98,9 +97,9 @@ struct GradHist {
 };
 
 // Saved forward state of a graph-attention layer: z = h W for all inner rows and halo positions of the graph, the attention
-// scores s_src (inner, halo), s_dst and the log-sum-exp of every inner row (scal = [s_in | s_dst | lse | s_halo]).
+// scores s_src (inner, halo), s_dst (scal = [s_in | s_dst | s_halo]) and the softmax weights as entries {column, alpha} of the local CSR.
 struct GatState {
-    DevBuf z_in, z_halo, scal;
+    DevBuf z_in, z_halo, scal, ent;
     int32_t d_out = 0;
     int relu = 0;
     std::vector<uint8_t> valid;
@@ -193,13 +192,11 @@ struct sat_ctx {
     int32_t n_hlong = 0;
     std::vector<int32_t> h_hlong_off;
     int32_t *halo_tile_order = nullptr;  // [ceil(n_halo / 128)] tiles of 128 halo rows ordered by the cache slot of their first row (built on first use)
-    // work items of the attention layer (rows cut into chunks of SAT_SPMM_CHUNK edges)
-    int32_t *first_item = nullptr; // [n+1]
-    int32_t *item_row = nullptr;   // [n_items]
-    int32_t *item_mslot = nullptr; // [n_items] index of the partial-sum row for items of multi-chunk rows, else -1
-    int32_t *mrows = nullptr;      // [n_mrows] rows with more than one chunk
-    int32_t n_items = 0, n_mrows = 0, n_mitems = 0;
-    std::vector<int32_t> h_inner_off, h_push_off, h_item_off, h_mrow_off, h_mitem_off;
+    uint32_t *gat_rev = nullptr;   // [nnz+n] (attention layer, built on first use) mirror image of every inner entry
+    uint32_t *gat_hmap = nullptr;  // [nnz_cut] local-CSR entry of every halo-row entry
+    int32_t *gat_long = nullptr;   // rows of more than SAT_HROW_LONG entries
+    std::vector<int64_t> h_gat_long_off;
+    std::vector<int32_t> h_inner_off, h_push_off;
     std::vector<int64_t> h_halo_off, h_lnnz_off, h_hrow_off;
 
     // ---- cache ----
@@ -318,9 +315,6 @@ sat_status sat_codec_roundtrip(sat_ctx *ctx, float *x, int32_t ld, int64_t rows,
 struct PartView {
     int32_t row0, n_rows;     // partition-major rows
     int64_t halo0, n_halo;    // halo positions
-    int32_t item0, n_items;   // SpMM work items
-    int32_t mrow0, n_mrows;   // multi-chunk rows
-    int32_t mitem0, n_mitems; // partial-sum rows
     int32_t push0, n_push;
     int32_t hlong0, n_hlong;  // long halo rows
     int p0, p1;               // partitions [p0, p1)
@@ -342,6 +336,18 @@ enum class SpmmHalo { by_position, by_gid, by_slot };
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask = nullptr,
                     int32_t omask_words = 0, SpmmHalo halo_kind = SpmmHalo::by_position, bool in_global = false);
+// the same kernels on weights of the caller's: out[row] = epilogue(sum_e w_e * src(col_e)) with ent[e] = {column, weight} indexed like
+// the entries of the mode (0: local rows; 1: their inner prefix; 3: halo rows, columns = partition-major rows)
+struct SpmmEpilogue {
+    const float *bias = nullptr;                              // [d]
+    int relu = 0;
+    const float *s1 = nullptr, *v1 = nullptr, *s2 = nullptr, *v2 = nullptr;   // + s1[row] v1[col] + s2[row] v2[col]
+    int32_t d = 0;
+};
+sat_status sat_spmm_entries(sat_ctx *ctx, const PartView &v, int mode, int32_t d, const int2 *ent, const float *in_base, int32_t ld_in,
+                            const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const SpmmEpilogue &ep);
+// the work items such a product walks at width d
+sat_status sat_spmm_items(sat_ctx *ctx, const PartView &v, int mode, int32_t d, const int4 **items, int64_t *n_items);
 //   halo-row products: out[j] = sum_{e in hrow(j)} dinv[halo j] dinv[inner e] * src[pos_e], or with by_slot the rows of src by cache
 //   slot, including the self term
 sat_status sat_spmm_hrow(sat_ctx *ctx, const PartView &v, int32_t d, const float *src_base, int32_t ld_src, int by_slot, float *out_base,
@@ -465,9 +471,10 @@ struct TcEpilogueHost {
 };
 // tensor-core path on / off for a contraction with n outputs and k terms (SAT_NO_TC=1 in the environment forces the CUDA cores)
 bool sat_use_tc(int32_t n, int32_t k);
-// dst = src o mask (skipped when dst is null) and colsum (+)= 1^T (src o mask) (skipped when colsum is null)
+// dst = src o mask (skipped when dst is null) and colsum (+)= 1^T (src o mask) (skipped when colsum is null); with `act` the mask is
+// act > 0 instead of the bits
 sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t rows, int32_t d, const uint32_t *mask, int32_t mask_words,
-                         float *dst, int32_t ld_dst, float *colsum, int accumulate);
+                         float *dst, int32_t ld_dst, float *colsum, int accumulate, const float *act = nullptr, int32_t ld_act = 0);
 // weight planes in `buf`; transpose = 1 for W given as [K x N], 0 for [N x K]; optional second source continuing along K
 // gate_h > 0: the n = 4 gate_h columns (gate blocks i | f | g | o) are interleaved so that packed column 4 j + gate is gate `gate`
 // of hidden unit j (what the fused LSTM epilogue expects)

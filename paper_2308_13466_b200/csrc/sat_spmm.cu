@@ -421,18 +421,38 @@ static sat_status list_build(sat_ctx *ctx, const ListKey &want, SpmmList **out)
 // kernel spills), descriptors of the next item fetched ahead (20-60 % slower), 6-8 blocks per SM at NV = 2 (fewer registers:
 // fewer rows in flight).
 // -------------------------------------------------------------------------------------
-template <int G, int NV, int U, int MINB>
+// result of row `row`, float4 column c, before the store: act(s * acc + bias + s1[row] v1 + s2[row] v2) (attention layer)
+__device__ __forceinline__ float4 spmm_epilogue(const SpmmEpilogue &ep, int64_t row, int c, float4 r)
+{
+    float x[4] = {r.x, r.y, r.z, r.w};
+    const float s1 = ep.s1 ? __ldg(ep.s1 + row) : 0.f, s2 = ep.s2 ? __ldg(ep.s2 + row) : 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int col = 4 * c + k;
+        if (col >= ep.d) {   // padding columns hold zeros
+            x[k] = 0.f;
+            continue;
+        }
+        if (ep.bias) x[k] += __ldg(ep.bias + col);
+        if (ep.s1) x[k] += s1 * __ldg(ep.v1 + col);
+        if (ep.s2) x[k] += s2 * __ldg(ep.v2 + col);
+        if (ep.relu) x[k] = fmaxf(x[k], 0.f);
+    }
+    return make_float4(x[0], x[1], x[2], x[3]);
+}
+
+template <int G, int NV, int U, int MINB, bool EPI>
 __global__ void __launch_bounds__(256, MINB)
 k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const int2 *__restrict__ ent, const float *__restrict__ scale, int32_t n,
        int32_t d4, const float *__restrict__ in_base, int64_t ld_in, const float *__restrict__ halo_base, int64_t ld_halo, float *__restrict__ out_base,
-       int64_t ld_out, float *__restrict__ partial, const uint32_t *__restrict__ omask, int32_t omask_words, DbgLimits dbg)
+       int64_t ld_out, float *__restrict__ partial, const uint32_t *__restrict__ omask, int32_t omask_words, SpmmEpilogue ep, DbgLimits dbg)
 {
     const int lane = threadIdx.x & (G - 1);
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     if (gid >= n_items) return;
     const int col = blockIdx.y * (G * NV) + lane;
     const int4 it = __ldg(items + gid);
-    const int2 *__restrict__ ep = ent + ((int64_t)(uint32_t)it.z | ((int64_t)(it.w & 0xffff) << 32));
+    const int2 *__restrict__ ents = ent + ((int64_t)(uint32_t)it.z | ((int64_t)(it.w & 0xffff) << 32));
     const int32_t len = it.w >> 16;
     // columns below n index the inner matrix, the others the halo matrix (addressed from its virtual row -n): one multiply-add
     // per row either way
@@ -452,7 +472,7 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
     for (; e + U <= len; e += U) {
         int2 q[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) q[u] = __ldg(ep + e + u);
+        for (int u = 0; u < U; ++u) q[u] = __ldg(ents + e + u);
         float4 x[U][NV];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -466,7 +486,7 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
             for (int v = 0; v < NV; ++v) fma4(acc[v], __int_as_float(q[u].y), x[u][v]);
     }
     for (; e < len; ++e) {
-        const int2 q = __ldg(ep + e);
+        const int2 q = __ldg(ents + e);
         const float4 *src = row_of(q.x);
 #pragma unroll
         for (int v = 0; v < NV; ++v)
@@ -474,13 +494,14 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
     }
     if (it.y < 0) {
         const int64_t row = SAT_IDX((int64_t)it.x, dbg.out_lo, dbg.out_hi, dbg.status);
-        const float s = __ldg(scale + row);
+        const float s = EPI ? 1.f : __ldg(scale + row);
         float4 *o = reinterpret_cast<float4 *>(out_base + row * ld_out) + col;
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             if (col + v * G < d4) {
                 float4 r = make_float4(s * acc[v].x, s * acc[v].y, s * acc[v].z, s * acc[v].w);
-                if (omask) mask4(r, omask, row * omask_words, col + v * G);
+                if (EPI) r = spmm_epilogue(ep, row, col + v * G, r);
+                else if (omask) mask4(r, omask, row * omask_words, col + v * G);
                 o[v * G] = r;
             }
         }
@@ -517,7 +538,7 @@ __device__ __forceinline__ float4 fixup_range(const float4 *__restrict__ p, int3
 __global__ void __launch_bounds__(256)
 k_spmm_fixup(const int32_t *__restrict__ hrows, int32_t n_hrows, const int32_t *__restrict__ mrows, int32_t n_mrows, const int32_t *__restrict__ slot0,
              const int32_t *__restrict__ tot, int64_t slot_base, const float *__restrict__ scale, int32_t d4, const float *__restrict__ partial,
-             float *__restrict__ out_base, int64_t ld_out, const uint32_t *__restrict__ omask, int32_t omask_words, DbgLimits dbg)
+             float *__restrict__ out_base, int64_t ld_out, const uint32_t *__restrict__ omask, int32_t omask_words, SpmmEpilogue ep, DbgLimits dbg)
 {
     __shared__ float4 part[8][32];
     const int32_t slabs = (d4 + 31) / 32;
@@ -551,15 +572,17 @@ k_spmm_fixup(const int32_t *__restrict__ hrows, int32_t n_hrows, const int32_t *
         row = SAT_IDX((int64_t)mrows[i], dbg.out_lo, dbg.out_hi, dbg.status);
         a = fixup_range(reinterpret_cast<const float4 *>(partial) + ((int64_t)slot0[row] - slot_base) * d4 + c, 0, tot[row], d4);
     }
-    const float s = scale[row];
+    const float s = scale ? scale[row] : 1.f;
     float4 r = make_float4(s * a.x, s * a.y, s * a.z, s * a.w);
-    if (omask) mask4(r, omask, row * omask_words, c);
+    if (!scale) r = spmm_epilogue(ep, row, c, r);
+    else if (omask) mask4(r, omask, row * omask_words, c);
     *reinterpret_cast<float4 *>(out_base + row * ld_out + 4 * c) = r;
 }
 
 struct SpmmArgs {
     const int2 *ent;
-    const float *scale;          // per row of the list
+    const float *scale;          // per row of the list; null: no scaling, and the epilogue `ep` instead of the mask
+    SpmmEpilogue ep;
     int32_t n;                   // columns below n address `in`, the others `halo`
     const float *in_base, *halo_base;
     int32_t ld_in, ld_halo;
@@ -574,8 +597,13 @@ template <int G, int NV, int U, int MINB>
 static void launch_spmm(sat_ctx *ctx, const int4 *items, int32_t n_items, int64_t slot_base, int32_t d4, const SpmmArgs &a, float *partial)
 {
     dim3 grid((unsigned)cdiv64((int64_t)n_items * G, 256), (unsigned)cdiv64(d4, G * NV));
-    k_spmm<G, NV, U, MINB><<<grid, 256, 0, ctx->stream>>>(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
-                                                          a.out_base, a.ld_out, partial, a.omask, a.omask_words, dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1));
+    const DbgLimits dbg = dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1);
+    if (a.scale)
+        k_spmm<G, NV, U, MINB, false><<<grid, 256, 0, ctx->stream>>>(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
+                                                                     a.out_base, a.ld_out, partial, a.omask, a.omask_words, a.ep, dbg);
+    else
+        k_spmm<G, NV, U, MINB, true><<<grid, 256, 0, ctx->stream>>>(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
+                                                                    a.out_base, a.ld_out, partial, a.omask, a.omask_words, a.ep, dbg);
 }
 
 // walks partitions [v.p0, v.p1) of a list
@@ -608,7 +636,7 @@ static sat_status run_list(sat_ctx *ctx, const PartView &v, const SpmmList &l, i
     if (n_slots > 0) {
         k_spmm_fixup<<<(unsigned)(n_hrows * cdiv64(d4, 32) + cdiv64(n_mrows * d4, 256)), 256, 0, ctx->stream>>>(
             l.hrows + hrow0, (int32_t)n_hrows, l.mrows + mrow0, (int32_t)n_mrows, l.slot0, l.tot, slot_base, a.scale, d4, partial, a.out_base, a.ld_out, a.omask,
-            a.omask_words, dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1));
+            a.omask_words, a.ep, dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1));
         SAT_LAUNCHED(ctx);
     }
     return SAT_OK;
@@ -689,6 +717,40 @@ sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, 
     a.omask = omask;
     a.omask_words = omask_words;
     return run_list(ctx, v, *l, d4, a);
+}
+
+sat_status sat_spmm_entries(sat_ctx *ctx, const PartView &v, int mode, int32_t d, const int2 *ent, const float *in_base, int32_t ld_in,
+                            const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const SpmmEpilogue &ep)
+{
+    SpmmList *l = nullptr;
+    SAT_TRY(list_build(ctx, list_key((d + 3) / 4, mode), &l));
+    SpmmArgs a;
+    a.ent = ent;
+    a.scale = nullptr;
+    a.ep = ep;
+    a.ep.d = d;
+    a.n = mode == 0 ? ctx->n : INT32_MAX;
+    a.in_base = in_base;
+    a.ld_in = ld_in;
+    a.halo_base = halo_base;
+    a.ld_halo = ld_halo;
+    a.out_base = out_base;
+    a.ld_out = ld_out;
+    a.omask = nullptr;
+    a.omask_words = 0;
+    a.src = DbgRange{v.row0, (int64_t)v.row0 + v.n_rows};
+    a.halo = DbgRange{v.halo0, v.halo0 + v.n_halo};
+    a.out = mode == 3 ? a.halo : a.src;
+    return run_list(ctx, v, *l, (d + 3) / 4, a);
+}
+
+sat_status sat_spmm_items(sat_ctx *ctx, const PartView &v, int mode, int32_t d, const int4 **items, int64_t *n_items)
+{
+    SpmmList *l = nullptr;
+    SAT_TRY(list_build(ctx, list_key((d + 3) / 4, mode), &l));
+    *items = l->item + l->off[v.p0];
+    *n_items = l->off[v.p1] - l->off[v.p0];
+    return SAT_OK;
 }
 
 extern "C" sat_status sat_spmm_plan(sat_ctx *ctx, int32_t part, int32_t d, int32_t *n_blocks, int64_t *n_items, int64_t *n_partial_rows)
