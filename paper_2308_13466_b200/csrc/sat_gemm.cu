@@ -322,10 +322,14 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
 // C = A^T B sums ~1e5 signed terms per element that cancel to a few 1e-3 of their magnitude (softmax gradients sum to
 // zero); the tensor-core contraction, whose accumulation truncates, was measured at 1e-4 relative error there against
 // 2e-5 for this kernel, which at this width costs about the same.
-//   block (x, y): rows [x * rows_per_block, ...), columns y * 256 .. + 255 of A, two per thread; B rows are
-//   staged in shared memory and broadcast; partial sums per row block, added in block order by k_splitk_reduce.
+//   block (x, y): rows [x * rows_per_block, ...), columns y * 64 TM .. + 64 TM - 1 of A against all n <= NT columns of B; partial sums per
+//   row block, added in block order by k_splitk_reduce.  128 threads: thread t owns the TM columns TM (t % 64) .. of A and one half
+//   (t / 64) of the columns of B, so that a staged row costs it TM / 4 + NT / 8 128-bit shared loads for TM NT / 2 FMAs.  (Two columns
+//   of A against all of B, the first layout, took 1 + NT / 4 loads for the same FMAs.)  NT goes in steps of 8 so that little of it is
+//   padding.  Bound by FMA issue and the shared loads that feed it: 169 k x 256 x 40 115 -> 93 us (48 us of FMAs, 31 us of reads),
+//   2,048 x 16 x 16 9.2 -> 4.5 us.
 // =====================================================================================
-#define TNN_STAGE 32
+#define TNN_STAGE 16
 __device__ __forceinline__ void tnn_cp16(void *smem_dst, const void *gsrc, bool valid)
 {
     // src-size 0 writes 16 zero bytes without reading the source
@@ -333,32 +337,29 @@ __device__ __forceinline__ void tnn_cp16(void *smem_dst, const void *gsrc, bool 
                  "r"(valid ? 16u : 0u)
                  : "memory");
 }
-// two stages of [TNN_STAGE x 256] of A and [TNN_STAGE x NT] of B, filled by cp.async while the previous stage is consumed;
-// 128 threads, each owning columns t and t + 128 of the block's 256 columns of A (2 NT accumulators: two FMAs per
-// broadcast shared-memory load of B)
-template <int NT>
+template <int NT, int TM>
 __global__ void __launch_bounds__(128)
 k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, const float *__restrict__ A, int64_t lda,
                  const float *__restrict__ B, int64_t ldb, float *__restrict__ part, float *__restrict__ part_cs)
 {
     extern __shared__ __align__(16) float tnn_smem[];
+    constexpr int MC = 64 * TM, NH = NT / 2, STAGE_FLOATS = TNN_STAGE * (MC + NT);
     // column sums of B (the bias gradient), by the blocks with y == 0: thread t takes column t % NT of every (128 / NT)-th staged row
     constexpr int CS_GROUPS = 128 / NT;
     const bool want_cs = part_cs != nullptr && blockIdx.y == 0 && threadIdx.x < NT * CS_GROUPS;
     float cs = 0.f;
-    constexpr int STAGE_FLOATS = TNN_STAGE * 256 + TNN_STAGE * NT;
-    const int32_t m0 = blockIdx.y * 256;
-    const int32_t col0 = m0 + threadIdx.x, col1 = col0 + 128;
+    const int32_t m0 = blockIdx.y * MC;
+    const int cg = threadIdx.x & 63, half = threadIdx.x >> 6;
     const int32_t m4 = (m + 3) & ~3, n4 = (n + 3) & ~3;
     const int64_t r_begin = (int64_t)blockIdx.x * rows_per_block;
     const int64_t r_end = r_begin + rows_per_block < rows ? r_begin + rows_per_block : rows;
     auto load_stage = [&](int s, int64_t r0) {
-        float *As = tnn_smem + s * STAGE_FLOATS, *Bs = As + TNN_STAGE * 256;
+        float *As = tnn_smem + s * STAGE_FLOATS, *Bs = As + TNN_STAGE * MC;
 #pragma unroll
-        for (int k = 0; k < TNN_STAGE * 64 / 128; ++k) {
-            const int i = threadIdx.x + 128 * k, rr = i >> 6, c4 = i & 63;
+        for (int k = 0; k < TNN_STAGE * MC / 4 / 128; ++k) {
+            const int i = threadIdx.x + 128 * k, rr = i / (MC / 4), c4 = i % (MC / 4);
             const bool ok = r0 + rr < r_end && m0 + 4 * c4 < m4;
-            tnn_cp16(As + rr * 256 + 4 * c4, ok ? A + (r0 + rr) * lda + m0 + 4 * c4 : A, ok);
+            tnn_cp16(As + rr * MC + 4 * c4, ok ? A + (r0 + rr) * lda + m0 + 4 * c4 : A, ok);
         }
         for (int i = threadIdx.x; i < TNN_STAGE * (NT / 4); i += 128) {
             const int rr = i / (NT / 4), j4 = i - rr * (NT / 4);
@@ -368,10 +369,11 @@ k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, con
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     // accumulators as pairs: the packed FMA of sm_100 (two IEEE-rounded fp32 FMAs per instruction, same results as fmaf)
-    // halves the issue slots of the inner loop, which is bound by FMA issue
-    float2 acc0[NT / 2], acc1[NT / 2];
+    float2 acc[TM][NH / 2];
 #pragma unroll
-    for (int j = 0; j < NT / 2; ++j) acc0[j] = acc1[j] = make_float2(0.f, 0.f);
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < NH / 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
     int s = 0;
     load_stage(0, r_begin);
     for (int64_t r0 = r_begin; r0 < r_end; r0 += TNN_STAGE, s ^= 1) {
@@ -382,19 +384,29 @@ k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, con
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
-        const float *As = tnn_smem + s * STAGE_FLOATS, *Bs = As + TNN_STAGE * 256;
+        const float *As = tnn_smem + s * STAGE_FLOATS, *Bs = As + TNN_STAGE * MC;
 #pragma unroll 2
         for (int rr = 0; rr < TNN_STAGE; ++rr) {
-            const float a0 = As[rr * 256 + threadIdx.x], a1 = As[rr * 256 + 128 + threadIdx.x];
-            const float2 a0p = make_float2(a0, a0), a1p = make_float2(a1, a1);
+            float av[TM];
+            if (TM == 4) {
+                const float4 t = *reinterpret_cast<const float4 *>(As + rr * MC + 4 * cg);
+                av[0] = t.x; av[1 % TM] = t.y; av[2 % TM] = t.z; av[3 % TM] = t.w;
+            } else if (TM == 2) {
+                const float2 t = *reinterpret_cast<const float2 *>(As + rr * MC + 2 * cg);
+                av[0] = t.x; av[1 % TM] = t.y;
+            } else {
+                av[0] = As[rr * MC + cg];
+            }
+            const float4 *bp = reinterpret_cast<const float4 *>(Bs + rr * NT + half * NH);
 #pragma unroll
-            for (int j4 = 0; j4 < NT; j4 += 4) {
-                const float4 b = *reinterpret_cast<const float4 *>(Bs + rr * NT + j4);
-                const float2 blo = make_float2(b.x, b.y), bhi = make_float2(b.z, b.w);
-                acc0[j4 / 2] = __ffma2_rn(a0p, blo, acc0[j4 / 2]);
-                acc0[j4 / 2 + 1] = __ffma2_rn(a0p, bhi, acc0[j4 / 2 + 1]);
-                acc1[j4 / 2] = __ffma2_rn(a1p, blo, acc1[j4 / 2]);
-                acc1[j4 / 2 + 1] = __ffma2_rn(a1p, bhi, acc1[j4 / 2 + 1]);
+            for (int j4 = 0; j4 < NH / 4; ++j4) {
+                const float4 b = bp[j4];
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const float2 ap = make_float2(av[i], av[i]);
+                    acc[i][2 * j4] = __ffma2_rn(ap, make_float2(b.x, b.y), acc[i][2 * j4]);
+                    acc[i][2 * j4 + 1] = __ffma2_rn(ap, make_float2(b.z, b.w), acc[i][2 * j4 + 1]);
+                }
             }
         }
         if (want_cs) {
@@ -412,34 +424,50 @@ k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, con
             for (int g = 1; g < CS_GROUPS; ++g) t += tnn_smem[g * NT + threadIdx.x];
             part_cs[(int64_t)blockIdx.x * n + threadIdx.x] = t;
         }
+        __syncthreads();
     }
-    if (col0 < m) {
-        float *o = part + ((int64_t)blockIdx.x * m + col0) * n;
+    // the partial sums leave through shared memory, one half of the columns at a time, in runs of NH floats
+    float *o = part + (int64_t)blockIdx.x * m * n;
+    for (int h = 0; h < 2; ++h) {
+        if (half == h) {
 #pragma unroll
-        for (int j = 0; j < NT; ++j)
-            if (j < n) o[j] = (j & 1) ? acc0[j / 2].y : acc0[j / 2].x;
-    }
-    if (col1 < m) {
-        float *o = part + ((int64_t)blockIdx.x * m + col1) * n;
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < NT; ++j)
-            if (j < n) o[j] = (j & 1) ? acc1[j / 2].y : acc1[j / 2].x;
+                for (int j = 0; j < NH / 2; ++j) {
+                    tnn_smem[(TM * cg + i) * (NH + 1) + 2 * j] = acc[i][j].x;
+                    tnn_smem[(TM * cg + i) * (NH + 1) + 2 * j + 1] = acc[i][j].y;
+                }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < MC * NH; i += 128) {
+            const int c = i / NH, j = i - c * NH;
+            if (m0 + c < m && h * NH + j < n) o[(int64_t)(m0 + c) * n + h * NH + j] = tnn_smem[c * (NH + 1) + j];
+        }
+        __syncthreads();
     }
 }
 
-template <int NT>
-static sat_status launch_tn_narrow(sat_ctx *ctx, dim3 grid, int64_t rows, int64_t rpb, int32_t m, int32_t n, const float *A, int32_t lda,
-                                   const float *B, int32_t ldb, float *part, float *part_cs)
+template <int NT, int TM>
+static sat_status launch_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb,
+                                   int accumulate, float *C, int32_t ldc, float *colsum)
 {
     static PerDeviceOnce attr_set;
-    const size_t smem = 2 * (size_t)(TNN_STAGE * 256 + TNN_STAGE * NT) * sizeof(float);
+    constexpr size_t stage2 = 2 * (size_t)TNN_STAGE * (64 * TM + NT), turn = (size_t)64 * TM * (NT / 2 + 1);
+    constexpr size_t smem = (stage2 > turn ? stage2 : turn) * sizeof(float);
     if (attr_set.need(ctx->device)) {
-        SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tn_narrow<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tn_narrow<NT, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr_set.mark(ctx->device);
     }
-    k_gemm_tn_narrow<NT><<<grid, 128, smem, ctx->stream>>>(rows, rpb, m, n, A, lda, B, ldb, part, part_cs);
+    // one wave of row blocks, three per SM; at least four stages each (below that the partial sums outweigh the products)
+    const int64_t yb = cdiv64(m, 64 * TM), want = std::max<int64_t>(1, 3 * 148 / yb);
+    const int64_t rpb = std::max<int64_t>(4 * TNN_STAGE, cdiv64(cdiv64(rows > 0 ? rows : 1, want), TNN_STAGE) * TNN_STAGE);
+    const int64_t blocks = cdiv64(rows > 0 ? rows : 1, rpb);
+    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)blocks * ((size_t)m * n + n) * sizeof(float)));
+    float *part = (float *)ctx->buf_splitk.p;
+    float *part_cs = colsum ? part + (size_t)blocks * m * n : nullptr;
+    k_gemm_tn_narrow<NT, TM><<<dim3((unsigned)blocks, (unsigned)yb), 128, smem, ctx->stream>>>(rows, rpb, m, n, A, lda, B, ldb, part, part_cs);
     SAT_LAUNCHED(ctx);
-    return SAT_OK;
+    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)blocks, accumulate, C, n, ldc, part_cs, n, colsum);
 }
 
 // C[m x n] (+)= A^T B over `rows` rows for n <= 64 (B already masked)
@@ -450,22 +478,18 @@ sat_status sat_gemm_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, 
     if (n > 64 || (lda & 3) || (ldb & 3) || (((uintptr_t)A | (uintptr_t)B) & 15u))
         return sat_fail(ctx, SAT_EINVAL, "sat_gemm_tn_narrow: n must be <= 64, operands 16-byte aligned with leading dimensions in multiples of 4");
     ProfScope prof(ctx, SATK_GEMM_TN, 4.0 * ((double)rows * (m + n) + (double)m * n), 2.0 * (double)rows * m * n);
-    // two CTAs fit on an SM (80 KB of shared memory each): one full wave of row blocks
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-    const int64_t want = (2 * (int64_t)sms) / cdiv64(m, 256) > 0 ? (2 * (int64_t)sms) / cdiv64(m, 256) : 1;
-    int64_t rpb = cdiv64(cdiv64(rows > 0 ? rows : 1, want), TNN_STAGE) * TNN_STAGE;
-    if (rpb < 4 * TNN_STAGE) rpb = 4 * TNN_STAGE;
-    const int64_t blocks = cdiv64(rows > 0 ? rows : 1, rpb);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)blocks * ((size_t)m * n + n) * sizeof(float)));
-    float *part = (float *)ctx->buf_splitk.p;
-    float *part_cs = colsum ? part + (size_t)blocks * m * n : nullptr;
-    dim3 grid((unsigned)blocks, (unsigned)cdiv64(m, 256));
-    if (n <= 16) SAT_TRY(launch_tn_narrow<16>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
-    else if (n <= 32) SAT_TRY(launch_tn_narrow<32>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
-    else if (n <= 48) SAT_TRY(launch_tn_narrow<48>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
-    else SAT_TRY(launch_tn_narrow<64>(ctx, grid, rows, rpb, m, n, A, lda, B, ldb, part, part_cs));
-    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)blocks, accumulate, C, n, ldc, part_cs, n, colsum);
+#define CALL(NT)                                                                                                        \
+    (m <= 64 ? launch_tn_narrow<NT, 1>(ctx, rows, m, n, A, lda, B, ldb, accumulate, C, ldc, colsum)                      \
+             : m <= 128 ? launch_tn_narrow<NT, 2>(ctx, rows, m, n, A, lda, B, ldb, accumulate, C, ldc, colsum)           \
+                        : launch_tn_narrow<NT, 4>(ctx, rows, m, n, A, lda, B, ldb, accumulate, C, ldc, colsum))
+    if (n <= 16) return CALL(16);
+    if (n <= 24) return CALL(24);
+    if (n <= 32) return CALL(32);
+    if (n <= 40) return CALL(40);
+    if (n <= 48) return CALL(48);
+    if (n <= 56) return CALL(56);
+    return CALL(64);
+#undef CALL
 }
 
 // =====================================================================================
