@@ -96,7 +96,7 @@ extern "C" sat_status sat_create(sat_ctx **out, int device, void *cuda_stream)
     ctx->device = device;
     ctx->stream = (cudaStream_t)cuda_stream;
     if (cudaMalloc((void **)&ctx->d_flag, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMallocHost((void **)&ctx->h_flag, sizeof(int)) != cudaSuccess) {
+        cudaMallocHost((void **)&ctx->h_flag, 4 * sizeof(int)) != cudaSuccess) {
         delete ctx;
         return SAT_ENOMEM;
     }
