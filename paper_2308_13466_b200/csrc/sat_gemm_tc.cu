@@ -13,7 +13,7 @@
 //                 (weight gradient)
 // Warp roles of k_gemm_tc_k (512 threads): warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, then 6 converter and
 // 8 epilogue warps (two per TMEM lane quadrant), or 2 + 12 for the K = h variants with a side operand.  k_gemm_tc_mn:
-// warps 0 / 1 as above, warps 2..5 convert during the main loop and then run the epilogue.  Every mbarrier wait is
+// warps 0 / 1 as above, warps 2..9 convert during the main loop and then run the epilogue.  Every mbarrier wait is
 // bounded; a timeout raises a status word and lets the CTA drain (TMEM is freed, the kernel returns).
 #include <cuda.h>
 
@@ -21,7 +21,6 @@
 
 #define TC_BM 128
 #define TC_BK 16          /* fp32 elements per k-block: 64-byte rows */
-#define TC_THREADS 192
 #define TC_WAIT_LIMIT (1u << 22)
 
 // =====================================================================================
@@ -157,7 +156,7 @@ __host__ __device__ inline uint32_t make_idesc(int n, int a_mn_major, int b_mn_m
 // The tensor core reads an fp32 container as TF32 by ignoring the low 13 mantissa bits.  split_tile_residual uses that:
 // the raw tile already is the "hi" operand (hi = x with those bits cleared) and only lo = tf32_rn(x - hi) is written, to
 // the second tile (x - hi is exact; rounding lo to nearest keeps the representation error |x - hi - lo| <= 2^-21 |x|
-// free of bias).  split_tile_round rounds hi to nearest as well and rewrites the raw tile in place: hi and lo are then
+// free of bias).  split4 rounds hi to nearest as well and the weight gradient rewrites the raw tile in place: hi and lo are then
 // symmetric around x, which matters for the weight gradient (a small difference of ~1e5 signed terms per element).
 // =====================================================================================
 __device__ __forceinline__ float tf32_round(float x)
@@ -188,26 +187,6 @@ __device__ __forceinline__ void split_tile_residual(const uint8_t *hi_tile, uint
         if (two) x2 = *reinterpret_cast<const float4 *>(hi_tile + off2);
         *reinterpret_cast<float4 *>(lo_tile + off) = residual4(x1);
         if (two) *reinterpret_cast<float4 *>(lo_tile + off2) = residual4(x2);
-    }
-}
-__device__ __forceinline__ void split_tile_round(uint8_t *hi_tile, uint8_t *lo_tile, uint32_t bytes, int tid, int nthreads)
-{
-    const uint32_t step = (uint32_t)nthreads * 16;
-    for (uint32_t off = (uint32_t)tid * 16; off < bytes; off += 2 * step) {
-        const uint32_t off2 = off + step;
-        const bool two = off2 < bytes;
-        const float4 x1 = *reinterpret_cast<float4 *>(hi_tile + off);
-        float4 x2 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (two) x2 = *reinterpret_cast<float4 *>(hi_tile + off2);
-        float4 h1, l1, h2, l2;
-        split4(x1, h1, l1);
-        split4(x2, h2, l2);
-        *reinterpret_cast<float4 *>(hi_tile + off) = h1;
-        *reinterpret_cast<float4 *>(lo_tile + off) = l1;
-        if (two) {
-            *reinterpret_cast<float4 *>(hi_tile + off2) = h2;
-            *reinterpret_cast<float4 *>(lo_tile + off2) = l2;
-        }
     }
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
@@ -253,15 +232,12 @@ struct TcShared {
     uint64_t full[4];       // TMA bytes of the stage have landed
     uint64_t conv[4];       // the converter threads have split the stage
     uint64_t empty[4];      // the MMAs reading the stage have completed
-    uint64_t accum;         // (MN-major kernel) all MMAs of the tile have completed
-    uint64_t acc_full[2];   // (K-major kernel) accumulator buffer holds a finished tile
-    uint64_t acc_empty[2];  // (K-major kernel) accumulator buffer has been drained by the epilogue
+    uint64_t acc_full[2];   // accumulator buffer holds a finished tile
+    uint64_t acc_empty[2];  // accumulator buffer has been drained by the epilogue
     uint32_t tmem_base;
     int dead;
 };
 
-#define TC_CONV_THREADS 128
-#define TC_EPI_THREADS 128
 /* 512 threads, 128 registers each: warp 0 TMA, warp 1 MMA, then the converter warps, then the epilogue warps.  The split
  * between converters and epilogue depends on the epilogue variant (TckCfg): the K = h variants with a side operand have
  * four k-blocks per tile and an epilogue bound by instruction issue, so they run 2 + 12 instead of 6 + 8.
@@ -727,31 +703,47 @@ done:
 // MN-major kernel (weight gradient): block (x, y, z) = tile (x, y) of A^T B over rows [z * rps, (z + 1) * rps); the blocks with x == 0
 // also leave the column sums of their rows of B (the bias gradient) in part_cs [z x N] when it is given: the converters hold every
 // value of B in registers anyway, which saves a pass over it (34 us for 169 k x 256).
-// The main loop is bound by shared-memory traffic: per k-block of 16 rows at N = 256 the TMA writes 24 KB, the converters read 24
-// and write 48 KB and the MMAs read 72 KB, 0.7 us at 128 B per clock against 0.4 us of tensor work.
+//
+// Tile: up to 256 columns of A (two accumulators of 128 TMEM lanes) by up to 256 of B, one CTA per SM (two where m <= 128).  Both operands are activations
+// and have to be split in the kernel; a 256-column tile of A converts and fetches B once where two 128-column CTAs did it twice, and the
+// ring holds three stages of 64 KB instead of two per CTA.  Per k-block of 16 rows at 256 x 256 the TMA writes 32 KB, eight converter
+// warps read 32 and write 64 KB and the MMAs read 144 KB: 1.1 us at 128 B per clock, as much as the tensor work (1.1 us).
 // =====================================================================================
-__global__ void __launch_bounds__(TC_THREADS, 2)
-k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int32_t Mdim, int32_t N, int64_t rps,
-             int32_t bn, int32_t stages, int32_t tmem_cols, float *part_C, float *part_cs, int *status)
+#define MN_STAGES_MAX 6
+#define MN_CONV_THREADS 256
+#define MN_THREADS (64 + MN_CONV_THREADS)
+#define MN_SMEM_MAX (227 * 1024)
+#define MN_TURN_BYTES (8u * 32 * 33 * 4)   /* the epilogue turns eight 32 x 32 blocks around in the stages */
+struct MnShared {
+    uint64_t full[MN_STAGES_MAX], conv[MN_STAGES_MAX], empty[MN_STAGES_MAX];
+    uint64_t accum;
+    uint32_t tmem_base;
+    int dead;
+};
+
+__global__ void __launch_bounds__(MN_THREADS, 2)
+k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int32_t Mdim, int32_t N, int64_t rps, int64_t rows,
+             int32_t mt_max, int32_t bn, int32_t stages, uint32_t tmem_cols, float *part_C, float *part_cs, int *status)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const uint32_t blk_bytes = TC_BK * 128;                // one 32-column block of a k-block: 16 rows x 128 B
+    constexpr uint32_t blk_bytes = TC_BK * 128;            // one 32-column block of a k-block: 16 rows x 128 B
+    constexpr uint32_t sub_bytes = (TC_BM / 32) * blk_bytes;  // one plane of 128 columns of A
     const int n_blks_b = (bn + 31) / 32;
-    const uint32_t a_bytes = (TC_BM / 32) * blk_bytes;     // one plane of A: 128 columns
-    const uint32_t b_bytes = (uint32_t)n_blks_b * blk_bytes;
+    const uint32_t a_bytes = (uint32_t)mt_max * sub_bytes, b_bytes = (uint32_t)n_blks_b * blk_bytes;
     const uint32_t stage_bytes = 2 * a_bytes + 2 * b_bytes;  // [A hi | A lo | B hi | B lo]
-    TcShared *sh = (TcShared *)(smem + (size_t)stages * stage_bytes);
+    const uint32_t stage_area = (uint32_t)stages * stage_bytes > MN_TURN_BYTES ? (uint32_t)stages * stage_bytes : MN_TURN_BYTES;
+    MnShared *sh = (MnShared *)(smem + stage_area);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int32_t m0 = blockIdx.x * TC_BM;
-    const int32_t n0 = blockIdx.y * bn;
-    const int64_t r0 = (int64_t)blockIdx.z * rps;
-    const int32_t nkb = (int32_t)(rps / TC_BK);
+    const int32_t m0 = blockIdx.x * (mt_max * TC_BM), n0 = blockIdx.y * bn;
+    const int32_t mt = (Mdim - m0 + TC_BM - 1) / TC_BM < mt_max ? (Mdim - m0 + TC_BM - 1) / TC_BM : mt_max;   // 128-column sub-tiles in use
+    const int64_t r0 = (int64_t)blockIdx.z * rps, r1 = r0 + rps < rows ? r0 + rps : rows;
+    const int32_t nkb = (int32_t)((r1 - r0 + TC_BK - 1) / TC_BK);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
             mbar_init(&sh->full[s], 1);
-            mbar_init(&sh->conv[s], TC_CONV_THREADS);
+            mbar_init(&sh->conv[s], MN_CONV_THREADS);
             mbar_init(&sh->empty[s], 1);
         }
         mbar_init(&sh->accum, 1);
@@ -759,8 +751,7 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"((uint32_t)tmem_cols)
-                     : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"(tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -777,34 +768,35 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
                 if (!mbar_wait(&sh->empty[s], ph ^ 1u, dead, status)) break;
                 uint8_t *st = smem + (size_t)s * stage_bytes;
                 const int32_t r = (int32_t)(r0 + (int64_t)kb * TC_BK);
-                mbar_expect_tx(&sh->full[s], a_bytes + b_bytes);
-                for (int bl = 0; bl < TC_BM / 32; ++bl) tma_load_2d(st + bl * blk_bytes, &mapA, &sh->full[s], m0 + bl * 32, r);
+                mbar_expect_tx(&sh->full[s], (uint32_t)mt * sub_bytes + b_bytes);
+                for (int bl = 0; bl < mt * (TC_BM / 32); ++bl) tma_load_2d(st + bl * blk_bytes, &mapA, &sh->full[s], m0 + bl * 32, r);
                 for (int bl = 0; bl < n_blks_b; ++bl) tma_load_2d(st + 2 * a_bytes + bl * blk_bytes, &mapB, &sh->full[s], n0 + bl * 32, r);
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             const uint32_t idesc = make_idesc(bn, 1, 1);
+            // MN-major 32-bit operands use the 128-byte swizzle with 32-byte atoms (the only layout the tensor core accepts for them):
+            // 32-column blocks blk_bytes apart (leading offset), groups of 4 k-rows 512 B apart (stride offset); a k-step is 8 rows =
+            // 1024 B.  Only the 14-bit start-address field (bytes >> 4) differs between the descriptors.
+            const uint64_t desc0 = make_desc(smem_u32(smem), blk_bytes, 512, 1);
             for (int32_t kb = 0; kb < nkb; ++kb) {
                 const int s = kb % stages;
                 const uint32_t ph = (uint32_t)(kb / stages) & 1u;
                 // the converters arrive on conv[s] only after they have seen full[s] (the TMA bytes) themselves
                 if (!mbar_wait(&sh->conv[s], ph, dead, status)) break;
                 tc_fence_after();
-                const uint32_t st = smem_u32(smem + (size_t)s * stage_bytes);
+                const uint64_t st = desc0 + (uint64_t)(((uint32_t)s * stage_bytes) >> 4);
 #pragma unroll
                 for (int ks = 0; ks < TC_BK / 8; ++ks) {
-                    // MN-major 32-bit operands use the 128-byte swizzle with 32-byte atoms (the only layout the tensor core
-                    // accepts for them): 32-column blocks blk_bytes apart (leading offset), groups of 4 k-rows 512 B apart
-                    // (stride offset); a k-step is 8 rows = 1024 B
-                    const uint32_t koff = ks * 1024;
-                    const uint64_t a_hi = make_desc(st + koff, blk_bytes, 512, 1);
-                    const uint64_t a_lo = make_desc(st + a_bytes + koff, blk_bytes, 512, 1);
-                    const uint64_t b_hi = make_desc(st + 2 * a_bytes + koff, blk_bytes, 512, 1);
-                    const uint64_t b_lo = make_desc(st + 2 * a_bytes + b_bytes + koff, blk_bytes, 512, 1);
-                    tc_mma(tmem, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-                    tc_mma(tmem, a_hi, b_lo, idesc, 1u);
-                    tc_mma(tmem, a_lo, b_hi, idesc, 1u);
+                    const uint64_t b_hi = st + (uint64_t)((2 * a_bytes + ks * 1024) >> 4), b_lo = b_hi + (b_bytes >> 4);
+                    for (int i = 0; i < mt; ++i) {
+                        const uint64_t a_hi = st + (uint64_t)(((uint32_t)i * sub_bytes + ks * 1024) >> 4), a_lo = a_hi + (a_bytes >> 4);
+                        const uint32_t acc = tmem + (uint32_t)i * 256u;
+                        tc_mma(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                        tc_mma(acc, a_hi, b_lo, idesc, 1u);
+                        tc_mma(acc, a_lo, b_hi, idesc, 1u);
+                    }
                 }
                 tc_commit(&sh->empty[s]);
             }
@@ -813,51 +805,65 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     } else {
         const int ctid = threadIdx.x - 64;
         const bool want_cs = part_cs != nullptr && blockIdx.x == 0;
-        float4 cs[8];   // this thread's share of the column sums: one 16-byte piece of every 32-column block, row ctid / 8 of each k-block
+        // thread t takes 16-byte piece t % 128 of every second 32-column block; row (t % 128) / 8 of each k-block
+        const uint32_t off = (uint32_t)(ctid & 127) * 16, half = (uint32_t)(ctid >> 7);
+        float4 cs[4];
 #pragma unroll
-        for (int bl = 0; bl < 8; ++bl) cs[bl] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < 4; ++i) cs[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         bool alive = true;
         for (int32_t kb = 0; kb < nkb && alive; ++kb) {
             const int s = kb % stages;
             const uint32_t ph = (uint32_t)(kb / stages) & 1u;
             alive = mbar_wait(&sh->full[s], ph, dead, status);
             if (!alive) break;
-            uint8_t *st = smem + (size_t)s * stage_bytes;
-            split_tile_round(st, st + a_bytes, a_bytes, ctid, TC_CONV_THREADS);
-            if (!want_cs) {
-                split_tile_round(st + 2 * a_bytes, st + 2 * a_bytes + b_bytes, b_bytes, ctid, TC_CONV_THREADS);
-            } else {
-                uint8_t *bh = st + 2 * a_bytes + ctid * 16, *bl_ = bh + b_bytes;
+            uint8_t *ah = smem + (size_t)s * stage_bytes + off + half * blk_bytes, *bh = ah + 2 * a_bytes;
+            float4 x[4];
+            // loads first, four 16-byte pieces at a time (the loop is latency-bound otherwise)
 #pragma unroll
-                for (int bl = 0; bl < 8; ++bl) {
-                    if (bl < n_blks_b) {
-                        const float4 x = *reinterpret_cast<const float4 *>(bh + bl * blk_bytes);
-                        float4 h, l;
-                        split4(x, h, l);
-                        *reinterpret_cast<float4 *>(bh + bl * blk_bytes) = h;
-                        *reinterpret_cast<float4 *>(bl_ + bl * blk_bytes) = l;
-                        cs[bl].x += x.x;
-                        cs[bl].y += x.y;
-                        cs[bl].z += x.z;
-                        cs[bl].w += x.w;
-                    }
+            for (int i = 0; i < 4; ++i)
+                if ((int)half + 2 * i < n_blks_b) x[i] = *reinterpret_cast<const float4 *>(bh + 2 * i * blk_bytes);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if ((int)half + 2 * i < n_blks_b) {
+                    float4 h, l;
+                    split4(x[i], h, l);
+                    *reinterpret_cast<float4 *>(bh + 2 * i * blk_bytes) = h;
+                    *reinterpret_cast<float4 *>(bh + 2 * i * blk_bytes + b_bytes) = l;
+                    cs[i].x += x[i].x;
+                    cs[i].y += x[i].y;
+                    cs[i].z += x[i].z;
+                    cs[i].w += x[i].w;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < 2 * mt) x[i] = *reinterpret_cast<const float4 *>(ah + 2 * i * blk_bytes);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i < 2 * mt) {
+                    float4 h, l;
+                    split4(x[i], h, l);
+                    *reinterpret_cast<float4 *>(ah + 2 * i * blk_bytes) = h;
+                    *reinterpret_cast<float4 *>(ah + 2 * i * blk_bytes + a_bytes) = l;
                 }
             }
             fence_async_smem();
             mbar_arrive(&sh->conv[s]);
         }
-        const int q = warp & 3;
+        const int q = warp & 3, e = (warp - 2) >> 2;
         const bool ok = alive && mbar_wait(&sh->accum, 0, dead, status);   // every MMA has completed: the stages are free
         tc_fence_after();
         if (ok) {
-            // each warp turns its 32 x 32 block around in shared memory and writes whole row segments: with one row per lane a store
-            // instruction touched 32 lines, and the partial sums of a tile took 35 us
-            float *tb = reinterpret_cast<float *>(smem) + q * (32 * 33);
+            // two warps per TMEM lane quadrant: one per sub-tile, or alternate chunks of the only one.  Each turns its 32 x 32 blocks
+            // around in shared memory and writes whole row segments: with one row per lane a store instruction touched 32 lines, and
+            // the partial sums of a tile took 35 us
+            float *tb = reinterpret_cast<float *>(smem) + (warp - 2) * (32 * 33);
             float *pc = part_C + (int64_t)blockIdx.z * Mdim * N;
-            const int32_t row0 = m0 + q * 32;
-            for (int c0 = 0; c0 < bn; c0 += 32) {
+            const int sub = mt > 1 ? e : 0;
+            const int32_t row0 = m0 + sub * TC_BM + q * 32;
+            for (int c0 = mt > 1 ? 0 : 32 * e; c0 < bn; c0 += mt > 1 ? 32 : 64) {
                 uint32_t r[32];
-                tc_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
+                tc_ld32(tmem + (uint32_t)sub * 256u + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < 32; ++j) tb[lane * 33 + j] = __uint_as_float(r[j]);
@@ -872,14 +878,16 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
         }
         if (want_cs) {
             // the 16 rows of a k-block lie in 16 groups of eight threads; the 32-byte atoms of a row are exchanged by its low two bits
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            asm volatile("bar.sync 1, 256;" ::: "memory");
             float *cb = reinterpret_cast<float *>(smem);   // [16][n_blks_b * 32]
-            const int rr = ctid >> 3, piece = (ctid & 7) ^ ((rr & 3) << 1), w = n_blks_b * 32;
+            const int rr = (ctid & 127) >> 3, piece = (ctid & 7) ^ ((rr & 3) << 1), w = n_blks_b * 32;
 #pragma unroll
-            for (int bl = 0; bl < 8; ++bl)
-                if (bl < n_blks_b && ok) *reinterpret_cast<float4 *>(cb + rr * w + bl * 32 + piece * 4) = cs[bl];
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            for (int c = ctid; c < w; c += TC_CONV_THREADS) {
+            for (int i = 0; i < 4; ++i) {
+                const int bl = (int)half + 2 * i;
+                if (bl < n_blks_b && ok) *reinterpret_cast<float4 *>(cb + rr * w + bl * 32 + piece * 4) = cs[i];
+            }
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            for (int c = ctid; c < w; c += MN_CONV_THREADS) {
                 float t = cb[c];
                 for (int g = 1; g < 16; ++g) t += cb[g * w + c];
                 if (n0 + c < N && c < bn) part_cs[(int64_t)blockIdx.z * N + n0 + c] = t;
@@ -890,7 +898,7 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)tmem_cols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
     }
 }
 
@@ -1046,8 +1054,12 @@ static sat_status make_map(sat_ctx *ctx, CUtensorMap *map, const void *base, int
     return SAT_OK;
 }
 
-static int tmem_cols_for(int bn) { return bn <= 32 ? 32 : bn <= 64 ? 64 : bn <= 128 ? 128 : 256; }
-static int tile_n_for(int n) { return n >= 256 ? 256 : (n + 31) / 32 * 32; }
+// output columns per tile: as few tiles of at most 256 as possible, of equal width (a multiple of 32)
+static int tile_n_for(int n)
+{
+    const int tiles = (n + 255) / 256;
+    return ((n + tiles - 1) / tiles + 31) / 32 * 32;
+}
 
 bool sat_use_tc(int32_t n, int32_t k)
 {
@@ -1116,7 +1128,6 @@ sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeig
 }
 
 static PerDeviceOnce g_attr_mn;
-#define TC_SMEM_BUDGET (100 * 1024)
 
 struct TckLaunch {
     CUtensorMap mA, mA2, mB, mBlo, mC;
@@ -1227,25 +1238,23 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
 {
     if (m == 0 || n == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_GEMM_TN, 4.0 * ((double)rows * (m + n) + (double)m * n), 2.0 * (double)rows * m * n);
-    const int32_t bn = tile_n_for(n);
-    const int n_blks_b = (bn + 31) / 32;
-    const uint32_t stage_bytes = 2 * ((TC_BM / 32) * TC_BK * 128) + 2 * (uint32_t)n_blks_b * TC_BK * 128;
-    int stages = (int)(TC_SMEM_BUDGET / stage_bytes);
-    if (stages > 4) stages = 4;
-    if (stages < 2) stages = 2;
-    const size_t smem = (size_t)stages * stage_bytes + sizeof(TcShared) + 1024;
-    const int64_t tiles = cdiv64(m, TC_BM) * cdiv64(n, bn);
-    // Two CTAs fit on an SM: one wave of 2 x 148 for tall inputs.  Below ~100 k-blocks per CTA of such a wave, half as many splits: the
-    // m x n partial sums of a split cost as much as ~10 of its k-blocks (21 k rows, 256 x 256: 65 us with 148 splits of the old store,
-    // see the epilogue)
-    const int64_t kblocks = cdiv64(rows > 0 ? rows : 1, TC_BK);
-    int64_t splits = (2 * 148 + tiles - 1) / tiles;
-    if (kblocks < 40 * splits) splits = (148 + tiles - 1) / tiles;
-    const int64_t max_splits = cdiv64(rows > 0 ? rows : 1, 8 * TC_BK);
-    if (splits > max_splits) splits = max_splits;
-    if (splits < 1) splits = 1;
-    const int64_t rps = cdiv64(cdiv64(rows > 0 ? rows : 1, splits), TC_BK) * TC_BK;
-    splits = cdiv64(rows > 0 ? rows : 1, rps);
+    const int32_t bn = tile_n_for(n), mt = m > TC_BM ? 2 : 1;
+    const uint32_t stage_bytes = 2 * (uint32_t)mt * (TC_BM / 32) * TC_BK * 128 + 2 * (uint32_t)((bn + 31) / 32) * TC_BK * 128;
+    const int64_t r1 = rows > 0 ? rows : 1, kblocks = cdiv64(r1, TC_BK);
+    // One wave: a CTA per SM, or two where the tile is 128 columns of A (256 of the 512 TMEM columns each; the shorter chains also keep
+    // the truncating accumulation error down).  Not less than six k-blocks each: the m x n partial sums of a split, written and read
+    // again, cost about as much as that.
+    const int per_sm = mt == 1 ? 2 : 1;
+    const int64_t tiles = cdiv64(m, mt * TC_BM) * cdiv64(n, bn);
+    int64_t splits = tiles < 148 * per_sm ? 148 * per_sm / tiles : 1;
+    if (splits > cdiv64(kblocks, 6)) splits = cdiv64(kblocks, 6);
+    const int64_t kpb = cdiv64(kblocks, splits), rps = kpb * TC_BK;
+    splits = cdiv64(r1, rps);
+    int64_t stages = (MN_SMEM_MAX / per_sm - 1024 - (int)sizeof(MnShared) - 1024) / stage_bytes;
+    if (stages > MN_STAGES_MAX) stages = MN_STAGES_MAX;
+    if (stages > kpb) stages = kpb;
+    const size_t need = (size_t)stages * stage_bytes, turn = MN_TURN_BYTES;
+    const size_t smem = (need > turn ? need : turn) + sizeof(MnShared) + 1024;
     SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)splits * ((size_t)m * n + n) * sizeof(float)));
     float *part = (float *)ctx->buf_splitk.p;
     float *part_cs = colsum ? part + (size_t)splits * m * n : nullptr;
@@ -1253,11 +1262,12 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
     SAT_TRY(make_map(ctx, &mA, A, m, rows, lda, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
     SAT_TRY(make_map(ctx, &mB, B, n, rows, ldb, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
     if (g_attr_mn.need(ctx->device)) {
-        SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_mn, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024));
+        SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_mn, cudaFuncAttributeMaxDynamicSharedMemorySize, MN_SMEM_MAX));
         g_attr_mn.mark(ctx->device);
     }
-    dim3 grid((unsigned)cdiv64(m, TC_BM), (unsigned)cdiv64(n, bn), (unsigned)splits);
-    k_gemm_tc_mn<<<grid, TC_THREADS, smem, ctx->stream>>>(mA, mB, m, n, rps, bn, stages, tmem_cols_for(bn), part, part_cs, ctx->d_flag + 1);
+    dim3 grid((unsigned)cdiv64(m, mt * TC_BM), (unsigned)cdiv64(n, bn), (unsigned)splits);
+    k_gemm_tc_mn<<<grid, MN_THREADS, smem, ctx->stream>>>(mA, mB, m, n, rps, r1, mt, bn, (int32_t)stages, mt == 1 ? 256u : 512u, part, part_cs,
+                                                       ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
     return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, part_cs, n, colsum);
 }
