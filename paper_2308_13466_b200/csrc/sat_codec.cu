@@ -91,6 +91,7 @@ __device__ __forceinline__ Q codec_scan(Q x, int lane, Q *total)
 __global__ void __launch_bounds__(256)
 k_codec_sizes(const float *__restrict__ x, int64_t ld, int64_t rows, int32_t d, int vec, float scale32, double scale, int32_t *__restrict__ row_bytes)
 {
+    sat_grid_wait();
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (r >= rows) return;
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(256)
 k_codec_encode(const float *__restrict__ x, int64_t ld, int64_t rows, int32_t d, int vec, float scale32, double scale,
                const int64_t *__restrict__ offsets, uint8_t *__restrict__ out)
 {
+    sat_grid_wait();
     __shared__ __align__(16) uint8_t bufs[8][CODEC_BUF + 16];
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -254,6 +256,7 @@ __global__ void __launch_bounds__(256)
 k_codec_decode(const uint8_t *__restrict__ in, int64_t in_bytes, const int64_t *__restrict__ offsets, int64_t rows, int32_t d, float scale32,
                double scale, float *__restrict__ x, int64_t ld, int *__restrict__ status)
 {
+    sat_grid_wait();
     __shared__ __align__(16) uint8_t wins[8][16 + CODEC_WIN + 16];   // the last 16 bytes of the window before, the window (63 subtracted)
     __shared__ uint16_t lists[8][CODEC_WIN];
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -395,7 +398,7 @@ static sat_status codec_plan(sat_ctx *ctx, const float *x, int32_t ld, int64_t r
     int32_t *sizes = (int32_t *)ctx->buf_codec_sizes.p;
     if (rows > 0) {
         ProfScope prof(ctx, SATK_CODEC, 4.0 * (double)rows * d + 12.0 * (double)rows, 0.0);
-        k_codec_sizes<<<(unsigned)cdiv64(rows * 32, 256), 256, 0, ctx->stream>>>(x, ld, rows, d, codec_vec(x, ld), (float)codec_scale(precision),
+        sat_pdl(ctx->stream, k_codec_sizes, (unsigned)cdiv64(rows * 32, 256), 256, 0)(x, ld, rows, d, codec_vec(x, ld), (float)codec_scale(precision),
                                                                              codec_scale(precision), sizes);
         SAT_LAUNCHED(ctx);
     }
@@ -420,7 +423,7 @@ static sat_status codec_encode(sat_ctx *ctx, const float *x, int32_t ld, int64_t
 {
     if (rows == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_CODEC, 4.0 * (double)rows * d + 8.0 * (double)rows + (double)total, 0.0);
-    k_codec_encode<<<(unsigned)cdiv64(rows * 32, 256), 256, 0, ctx->stream>>>(x, ld, rows, d, codec_vec(x, ld), (float)codec_scale(precision), codec_scale(precision),
+    sat_pdl(ctx->stream, k_codec_encode, (unsigned)cdiv64(rows * 32, 256), 256, 0)(x, ld, rows, d, codec_vec(x, ld), (float)codec_scale(precision), codec_scale(precision),
                                                                              row_offsets, out);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -444,7 +447,7 @@ static sat_status codec_decode(sat_ctx *ctx, const uint8_t *in, int64_t in_bytes
 {
     if (rows == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_CODEC, 4.0 * (double)rows * d + 8.0 * (double)rows + (double)in_bytes, 0.0);
-    k_codec_decode<<<(unsigned)cdiv64(rows * 32, 256), 256, 0, ctx->stream>>>(in, in_bytes, row_offsets, rows, d, (float)codec_scale(precision), codec_scale(precision), x, ld,
+    sat_pdl(ctx->stream, k_codec_decode, (unsigned)cdiv64(rows * 32, 256), 256, 0)(in, in_bytes, row_offsets, rows, d, (float)codec_scale(precision), codec_scale(precision), x, ld,
                                                                              ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
     return SAT_OK;

@@ -338,6 +338,7 @@ extern "C" sat_status sat_profile_read(sat_ctx *ctx, int32_t family, const char 
 
 __global__ void k_scan_tile_sums(const int32_t *__restrict__ in, int64_t count, int64_t *__restrict__ tile_sum)
 {
+    sat_grid_wait();
     __shared__ long long red[SCAN_THREADS];
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     long long s = 0;
@@ -357,6 +358,7 @@ __global__ void k_scan_tile_sums(const int32_t *__restrict__ in, int64_t count, 
 // single block: exclusive scan of the tile sums in place (serial over chunks, tiny)
 __global__ void k_scan_tile_offsets(int64_t *tile_sum, int64_t n_tiles, int64_t *total)
 {
+    sat_grid_wait();
     __shared__ long long sh[SCAN_THREADS];
     __shared__ long long carry;
     if (threadIdx.x == 0) carry = 0;
@@ -384,6 +386,7 @@ __global__ void k_scan_tile_offsets(int64_t *tile_sum, int64_t n_tiles, int64_t 
 __global__ void k_scan_write(const int32_t *__restrict__ in, int64_t count, const int64_t *__restrict__ tile_off,
                              int64_t *__restrict__ out)
 {
+    sat_grid_wait();
     // each thread owns SCAN_TILE / SCAN_THREADS consecutive elements
     const int PER = SCAN_TILE / SCAN_THREADS;
     __shared__ long long sh[SCAN_THREADS];
@@ -418,11 +421,11 @@ sat_status sat_scan_i32(sat_ctx *ctx, const int32_t *in, int64_t count, int64_t 
     int64_t n_tiles = cdiv64(count > 0 ? count : 1, SCAN_TILE);
     SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)(n_tiles + 1) * sizeof(int64_t)));
     int64_t *tiles = (int64_t *)ctx->buf_misc.p;
-    k_scan_tile_sums<<<(unsigned)n_tiles, SCAN_THREADS, 0, ctx->stream>>>(in, count, tiles);
+    sat_pdl(ctx->stream, k_scan_tile_sums, (unsigned)n_tiles, SCAN_THREADS, 0)(in, count, tiles);
     SAT_LAUNCHED(ctx);
-    k_scan_tile_offsets<<<1, SCAN_THREADS, 0, ctx->stream>>>(tiles, n_tiles, out + count);
+    sat_pdl(ctx->stream, k_scan_tile_offsets, 1, SCAN_THREADS, 0)(tiles, n_tiles, out + count);
     SAT_LAUNCHED(ctx);
-    k_scan_write<<<(unsigned)n_tiles, SCAN_THREADS, 0, ctx->stream>>>(in, count, tiles, out);
+    sat_pdl(ctx->stream, k_scan_write, (unsigned)n_tiles, SCAN_THREADS, 0)(in, count, tiles, out);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }

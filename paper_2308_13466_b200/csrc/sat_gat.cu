@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(256)
 k_gat_scores(const float *__restrict__ z, int64_t ld, int64_t rows, int32_t d, const float *__restrict__ a_src, const float *__restrict__ a_dst,
              float *__restrict__ s_src, float *__restrict__ s_dst)
 {
+    sat_grid_wait();
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (r >= rows) return;
@@ -139,6 +140,7 @@ k_gat_alpha(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ len
             const int32_t *__restrict__ long_rows, int32_t n_long, const float *__restrict__ s_in, const float *__restrict__ s_halo,
             const float *__restrict__ s_dst, int2 *__restrict__ ent)
 {
+    sat_grid_wait();
     __shared__ float sh[8];
     if ((int32_t)blockIdx.x < n_long) {
         const int32_t row = long_rows[blockIdx.x];
@@ -161,6 +163,7 @@ __global__ void __launch_bounds__(256, NV <= 2 ? 3 : NV <= 4 ? 2 : 1)
 k_gat_dots(const int4 *__restrict__ items, int32_t n_items, const int32_t *__restrict__ lenc, int32_t n, int32_t d4, const float *__restrict__ z_in,
            const float *__restrict__ z_halo, uint32_t ldz4, const float *__restrict__ D, double *__restrict__ dots)
 {
+    sat_grid_wait();
     const int lane = threadIdx.x & (G - 1);
     const int64_t gid = ((int64_t)blockIdx.x * 256 + threadIdx.x) / G;
     if (gid >= n_items) return;
@@ -255,6 +258,7 @@ k_gat_rows(const int64_t *__restrict__ lrowptr, const int2 *__restrict__ ent, in
            int32_t n_long, const float *__restrict__ s_in, const float *__restrict__ s_halo, const float *__restrict__ s_dst, double *dots,
            float *__restrict__ ds_dst)
 {
+    sat_grid_wait();
     __shared__ double sh[8];
     if ((int32_t)blockIdx.x < n_long) {
         const int32_t row = long_rows[blockIdx.x];
@@ -290,6 +294,7 @@ k_gat_cols(const int64_t *__restrict__ ptr, const int32_t *__restrict__ cnt, int
            const int32_t *__restrict__ idx, const uint32_t *__restrict__ map, const float2 *__restrict__ edge, int2 *__restrict__ ent_out,
            float *__restrict__ ds_src)
 {
+    sat_grid_wait();
     __shared__ double sh[8];
     if ((int32_t)blockIdx.x < n_long) {
         const int32_t u = long_u[blockIdx.x];
@@ -351,6 +356,7 @@ __global__ void __launch_bounds__(256)
 k_gat_wcolsum(const float *__restrict__ x, int64_t ld, int64_t rows, int32_t d, int32_t tpr, const float *__restrict__ w1, const float *__restrict__ w2,
               float *__restrict__ part1, float *__restrict__ part2)
 {
+    sat_grid_wait();
     __shared__ float4 red[2][256];
     const int c4 = threadIdx.x % tpr, rg = threadIdx.x / tpr, n_rg = 256 / tpr, d4 = (d + 3) >> 2;
     const int64_t r0 = (int64_t)blockIdx.x * GAT_WSUM_ROWS, r1 = r0 + GAT_WSUM_ROWS < rows ? r0 + GAT_WSUM_ROWS : rows;
@@ -455,7 +461,7 @@ static sat_status gat_wcolsum(sat_ctx *ctx, const float *x, int32_t ld, int64_t 
     float *p1 = (float *)ctx->buf_colsum.p, *p2 = w2 ? p1 + (size_t)blocks * d : nullptr;
     int tpr = 1;
     while (tpr < (d + 3) / 4) tpr <<= 1;   // d <= 1024: at most 256
-    k_gat_wcolsum<<<(unsigned)blocks, 256, 0, ctx->stream>>>(x, ld, rows, d, tpr, w1, w2, p1, p2);
+    sat_pdl(ctx->stream, k_gat_wcolsum, (unsigned)blocks, 256, 0)(x, ld, rows, d, tpr, w1, w2, p1, p2);
     SAT_LAUNCHED(ctx);
     return sat_splitk_reduce(ctx, p1, d, (int32_t)blocks, accumulate, out1, d, d, p2, d, out2);
 }
@@ -545,18 +551,18 @@ extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int
     SAT_TRY(gat_nn(ctx, v.n_halo, d_out, d_in, h_halo, ld_halo, W, z_halo + v.halo0 * ld_z, ld_z));
     ProfScope prof(ctx, SATK_GAT, 0.0, 0.0);
     if (v.n_rows > 0) {
-        k_gat_scores<<<(unsigned)cdiv64((int64_t)v.n_rows * 32, 256), 256, 0, ctx->stream>>>(z_in + (int64_t)v.row0 * ld_z, ld_z, v.n_rows, d_out, a_src, a_dst,
+        sat_pdl(ctx->stream, k_gat_scores, (unsigned)cdiv64((int64_t)v.n_rows * 32, 256), 256, 0)(z_in + (int64_t)v.row0 * ld_z, ld_z, v.n_rows, d_out, a_src, a_dst,
                                                                                            s_in + v.row0, s_dst + v.row0);
         SAT_LAUNCHED(ctx);
     }
     if (v.n_halo > 0) {
-        k_gat_scores<<<(unsigned)cdiv64(v.n_halo * 32, 256), 256, 0, ctx->stream>>>(z_halo + v.halo0 * ld_z, ld_z, v.n_halo, d_out, a_src, nullptr,
+        sat_pdl(ctx->stream, k_gat_scores, (unsigned)cdiv64(v.n_halo * 32, 256), 256, 0)(z_halo + v.halo0 * ld_z, ld_z, v.n_halo, d_out, a_src, nullptr,
                                                                                   s_halo + v.halo0, nullptr);
         SAT_LAUNCHED(ctx);
     }
     if (v.n_rows > 0) {
         const int64_t l0 = ctx->h_gat_long_off[v.p0], n_long = ctx->h_gat_long_off[v.p1] - l0;
-        k_gat_alpha<<<(unsigned)(n_long + cdiv64((int64_t)v.n_rows * GAT_TEAM, 256)), 256, 0, ctx->stream>>>(
+        sat_pdl(ctx->stream, k_gat_alpha, (unsigned)(n_long + cdiv64((int64_t)v.n_rows * GAT_TEAM, 256)), 256, 0)(
             ctx->lrowptr, ctx->lenc, ctx->n, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, s_in, s_halo, s_dst, (int2 *)G.ent.p);
         SAT_LAUNCHED(ctx);
         SpmmEpilogue ep;
@@ -635,7 +641,7 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
         int64_t n_items = 0;
         SAT_TRY(sat_spmm_items(ctx, v, 0, d_out, &items, &n_items));
 #define CALL(GG, NV)                                                                                                                            \
-    k_gat_dots<GG, NV><<<(unsigned)cdiv64(n_items * GG, 256), 256, 0, ctx->stream>>>(items, (int32_t)n_items, ctx->lenc, ctx->n, d4, z_in, z_halo, \
+    sat_pdl(ctx->stream, k_gat_dots<GG, NV>, (unsigned)cdiv64(n_items * GG, 256), 256, 0)(items, (int32_t)n_items, ctx->lenc, ctx->n, d4, z_in, z_halo, \
                                                                                      (uint32_t)(ld_z / 4), Db, dots_b)
         if (d4 <= 8) CALL(8, 1);
         else if (d4 <= 16) CALL(16, 1);
@@ -647,10 +653,10 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
         SAT_LAUNCHED(ctx);
         const int64_t l0 = ctx->h_gat_long_off[v.p0], n_long = ctx->h_gat_long_off[v.p1] - l0;
         const unsigned grid = (unsigned)(n_long + cdiv64((int64_t)v.n_rows * GAT_TEAM, 256));
-        k_gat_rows<<<grid, 256, 0, ctx->stream>>>(ctx->lrowptr, (const int2 *)G.ent.p, ctx->n, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, s_in,
+        sat_pdl(ctx->stream, k_gat_rows, grid, 256, 0)(ctx->lrowptr, (const int2 *)G.ent.p, ctx->n, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, s_in,
                                                   s_halo, s_dst, dots_b, ds_dst_b);
         SAT_LAUNCHED(ctx);
-        k_gat_cols<<<grid, 256, 0, ctx->stream>>>(ctx->lrowptr, ctx->inner_cnt, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, ctx->lenc,
+        sat_pdl(ctx->stream, k_gat_cols, grid, 256, 0)(ctx->lrowptr, ctx->inner_cnt, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, ctx->lenc,
                                                   ctx->gat_rev, (const float2 *)dots_b, ent_in_b, ds_in_b);
         SAT_LAUNCHED(ctx);
         SpmmEpilogue ep;
@@ -664,7 +670,7 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
     }
     if (v.n_halo > 0 && v.n_rows > 0) {
         ProfScope prof(ctx, SATK_GAT, 0.0, 0.0);
-        k_gat_cols<<<(unsigned)(v.n_hlong + cdiv64(v.n_halo * GAT_TEAM, 256)), 256, 0, ctx->stream>>>(
+        sat_pdl(ctx->stream, k_gat_cols, (unsigned)(v.n_hlong + cdiv64(v.n_halo * GAT_TEAM, 256)), 256, 0)(
             ctx->hrow_ptr, nullptr, v.halo0, v.n_halo, ctx->hlong ? ctx->hlong + v.hlong0 : nullptr, v.n_hlong, ctx->hrow_pos, ctx->gat_hmap,
             (const float2 *)dots_b, ent_halo_b, ds_halo_b);
         SAT_LAUNCHED(ctx);

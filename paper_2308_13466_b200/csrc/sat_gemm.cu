@@ -33,6 +33,7 @@ k_gemm_nn(int64_t m, int32_t n, int32_t k1, const float *__restrict__ A, int64_t
           float *__restrict__ C, int64_t ldc, const float *__restrict__ bias, int relu, uint32_t *__restrict__ mask_out,
           int32_t mask_words, const float *__restrict__ resid, const int32_t *__restrict__ resid_idx, int64_t ld_resid)
 {
+    sat_grid_wait();
     // the contraction runs over the virtual concatenation [A | A2] [B ; B2] (k2 may be 0)
     const int32_t k = k1 + k2;
     __shared__ float As[BK][BM + 4];
@@ -101,7 +102,7 @@ sat_status sat_gemm_nn(sat_ctx *ctx, int64_t m, int32_t n, int32_t k, const floa
     if (m == 0 || n == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_GEMM_NN, 4.0 * ((double)m * (k + n) + (double)k * n), 2.0 * (double)m * n * k);
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN));
-    k_gemm_nn<<<grid, 256, 0, ctx->stream>>>(m, n, k, A, lda, B, ldb, 0, nullptr, 0, nullptr, 0, C, ldc, ep.bias, ep.relu, ep.mask_out,
+    sat_pdl(ctx->stream, k_gemm_nn, grid, 256, 0)(m, n, k, A, lda, B, ldb, 0, nullptr, 0, nullptr, 0, C, ldc, ep.bias, ep.relu, ep.mask_out,
                                              ep.mask_words, ep.resid, ep.resid_idx, ep.ld_resid);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -114,7 +115,7 @@ sat_status sat_gemm_nn_dual(sat_ctx *ctx, int64_t m, int32_t n, int32_t k1, cons
     if (m == 0 || n == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_GEMM_NN, 4.0 * ((double)m * (k1 + k2 + n) + (double)(k1 + k2) * n), 2.0 * (double)m * n * (k1 + k2));
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN));
-    k_gemm_nn<<<grid, 256, 0, ctx->stream>>>(m, n, k1, A1, lda1, B1, ldb1, k2, A2, lda2, B2, ldb2, C, ldc, bias, 0, nullptr, 0, nullptr,
+    sat_pdl(ctx->stream, k_gemm_nn, grid, 256, 0)(m, n, k1, A1, lda1, B1, ldb1, k2, A2, lda2, B2, ldb2, C, ldc, bias, 0, nullptr, 0, nullptr,
                                              nullptr, 0);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -124,6 +125,7 @@ __global__ void __launch_bounds__(256)
 k_gemm_nt(int64_t m, int32_t n, int32_t k, const float *__restrict__ A, int64_t lda, const uint32_t *__restrict__ mask,
           int32_t mask_words, const float *__restrict__ B, int64_t ldb, float *__restrict__ C, int64_t ldc)
 {
+    sat_grid_wait();
     __shared__ float As[BK][BM + 4];
     __shared__ float Bs[BK][BN + 4];
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -174,7 +176,7 @@ sat_status sat_gemm_nt(sat_ctx *ctx, int64_t m, int32_t n, int32_t k, const floa
     if (m == 0 || n == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_GEMM_NT, 4.0 * ((double)m * (k + n) + (double)k * n), 2.0 * (double)m * n * k);
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN));
-    k_gemm_nt<<<grid, 256, 0, ctx->stream>>>(m, n, k, A, lda, mask, mask_words, B, ldb, C, ldc);
+    sat_pdl(ctx->stream, k_gemm_nt, grid, 256, 0)(m, n, k, A, lda, mask, mask_words, B, ldb, C, ldc);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
@@ -186,6 +188,7 @@ k_gemm_tn(int64_t rows, int64_t rows_per_split, int32_t m, int32_t n, const floa
           const float *__restrict__ B, int64_t ldb, const uint32_t *__restrict__ mask, int32_t mask_words,
           float *__restrict__ part_C /* [splits x m x n] */, float *__restrict__ part_cs /* [splits x n] or null */)
 {
+    sat_grid_wait();
     __shared__ float As[BK][BM + 4];
     __shared__ float Bs[BK][BN + 4];
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -250,6 +253,7 @@ __global__ void __launch_bounds__(256)
 k_splitk_reduce(const float *__restrict__ part, int64_t count, int32_t splits, int accumulate, float *__restrict__ out,
                 int32_t ncols, int64_t ld_out, int64_t blocks1, const float *__restrict__ part2, int64_t count2, float *__restrict__ out2)
 {
+    sat_grid_wait();
     __shared__ float red[8][32];
     const int o = threadIdx.x & 31, zl = threadIdx.x >> 5;
     int64_t blk = blockIdx.x;
@@ -290,7 +294,7 @@ sat_status sat_splitk_reduce(sat_ctx *ctx, const float *part, int64_t count, int
 {
     if (count == 0) return SAT_OK;
     const int64_t b1 = cdiv64(count, 32), b2 = out2 ? cdiv64(count2, 32) : 0;
-    k_splitk_reduce<<<(unsigned)(b1 + b2), 256, 0, ctx->stream>>>(part, count, splits, accumulate, out, ncols, ld_out, b1, part2, count2, out2);
+    sat_pdl(ctx->stream, k_splitk_reduce, (unsigned)(b1 + b2), 256, 0)(part, count, splits, accumulate, out, ncols, ld_out, b1, part2, count2, out2);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
@@ -312,7 +316,7 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
     float *part_C = (float *)ctx->buf_splitk.p;
     float *part_cs = colsum ? part_C + (size_t)splits * m * n : nullptr;
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN), (unsigned)splits);
-    k_gemm_tn<<<grid, 256, 0, ctx->stream>>>(rows, rows_per_split, m, n, A, lda, B, ldb, mask, mask_words, part_C, part_cs);
+    sat_pdl(ctx->stream, k_gemm_tn, grid, 256, 0)(rows, rows_per_split, m, n, A, lda, B, ldb, mask, mask_words, part_C, part_cs);
     SAT_LAUNCHED(ctx);
     return sat_splitk_reduce(ctx, part_C, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, part_cs, n, colsum);
 }
@@ -342,6 +346,7 @@ __global__ void __launch_bounds__(128)
 k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, const float *__restrict__ A, int64_t lda,
                  const float *__restrict__ B, int64_t ldb, float *__restrict__ part, float *__restrict__ part_cs)
 {
+    sat_grid_wait();
     extern __shared__ __align__(16) float tnn_smem[];
     constexpr int MC = 64 * TM, NH = NT / 2, STAGE_FLOATS = TNN_STAGE * (MC + NT);
     // column sums of B (the bias gradient), by the blocks with y == 0: thread t takes column t % NT of every (128 / NT)-th staged row
@@ -465,7 +470,7 @@ static sat_status launch_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_
     SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)blocks * ((size_t)m * n + n) * sizeof(float)));
     float *part = (float *)ctx->buf_splitk.p;
     float *part_cs = colsum ? part + (size_t)blocks * m * n : nullptr;
-    k_gemm_tn_narrow<NT, TM><<<dim3((unsigned)blocks, (unsigned)yb), 128, smem, ctx->stream>>>(rows, rpb, m, n, A, lda, B, ldb, part, part_cs);
+    sat_pdl(ctx->stream, k_gemm_tn_narrow<NT, TM>, dim3((unsigned)blocks, (unsigned)yb), 128, smem)(rows, rpb, m, n, A, lda, B, ldb, part, part_cs);
     SAT_LAUNCHED(ctx);
     return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)blocks, accumulate, C, n, ldc, part_cs, n, colsum);
 }
@@ -562,11 +567,11 @@ extern "C" sat_status sat_dense_tn_static(void *cuda_stream, int64_t rows, int32
     // every element of the `splits` partial blocks is written by exactly one thread block below, so nothing left over from
     // an earlier call is ever read and no clearing is needed
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN), (unsigned)splits);
-    k_gemm_tn<<<grid, 256, 0, st>>>(rows, rows_per_split, m, n, A, lda, B, ldb, nullptr, 0, scratch, nullptr);
+    sat_pdl(st, k_gemm_tn, grid, 256, 0)(rows, rows_per_split, m, n, A, lda, B, ldb, nullptr, 0, scratch, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return static_fail(errbuf, errbuf_len, SAT_ECUDA, "sat_dense_tn_static: launch failed (%s)", cudaGetErrorString(e));
     const int64_t b1 = cdiv64((int64_t)m * n, 32);
-    k_splitk_reduce<<<(unsigned)b1, 256, 0, st>>>(scratch, (int64_t)m * n, (int32_t)splits, 0, C, n, n, b1, nullptr, 0, nullptr);
+    sat_pdl(st, k_splitk_reduce, (unsigned)b1, 256, 0)(scratch, (int64_t)m * n, (int32_t)splits, 0, C, n, n, b1, nullptr, 0, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return static_fail(errbuf, errbuf_len, SAT_ECUDA, "sat_dense_tn_static: launch failed (%s)", cudaGetErrorString(e));
     return SAT_OK;

@@ -325,6 +325,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
     volatile int *dead = &sh->dead;
+    sat_grid_wait();   // everything above is set-up of this block; no global memory has been touched
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -759,6 +760,7 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
     volatile int *dead = &sh->dead;
+    sat_grid_wait();   // everything above is set-up of this block; no global memory has been touched
 
     if (warp == 0) {
         if (lane == 0) {
@@ -915,6 +917,7 @@ k_mask_rows(const float *__restrict__ src, int64_t ld, int64_t rows, int32_t d, 
             int32_t mask_words, const float *__restrict__ act, int64_t ld_act, int act_vec, float *__restrict__ dst, int64_t ld_dst,
             float *__restrict__ colsum_part)
 {
+    sat_grid_wait();
     __shared__ float4 red[256];
     const int c4 = threadIdx.x % tpr, rg = threadIdx.x / tpr, n_rg = 256 / tpr;
     const int64_t r0 = (int64_t)blockIdx.x * MASK_ROWS_PER_BLOCK;
@@ -991,6 +994,7 @@ k_mask_rows(const float *__restrict__ src, int64_t ld, int64_t rows, int32_t d, 
 // zero-padded bias for the tile width (optionally with the same gate interleave as the weights)
 __global__ void k_pack_bias(const float *__restrict__ bias, int32_t n, int32_t n_pad, int32_t gate_h, float *__restrict__ out)
 {
+    sat_grid_wait();
     const int32_t np = blockIdx.x * blockDim.x + threadIdx.x;
     if (np >= n_pad) return;
     const int32_t nn = gate_h > 0 ? (np & 3) * gate_h + (np >> 2) : np;
@@ -1005,6 +1009,7 @@ __global__ void k_split_weights(const float *__restrict__ W, int64_t ldw, int32_
                                 int64_t ldw2, int32_t k2, int32_t n, int32_t n_pad, int32_t k_pad, int transpose, int32_t gate_h,
                                 float *__restrict__ hi, float *__restrict__ lo)
 {
+    sat_grid_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)n_pad * k_pad) return;
     const int32_t np = (int32_t)(i / k_pad), kk = (int32_t)(i - (int64_t)np * k_pad);
@@ -1085,7 +1090,7 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
     }
     int tpr = 1;
     while (tpr < (d + 3) / 4 && tpr < 256) tpr <<= 1;
-    k_mask_rows<<<(unsigned)blocks, 256, 0, ctx->stream>>>(src, ld, rows, d, tpr, mask, mask_words, act, ld_act, aligned16(act) && !(ld_act & 3),
+    sat_pdl(ctx->stream, k_mask_rows, (unsigned)blocks, 256, 0)(src, ld, rows, d, tpr, mask, mask_words, act, ld_act, aligned16(act) && !(ld_act & 3),
                                                             dst, ld_dst, part);
     SAT_LAUNCHED(ctx);
     if (colsum) SAT_TRY(sat_splitk_reduce(ctx, part, d, (int32_t)blocks, accumulate, colsum, d, d));
@@ -1106,7 +1111,7 @@ sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1,
     out->lo = (float *)((char *)buf.p + plane);
     out->ld = k_pad;
     out->n_pad = n_pad;
-    k_split_weights<<<(unsigned)cdiv64((int64_t)n_pad * k_pad, 256), 256, 0, ctx->stream>>>(W, ldw, k1, k1_pad, W2, ldw2, k2, n, n_pad, k_pad,
+    sat_pdl(ctx->stream, k_split_weights, (unsigned)cdiv64((int64_t)n_pad * k_pad, 256), 256, 0)(W, ldw, k1, k1_pad, W2, ldw2, k2, n, n_pad, k_pad,
                                                                                           transpose, gate_h, out->hi, out->lo);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -1150,7 +1155,7 @@ static sat_status launch_tck(sat_ctx *ctx, const TckLaunch &L, const TcEpilogue 
         SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_k<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set.mark(ctx->device);
     }
-    k_gemm_tc_k<EPI><<<L.grid, TCK_THREADS, smem, ctx->stream>>>(L.mA, L.mA2, L.mB, L.mBlo, L.mC, L.use_tma_store, L.m, L.n, L.nkb1, L.nkb2, L.bn, L.n_tiles_n,
+    sat_pdl(ctx->stream, k_gemm_tc_k<EPI>, L.grid, TCK_THREADS, smem)(L.mA, L.mA2, L.mB, L.mBlo, L.mC, L.use_tma_store, L.m, L.n, L.nkb1, L.nkb2, L.bn, L.n_tiles_n,
                                                                 L.n_tiles, ep, ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -1188,7 +1193,7 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
         DevBuf &home = eh.bias_home ? *eh.bias_home : ctx->buf_bias;
         if (!(eh.bias_home && eh.bias_ready && home.bytes >= padded * sizeof(float))) {
             SAT_TRY(sat_ensure(ctx, home, padded * sizeof(float)));
-            k_pack_bias<<<(unsigned)cdiv64(padded, 256), 256, 0, ctx->stream>>>(eh.bias, n, (int32_t)padded, eh.lstm_h > 0 ? eh.lstm_h : eh.pack_gate_h,
+            sat_pdl(ctx->stream, k_pack_bias, (unsigned)cdiv64(padded, 256), 256, 0)(eh.bias, n, (int32_t)padded, eh.lstm_h > 0 ? eh.lstm_h : eh.pack_gate_h,
                                                                                 (float *)home.p);
             SAT_LAUNCHED(ctx);
         }
@@ -1266,7 +1271,7 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
         g_attr_mn.mark(ctx->device);
     }
     dim3 grid((unsigned)cdiv64(m, mt * TC_BM), (unsigned)cdiv64(n, bn), (unsigned)splits);
-    k_gemm_tc_mn<<<grid, MN_THREADS, smem, ctx->stream>>>(mA, mB, m, n, rps, r1, mt, bn, (int32_t)stages, mt == 1 ? 256u : 512u, part, part_cs,
+    sat_pdl(ctx->stream, k_gemm_tc_mn, grid, MN_THREADS, smem)(mA, mB, m, n, rps, r1, mt, bn, (int32_t)stages, mt == 1 ? 256u : 512u, part, part_cs,
                                                        ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
     return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, part_cs, n, colsum);

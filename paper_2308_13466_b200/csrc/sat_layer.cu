@@ -250,6 +250,7 @@ extern "C" sat_status sat_cache_import(sat_ctx *ctx, int32_t layer, const float 
 // this kernel applies the cell:  c = f c + i g ; s = o tanh(c).
 __global__ void k_lstm_cell(const float *__restrict__ gates, int64_t rows, int32_t h, int first, float *__restrict__ c, float *__restrict__ s)
 {
+    sat_grid_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= rows * h) return;
     const int64_t r = sat_div(t, h);
@@ -273,6 +274,7 @@ sat_status sat_gemm_nn_dual(sat_ctx *ctx, int64_t m, int32_t n, int32_t k1, cons
 // first LSTM step from a cached input projection (gate-interleaved columns 4 j + gate): previous state is zero
 __global__ void k_lstm_cell_first(const float *__restrict__ proj, int64_t rows, int32_t h, float *__restrict__ c, float *__restrict__ s)
 {
+    sat_grid_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= rows * h) return;
     const float4 a = __ldg(reinterpret_cast<const float4 *>(proj) + t);  // (i, f, g, o) of unit t % h of row t / h
@@ -345,7 +347,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
         eh.lstm_c = cell;
         if (cached && t == 0) {
             ProfScope prof(ctx, SATK_LSTM_CELL, 4.0 * (double)rows * h * 6.0, 0.0);
-            k_lstm_cell_first<<<(unsigned)cdiv64(rows * h, 256), 256, 0, ctx->stream>>>(pr, rows, h, cell, c->S);
+            sat_pdl(ctx->stream, k_lstm_cell_first, (unsigned)cdiv64(rows * h, 256), 256, 0)(pr, rows, h, cell, c->S);
             SAT_LAUNCHED(ctx);
         } else if (cached) {
             if (!have_up) {
@@ -381,6 +383,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
 __global__ void k_gru_cell(const float *__restrict__ gx, const float *__restrict__ gh, const float *__restrict__ b_hn, int64_t rows, int32_t h,
                            float *__restrict__ s)
 {
+    sat_grid_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= rows * h) return;
     const int64_t r0 = sat_div(t, h);
@@ -452,7 +455,7 @@ static sat_status run_gru(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p)
             }
         }
         ProfScope prof(ctx, SATK_LSTM_CELL, 4.0 * (double)rows * h * 8.0, 0.0);
-        k_gru_cell<<<(unsigned)cdiv64(rows * h, 256), 256, 0, ctx->stream>>>(gx, t > 0 ? gh : nullptr, p->b + 3 * h, rows, h, c->S);
+        sat_pdl(ctx->stream, k_gru_cell, (unsigned)cdiv64(rows * h, 256), 256, 0)(gx, t > 0 ? gh : nullptr, p->b + 3 * h, rows, h, c->S);
         SAT_LAUNCHED(ctx);
     }
     c->S_valid = true;
@@ -515,7 +518,7 @@ static sat_status run_lstm(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p
         }
         if (!fused) {
             ProfScope prof(ctx, SATK_LSTM_CELL, 4.0 * (double)rows * h * 7.0, 0.0);
-            k_lstm_cell<<<(unsigned)cdiv64(rows * h, 256), 256, 0, ctx->stream>>>(gates, rows, h, t == 0, cell, c->S);
+            sat_pdl(ctx->stream, k_lstm_cell, (unsigned)cdiv64(rows * h, 256), 256, 0)(gates, rows, h, t == 0, cell, c->S);
             SAT_LAUNCHED(ctx);
         }
     }
@@ -980,6 +983,7 @@ __global__ void __launch_bounds__(256)
 k_loss_ce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const int32_t *__restrict__ y, float scale,
           float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
 {
+    sat_grid_wait();
     const int lane = threadIdx.x & 7;
     double acc = 0.0;
     // whole warps stay together (the shuffles name every lane): a warp walks four rows at a time
@@ -1024,6 +1028,7 @@ __global__ void __launch_bounds__(256)
 k_loss_ce_wide(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const int32_t *__restrict__ y, float scale,
                float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
 {
+    sat_grid_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double acc = 0.0;
     for (int64_t r = (int64_t)blockIdx.x * 8 + warp; r < rows; r += (int64_t)gridDim.x * 8) {
@@ -1050,6 +1055,7 @@ __global__ void __launch_bounds__(256)
 k_loss_bce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const uint8_t *__restrict__ y, float scale,
            float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
 {
+    sat_grid_wait();
     const float sc = scale / (float)C;
     const int32_t cv = C / V;
     const int64_t count = rows * cv;
@@ -1103,15 +1109,15 @@ extern "C" sat_status sat_loss_grad(sat_ctx *ctx, int32_t part, int kind, int32_
 #define ARGS v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial, ticket, loss_sum
     if (kind == SAT_LOSS_SOFTMAX_CE) {
         const int32_t *yl = (const int32_t *)labels;
-        if (n_classes <= 16) k_loss_ce<2><<<blocks, 256, 0, ctx->stream>>>(ARGS);
-        else if (n_classes <= 32) k_loss_ce<4><<<blocks, 256, 0, ctx->stream>>>(ARGS);
-        else if (n_classes <= 64) k_loss_ce<8><<<blocks, 256, 0, ctx->stream>>>(ARGS);
-        else if (n_classes <= 128) k_loss_ce<16><<<blocks, 256, 0, ctx->stream>>>(ARGS);
-        else k_loss_ce_wide<<<blocks, 256, 0, ctx->stream>>>(ARGS);
+        if (n_classes <= 16) sat_pdl(ctx->stream, k_loss_ce<2>, blocks, 256, 0)(ARGS);
+        else if (n_classes <= 32) sat_pdl(ctx->stream, k_loss_ce<4>, blocks, 256, 0)(ARGS);
+        else if (n_classes <= 64) sat_pdl(ctx->stream, k_loss_ce<8>, blocks, 256, 0)(ARGS);
+        else if (n_classes <= 128) sat_pdl(ctx->stream, k_loss_ce<16>, blocks, 256, 0)(ARGS);
+        else sat_pdl(ctx->stream, k_loss_ce_wide, blocks, 256, 0)(ARGS);
     } else {
         const uint8_t *yl = (const uint8_t *)labels;
-        if (vec4) k_loss_bce<4><<<blocks, 256, 0, ctx->stream>>>(ARGS);
-        else k_loss_bce<1><<<blocks, 256, 0, ctx->stream>>>(ARGS);
+        if (vec4) sat_pdl(ctx->stream, k_loss_bce<4>, blocks, 256, 0)(ARGS);
+        else sat_pdl(ctx->stream, k_loss_bce<1>, blocks, 256, 0)(ARGS);
     }
 #undef ARGS
     SAT_LAUNCHED(ctx);
@@ -1124,6 +1130,7 @@ k_staleness(const int32_t *__restrict__ halo_gid, const int32_t *__restrict__ po
             const float *__restrict__ fresh, int64_t ld, const float *__restrict__ used, int64_t ld_used, double *__restrict__ block_partial,
             int *__restrict__ ticket, double *total)
 {
+    sat_grid_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double acc = 0.0;
     for (int64_t j = (int64_t)blockIdx.x * 8 + warp; j < n_halo; j += (int64_t)gridDim.x * 8) {
@@ -1152,7 +1159,7 @@ extern "C" sat_status sat_staleness(sat_ctx *ctx, int32_t part, int32_t d, const
     const int64_t groups = cdiv64(v.n_halo, 8);
     const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS ? groups : LOSS_MAX_BLOCKS);
     SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS * sizeof(double)));
-    k_staleness<<<blocks, 256, 0, ctx->stream>>>(ctx->halo_gid, ctx->pos, v.halo0, v.n_halo, d, h_fresh, ld, h_used_halo, ld_halo,
+    sat_pdl(ctx->stream, k_staleness, blocks, 256, 0)(ctx->halo_gid, ctx->pos, v.halo0, v.n_halo, d, h_fresh, ld, h_used_halo, ld_halo,
                                                  (double *)ctx->buf_misc.p, ctx->d_flag + 2, sq_sum);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -1160,6 +1167,7 @@ extern "C" sat_status sat_staleness(sat_ctx *ctx, int32_t part, int32_t d, const
 
 __global__ void k_sgd(int64_t count, float *__restrict__ w, const float *__restrict__ g, float lr)
 {
+    sat_grid_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) w[i] = w[i] - lr * g[i];
 }
@@ -1169,7 +1177,7 @@ extern "C" sat_status sat_sgd_step(sat_ctx *ctx, int64_t count, float *w, const 
     CHECK_CTX(ctx);
     if (count < 0 || (count > 0 && (!w || !g))) return sat_fail(ctx, SAT_EINVAL, "sat_sgd_step: null tensor");
     if (count == 0) return SAT_OK;
-    k_sgd<<<(unsigned)cdiv64(count, 256), 256, 0, ctx->stream>>>(count, w, g, lr);
+    sat_pdl(ctx->stream, k_sgd, (unsigned)cdiv64(count, 256), 256, 0)(count, w, g, lr);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
@@ -1185,6 +1193,7 @@ struct SgdBatch {
 
 __global__ void k_sgd_many(SgdBatch b, float lr)
 {
+    sat_grid_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= b.end[b.n - 1]) return;
     int t = 0;
@@ -1211,7 +1220,7 @@ extern "C" sat_status sat_sgd_steps(sat_ctx *ctx, int32_t n_arrays, const int64_
             ++b.n;
         }
         if (b.n == 0) continue;
-        k_sgd_many<<<(unsigned)cdiv64(total, 256), 256, 0, ctx->stream>>>(b, lr);
+        sat_pdl(ctx->stream, k_sgd_many, (unsigned)cdiv64(total, 256), 256, 0)(b, lr);
         SAT_LAUNCHED(ctx);
     }
     return SAT_OK;

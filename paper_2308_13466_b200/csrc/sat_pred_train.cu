@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(256)
 k_pt_cell_fwd(float *__restrict__ z, int64_t rows, int32_t h, const float *__restrict__ c_prev, float *__restrict__ c_out,
               float *__restrict__ h_out)
 {
+    sat_grid_wait();
     const int h4 = h >> 2, rpp = 256 / h4;
     const int q = threadIdx.x % h4, rr = threadIdx.x / h4;
     if (rr >= rpp) return;
@@ -62,6 +63,7 @@ __global__ void __launch_bounds__(256)
 k_pt_cell_bwd(float *__restrict__ gz, int64_t rows, int32_t h, const float *__restrict__ c_prev, const float *__restrict__ c_cur,
               const float *__restrict__ dh, const float *dc_in, float *dc_out, float *__restrict__ colsum_part)
 {
+    sat_grid_wait();
     extern __shared__ float red[];   // [rpp][4h]
     const int h4 = h >> 2, rpp = 256 / h4;
     const int q = threadIdx.x % h4, rr = threadIdx.x / h4;
@@ -123,6 +125,7 @@ k_pt_error(float *__restrict__ pred, int64_t ld, int64_t n_halo, int32_t d, cons
            const int32_t *__restrict__ halo_slot, const float *__restrict__ row_weight, const int64_t *__restrict__ halo_off, int32_t M,
            double *__restrict__ block_partial, float *__restrict__ colsum_part)
 {
+    sat_grid_wait();
     extern __shared__ float4 cs4[];   // [8 warps][d rounded up to 4]
     float *cs = reinterpret_cast<float *>(cs4);
     __shared__ double red[8];
@@ -193,6 +196,7 @@ k_pt_error(float *__restrict__ pred, int64_t ld, int64_t n_halo, int32_t d, cons
 // in index order; the association is fixed, so the total does not depend on scheduling
 __global__ void __launch_bounds__(256) k_pt_sum(const double *__restrict__ block_partial, int64_t count, double *total)
 {
+    sat_grid_wait();
     __shared__ double part[256];
     double s = 0.0;
     for (int64_t i = threadIdx.x; i < count; i += 256) s += block_partial[i];
@@ -319,7 +323,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
             SAT_TRY(sat_gemm_nn_dual(ctx, R, 4 * h, d, x, c->ld, params->Wx, 4 * h, t ? h : 0, h_prev, h, params->Uh, 4 * h, params->b, z, 4 * h));
         }
         ProfScope prof(ctx, SATK_PRED_TRAIN, 4.0 * (double)plane_s * 11.0, 0.0);
-        k_pt_cell_fwd<<<cell_grid, 256, 0, ctx->stream>>>(z, R, h, t ? cs + (t - 1) * plane_s : nullptr, cs + t * plane_s, hs + t * plane_s);
+        sat_pdl(ctx->stream, k_pt_cell_fwd, cell_grid, 256, 0)(z, R, h, t ? cs + (t - 1) * plane_s : nullptr, cs + t * plane_s, hs + t * plane_s);
         SAT_LAUNCHED(ctx);
     }
     // ---- graph convolution on the final state, output layer, skip connection ----
@@ -353,11 +357,11 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     {
         ProfScope prof(ctx, SATK_PRED_TRAIN, 4.0 * (double)nb * d * 3.0, 0.0);
         SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)n_blocks * d * sizeof(float)));
-        k_pt_error<<<(unsigned)n_blocks, 256, (size_t)8 * ld_d * sizeof(float), ctx->stream>>>(E, ld_d, nb, d, ring_buf(ctx, c, ctx->write_idx), c->ld,
+        sat_pdl(ctx->stream, k_pt_error, (unsigned)n_blocks, 256, (size_t)8 * ld_d * sizeof(float))(E, ld_d, nb, d, ring_buf(ctx, c, ctx->write_idx), c->ld,
                                                                                            ctx->halo_slot, row_weight, halo_off, M, partial,
                                                                                            (float *)ctx->buf_colsum.p);
         SAT_LAUNCHED(ctx);
-        k_pt_sum<<<1, 256, 0, ctx->stream>>>(partial, n_blocks, partial + n_blocks);
+        sat_pdl(ctx->stream, k_pt_sum, 1, 256, 0)(partial, n_blocks, partial + n_blocks);
         SAT_LAUNCHED(ctx);
     }
     SAT_TRY(sat_splitk_reduce(ctx, (const float *)ctx->buf_colsum.p, d, (int32_t)n_blocks, 0, g_bg, d, d));
@@ -376,7 +380,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
             {
                 ProfScope prof(ctx, SATK_PRED_TRAIN, 4.0 * (double)plane_s * 13.0, 0.0);
                 SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)bwd_grid * 4 * h * sizeof(float)));
-                k_pt_cell_bwd<<<bwd_grid, 256, cell_smem, ctx->stream>>>(z, R, h, t ? cs + (t - 1) * plane_s : nullptr, cs + t * plane_s, dh,
+                sat_pdl(ctx->stream, k_pt_cell_bwd, bwd_grid, 256, cell_smem)(z, R, h, t ? cs + (t - 1) * plane_s : nullptr, cs + t * plane_s, dh,
                                                                           t == k - 1 ? nullptr : dc, dc, (float *)ctx->buf_colsum.p);
                 SAT_LAUNCHED(ctx);
             }

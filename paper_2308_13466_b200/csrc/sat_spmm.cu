@@ -447,6 +447,7 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
        int32_t d4, const float *__restrict__ in_base, int64_t ld_in, const float *__restrict__ halo_base, int64_t ld_halo, float *__restrict__ out_base,
        int64_t ld_out, float *__restrict__ partial, const uint32_t *__restrict__ omask, int32_t omask_words, SpmmEpilogue ep, DbgLimits dbg)
 {
+    sat_grid_wait();
     const int lane = threadIdx.x & (G - 1);
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     if (gid >= n_items) return;
@@ -540,6 +541,7 @@ k_spmm_fixup(const int32_t *__restrict__ hrows, int32_t n_hrows, const int32_t *
              const int32_t *__restrict__ tot, int64_t slot_base, const float *__restrict__ scale, int32_t d4, const float *__restrict__ partial,
              float *__restrict__ out_base, int64_t ld_out, const uint32_t *__restrict__ omask, int32_t omask_words, SpmmEpilogue ep, DbgLimits dbg)
 {
+    sat_grid_wait();
     __shared__ float4 part[8][32];
     const int32_t slabs = (d4 + 31) / 32;
     const int64_t n_hblk = (int64_t)n_hrows * slabs;
@@ -599,10 +601,10 @@ static void launch_spmm(sat_ctx *ctx, const int4 *items, int32_t n_items, int64_
     dim3 grid((unsigned)cdiv64((int64_t)n_items * G, 256), (unsigned)cdiv64(d4, G * NV));
     const DbgLimits dbg = dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1);
     if (a.scale)
-        k_spmm<G, NV, U, MINB, false><<<grid, 256, 0, ctx->stream>>>(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
+        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, false>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
                                                                      a.out_base, a.ld_out, partial, a.omask, a.omask_words, a.ep, dbg);
     else
-        k_spmm<G, NV, U, MINB, true><<<grid, 256, 0, ctx->stream>>>(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
+        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, true>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
                                                                     a.out_base, a.ld_out, partial, a.omask, a.omask_words, a.ep, dbg);
 }
 
@@ -634,7 +636,7 @@ static sat_status run_list(sat_ctx *ctx, const PartView &v, const SpmmList &l, i
 #undef ARGS
     SAT_LAUNCHED(ctx);
     if (n_slots > 0) {
-        k_spmm_fixup<<<(unsigned)(n_hrows * cdiv64(d4, 32) + cdiv64(n_mrows * d4, 256)), 256, 0, ctx->stream>>>(
+        sat_pdl(ctx->stream, k_spmm_fixup, (unsigned)(n_hrows * cdiv64(d4, 32) + cdiv64(n_mrows * d4, 256)), 256, 0)(
             l.hrows + hrow0, (int32_t)n_hrows, l.mrows + mrow0, (int32_t)n_mrows, l.slot0, l.tot, slot_base, a.scale, d4, partial, a.out_base, a.ld_out, a.omask,
             a.omask_words, a.ep, dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1));
         SAT_LAUNCHED(ctx);
@@ -832,6 +834,7 @@ sat_status sat_spmm_hrow(sat_ctx *ctx, const PartView &v, int32_t d, const float
 __global__ void k_gather_rows(const int32_t *__restrict__ idx, int64_t count, int32_t d4, const float *__restrict__ src, int64_t ld_src,
                               float *__restrict__ out, int64_t ld_out, DbgLimits dbg)
 {
+    sat_grid_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = sat_div(t, d4);
     const int c = (int)(t - i * d4);
@@ -846,7 +849,7 @@ sat_status sat_gather(sat_ctx *ctx, const int32_t *idx, int64_t count, int32_t d
     if (count == 0) return SAT_OK;
     const int32_t d4 = (d + 3) / 4;
     ProfScope prof(ctx, SATK_GATHER, (8.0 * d + 4.0) * (double)count, 0.0);
-    k_gather_rows<<<(unsigned)cdiv64(count * d4, 256), 256, 0, ctx->stream>>>(idx, count, d4, src, ld_src, out, ld_out,
+    sat_pdl(ctx->stream, k_gather_rows, (unsigned)cdiv64(count * d4, 256), 256, 0)(idx, count, d4, src, ld_src, out, ld_out,
                                                                               dbg_limits(src_rows, DbgRange{0, 0}, DbgRange{0, count}, ctx->d_flag + 1));
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -855,6 +858,7 @@ sat_status sat_gather(sat_ctx *ctx, const int32_t *idx, int64_t count, int32_t d
 __global__ void k_scatter_rows(const int32_t *__restrict__ src_row, const int32_t *__restrict__ dst_row, int64_t count, int32_t d4,
                                const float *__restrict__ src_base, int64_t ld_src, float *__restrict__ dst, int64_t ld_dst, DbgLimits dbg)
 {
+    sat_grid_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = sat_div(t, d4);
     const int c = (int)(t - i * d4);
@@ -869,7 +873,7 @@ sat_status sat_scatter(sat_ctx *ctx, const int32_t *src_row, const int32_t *dst_
     if (count == 0) return SAT_OK;
     const int32_t d4 = (d + 3) / 4;
     ProfScope prof(ctx, SATK_SCATTER, (8.0 * d + 8.0) * (double)count, 0.0);
-    k_scatter_rows<<<(unsigned)cdiv64(count * d4, 256), 256, 0, ctx->stream>>>(src_row, dst_row, count, d4, src_base, ld_src, dst, ld_dst,
+    sat_pdl(ctx->stream, k_scatter_rows, (unsigned)cdiv64(count * d4, 256), 256, 0)(src_row, dst_row, count, d4, src_base, ld_src, dst, ld_dst,
                                                                                dbg_limits(src_rows, DbgRange{0, 0}, dst_rows, ctx->d_flag + 1));
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -879,6 +883,7 @@ __global__ void k_scatter_add_rows(const int32_t *__restrict__ src_row, const in
                                    const float *__restrict__ src_base, int64_t ld_src, float *__restrict__ dst, int64_t ld_dst,
                                    const uint32_t *__restrict__ mask, int32_t mask_words, DbgLimits dbg)
 {
+    sat_grid_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = sat_div(t, d4);
     const int c = (int)(t - i * d4);
@@ -901,7 +906,7 @@ sat_status sat_scatter_add(sat_ctx *ctx, const int32_t *src_row, const int32_t *
     if (count == 0) return SAT_OK;
     const int32_t d4 = (d + 3) / 4;
     ProfScope prof(ctx, SATK_SCATTER, (12.0 * d + 8.0) * (double)count, 0.0);
-    k_scatter_add_rows<<<(unsigned)cdiv64(count * d4, 256), 256, 0, ctx->stream>>>(src_row, dst_row, count, d4, src_base, ld_src, dst, ld_dst, mask,
+    sat_pdl(ctx->stream, k_scatter_add_rows, (unsigned)cdiv64(count * d4, 256), 256, 0)(src_row, dst_row, count, d4, src_base, ld_src, dst, ld_dst, mask,
                                                                                    mask_words, dbg_limits(src_rows, DbgRange{0, 0}, dst_rows, ctx->d_flag + 1));
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -971,6 +976,7 @@ k_sum_by_slot(const int64_t *__restrict__ hs_ptr, const int32_t *__restrict__ hs
               int32_t n, int32_t d4, const float *__restrict__ src, int64_t ld_src, int self_scale, int add, float *__restrict__ out, int64_t ld_out,
               DbgLimits dbg)
 {
+    sat_grid_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t s = sat_div(t, d4);
     const int c = (int)(t - s * d4);
@@ -1009,7 +1015,7 @@ sat_status sat_sum_by_slot(sat_ctx *ctx, int32_t d, const float *src, int32_t ld
     SAT_TRY(build_halo_by_slot(ctx));
     const int32_t d4 = (d + 3) / 4;
     ProfScope prof(ctx, SATK_SCATTER, 8.0 * (double)ctx->nb + 4.0 * d * ((double)ctx->nb + (add ? 2.0 : 1.0) * ctx->n_slots), 0.0);
-    k_sum_by_slot<<<(unsigned)cdiv64((int64_t)ctx->n_slots * d4, 256), 256, 0, ctx->stream>>>(ctx->hs_ptr, ctx->hs_pos, ctx->n_slots, ctx->dinv_enc,
+    sat_pdl(ctx->stream, k_sum_by_slot, (unsigned)cdiv64((int64_t)ctx->n_slots * d4, 256), 256, 0)(ctx->hs_ptr, ctx->hs_pos, ctx->n_slots, ctx->dinv_enc,
                                                                                               ctx->n, d4, src, ld_src, self_scale, add, out, ld_out,
                                                                                               dbg_limits(DbgRange{0, ctx->nb}, DbgRange{0, 0}, DbgRange{0, ctx->n_slots}, ctx->d_flag + 1));
     SAT_LAUNCHED(ctx);
