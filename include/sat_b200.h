@@ -378,6 +378,43 @@ sat_status sat_sgd_step(sat_ctx *ctx, int64_t count, float *w, const float *g, f
 sat_status sat_sgd_steps(sat_ctx *ctx, int32_t n_arrays, const int64_t *counts, float *const *w, const float *const *g, float lr);
 
 /* ---------------------------------------------------------------------------------------
+ * sat_epoch — the epoch body of Algorithm 1 in one call: the calls of this header, in the order of the algorithm, on buffers
+ * described once.  Per partition (or for all of them at once): for l = 1..L  sat_predict of cached layer l-1 where pred[l-2] is
+ * given (SAT_FWD_HALO_CACHED where not), sat_layer_fwd with ReLU and SAT_FWD_PUSH (l < L; layer 1 reads x with
+ * SAT_FWD_INPUT_GLOBAL);  sat_loss_grad;  sat_layer_bwd for l = L..1 with the fused ReLU masks.  Results are those of these calls.
+ *   order     n_order = 0: all partitions per launch.  Otherwise the partitions to run, one after the other (HOST array): the first
+ *             one runs the predictor's recurrence and overwrites the gradients, the others reuse the state table and add to them.
+ *   flags     SAT_EPOCH_GRAD_HISTORY: SAT_BWD_GRAD_HISTORY on layers >= 2;  SAT_EPOCH_COMMIT: sat_cache_commit afterwards;
+ *             SAT_EPOCH_STEP: w <- w - lr gw, b <- b - lr gb afterwards;  SAT_EPOCH_CONTINUE: this call goes on with an epoch that an
+ *             earlier one began (partitions of `order` that are yet to run): its first partition too reuses the state table and adds to
+ *             the gradients and to the loss
+ * All arrays of pointers / sizes are HOST, the arrays they point to DEVICE.  *loss_sum is overwritten (unless continuing).
+ * ------------------------------------------------------------------------------------- */
+typedef struct sat_epoch_buffers {
+    int32_t n_layers;
+    const int32_t *dims;                  /* [L+1] */
+    const float *x;                       /* features of all n nodes in global id order [n x ld_x] */
+    int32_t ld_x;
+    int32_t loss_kind;                    /* SAT_LOSS_* */
+    const void *labels;                   /* partition-major rows, as for sat_loss_grad */
+    float *const *h;                      /* [L] outputs of the layers, [n x ld_h[l]] in partition-major row order */
+    const int32_t *ld_h;
+    float *const *g;                      /* [L] gradients with respect to them, [n x ld_g[l]] */
+    const int32_t *ld_g;
+    float *halo;                          /* [sum_m b_m x ld_halo] room for predicted rows (NULL without predictors) */
+    int32_t ld_halo;
+    float *const *w, *const *b;           /* [L] parameters (b[l] may be NULL) */
+    float *const *gw, *const *gb;         /* [L] their gradients */
+    const sat_pred_params *const *pred;   /* [L-1] predictor of cached layer l (NULL: plain historical embeddings), or NULL */
+    double *loss_sum;                     /* may be NULL */
+} sat_epoch_buffers;
+#define SAT_EPOCH_GRAD_HISTORY 1
+#define SAT_EPOCH_COMMIT 2
+#define SAT_EPOCH_STEP 4
+#define SAT_EPOCH_CONTINUE 8
+sat_status sat_epoch(sat_ctx *ctx, const sat_epoch_buffers *buffers, const int32_t *order, int32_t n_order, int flags, float lr);
+
+/* ---------------------------------------------------------------------------------------
  * The dense contractions of the layer step on caller tensors (all DEVICE fp32; the paper has no counterpart:
  * they are the matrix products inside the forward / backward formulas of the Appendix, exposed so that the
  * kernels can be exercised and measured in isolation).  Same kernels and same path selection as inside

@@ -44,6 +44,15 @@ class sat_pred_params(C.Structure):
 
 
 SAT_CELL_LSTM, SAT_CELL_GRU = 0, 1
+SAT_EPOCH_GRAD_HISTORY, SAT_EPOCH_COMMIT, SAT_EPOCH_STEP, SAT_EPOCH_CONTINUE = 1, 2, 4, 8
+
+
+class sat_epoch_buffers(C.Structure):
+    """Host description of an epoch's buffers (sat_epoch); `_keep` holds the arrays and tensors behind the pointers."""
+    _fields_ = [("n_layers", C.c_int32), ("dims", C.c_void_p), ("x", C.c_void_p), ("ld_x", C.c_int32), ("loss_kind", C.c_int32),
+                ("labels", C.c_void_p), ("h", C.c_void_p), ("ld_h", C.c_void_p), ("g", C.c_void_p), ("ld_g", C.c_void_p),
+                ("halo", C.c_void_p), ("ld_halo", C.c_int32), ("w", C.c_void_p), ("b", C.c_void_p), ("gw", C.c_void_p), ("gb", C.c_void_p),
+                ("pred", C.c_void_p), ("loss_sum", C.c_void_p)]
 
 
 def _load():
@@ -67,7 +76,7 @@ EXPORTS = [
     "sat_predict_state", "sat_layer_fwd", "sat_layer_bwd", "sat_cache_update", "sat_cache_commit", "sat_cache_state",
     "sat_cache_read", "sat_cache_export", "sat_cache_import", "sat_cache_set_state", "sat_loss_grad", "sat_sgd_step", "sat_sgd_steps",
     "sat_dense_nn", "sat_dense_nt", "sat_dense_tn", "sat_dense_tn_static", "sat_launch_count", "sat_profile_families", "sat_profile_enable", "sat_profile_select", "sat_profile_read",
-    "sat_codec_plan", "sat_codec_encode", "sat_codec_decode", "sat_cache_requantise", "sat_staleness", "sat_pred_grad", "sat_grad_history_read", "sat_grad_history_write", "sat_gat_fwd", "sat_gat_bwd", "sat_gat_scores", "sat_profile_l2_rates", "sat_debug_poke_index", "sat_spmm_plan",
+    "sat_epoch", "sat_codec_plan", "sat_codec_encode", "sat_codec_decode", "sat_cache_requantise", "sat_staleness", "sat_pred_grad", "sat_grad_history_read", "sat_grad_history_write", "sat_gat_fwd", "sat_gat_bwd", "sat_gat_scores", "sat_profile_l2_rates", "sat_debug_poke_index", "sat_spmm_plan",
 ]
 
 
@@ -237,6 +246,35 @@ def sat_layer_bwd(ctx, part: int, layer: int, g_out, W, g_W, g_b, accumulate: in
                                    _dev(g_W), _dev(g_b), C.c_int(accumulate),
                                    _dev(g_in), C.c_int32(_ld(g_in) if g_in is not None else 0),
                                    _dev(g_halo), C.c_int32(_ld(g_halo) if g_halo is not None else 0)))
+
+
+def make_epoch_buffers(dims, X, labels, loss_kind: int, H, G, halo, W, b, gW, gb, pred, loss_sum) -> sat_epoch_buffers:
+    """Description for sat_epoch: H, G the layers' outputs and gradients (row strides multiples of 4), W, b, gW, gb contiguous
+    CUDA fp32 lists, pred a list of sat_pred_params or None per cached layer, or None."""
+    for l, (w, gw, bb, gbb) in enumerate(zip(W, gW, b, gb)):
+        assert w.is_cuda and w.is_contiguous() and gw.is_contiguous() and tuple(w.shape) == tuple(gw.shape) == (dims[l], dims[l + 1])
+        assert bb is None or (bb.is_cuda and bb.is_contiguous() and bb.numel() == gbb.numel() == dims[l + 1])
+    n = len(W)
+    ptrs = lambda ts: (C.c_void_p * max(len(ts), 1))(*[None if t is None else t.data_ptr() for t in ts])
+    lds = lambda ts: (C.c_int32 * len(ts))(*[_ld(t) for t in ts])
+    adr = lambda a: C.cast(a, C.c_void_p).value
+    arr = dict(dims=(C.c_int32 * (n + 1))(*dims), h=ptrs(H), ld_h=lds(H), g=ptrs(G), ld_g=lds(G), w=ptrs(W), b=ptrs(b), gw=ptrs(gW), gb=ptrs(gb))
+    e = sat_epoch_buffers(n_layers=n, x=_dev(X).value, ld_x=_ld(X), loss_kind=loss_kind, labels=_dev(labels).value, halo=_dev(halo).value,
+                          ld_halo=_ld(halo), loss_sum=None if loss_sum is None else loss_sum.data_ptr(), **{k: adr(v) for k, v in arr.items()})
+    if pred is not None:
+        arr["pred"] = (C.c_void_p * max(n - 1, 1))(*[None if p is None else C.addressof(p) for p in pred[:n - 1]])
+        e.pred = adr(arr["pred"])
+    e._keep = (arr, X, labels, list(H), list(G), halo, list(W), list(b), list(gW), list(gb), None if pred is None else list(pred), loss_sum)
+    return e
+
+
+def sat_epoch(ctx, buffers: sat_epoch_buffers, order=None, flags: int = SAT_EPOCH_COMMIT, lr: float = 0.0):
+    """order: partitions to run one after the other, or None for all of them per launch."""
+    if order is None:
+        st = _lib.sat_epoch(ctx, C.byref(buffers), None, 0, flags, C.c_float(lr))
+    else:
+        st = _lib.sat_epoch(ctx, C.byref(buffers), (C.c_int32 * max(len(order), 1))(*order), len(order), flags, C.c_float(lr))
+    _check(ctx, st)
 
 
 def sat_cache_update(ctx, part: int, layer: int, h_out):

@@ -94,6 +94,7 @@ extern "C" sat_status sat_create(sat_ctx **out, int device, void *cuda_stream)
     sat_ctx *ctx = new (std::nothrow) sat_ctx();
     if (!ctx) return SAT_ENOMEM;
     ctx->device = device;
+    cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, device);
     ctx->stream = (cudaStream_t)cuda_stream;
     if (cudaMalloc((void **)&ctx->d_flag, 4 * sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void **)&ctx->h_flag, 4 * sizeof(int)) != cudaSuccess) {

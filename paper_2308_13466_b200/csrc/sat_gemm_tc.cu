@@ -1222,9 +1222,7 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.tile_order = eh.tile_order;
     const int32_t n_tiles_n = (int32_t)cdiv64(n, bn);
     const int64_t n_tiles = cdiv64(m, TC_BM) * n_tiles_n;
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-    const unsigned grid = (unsigned)(n_tiles < sms ? n_tiles : sms);
+    const unsigned grid = (unsigned)(n_tiles < ctx->sms ? n_tiles : ctx->sms);
     TckLaunch L;
     L.mA = mA; L.mA2 = mA2; L.mB = mB; L.mBlo = mBlo; L.mC = mC;
     L.use_tma_store = use_tma_store;

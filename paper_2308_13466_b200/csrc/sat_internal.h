@@ -142,6 +142,7 @@ struct sat_ctx {
     uint64_t prof_mask = ~0ull;  // families that are bracketed while prof_on
     std::vector<ProfRec> prof;
     int device = 0;
+    int sms = 148;           // multiprocessors of the device
     cudaStream_t stream = nullptr;
     char err[512] = {0};
     bool cuda_failed = false;
@@ -369,6 +370,10 @@ sat_status sat_sum_by_slot(sat_ctx *ctx, int32_t d, const float *src, int32_t ld
 sat_status sat_scatter_add(sat_ctx *ctx, const int32_t *src_row, const int32_t *dst_row, int64_t count, int32_t d, const float *src_base,
                            int32_t ld_src, float *dst, int32_t ld_dst, const uint32_t *mask, int32_t mask_words, DbgRange src_rows = SAT_ANY_ROW,
                            DbgRange dst_rows = SAT_ANY_ROW);
+
+// sat_loss_grad with the choice of overwriting *loss_sum instead of adding to it
+sat_status sat_loss_into(sat_ctx *ctx, int32_t part, int kind, int32_t n_classes, const float *z, int32_t ld_z, const void *labels, double *loss_sum,
+                         float *g, int32_t ld_g, int overwrite);
 
 // GEMM family (sat_gemm.cu)
 // C[m x n] = A[m x k] B[k x n] (+ bias) with optional ReLU, sign-mask output, row-gathered residual add.

@@ -943,7 +943,7 @@ extern "C" sat_status sat_dense_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_
 // partials in fixed order: which rows a thread owns depends on the row count alone, so the total does not depend on scheduling.
 #define LOSS_MAX_BLOCKS (148 * 6)
 
-__device__ __forceinline__ void loss_finish(double thread_sum, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
+__device__ __forceinline__ void loss_finish(double thread_sum, double *__restrict__ block_partial, int *__restrict__ ticket, double *total, int overwrite)
 {
     __shared__ double red[256];
     __shared__ int last;
@@ -971,7 +971,7 @@ __device__ __forceinline__ void loss_finish(double thread_sum, double *__restric
     }
     if (threadIdx.x == 0) {
         *ticket = 0;   // the next launch on this stream starts from zero again
-        if (total) *total += red[0];
+        if (total) *total = overwrite ? red[0] : *total + red[0];
     }
 }
 
@@ -981,7 +981,8 @@ __device__ __forceinline__ void loss_finish(double thread_sum, double *__restric
 template <int CPL>
 __global__ void __launch_bounds__(256)
 k_loss_ce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const int32_t *__restrict__ y, float scale,
-          float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
+          float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total,
+          int overwrite)
 {
     sat_grid_wait();
     const int lane = threadIdx.x & 7;
@@ -1020,13 +1021,14 @@ k_loss_ce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, co
         }
         if (lane == 0) acc += (double)(scale * (mx + logf(se) - zy));
     }
-    loss_finish(acc, block_partial, ticket, total);
+    loss_finish(acc, block_partial, ticket, total, overwrite);
 }
 
 // any number of classes: three passes over the row
 __global__ void __launch_bounds__(256)
 k_loss_ce_wide(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const int32_t *__restrict__ y, float scale,
-               float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
+               float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total,
+          int overwrite)
 {
     sat_grid_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1044,7 +1046,7 @@ k_loss_ce_wide(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_
         for (int c = lane; c < C; c += 32) g[r * ld_g + c] = scale * (expf(zr[c] - mx) * inv - (c == yr ? 1.f : 0.f));
         if (lane == 0) acc += (double)(scale * (mx + logf(se) - zr[yr]));
     }
-    loss_finish(acc, block_partial, ticket, total);
+    loss_finish(acc, block_partial, ticket, total, overwrite);
 }
 
 // Sigmoid cross-entropy, element by element (the loss is a plain sum over nodes and labels): V consecutive labels per thread, V = 4
@@ -1053,7 +1055,8 @@ k_loss_ce_wide(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_
 template <int V>
 __global__ void __launch_bounds__(256)
 k_loss_bce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, const uint8_t *__restrict__ y, float scale,
-           float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total)
+           float *__restrict__ g, int64_t ld_g, double *__restrict__ block_partial, int *__restrict__ ticket, double *total,
+          int overwrite)
 {
     sat_grid_wait();
     const float sc = scale / (float)C;
@@ -1084,17 +1087,26 @@ k_loss_bce(int64_t rows, int32_t C, const float *__restrict__ z, int64_t ld_z, c
         else g[r * ld_g + c] = gx[0];
         acc += (double)(sc * a);
     }
-    loss_finish(acc, block_partial, ticket, total);
+    loss_finish(acc, block_partial, ticket, total, overwrite);
 }
 
 extern "C" sat_status sat_loss_grad(sat_ctx *ctx, int32_t part, int kind, int32_t n_classes, const float *z, int32_t ld_z,
                                     const void *labels, double *loss_sum, float *g, int32_t ld_g)
 {
     CHECK_CTX(ctx);
+    return sat_loss_into(ctx, part, kind, n_classes, z, ld_z, labels, loss_sum, g, ld_g, 0);
+}
+
+sat_status sat_loss_into(sat_ctx *ctx, int32_t part, int kind, int32_t n_classes, const float *z, int32_t ld_z, const void *labels, double *loss_sum,
+                         float *g, int32_t ld_g, int overwrite)
+{
     PartView v;
     SAT_TRY(sat_part_view(ctx, part, &v));
     if (kind != SAT_LOSS_SOFTMAX_CE && kind != SAT_LOSS_SIGMOID_BCE) return sat_fail(ctx, SAT_EINVAL, "sat_loss_grad: unknown loss");
-    if (v.n_rows == 0) return SAT_OK;
+    if (v.n_rows == 0) {
+        if (overwrite && loss_sum) SAT_CUDA(ctx, cudaMemsetAsync(loss_sum, 0, sizeof(double), ctx->stream));
+        return SAT_OK;
+    }
     if (n_classes <= 0 || !z || !labels || !g || ld_z < n_classes || ld_g < n_classes) return sat_fail(ctx, SAT_EINVAL, "sat_loss_grad: null tensor or bad shape");
     const bool vec4 = kind == SAT_LOSS_SIGMOID_BCE && !(n_classes & 3) && !(ld_z & 3) && !(ld_g & 3) && aligned16(z) && aligned16(g) &&
                       (((uintptr_t)labels) & 3u) == 0;
@@ -1106,7 +1118,7 @@ extern "C" sat_status sat_loss_grad(sat_ctx *ctx, int32_t part, int kind, int32_
     int *ticket = ctx->d_flag + 2;
     const float scale = 1.0f / (float)ctx->n;
     ProfScope prof(ctx, SATK_LOSS, 8.0 * (double)v.n_rows * n_classes, 0.0);
-#define ARGS v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial, ticket, loss_sum
+#define ARGS v.n_rows, n_classes, z, ld_z, yl, scale, g, ld_g, block_partial, ticket, loss_sum, overwrite
     if (kind == SAT_LOSS_SOFTMAX_CE) {
         const int32_t *yl = (const int32_t *)labels;
         if (n_classes <= 16) sat_pdl(ctx->stream, k_loss_ce<2>, blocks, 256, 0)(ARGS);
@@ -1128,7 +1140,8 @@ extern "C" sat_status sat_loss_grad(sat_ctx *ctx, int32_t part, int kind, int32_
 __global__ void __launch_bounds__(256)
 k_staleness(const int32_t *__restrict__ halo_gid, const int32_t *__restrict__ pos, int64_t halo0, int64_t n_halo, int32_t d,
             const float *__restrict__ fresh, int64_t ld, const float *__restrict__ used, int64_t ld_used, double *__restrict__ block_partial,
-            int *__restrict__ ticket, double *total)
+            int *__restrict__ ticket, double *total,
+          int overwrite)
 {
     sat_grid_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1143,7 +1156,7 @@ k_staleness(const int32_t *__restrict__ halo_gid, const int32_t *__restrict__ po
         }
         acc += s;
     }
-    loss_finish(acc, block_partial, ticket, total);
+    loss_finish(acc, block_partial, ticket, total, overwrite);
 }
 
 extern "C" sat_status sat_staleness(sat_ctx *ctx, int32_t part, int32_t d, const float *h_fresh, int32_t ld, const float *h_used_halo,
@@ -1153,14 +1166,16 @@ extern "C" sat_status sat_staleness(sat_ctx *ctx, int32_t part, int32_t d, const
     PartView v;
     SAT_TRY(sat_part_view(ctx, part, &v));
     if (!sq_sum || d <= 0) return sat_fail(ctx, SAT_EINVAL, "sat_staleness: null result or bad width");
-    SAT_CUDA(ctx, cudaMemsetAsync(sq_sum, 0, sizeof(double), ctx->stream));
-    if (v.n_halo == 0) return SAT_OK;
+    if (v.n_halo == 0) {
+        SAT_CUDA(ctx, cudaMemsetAsync(sq_sum, 0, sizeof(double), ctx->stream));
+        return SAT_OK;
+    }
     if (!h_fresh || !h_used_halo || ld < d || ld_halo < d) return sat_fail(ctx, SAT_EINVAL, "sat_staleness: null tensor or bad leading dimension");
     const int64_t groups = cdiv64(v.n_halo, 8);
     const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS ? groups : LOSS_MAX_BLOCKS);
     SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS * sizeof(double)));
     sat_pdl(ctx->stream, k_staleness, blocks, 256, 0)(ctx->halo_gid, ctx->pos, v.halo0, v.n_halo, d, h_fresh, ld, h_used_halo, ld_halo,
-                                                 (double *)ctx->buf_misc.p, ctx->d_flag + 2, sq_sum);
+                                                 (double *)ctx->buf_misc.p, ctx->d_flag + 2, sq_sum, 1);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }

@@ -1,8 +1,9 @@
 """One SAT epoch as a sequence of library calls (Algorithm 1 of the paper, epoch body).
 
-This module only owns device buffers (torch tensors) and strings the C entry points
-together in the order of Algorithm 1:  for every layer: pull (predict) -> forward ->
-push;  then loss, backward, commit.  It contains no arithmetic of its own.
+This module only owns device buffers (torch tensors) and hands them to the library's epoch
+call (Algorithm 1:  for every layer: pull (predict) -> forward -> push;  then loss, backward,
+commit), or strings the C entry points together in that order where the epoch has other
+steps in between.  It contains no arithmetic of its own.
 """
 from __future__ import annotations
 
@@ -56,13 +57,15 @@ class SatEpoch:
         self.loss_sum = torch.zeros(1, dtype=torch.float64, device=dev)
         self.X = None
         self.labels = None
+        self._epoch_key = None
+        self._epoch_buf = None
 
     def close(self):
         """Destroys the context and drops the activation / gradient buffers (sizes and offsets stay readable)."""
         if self.ctx is not None:
             B.sat_destroy(self.ctx)
             self.ctx = None
-        self.H = self.G = self.halo = self.X_in = self.X = self.labels = None
+        self.H = self.G = self.halo = self.X_in = self.X = self.labels = self._epoch_key = self._epoch_buf = None
         if hasattr(self, "gat_halo"):
             self.gat_halo = None
 
@@ -96,37 +99,24 @@ class SatEpoch:
         return t[self.inner_off[m]:self.inner_off[m + 1]]
 
     # ---- one epoch ----------------------------------------------------------------
+    def _described(self, W, b, pred) -> B.sat_epoch_buffers:
+        """The buffers of an epoch as the library takes them; made anew when any tensor behind them is another one."""
+        key = (self.X, self.labels, *W, *b, *(pred or ()), pred is None)
+        ptrs = [t.data_ptr() for t in W]
+        ptrs += [None if t is None else t.data_ptr() for t in b]
+        old = self._epoch_key
+        if old is None or len(old[0]) != len(key) or any(x is not y for x, y in zip(old[0], key)) or old[1] != ptrs:
+            kind = B.SAT_LOSS_SOFTMAX_CE if self.loss == "ce" else B.SAT_LOSS_SIGMOID_BCE
+            self._epoch_buf = B.make_epoch_buffers(self.dims, self.X, self.labels, kind, self.H[1:], self.G[1:], self.halo, W, b, self.gW, self.gb,
+                                                   pred, self.loss_sum)
+            self._epoch_key = (key, ptrs)
+        return self._epoch_buf
+
     def _forward_backward(self, m: int, W, b, pred, accumulate: int, reuse_state: int, grad_history: bool = False):
-        ctx, L = self.ctx, self.L
-        h_in = None
-        for l in range(1, L + 1):
-            act = (B.SAT_ACT_RELU | B.SAT_FWD_PUSH) if l < L else B.SAT_ACT_NONE
-            if l == 1:
-                # layer 1: in- and out-of-subgraph rows are raw features, exact; the layer reads both from the feature matrix
-                # itself (global id order) through the partition's inner and halo lists: no gathered copies, no pull
-                h_in, hv = self.X, None
-                act |= B.SAT_FWD_INPUT_GLOBAL
-            elif pred is None or pred[l - 2] is None:
-                hv = None                            # plain historical embeddings: the layer reads them from the ring itself
-                act |= B.SAT_FWD_HALO_CACHED
-            else:
-                hv = self.halo_view(l - 1, m)
-                B.sat_predict(ctx, l - 1, m, pred[l - 2], reuse_state, hv)  # pull predicted
-            h_out = self.rows(self.H[l], m)
-            # forward; for the cached layers the push of the boundary rows rides on the transform's epilogue
-            B.sat_layer_fwd(ctx, m, l, h_in, hv, W[l - 1], b[l - 1], act, h_out)
-            h_in = h_out
-        kind = B.SAT_LOSS_SOFTMAX_CE if self.loss == "ce" else B.SAT_LOSS_SIGMOID_BCE
-        g = self.rows(self.G[L], m)
-        B.sat_loss_grad(ctx, m, kind, self.rows(self.H[L], m), self.rows(self.labels, m), self.loss_sum, g)
-        for l in range(L, 0, -1):
-            g_in = self.rows(self.G[l - 1], m) if l > 1 else None
-            # the gradient handed down is written already multiplied by the ReLU mask of the layer below (no separate pass)
-            flags = accumulate | (B.SAT_BWD_MASK_G_IN if l > 1 else 0) | (B.SAT_BWD_G_OUT_MASKED if l < L else 0)
-            if grad_history and l > 1:
-                flags |= B.SAT_BWD_GRAD_HISTORY      # stale-gradient term of the Appendix's back-propagation
-            B.sat_layer_bwd(ctx, m, l, g, W[l - 1], self.gW[l - 1], self.gb[l - 1], flags, g_in, None)
-            g = g_in
+        """Forward and backward of one partition (or all) without the commit; accumulate and reuse_state: it is not the first one."""
+        assert bool(accumulate) == bool(reuse_state)
+        flags = (B.SAT_EPOCH_CONTINUE if accumulate else 0) | (B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0)
+        B.sat_epoch(self.ctx, self._described(W, b, pred), None if m == B.SAT_ALL_PARTS else [m], flags)
 
     def pred_update(self, pred, lr: float, max_steps: int = 1, min_gain: float | None = None, row_weight=None):
         """Algorithm 1 "Embedding predictor update", to be called after the pushes of an epoch and before the commit:
@@ -161,22 +151,21 @@ class SatEpoch:
         """All partitions per launch.  W, b: lists of CUDA tensors; pred: list of sat_pred_params or None.
         pred_lr: also run one predictor update (pred_update) before the ring is committed.
         grad_history: back-propagate with the stale-gradient term (gradient-side history of the previous epoch)."""
-        self.loss_sum.zero_()
+        flags = B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0
+        if pred_lr is None or pred is None:
+            flags |= B.SAT_EPOCH_COMMIT | (B.SAT_EPOCH_STEP if lr is not None else 0)
+            B.sat_epoch(self.ctx, self._described(W, b, pred), None, flags, lr or 0.0)
+            return
         self._forward_backward(B.SAT_ALL_PARTS, W, b, pred, 0, 0, grad_history)
-        if pred_lr is not None and pred is not None:
-            self.pred_update(pred, pred_lr)
+        self.pred_update(pred, pred_lr)
         B.sat_cache_commit(self.ctx)
         if lr is not None:
             B.sat_sgd_steps(self.ctx, list(W) + list(b), list(self.gW) + list(self.gb), lr)
 
     def step_per_partition(self, W, b, pred, order=None, lr: float | None = None, grad_history: bool = False):
         """Same epoch, one partition at a time (the LSTM state table is computed by the first call of every layer)."""
-        self.loss_sum.zero_()
-        for i, m in enumerate(order if order is not None else range(self.M)):
-            self._forward_backward(m, W, b, pred, 0 if i == 0 else 1, 0 if i == 0 else 1, grad_history)
-        B.sat_cache_commit(self.ctx)
-        if lr is not None:
-            B.sat_sgd_steps(self.ctx, list(W) + list(b), list(self.gW) + list(self.gb), lr)
+        flags = B.SAT_EPOCH_COMMIT | (B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0) | (B.SAT_EPOCH_STEP if lr is not None else 0)
+        B.sat_epoch(self.ctx, self._described(W, b, pred), order if order is not None else range(self.M), flags, lr or 0.0)
 
     # ---- graph-attention backbone ---------------------------------------------------
     def step_gat(self, params, pred, lr: float | None = None):
