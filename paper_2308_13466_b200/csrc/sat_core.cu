@@ -101,7 +101,7 @@ extern "C" sat_status sat_create(sat_ctx **out, int device, void *cuda_stream)
         delete ctx;
         return SAT_ENOMEM;
     }
-    cudaMemsetAsync(ctx->d_flag, 0, 4 * sizeof(int), ctx->stream);  // [0] validation flags, [1] kernel wait time-outs, [2] ticket of loss_finish
+    cudaMemsetAsync(ctx->d_flag, 0, 4 * sizeof(int), ctx->stream);  // [0] validation flags, [1] kernel wait time-outs, [2] ticket of loss_finish, [3] longest row (list_build)
     *out = ctx;
     return SAT_OK;
 }
@@ -193,6 +193,7 @@ extern "C" sat_status sat_destroy(sat_ctx *ctx)
     dev_free(&ctx->col);
     dev_free(&ctx->dinv);
     sat_free_buf(ctx->buf_partial);
+    sat_free_buf(ctx->buf_ticket);
     sat_free_buf(ctx->buf_gagg);
     sat_free_buf(ctx->buf_splitk);
     sat_free_buf(ctx->buf_lstm_c);

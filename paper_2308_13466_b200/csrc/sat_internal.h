@@ -132,8 +132,9 @@ struct SpmmList {
     int4 *item = nullptr;      // {row, partial slot or -1, first entry: low 32 bits, first entry: high 16 bits | entries << 16}
     int32_t *slot0 = nullptr;  // per row: first partial slot of a row with several runs (one allocation with the three below)
     int32_t *tot = nullptr;    // per row: runs of the row
-    int32_t *mrows = nullptr;  // rows with a few runs
-    int32_t *hrows = nullptr;  // rows with many runs
+    int32_t *mrows = nullptr;  // rows with a few runs that k_spmm_fixup adds
+    int32_t *hrows = nullptr;  // rows with many
+    int32_t last_max = 0;      // rows of up to this many runs are added inside k_spmm, by the run that ends last
     std::vector<int64_t> off;  // [4 x (M+1)] first item, first partial slot, first entry of mrows and of hrows of every partition
 };
 
@@ -213,7 +214,7 @@ struct sat_ctx {
 
     // ---- scratch ----
     DevBuf buf_codec_sizes, buf_codec_off, buf_codec_bytes;  // embedding codec scratch
-    DevBuf buf_partial, buf_gagg, buf_splitk, buf_lstm_c, buf_lstm_s, buf_lstm_w, buf_pred_a, buf_misc, buf_colsum, buf_dmask,
+    DevBuf buf_ticket, buf_partial, buf_gagg, buf_splitk, buf_lstm_c, buf_lstm_s, buf_lstm_w, buf_pred_a, buf_misc, buf_colsum, buf_dmask,
         buf_wsplit, buf_wsplit2, buf_wsplit3, buf_bias, buf_pred_train, buf_ghist_halo, buf_ghist_rows, buf_ghist_out, buf_gat, buf_gat_items;
 };
 

@@ -33,7 +33,7 @@ __device__ __forceinline__ void mask4(float4 &r, const uint32_t *__restrict__ om
 //   0  local CSR rows, all entries (forward)            1  their inner prefix (backward, P_in^T = P_in)
 //   2  their halo suffix (transposed predictor convolution; rows without one are not in the list and are not written)
 //   3  halo rows (halo-row CSR, columns = inner rows)    4  halo rows by cache slot, the self entry first
-// Rows longer than a chunk leave one un-scaled partial sum per run, added in run order by k_spmm_fixup (fixed order:
+// Rows longer than a chunk leave one un-scaled partial sum per run, added in run order by k_spmm_fixup or by the run that ends last (fixed order:
 // reproducible, and identical for one partition alone or all at once).
 //
 // Three things decide how fast such a list is walked (measured on the kernels below, graphs with the degree skew of the tests):
@@ -49,18 +49,23 @@ __device__ __forceinline__ void mask4(float4 &r, const uint32_t *__restrict__ om
 //    partial sum per (row, block) and the pass that adds them.
 // -------------------------------------------------------------------------------------
 #define LIST_WINDOW 2048
-#define FIXUP_HEAVY 16   /* rows with more runs than this are added by a thread block, the others by a thread per column */
+#define FIXUP_HEAVY 16      /* k_spmm_fixup: rows with more runs than this are added by a thread block, the others by a thread per column */
+#define LAST_RUN_MAX 64     /* small lists: up to this many runs the one that ends last adds them inside k_spmm (no second launch) */
 
 // Longest run of a list with `entries` entries over `rows` rows.  Short runs balance a launch, but every run of a longer row costs a
 // partial sum that is written and read again, so the length grows with the launch: 32 while the chip is not full and the longest
 // run is the launch's duration, 64 / 128 / 256 from 1 / 8 / 16 M entries (on a skewed graph of 32 M entries, 64-entry runs
 // moved 1.7 ms per epoch into the partial sums and gained 0.4 ms); and not below the mean row (rounded up to a power of two), so that an
-// ordinary row of a dense graph stays in one piece.
+// ordinary row of a dense graph stays in one piece (up to 512: 2 % of an epoch with 490 entries a row against 256).
+//
+// Small lists have no second launch: the run of a row that ends last adds the row's partial sums (epoch of 900 nodes 99 -> 89 us, of
+// 2708 nodes 285 -> 269); their chunk grows until every row has at most LAST_RUN_MAX runs.  Large lists keep k_spmm_fixup: the fence
+// and ticket of every partial run cost more there than a launch (32 M entries: +4 %).
 static int32_t list_chunk(int64_t entries, int64_t rows)
 {
     const int64_t M = (int64_t)1 << 20;
     int32_t c = entries <= M ? 32 : entries <= 8 * M ? 64 : entries <= 16 * M ? 128 : 256;
-    while (c < 256 && (int64_t)c * rows < entries) c <<= 1;
+    while (c < 512 && (int64_t)c * rows < entries) c <<= 1;
     return c;
 }
 
@@ -136,7 +141,7 @@ __global__ void k_list_count(ListRows L, ListPart P, const int32_t *__restrict__
 }
 
 __global__ void k_list_row_totals(const int32_t *__restrict__ count, ListPart P, int32_t *__restrict__ tot, int32_t *__restrict__ slots,
-                                  int32_t *__restrict__ multi, int32_t *__restrict__ heavy)
+                                  int32_t *__restrict__ multi, int32_t *__restrict__ heavy, int32_t last_max)
 {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= P.n_rows) return;
@@ -144,8 +149,9 @@ __global__ void k_list_row_totals(const int32_t *__restrict__ count, ListPart P,
     for (int32_t j = 0; j < P.n_blocks; ++j) s += count[(int64_t)j * P.n_rows + r];
     tot[P.row0 + r] = s;
     slots[P.row0 + r] = s > 1 ? s : 0;
-    multi[P.row0 + r] = s > 1 && s <= FIXUP_HEAVY ? 1 : 0;
-    heavy[P.row0 + r] = s > FIXUP_HEAVY ? 1 : 0;
+    const bool fixup = s > 1 && s > last_max;
+    multi[P.row0 + r] = fixup && s <= FIXUP_HEAVY ? 1 : 0;
+    heavy[P.row0 + r] = fixup && s > FIXUP_HEAVY ? 1 : 0;
 }
 
 __global__ void k_list_fill(ListRows L, ListPart P, const int32_t *__restrict__ lenc, const int32_t *__restrict__ count,
@@ -196,6 +202,19 @@ __global__ void k_list_offsets(const int64_t *__restrict__ cbase, const int64_t 
     out[3 * (M + 1) + m] = hrow_off[row_off[m]];
 }
 
+// longest row of a list
+__global__ void k_list_max(ListRows L, int64_t n_rows, int32_t *__restrict__ out)
+{
+    int32_t mx = 0;
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_rows; r += (int64_t)gridDim.x * blockDim.x) {
+        int64_t rb, re;
+        list_row(L, r, &rb, &re);
+        mx = max(mx, (int32_t)(re - rb));
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, mx);
+}
+
 // orders the items of one window by length, longest first (a counting sort; the order among equal lengths does not matter)
 __global__ void __launch_bounds__(256) k_list_sort(int4 *__restrict__ item, int64_t item0, int64_t n_items)
 {
@@ -212,7 +231,7 @@ __global__ void __launch_bounds__(256) k_list_sort(int4 *__restrict__ item, int6
         const int64_t i = w0 + threadIdx.x + 256 * k;
         if (i < w1) {
             it[k] = item[i];
-            atomicAdd(&head[256 - (it[k].w >> 16)], 1);   // bin 0 = the longest possible run (256 entries)
+            atomicAdd(&head[256 - (it[k].w >> 17)], 1);   // bin 0 = the longest possible run (512 entries); pairs of lengths share a bin
         }
     }
     __syncthreads();
@@ -233,7 +252,7 @@ __global__ void __launch_bounds__(256) k_list_sort(int4 *__restrict__ item, int6
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int64_t i = w0 + threadIdx.x + 256 * k;
-        if (i < w1) item[w0 + atomicAdd(&head[256 - (it[k].w >> 16)], 1)] = it[k];
+        if (i < w1) item[w0 + atomicAdd(&head[256 - (it[k].w >> 17)], 1)] = it[k];
     }
 }
 
@@ -309,8 +328,21 @@ static sat_status list_build(sat_ctx *ctx, const ListKey &want, SpmmList **out)
     const int64_t n_rows = halo_rows ? ctx->nb : n;
     const int64_t cut = ctx->h_hrow_off.empty() ? 0 : ctx->h_hrow_off[M], all = ctx->nnz + n;
     const int64_t entries = mode == 0 ? all : mode == 1 ? all - cut : mode == 4 ? cut + ctx->nb : cut;
-    const int32_t chunk = list_chunk(entries, mode == 2 ? (ctx->n_slots > 0 ? ctx->n_slots : 1) : (n_rows > 0 ? n_rows : 1));
+    int32_t chunk = list_chunk(entries, mode == 2 ? (ctx->n_slots > 0 ? ctx->n_slots : 1) : (n_rows > 0 ? n_rows : 1));
     ListRows L{halo_rows ? ctx->hrow_ptr : ctx->lrowptr, ctx->inner_cnt, mode};
+    int32_t last_max = 0;
+    if (chunk == 32 && n_rows > 0) {
+        last_max = LAST_RUN_MAX;
+        // a small launch: runs up to 128 entries where that lets the last run of the longest row do the adding (no second launch)
+        int32_t longest = 0;
+        SAT_CUDA(ctx, cudaMemsetAsync(ctx->d_flag + 3, 0, sizeof(int32_t), ctx->stream));
+        k_list_max<<<(unsigned)std::min<int64_t>(cdiv64(n_rows, 256), 148), 256, 0, ctx->stream>>>(L, n_rows, ctx->d_flag + 3);
+        SAT_LAUNCHED(ctx);
+        SAT_CUDA(ctx, cudaMemcpyAsync(&longest, ctx->d_flag + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+        SAT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        const int32_t want = (int32_t)cdiv64(cdiv64(longest, LAST_RUN_MAX), 8) * 8;
+        if (want > chunk && want <= 128) chunk = want;
+    }
     std::vector<ListPart> parts((size_t)M);
     std::vector<int64_t> off(2 * ((size_t)M + 1), 0);   // [first count | first row] of every partition
     int64_t *cbase = off.data(), *row_off = cbase + M + 1;
@@ -329,6 +361,7 @@ static sat_status list_build(sat_ctx *ctx, const ListKey &want, SpmmList **out)
     SpmmList l;
     l.asked = want;
     l.key = key;
+    l.last_max = last_max;
     auto cleanup = [&](bool drop) {
         cudaFree(tmp);
         if (drop) { cudaFree(l.item); cudaFree(l.slot0); }
@@ -363,7 +396,7 @@ static sat_status list_build(sat_ctx *ctx, const ListKey &want, SpmmList **out)
         const ListPart &P = parts[m];
         if (P.n_rows == 0) continue;
         k_list_count<<<(unsigned)cdiv64((int64_t)P.n_rows * P.n_blocks, 256), 256, 0, ctx->stream>>>(L, P, ctx->lenc, count + cbase[m]);
-        k_list_row_totals<<<(unsigned)cdiv64(P.n_rows, 256), 256, 0, ctx->stream>>>(count + cbase[m], P, l.tot, slots, multi, heavy);
+        k_list_row_totals<<<(unsigned)cdiv64(P.n_rows, 256), 256, 0, ctx->stream>>>(count + cbase[m], P, l.tot, slots, multi, heavy, l.last_max);
         ctx->launches += 2;
     }
     LB_CUDA(cudaGetLastError());
@@ -413,7 +446,7 @@ static sat_status list_build(sat_ctx *ctx, const ListKey &want, SpmmList **out)
 // (blockIdx.y).  Every lane reads the 8-byte entry itself (one broadcast transaction per group; sharing it through two
 // shuffles was slower below 256 columns and equal there), U entries in flight, packed fp32 FMAs.
 //   single-run rows write  out[row] = scale[row] * sum_e w_e * src[col_e]  (masked on request)
-//   runs of longer rows write their un-scaled partial sum to `partial`; k_spmm_fixup adds them in run order.
+//   runs of longer rows write their un-scaled partial sum to `partial`, added in run order afterwards.
 // Bound by the L2 -> SM path where the sources fit the L2 (dense graphs: 20 TB/s of gathered rows at d = 256, the rate of random
 // rows out of an L2-resident buffer), by the latency of the short rows' chains (descriptor -> entries -> rows) and DRAM
 // elsewhere.  Measured and dropped: cp.async rings (7 % faster than this at d = 256 on sparse graphs, 35 % slower on dense
@@ -441,11 +474,32 @@ __device__ __forceinline__ float4 spmm_epilogue(const SpmmEpilogue &ep, int64_t 
     return make_float4(x[0], x[1], x[2], x[3]);
 }
 
+// K entries: their columns and weights, their rows (all in flight together), the sums
+template <int G, int NV, int K, typename F>
+__device__ __forceinline__ void spmm_step(const int2 *__restrict__ ents, const F &row_of, int col, int32_t d4, float4 (&acc)[NV])
+{
+    int2 q[K];
+#pragma unroll
+    for (int u = 0; u < K; ++u) q[u] = __ldg(ents + u);
+    float4 x[K][NV];
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        const float4 *src = row_of(q[u].x);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) x[u][v] = col + v * G < d4 ? __ldg(src + v * G) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) fma4(acc[v], __int_as_float(q[u].y), x[u][v]);
+}
+
 template <int G, int NV, int U, int MINB, bool EPI>
 __global__ void __launch_bounds__(256, MINB)
 k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const int2 *__restrict__ ent, const float *__restrict__ scale, int32_t n,
        int32_t d4, const float *__restrict__ in_base, int64_t ld_in, const float *__restrict__ halo_base, int64_t ld_halo, float *__restrict__ out_base,
-       int64_t ld_out, float *__restrict__ partial, const uint32_t *__restrict__ omask, int32_t omask_words, SpmmEpilogue ep, DbgLimits dbg)
+       int64_t ld_out, float *partial, const int32_t *__restrict__ slot0, const int32_t *__restrict__ tot, int32_t *ticket,
+       int32_t last_max, const uint32_t *__restrict__ omask, int32_t omask_words, SpmmEpilogue ep, DbgLimits dbg)
 {
     sat_grid_wait();
     const int lane = threadIdx.x & (G - 1);
@@ -470,47 +524,71 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
 #pragma unroll
     for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     int32_t e = 0;
-    for (; e + U <= len; e += U) {
-        int2 q[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) q[u] = __ldg(ents + e + u);
-        float4 x[U][NV];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const float4 *src = row_of(q[u].x);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) x[u][v] = col + v * G < d4 ? __ldg(src + v * G) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int v = 0; v < NV; ++v) fma4(acc[v], __int_as_float(q[u].y), x[u][v]);
+    for (; e + U <= len; e += U) spmm_step<G, NV, U>(ents + e, row_of, col, d4, acc);
+    // the remainder by halves: each step is one chain of latencies (entry -> row), whatever its width
+    if (U > 4 && ((len - e) & 4)) {
+        spmm_step<G, NV, U < 4 ? U : 4>(ents + e, row_of, col, d4, acc);
+        e += 4;
     }
-    for (; e < len; ++e) {
-        const int2 q = __ldg(ents + e);
-        const float4 *src = row_of(q.x);
+    if ((len - e) & 2) {
+        spmm_step<G, NV, 2>(ents + e, row_of, col, d4, acc);
+        e += 2;
+    }
+    if ((len - e) & 1) spmm_step<G, NV, 1>(ents + e, row_of, col, d4, acc);
+    float4 *pr = reinterpret_cast<float4 *>(partial) + ((int64_t)it.y - slot_base) * d4 + col;
+    if (it.y >= 0) {
+        // a run of a longer row: leave the partial sum.  Small launches: the group that finishes a row last (by its ticket) adds all of
+        // them in run order.  (In large ones the fences in front of the tickets cost more than the second launch.)
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-            if (col + v * G < d4) fma4(acc[v], __int_as_float(q.y), __ldg(src + v * G));
-    }
-    if (it.y < 0) {
-        const int64_t row = SAT_IDX((int64_t)it.x, dbg.out_lo, dbg.out_hi, dbg.status);
-        const float s = EPI ? 1.f : __ldg(scale + row);
-        float4 *o = reinterpret_cast<float4 *>(out_base + row * ld_out) + col;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            if (col + v * G < d4) {
-                float4 r = make_float4(s * acc[v].x, s * acc[v].y, s * acc[v].z, s * acc[v].w);
-                if (EPI) r = spmm_epilogue(ep, row, col + v * G, r);
-                else if (omask) mask4(r, omask, row * omask_words, col + v * G);
-                o[v * G] = r;
-            }
+            if (col + v * G < d4) pr[v * G] = acc[v];
+        if (last_max == 0) return;
+        const int32_t first = __ldg(slot0 + it.x), cnt = __ldg(tot + it.x);
+        if (cnt > last_max) return;   // k_spmm_fixup
+        const unsigned mask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+        __threadfence();
+        __syncwarp(mask);
+        int32_t before = 0;
+        int32_t *t = ticket + (first - slot_base) * gridDim.y + blockIdx.y;
+        if (lane == 0) {
+            before = atomicAdd(t, 1);
+            if (before == cnt - 1) *t = 0;   // zero again for the next launch
         }
-    } else {
-        float4 *o = reinterpret_cast<float4 *>(partial) + ((int64_t)it.y - slot_base) * d4 + col;
+        before = __shfl_sync(mask, before, 0, G);
+        if (before != cnt - 1) return;
+        __threadfence();
+        const float4 *p0 = reinterpret_cast<const float4 *>(partial) + ((int64_t)first - slot_base) * d4 + col;
 #pragma unroll
-        for (int v = 0; v < NV; ++v)
-            if (col + v * G < d4) o[v * G] = acc[v];
+        for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int32_t q = 0; q < cnt; q += 4) {
+            float4 x[4][NV];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < NV; ++v)
+                    x[u][v] = q + u < cnt && col + v * G < d4 ? __ldcg(p0 + (int64_t)(q + u) * d4 + v * G) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    acc[v].x += x[u][v].x;
+                    acc[v].y += x[u][v].y;
+                    acc[v].z += x[u][v].z;
+                    acc[v].w += x[u][v].w;
+                }
+        }
+    }
+    const int64_t row = SAT_IDX((int64_t)it.x, dbg.out_lo, dbg.out_hi, dbg.status);
+    const float s = EPI ? 1.f : __ldg(scale + row);
+    float4 *o = reinterpret_cast<float4 *>(out_base + row * ld_out) + col;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        if (col + v * G < d4) {
+            float4 r = make_float4(s * acc[v].x, s * acc[v].y, s * acc[v].z, s * acc[v].w);
+            if (EPI) r = spmm_epilogue(ep, row, col + v * G, r);
+            else if (omask) mask4(r, omask, row * omask_words, col + v * G);
+            o[v * G] = r;
+        }
     }
 }
 
@@ -596,16 +674,16 @@ struct SpmmArgs {
 };
 
 template <int G, int NV, int U, int MINB>
-static void launch_spmm(sat_ctx *ctx, const int4 *items, int32_t n_items, int64_t slot_base, int32_t d4, const SpmmArgs &a, float *partial)
+static void launch_spmm(sat_ctx *ctx, const SpmmList &l, const int4 *items, int32_t n_items, int64_t slot_base, int32_t d4, const SpmmArgs &a, float *partial)
 {
     dim3 grid((unsigned)cdiv64((int64_t)n_items * G, 256), (unsigned)cdiv64(d4, G * NV));
     const DbgLimits dbg = dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1);
     if (a.scale)
         sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, false>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
-                                                                     a.out_base, a.ld_out, partial, a.omask, a.omask_words, a.ep, dbg);
+                                                                     a.out_base, a.ld_out, partial, l.slot0, l.tot, (int32_t *)ctx->buf_ticket.p, l.last_max, a.omask, a.omask_words, a.ep, dbg);
     else
         sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, true>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
-                                                                    a.out_base, a.ld_out, partial, a.omask, a.omask_words, a.ep, dbg);
+                                                                    a.out_base, a.ld_out, partial, l.slot0, l.tot, (int32_t *)ctx->buf_ticket.p, l.last_max, a.omask, a.omask_words, a.ep, dbg);
 }
 
 // walks partitions [v.p0, v.p1) of a list
@@ -622,20 +700,28 @@ static sat_status run_list(sat_ctx *ctx, const PartView &v, const SpmmList &l, i
         // sized for all partitions at once: calls on one partition after the other would grow it again and again
         SAT_TRY(sat_ensure(ctx, ctx->buf_partial, (size_t)l.off[M1 + ctx->M] * d4 * 16));
         partial = (float *)ctx->buf_partial.p;
+        // a ticket per (slot, column slice), all zero between launches
+        const size_t need = l.last_max > 0 ? (size_t)l.off[M1 + ctx->M] * cdiv64(d4, 64) * sizeof(int32_t) : 0;
+        if (need > ctx->buf_ticket.bytes) {
+            SAT_TRY(sat_ensure(ctx, ctx->buf_ticket, need));
+            SAT_CUDA(ctx, cudaMemsetAsync(ctx->buf_ticket.p, 0, ctx->buf_ticket.bytes, ctx->stream));
+        }
     }
     // Lane groups by width.  Above 256 columns the launch walks slices of 256: a slice's sources fit the L2 twice as often, and two
     // passes of the 2-vector shape beat one pass of a 4-vector one (d = 512: 484 -> 391 us on the sparse graph, 1,334 -> 1,190 on
     // the dense one).
     const int4 *items = l.item + item0;
-#define ARGS ctx, items, (int32_t)n_items, slot_base, d4, a, partial
-    if (d4 <= 4) launch_spmm<4, 1, 4, 6>(ARGS);
-    else if (d4 <= 8) launch_spmm<8, 1, 4, 6>(ARGS);
-    else if (d4 <= 16) launch_spmm<16, 1, 4, 6>(ARGS);
-    else if (d4 <= 32) launch_spmm<16, 2, 4, 5>(ARGS);
-    else launch_spmm<32, 2, 4, 5>(ARGS);
+#define ARGS ctx, l, items, (int32_t)n_items, slot_base, d4, a, partial
+    // A launch that leaves most of the chip idle is as long as its longest run: eight entries in flight per step then
+    const bool small = n_items * 32 <= 148 * 768;
+    if (d4 <= 4) small ? launch_spmm<4, 1, 8, 3>(ARGS) : launch_spmm<4, 1, 4, 6>(ARGS);
+    else if (d4 <= 8) small ? launch_spmm<8, 1, 8, 3>(ARGS) : launch_spmm<8, 1, 4, 6>(ARGS);
+    else if (d4 <= 16) small ? launch_spmm<16, 1, 8, 3>(ARGS) : launch_spmm<16, 1, 4, 6>(ARGS);
+    else if (d4 <= 32) small ? launch_spmm<16, 2, 8, 3>(ARGS) : launch_spmm<16, 2, 4, 5>(ARGS);
+    else small ? launch_spmm<32, 2, 8, 3>(ARGS) : launch_spmm<32, 2, 4, 5>(ARGS);
 #undef ARGS
     SAT_LAUNCHED(ctx);
-    if (n_slots > 0) {
+    if (n_hrows + n_mrows > 0) {
         sat_pdl(ctx->stream, k_spmm_fixup, (unsigned)(n_hrows * cdiv64(d4, 32) + cdiv64(n_mrows * d4, 256)), 256, 0)(
             l.hrows + hrow0, (int32_t)n_hrows, l.mrows + mrow0, (int32_t)n_mrows, l.slot0, l.tot, slot_base, a.scale, d4, partial, a.out_base, a.ld_out, a.omask,
             a.omask_words, a.ep, dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1));
