@@ -209,7 +209,7 @@ struct TcEpilogue {
     const float *resid;  // C += resid[resid_idx[row]]  (row gather)
     const int32_t *resid_idx;
     int64_t ld_resid;
-    int32_t lstm_h;      // > 0: fused LSTM cell, C = hidden state [M x lstm_h], lstm_c = cell state
+    int32_t lstm_h;      // > 0: fused recurrent cell, C = hidden state [M x lstm_h], lstm_c = cell state (LSTM only)
     int lstm_first;
     float *lstm_c;       // cell state in the blocked layout of sat_cell_offset
     const float *addend; // [M x ld_addend] added to the gate pre-activations (cached input projection), or null
@@ -255,10 +255,11 @@ struct TcShared {
 // LSTM input projection) keep a ring of 32 x 32 side tiles per epilogue warp in shared memory, filled by cp.async ahead of
 // the consumer: one chunk in flight per warp left the loads latency-bound at ~2 TB/s.  Those variants contract over a
 // small K (the predictor width), so they give up main-loop stages for the ring.
-enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_LSTM = 2, EPI_LSTM_ADD = 3, EPI_PUSH = 4 };   // EPI_PUSH = EPI_PLAIN + a second copy of the rows that have a cache slot
+enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_LSTM = 2, EPI_LSTM_ADD = 3, EPI_PUSH = 4, EPI_GRU = 5 };   // EPI_PUSH = EPI_PLAIN + a second copy of the rows that have a cache slot
 template <int EPI> struct TckCfg { static constexpr int stages = 4, ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = epi_warps * 4096; };
 template <> struct TckCfg<EPI_RESID> { static constexpr int stages = 2, ring = 1, conv_warps = 2, epi_warps = 12, out_bytes = epi_warps * 4096; };
 template <> struct TckCfg<EPI_LSTM> { static constexpr int stages = 4, ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = 0; };
+template <> struct TckCfg<EPI_GRU> : TckCfg<EPI_LSTM> {};
 template <> struct TckCfg<EPI_LSTM_ADD> { static constexpr int stages = 2, ring = 2, conv_warps = 2, epi_warps = 12, out_bytes = 0; };
 static_assert(TckCfg<EPI_PLAIN>::stages % TCK_CONV_GROUPS == 0 && TckCfg<EPI_RESID>::stages % TCK_CONV_GROUPS == 0 &&
                   TckCfg<EPI_LSTM>::stages % TCK_CONV_GROUPS == 0 && TckCfg<EPI_LSTM_ADD>::stages % TCK_CONV_GROUPS == 0,
@@ -404,7 +405,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         // ---------------- epilogue ----------------
         // warp w reads TMEM lanes 32 (w % 4) .. +31 = rows of the tile, one row per thread; the warps of a lane quadrant
         // take alternate 32-column chunks.
-        constexpr bool LSTM = EPI == EPI_LSTM || EPI == EPI_LSTM_ADD;
+        constexpr bool LSTM = EPI == EPI_LSTM || EPI == EPI_LSTM_ADD || EPI == EPI_GRU;   // a recurrent cell
         const int e = warp - EPI_WARP0;
         const int q = warp & 3;
         const int c_first = 32 * (e >> 2);
@@ -515,13 +516,13 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 }
             }
             float4 side[8], cside[2];
-            // previous cell state of the next chunk, fetched one chunk ahead (two 128-bit loads per thread)
+            // previous cell state (GRU: hidden state) of the next chunk, fetched one chunk ahead (two 128-bit loads per thread)
             auto load_cell = [&](int c0) {
                 if (LSTM) {
                     cside[0] = cside[1] = zero4;
                     const int32_t j0 = (n0 + c0) >> 2;
                     if (row_ok && lstm_full && !ep.lstm_first && j0 + 7 < ep.lstm_h) {
-                        const float *cp = ep.lstm_c + sat_cell_offset(row, j0, ep.lstm_h);
+                        const float *cp = EPI == EPI_GRU ? crow + j0 : ep.lstm_c + sat_cell_offset(row, j0, ep.lstm_h);
                         cside[0] = *reinterpret_cast<const float4 *>(cp);
                         cside[1] = *reinterpret_cast<const float4 *>(cp + 4);
                     }
@@ -566,12 +567,19 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         if (!ep.lstm_first && !full) {
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
-                                if (j0 + u < ep.lstm_h) cprev[u] = ep.lstm_c[sat_cell_offset(row, j0 + u, ep.lstm_h)];
+                                if (j0 + u < ep.lstm_h) cprev[u] = EPI == EPI_GRU ? crow[j0 + u] : ep.lstm_c[sat_cell_offset(row, j0 + u, ep.lstm_h)];
                         }
                         if (c0 + CHUNK_STEP < bn) load_cell(c0 + CHUNK_STEP);
                         float sv[8], cv[8];
 #pragma unroll
                         for (int u = 0; u < 8; ++u) {
+                            if (EPI == EPI_GRU) {   // (r, z, n from the input, n from the state)
+                                const float gr = 1.f / (1.f + expf(-__uint_as_float(r[4 * u])));
+                                const float gz = 1.f / (1.f + expf(-__uint_as_float(r[4 * u + 1])));
+                                const float gn = tanhf(__uint_as_float(r[4 * u + 2]) + gr * __uint_as_float(r[4 * u + 3]));
+                                sv[u] = (1.f - gz) * gn + gz * cprev[u];
+                                continue;
+                            }
                             const float gi = sigmoid_fast(__uint_as_float(r[4 * u]));
                             const float gf = sigmoid_fast(__uint_as_float(r[4 * u + 1]));
                             const float gg = tanh_fast(__uint_as_float(r[4 * u + 2]));
@@ -580,17 +588,19 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                             sv[u] = go * tanh_fast(cv[u]);
                         }
                         if (full) {
-                            float4 *cd = reinterpret_cast<float4 *>(ep.lstm_c + sat_cell_offset(row, j0, ep.lstm_h));
                             float4 *sd = reinterpret_cast<float4 *>(ep.C + row * ep.ldc + j0);
-                            cd[0] = make_float4(cv[0], cv[1], cv[2], cv[3]);
-                            cd[1] = make_float4(cv[4], cv[5], cv[6], cv[7]);
+                            if (EPI != EPI_GRU) {
+                                float4 *cd = reinterpret_cast<float4 *>(ep.lstm_c + sat_cell_offset(row, j0, ep.lstm_h));
+                                cd[0] = make_float4(cv[0], cv[1], cv[2], cv[3]);
+                                cd[1] = make_float4(cv[4], cv[5], cv[6], cv[7]);
+                            }
                             sd[0] = make_float4(sv[0], sv[1], sv[2], sv[3]);
                             sd[1] = make_float4(sv[4], sv[5], sv[6], sv[7]);
                         } else {
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
                                 if (j0 + u < ep.lstm_h) {
-                                    ep.lstm_c[sat_cell_offset(row, j0 + u, ep.lstm_h)] = cv[u];
+                                    if (EPI != EPI_GRU) ep.lstm_c[sat_cell_offset(row, j0 + u, ep.lstm_h)] = cv[u];
                                     ep.C[row * ep.ldc + j0 + u] = sv[u];
                                 }
                         }
@@ -1005,17 +1015,20 @@ __global__ void k_pack_bias(const float *__restrict__ bias, int32_t n, int32_t n
 //   transpose = 1: W is [K x N] row-major (ldw) -> B[n][k] = W[k][n]          (C = A W)
 //   transpose = 0: W is [N x K] row-major (ldw) -> B[n][k] = W[n][k]          (C = A W^T)
 // A second source W2 (same orientation, k2 rows) continues along K at column offset k1_pad.
+// gate_h > 0: packed column 4 j + g is gate g of hidden unit j.  gates = 4: the sources have the columns i | f | g | o.  gates = 3 (GRU,
+// sources r | z | n): the candidate's two parts stay apart, column 4 j + 2 takes n of the first source only and 4 j + 3 n of the second.
 __global__ void k_split_weights(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t k1_pad, const float *__restrict__ W2,
-                                int64_t ldw2, int32_t k2, int32_t n, int32_t n_pad, int32_t k_pad, int transpose, int32_t gate_h,
+                                int64_t ldw2, int32_t k2, int32_t n, int32_t n_pad, int32_t k_pad, int transpose, int32_t gate_h, int gates,
                                 float *__restrict__ hi, float *__restrict__ lo)
 {
     sat_grid_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)n_pad * k_pad) return;
     const int32_t np = (int32_t)(i / k_pad), kk = (int32_t)(i - (int64_t)np * k_pad);
-    const int32_t nn = gate_h > 0 ? (np & 3) * gate_h + (np >> 2) : np;  // packed row -> logical column
+    const int32_t g = np & 3;
+    const int32_t nn = gate_h > 0 ? (gates == 3 && g == 3 ? 2 : g) * gate_h + (np >> 2) : np;  // packed row -> logical column
     float x = 0.f;
-    if (np < n) {
+    if (np < n && !(gates == 3 && g == (kk < k1 ? 3 : 2))) {
         if (kk < k1) x = transpose ? W[(int64_t)kk * ldw + nn] : W[(int64_t)nn * ldw + kk];
         else if (kk >= k1_pad && kk - k1_pad < k2) x = transpose ? W2[(int64_t)(kk - k1_pad) * ldw2 + nn] : W2[(int64_t)nn * ldw2 + (kk - k1_pad)];
     }
@@ -1098,7 +1111,7 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
 }
 
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
-                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h)
+                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h, int gates)
 {
     const int32_t k1_pad = W2 ? (k1 + TC_BK - 1) / TC_BK * TC_BK : k1;
     const int32_t k_tot = k1_pad + (W2 ? k2 : 0);
@@ -1112,7 +1125,7 @@ sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1,
     out->ld = k_pad;
     out->n_pad = n_pad;
     sat_pdl(ctx->stream, k_split_weights, (unsigned)cdiv64((int64_t)n_pad * k_pad, 256), 256, 0)(W, ldw, k1, k1_pad, W2, ldw2, k2, n, n_pad, k_pad,
-                                                                                          transpose, gate_h, out->hi, out->lo);
+                                                                                          transpose, gate_h, gates, out->hi, out->lo);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
@@ -1172,7 +1185,7 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     // algorithmic bytes: operands once, results once.  Plain: A, B, C.  Gathered residual: + the residual rows.  LSTM cell:
     // the output is the hidden state [m x h] plus the cell state read and written, and the cached projection if it is added.
     double alg_bytes = 4.0 * ((double)m * (k1 + k2) + (double)(k1 + k2) * n);
-    if (eh.lstm_h > 0) alg_bytes += 4.0 * (double)m * eh.lstm_h * (eh.lstm_first ? 2.0 : 3.0) + (eh.addend ? 4.0 * (double)m * n : 0.0);
+    if (eh.lstm_h > 0) alg_bytes += 4.0 * (double)m * eh.lstm_h * (eh.gru ? 1.0 : eh.lstm_first ? 2.0 : 3.0) + (eh.addend ? 4.0 * (double)m * n : 0.0);
     else alg_bytes += 4.0 * (double)m * n * (eh.resid_idx ? 2.0 : 1.0);
     ProfScope prof(ctx, family, alg_bytes, 2.0 * (double)m * n * (k1 + k2));
     CUtensorMap mA, mA2, mB, mBlo, mC;
@@ -1209,8 +1222,8 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.lstm_c = eh.lstm_c;
     ep.addend = eh.addend;
     ep.ld_addend = eh.ld_addend;
-    if (eh.lstm_h > 0 && ((!eh.bias && !eh.addend) || !eh.lstm_c || n != 4 * eh.lstm_h || (eh.addend && (eh.ld_addend & 3))))
-        return sat_fail(ctx, SAT_EINVAL, "fused LSTM epilogue needs bias or addend, cell state and n = 4h");
+    if (eh.lstm_h > 0 && ((!eh.bias && !eh.addend) || (eh.gru ? eh.addend != nullptr : !eh.lstm_c) || n != 4 * eh.lstm_h || (eh.addend && (eh.ld_addend & 3))))
+        return sat_fail(ctx, SAT_EINVAL, "fused recurrent epilogue needs bias or addend, cell state (LSTM) and n = 4h");
     if (eh.resid_idx && (eh.mask_out || eh.lstm_h > 0))
         return sat_fail(ctx, SAT_EINVAL, "gathered-residual epilogue cannot be combined with a mask output or the LSTM cell");
     ep.relu = eh.relu;
@@ -1229,6 +1242,7 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     L.m = m; L.n = n; L.nkb1 = nkb1; L.nkb2 = nkb2; L.bn = bn; L.n_tiles_n = n_tiles_n; L.n_tiles = n_tiles;
     L.grid = grid;
     L.stage_bytes = stage_bytes;
+    if (eh.gru) return launch_tck<EPI_GRU>(ctx, L, ep);
     if (ep.lstm_h > 0) return ep.addend ? launch_tck<EPI_LSTM_ADD>(ctx, L, ep) : launch_tck<EPI_LSTM>(ctx, L, ep);
     if (ep.resid_idx) return launch_tck<EPI_RESID>(ctx, L, ep);
     if (ep.push_dst) return launch_tck<EPI_PUSH>(ctx, L, ep);

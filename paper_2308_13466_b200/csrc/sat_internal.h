@@ -502,7 +502,8 @@ struct TcEpilogueHost {
     // fused LSTM cell (the weights must have been packed with gate interleave): the n = 4h outputs of a row are the gate
     // pre-activations; the epilogue applies c = f c + i g, s = o tanh(c) and writes s to C [m x h] and c to lstm_c [m x h]
     int32_t lstm_h = 0;
-    int lstm_first = 0;                // first step: previous cell state is zero
+    int lstm_first = 0;                // first step: previous cell state (GRU: hidden state) is zero
+    int gru = 0;                       // GRU cell instead (weights packed with gates = 3): C is also the previous hidden state, no lstm_c
     float *lstm_c = nullptr;
     const float *addend = nullptr;     // dense [m x ld_addend], added to the accumulators before the LSTM cell (row-aligned)
     int32_t ld_addend = 0;
@@ -525,9 +526,9 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
                          float *dst, int32_t ld_dst, float *colsum, int accumulate, const float *act = nullptr, int32_t ld_act = 0);
 // weight planes in `buf`; transpose = 1 for W given as [K x N], 0 for [N x K]; optional second source continuing along K
 // gate_h > 0: the n = 4 gate_h columns (gate blocks i | f | g | o) are interleaved so that packed column 4 j + gate is gate `gate`
-// of hidden unit j (what the fused LSTM epilogue expects)
+// of hidden unit j (what the fused LSTM epilogue expects); gates = 3: the GRU's, see k_split_weights
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
-                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0);
+                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0, int gates = 4);
 sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out);
 // C[m x n] = [A | A2] B^T (+ epilogue)
 sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32_t lda, int32_t k1, const float *A2, int32_t lda2, int32_t k2,

@@ -403,7 +403,10 @@ __global__ void k_gru_cell(const float *__restrict__ gx, const float *__restrict
     s[t] = (1.f - z) * n + z * sp;
 }
 
-// GRU-GCN variant: two plain contractions per step (input side with the bias, hidden side) and the cell kernel
+// GRU-GCN variant.  With one tile over all gates (h <= 64) a step is one contraction over [x | s] with 4 h outputs -- r, z and the
+// candidate's input and state parts apart, since r multiplies only the latter -- and the cell in its epilogue, the state updated in place as
+// for the LSTM.  A third of the B operand is zeros, which costs less than the two pre-activation matrices written and read again (84671
+// nodes, 256 -> 64, four steps: epoch 2092 -> 1786 us).  Wider: two plain contractions per step (input side with the bias, hidden side) and the cell kernel.
 static sat_status run_gru(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p)
 {
     const int32_t h = p->h, d = c->width;
@@ -420,6 +423,24 @@ static sat_status run_gru(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p)
     const int32_t k = ctx->n_valid < ctx->tau ? ctx->n_valid : ctx->tau;
     if (k == 0 || rows == 0) {
         SAT_CUDA(ctx, cudaMemsetAsync(c->S, 0, (size_t)(rows > 0 ? rows : 1) * h * sizeof(float), ctx->stream));
+        c->S_valid = true;
+        return SAT_OK;
+    }
+    if (sat_use_tc(4 * h, d) && 4 * h <= 256) {
+        TcWeights W1, W2;   // first step: x alone
+        SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, h, 3));
+        if (k > 1) SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, p->Uh, 3 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, h, 3));
+        for (int32_t t = 0; t < k; ++t) {
+            TcEpilogueHost eh;
+            eh.C = c->S;
+            eh.ldc = h;
+            eh.bias = p->b;   // b_r | b_z | b_n | b_hn: the interleave of four gates
+            eh.lstm_h = h;
+            eh.gru = 1;
+            eh.lstm_first = t == 0;
+            SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, ring_buf(ctx, c, ring_index(ctx, k - 1 - t)), c->ld, d, t == 0 ? nullptr : c->S, h, t == 0 ? 0 : h,
+                                t == 0 ? W1 : W2, eh, SATK_GEMM_NN));
+        }
         c->S_valid = true;
         return SAT_OK;
     }

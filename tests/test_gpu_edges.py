@@ -204,3 +204,48 @@ def test_losses(B, rows, C, kind):
         B.sat_sync_status(ctx)
     finally:
         B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("d", [16, 17, 100, 256])
+@pytest.mark.parametrize("h", [4, 8, 20, 60, 64, 68])       # 4 h gate columns: one tile up to h = 64, contractions and a cell kernel above
+@pytest.mark.parametrize("steps", [1, 2, 5])
+def test_gru_state(B, d, h, steps):
+    """sat_predict_state against the cell in fp64.  With e the error of a pre-activation (bound of the module's docstring plus what the
+    previous state brings through Uh) and sigma' <= 1/4, tanh' <= 1:  |ds| <= e_z / 2 + e_n + e_hn + |hn| e_r / 4 + |ds_prev| + 2^-20."""
+    n, M = 700, 3
+    A = _graph([300, 40], n)
+    rng = np.random.default_rng(d + h)
+    part = rng.integers(0, M, n).astype(np.int32)
+    perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+    W, Uh, b = rng.standard_normal((d, 3 * h)) / d ** 0.5, rng.standard_normal((h, 3 * h)) / h ** 0.5, rng.standard_normal(4 * h) / 4
+    Wg, bg = np.zeros((h, d)), np.zeros(d)
+    W, Uh, b, Wg, bg = (x.astype(np.float32) for x in (W, Uh, b, Wg, bg))
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        B.sat_cache_init(ctx, [d], 5)
+        n_halo = sum(B.sat_part_sizes(ctx, m)[1] for m in range(M))
+        n_slots = B.sat_slot_map(ctx, n)[2]
+        for _ in range(steps):
+            B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, dev2d(rng.standard_normal((n, d)).astype(np.float32)[perm]))
+            B.sat_cache_commit(ctx)
+        snaps = [B.sat_cache_read(ctx, 1, age, n_slots, d).astype(np.float64) for age in range(steps - 1, -1, -1)]
+        params = B.make_pred_params(dev(W), dev(Uh), dev(b), dev(Wg), dev(bg), h, 0, B.SAT_CELL_GRU)
+        B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, params, 0, empty2d(n_halo, d))
+        S = B.sat_predict_state(ctx, 1, n_slots, h)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    s, ds = np.zeros((n_slots, h)), np.zeros((n_slots, h))
+    sig = lambda v: 1 / (1 + np.exp(-v))
+    U64 = Uh.astype(np.float64)
+    for x in snaps:
+        ax, ah = x @ W + b[:3 * h], s @ U64
+        e = ((d + h + 2) * U + 2.0 ** -20) * (np.abs(x) @ np.abs(W) + np.abs(s) @ np.abs(U64) + np.abs(b[:3 * h])) + ds @ np.abs(U64)
+        hn = ah[:, 2 * h:] + b[3 * h:]
+        r, z = sig(ax[:, :h] + ah[:, :h]), sig(ax[:, h:2 * h] + ah[:, h:2 * h])
+        cand = np.tanh(ax[:, 2 * h:] + r * hn)
+        ds = e[:, h:2 * h] / 2 + 2 * e[:, 2 * h:] + np.abs(hn) * e[:, :h] / 4 + ds + 2.0 ** -20
+        s = (1 - z) * cand + z * s
+    assert (np.abs(S - s) <= ds).all()
