@@ -7,7 +7,7 @@
 // (see "TF32 split of a shared-memory tile" below for the two variants).  Weights are repacked once per call into the
 // K-major operand layout.
 //
-//   k_gemm_tc_k   C[M x N] = A[M x K] B[N x K]^T   both operands K-major, 64-byte swizzle, BLOCK_K = 16, persistent
+//   k_gemm_tc_k   C[M x N] = A[M x K] B[N x K]^T   both operands K-major, 64-byte swizzle, BLOCK_K = 16, persistent CTA pairs
 //                 (layer transform, LSTM gates with two A operands or a cached projection, predictor output, input gradient)
 //   k_gemm_tc_mn  C[M x N] = A[R x M]^T B[R x N]   both operands MN-major, 128-byte swizzle with 32-byte atoms, split over R
 //                 (weight gradient)
@@ -72,6 +72,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, v
     if (!ok) return false;
     return mbar_wait(bar, parity, dead, status);
 }
+// every lane waits; the result is that of the whole warp
+__device__ __forceinline__ bool mbar_wait_all(uint64_t *bar, uint32_t parity, volatile int *dead, int *status)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, dead, status));
+}
 __device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int32_t x, int32_t y)
 {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
@@ -93,22 +98,71 @@ __device__ __forceinline__ void tma_store_wait_read()
     asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// One warp; GROUP = 2: one warp of each CTA of the pair, which get the same columns
+template <int GROUP>
+__device__ __forceinline__ void tc_alloc(uint32_t *base, uint32_t cols)
+{
+    if (GROUP == 2) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(base)), "r"(cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(base)), "r"(cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+}
+template <int GROUP>
+__device__ __forceinline__ void tc_dealloc(uint32_t base, uint32_t cols)
+{
+    if (GROUP == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+// arrives on the barrier once this thread's MMAs so far have completed; GROUP = 2: on that of both CTAs of the pair
+template <int GROUP>
 __device__ __forceinline__ void tc_commit(uint64_t *bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+    if (GROUP == 2)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+                     "h"((uint16_t)3)
+                     : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// D (+)= A B.  USE_A: what becomes of the A tile in the tensor core's operand collector -- 1: it stays, 2: it is taken from there for
+// the last time.  (The two products with A hi read it from shared memory once: 1.3 % of a 179250 x 512 x 512 contraction.)
+#define TC_MMA_ASM(G, COLLECTOR)                                                                       \
+    asm volatile(                                                                                      \
+        "{\n\t"                                                                                        \
+        ".reg .pred p;\n\t"                                                                            \
+        "setp.ne.b32 p, %4, 0;\n\t"                                                                    \
+        "tcgen05.mma.cta_group::" G ".kind::tf32" COLLECTOR " [%0], %1, %2, %3, p;\n\t"                     \
+        "}" ::"r"(tmem_d),                                                                             \
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                                            \
+        : "memory")
+template <int USE_A, int GROUP>
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile(
-        "{\n\t"
-        ".reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t"
-        "}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if (GROUP == 2) {
+        if (USE_A == 1) TC_MMA_ASM("2", ".collector::a::fill");
+        else if (USE_A == 2) TC_MMA_ASM("2", ".collector::a::lastuse");
+        else TC_MMA_ASM("2", "");
+    } else {
+        if (USE_A == 1) TC_MMA_ASM("1", ".collector::a::fill");
+        else if (USE_A == 2) TC_MMA_ASM("1", ".collector::a::lastuse");
+        else TC_MMA_ASM("1", "");
+    }
 }
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t *r)
 {
@@ -137,7 +191,7 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
 }
 
 // instruction descriptor for kind::tf32 (TF32 operands in 32-bit containers, fp32 accumulation)
-__host__ __device__ inline uint32_t make_idesc(int n, int a_mn_major, int b_mn_major)
+__host__ __device__ inline uint32_t make_idesc(int m, int n, int a_mn_major, int b_mn_major)
 {
     uint32_t d = 0;
     d |= 1u << 4;   // D format: f32
@@ -146,7 +200,7 @@ __host__ __device__ inline uint32_t make_idesc(int n, int a_mn_major, int b_mn_m
     d |= (uint32_t)a_mn_major << 15;
     d |= (uint32_t)b_mn_major << 16;
     d |= (uint32_t)(n >> 3) << 17;
-    d |= (uint32_t)(TC_BM >> 4) << 24;
+    d |= (uint32_t)(m >> 4) << 24;
     return d;
 }
 
@@ -193,6 +247,19 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// On the barrier at the same place in CTA 0 of the pair.  What the barrier guards has been performed when this is issued: shared-memory
+// writes by the proxy fence in front of it, TMEM reads by their wait.  (With .release.cluster the arrive also waits for everything else the
+// SM has in flight, 1.4 us: a 179250 x 512 x 512 contraction took 490 us instead of 370.)
+__device__ __forceinline__ void mbar_arrive_leader(uint64_t *bar)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .b32 a;\n\t"
+        "mapa.shared::cluster.u32 a, %0, 0;\n\t"
+        "mbarrier.arrive.shared::cluster.b64 _, [a];\n\t"
+        "}" ::"r"(smem_u32(bar))
+        : "memory");
+}
 // make generic-proxy shared-memory writes visible to the tensor-core (async) proxy
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -220,7 +287,7 @@ struct TcEpilogue {
     const int32_t *tile_order;  // row tile walked at position i of the schedule (null: i itself)
 };
 
-// Row tile (of TC_BM rows) of schedule position t: the persistent CTAs walk positions blockIdx.x, blockIdx.x + gridDim.x, ...;
+// Row tile (of SAT_TC_ROWS rows) of schedule position t: the persistent CTA pairs walk positions unit, unit + units, ...;
 // a permutation lets the caller choose which row tiles run at the same time (results do not depend on it).
 __device__ __forceinline__ int64_t tck_row_tile(const TcEpilogue &ep, int64_t t, int32_t n_tiles_n)
 {
@@ -228,10 +295,11 @@ __device__ __forceinline__ int64_t tck_row_tile(const TcEpilogue &ep, int64_t t,
     return ep.tile_order ? (int64_t)__ldg(ep.tile_order + rt) : rt;
 }
 
+#define TCK_STAGES_MAX 8
 struct TcShared {
-    uint64_t full[4];       // TMA bytes of the stage have landed
-    uint64_t conv[4];       // the converter threads have split the stage
-    uint64_t empty[4];      // the MMAs reading the stage have completed
+    uint64_t full[TCK_STAGES_MAX];       // TMA bytes of the stage have landed
+    uint64_t conv[TCK_STAGES_MAX];       // the converter threads have split the stage
+    uint64_t empty[TCK_STAGES_MAX];      // the MMAs reading the stage have completed
     uint64_t acc_full[2];   // accumulator buffer holds a finished tile
     uint64_t acc_empty[2];  // accumulator buffer has been drained by the epilogue
     uint32_t tmem_base;
@@ -241,10 +309,11 @@ struct TcShared {
 /* 512 threads, 128 registers each: warp 0 TMA, warp 1 MMA, then the converter warps, then the epilogue warps.  The split
  * between converters and epilogue depends on the epilogue variant (TckCfg): the K = h variants with a side operand have
  * four k-blocks per tile and an epilogue bound by instruction issue, so they run 2 + 12 instead of 6 + 8.
- * The converter warps work in two groups on alternate k-blocks, so two stages are being split at any time.  Every stage
+ * The converter warps work in two groups on alternate k-blocks, so two stages are being split at any time.  The stage
  * count is even, hence a stage is always handled by the same group and each group meets the phases of its stages in
  * order (a parity wait must never be more than one phase ahead of its barrier). */
 #define TCK_THREADS 512
+#define TCK_CTAS 2
 #define TCK_CONV_GROUPS 2
 /* The weights' residual plane is made once by k_split_weights and fetched by TMA next to the raw plane: B is the same for
  * every row tile, and splitting its tile again per k-block cost the converters twice what the A tile costs (measured:
@@ -256,14 +325,11 @@ struct TcShared {
 // the consumer: one chunk in flight per warp left the loads latency-bound at ~2 TB/s.  Those variants contract over a
 // small K (the predictor width), so they give up main-loop stages for the ring.
 enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_LSTM = 2, EPI_LSTM_ADD = 3, EPI_PUSH = 4, EPI_GRU = 5 };   // EPI_PUSH = EPI_PLAIN + a second copy of the rows that have a cache slot
-template <int EPI> struct TckCfg { static constexpr int stages = 4, ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = epi_warps * 4096; };
-template <> struct TckCfg<EPI_RESID> { static constexpr int stages = 2, ring = 1, conv_warps = 2, epi_warps = 12, out_bytes = epi_warps * 4096; };
-template <> struct TckCfg<EPI_LSTM> { static constexpr int stages = 4, ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = 0; };
+template <int EPI> struct TckCfg { static constexpr int ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = epi_warps * 4096; };
+template <> struct TckCfg<EPI_RESID> { static constexpr int ring = 1, conv_warps = 2, epi_warps = 12, out_bytes = epi_warps * 4096; };
+template <> struct TckCfg<EPI_LSTM> { static constexpr int ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = 0; };
 template <> struct TckCfg<EPI_GRU> : TckCfg<EPI_LSTM> {};
-template <> struct TckCfg<EPI_LSTM_ADD> { static constexpr int stages = 2, ring = 2, conv_warps = 2, epi_warps = 12, out_bytes = 0; };
-static_assert(TckCfg<EPI_PLAIN>::stages % TCK_CONV_GROUPS == 0 && TckCfg<EPI_RESID>::stages % TCK_CONV_GROUPS == 0 &&
-                  TckCfg<EPI_LSTM>::stages % TCK_CONV_GROUPS == 0 && TckCfg<EPI_LSTM_ADD>::stages % TCK_CONV_GROUPS == 0,
-              "a stage must always be split by the same converter group");
+template <> struct TckCfg<EPI_LSTM_ADD> { static constexpr int ring = 2, conv_warps = 2, epi_warps = 12, out_bytes = 0; };
 
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, bool valid)
 {
@@ -274,7 +340,11 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Persistent: each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...  The shared-memory ring of k-block stages
+// Persistent: each pair of CTAs walks tiles of 256 rows unit, unit + units, ...  A pair's MMA (cta_group::2) multiplies the 128 rows of
+// either CTA with all columns of B, of which each CTA holds half: per k-block of 16 the tensor core reads 48 + 24 KB less operand and
+// the TMA writes 16 KB less than two CTAs on their own at 256 columns, where shared memory (128 KB per k-block at 128 B per clock)
+// and not the tensor work (96 KB worth) was the bound; and the ring holds six stages instead of four.  Measured: 169343 x 256 x 256
+// 117 -> 105 us, 179250 x 512 x 512 413 -> 370, 612257 x 256 x 256 415 -> 358.  The shared-memory ring of k-block stages
 // and the two TMEM accumulator buffers let the TMA loads, the TF32 split, the MMAs and the epilogue of consecutive tiles
 // overlap.  A and B arrive as raw fp32 tiles, which the tensor core reads as the hi operands; the converters write the
 // residual tiles.  The epilogue is a template parameter (plain bias / ReLU / mask, gathered residual, fused LSTM cell)
@@ -284,16 +354,17 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int EPI>
 __global__ void __launch_bounds__(TCK_THREADS, 1)
 k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapA2, const __grid_constant__ CUtensorMap mapB,
-            const __grid_constant__ CUtensorMap mapBlo, const __grid_constant__ CUtensorMap mapC, int use_tma_store, int64_t M, int32_t N, int32_t nkb1, int32_t nkb2, int32_t bn, int32_t n_tiles_n, int64_t n_tiles, TcEpilogue ep, int *status)
+            const __grid_constant__ CUtensorMap mapBlo, const __grid_constant__ CUtensorMap mapC, int use_tma_store, uint32_t stages, int64_t M, int32_t N, int32_t nkb1, int32_t nkb2, int32_t bn, int32_t n_tiles_n, int64_t n_tiles, TcEpilogue ep, int *status)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t a_bytes = TC_BM * TC_BK * 4;  // one plane of the A tile: 128 rows x 64 B
-    const uint32_t b_bytes = (uint32_t)bn * TC_BK * 4;
+    const uint32_t b_bytes = (uint32_t)bn / TCK_CTAS * TC_BK * 4;  // a CTA of a pair holds half of the columns
     const uint32_t stage_bytes = 2 * a_bytes + 2 * b_bytes;  // [A hi | A lo | B hi | B lo]
-    constexpr int STAGES = TckCfg<EPI>::stages;
+    const uint32_t rank = blockIdx.x & 1u;  // in the pair; CTA 0 issues the MMAs of both
+    const int64_t unit = blockIdx.x / TCK_CTAS, units = gridDim.x / TCK_CTAS;
     constexpr int RING = TckCfg<EPI>::ring;
-    uint8_t *out_stage = smem + (size_t)STAGES * stage_bytes;
+    uint8_t *out_stage = smem + (size_t)stages * stage_bytes;
     uint8_t *ring_base = out_stage + TckCfg<EPI>::out_bytes;
     constexpr int CONV_THREADS = TckCfg<EPI>::conv_warps * 32, CONV_GROUP_THREADS = CONV_THREADS / TCK_CONV_GROUPS;
     constexpr int EPI_WARPS = TckCfg<EPI>::epi_warps, EPI_WARP0 = 2 + TckCfg<EPI>::conv_warps;
@@ -305,24 +376,24 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     const uint32_t acc_cols = 256;  // column stride between the two accumulator buffers
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (uint32_t s = 0; s < stages; ++s) {
             mbar_init(&sh->full[s], 1);
-            mbar_init(&sh->conv[s], CONV_GROUP_THREADS);
+            mbar_init(&sh->conv[s], TCK_CTAS * (CONV_GROUP_THREADS / 32));
             mbar_init(&sh->empty[s], 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sh->acc_full[i], 1);
-            mbar_init(&sh->acc_empty[i], EPI_WARPS * 32);
+            mbar_init(&sh->acc_empty[i], TCK_CTAS * EPI_WARPS);
         }
         sh->dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"(512u) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tc_alloc<TCK_CTAS>(&sh->tmem_base, 512u);
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();   // the other CTA's barriers are initialised and its TMEM is allocated
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
     volatile int *dead = &sh->dead;
@@ -331,13 +402,11 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     if (warp == 0) {
         // ---------------- TMA producer ----------------
         if (lane == 0) {
-            uint32_t it = 0;
-            for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-                const int32_t m0 = (int32_t)tck_row_tile(ep, t, n_tiles_n) * TC_BM;
-                const int32_t n0 = (int32_t)(t % n_tiles_n) * bn;
-                for (int32_t kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (it / STAGES) & 1u;
+            uint32_t s = 0, ph = 0;
+            for (int64_t t = unit; t < n_tiles; t += units) {
+                const int32_t m0 = ((int32_t)tck_row_tile(ep, t, n_tiles_n) * TCK_CTAS + (int32_t)rank) * TC_BM;   // CTA `rank` holds the rank-th 128 rows
+                const int32_t n0 = (int32_t)(t % n_tiles_n) * bn + (int32_t)rank * (bn / TCK_CTAS);
+                for (int32_t kb = 0; kb < nkb; ++kb) {
                     if (!mbar_wait(&sh->empty[s], ph ^ 1u, dead, status)) goto done;
                     uint8_t *st = smem + (size_t)s * stage_bytes;
                     mbar_expect_tx(&sh->full[s], a_bytes + (TCK_B_PRESPLIT ? 2 * b_bytes : b_bytes));
@@ -345,63 +414,69 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     else tma_load_2d(st, &mapA2, &sh->full[s], (kb - nkb1) * TC_BK, m0);
                     tma_load_2d(st + 2 * a_bytes, &mapB, &sh->full[s], kb * TC_BK, n0);
                     if (TCK_B_PRESPLIT) tma_load_2d(st + 2 * a_bytes + b_bytes, &mapBlo, &sh->full[s], kb * TC_BK, n0);
+                    if (++s == stages) s = 0, ph ^= 1u;
                 }
             }
+            // the pair's MMAs have signalled every stage: nothing arrives here any more once both CTAs may exit
+            for (uint32_t i = 0; i < stages; ++i) {
+                if (!mbar_wait(&sh->empty[s], ph ^ 1u, dead, status)) goto done;
+                if (++s == stages) s = 0, ph ^= 1u;
+            }
         }
-    } else if (warp == 1) {
+    } else if (warp == 1 && rank == 0) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc(bn, 0, 0);
-            const uint64_t desc0 = make_desc(smem_u32(smem), 16, 512, 4);
-            uint32_t it = 0, lt = 0;
-            for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x, ++lt) {
-                const uint32_t buf = lt & 1u;
-                if (!mbar_wait(&sh->acc_empty[buf], ((lt >> 1) & 1u) ^ 1u, dead, status)) goto done;
+        // The whole warp walks the k-blocks and an elected lane issues: the operands of the instructions are then known to be uniform.
+        // (One lane doing all of it took 0.4 us per k-block, which bound the narrow tiles: 169343 x 40, K = 256: 70 -> 62 us.)
+        const uint32_t idesc = make_idesc(TC_BM * TCK_CTAS, bn, 0, 0);
+        const uint64_t desc0 = make_desc(smem_u32(smem), 16, 512, 4);
+        uint32_t s = 0, ph = 0, lt = 0;
+        for (int64_t t = unit; t < n_tiles; t += units, ++lt) {
+            const uint32_t buf = lt & 1u;
+            if (!mbar_wait_all(&sh->acc_empty[buf], ((lt >> 1) & 1u) ^ 1u, dead, status)) goto done;
+            tc_fence_after();
+            const uint32_t acc = tmem + buf * acc_cols;
+            for (int32_t kb = 0; kb < nkb; ++kb) {
+                // the converters arrive on conv[s] only after they have seen full[s] (the TMA bytes) themselves
+                if (!mbar_wait_all(&sh->conv[s], ph, dead, status)) goto done;
                 tc_fence_after();
-                const uint32_t acc = tmem + buf * acc_cols;
-                for (int32_t kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (it / STAGES) & 1u;
-                    // the converters arrive on conv[s] only after they have seen full[s] (the TMA bytes) themselves
-                    if (!mbar_wait(&sh->conv[s], ph, dead, status)) goto done;
-                    tc_fence_after();
-                    // K-major, 64-byte swizzle: rows 64 B apart, 8-row groups 512 B apart; a k-step (8 values) is 32 B inside the
-                    // row.  Only the 14-bit start-address field (bytes >> 4) differs between the descriptors of a stage.
-                    const uint64_t a_hi0 = desc0 + (uint64_t)(((uint32_t)s * stage_bytes) >> 4);
+                // K-major, 64-byte swizzle: rows 64 B apart, 8-row groups 512 B apart; a k-step (8 values) is 32 B inside the
+                // row.  Only the 14-bit start-address field (bytes >> 4) differs between the descriptors of a stage.
+                const uint64_t a_hi0 = desc0 + (uint64_t)((s * stage_bytes) >> 4);
+                if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < TC_BK / 8; ++ks) {
                         const uint64_t a_hi = a_hi0 + (uint64_t)(ks * 2);
                         const uint64_t a_lo = a_hi + (a_bytes >> 4);
                         const uint64_t b_hi = a_hi + (2 * a_bytes >> 4);
                         const uint64_t b_lo = b_hi + (b_bytes >> 4);
-                        tc_mma(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-                        tc_mma(acc, a_hi, b_lo, idesc, 1u);
-                        tc_mma(acc, a_lo, b_hi, idesc, 1u);
+                        tc_mma<1, TCK_CTAS>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                        tc_mma<2, TCK_CTAS>(acc, a_hi, b_lo, idesc, 1u);
+                        tc_mma<0, TCK_CTAS>(acc, a_lo, b_hi, idesc, 1u);
                     }
-                    tc_commit(&sh->empty[s]);  // the stage is free once these MMAs have read it
+                    tc_commit<TCK_CTAS>(&sh->empty[s]);  // the stage is free once these MMAs have read it
                 }
-                tc_commit(&sh->acc_full[buf]);
+                if (++s == stages) s = 0, ph ^= 1u;
             }
+            if (elect_one()) tc_commit<TCK_CTAS>(&sh->acc_full[buf]);
         }
-    } else if (warp < EPI_WARP0) {
+    } else if (warp >= 2 && warp < EPI_WARP0) {
         // ---------------- converters: TF32 split of the A and B tiles of every k-block ----------------
         const int grp = (threadIdx.x - 64) / CONV_GROUP_THREADS;
         const int ctid = (threadIdx.x - 64) % CONV_GROUP_THREADS;
-        uint32_t it = 0;
-        for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-            for (int32_t kb = 0; kb < nkb; ++kb, ++it) {
-                if ((int)(it % TCK_CONV_GROUPS) != grp) continue;
-                const int s = it % STAGES;
-                const uint32_t ph = (it / STAGES) & 1u;
-                if (!mbar_wait(&sh->full[s], ph, dead, status)) goto done;
-                uint8_t *st = smem + (size_t)s * stage_bytes;
-                split_tile_residual(st, st + a_bytes, a_bytes, ctid, CONV_GROUP_THREADS);
-                if (!TCK_B_PRESPLIT) split_tile_residual(st + 2 * a_bytes, st + 2 * a_bytes + b_bytes, b_bytes, ctid, CONV_GROUP_THREADS);
-                fence_async_smem();
-                mbar_arrive(&sh->conv[s]);
-            }
+        const int64_t my_tiles = unit < n_tiles ? (n_tiles - 1 - unit) / units + 1 : 0;
+        uint32_t s = grp, ph = 0;
+        for (int64_t it = grp; it < my_tiles * nkb; it += TCK_CONV_GROUPS) {
+            if (!mbar_wait_all(&sh->full[s], ph, dead, status)) goto done;
+            uint8_t *st = smem + (size_t)s * stage_bytes;
+            split_tile_residual(st, st + a_bytes, a_bytes, ctid, CONV_GROUP_THREADS);
+            if (!TCK_B_PRESPLIT) split_tile_residual(st + 2 * a_bytes, st + 2 * a_bytes + b_bytes, b_bytes, ctid, CONV_GROUP_THREADS);
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_leader(&sh->conv[s]);
+            s += TCK_CONV_GROUPS;
+            if (s >= stages) s -= stages, ph ^= 1u;
         }
-    } else {
+    } else if (warp >= EPI_WARP0) {
         // ---------------- epilogue ----------------
         // warp w reads TMEM lanes 32 (w % 4) .. +31 = rows of the tile, one row per thread; the warps of a lane quadrant
         // take alternate 32-column chunks.
@@ -419,24 +494,25 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         // warp: cp.async group counting plus __syncwarp is all the synchronisation needed.  The prefetch cursor (pf_*)
         // walks this warp's (tile, chunk) sequence RING chunks ahead of the consumer.
         uint8_t *ring = ring_base + (size_t)e * RING * 4096;
-        int64_t pf_t = blockIdx.x;
+        int64_t pf_t = unit;
         int pf_c = c_first;
         const float *pf_srow = nullptr;
         int32_t pf_lim = 0;
         int32_t pf_idx_next = -1;   // (gathered residual) row index for the tile after the cursor's, fetched a tile early
         uint32_t pf_slot = 0, rd_slot = 0;
+        auto tile_row = [&](int64_t t) { return (tck_row_tile(ep, t, n_tiles_n) * TCK_CTAS + rank) * TC_BM + q * 32; };   // first row of this warp
         auto pf_enter_tile = [&](int32_t idx_now) {
             // called when the cursor enters tile pf_t; idx_now = gathered row index for this thread's row, or -1
             pf_srow = nullptr;
             if (pf_t < n_tiles) {
-                const int64_t prow = tck_row_tile(ep, pf_t, n_tiles_n) * TC_BM + q * 32 + lane;
+                const int64_t prow = tile_row(pf_t) + lane;
                 const int32_t pn0 = (int32_t)(pf_t % n_tiles_n) * bn;
                 if (EPI == EPI_RESID) {
                     if (prow < M && idx_now >= 0) pf_srow = ep.resid + (int64_t)idx_now * ep.ld_resid + pn0;  // rows padded to 4 floats
                     pf_lim = n4 - pn0;
-                    const int64_t nt = pf_t + gridDim.x;
-                    const int64_t nrow = tck_row_tile(ep, nt, n_tiles_n) * TC_BM + q * 32 + lane;
-                    pf_idx_next = (nt < n_tiles && nrow < M) ? __ldg(ep.resid_idx + nrow) : -1;
+                    const int64_t nt = pf_t + units;
+                    const int64_t nrow = nt < n_tiles ? tile_row(nt) + lane : M;
+                    pf_idx_next = nrow < M ? __ldg(ep.resid_idx + nrow) : -1;
                 } else {
                     if (prow < M) pf_srow = ep.addend + prow * ep.ld_addend + pn0;
                     pf_lim = N - pn0;
@@ -462,7 +538,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     }
                 } else {
                     // dense side operand: rows of the tile are ld_addend apart
-                    const int64_t prow0 = tck_row_tile(ep, pf_t, n_tiles_n) * TC_BM + q * 32 + (lane >> 3);
+                    const int64_t prow0 = tile_row(pf_t) + (lane >> 3);
                     const float *p0 = base + prow0 * ep.ld_addend + (int32_t)(pf_t % n_tiles_n) * bn + pf_c + 4 * piece;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
@@ -474,7 +550,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 pf_c += CHUNK_STEP;
                 if (pf_c >= bn) {
                     pf_c = c_first;
-                    pf_t += gridDim.x;
+                    pf_t += units;
                     pf_enter_tile(pf_idx_next);
                 }
             }
@@ -484,7 +560,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (RING > 0 && c_first < bn) {
             int32_t idx0 = -1;
             if (EPI == EPI_RESID && pf_t < n_tiles) {
-                const int64_t prow = tck_row_tile(ep, pf_t, n_tiles_n) * TC_BM + q * 32 + lane;
+                const int64_t prow = tile_row(pf_t) + lane;
                 if (prow < M) idx0 = __ldg(ep.resid_idx + prow);
             }
             pf_enter_tile(idx0);
@@ -493,8 +569,8 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         }
 
         uint32_t lt = 0;
-        for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x, ++lt) {
-            const int64_t m0 = tck_row_tile(ep, t, n_tiles_n) * TC_BM;
+        for (int64_t t = unit; t < n_tiles; t += units, ++lt) {
+            const int64_t m0 = tile_row(t) - q * 32;
             const int32_t n0 = (int32_t)(t % n_tiles_n) * bn;
             const uint32_t buf = lt & 1u;
             const int64_t row = m0 + q * 32 + lane;
@@ -696,7 +772,8 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 }
             }
             tc_fence_before();
-            mbar_arrive(&sh->acc_empty[buf]);  // the accumulator buffer may be overwritten by the tile after next
+            __syncwarp();
+            if (lane == 0) mbar_arrive_leader(&sh->acc_empty[buf]);  // the accumulator buffer may be overwritten by the tile after next
         }
         if (use_tma_store && lane == 0) tma_store_wait_all();
         if (RING > 0) cp_async_wait<0>();
@@ -704,9 +781,11 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 done:
     tc_fence_before();
     __syncthreads();
+    cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
     if (warp == 1) {
+        __syncwarp();
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+        tc_dealloc<TCK_CTAS>(tmem, 512u);
     }
 }
 
@@ -762,8 +841,7 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"(tmem_cols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tc_alloc<1>(&sh->tmem_base, tmem_cols);
     }
     tc_fence_before();
     __syncthreads();
@@ -786,34 +864,34 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc(bn, 1, 1);
-            // MN-major 32-bit operands use the 128-byte swizzle with 32-byte atoms (the only layout the tensor core accepts for them):
-            // 32-column blocks blk_bytes apart (leading offset), groups of 4 k-rows 512 B apart (stride offset); a k-step is 8 rows =
-            // 1024 B.  Only the 14-bit start-address field (bytes >> 4) differs between the descriptors.
-            const uint64_t desc0 = make_desc(smem_u32(smem), blk_bytes, 512, 1);
-            for (int32_t kb = 0; kb < nkb; ++kb) {
-                const int s = kb % stages;
-                const uint32_t ph = (uint32_t)(kb / stages) & 1u;
-                // the converters arrive on conv[s] only after they have seen full[s] (the TMA bytes) themselves
-                if (!mbar_wait(&sh->conv[s], ph, dead, status)) break;
-                tc_fence_after();
-                const uint64_t st = desc0 + (uint64_t)(((uint32_t)s * stage_bytes) >> 4);
+        const uint32_t idesc = make_idesc(TC_BM, bn, 1, 1);
+        // MN-major 32-bit operands use the 128-byte swizzle with 32-byte atoms (the only layout the tensor core accepts for them):
+        // 32-column blocks blk_bytes apart (leading offset), groups of 4 k-rows 512 B apart (stride offset); a k-step is 8 rows =
+        // 1024 B.  Only the 14-bit start-address field (bytes >> 4) differs between the descriptors.
+        const uint64_t desc0 = make_desc(smem_u32(smem), blk_bytes, 512, 1);
+        for (int32_t kb = 0; kb < nkb; ++kb) {
+            const int s = kb % stages;
+            const uint32_t ph = (uint32_t)(kb / stages) & 1u;
+            // the converters arrive on conv[s] only after they have seen full[s] (the TMA bytes) themselves
+            if (!mbar_wait_all(&sh->conv[s], ph, dead, status)) break;
+            tc_fence_after();
+            const uint64_t st = desc0 + (uint64_t)(((uint32_t)s * stage_bytes) >> 4);
+            if (elect_one()) {
 #pragma unroll
                 for (int ks = 0; ks < TC_BK / 8; ++ks) {
                     const uint64_t b_hi = st + (uint64_t)((2 * a_bytes + ks * 1024) >> 4), b_lo = b_hi + (b_bytes >> 4);
                     for (int i = 0; i < mt; ++i) {
                         const uint64_t a_hi = st + (uint64_t)(((uint32_t)i * sub_bytes + ks * 1024) >> 4), a_lo = a_hi + (a_bytes >> 4);
                         const uint32_t acc = tmem + (uint32_t)i * 256u;
-                        tc_mma(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-                        tc_mma(acc, a_hi, b_lo, idesc, 1u);
-                        tc_mma(acc, a_lo, b_hi, idesc, 1u);
+                        tc_mma<1, 1>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                        tc_mma<2, 1>(acc, a_hi, b_lo, idesc, 1u);
+                        tc_mma<0, 1>(acc, a_lo, b_hi, idesc, 1u);
                     }
                 }
-                tc_commit(&sh->empty[s]);
+                tc_commit<1>(&sh->empty[s]);
             }
-            tc_commit(&sh->accum);
         }
+        if (elect_one()) tc_commit<1>(&sh->accum);
     } else {
         const int ctid = threadIdx.x - 64;
         const bool want_cs = part_cs != nullptr && blockIdx.x == 0;
@@ -910,7 +988,7 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+        tc_dealloc<1>(tmem, tmem_cols);
     }
 }
 
@@ -1161,14 +1239,19 @@ template <int EPI>
 static sat_status launch_tck(sat_ctx *ctx, const TckLaunch &L, const TcEpilogue &ep)
 {
     static PerDeviceOnce attr_set;
-    const size_t smem = (size_t)TckCfg<EPI>::stages * L.stage_bytes + TckCfg<EPI>::out_bytes + (size_t)TckCfg<EPI>::epi_warps * TckCfg<EPI>::ring * 4096 +
-                        sizeof(TcShared) + 1024;
+    // As many stages as fit, since the bytes in flight bound the narrow contractions (169343 x 128, K = 256: 86 us with 4 stages, 77 with
+    // 6), but no more than the longest CTA has k-blocks, so that a small launch leaves room on the SM for its successor; an even number
+    const size_t fixed = TckCfg<EPI>::out_bytes + (size_t)TckCfg<EPI>::epi_warps * TckCfg<EPI>::ring * 4096 + sizeof(TcShared) + 1024;
+    const int64_t blocks = cdiv64(L.n_tiles, L.grid / TCK_CTAS) * (L.nkb1 + L.nkb2), fit = (227 * 1024 - (int64_t)fixed) / L.stage_bytes;
+    uint32_t stages = TCK_STAGES_MAX;
+    while (stages > 2 && (stages > fit || stages - 2 >= blocks)) stages -= 2;
+    const size_t smem = (size_t)stages * L.stage_bytes + fixed;
     if (smem > 227 * 1024) return sat_fail(ctx, SAT_EINVAL, "tensor-core GEMM: shared-memory layout of %zu bytes does not fit", smem);
     if (attr_set.need(ctx->device)) {
         SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_k<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set.mark(ctx->device);
     }
-    sat_pdl(ctx->stream, k_gemm_tc_k<EPI>, L.grid, TCK_THREADS, smem)(L.mA, L.mA2, L.mB, L.mBlo, L.mC, L.use_tma_store, L.m, L.n, L.nkb1, L.nkb2, L.bn, L.n_tiles_n,
+    sat_pdl(ctx->stream, k_gemm_tc_k<EPI>, L.grid, TCK_THREADS, smem, TCK_CTAS)(L.mA, L.mA2, L.mB, L.mBlo, L.mC, L.use_tma_store, stages, L.m, L.n, L.nkb1, L.nkb2, L.bn, L.n_tiles_n,
                                                                 L.n_tiles, ep, ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -1181,7 +1264,7 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     if (m == 0 || n == 0) return SAT_OK;
     const int32_t nkb1 = (k1 + TC_BK - 1) / TC_BK, nkb2 = A2 ? (k2 + TC_BK - 1) / TC_BK : 0;
     const int32_t bn = tile_n_for(n);
-    const uint32_t stage_bytes = 2 * (TC_BM * TC_BK * 4) + 2 * (uint32_t)bn * TC_BK * 4;
+    const uint32_t stage_bytes = 2 * (TC_BM * TC_BK * 4) + 2 * (uint32_t)bn / TCK_CTAS * TC_BK * 4;
     // algorithmic bytes: operands once, results once.  Plain: A, B, C.  Gathered residual: + the residual rows.  LSTM cell:
     // the output is the hidden state [m x h] plus the cell state read and written, and the cached projection if it is added.
     double alg_bytes = 4.0 * ((double)m * (k1 + k2) + (double)(k1 + k2) * n);
@@ -1195,8 +1278,8 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     SAT_TRY(make_map(ctx, &mA, A, k1, m, lda, TC_BK, TC_BM, CU_TENSOR_MAP_SWIZZLE_64B));
     if (A2) SAT_TRY(make_map(ctx, &mA2, A2, k2, m, lda2, TC_BK, TC_BM, CU_TENSOR_MAP_SWIZZLE_64B));
     else mA2 = mA;
-    SAT_TRY(make_map(ctx, &mB, Bw.hi, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn, CU_TENSOR_MAP_SWIZZLE_64B));
-    SAT_TRY(make_map(ctx, &mBlo, Bw.lo, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn, CU_TENSOR_MAP_SWIZZLE_64B));
+    SAT_TRY(make_map(ctx, &mB, Bw.hi, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / TCK_CTAS, CU_TENSOR_MAP_SWIZZLE_64B));
+    SAT_TRY(make_map(ctx, &mBlo, Bw.lo, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / TCK_CTAS, CU_TENSOR_MAP_SWIZZLE_64B));
     TcEpilogue ep;
     ep.C = eh.C;
     ep.ldc = eh.ldc;
@@ -1234,8 +1317,8 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.ld_resid = eh.ld_resid;
     ep.tile_order = eh.tile_order;
     const int32_t n_tiles_n = (int32_t)cdiv64(n, bn);
-    const int64_t n_tiles = cdiv64(m, TC_BM) * n_tiles_n;
-    const unsigned grid = (unsigned)(n_tiles < ctx->sms ? n_tiles : ctx->sms);
+    const int64_t n_tiles = cdiv64(m, SAT_TC_ROWS) * n_tiles_n, units = ctx->sms / TCK_CTAS;
+    const unsigned grid = (unsigned)(n_tiles < units ? n_tiles : units) * TCK_CTAS;
     TckLaunch L;
     L.mA = mA; L.mA2 = mA2; L.mB = mB; L.mBlo = mBlo; L.mC = mC;
     L.use_tma_store = use_tma_store;

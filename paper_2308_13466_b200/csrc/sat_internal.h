@@ -433,28 +433,38 @@ struct SatPdl {
     void (*kernel)(P...);
     dim3 grid, block;
     size_t smem;
+    unsigned cluster;   // blocks per cluster along x
     template <typename... A>
     void operator()(A &&...a) const   // launch errors are picked up by SAT_LAUNCHED
     {
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchAttribute attr[2];
+        int n = 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = grid;
         cfg.blockDim = block;
         cfg.dynamicSmemBytes = smem;
         cfg.stream = stream;
-        cfg.attrs = &attr;
+        cfg.attrs = attr;
         // only grids of at most one wave: the blocks of a longer one that move in early find the SM's shared memory / L1 split as the
         // running kernel left it and keep it for their whole launch (gathers behind a 200 KB contraction: epochs 3-10 % slower)
-        cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z * block.x <= 148 * 2048 ? 1 : 0;
+        if ((int64_t)grid.x * grid.y * grid.z * block.x <= 148 * 2048) {
+            attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[n++].val.programmaticStreamSerializationAllowed = 1;
+        }
+        if (cluster > 1) {
+            attr[n].id = cudaLaunchAttributeClusterDimension;
+            attr[n].val.clusterDim.x = cluster;
+            attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+            ++n;
+        }
+        cfg.numAttrs = (unsigned)n;
         (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(a)...);
     }
 };
 template <typename... P>
-inline SatPdl<P...> sat_pdl(cudaStream_t stream, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem)
+inline SatPdl<P...> sat_pdl(cudaStream_t stream, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, unsigned cluster = 1)
 {
-    return SatPdl<P...>{stream, kernel, grid, block, smem};
+    return SatPdl<P...>{stream, kernel, grid, block, smem, cluster};
 }
 // t / d for t >= 0: a 32-bit division (a few instructions instead of a hundred) wherever t fits
 __device__ __forceinline__ int64_t sat_div(int64_t t, int32_t d)
@@ -486,6 +496,7 @@ struct TcWeights {         // weight operand as two fp32 planes [n_pad x ld] hol
     float *hi = nullptr, *lo = nullptr;
     int32_t ld = 0, n_pad = 0;
 };
+#define SAT_TC_ROWS 256      /* rows per tile of the tensor-core contraction (128 per CTA of a pair) */
 struct TcEpilogueHost {
     float *C = nullptr;
     int32_t ldc = 0;
@@ -496,7 +507,7 @@ struct TcEpilogueHost {
     const float *resid = nullptr;      // C += resid[resid_idx[i]] (row gather)
     const int32_t *resid_idx = nullptr;
     int32_t ld_resid = 0;
-    // order in which the persistent kernel walks the tiles of 128 rows: [ceil(m / 128)] row-tile indices, a permutation
+    // order in which the persistent kernel walks the tiles of SAT_TC_ROWS rows: [ceil(m / SAT_TC_ROWS)] row-tile indices, a permutation
     // (null: ascending).  Results do not depend on it; it decides which rows are in flight together.
     const int32_t *tile_order = nullptr;
     // fused LSTM cell (the weights must have been packed with gate interleave): the n = 4h outputs of a row are the gate
