@@ -247,18 +247,26 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// On the barrier at the same place in CTA 0 of the pair.  What the barrier guards has been performed when this is issued: shared-memory
-// writes by the proxy fence in front of it, TMEM reads by their wait.  (With .release.cluster the arrive also waits for everything else the
-// SM has in flight, 1.4 us: a 179250 x 512 x 512 contraction took 490 us instead of 370.)
-__device__ __forceinline__ void mbar_arrive_leader(uint64_t *bar)
+// A warp's arrival on a barrier that the MMA issuer waits for.  CTAS = 1: every lane arrives.  2: lane 0 does, on the barrier at the same
+// place in CTA 0 of the pair.  What the barrier guards has been performed when the arrive is issued: shared-memory writes by the proxy
+// fence in front of it, TMEM reads by their wait.  (With .release.cluster it also waits for everything else the SM has in flight,
+// 1.4 us: a 179250 x 512 x 512 contraction took 490 us instead of 370.)
+template <int CTAS>
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t *bar, int lane)
 {
-    asm volatile(
-        "{\n\t"
-        ".reg .b32 a;\n\t"
-        "mapa.shared::cluster.u32 a, %0, 0;\n\t"
-        "mbarrier.arrive.shared::cluster.b64 _, [a];\n\t"
-        "}" ::"r"(smem_u32(bar))
-        : "memory");
+    if (CTAS == 1) {
+        mbar_arrive(bar);
+        return;
+    }
+    __syncwarp();
+    if (lane == 0)
+        asm volatile(
+            "{\n\t"
+            ".reg .b32 a;\n\t"
+            "mapa.shared::cluster.u32 a, %0, 0;\n\t"
+            "mbarrier.arrive.shared::cluster.b64 _, [a];\n\t"
+            "}" ::"r"(smem_u32(bar))
+            : "memory");
 }
 // make generic-proxy shared-memory writes visible to the tensor-core (async) proxy
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -287,7 +295,7 @@ struct TcEpilogue {
     const int32_t *tile_order;  // row tile walked at position i of the schedule (null: i itself)
 };
 
-// Row tile (of SAT_TC_ROWS rows) of schedule position t: the persistent CTA pairs walk positions unit, unit + units, ...;
+// Row tile (of 128 rows per CTA of a unit) of schedule position t: the persistent CTAs or CTA pairs walk positions unit, unit + units, ...;
 // a permutation lets the caller choose which row tiles run at the same time (results do not depend on it).
 __device__ __forceinline__ int64_t tck_row_tile(const TcEpilogue &ep, int64_t t, int32_t n_tiles_n)
 {
@@ -313,7 +321,6 @@ struct TcShared {
  * count is even, hence a stage is always handled by the same group and each group meets the phases of its stages in
  * order (a parity wait must never be more than one phase ahead of its barrier). */
 #define TCK_THREADS 512
-#define TCK_CTAS 2
 #define TCK_CONV_GROUPS 2
 /* The weights' residual plane is made once by k_split_weights and fetched by TMA next to the raw plane: B is the same for
  * every row tile, and splitting its tile again per k-block cost the converters twice what the A tile costs (measured:
@@ -340,18 +347,18 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Persistent: each pair of CTAs walks tiles of 256 rows unit, unit + units, ...  A pair's MMA (cta_group::2) multiplies the 128 rows of
-// either CTA with all columns of B, of which each CTA holds half: per k-block of 16 the tensor core reads 48 + 24 KB less operand and
-// the TMA writes 16 KB less than two CTAs on their own at 256 columns, where shared memory (128 KB per k-block at 128 B per clock)
-// and not the tensor work (96 KB worth) was the bound; and the ring holds six stages instead of four.  Measured: 169343 x 256 x 256
-// 117 -> 105 us, 179250 x 512 x 512 413 -> 370, 612257 x 256 x 256 415 -> 358.  The shared-memory ring of k-block stages
+// Persistent: each CTA (CTAS = 1) or pair of CTAs (2) walks tiles unit, unit + units, ... of 128 or 256 rows.  A pair's MMA
+// (cta_group::2) multiplies the 128 rows of either CTA with all columns of B, of which each CTA holds half: per k-block of 16 at 256
+// columns the tensor core reads 24 KB and the TMA writes 16 KB less per SM than with single CTAs, where shared memory (128 KB per k-block
+// at 128 B per clock) and not the tensor work (96 KB worth) was the bound; and the ring holds six stages instead of four.  Measured:
+// 169343 x 256 x 256 117 -> 105 us, 179250 x 512 x 512 413 -> 370, 612257 x 256 x 256 415 -> 358.  The shared-memory ring of k-block stages
 // and the two TMEM accumulator buffers let the TMA loads, the TF32 split, the MMAs and the epilogue of consecutive tiles
 // overlap.  A and B arrive as raw fp32 tiles, which the tensor core reads as the hi operands; the converters write the
 // residual tiles.  The epilogue is a template parameter (plain bias / ReLU / mask, gathered residual, fused LSTM cell)
 // and runs on eight or twelve warps, two or three per TMEM lane quadrant taking 32-column chunks in turn: with one warp
 // per scheduler the epilogue was bound by instruction issue and load latency (9 - 14 us per 128 x 256 tile, longer than
 // the main loop of a K = 256 tile).
-template <int EPI>
+template <int EPI, int CTAS>
 __global__ void __launch_bounds__(TCK_THREADS, 1)
 k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapA2, const __grid_constant__ CUtensorMap mapB,
             const __grid_constant__ CUtensorMap mapBlo, const __grid_constant__ CUtensorMap mapC, int use_tma_store, uint32_t stages, int64_t M, int32_t N, int32_t nkb1, int32_t nkb2, int32_t bn, int32_t n_tiles_n, int64_t n_tiles, TcEpilogue ep, int *status)
@@ -359,10 +366,10 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t a_bytes = TC_BM * TC_BK * 4;  // one plane of the A tile: 128 rows x 64 B
-    const uint32_t b_bytes = (uint32_t)bn / TCK_CTAS * TC_BK * 4;  // a CTA of a pair holds half of the columns
+    const uint32_t b_bytes = (uint32_t)bn / CTAS * TC_BK * 4;  // a CTA of a pair holds half of the columns
     const uint32_t stage_bytes = 2 * a_bytes + 2 * b_bytes;  // [A hi | A lo | B hi | B lo]
-    const uint32_t rank = blockIdx.x & 1u;  // in the pair; CTA 0 issues the MMAs of both
-    const int64_t unit = blockIdx.x / TCK_CTAS, units = gridDim.x / TCK_CTAS;
+    const uint32_t rank = CTAS == 2 ? blockIdx.x & 1u : 0u;  // in the pair; CTA 0 issues the MMAs of both
+    const int64_t unit = blockIdx.x / CTAS, units = gridDim.x / CTAS;
     constexpr int RING = TckCfg<EPI>::ring;
     uint8_t *out_stage = smem + (size_t)stages * stage_bytes;
     uint8_t *ring_base = out_stage + TckCfg<EPI>::out_bytes;
@@ -378,22 +385,22 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < stages; ++s) {
             mbar_init(&sh->full[s], 1);
-            mbar_init(&sh->conv[s], TCK_CTAS * (CONV_GROUP_THREADS / 32));
+            mbar_init(&sh->conv[s], CTAS == 2 ? 2 * (CONV_GROUP_THREADS / 32) : CONV_GROUP_THREADS);
             mbar_init(&sh->empty[s], 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sh->acc_full[i], 1);
-            mbar_init(&sh->acc_empty[i], TCK_CTAS * EPI_WARPS);
+            mbar_init(&sh->acc_empty[i], CTAS == 2 ? 2 * EPI_WARPS : EPI_WARPS * 32);
         }
         sh->dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        tc_alloc<TCK_CTAS>(&sh->tmem_base, 512u);
+        tc_alloc<CTAS>(&sh->tmem_base, 512u);
     }
     tc_fence_before();
     __syncthreads();
-    cluster_sync();   // the other CTA's barriers are initialised and its TMEM is allocated
+    if (CTAS == 2) cluster_sync();   // the other CTA's barriers are initialised and its TMEM is allocated
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
     volatile int *dead = &sh->dead;
@@ -404,8 +411,8 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (lane == 0) {
             uint32_t s = 0, ph = 0;
             for (int64_t t = unit; t < n_tiles; t += units) {
-                const int32_t m0 = ((int32_t)tck_row_tile(ep, t, n_tiles_n) * TCK_CTAS + (int32_t)rank) * TC_BM;   // CTA `rank` holds the rank-th 128 rows
-                const int32_t n0 = (int32_t)(t % n_tiles_n) * bn + (int32_t)rank * (bn / TCK_CTAS);
+                const int32_t m0 = ((int32_t)tck_row_tile(ep, t, n_tiles_n) * CTAS + (int32_t)rank) * TC_BM;   // CTA `rank` holds the rank-th 128 rows
+                const int32_t n0 = (int32_t)(t % n_tiles_n) * bn + (int32_t)rank * (bn / CTAS);
                 for (int32_t kb = 0; kb < nkb; ++kb) {
                     if (!mbar_wait(&sh->empty[s], ph ^ 1u, dead, status)) goto done;
                     uint8_t *st = smem + (size_t)s * stage_bytes;
@@ -418,7 +425,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 }
             }
             // the pair's MMAs have signalled every stage: nothing arrives here any more once both CTAs may exit
-            for (uint32_t i = 0; i < stages; ++i) {
+            for (uint32_t i = 0; CTAS == 2 && i < stages; ++i) {
                 if (!mbar_wait(&sh->empty[s], ph ^ 1u, dead, status)) goto done;
                 if (++s == stages) s = 0, ph ^= 1u;
             }
@@ -427,7 +434,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         // ---------------- MMA issuer ----------------
         // The whole warp walks the k-blocks and an elected lane issues: the operands of the instructions are then known to be uniform.
         // (One lane doing all of it took 0.4 us per k-block, which bound the narrow tiles: 169343 x 40, K = 256: 70 -> 62 us.)
-        const uint32_t idesc = make_idesc(TC_BM * TCK_CTAS, bn, 0, 0);
+        const uint32_t idesc = make_idesc(TC_BM * CTAS, bn, 0, 0);
         const uint64_t desc0 = make_desc(smem_u32(smem), 16, 512, 4);
         uint32_t s = 0, ph = 0, lt = 0;
         for (int64_t t = unit; t < n_tiles; t += units, ++lt) {
@@ -449,15 +456,15 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         const uint64_t a_lo = a_hi + (a_bytes >> 4);
                         const uint64_t b_hi = a_hi + (2 * a_bytes >> 4);
                         const uint64_t b_lo = b_hi + (b_bytes >> 4);
-                        tc_mma<1, TCK_CTAS>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-                        tc_mma<2, TCK_CTAS>(acc, a_hi, b_lo, idesc, 1u);
-                        tc_mma<0, TCK_CTAS>(acc, a_lo, b_hi, idesc, 1u);
+                        tc_mma<1, CTAS>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                        tc_mma<2, CTAS>(acc, a_hi, b_lo, idesc, 1u);
+                        tc_mma<0, CTAS>(acc, a_lo, b_hi, idesc, 1u);
                     }
-                    tc_commit<TCK_CTAS>(&sh->empty[s]);  // the stage is free once these MMAs have read it
+                    tc_commit<CTAS>(&sh->empty[s]);  // the stage is free once these MMAs have read it
                 }
                 if (++s == stages) s = 0, ph ^= 1u;
             }
-            if (elect_one()) tc_commit<TCK_CTAS>(&sh->acc_full[buf]);
+            if (elect_one()) tc_commit<CTAS>(&sh->acc_full[buf]);
         }
     } else if (warp >= 2 && warp < EPI_WARP0) {
         // ---------------- converters: TF32 split of the A and B tiles of every k-block ----------------
@@ -466,13 +473,12 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         const int64_t my_tiles = unit < n_tiles ? (n_tiles - 1 - unit) / units + 1 : 0;
         uint32_t s = grp, ph = 0;
         for (int64_t it = grp; it < my_tiles * nkb; it += TCK_CONV_GROUPS) {
-            if (!mbar_wait_all(&sh->full[s], ph, dead, status)) goto done;
+            if (CTAS == 2 ? !mbar_wait_all(&sh->full[s], ph, dead, status) : !mbar_wait(&sh->full[s], ph, dead, status)) goto done;
             uint8_t *st = smem + (size_t)s * stage_bytes;
             split_tile_residual(st, st + a_bytes, a_bytes, ctid, CONV_GROUP_THREADS);
             if (!TCK_B_PRESPLIT) split_tile_residual(st + 2 * a_bytes, st + 2 * a_bytes + b_bytes, b_bytes, ctid, CONV_GROUP_THREADS);
             fence_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_leader(&sh->conv[s]);
+            mbar_arrive_warp<CTAS>(&sh->conv[s], lane);
             s += TCK_CONV_GROUPS;
             if (s >= stages) s -= stages, ph ^= 1u;
         }
@@ -500,7 +506,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         int32_t pf_lim = 0;
         int32_t pf_idx_next = -1;   // (gathered residual) row index for the tile after the cursor's, fetched a tile early
         uint32_t pf_slot = 0, rd_slot = 0;
-        auto tile_row = [&](int64_t t) { return (tck_row_tile(ep, t, n_tiles_n) * TCK_CTAS + rank) * TC_BM + q * 32; };   // first row of this warp
+        auto tile_row = [&](int64_t t) { return (tck_row_tile(ep, t, n_tiles_n) * CTAS + rank) * TC_BM + q * 32; };   // first row of this warp
         auto pf_enter_tile = [&](int32_t idx_now) {
             // called when the cursor enters tile pf_t; idx_now = gathered row index for this thread's row, or -1
             pf_srow = nullptr;
@@ -772,8 +778,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 }
             }
             tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_leader(&sh->acc_empty[buf]);  // the accumulator buffer may be overwritten by the tile after next
+            mbar_arrive_warp<CTAS>(&sh->acc_empty[buf], lane);  // the accumulator buffer may be overwritten by the tile after next
         }
         if (use_tma_store && lane == 0) tma_store_wait_all();
         if (RING > 0) cp_async_wait<0>();
@@ -781,11 +786,11 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 done:
     tc_fence_before();
     __syncthreads();
-    cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
+    if (CTAS == 2) cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        tc_dealloc<TCK_CTAS>(tmem, 512u);
+        tc_dealloc<CTAS>(tmem, 512u);
     }
 }
 
@@ -1235,23 +1240,23 @@ struct TckLaunch {
     uint32_t stage_bytes;
 };
 
-template <int EPI>
+template <int EPI, int CTAS>
 static sat_status launch_tck(sat_ctx *ctx, const TckLaunch &L, const TcEpilogue &ep)
 {
     static PerDeviceOnce attr_set;
     // As many stages as fit, since the bytes in flight bound the narrow contractions (169343 x 128, K = 256: 86 us with 4 stages, 77 with
     // 6), but no more than the longest CTA has k-blocks, so that a small launch leaves room on the SM for its successor; an even number
     const size_t fixed = TckCfg<EPI>::out_bytes + (size_t)TckCfg<EPI>::epi_warps * TckCfg<EPI>::ring * 4096 + sizeof(TcShared) + 1024;
-    const int64_t blocks = cdiv64(L.n_tiles, L.grid / TCK_CTAS) * (L.nkb1 + L.nkb2), fit = (227 * 1024 - (int64_t)fixed) / L.stage_bytes;
+    const int64_t blocks = cdiv64(L.n_tiles, L.grid / CTAS) * (L.nkb1 + L.nkb2), fit = (227 * 1024 - (int64_t)fixed) / L.stage_bytes;
     uint32_t stages = TCK_STAGES_MAX;
     while (stages > 2 && (stages > fit || stages - 2 >= blocks)) stages -= 2;
     const size_t smem = (size_t)stages * L.stage_bytes + fixed;
     if (smem > 227 * 1024) return sat_fail(ctx, SAT_EINVAL, "tensor-core GEMM: shared-memory layout of %zu bytes does not fit", smem);
     if (attr_set.need(ctx->device)) {
-        SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_k<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_k<EPI, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set.mark(ctx->device);
     }
-    sat_pdl(ctx->stream, k_gemm_tc_k<EPI>, L.grid, TCK_THREADS, smem, TCK_CTAS)(L.mA, L.mA2, L.mB, L.mBlo, L.mC, L.use_tma_store, stages, L.m, L.n, L.nkb1, L.nkb2, L.bn, L.n_tiles_n,
+    sat_pdl(ctx->stream, k_gemm_tc_k<EPI, CTAS>, L.grid, TCK_THREADS, smem, CTAS)(L.mA, L.mA2, L.mB, L.mBlo, L.mC, L.use_tma_store, stages, L.m, L.n, L.nkb1, L.nkb2, L.bn, L.n_tiles_n,
                                                                 L.n_tiles, ep, ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
@@ -1264,7 +1269,13 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     if (m == 0 || n == 0) return SAT_OK;
     const int32_t nkb1 = (k1 + TC_BK - 1) / TC_BK, nkb2 = A2 ? (k2 + TC_BK - 1) / TC_BK : 0;
     const int32_t bn = tile_n_for(n);
-    const uint32_t stage_bytes = 2 * (TC_BM * TC_BK * 4) + 2 * (uint32_t)bn / TCK_CTAS * TC_BK * 4;
+    // CTA pairs for launches of more than one wave of single CTAs (below, the pair only adds its synchronisation: 6000 x 72, K = 50: 12.0
+    // -> 12.9 us), except with a side operand: those contract over the predictor width and are bound by the side operand's
+    // stream, which the pair holds up (gathered residual 145 -> 161 us, cached projection 92 -> 95 at 169343 rows)
+    const int32_t n_tiles_n = (int32_t)cdiv64(n, bn);
+    const bool pair = !eh.resid_idx && !eh.addend && cdiv64(m, TC_BM) * n_tiles_n > ctx->sms;
+    const int ctas = pair ? 2 : 1;
+    const uint32_t stage_bytes = 2 * (TC_BM * TC_BK * 4) + 2 * (uint32_t)bn / ctas * TC_BK * 4;
     // algorithmic bytes: operands once, results once.  Plain: A, B, C.  Gathered residual: + the residual rows.  LSTM cell:
     // the output is the hidden state [m x h] plus the cell state read and written, and the cached projection if it is added.
     double alg_bytes = 4.0 * ((double)m * (k1 + k2) + (double)(k1 + k2) * n);
@@ -1278,8 +1289,8 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     SAT_TRY(make_map(ctx, &mA, A, k1, m, lda, TC_BK, TC_BM, CU_TENSOR_MAP_SWIZZLE_64B));
     if (A2) SAT_TRY(make_map(ctx, &mA2, A2, k2, m, lda2, TC_BK, TC_BM, CU_TENSOR_MAP_SWIZZLE_64B));
     else mA2 = mA;
-    SAT_TRY(make_map(ctx, &mB, Bw.hi, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / TCK_CTAS, CU_TENSOR_MAP_SWIZZLE_64B));
-    SAT_TRY(make_map(ctx, &mBlo, Bw.lo, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / TCK_CTAS, CU_TENSOR_MAP_SWIZZLE_64B));
+    SAT_TRY(make_map(ctx, &mB, Bw.hi, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / ctas, CU_TENSOR_MAP_SWIZZLE_64B));
+    SAT_TRY(make_map(ctx, &mBlo, Bw.lo, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / ctas, CU_TENSOR_MAP_SWIZZLE_64B));
     TcEpilogue ep;
     ep.C = eh.C;
     ep.ldc = eh.ldc;
@@ -1316,20 +1327,20 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.resid_idx = eh.resid_idx;
     ep.ld_resid = eh.ld_resid;
     ep.tile_order = eh.tile_order;
-    const int32_t n_tiles_n = (int32_t)cdiv64(n, bn);
-    const int64_t n_tiles = cdiv64(m, SAT_TC_ROWS) * n_tiles_n, units = ctx->sms / TCK_CTAS;
-    const unsigned grid = (unsigned)(n_tiles < units ? n_tiles : units) * TCK_CTAS;
+    const int64_t n_tiles = cdiv64(m, TC_BM * ctas) * n_tiles_n, units = ctx->sms / ctas;
+    const unsigned grid = (unsigned)(n_tiles < units ? n_tiles : units) * ctas;
     TckLaunch L;
     L.mA = mA; L.mA2 = mA2; L.mB = mB; L.mBlo = mBlo; L.mC = mC;
     L.use_tma_store = use_tma_store;
     L.m = m; L.n = n; L.nkb1 = nkb1; L.nkb2 = nkb2; L.bn = bn; L.n_tiles_n = n_tiles_n; L.n_tiles = n_tiles;
     L.grid = grid;
     L.stage_bytes = stage_bytes;
-    if (eh.gru) return launch_tck<EPI_GRU>(ctx, L, ep);
-    if (ep.lstm_h > 0) return ep.addend ? launch_tck<EPI_LSTM_ADD>(ctx, L, ep) : launch_tck<EPI_LSTM>(ctx, L, ep);
-    if (ep.resid_idx) return launch_tck<EPI_RESID>(ctx, L, ep);
-    if (ep.push_dst) return launch_tck<EPI_PUSH>(ctx, L, ep);
-    return launch_tck<EPI_PLAIN>(ctx, L, ep);
+    if (eh.gru) return pair ? launch_tck<EPI_GRU, 2>(ctx, L, ep) : launch_tck<EPI_GRU, 1>(ctx, L, ep);
+    if (ep.lstm_h > 0 && ep.addend) return launch_tck<EPI_LSTM_ADD, 1>(ctx, L, ep);
+    if (ep.lstm_h > 0) return pair ? launch_tck<EPI_LSTM, 2>(ctx, L, ep) : launch_tck<EPI_LSTM, 1>(ctx, L, ep);
+    if (ep.resid_idx) return launch_tck<EPI_RESID, 1>(ctx, L, ep);
+    if (ep.push_dst) return pair ? launch_tck<EPI_PUSH, 2>(ctx, L, ep) : launch_tck<EPI_PUSH, 1>(ctx, L, ep);
+    return pair ? launch_tck<EPI_PLAIN, 2>(ctx, L, ep) : launch_tck<EPI_PLAIN, 1>(ctx, L, ep);
 }
 
 // C[m x n] (+)= A^T B over `rows` rows: A fp32 [rows x m] (lda), B fp32 [rows x n] (ldb)

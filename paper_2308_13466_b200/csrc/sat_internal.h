@@ -496,7 +496,6 @@ struct TcWeights {         // weight operand as two fp32 planes [n_pad x ld] hol
     float *hi = nullptr, *lo = nullptr;
     int32_t ld = 0, n_pad = 0;
 };
-#define SAT_TC_ROWS 256      /* rows per tile of the tensor-core contraction (128 per CTA of a pair) */
 struct TcEpilogueHost {
     float *C = nullptr;
     int32_t ldc = 0;
@@ -507,7 +506,7 @@ struct TcEpilogueHost {
     const float *resid = nullptr;      // C += resid[resid_idx[i]] (row gather)
     const int32_t *resid_idx = nullptr;
     int32_t ld_resid = 0;
-    // order in which the persistent kernel walks the tiles of SAT_TC_ROWS rows: [ceil(m / SAT_TC_ROWS)] row-tile indices, a permutation
+    // (with a gathered residual) order in which the persistent kernel walks the tiles of 128 rows: [ceil(m / 128)] row-tile indices, a permutation
     // (null: ascending).  Results do not depend on it; it decides which rows are in flight together.
     const int32_t *tile_order = nullptr;
     // fused LSTM cell (the weights must have been packed with gate interleave): the n = 4h outputs of a row are the gate

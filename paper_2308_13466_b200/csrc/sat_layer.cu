@@ -547,7 +547,7 @@ static sat_status run_lstm(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p
     return SAT_OK;
 }
 
-// Schedule of the predictor-output contraction over the halo rows of all partitions: tiles of SAT_TC_ROWS rows ordered by the
+// Schedule of the predictor-output contraction over the halo rows of all partitions: tiles of 128 rows ordered by the
 // cache slot of their first row.  Every partition's halo list is sorted by node id, hence by slot, so a tile covers a
 // narrow slot range; walking the tiles of all partitions in slot order puts the (on average 3-4) halo copies of a cached
 // node in flight together, and its newest-snapshot row — the skip connection the epilogue gathers — is read from DRAM once
@@ -555,13 +555,13 @@ static sat_status run_lstm(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p
 __global__ void k_tile_keys(const int32_t *__restrict__ halo_slot, int64_t n_halo, int64_t n_tiles, int32_t *__restrict__ keys)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n_tiles) keys[t] = halo_slot[t * SAT_TC_ROWS < n_halo ? t * SAT_TC_ROWS : n_halo - 1];
+    if (t < n_tiles) keys[t] = halo_slot[t * 128 < n_halo ? t * 128 : n_halo - 1];
 }
 
 static sat_status halo_tile_order(sat_ctx *ctx, int64_t n_halo, const int32_t **out)
 {
     if (!ctx->halo_tile_order) {
-        const int64_t n_tiles = cdiv64(n_halo, SAT_TC_ROWS);
+        const int64_t n_tiles = cdiv64(n_halo, 128);
         int32_t *d = nullptr;
         SAT_CUDA(ctx, cudaMalloc((void **)&d, (size_t)n_tiles * sizeof(int32_t)));
         k_tile_keys<<<(unsigned)cdiv64(n_tiles, 256), 256, 0, ctx->stream>>>(ctx->halo_slot, n_halo, n_tiles, d);

@@ -249,3 +249,23 @@ def test_gru_state(B, d, h, steps):
         ds = e[:, h:2 * h] / 2 + 2 * e[:, 2 * h:] + np.abs(hn) * e[:, :h] / 4 + ds + 2.0 ** -20
         s = (1 - z) * cand + z * s
     assert (np.abs(S - s) <= ds).all()
+
+
+@pytest.mark.parametrize("n,k", [(16, 16), (40, 100), (72, 17), (128, 256), (256, 64), (257, 40), (300, 602)])
+@pytest.mark.parametrize("rows", [-1, 0, 1, 128, 129, 256, 20000])      # relative to a wave of single CTAs (128 rows each): pairs above it
+def test_contraction_by_single_ctas_and_by_pairs(B, n, k, rows):
+    tiles_n = -(-n // 256)
+    m = 128 * (torch.cuda.get_device_properties(0).multi_processor_count // tiles_n) + rows
+    rng = np.random.default_rng(n + k)
+    A, W, b = (rng.standard_normal(s).astype(np.float32) for s in ((m, k), (k, n), (n,)))
+    ctx = B.sat_create(0, 0)
+    try:
+        out = empty2d(m, n)
+        B.sat_dense_nn(ctx, dev2d(A), dev(W), dev(b), out)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    sel = np.unique(np.concatenate([np.arange(300), np.arange(m - 300, m), rng.integers(0, m, 300)]))
+    a = A[sel].astype(np.float64)
+    bound = ((k + 2) * U + 2.0 ** -20) * (np.abs(a) @ np.abs(W) + np.abs(b))
+    assert (np.abs(out.cpu().numpy()[sel] - (a @ W + b)) <= bound).all()
