@@ -12,7 +12,7 @@
 //   k_gemm_tc_mn  C[M x N] = A[R x M]^T B[R x N]   both operands MN-major, 128-byte swizzle with 32-byte atoms, split over R
 //                 (weight gradient)
 // Warp roles of k_gemm_tc_k (512 threads): warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, then 6 converter and
-// 8 epilogue warps (two per TMEM lane quadrant), or 2 + 12 for the K = h variants with a side operand.  k_gemm_tc_mn:
+// 8 epilogue warps (two per TMEM lane quadrant), or 2 + 12 with a gathered residual (K = h).  k_gemm_tc_mn:
 // warps 0 / 1 as above, warps 2..9 convert during the main loop and then run the epilogue.  Every mbarrier wait is
 // bounded; a timeout raises a status word and lets the CTA drain (TMEM is freed, the kernel returns).
 #include <cuda.h>
@@ -287,8 +287,7 @@ struct TcEpilogue {
     int32_t lstm_h;      // > 0: fused recurrent cell, C = hidden state [M x lstm_h], lstm_c = cell state (LSTM only)
     int lstm_first;
     float *lstm_c;       // cell state in the blocked layout of sat_cell_offset
-    const float *addend; // [M x ld_addend] added to the gate pre-activations (cached input projection), or null
-    int64_t ld_addend;
+    int32_t proj_h;      // (EPI_PROJ) hidden units: C is a projection plane, see sat_proj_floats
     float *push_dst;     // (EPI_PUSH) row i is also written to push_dst + push_slot[i] * ld_push when push_slot[i] >= 0
     const int32_t *push_slot;
     int64_t ld_push;
@@ -331,12 +330,12 @@ struct TcShared {
 // LSTM input projection) keep a ring of 32 x 32 side tiles per epilogue warp in shared memory, filled by cp.async ahead of
 // the consumer: one chunk in flight per warp left the loads latency-bound at ~2 TB/s.  Those variants contract over a
 // small K (the predictor width), so they give up main-loop stages for the ring.
-enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_LSTM = 2, EPI_LSTM_ADD = 3, EPI_PUSH = 4, EPI_GRU = 5 };   // EPI_PUSH = EPI_PLAIN + a second copy of the rows that have a cache slot
+enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_LSTM = 2, EPI_PROJ = 3, EPI_PUSH = 4, EPI_GRU = 5 };   // EPI_PUSH = EPI_PLAIN + a second copy of the rows that have a cache slot
 template <int EPI> struct TckCfg { static constexpr int ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = epi_warps * 4096; };
 template <> struct TckCfg<EPI_RESID> { static constexpr int ring = 1, conv_warps = 2, epi_warps = 12, out_bytes = epi_warps * 4096; };
 template <> struct TckCfg<EPI_LSTM> { static constexpr int ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = 0; };
 template <> struct TckCfg<EPI_GRU> : TckCfg<EPI_LSTM> {};
-template <> struct TckCfg<EPI_LSTM_ADD> { static constexpr int ring = 2, conv_warps = 2, epi_warps = 12, out_bytes = 0; };
+template <> struct TckCfg<EPI_PROJ> : TckCfg<EPI_LSTM> {};
 
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, bool valid)
 {
@@ -486,7 +485,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         // ---------------- epilogue ----------------
         // warp w reads TMEM lanes 32 (w % 4) .. +31 = rows of the tile, one row per thread; the warps of a lane quadrant
         // take alternate 32-column chunks.
-        constexpr bool LSTM = EPI == EPI_LSTM || EPI == EPI_LSTM_ADD || EPI == EPI_GRU;   // a recurrent cell
+        constexpr bool LSTM = EPI == EPI_LSTM || EPI == EPI_GRU;   // a recurrent cell
         const int e = warp - EPI_WARP0;
         const int q = warp & 3;
         const int c_first = 32 * (e >> 2);
@@ -513,16 +512,11 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             if (pf_t < n_tiles) {
                 const int64_t prow = tile_row(pf_t) + lane;
                 const int32_t pn0 = (int32_t)(pf_t % n_tiles_n) * bn;
-                if (EPI == EPI_RESID) {
-                    if (prow < M && idx_now >= 0) pf_srow = ep.resid + (int64_t)idx_now * ep.ld_resid + pn0;  // rows padded to 4 floats
-                    pf_lim = n4 - pn0;
-                    const int64_t nt = pf_t + units;
-                    const int64_t nrow = nt < n_tiles ? tile_row(nt) + lane : M;
-                    pf_idx_next = nrow < M ? __ldg(ep.resid_idx + nrow) : -1;
-                } else {
-                    if (prow < M) pf_srow = ep.addend + prow * ep.ld_addend + pn0;
-                    pf_lim = N - pn0;
-                }
+                if (prow < M && idx_now >= 0) pf_srow = ep.resid + (int64_t)idx_now * ep.ld_resid + pn0;  // rows padded to 4 floats
+                pf_lim = n4 - pn0;
+                const int64_t nt = pf_t + units;
+                const int64_t nrow = nt < n_tiles ? tile_row(nt) + lane : M;
+                pf_idx_next = nrow < M ? __ldg(ep.resid_idx + nrow) : -1;
             }
         };
         auto pf_issue = [&]() {
@@ -531,27 +525,14 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             // matters because the load/store unit handles one line per cycle.
             if (pf_t < n_tiles && pf_c < bn) {
                 uint8_t *slot = ring + pf_slot * 4096;
-                const float *base = EPI == EPI_RESID ? ep.resid : ep.addend;
                 const int piece = lane & 7;
                 const bool col_ok = pf_c + 4 * piece < pf_lim;
-                if (EPI == EPI_RESID) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {  // gathered rows: the row pointer lives in the lane that owns the row
-                        const int rr = (lane >> 3) + 4 * i;
-                        const float *rowp = reinterpret_cast<const float *>(__shfl_sync(0xffffffffu, (unsigned long long)(uintptr_t)pf_srow, rr));
-                        const bool valid = rowp != nullptr && col_ok;
-                        cp_async16(slot + rr * 128 + ((piece ^ (rr & 7)) << 4), (valid ? rowp : base) + pf_c + 4 * piece, valid);
-                    }
-                } else {
-                    // dense side operand: rows of the tile are ld_addend apart
-                    const int64_t prow0 = tile_row(pf_t) + (lane >> 3);
-                    const float *p0 = base + prow0 * ep.ld_addend + (int32_t)(pf_t % n_tiles_n) * bn + pf_c + 4 * piece;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int rr = (lane >> 3) + 4 * i;
-                        const bool valid = prow0 + 4 * i < M && col_ok;
-                        cp_async16(slot + rr * 128 + ((piece ^ (rr & 7)) << 4), valid ? p0 + (int64_t)(4 * i) * ep.ld_addend : base, valid);
-                    }
+                for (int i = 0; i < 8; ++i) {  // the row pointer lives in the lane that owns the row
+                    const int rr = (lane >> 3) + 4 * i;
+                    const float *rowp = reinterpret_cast<const float *>(__shfl_sync(0xffffffffu, (unsigned long long)(uintptr_t)pf_srow, rr));
+                    const bool valid = rowp != nullptr && col_ok;
+                    cp_async16(slot + rr * 128 + ((piece ^ (rr & 7)) << 4), (valid ? rowp : ep.resid) + pf_c + 4 * piece, valid);
                 }
                 pf_c += CHUNK_STEP;
                 if (pf_c >= bn) {
@@ -565,7 +546,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         };
         if (RING > 0 && c_first < bn) {
             int32_t idx0 = -1;
-            if (EPI == EPI_RESID && pf_t < n_tiles) {
+            if (pf_t < n_tiles) {
                 const int64_t prow = tile_row(pf_t) + lane;
                 if (prow < M) idx0 = __ldg(ep.resid_idx + prow);
             }
@@ -633,7 +614,7 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         const bool full = lstm_full && j0 + 7 < ep.lstm_h;
 #pragma unroll
                         for (int u = 0; u < 8; ++u) {
-                            float4 b4 = EPI == EPI_LSTM_ADD ? side[u] : zero4;
+                            float4 b4 = zero4;
                             if (ep.bias) {
                                 const float4 bb = __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + c0) + u);
                                 b4.x += bb.x; b4.y += bb.y; b4.z += bb.z; b4.w += bb.w;
@@ -714,6 +695,18 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(fmaxf(__uint_as_float(r[j]), 0.f));
                     }
                 }
+                if (EPI == EPI_PROJ) {   // a warp's store of a unit is 512 contiguous bytes
+                    if (row_ok) {
+                        const int32_t j0 = (n0 + c0) >> 2;
+                        float4 *dst = reinterpret_cast<float4 *>(ep.C) + ((row >> 7) * ep.proj_h + j0) * 128 + (row & 127);
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (j0 + u < ep.proj_h)
+                                dst[u * 128] = make_float4(__uint_as_float(r[4 * u]), __uint_as_float(r[4 * u + 1]), __uint_as_float(r[4 * u + 2]),
+                                                           __uint_as_float(r[4 * u + 3]));
+                    }
+                    continue;
+                }
                 if (EPI == EPI_PUSH && prow) {   // one full 128-byte line per thread and chunk
 #pragma unroll
                     for (int j4 = 0; j4 < 32; j4 += 4) {
@@ -791,6 +784,220 @@ done:
         __syncwarp();
         tc_fence_after();
         tc_dealloc<CTAS>(tmem, 512u);
+    }
+}
+
+// =====================================================================================
+// LSTM steps over cached input projections, all in one kernel: z = proj_t + s Uh, c = f c + i g, s = o tanh(c) for consecutive steps t.
+//
+// One launch per step moved the state s and c through memory every time and fetched Uh for every tile: 345 MB a step at 169343 rows and
+// h = 64, half of it the projection (83 us a step, and 54 for the first one).  Here a row tile stays on the SM for all steps: s as the
+// A operand in shared memory, c in registers, Uh resident; a step reads its projection and nothing else.
+//
+// A CTA pair (cta_group::2) works on two slots of 256 rows (128 per CTA) in turn, so that one slot's MMA runs under the other's
+// cell arithmetic: Uh takes 64 KB per CTA (half of the columns, both planes, h = 64), the two slots 64 KB each, and the accumulators
+// all of TMEM.  Eight warps per slot, two per lane quadrant with alternate quads of four units: one row per thread.  Projections are stored
+// [row tile of 128][unit][row] float4 (sat_proj_floats), so a warp reads 512 contiguous bytes and the next step's block of a tile is one
+// bulk prefetch into L2.  Bound by the hardware exponential and reciprocal (ten per unit and step: 2.7 us per 128 rows at h = 64) next to
+// the projection stream (3.0 us).
+// =====================================================================================
+#define SEQ_THREADS (17 * 32)
+struct SeqSteps {
+    const float *proj[SAT_SEQ_MAX];
+};
+struct SeqShared {
+    uint64_t b_full, b_ready;           // Uh has landed in this CTA; in both
+    uint64_t a_ready[2], acc_full[2];   // per slot: the state is in place; the product is done
+    uint32_t tmem_base;
+    int dead;
+};
+
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t *r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(SEQ_THREADS, 1)
+k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo, const __grid_constant__ SeqSteps steps, int32_t n_steps,
+           int first, int64_t rows, int32_t h, int32_t bn, int32_t nkb, float *S, float *cell, int write_cell, int *status)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    constexpr uint32_t a_plane = TC_BM * TC_BK * 4;               // one plane of a k-block of the state: 128 rows x 64 B, 64-byte swizzle
+    const uint32_t b_plane = (uint32_t)bn / 2 * TC_BK * 4;
+    const uint32_t slot_bytes = (uint32_t)nkb * 2 * a_plane;      // [k-block][hi | lo]
+    uint8_t *Bs = smem + 2 * slot_bytes;                          // [k-block][hi | lo]
+    SeqShared *sh = (SeqShared *)(Bs + (size_t)nkb * 2 * b_plane);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = blockIdx.x & 1u;
+    const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1, n_pt = (rows + 255) / 256;
+    const int32_t mine = unit < n_pt ? (int32_t)((n_pt - 1 - unit) / units + 1) : 0;   // tiles of the pair, alternately in slot 0 and 1
+
+    for (uint32_t o = threadIdx.x * 16; o < 2 * slot_bytes; o += SEQ_THREADS * 16) *reinterpret_cast<float4 *>(smem + o) = make_float4(0.f, 0.f, 0.f, 0.f);
+    fence_async_smem();   // (the columns h .. 16 nkb stay zero)
+    if (threadIdx.x == 0) {
+        mbar_init(&sh->b_full, 1);
+        mbar_init(&sh->b_ready, 2);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sh->a_ready[i], 2 * 8);
+            mbar_init(&sh->acc_full[i], 1);
+        }
+        sh->dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 16) tc_alloc<2>(&sh->tmem_base, 512u);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    tc_fence_after();
+    const uint32_t tmem = sh->tmem_base;
+    volatile int *dead = &sh->dead;
+    sat_grid_wait();
+
+    if (warp == 16) {
+        if (lane == 0) {
+            mbar_expect_tx(&sh->b_full, (uint32_t)nkb * 2 * b_plane);
+            for (int32_t kb = 0; kb < nkb; ++kb) {
+                tma_load_2d(Bs + (size_t)kb * 2 * b_plane, &mapB, &sh->b_full, kb * TC_BK, (int32_t)rank * (bn / 2));
+                tma_load_2d(Bs + ((size_t)kb * 2 + 1) * b_plane, &mapBlo, &sh->b_full, kb * TC_BK, (int32_t)rank * (bn / 2));
+            }
+        }
+        if (!mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
+        mbar_arrive_warp<2>(&sh->b_ready, lane);
+        if (rank == 0) {
+            if (!mbar_wait_all(&sh->b_ready, 0, dead, status)) goto done;
+            const uint32_t idesc = make_idesc(2 * TC_BM, bn, 0, 0);
+            const uint64_t a0 = make_desc(smem_u32(smem), 16, 512, 4), b0 = make_desc(smem_u32(Bs), 16, 512, 4);
+            const int32_t products = n_steps - (first ? 1 : 0);   // per tile: the first step has no state yet
+            const int32_t count0 = (mine + 1) / 2 * products, count1 = mine / 2 * products;
+            for (int32_t i = 0; i < count0; ++i)
+                for (int sl = 0; sl < 2; ++sl) {
+                    if (sl == 1 && i >= count1) continue;
+                    if (!mbar_wait_all(&sh->a_ready[sl], (uint32_t)i & 1u, dead, status)) goto done;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint32_t acc = tmem + (uint32_t)sl * 256u;
+                        for (int32_t kb = 0; kb < nkb; ++kb) {
+#pragma unroll
+                            for (int ks = 0; ks < TC_BK / 8; ++ks) {
+                                const uint64_t a_hi = a0 + (uint64_t)(((uint32_t)sl * slot_bytes + (uint32_t)kb * 2 * a_plane) >> 4) + (uint64_t)(ks * 2);
+                                const uint64_t b_hi = b0 + (uint64_t)(((uint32_t)kb * 2 * b_plane) >> 4) + (uint64_t)(ks * 2);
+                                const uint64_t a_lo = a_hi + (a_plane >> 4), b_lo = b_hi + (b_plane >> 4);
+                                tc_mma<1, 2>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                                tc_mma<2, 2>(acc, a_hi, b_lo, idesc, 1u);
+                                tc_mma<0, 2>(acc, a_lo, b_hi, idesc, 1u);
+                            }
+                        }
+                        tc_commit<2>(&sh->acc_full[sl]);
+                    }
+                }
+        }
+    } else {
+        const int slot = warp >> 3, q = warp & 3, half = (warp >> 2) & 1;
+        const int32_t nq = h >> 2;                       // quads of four units
+        const int r_in = q * 32 + lane;                  // this thread's row of the tile
+        uint8_t *A = smem + (uint32_t)slot * slot_bytes + r_in * 64;
+        const uint32_t swz = (uint32_t)(r_in >> 1) & 3u; // 64-byte swizzle: 16-byte piece c of row r sits at c ^ ((r >> 1) & 3)
+        auto put = [&](int qd, const float4 &v) {
+            uint8_t *d = A + (uint32_t)(qd >> 2) * 2 * a_plane + ((((uint32_t)qd & 3u) ^ swz) << 4);
+            *reinterpret_cast<float4 *>(d) = v;
+            *reinterpret_cast<float4 *>(d + a_plane) = residual4(v);
+        };
+        uint32_t ph = 0;
+        for (int32_t k = slot; k < mine; k += 2) {
+            const int64_t rt = (unit + (int64_t)k * units) * 2 + rank;   // row tile of 128
+            const int64_t row = rt * TC_BM + r_in;
+            const bool row_ok = row < rows, tile_ok = rt * TC_BM < rows;
+            float4 c[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int32_t qd = half + 2 * i;
+                c[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (!first && qd < nq) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (row_ok) {
+                        v = *reinterpret_cast<const float4 *>(S + row * h + 4 * qd);
+                        c[i] = *reinterpret_cast<const float4 *>(cell + sat_cell_offset(row, 4 * qd, h));
+                    }
+                    put(qd, v);
+                }
+            }
+            for (int32_t t = 0; t < n_steps; ++t) {
+                const bool product = t > 0 || !first, last = t + 1 == n_steps;
+                if (product) {
+                    fence_async_smem();
+                    tc_fence_before();
+                    mbar_arrive_warp<2>(&sh->a_ready[slot], lane);
+                }
+                const float4 *pr = reinterpret_cast<const float4 *>(steps.proj[t]) + rt * h * 128 + r_in;
+                if ((warp & 7) == 0 && lane == 0) {   // what this slot reads next, into L2
+                    const int64_t rn = last ? (unit + (int64_t)(k + 2) * units) * 2 + rank : rt;
+                    if (rn * TC_BM < rows && (!last || k + 2 < mine)) {
+                        const float *nx = steps.proj[last ? 0 : t + 1] + rn * h * 512;
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(nx), "r"((uint32_t)h * 2048u) : "memory");
+                    }
+                }
+                float4 nx[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) nx[u] = tile_ok && half < nq ? __ldg(pr + (4 * half + u) * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (product) {
+                    if (!mbar_wait_all(&sh->acc_full[slot], ph, dead, status)) goto done;
+                    ph ^= 1u;
+                    tc_fence_after();
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int32_t qd = half + 2 * i;
+                    if (qd < nq) {
+                        float4 z[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            z[u] = nx[u];
+                            if (tile_ok && qd + 2 < nq) nx[u] = __ldg(pr + (4 * (qd + 2) + u) * 128);
+                        }
+                        if (product) {
+                            uint32_t r[16];
+                            tc_ld16(tmem + (uint32_t)slot * 256u + ((uint32_t)(q * 32) << 16) + 16u * (uint32_t)qd, r);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                z[u].x += __uint_as_float(r[4 * u]);
+                                z[u].y += __uint_as_float(r[4 * u + 1]);
+                                z[u].z += __uint_as_float(r[4 * u + 2]);
+                                z[u].w += __uint_as_float(r[4 * u + 3]);
+                            }
+                        }
+                        float4 sv;
+                        float *cf = reinterpret_cast<float *>(&c[i]), *sf = reinterpret_cast<float *>(&sv);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {   // (i, f, g, o) of unit 4 qd + u
+                            const float gi = sigmoid_fast(z[u].x), gf = sigmoid_fast(z[u].y), gg = tanh_fast(z[u].z), go = sigmoid_fast(z[u].w);
+                            cf[u] = gf * cf[u] + gi * gg;
+                            sf[u] = go * tanh_fast(cf[u]);
+                        }
+                        if (!last) {
+                            put(qd, sv);
+                        } else if (row_ok) {
+                            *reinterpret_cast<float4 *>(S + row * h + 4 * qd) = sv;
+                            if (write_cell) *reinterpret_cast<float4 *>(cell + sat_cell_offset(row, 4 * qd, h)) = c[i];
+                        }
+                    }
+                }
+            }
+        }
+    }
+done:
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
+    if (warp == 16) {
+        __syncwarp();
+        tc_fence_after();
+        tc_dealloc<2>(tmem, 512u);
     }
 }
 
@@ -1270,20 +1477,20 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     const int32_t nkb1 = (k1 + TC_BK - 1) / TC_BK, nkb2 = A2 ? (k2 + TC_BK - 1) / TC_BK : 0;
     const int32_t bn = tile_n_for(n);
     // CTA pairs for launches of more than one wave of single CTAs (below, the pair only adds its synchronisation: 6000 x 72, K = 50: 12.0
-    // -> 12.9 us), except with a side operand: those contract over the predictor width and are bound by the side operand's
-    // stream, which the pair holds up (gathered residual 145 -> 161 us, cached projection 92 -> 95 at 169343 rows)
+    // -> 12.9 us), except with a gathered residual: that contracts over the predictor width and is bound by the residual's
+    // stream, which the pair holds up (145 -> 161 us at 169343 rows)
     const int32_t n_tiles_n = (int32_t)cdiv64(n, bn);
-    const bool pair = !eh.resid_idx && !eh.addend && cdiv64(m, TC_BM) * n_tiles_n > ctx->sms;
+    const bool pair = !eh.resid_idx && cdiv64(m, TC_BM) * n_tiles_n > ctx->sms;
     const int ctas = pair ? 2 : 1;
     const uint32_t stage_bytes = 2 * (TC_BM * TC_BK * 4) + 2 * (uint32_t)bn / ctas * TC_BK * 4;
     // algorithmic bytes: operands once, results once.  Plain: A, B, C.  Gathered residual: + the residual rows.  LSTM cell:
     // the output is the hidden state [m x h] plus the cell state read and written, and the cached projection if it is added.
     double alg_bytes = 4.0 * ((double)m * (k1 + k2) + (double)(k1 + k2) * n);
-    if (eh.lstm_h > 0) alg_bytes += 4.0 * (double)m * eh.lstm_h * (eh.gru ? 1.0 : eh.lstm_first ? 2.0 : 3.0) + (eh.addend ? 4.0 * (double)m * n : 0.0);
+    if (eh.lstm_h > 0) alg_bytes += 4.0 * (double)m * eh.lstm_h * (eh.gru ? 1.0 : eh.lstm_first ? 2.0 : 3.0);
     else alg_bytes += 4.0 * (double)m * n * (eh.resid_idx ? 2.0 : 1.0);
     ProfScope prof(ctx, family, alg_bytes, 2.0 * (double)m * n * (k1 + k2));
     CUtensorMap mA, mA2, mB, mBlo, mC;
-    const int use_tma_store = eh.lstm_h == 0 && ((eh.ldc & 3) == 0) && ((((uintptr_t)eh.C) & 15u) == 0);
+    const int use_tma_store = eh.lstm_h == 0 && eh.proj_h == 0 && ((eh.ldc & 3) == 0) && ((((uintptr_t)eh.C) & 15u) == 0);
     if (use_tma_store) SAT_TRY(make_map(ctx, &mC, eh.C, n, m, eh.ldc, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B));
     else memset(&mC, 0, sizeof(mC));
     SAT_TRY(make_map(ctx, &mA, A, k1, m, lda, TC_BK, TC_BM, CU_TENSOR_MAP_SWIZZLE_64B));
@@ -1300,7 +1507,7 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
         DevBuf &home = eh.bias_home ? *eh.bias_home : ctx->buf_bias;
         if (!(eh.bias_home && eh.bias_ready && home.bytes >= padded * sizeof(float))) {
             SAT_TRY(sat_ensure(ctx, home, padded * sizeof(float)));
-            sat_pdl(ctx->stream, k_pack_bias, (unsigned)cdiv64(padded, 256), 256, 0)(eh.bias, n, (int32_t)padded, eh.lstm_h > 0 ? eh.lstm_h : eh.pack_gate_h,
+            sat_pdl(ctx->stream, k_pack_bias, (unsigned)cdiv64(padded, 256), 256, 0)(eh.bias, n, (int32_t)padded, eh.lstm_h > 0 ? eh.lstm_h : eh.proj_h,
                                                                                 (float *)home.p);
             SAT_LAUNCHED(ctx);
         }
@@ -1314,10 +1521,9 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.lstm_h = eh.lstm_h;
     ep.lstm_first = eh.lstm_first;
     ep.lstm_c = eh.lstm_c;
-    ep.addend = eh.addend;
-    ep.ld_addend = eh.ld_addend;
-    if (eh.lstm_h > 0 && ((!eh.bias && !eh.addend) || (eh.gru ? eh.addend != nullptr : !eh.lstm_c) || n != 4 * eh.lstm_h || (eh.addend && (eh.ld_addend & 3))))
-        return sat_fail(ctx, SAT_EINVAL, "fused recurrent epilogue needs bias or addend, cell state (LSTM) and n = 4h");
+    ep.proj_h = eh.proj_h;
+    if (eh.lstm_h > 0 && (!eh.bias || (!eh.gru && !eh.lstm_c) || n != 4 * eh.lstm_h))
+        return sat_fail(ctx, SAT_EINVAL, "fused recurrent epilogue needs bias, cell state (LSTM) and n = 4h");
     if (eh.resid_idx && (eh.mask_out || eh.lstm_h > 0))
         return sat_fail(ctx, SAT_EINVAL, "gathered-residual epilogue cannot be combined with a mask output or the LSTM cell");
     ep.relu = eh.relu;
@@ -1336,11 +1542,36 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     L.grid = grid;
     L.stage_bytes = stage_bytes;
     if (eh.gru) return pair ? launch_tck<EPI_GRU, 2>(ctx, L, ep) : launch_tck<EPI_GRU, 1>(ctx, L, ep);
-    if (ep.lstm_h > 0 && ep.addend) return launch_tck<EPI_LSTM_ADD, 1>(ctx, L, ep);
+    if (ep.proj_h > 0) return pair ? launch_tck<EPI_PROJ, 2>(ctx, L, ep) : launch_tck<EPI_PROJ, 1>(ctx, L, ep);
     if (ep.lstm_h > 0) return pair ? launch_tck<EPI_LSTM, 2>(ctx, L, ep) : launch_tck<EPI_LSTM, 1>(ctx, L, ep);
     if (ep.resid_idx) return launch_tck<EPI_RESID, 1>(ctx, L, ep);
     if (ep.push_dst) return pair ? launch_tck<EPI_PUSH, 2>(ctx, L, ep) : launch_tck<EPI_PUSH, 1>(ctx, L, ep);
     return pair ? launch_tck<EPI_PLAIN, 2>(ctx, L, ep) : launch_tck<EPI_PLAIN, 1>(ctx, L, ep);
+}
+
+sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
+                        float *cell, int write_cell)
+{
+    if (rows == 0 || n_steps == 0) return SAT_OK;
+    if (n_steps > SAT_SEQ_MAX || h > 64 || (h & 3)) return sat_fail(ctx, SAT_EINVAL, "sat_lstm_seq: at most %d steps and 64 units", SAT_SEQ_MAX);
+    ProfScope prof(ctx, SATK_GEMM_SIDE, 4.0 * (double)rows * h * (4.0 * n_steps + 1.0 + (first ? 0.0 : 2.0)), 8.0 * (double)rows * h * h * (n_steps - (first ? 1 : 0)));
+    const int32_t bn = tile_n_for(4 * h), nkb = (h + TC_BK - 1) / TC_BK;
+    const size_t smem = (size_t)2 * nkb * 2 * TC_BM * TC_BK * 4 + (size_t)nkb * 2 * (bn / 2) * TC_BK * 4 + sizeof(SeqShared) + 1024;
+    static PerDeviceOnce attr_set;
+    if (attr_set.need(ctx->device)) {
+        SAT_CUDA(ctx, cudaFuncSetAttribute(k_lstm_seq, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        attr_set.mark(ctx->device);
+    }
+    CUtensorMap mB, mBlo;
+    SAT_TRY(make_map(ctx, &mB, Uh.hi, Uh.ld, Uh.n_pad, Uh.ld, TC_BK, bn / 2, CU_TENSOR_MAP_SWIZZLE_64B));
+    SAT_TRY(make_map(ctx, &mBlo, Uh.lo, Uh.ld, Uh.n_pad, Uh.ld, TC_BK, bn / 2, CU_TENSOR_MAP_SWIZZLE_64B));
+    SeqSteps st;
+    for (int32_t t = 0; t < SAT_SEQ_MAX; ++t) st.proj[t] = t < n_steps ? proj[t] : nullptr;
+    const int64_t tiles = cdiv64(rows, 2 * TC_BM), units = ctx->sms / 2;
+    sat_pdl(ctx->stream, k_lstm_seq, (unsigned)(tiles < units ? tiles : units) * 2, SEQ_THREADS, smem, 2)(mB, mBlo, st, n_steps, first, rows, h, bn, nkb, S, cell,
+                                                                                                write_cell, ctx->d_flag + 1);
+    SAT_LAUNCHED(ctx);
+    return SAT_OK;
 }
 
 // C[m x n] (+)= A^T B over `rows` rows: A fp32 [rows x m] (lda), B fp32 [rows x n] (ldb)

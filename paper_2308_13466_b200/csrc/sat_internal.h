@@ -77,7 +77,7 @@ struct CacheLayer {
     int32_t S_h = 0;
     bool S_valid = false;
     // input projections x Wx + b of the ring buffers (gate-interleaved columns), reused while the caller's parameter
-    // version stays the same: [(tau+1) x n_slots x 4 proj_h]; proj_tag[i] = version the projection of buffer i was made with
+    // version stays the same: [(tau+1) x sat_proj_floats]; proj_tag[i] = version the projection of buffer i was made with
     float *proj = nullptr;
     int32_t proj_h = 0;
     std::vector<uint64_t> proj_tag;
@@ -515,9 +515,8 @@ struct TcEpilogueHost {
     int lstm_first = 0;                // first step: previous cell state (GRU: hidden state) is zero
     int gru = 0;                       // GRU cell instead (weights packed with gates = 3): C is also the previous hidden state, no lstm_c
     float *lstm_c = nullptr;
-    const float *addend = nullptr;     // dense [m x ld_addend], added to the accumulators before the LSTM cell (row-aligned)
-    int32_t ld_addend = 0;
-    int32_t pack_gate_h = 0;           // > 0: the bias is interleaved like weights packed with gate_h (without the LSTM epilogue)
+    // > 0: an input projection of the LSTM with this many units: weights packed with gate_h, bias interleaved alike, C a projection plane
+    int32_t proj_h = 0;
     // second destination of the rows that have a cache slot (the push of Algorithm 1 fused into the layer transform):
     // row i also goes to push_dst + push_slot[i] * ld_push when push_slot[i] >= 0
     float *push_dst = nullptr;
@@ -540,6 +539,13 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
                           int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0, int gates = 4);
 sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out);
+// Plane of an input projection x Wx + b of the LSTM, [row tile of 128][unit][row of the tile][i f g o]
+inline int64_t sat_proj_floats(int64_t rows, int32_t h) { return (rows + 127) / 128 * 512 * h; }
+// LSTM steps over `n_steps` projection planes, oldest first, on the state S [rows x h] and the cell state (sat_cell_offset layout; read
+// unless `first`, i.e. both start from zero; written with write_cell).  Uh packed with gate_h; h a multiple of 4 up to 64.
+#define SAT_SEQ_MAX 32
+sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
+                        float *cell, int write_cell);
 // C[m x n] = [A | A2] B^T (+ epilogue)
 sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32_t lda, int32_t k1, const float *A2, int32_t lda2, int32_t k2,
                        const TcWeights &Bw, const TcEpilogueHost &eh, int family);

@@ -271,24 +271,8 @@ sat_status sat_gemm_nn_dual(sat_ctx *ctx, int64_t m, int32_t n, int32_t k1, cons
                             int32_t k2, const float *A2, int32_t lda2, const float *B2, int32_t ldb2, const float *bias, float *C,
                             int32_t ldc);
 
-// first LSTM step from a cached input projection (gate-interleaved columns 4 j + gate): previous state is zero
-__global__ void k_lstm_cell_first(const float *__restrict__ proj, int64_t rows, int32_t h, float *__restrict__ c, float *__restrict__ s)
-{
-    sat_grid_wait();
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= rows * h) return;
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(proj) + t);  // (i, f, g, o) of unit t % h of row t / h
-    const float gi = sigmoid_fast(a.x);   // same gate arithmetic as the fused cell of the later steps
-    const float gg = tanh_fast(a.z);
-    const float go = sigmoid_fast(a.w);
-    const float cn = gi * gg;
-    const int64_t r = sat_div(t, h);
-    c[sat_cell_offset(r, (int32_t)(t - r * h), h)] = cn;
-    s[t] = go * tanh_fast(cn);
-}
-
 // LSTM with cached input projections (parameter version promised by the caller).  A snapshot whose projection x Wx + b is
-// cached runs its step as a contraction over h only, with the projection added in the epilogue.  A missing projection is
+// cached needs a contraction over h only, and consecutive ones run as one launch (sat_lstm_seq).  A missing projection is
 // computed (and kept) only for the newest snapshot, which has tau - 1 further epochs of use ahead; an older snapshot
 // without one (after a version bump) runs its step as the contraction over [x | s] instead, which costs less than
 // projecting it for the one or two epochs it has left.
@@ -296,7 +280,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
 {
     const int32_t h = p->h, d = c->width;
     const int64_t rows = ctx->n_slots;
-    const int64_t plane = rows * 4 * h;
+    const int64_t plane = sat_proj_floats(rows, h);
     if (!c->proj || c->proj_h != h) {
         SAT_TRY(dev_realloc(ctx, &c->proj, (int64_t)(ctx->tau + 1) * plane));
         c->proj_h = h;
@@ -327,29 +311,22 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
         eh.C = c->proj + (int64_t)newest * plane;
         eh.ldc = 4 * h;
         eh.bias = p->b;
-        eh.pack_gate_h = h;
+        eh.proj_h = h;
         eh.bias_home = &c->pk_b;
         eh.bias_ready = c->tag_b == p->version;
         c->tag_b = p->version;
         SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, ring_buf(ctx, c, newest), c->ld, d, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
         c->proj_tag[newest] = p->version;
     }
-    // (Running the steps row block by row block, so that a block's state stays in L2 between two steps, was measured and
-    // was slower: the smaller launches cost more than the state traffic they save.)
-    for (int32_t t = 0; t < k; ++t) {
-        const int32_t idx = ring_index(ctx, k - 1 - t);  // oldest first
-        const bool cached = c->proj_tag[idx] == p->version;
-        const float *pr = c->proj + (int64_t)idx * plane;
-        TcEpilogueHost eh;
-        eh.C = c->S;
-        eh.ldc = h;
-        eh.lstm_h = h;
-        eh.lstm_c = cell;
-        if (cached && t == 0) {
-            ProfScope prof(ctx, SATK_LSTM_CELL, 4.0 * (double)rows * h * 6.0, 0.0);
-            sat_pdl(ctx->stream, k_lstm_cell_first, (unsigned)cdiv64(rows * h, 256), 256, 0)(pr, rows, h, cell, c->S);
-            SAT_LAUNCHED(ctx);
-        } else if (cached) {
+    auto is_cached = [&](int32_t t) { return c->proj_tag[ring_index(ctx, k - 1 - t)] == p->version; };   // step t, oldest first
+    for (int32_t t = 0; t < k;) {
+        if (is_cached(t)) {
+            const float *planes[SAT_SEQ_MAX];
+            int32_t n = 0;
+            while (t + n < k && n < SAT_SEQ_MAX && is_cached(t + n)) {
+                planes[n] = c->proj + (int64_t)ring_index(ctx, k - 1 - t - n) * plane;
+                ++n;
+            }
             if (!have_up) {
                 if (c->tag_uh == p->version) {
                     SAT_TRY(sat_tc_weights_layout(h, 4 * h, c->pk_uh, &Up));
@@ -359,20 +336,27 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
                 }
             }
             have_up = true;
-            eh.addend = pr;
-            eh.ld_addend = 4 * h;
-            SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, c->S, h, h, nullptr, 0, 0, Up, eh, SATK_GEMM_SIDE));
-        } else if (t == 0) {
+            SAT_TRY(sat_lstm_seq(ctx, rows, h, Up, planes, n, t == 0, c->S, cell, t + n < k));
+            t += n;
+            continue;
+        }
+        const float *x = ring_buf(ctx, c, ring_index(ctx, k - 1 - t));
+        TcEpilogueHost eh;
+        eh.C = c->S;
+        eh.ldc = h;
+        eh.lstm_h = h;
+        eh.lstm_c = cell;
+        eh.bias = p->b;
+        if (t == 0) {
             SAT_TRY(pack_wx());
-            eh.bias = p->b;
             eh.lstm_first = 1;
-            SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, ring_buf(ctx, c, idx), c->ld, d, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
+            SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, x, c->ld, d, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
         } else {
             if (!have_wxu) SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, p->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit3, &Wxu, h));
             have_wxu = true;
-            eh.bias = p->b;
-            SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, ring_buf(ctx, c, idx), c->ld, d, c->S, h, h, Wxu, eh, SATK_GEMM_NN));
+            SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, x, c->ld, d, c->S, h, h, Wxu, eh, SATK_GEMM_NN));
         }
+        ++t;
     }
     c->S_valid = true;
     return SAT_OK;

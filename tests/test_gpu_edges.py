@@ -269,3 +269,51 @@ def test_contraction_by_single_ctas_and_by_pairs(B, n, k, rows):
     a = A[sel].astype(np.float64)
     bound = ((k + 2) * U + 2.0 ** -20) * (np.abs(a) @ np.abs(W) + np.abs(b))
     assert (np.abs(out.cpu().numpy()[sel] - (a @ W + b)) <= bound).all()
+
+
+@pytest.mark.parametrize("n,h,d,versions", [(700, h, d, v) for h in (16, 20, 32, 48, 60, 64) for d, v in ((16, [1]), (100, [1, 1]), (40, [1] * 6))] +
+                         [(700, 64, 40, [1, 1, 2, 1, 1]), (700, 24, 40, [2, 1, 1, 1]), (45000, 64, 40, [1, 1, 1]), (45000, 20, 16, [1, 2, 1, 1])])
+def test_lstm_state_over_cached_projections(B, n, h, d, versions):
+    """State of the predictor after every epoch, its parameter version as given (steps over cached projections run as one launch, others on
+    their own; more than 256 rows a CTA pair at the larger size) against the cell in fp64.  With e the error of a pre-activation (bound
+    of the module's docstring, and what the previous state brings through Uh), eta = 2^-20 that of a gate, sigma' <= 1/4, tanh' <= 1:
+    |dc| <= |c| (e_f / 4 + eta) + |dc_prev| + |g| (e_i / 4 + eta) + e_g + eta,  |ds| <= e_o / 4 + eta + |dc| + eta."""
+    tau, M = 5, 3
+    A = _graph([300, 40], n)
+    rng = np.random.default_rng(d + h)
+    part = rng.integers(0, M, n).astype(np.int32)
+    perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+    W, Uh, b = rng.standard_normal((d, 4 * h)) / d ** 0.5, rng.standard_normal((h, 4 * h)) / h ** 0.5, rng.standard_normal(4 * h) / 4
+    W, Uh, b, Wg, bg = (x.astype(np.float32) for x in (W, Uh, b, np.zeros((h, d)), np.zeros(d)))
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        B.sat_cache_init(ctx, [d], tau)
+        out = empty2d(sum(B.sat_part_sizes(ctx, m)[1] for m in range(M)), d)
+        n_slots = B.sat_slot_map(ctx, n)[2]
+        weights = [dev(x) for x in (W, Uh, b, Wg, bg)]
+        for version in versions:
+            B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, dev2d(rng.standard_normal((n, d)).astype(np.float32)[perm]))
+            B.sat_cache_commit(ctx)
+            B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, B.make_pred_params(*weights, h, version, B.SAT_CELL_LSTM), 0, out)
+        S = B.sat_predict_state(ctx, 1, n_slots, h)
+        B.sat_sync_status(ctx)
+        snaps = [B.sat_cache_read(ctx, 1, age, n_slots, d) for age in range(min(len(versions), tau) - 1, -1, -1)]
+    finally:
+        B.sat_destroy(ctx)
+    sel = np.unique(np.concatenate([np.arange(300), np.arange(n_slots - 300, n_slots), rng.integers(0, n_slots, 400)]))
+    s, c, ds, dc = (np.zeros((len(sel), h)) for _ in range(4))
+    sig = lambda v: 1 / (1 + np.exp(-v))
+    U64, eta = Uh.astype(np.float64), 2.0 ** -20
+    for x in snaps:
+        x = x[sel].astype(np.float64)
+        z = x @ W + s @ U64 + b
+        e = ((d + h + 2) * U + 2.0 ** -20) * (np.abs(x) @ np.abs(W) + np.abs(s) @ np.abs(U64) + np.abs(b)) + ds @ np.abs(U64)
+        (zi, zf, zg, zo), (ei, ef, eg, eo) = (np.split(v, 4, axis=1) for v in (z, e))
+        g = np.tanh(zg)
+        dc = np.abs(c) * (ef / 4 + eta) + dc + np.abs(g) * (ei / 4 + eta) + eg + eta
+        c = sig(zf) * c + sig(zi) * g
+        s = sig(zo) * np.tanh(c)
+        ds = eo / 4 + eta + dc + eta
+    assert (np.abs(S[sel] - s) <= ds).all()
