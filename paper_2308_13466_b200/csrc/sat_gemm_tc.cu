@@ -794,14 +794,15 @@ done:
 // h = 64, half of it the projection (83 us a step, and 54 for the first one).  Here a row tile stays on the SM for all steps: s as the
 // A operand in shared memory, c in registers, Uh resident; a step reads its projection and nothing else.
 //
-// A CTA pair (cta_group::2) works on two slots of 256 rows (128 per CTA) in turn, so that one slot's MMA runs under the other's
-// cell arithmetic: Uh takes 64 KB per CTA (half of the columns, both planes, h = 64), the two slots 64 KB each, and the accumulators
-// all of TMEM.  Eight warps per slot, two per lane quadrant with alternate quads of four units: one row per thread.  Projections are stored
-// [row tile of 128][unit][row] float4 (sat_proj_floats), so a warp reads 512 contiguous bytes and the next step's block of a tile is one
-// bulk prefetch into L2.  Bound by the hardware exponential and reciprocal (ten per unit and step: 2.7 us per 128 rows at h = 64) next to
-// the projection stream (3.0 us).
+// A CTA pair (cta_group::2) works on two slots of 256 rows (128 per CTA) so that one slot's product runs under the other's cell
+// arithmetic: Uh takes 64 KB per CTA (half of the columns, both planes, h = 64), the two slots 64 KB each, and the accumulators all of
+// TMEM.  Eight warps per slot, two per lane quadrant with alternate quads of four units: one row per thread; the slot's first warp also
+// issues its products.  Projections are stored [row tile of 128][unit][row] float4 (sat_proj_floats), so a warp reads 512 contiguous
+// bytes.  160000 rows, h = 64: 198 us for four steps, 692 MB of projections at 3.5 TB/s.  Bound by latency: sixteen warps of 128 registers are all that fit,
+// and each step of a slot is a chain of product, load, gates and store.  (Without the loads 151 us, without the products 163, without
+// exponentials and reciprocals 209 of 226.  An issuing warp of its own left 96 registers: 213; bulk prefetches into L2: +13.)
 // =====================================================================================
-#define SEQ_THREADS (17 * 32)
+#define SEQ_THREADS 512   /* 128 registers a thread */
 struct SeqSteps {
     const float *proj[SAT_SEQ_MAX];
 };
@@ -850,7 +851,7 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
         sh->dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 16) tc_alloc<2>(&sh->tmem_base, 512u);
+    if (warp == 0) tc_alloc<2>(&sh->tmem_base, 512u);
     tc_fence_before();
     __syncthreads();
     cluster_sync();
@@ -859,7 +860,7 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
     volatile int *dead = &sh->dead;
     sat_grid_wait();
 
-    if (warp == 16) {
+    if (warp == 0) {
         if (lane == 0) {
             mbar_expect_tx(&sh->b_full, (uint32_t)nkb * 2 * b_plane);
             for (int32_t kb = 0; kb < nkb; ++kb) {
@@ -869,36 +870,12 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
         }
         if (!mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
         mbar_arrive_warp<2>(&sh->b_ready, lane);
-        if (rank == 0) {
-            if (!mbar_wait_all(&sh->b_ready, 0, dead, status)) goto done;
-            const uint32_t idesc = make_idesc(2 * TC_BM, bn, 0, 0);
-            const uint64_t a0 = make_desc(smem_u32(smem), 16, 512, 4), b0 = make_desc(smem_u32(Bs), 16, 512, 4);
-            const int32_t products = n_steps - (first ? 1 : 0);   // per tile: the first step has no state yet
-            const int32_t count0 = (mine + 1) / 2 * products, count1 = mine / 2 * products;
-            for (int32_t i = 0; i < count0; ++i)
-                for (int sl = 0; sl < 2; ++sl) {
-                    if (sl == 1 && i >= count1) continue;
-                    if (!mbar_wait_all(&sh->a_ready[sl], (uint32_t)i & 1u, dead, status)) goto done;
-                    tc_fence_after();
-                    if (elect_one()) {
-                        const uint32_t acc = tmem + (uint32_t)sl * 256u;
-                        for (int32_t kb = 0; kb < nkb; ++kb) {
-#pragma unroll
-                            for (int ks = 0; ks < TC_BK / 8; ++ks) {
-                                const uint64_t a_hi = a0 + (uint64_t)(((uint32_t)sl * slot_bytes + (uint32_t)kb * 2 * a_plane) >> 4) + (uint64_t)(ks * 2);
-                                const uint64_t b_hi = b0 + (uint64_t)(((uint32_t)kb * 2 * b_plane) >> 4) + (uint64_t)(ks * 2);
-                                const uint64_t a_lo = a_hi + (a_plane >> 4), b_lo = b_hi + (b_plane >> 4);
-                                tc_mma<1, 2>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-                                tc_mma<2, 2>(acc, a_hi, b_lo, idesc, 1u);
-                                tc_mma<0, 2>(acc, a_lo, b_hi, idesc, 1u);
-                            }
-                        }
-                        tc_commit<2>(&sh->acc_full[sl]);
-                    }
-                }
-        }
-    } else {
+    }
+    {
         const int slot = warp >> 3, q = warp & 3, half = (warp >> 2) & 1;
+        const bool issuer = rank == 0 && (warp & 7) == 0;   // of its slot's products
+        const uint32_t idesc = make_idesc(2 * TC_BM, bn, 0, 0), acc = tmem + (uint32_t)slot * 256u;
+        const uint64_t a0 = make_desc(smem_u32(smem) + (uint32_t)slot * slot_bytes, 16, 512, 4), b0 = make_desc(smem_u32(Bs), 16, 512, 4);
         const int32_t nq = h >> 2;                       // quads of four units
         const int r_in = q * 32 + lane;                  // this thread's row of the tile
         uint8_t *A = smem + (uint32_t)slot * slot_bytes + r_in * 64;
@@ -908,6 +885,7 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
             *reinterpret_cast<float4 *>(d) = v;
             *reinterpret_cast<float4 *>(d + a_plane) = residual4(v);
         };
+        if (issuer && !mbar_wait_all(&sh->b_ready, 0, dead, status)) goto done;
         uint32_t ph = 0;
         for (int32_t k = slot; k < mine; k += 2) {
             const int64_t rt = (unit + (int64_t)k * units) * 2 + rank;   // row tile of 128
@@ -935,17 +913,34 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
                     mbar_arrive_warp<2>(&sh->a_ready[slot], lane);
                 }
                 const float4 *pr = reinterpret_cast<const float4 *>(steps.proj[t]) + rt * h * 128 + r_in;
-                if ((warp & 7) == 0 && lane == 0) {   // what this slot reads next, into L2
-                    const int64_t rn = last ? (unit + (int64_t)(k + 2) * units) * 2 + rank : rt;
-                    if (rn * TC_BM < rows && (!last || k + 2 < mine)) {
-                        const float *nx = steps.proj[last ? 0 : t + 1] + rn * h * 512;
-                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(nx), "r"((uint32_t)h * 2048u) : "memory");
-                    }
-                }
-                float4 nx[4];
+                // projections are fetched two quads ahead
+                float4 nx[2][4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) nx[u] = tile_ok && half < nq ? __ldg(pr + (4 * half + u) * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        nx[i][u] = tile_ok && half + 2 * i < nq ? __ldg(pr + (4 * (half + 2 * i) + u) * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const uint32_t mine_acc = acc + ((uint32_t)(q * 32) << 16);
                 if (product) {
+                    if (issuer) {
+                        if (!mbar_wait_all(&sh->a_ready[slot], ph, dead, status)) goto done;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            for (int32_t kb = 0; kb < nkb; ++kb) {
+#pragma unroll
+                                for (int ks = 0; ks < TC_BK / 8; ++ks) {
+                                    const uint64_t a_hi = a0 + (uint64_t)(((uint32_t)kb * 2 * a_plane) >> 4) + (uint64_t)(ks * 2);
+                                    const uint64_t b_hi = b0 + (uint64_t)(((uint32_t)kb * 2 * b_plane) >> 4) + (uint64_t)(ks * 2);
+                                    const uint64_t a_lo = a_hi + (a_plane >> 4), b_lo = b_hi + (b_plane >> 4);
+                                    tc_mma<1, 2>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                                    tc_mma<2, 2>(acc, a_hi, b_lo, idesc, 1u);
+                                    tc_mma<0, 2>(acc, a_lo, b_hi, idesc, 1u);
+                                }
+                            }
+                            tc_commit<2>(&sh->acc_full[slot]);
+                        }
+                        __syncwarp();
+                    }
                     if (!mbar_wait_all(&sh->acc_full[slot], ph, dead, status)) goto done;
                     ph ^= 1u;
                     tc_fence_after();
@@ -957,12 +952,12 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
                         float4 z[4];
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            z[u] = nx[u];
-                            if (tile_ok && qd + 2 < nq) nx[u] = __ldg(pr + (4 * (qd + 2) + u) * 128);
+                            z[u] = nx[i & 1][u];
+                            if (tile_ok && qd + 4 < nq) nx[i & 1][u] = __ldg(pr + (4 * (qd + 4) + u) * 128);
                         }
                         if (product) {
                             uint32_t r[16];
-                            tc_ld16(tmem + (uint32_t)slot * 256u + ((uint32_t)(q * 32) << 16) + 16u * (uint32_t)qd, r);
+                            tc_ld16(mine_acc + 16u * (uint32_t)qd, r);
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
                                 z[u].x += __uint_as_float(r[4 * u]);
@@ -994,7 +989,7 @@ done:
     tc_fence_before();
     __syncthreads();
     cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
-    if (warp == 16) {
+    if (warp == 0) {
         __syncwarp();
         tc_fence_after();
         tc_dealloc<2>(tmem, 512u);
