@@ -997,7 +997,8 @@ done:
 }
 
 // =====================================================================================
-// MN-major kernel (weight gradient): block (x, y, z) = tile (x, y) of A^T B over rows [z * rps, (z + 1) * rps); the blocks with x == 0
+// MN-major kernel (weight gradient): block (x, y, z) = tile (x, y) of A^T B over rows [z' * rps, (z' + 1) * rps) of segment z / seg_splits,
+// z' = z % seg_splits (several products of the same shape summed into one result: the steps of the predictor); the blocks with x == 0
 // also leave the column sums of their rows of B (the bias gradient) in part_cs [z x N] when it is given: the converters hold every
 // value of B in registers anyway, which saves a pass over it (34 us for 169 k x 256).
 //
@@ -1007,6 +1008,9 @@ done:
 // warps read 32 and write 64 KB and the MMAs read 144 KB: 1.1 us at 128 B per clock, as much as the tensor work (1.1 us).
 // =====================================================================================
 #define MN_STAGES_MAX 6
+struct MnMaps {   // operands of the segments: C = sum over segments of A^T B
+    CUtensorMap a[SAT_TN_SEGMENTS], b[SAT_TN_SEGMENTS];
+};
 #define MN_CONV_THREADS 256
 #define MN_THREADS (64 + MN_CONV_THREADS)
 #define MN_SMEM_MAX (227 * 1024)
@@ -1019,7 +1023,7 @@ struct MnShared {
 };
 
 __global__ void __launch_bounds__(MN_THREADS, 2)
-k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int32_t Mdim, int32_t N, int64_t rps, int64_t rows,
+k_gemm_tc_mn(const __grid_constant__ MnMaps maps, int32_t seg_splits, int32_t Mdim, int32_t N, int64_t rps, int64_t rows,
              int32_t mt_max, int32_t bn, int32_t stages, uint32_t tmem_cols, float *part_C, float *part_cs, int *status)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -1034,7 +1038,8 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t m0 = blockIdx.x * (mt_max * TC_BM), n0 = blockIdx.y * bn;
     const int32_t mt = (Mdim - m0 + TC_BM - 1) / TC_BM < mt_max ? (Mdim - m0 + TC_BM - 1) / TC_BM : mt_max;   // 128-column sub-tiles in use
-    const int64_t r0 = (int64_t)blockIdx.z * rps, r1 = r0 + rps < rows ? r0 + rps : rows;
+    const int32_t seg = (int32_t)blockIdx.z / seg_splits;
+    const int64_t r0 = (int64_t)((int32_t)blockIdx.z - seg * seg_splits) * rps, r1 = r0 + rps < rows ? r0 + rps : rows;
     const int32_t nkb = (int32_t)((r1 - r0 + TC_BK - 1) / TC_BK);
 
     if (threadIdx.x == 0) {
@@ -1066,8 +1071,8 @@ k_gemm_tc_mn(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
                 uint8_t *st = smem + (size_t)s * stage_bytes;
                 const int32_t r = (int32_t)(r0 + (int64_t)kb * TC_BK);
                 mbar_expect_tx(&sh->full[s], (uint32_t)mt * sub_bytes + b_bytes);
-                for (int bl = 0; bl < mt * (TC_BM / 32); ++bl) tma_load_2d(st + bl * blk_bytes, &mapA, &sh->full[s], m0 + bl * 32, r);
-                for (int bl = 0; bl < n_blks_b; ++bl) tma_load_2d(st + 2 * a_bytes + bl * blk_bytes, &mapB, &sh->full[s], n0 + bl * 32, r);
+                for (int bl = 0; bl < mt * (TC_BM / 32); ++bl) tma_load_2d(st + bl * blk_bytes, &maps.a[seg], &sh->full[s], m0 + bl * 32, r);
+                for (int bl = 0; bl < n_blks_b; ++bl) tma_load_2d(st + 2 * a_bytes + bl * blk_bytes, &maps.b[seg], &sh->full[s], n0 + bl * 32, r);
             }
         }
     } else if (warp == 1) {
@@ -1569,12 +1574,13 @@ sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &
     return SAT_OK;
 }
 
-// C[m x n] (+)= A^T B over `rows` rows: A fp32 [rows x m] (lda), B fp32 [rows x n] (ldb)
-sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb, float *C,
-                          int32_t ldc, int accumulate, float *colsum)
+// C[m x n] (+)= sum_i A[i]^T B[i] over `rows` rows each: A fp32 [rows x m] (lda), B fp32 [rows x n] (ldb)
+sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *const *A, int32_t lda, const float *const *B, int32_t ldb,
+                          int32_t segments, float *C, int32_t ldc, int accumulate, float *colsum)
 {
     if (m == 0 || n == 0) return SAT_OK;
-    ProfScope prof(ctx, SATK_GEMM_TN, 4.0 * ((double)rows * (m + n) + (double)m * n), 2.0 * (double)rows * m * n);
+    if (segments < 1 || segments > SAT_TN_SEGMENTS) return sat_fail(ctx, SAT_EINVAL, "sat_gemm_tc_tn: 1 to %d segments", SAT_TN_SEGMENTS);
+    ProfScope prof(ctx, SATK_GEMM_TN, 4.0 * ((double)rows * segments * (m + n) + (double)m * n), 2.0 * (double)rows * segments * m * n);
     const int32_t bn = tile_n_for(n), mt = m > TC_BM ? 2 : 1;
     const uint32_t stage_bytes = 2 * (uint32_t)mt * (TC_BM / 32) * TC_BK * 128 + 2 * (uint32_t)((bn + 31) / 32) * TC_BK * 128;
     const int64_t r1 = rows > 0 ? rows : 1, kblocks = cdiv64(r1, TC_BK);
@@ -1583,7 +1589,7 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
     // again, cost about as much as that.
     const int per_sm = mt == 1 ? 2 : 1;
     const int64_t tiles = cdiv64(m, mt * TC_BM) * cdiv64(n, bn);
-    int64_t splits = tiles < 148 * per_sm ? 148 * per_sm / tiles : 1;
+    int64_t splits = tiles * segments < 148 * per_sm ? 148 * per_sm / (tiles * segments) : 1;   // of a segment
     if (splits > cdiv64(kblocks, 6)) splits = cdiv64(kblocks, 6);
     const int64_t kpb = cdiv64(kblocks, splits), rps = kpb * TC_BK;
     splits = cdiv64(r1, rps);
@@ -1592,19 +1598,28 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
     if (stages > kpb) stages = kpb;
     const size_t need = (size_t)stages * stage_bytes, turn = MN_TURN_BYTES;
     const size_t smem = (need > turn ? need : turn) + sizeof(MnShared) + 1024;
-    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)splits * ((size_t)m * n + n) * sizeof(float)));
+    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)(splits * segments) * ((size_t)m * n + n) * sizeof(float)));
     float *part = (float *)ctx->buf_splitk.p;
-    float *part_cs = colsum ? part + (size_t)splits * m * n : nullptr;
-    CUtensorMap mA, mB;
-    SAT_TRY(make_map(ctx, &mA, A, m, rows, lda, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
-    SAT_TRY(make_map(ctx, &mB, B, n, rows, ldb, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
+    float *part_cs = colsum ? part + (size_t)(splits * segments) * m * n : nullptr;
+    MnMaps maps;
+    for (int32_t i = 0; i < segments; ++i) {
+        SAT_TRY(make_map(ctx, &maps.a[i], A[i], m, rows, lda, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
+        SAT_TRY(make_map(ctx, &maps.b[i], B[i], n, rows, ldb, 32, TC_BK, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B));
+    }
+    for (int32_t i = segments; i < SAT_TN_SEGMENTS; ++i) maps.a[i] = maps.a[0], maps.b[i] = maps.b[0];
     if (g_attr_mn.need(ctx->device)) {
         SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_mn, cudaFuncAttributeMaxDynamicSharedMemorySize, MN_SMEM_MAX));
         g_attr_mn.mark(ctx->device);
     }
-    dim3 grid((unsigned)cdiv64(m, mt * TC_BM), (unsigned)cdiv64(n, bn), (unsigned)splits);
-    sat_pdl(ctx->stream, k_gemm_tc_mn, grid, MN_THREADS, smem)(mA, mB, m, n, rps, r1, mt, bn, (int32_t)stages, mt == 1 ? 256u : 512u, part, part_cs,
+    dim3 grid((unsigned)cdiv64(m, mt * TC_BM), (unsigned)cdiv64(n, bn), (unsigned)(splits * segments));
+    sat_pdl(ctx->stream, k_gemm_tc_mn, grid, MN_THREADS, smem)(maps, (int32_t)splits, m, n, rps, r1, mt, bn, (int32_t)stages, mt == 1 ? 256u : 512u, part, part_cs,
                                                        ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
-    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)splits, accumulate, C, n, ldc, part_cs, n, colsum);
+    return sat_splitk_reduce(ctx, part, (int64_t)m * n, (int32_t)(splits * segments), accumulate, C, n, ldc, part_cs, n, colsum);
+}
+
+sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb, float *C,
+                          int32_t ldc, int accumulate, float *colsum)
+{
+    return sat_gemm_tc_tn(ctx, rows, m, n, &A, lda, &B, ldb, 1, C, ldc, accumulate, colsum);
 }

@@ -58,7 +58,7 @@ k_pt_cell_fwd(float *__restrict__ z, int64_t rows, int32_t h, const float *__res
 // to the gate pre-activations; dc carries the gradient of the cell state from the later steps (null at the last step) and
 // leaves as the gradient with respect to the previous cell state.  The column sums of the written gradients (the bias
 // gradient of the step) are accumulated on the way: per thread over its rows, then over the row groups of the block in
-// fixed order into colsum_part [gridDim.x x 4h].
+// fixed order into colsum_part [gridDim.x x 4h] (null: the weight gradient takes them along).
 __global__ void __launch_bounds__(256)
 k_pt_cell_bwd(float *__restrict__ gz, int64_t rows, int32_t h, const float *__restrict__ c_prev, const float *__restrict__ c_cur,
               const float *__restrict__ dh, const float *dc_in, float *dc_out, float *__restrict__ colsum_part)
@@ -97,12 +97,15 @@ k_pt_cell_bwd(float *__restrict__ gz, int64_t rows, int32_t h, const float *__re
             PT_MAP4(sg, el(sg, e) + el(dg, e));
             PT_MAP4(so, el(so, e) + el(dd, e));
         }
-        float *mine = red + (size_t)rr * 4 * h + 4 * q;
-        st4s(mine, si);
-        st4s(mine + h, sf);
-        st4s(mine + 2 * h, sg);
-        st4s(mine + 3 * h, so);
+        if (colsum_part) {
+            float *mine = red + (size_t)rr * 4 * h + 4 * q;
+            st4s(mine, si);
+            st4s(mine + h, sf);
+            st4s(mine + 2 * h, sg);
+            st4s(mine + 3 * h, so);
+        }
     }
+    if (!colsum_part) return;
     __syncthreads();
     for (int c = threadIdx.x; c < 4 * h; c += 256) {
         float s = 0.f;
@@ -374,23 +377,39 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
         SAT_TRY(sat_scatter(ctx, ctx->push_row, ctx->push_slot, R, h, g_rows, h, dh, h));
         SAT_TRY(sat_sum_by_slot(ctx, h, g_a, h, 1, 1, dh, h));
         // ---- back-propagation through time ----
+        // The parameter gradients are sums over the steps of products of one shape (every step keeps its gate gradients): on the tensor
+        // cores all steps are one launch and one reduction each for Wx (with the bias) and Uh (a launch costs 27 us besides the product; 84671 nodes, four
+        // steps: 18 launches of the epoch, 957 + 236 us).
+        const bool merged = sat_use_tc(4 * h, d) && sat_use_tc(4 * h, h) && 4 * h > 64 && R >= 256;
+        if (!merged) SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)bwd_grid * 4 * h * sizeof(float)));
         for (int32_t t = k - 1; t >= 0; --t) {
             const float *x = ring_buf(ctx, c, ring_index(ctx, k - 1 - t));
             float *z = gates + t * plane_g;
             {
                 ProfScope prof(ctx, SATK_PRED_TRAIN, 4.0 * (double)plane_s * 13.0, 0.0);
-                SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)bwd_grid * 4 * h * sizeof(float)));
                 sat_pdl(ctx->stream, k_pt_cell_bwd, bwd_grid, 256, cell_smem)(z, R, h, t ? cs + (t - 1) * plane_s : nullptr, cs + t * plane_s, dh,
-                                                                          t == k - 1 ? nullptr : dc, dc, (float *)ctx->buf_colsum.p);
+                                                                          t == k - 1 ? nullptr : dc, dc,
+                                                                          merged ? nullptr : (float *)ctx->buf_colsum.p);
                 SAT_LAUNCHED(ctx);
             }
             const int acc = t != k - 1;
-            SAT_TRY(sat_splitk_reduce(ctx, (const float *)ctx->buf_colsum.p, 4 * h, (int32_t)bwd_grid, acc, g_b, 4 * h, 4 * h));
-            SAT_TRY(pt_tn(ctx, R, d, 4 * h, x, c->ld, z, 4 * h, g_Wx, nullptr, acc));
+            if (!merged) SAT_TRY(sat_splitk_reduce(ctx, (const float *)ctx->buf_colsum.p, 4 * h, (int32_t)bwd_grid, acc, g_b, 4 * h, 4 * h));
+            if (!merged) SAT_TRY(pt_tn(ctx, R, d, 4 * h, x, c->ld, z, 4 * h, g_Wx, nullptr, acc));
             if (t > 0) {
-                SAT_TRY(pt_tn(ctx, R, h, 4 * h, hs + (t - 1) * plane_s, h, z, 4 * h, g_Uh, nullptr, acc));
+                if (!merged) SAT_TRY(pt_tn(ctx, R, h, 4 * h, hs + (t - 1) * plane_s, h, z, 4 * h, g_Uh, nullptr, acc));
                 SAT_TRY(pt_nt(ctx, R, h, 4 * h, z, 4 * h, params->Uh, dh, h));
             }
+        }
+        for (int32_t t0 = 0; merged && t0 < k; t0 += SAT_TN_SEGMENTS) {
+            const float *xs[SAT_TN_SEGMENTS], *ss[SAT_TN_SEGMENTS], *zs[SAT_TN_SEGMENTS];
+            const int32_t cnt = k - t0 < SAT_TN_SEGMENTS ? k - t0 : SAT_TN_SEGMENTS, skip = t0 == 0 ? 1 : 0;   // no state before the first step
+            for (int32_t i = 0; i < cnt; ++i) {
+                xs[i] = ring_buf(ctx, c, ring_index(ctx, k - 1 - t0 - i));
+                ss[i] = t0 + i > 0 ? hs + (t0 + i - 1) * plane_s : nullptr;
+                zs[i] = gates + (t0 + i) * plane_g;
+            }
+            SAT_TRY(sat_gemm_tc_tn(ctx, R, d, 4 * h, xs, c->ld, zs, 4 * h, cnt, g_Wx, 4 * h, t0 > 0, g_b));
+            if (cnt > skip) SAT_TRY(sat_gemm_tc_tn(ctx, R, h, 4 * h, ss + skip, h, zs + skip, 4 * h, cnt - skip, g_Uh, 4 * h, t0 > 0));
         }
     }
     if (loss_host) {

@@ -317,3 +317,9 @@ def test_lstm_state_over_cached_projections(B, n, h, d, versions):
         s = sig(zo) * np.tanh(c)
         ds = eo / 4 + eta + dc + eta
     assert (np.abs(S[sel] - s) <= ds).all()
+
+
+@pytest.mark.parametrize("tau,h", [(7, 20), (8, 32), (10, 24)])     # steps summed by one launch: up to eight, the rest by a second one
+def test_predictor_gradient_over_long_windows(B, tau, h):
+    from tests.test_gpu_pred_train import test_gradient_for_every_fill_level as check
+    check(B, "medium", 16, {"tau": tau, "h": h})
