@@ -318,6 +318,8 @@ sat_status sat_cache_commit(sat_ctx *ctx);
  *     z_u = h_u W ;  e_vu = LeakyReLU_0.2(a_dst . z_v + a_src . z_u) ;  alpha_vu = softmax_u(e_vu) ;
  *     h_out_v = act( sum_u alpha_vu z_u + bias ).
  * The GCN normalisation is not used.  W [d_in x d_out], a_src [d_out], a_dst [d_out], bias [d_out] or NULL: DEVICE, dense.
+ * act may carry SAT_FWD_PUSH: the rows of boundary nodes also go to the write buffer of cached layer `layer`, as sat_cache_update
+ * with h_out would do (SAT_ESTATE without such a layer, SAT_EINVAL if its width is not d_out).
  * sat_gat_fwd keeps z, the attention scores and the log-sum-exp of every row for sat_gat_bwd (memory: (n + sum_m b_m) *
  * d_out floats per layer, owned by the context).  d_out <= 1024.
  * sat_gat_bwd: g_out [n_m x ld_g] gradient w.r.t. h_out; h_out as written by sat_gat_fwd (used for the ReLU mask; may be

@@ -169,7 +169,7 @@ __device__ __forceinline__ double gat_scaled(float x)
     return __hiloint2double((b >> 3) & (int)0x8FFFFFFFu, b << 29);
 }
 template <int G, int NV>
-__global__ void __launch_bounds__(256, NV <= 2 ? 3 : NV <= 4 ? 2 : 1)
+__global__ void __launch_bounds__(256, NV <= 2 ? 4 : NV <= 4 ? 2 : 1)
 k_gat_dots(const int4 *__restrict__ items, int32_t n_items, const int32_t *__restrict__ lenc, int32_t n, int32_t d4, const float *__restrict__ z_in,
            const float *__restrict__ z_halo, uint32_t ldz4, const float *__restrict__ D, double *__restrict__ dots)
 {
@@ -530,11 +530,19 @@ extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int
                                   const float *bias, int act, float *h_out, int32_t ld_out)
 {
     CHECK_CTX(ctx);
+    const bool push = act & SAT_FWD_PUSH;
+    act &= ~SAT_FWD_PUSH;
     PartView v;
     SAT_TRY(sat_part_view(ctx, part, &v));
     if (layer < 1 || layer > SAT_MAX_LAYERS) return sat_fail(ctx, SAT_EINVAL, "sat_gat_fwd: layer must be in [1, %d]", SAT_MAX_LAYERS);
     if (d_in <= 0 || d_out <= 0 || d_out > 128 * GAT_MAX_NV || !W || !a_src || !a_dst) return sat_fail(ctx, SAT_EINVAL, "sat_gat_fwd: bad widths or null parameters");
     if (act != SAT_ACT_NONE && act != SAT_ACT_RELU) return sat_fail(ctx, SAT_EINVAL, "sat_gat_fwd: unknown activation");
+    CacheLayer *pc = nullptr;
+    if (push) {
+        if (!ctx->cache_ok || layer > ctx->n_cached) return sat_fail(ctx, SAT_ESTATE, "sat_gat_fwd: SAT_FWD_PUSH without a cached layer %d", layer);
+        pc = &ctx->cache[layer - 1];
+        if (pc->width != d_out) return sat_fail(ctx, SAT_EINVAL, "sat_gat_fwd: SAT_FWD_PUSH of %d columns into a cached layer of %d", d_out, pc->width);
+    }
     if (v.n_rows > 0 && (!h_in || !h_out || !ok_ld(ld_in, d_in) || !ok_ld(ld_out, d_out) || !aligned16(h_in) || !aligned16(h_out)))
         return sat_fail(ctx, SAT_EINVAL, "sat_gat_fwd: null / misaligned h_in / h_out or bad leading dimension");
     if (v.n_halo > 0 && (!h_halo || !ok_ld(ld_halo, d_in) || !aligned16(h_halo))) return sat_fail(ctx, SAT_EINVAL, "sat_gat_fwd: null / misaligned h_halo");
@@ -578,6 +586,12 @@ extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int
         SpmmEpilogue ep;
         ep.bias = bias;
         ep.relu = G.relu;
+        if (push && ctx->n_slots > 0) {   // boundary rows go to the ring from the product's epilogue (a pass of its own: 66 us of 169343 x 256)
+            SAT_TRY(sat_row_slots(ctx, &ep.push_slot));
+            ep.push = ring_buf(ctx, pc, ctx->write_idx);
+            ep.ld_push = pc->ld;
+            if (!pc->proj_tag.empty()) pc->proj_tag[ctx->write_idx] = 0;   // the buffer changes: its cached input projection is stale
+        }
         SAT_TRY(sat_spmm_entries(ctx, v, 0, d_out, (const int2 *)G.ent.p, z_in, ld_z, z_halo, ld_z, h_out - (int64_t)v.row0 * ld_out, ld_out, ep));
     }
     for (int m = (part == SAT_ALL_PARTS ? 0 : part); m < (part == SAT_ALL_PARTS ? ctx->M : part + 1); ++m) G.valid[m] = 1;

@@ -346,7 +346,12 @@ struct SpmmEpilogue {
     int relu = 0;
     const float *s1 = nullptr, *v1 = nullptr, *s2 = nullptr, *v2 = nullptr;   // + s1[row] v1[col] + s2[row] v2[col]
     int32_t d = 0;
+    float *push = nullptr;               // row i goes to row push_slot[i] of this matrix as well where that is >= 0
+    const int32_t *push_slot = nullptr;  // [rows]
+    int64_t ld_push = 0;
 };
+// cache slot of every row in partition-major order (-1: not a boundary node); made when first asked for
+sat_status sat_row_slots(sat_ctx *ctx, const int32_t **out);
 sat_status sat_spmm_entries(sat_ctx *ctx, const PartView &v, int mode, int32_t d, const int2 *ent, const float *in_base, int32_t ld_in,
                             const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const SpmmEpilogue &ep);
 // the work items such a product walks at width d

@@ -673,6 +673,17 @@ __global__ void k_row_slot(const int32_t *__restrict__ perm, const int32_t *__re
     if (r < n) row_slot[r] = slot[perm[r]];
 }
 
+sat_status sat_row_slots(sat_ctx *ctx, const int32_t **out)
+{
+    if (!ctx->row_slot) {
+        SAT_TRY(dev_realloc(ctx, &ctx->row_slot, (int64_t)ctx->n));
+        k_row_slot<<<(unsigned)cdiv64(ctx->n, 256), 256, 0, ctx->stream>>>(ctx->perm, ctx->slot, ctx->n, ctx->row_slot);
+        SAT_LAUNCHED(ctx);
+    }
+    *out = ctx->row_slot;
+    return SAT_OK;
+}
+
 extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int32_t d_in, int32_t d_out, const float *h_in,
                                     int32_t ld_in, const float *h_halo, int32_t ld_halo, const float *W, const float *bias, int act,
                                     float *h_out, int32_t ld_out)
@@ -740,13 +751,9 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
         eh.mask_out = mask_out;
         eh.mask_words = words;
         if (push && ctx->n_slots > 0) {   // the boundary rows go to the ring's write buffer from the epilogue
-            if (!ctx->row_slot) {
-                SAT_TRY(dev_realloc(ctx, &ctx->row_slot, (int64_t)ctx->n));
-                k_row_slot<<<(unsigned)cdiv64(ctx->n, 256), 256, 0, ctx->stream>>>(ctx->perm, ctx->slot, ctx->n, ctx->row_slot);
-                SAT_LAUNCHED(ctx);
-            }
+            SAT_TRY(sat_row_slots(ctx, &eh.push_slot));
+            eh.push_slot += v.row0;
             eh.push_dst = ring_buf(ctx, pc, ctx->write_idx);
-            eh.push_slot = ctx->row_slot + v.row0;
             eh.ld_push = pc->ld;
             if (!pc->proj_tag.empty()) pc->proj_tag[ctx->write_idx] = 0;
         }

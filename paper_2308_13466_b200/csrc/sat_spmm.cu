@@ -471,7 +471,12 @@ __device__ __forceinline__ float4 spmm_epilogue(const SpmmEpilogue &ep, int64_t 
         if (ep.s2) x[k] += s2 * __ldg(ep.v2 + col);
         if (ep.relu) x[k] = fmaxf(x[k], 0.f);
     }
-    return make_float4(x[0], x[1], x[2], x[3]);
+    const float4 out = make_float4(x[0], x[1], x[2], x[3]);
+    if (ep.push) {
+        const int32_t slot = __ldg(ep.push_slot + row);
+        if (slot >= 0) *reinterpret_cast<float4 *>(ep.push + slot * ep.ld_push + 4 * c) = out;
+    }
+    return out;
 }
 
 // K entries: their columns and weights, their rows (all in flight together), the sums

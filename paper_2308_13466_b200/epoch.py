@@ -187,9 +187,7 @@ class SatEpoch:
             else:
                 B.sat_predict(ctx, l - 1, m, pred[l - 2] if pred is not None else None, 0, hv)
             p = params[l - 1]
-            B.sat_gat_fwd(ctx, m, l, h_in, hv, p["W"], p["a_src"], p["a_dst"], p["b"], B.SAT_ACT_RELU if l < L else B.SAT_ACT_NONE, self.H[l])
-            if l < L:
-                B.sat_cache_update(ctx, m, l, self.H[l])
+            B.sat_gat_fwd(ctx, m, l, h_in, hv, p["W"], p["a_src"], p["a_dst"], p["b"], B.SAT_ACT_RELU | B.SAT_FWD_PUSH if l < L else B.SAT_ACT_NONE, self.H[l])
             ins.append(h_in)
             h_in = self.H[l]
         kind = B.SAT_LOSS_SOFTMAX_CE if self.loss == "ce" else B.SAT_LOSS_SIGMOID_BCE

@@ -323,3 +323,40 @@ def test_lstm_state_over_cached_projections(B, n, h, d, versions):
 def test_predictor_gradient_over_long_windows(B, tau, h):
     from tests.test_gpu_pred_train import test_gradient_for_every_fill_level as check
     check(B, "medium", 16, {"tau": tau, "h": h})
+
+
+@pytest.mark.parametrize("parts", [False, True])
+@pytest.mark.parametrize("d_out", [40, 43, 256, 300])                 # one launch per slice of 256 columns; rows of many runs by k_spmm_fixup or their last run
+def test_attention_layer_pushes_its_boundary_rows(B, d_out, parts):
+    """SAT_FWD_PUSH of sat_gat_fwd against sat_cache_update: same bits in the ring and in h_out."""
+    n, M, d = 3000, 3, 24
+    A = _graph(HUBS, n)
+    rng = np.random.default_rng(d_out)
+    part = rng.integers(0, M, n).astype(np.int32)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        B.sat_cache_init(ctx, [d_out], 2)
+        sizes = [B.sat_part_sizes(ctx, m) for m in range(M)]
+        n_slots = B.sat_slot_map(ctx, n)[2]
+        H, halo = dev2d(rng.standard_normal((n, d)).astype(np.float32)), dev2d(rng.standard_normal((sum(s[1] for s in sizes), d)).astype(np.float32))
+        W, a1, a2, b = (dev(rng.standard_normal(s).astype(np.float32)) for s in ((d, d_out), (d_out,), (d_out,), (d_out,)))
+        got = []
+        for push in (0, B.SAT_FWD_PUSH):
+            out = empty2d(n, d_out)
+            r0 = u0 = 0
+            for m in range(M) if parts else [B.SAT_ALL_PARTS]:
+                r1, u1 = (r0 + sizes[m][0], u0 + sizes[m][1]) if parts else (n, len(halo))
+                B.sat_gat_fwd(ctx, m, 1, H[r0:r1], halo[u0:u1], W, a1, a2, b, B.SAT_ACT_RELU | push, out[r0:r1])
+                if not push:
+                    B.sat_cache_update(ctx, m, 1, out[r0:r1])
+                r0, u0 = r1, u1
+            B.sat_cache_commit(ctx)
+            got.append((out.cpu().numpy()[:, :d_out], B.sat_cache_read(ctx, 1, 0, n_slots, d_out)))
+        assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+        with pytest.raises(B.SatError):                       # layer 2 is not cached
+            B.sat_gat_fwd(ctx, B.SAT_ALL_PARTS, 2, H, halo, W, a1, a2, b, B.SAT_ACT_RELU | B.SAT_FWD_PUSH, empty2d(n, d_out))
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
