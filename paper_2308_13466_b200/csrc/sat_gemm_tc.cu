@@ -8,7 +8,7 @@
 // K-major operand layout.
 //
 //   k_gemm_tc_k   C[M x N] = A[M x K] B[N x K]^T   both operands K-major, 64-byte swizzle, BLOCK_K = 16, persistent CTA pairs
-//                 (layer transform, LSTM gates with two A operands or a cached projection, predictor output, input gradient)
+//                 (layer transform, recurrent gates with two A operands, input projections, predictor output, input gradient)
 //   k_gemm_tc_mn  C[M x N] = A[R x M]^T B[R x N]   both operands MN-major, 128-byte swizzle with 32-byte atoms, split over R
 //                 (weight gradient)
 // Warp roles of k_gemm_tc_k (512 threads): warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, then 6 converter and
@@ -314,8 +314,8 @@ struct TcShared {
 };
 
 /* 512 threads, 128 registers each: warp 0 TMA, warp 1 MMA, then the converter warps, then the epilogue warps.  The split
- * between converters and epilogue depends on the epilogue variant (TckCfg): the K = h variants with a side operand have
- * four k-blocks per tile and an epilogue bound by instruction issue, so they run 2 + 12 instead of 6 + 8.
+ * between converters and epilogue depends on the epilogue variant (TckCfg): the one with a gathered residual has four
+ * k-blocks per tile (K = h) and an epilogue bound by latency, so it runs 2 + 12 instead of 6 + 8.
  * The converter warps work in two groups on alternate k-blocks, so two stages are being split at any time.  The stage
  * count is even, hence a stage is always handled by the same group and each group meets the phases of its stages in
  * order (a parity wait must never be more than one phase ahead of its barrier). */
@@ -326,10 +326,10 @@ struct TcShared {
  * K = 256 transform 132 -> 118 us, K = 64 LSTM step 98 -> 85 us) for 16 KB more L2 -> SM traffic per k-block. */
 #define TCK_B_PRESPLIT 1
 
-// Epilogue variants.  The ones with a per-row side operand streamed from global memory (gathered residual rows, cached
-// LSTM input projection) keep a ring of 32 x 32 side tiles per epilogue warp in shared memory, filled by cp.async ahead of
-// the consumer: one chunk in flight per warp left the loads latency-bound at ~2 TB/s.  Those variants contract over a
-// small K (the predictor width), so they give up main-loop stages for the ring.
+// Epilogue variants.  EPI_RESID streams a per-row side operand from global memory (gathered residual rows): a ring of 32 x 32 side tiles
+// per epilogue warp in shared memory, filled by cp.async ahead of the consumer.  It contracts over a small K (the predictor width), so
+// it gives up main-loop stages for the ring.  (Four slots with the results staged in place, which fits with eight epilogue
+// warps: 1018 -> 1232 us at 612257 nodes; the twelve warps are worth more than the deeper ring.)
 enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_LSTM = 2, EPI_PROJ = 3, EPI_PUSH = 4, EPI_GRU = 5 };   // EPI_PUSH = EPI_PLAIN + a second copy of the rows that have a cache slot
 template <int EPI> struct TckCfg { static constexpr int ring = 0, conv_warps = 6, epi_warps = 8, out_bytes = epi_warps * 4096; };
 template <> struct TckCfg<EPI_RESID> { static constexpr int ring = 1, conv_warps = 2, epi_warps = 12, out_bytes = epi_warps * 4096; };
