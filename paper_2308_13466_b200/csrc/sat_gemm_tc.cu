@@ -1305,14 +1305,16 @@ __global__ void k_pack_bias(const float *__restrict__ bias, int32_t n, int32_t n
 //   transpose = 1: W is [K x N] row-major (ldw) -> B[n][k] = W[k][n]          (C = A W)
 //   transpose = 0: W is [N x K] row-major (ldw) -> B[n][k] = W[n][k]          (C = A W^T)
 // A second source W2 (same orientation, k2 rows) continues along K at column offset k1_pad.
+// A bias [n] is packed alike, zero padded (four gates with gates = 3 too).
 // gate_h > 0: packed column 4 j + g is gate g of hidden unit j.  gates = 4: the sources have the columns i | f | g | o.  gates = 3 (GRU,
 // sources r | z | n): the candidate's two parts stay apart, column 4 j + 2 takes n of the first source only and 4 j + 3 n of the second.
 __global__ void k_split_weights(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t k1_pad, const float *__restrict__ W2,
                                 int64_t ldw2, int32_t k2, int32_t n, int32_t n_pad, int32_t k_pad, int transpose, int32_t gate_h, int gates,
-                                float *__restrict__ hi, float *__restrict__ lo)
+                                float *__restrict__ hi, float *__restrict__ lo, const float *__restrict__ bias, float *__restrict__ bias_out)
 {
     sat_grid_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (bias && i < n_pad) bias_out[i] = i < n ? bias[gate_h > 0 ? ((int32_t)i & 3) * gate_h + ((int32_t)i >> 2) : (int32_t)i] : 0.f;
     if (i >= (int64_t)n_pad * k_pad) return;
     const int32_t np = (int32_t)(i / k_pad), kk = (int32_t)(i - (int64_t)np * k_pad);
     const int32_t g = np & 3;
@@ -1401,7 +1403,7 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
 }
 
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
-                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h, int gates)
+                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h, int gates, const float *bias)
 {
     const int32_t k1_pad = W2 ? (k1 + TC_BK - 1) / TC_BK * TC_BK : k1;
     const int32_t k_tot = k1_pad + (W2 ? k2 : 0);
@@ -1409,13 +1411,14 @@ sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1,
     const int32_t bn = tile_n_for(n);
     const int32_t n_pad = (n + bn - 1) / bn * bn;
     const size_t plane = ((size_t)n_pad * k_pad * sizeof(float) + 255) & ~(size_t)255;
-    SAT_TRY(sat_ensure(ctx, buf, 2 * plane));
+    SAT_TRY(sat_ensure(ctx, buf, 2 * plane + (bias ? (size_t)n_pad * sizeof(float) : 0)));
     out->hi = (float *)buf.p;
     out->lo = (float *)((char *)buf.p + plane);
     out->ld = k_pad;
     out->n_pad = n_pad;
+    out->bias = bias ? (float *)((char *)buf.p + 2 * plane) : nullptr;
     sat_pdl(ctx->stream, k_split_weights, (unsigned)cdiv64((int64_t)n_pad * k_pad, 256), 256, 0)(W, ldw, k1, k1_pad, W2, ldw2, k2, n, n_pad, k_pad,
-                                                                                          transpose, gate_h, gates, out->hi, out->lo);
+                                                                                          transpose, gate_h, gates, out->hi, out->lo, bias, out->bias);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }
@@ -1432,6 +1435,7 @@ sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeig
     out->lo = (float *)((char *)buf.p + plane);
     out->ld = k_pad;
     out->n_pad = n_pad;
+    out->bias = nullptr;
     return SAT_OK;
 }
 
@@ -1502,7 +1506,9 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.C = eh.C;
     ep.ldc = eh.ldc;
     ep.bias = nullptr;
-    if (eh.bias) {  // zero-padded copy so that the epilogue can read whole 128-bit vectors
+    if (eh.bias && Bw.bias) {
+        ep.bias = Bw.bias;   // packed with the weights
+    } else if (eh.bias) {  // zero-padded copy so that the epilogue can read whole 128-bit vectors
         const size_t padded = (size_t)cdiv64(n, bn) * bn;
         DevBuf &home = eh.bias_home ? *eh.bias_home : ctx->buf_bias;
         if (!(eh.bias_home && eh.bias_ready && home.bytes >= padded * sizeof(float))) {

@@ -499,6 +499,7 @@ __device__ __forceinline__ float tanh_fast(float x) { return fmaf(-2.f, rcp_fast
 
 struct TcWeights {         // weight operand as two fp32 planes [n_pad x ld] holding the TF32 hi / lo terms, K-major
     float *hi = nullptr, *lo = nullptr;
+    float *bias = nullptr;  // [n_pad], where one was packed with them
     int32_t ld = 0, n_pad = 0;
 };
 struct TcEpilogueHost {
@@ -542,7 +543,7 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
 // gate_h > 0: the n = 4 gate_h columns (gate blocks i | f | g | o) are interleaved so that packed column 4 j + gate is gate `gate`
 // of hidden unit j (what the fused LSTM epilogue expects); gates = 3: the GRU's, see k_split_weights
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
-                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0, int gates = 4);
+                          int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0, int gates = 4, const float *bias = nullptr);
 sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out);
 // Plane of an input projection x Wx + b of the LSTM, [row tile of 128][unit][row of the tile][i f g o]
 inline int64_t sat_proj_floats(int64_t rows, int32_t h) { return (rows + 127) / 128 * 512 * h; }

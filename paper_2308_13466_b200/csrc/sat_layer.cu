@@ -352,7 +352,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
             eh.lstm_first = 1;
             SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, x, c->ld, d, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
         } else {
-            if (!have_wxu) SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, p->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit3, &Wxu, h));
+            if (!have_wxu) SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, p->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit3, &Wxu, h, 4, p->b));
             have_wxu = true;
             SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, x, c->ld, d, c->S, h, h, Wxu, eh, SATK_GEMM_NN));
         }
@@ -412,8 +412,8 @@ static sat_status run_gru(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p)
     }
     if (sat_use_tc(4 * h, d) && 4 * h <= 256) {
         TcWeights W1, W2;   // first step: x alone
-        SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, h, 3));
-        if (k > 1) SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, p->Uh, 3 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, h, 3));
+        SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, h, 3, p->b));
+        if (k > 1) SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, p->Uh, 3 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, h, 3, p->b));
         for (int32_t t = 0; t < k; ++t) {
             TcEpilogueHost eh;
             eh.C = c->S;
@@ -498,8 +498,8 @@ static sat_status run_lstm(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p
     if (fused && p->version != 0 && sat_use_tc(4 * h, h)) return run_lstm_cached(ctx, c, p, k, cell);
     TcWeights W1, W2;   // packed weights for the first step (x only) and the later steps ([x | s])
     if (tc) {
-        SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, fused ? h : 0));
-        if (k > 1) SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, p->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, fused ? h : 0));
+        SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, fused ? h : 0, 4, p->b));
+        if (k > 1) SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, p->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, fused ? h : 0, 4, p->b));
     }
     for (int32_t t = 0; t < k; ++t) {
         const float *x = ring_buf(ctx, c, ring_index(ctx, k - 1 - t));  // oldest first
@@ -624,7 +624,7 @@ extern "C" sat_status sat_predict(sat_ctx *ctx, int32_t layer, int32_t part, con
             eh.bias_ready = c->tag_bg == params->version;
             c->tag_bg = params->version;
         } else {
-            SAT_TRY(sat_tc_weights(ctx, params->Wg, d, h, nullptr, 0, 0, d, 1, ctx->buf_wsplit, &Wg));
+            SAT_TRY(sat_tc_weights(ctx, params->Wg, d, h, nullptr, 0, 0, d, 1, ctx->buf_wsplit, &Wg, 0, 4, params->bg));
         }
         eh.C = halo_out;
         eh.ldc = ld_out;
@@ -742,7 +742,7 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
     const float *agg = L.agg + (int64_t)v.row0 * ld_agg;
     if (sat_use_tc(d_out, d_in)) {
         TcWeights Wp;
-        SAT_TRY(sat_tc_weights(ctx, W, d_out, d_in, nullptr, 0, 0, d_out, 1, ctx->buf_wsplit, &Wp));
+        SAT_TRY(sat_tc_weights(ctx, W, d_out, d_in, nullptr, 0, 0, d_out, 1, ctx->buf_wsplit, &Wp, 0, 4, bias));
         TcEpilogueHost eh;
         eh.C = h_out;
         eh.ldc = ld_out;
@@ -908,7 +908,7 @@ extern "C" sat_status sat_dense_nn(sat_ctx *ctx, int64_t m, int32_t n, int32_t k
         return sat_fail(ctx, SAT_EINVAL, "sat_dense_nn: null / misaligned tensor or bad shape");
     if (sat_use_tc(n, k)) {
         TcWeights Wp;
-        SAT_TRY(sat_tc_weights(ctx, W, n, k, nullptr, 0, 0, n, 1, ctx->buf_wsplit, &Wp));
+        SAT_TRY(sat_tc_weights(ctx, W, n, k, nullptr, 0, 0, n, 1, ctx->buf_wsplit, &Wp, 0, 4, bias));
         TcEpilogueHost eh;
         eh.C = C;
         eh.ldc = ldc;

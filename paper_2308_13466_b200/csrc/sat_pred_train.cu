@@ -310,8 +310,8 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     // ---- LSTM forward over the snapshots, oldest first, gate values kept ----
     const bool tc_z = sat_use_tc(4 * h, d);
     TcWeights W1, W2;
-    if (tc_z && k > 0) SAT_TRY(sat_tc_weights(ctx, params->Wx, 4 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1));
-    if (tc_z && k > 1) SAT_TRY(sat_tc_weights(ctx, params->Wx, 4 * h, d, params->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2));
+    if (tc_z && k > 0) SAT_TRY(sat_tc_weights(ctx, params->Wx, 4 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, 0, 4, params->b));
+    if (tc_z && k > 1) SAT_TRY(sat_tc_weights(ctx, params->Wx, 4 * h, d, params->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, 0, 4, params->b));
     for (int32_t t = 0; t < k; ++t) {
         const float *x = ring_buf(ctx, c, ring_index(ctx, k - 1 - t));
         float *z = gates + t * plane_g;
@@ -335,7 +335,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     else SAT_CUDA(ctx, cudaMemsetAsync(a, 0, (size_t)nb * h * sizeof(float), ctx->stream));
     if (sat_use_tc(d, h)) {
         TcWeights Wg;
-        SAT_TRY(sat_tc_weights(ctx, params->Wg, d, h, nullptr, 0, 0, d, 1, ctx->buf_wsplit, &Wg));
+        SAT_TRY(sat_tc_weights(ctx, params->Wg, d, h, nullptr, 0, 0, d, 1, ctx->buf_wsplit, &Wg, 0, 4, params->bg));
         TcEpilogueHost eh;
         eh.C = E;
         eh.ldc = ld_d;
