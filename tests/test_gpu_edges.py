@@ -360,3 +360,29 @@ def test_attention_layer_pushes_its_boundary_rows(B, d_out, parts):
         B.sat_sync_status(ctx)
     finally:
         B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 31, 33, 100])          # four rows a warp
+@pytest.mark.parametrize("d", [4, 7, 128, 130, 260])
+def test_attention_scores(B, n, d):
+    """Scores kept by sat_gat_fwd against a . (h W) in fp64 (two contractions one after the other)."""
+    rng = np.random.default_rng(n + d)
+    m = sp.coo_matrix((np.ones(n - 1), (np.arange(n - 1), np.arange(1, n))), shape=(n, n))
+    A = (m + m.T).tocsr()
+    A.sort_indices()
+    k = 20
+    H, W, a1, a2 = (rng.standard_normal(s).astype(np.float32) for s in ((n, k), (k, d), (d,), (d,)))
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, 1, B.SAT_PART_GIVEN, np.zeros(n, np.int32))
+        out = empty2d(n, d)
+        B.sat_gat_fwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(H), None, dev(W), dev(a1), dev(a2), None, B.SAT_ACT_NONE, out)
+        s_src, s_dst, _ = B.sat_gat_scores(ctx, 1, n, 0)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    z, terms = H.astype(np.float64) @ W, np.abs(H).astype(np.float64) @ np.abs(W)
+    for got, a in ((s_src, a1), (s_dst, a2)):
+        bound = ((k + 2) * U + 2.0 ** -20) * (terms @ np.abs(a)) + (d + 2) * U * (np.abs(z) @ np.abs(a)) * (1 + 2.0 ** -10)
+        assert (np.abs(got - z @ a) <= bound + 1e-30).all()
