@@ -12,7 +12,7 @@
 //   forward   k_gat_alpha: softmax of every row, written as {column, alpha} entries; the weighted sums of z rows are then the product
 //             kernel of the GCN layer (sat_spmm_entries) with those entries and a bias / ReLU epilogue.
 //   backward  k_gat_dots: D_v . z_u of every entry, once (a gather of z rows, doubles out); k_gat_rows: t_v, ds_dst and the entry's
-//             alpha and dpre; k_gat_cols brings both to the column side through an index of mirrored entries (gat_prepare) and sums
+//             dpre; k_gat_cols brings alpha and dpre to the column side through an index of mirrored entries (gat_prepare) and sums
 //             ds_src; dZ is again the product kernel, with D rows gathered and the a_src / a_dst terms in its epilogue.
 // The first version recomputed alpha and the dot product in each of three gather sweeps and walked every halo row with one warp:
 // 169 k nodes, 2.6 M entries, 256 wide: 763 + 626 + 911 us per layer in its sweeps against 389 (dots) + 65 (rows, cols) + 370 (the two
@@ -231,9 +231,9 @@ k_gat_dots(const int4 *__restrict__ items, int32_t n_items, const int32_t *__res
     }
 }
 
-// per row v: t_v = sum alpha dot / sum alpha and ds_dst[v]; per entry, over the dot product: {alpha, dpre = alpha slope (dot - t_v)}
+// per row v: t_v = sum alpha dot / sum alpha and ds_dst[v]; per entry, over the dot product: dpre = alpha slope (dot - t_v)
 // (the sums in double and divided by sum alpha: the fp32 weights sum to 1 + eps, and ds_dst, exactly zero where all slopes agree,
-// would inherit -eps t_v)
+// would inherit -eps t_v; dpre stays in double until its column is summed, the dpre of a column cancel as well)
 template <int T>
 __device__ __forceinline__ void gat_row(int tid, int64_t e0, int64_t e1, float sd, const int2 *__restrict__ ent, int32_t n,
                                         const float *__restrict__ s_in, const float *__restrict__ s_halo, double *__restrict__ dots,
@@ -242,7 +242,7 @@ __device__ __forceinline__ void gat_row(int tid, int64_t e0, int64_t e1, float s
     auto slope = [&](int32_t c) { return sd + (c < n ? s_in[c] : s_halo[c - n]) > 0.f ? 1.f : GAT_SLOPE; };
     const int64_t ef = e0 + tid;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, p_first = 0.0;
-    float al_first = 0.f, as_first = 0.f;
+    float as_first = 0.f;
 #pragma unroll 4
     for (int64_t e = ef; e < e1; e += T) {
         const int2 q = ent[e];
@@ -254,7 +254,6 @@ __device__ __forceinline__ void gat_row(int tid, int64_t e0, int64_t e1, float s
         a3 += as;
         if (e == ef) {
             p_first = p;
-            al_first = al;
             as_first = al * sl;
         }
     }
@@ -264,13 +263,11 @@ __device__ __forceinline__ void gat_row(int tid, int64_t e0, int64_t e1, float s
     a3 = team_reduce<T>(a3, OpAdd(), sh);
     const double t = a1 / a0;
     if (tid == 0) *ds_dst = (float)(a2 / a0 - t * (a3 / a0));
-    float2 *edge = reinterpret_cast<float2 *>(dots);
-    if (ef < e1) edge[ef] = make_float2(al_first, (float)((double)as_first * (p_first - t)));
+    if (ef < e1) dots[ef] = (double)as_first * (p_first - t);
 #pragma unroll 4
     for (int64_t e = ef + T; e < e1; e += T) {
         const int2 q = ent[e];
-        const float al = __int_as_float(q.y);
-        edge[e] = make_float2(al, (float)((double)(al * slope(q.x)) * (dots[e] - t)));
+        dots[e] = (double)(__int_as_float(q.y) * slope(q.x)) * (dots[e] - t);
     }
 }
 
@@ -297,14 +294,15 @@ k_gat_rows(const int64_t *__restrict__ lrowptr, const int2 *__restrict__ ent, in
 // column side of node u: its entries are the mirror images map[e] of row entries (v, u); ent_out[e] = {v, alpha_vu}, ds_src[u] = sum dpre_vu
 template <int T>
 __device__ __forceinline__ void gat_col(int tid, int64_t e0, int64_t e1, const int32_t *__restrict__ idx, const uint32_t *__restrict__ map,
-                                        const float2 *__restrict__ edge, int2 *__restrict__ ent_out, float *__restrict__ ds_src, double *sh)
+                                        const int2 *__restrict__ ent, const double *__restrict__ dpre, int2 *__restrict__ ent_out,
+                                        float *__restrict__ ds_src, double *sh)
 {
     double s = 0.0;
 #pragma unroll 4
     for (int64_t e = e0 + tid; e < e1; e += T) {
-        const float2 x = edge[map[e]];
-        ent_out[e] = make_int2(idx[e], __float_as_int(x.x));
-        s += (double)x.y;
+        const uint32_t m = map[e];
+        ent_out[e] = make_int2(idx[e], ent[m].y);
+        s += dpre[m];
     }
     s = team_reduce<T>(s, OpAdd(), sh);
     if (tid == 0) *ds_src = (float)s;
@@ -312,21 +310,21 @@ __device__ __forceinline__ void gat_col(int tid, int64_t e0, int64_t e1, const i
 
 __global__ void __launch_bounds__(256)
 k_gat_cols(const int64_t *__restrict__ ptr, const int32_t *__restrict__ cnt, int64_t u0, int64_t n_u, const int32_t *__restrict__ long_u, int32_t n_long,
-           const int32_t *__restrict__ idx, const uint32_t *__restrict__ map, const float2 *__restrict__ edge, int2 *__restrict__ ent_out,
-           float *__restrict__ ds_src)
+           const int32_t *__restrict__ idx, const uint32_t *__restrict__ map, const int2 *__restrict__ ent, const double *__restrict__ dpre,
+           int2 *__restrict__ ent_out, float *__restrict__ ds_src)
 {
     sat_grid_wait();
     __shared__ double sh[8];
     if ((int32_t)blockIdx.x < n_long) {
         const int32_t u = long_u[blockIdx.x];
-        gat_col<256>(threadIdx.x, ptr[u], cnt ? ptr[u] + cnt[u] : ptr[u + 1], idx, map, edge, ent_out, ds_src + u, sh);
+        gat_col<256>(threadIdx.x, ptr[u], cnt ? ptr[u] + cnt[u] : ptr[u + 1], idx, map, ent, dpre, ent_out, ds_src + u, sh);
         return;
     }
     const int64_t w = ((int64_t)(blockIdx.x - n_long) * 256 + threadIdx.x) / GAT_TEAM;
     if (w >= n_u) return;
     const int64_t u = u0 + w, e0 = ptr[u];
     if (ptr[u + 1] - e0 > GAT_LONG) return;
-    gat_col<GAT_TEAM>(threadIdx.x & (GAT_TEAM - 1), e0, cnt ? e0 + cnt[u] : ptr[u + 1], idx, map, edge, ent_out, ds_src + u, sh);
+    gat_col<GAT_TEAM>(threadIdx.x & (GAT_TEAM - 1), e0, cnt ? e0 + cnt[u] : ptr[u + 1], idx, map, ent, dpre, ent_out, ds_src + u, sh);
 }
 
 // mirror images: entry e = (r, c) of the inner block is entry rev[e] = (c, r); entry i of halo row j (node u, inner neighbour v) is the
@@ -651,7 +649,7 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
     const int64_t n = ctx->n;
     float *z_in = (float *)G.z_in.p, *z_halo = (float *)G.z_halo.p;
     float *s_in = (float *)G.scal.p, *s_dst = s_in + n, *s_halo = s_dst + n;
-    // scratch of the call, by row / halo position / entry of the selection: dot products (then alpha and dpre), entries of the inner and
+    // scratch of the call, by row / halo position / entry of the selection: dot products (then dpre), entries of the inner and
     // of the halo column side, D, dZ, ds_dst, ds_src
     const int64_t ent0 = ctx->h_lnnz_off[v.p0], cut0 = ctx->h_hrow_off[v.p0];
     const size_t f_rows = (size_t)(v.n_rows > 0 ? v.n_rows : 1), f_halo = (size_t)(v.n_halo > 0 ? v.n_halo : 1), f_ent = (size_t)v.lnnz + 2,
@@ -692,7 +690,7 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
                                                   s_halo, s_dst, dots_b, ds_dst_b);
         SAT_LAUNCHED(ctx);
         sat_pdl(ctx->stream, k_gat_cols, grid, 256, 0)(ctx->lrowptr, ctx->inner_cnt, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, ctx->lenc,
-                                                  ctx->gat_rev, (const float2 *)dots_b, ent_in_b, ds_in_b);
+                                                  ctx->gat_rev, (const int2 *)G.ent.p, dots_b, ent_in_b, ds_in_b);
         SAT_LAUNCHED(ctx);
         SpmmEpilogue ep;
         ep.s1 = ds_in_b;
@@ -707,7 +705,7 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
         ProfScope prof(ctx, SATK_GAT, 0.0, 0.0);
         sat_pdl(ctx->stream, k_gat_cols, (unsigned)(v.n_hlong + cdiv64(v.n_halo * GAT_TEAM, 256)), 256, 0)(
             ctx->hrow_ptr, nullptr, v.halo0, v.n_halo, ctx->hlong ? ctx->hlong + v.hlong0 : nullptr, v.n_hlong, ctx->hrow_pos, ctx->gat_hmap,
-            (const float2 *)dots_b, ent_halo_b, ds_halo_b);
+            (const int2 *)G.ent.p, dots_b, ent_halo_b, ds_halo_b);
         SAT_LAUNCHED(ctx);
         SpmmEpilogue ep;
         ep.s1 = ds_halo_b;

@@ -184,3 +184,43 @@ def test_epochs_with_the_attention_backbone(B, name, shrink):
             params = [{k: (v - 0.5 * res["grads"][l][k]).astype(np.float32) for k, v in p.items()} for l, p in enumerate(params)]
     finally:
         ep.close()
+
+
+@pytest.mark.parametrize("M", [1, 2])
+def test_score_gradients_of_columns_that_cancel(B, M):
+    """ds_src of a node is a sum of dpre over its column that may cancel most of its size: the terms are summed in double and
+    rounded once.  Complete graphs of four nodes with zero attention vectors: alpha = 1/4 and slope 0.2f exactly, and with
+    gradients g in one column  ds_src[u] = c (z_u - mean z) sum_v g_v,  c = 0.25 * 0.2f.  The pairs of g cancel to 2^-16 of their
+    size, so a term rounded to fp32 (2^-25 of it) would show as 2^-9 of the result; what is left is one rounding of ds_src per node
+    and the fp32 sum over at most 2 n nodes and halo copies."""
+    import scipy.sparse as sp
+    blocks, d = 16, 4
+    n = 4 * blocks
+    A = sp.kron(sp.identity(blocks), np.ones((4, 4)) - np.eye(4)).tocsr()
+    A.eliminate_zeros()
+    rng = np.random.default_rng(5)
+    X = np.zeros((n, d), np.float32)
+    X[:, 0] = rng.standard_normal(n)
+    G = np.zeros((n, d), np.float32)
+    G[0::2, 0] = rng.standard_normal(n // 2)
+    G[1::2, 0] = -G[0::2, 0] * np.float32(1 + 2.0 ** -16)
+    part = (np.arange(n) // 2 % M).astype(np.int32)      # two partitions: the pairs of a block lie in different ones
+    perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        halo = np.concatenate([B.sat_part_lists(ctx, m)["halo_gid"] for m in range(M)])
+        h_in, h_halo, out, g_in = dev2d(X[perm]), dev2d(X[halo]) if M > 1 else None, empty2d(n, d), empty2d(n, d)
+        W, a = dev(np.eye(d, dtype=np.float32)), dev(np.zeros(d, np.float32))
+        gW, gas, gad, gb = dev(np.zeros((d, d), np.float32)), dev(np.zeros(d, np.float32)), dev(np.zeros(d, np.float32)), dev(np.zeros(d, np.float32))
+        B.sat_gat_fwd(ctx, B.SAT_ALL_PARTS, 1, h_in, h_halo, W, a, a, None, B.SAT_ACT_NONE, out)
+        B.sat_gat_bwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(G[perm]), None, h_in, h_halo, W, a, a, gW, gas, gad, gb, 0, g_in)
+        B.sat_sync_status(ctx)
+        got = float(gas[0])
+    finally:
+        B.sat_destroy(ctx)
+    z, g, c = X[:, 0].astype(np.float64), G[:, 0].astype(np.float64), float(np.float32(0.25) * np.float32(0.2))
+    pairs = (z - np.repeat(z.reshape(-1, 4).mean(1), 4)).reshape(-1, 4, 1) * c * g.reshape(-1, 1, 2, 2).sum(3)   # [block, u, pair]
+    terms = (pairs * z.reshape(-1, 4, 1)) if M > 1 else (pairs.sum(2, keepdims=True) * z.reshape(-1, 4, 1))
+    assert abs(got - terms.sum()) <= (2 * n + 4) * 2.0 ** -24 * np.abs(terms).sum()
