@@ -1587,15 +1587,21 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
     if (m == 0 || n == 0) return SAT_OK;
     if (segments < 1 || segments > SAT_TN_SEGMENTS) return sat_fail(ctx, SAT_EINVAL, "sat_gemm_tc_tn: 1 to %d segments", SAT_TN_SEGMENTS);
     ProfScope prof(ctx, SATK_GEMM_TN, 4.0 * ((double)rows * segments * (m + n) + (double)m * n), 2.0 * (double)rows * segments * m * n);
-    const int32_t bn = tile_n_for(n), mt = m > TC_BM ? 2 : 1;
+    // Tiles of 256 columns of A where they are all full, else of 128 with two CTAs per SM (256 of the 512 TMEM columns each): 179250 x
+    // 300 x 512 376 -> 370 us, 58241 x 602 x 256 119 -> 136 us with the splits below.
+    const int32_t bn = tile_n_for(n), subs = (int32_t)cdiv64(m, TC_BM), mt = subs % 2 == 0 ? 2 : 1;
     const uint32_t stage_bytes = 2 * (uint32_t)mt * (TC_BM / 32) * TC_BK * 128 + 2 * (uint32_t)((bn + 31) / 32) * TC_BK * 128;
     const int64_t r1 = rows > 0 ? rows : 1, kblocks = cdiv64(r1, TC_BK);
-    // One wave: a CTA per SM, or two where the tile is 128 columns of A (256 of the 512 TMEM columns each; the shorter chains also keep
-    // the truncating accumulation error down).  Not less than six k-blocks each: the m x n partial sums of a split, written and read
-    // again, cost about as much as that.
     const int per_sm = mt == 1 ? 2 : 1;
-    const int64_t tiles = cdiv64(m, mt * TC_BM) * cdiv64(n, bn);
-    int64_t splits = tiles * segments < 148 * per_sm ? 148 * per_sm / (tiles * segments) : 1;   // of a segment
+    const int64_t col_tiles = cdiv64(n, bn), tiles = cdiv64(m, mt * TC_BM) * col_tiles;
+    // Row splits of a segment, in whole waves.  The accumulation truncates, so the error of a split's sum grows with its length, while the
+    // partial sums are added with rounding: a split is not longer than with two 128-column tiles per SM, whatever the tile and however many
+    // segments share the launch (one wave over all segments: relative error of the predictor's gradients 8e-6 -> 6e-5 at 512 columns and
+    // eight steps; one wave of 256-column tiles over 300 columns 7.2e-5 -> 8.7e-5).  Not less than six k-blocks each: the m x n partial
+    // sums of a split, written and read again, cost about as much as that.
+    const int64_t least = cdiv64(2 * ctx->sms, (int64_t)subs * col_tiles), slots = (int64_t)ctx->sms * per_sm, per_split = tiles * segments;
+    const int64_t waves = cdiv64(least * per_split, slots);
+    int64_t splits = per_split < slots * waves ? slots * waves / per_split : 1;
     if (splits > cdiv64(kblocks, 6)) splits = cdiv64(kblocks, 6);
     const int64_t kpb = cdiv64(kblocks, splits), rps = kpb * TC_BK;
     splits = cdiv64(r1, rps);

@@ -386,3 +386,27 @@ def test_attention_scores(B, n, d):
     for got, a in ((s_src, a1), (s_dst, a2)):
         bound = ((k + 2) * U + 2.0 ** -20) * (terms @ np.abs(a)) + (d + 2) * U * (np.abs(z) @ np.abs(a)) * (1 + 2.0 ** -10)
         assert (np.abs(got - z @ a) <= bound + 1e-30).all()
+
+
+@pytest.mark.parametrize("m,n", [(300, 256), (384, 512)])
+def test_weight_gradient_error_with_an_odd_number_of_column_tiles(B, m, n):
+    """Sums of positive terms: what is lost is the truncating accumulation, which grows with the rows that a split adds up.  At most two
+    128-column tiles per SM decide that length; against 256 columns (two such tiles) the error may grow by the ratio of the lengths.
+    (1.2: the loss per addition, relative to the sum, moves by the place of the sum between two powers of two.)"""
+    rows, sms = 120000, torch.cuda.get_device_properties(0).multi_processor_count
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(m)
+    A, D = (torch.empty((rows, w), device="cuda").normal_(generator=gen).abs_() for w in (m, n))
+    lost, length = [], []
+    ctx = B.sat_create(0, torch.cuda.current_stream().cuda_stream)
+    try:
+        for k in (256, m):
+            C = torch.empty((k, n), device="cuda")
+            B.sat_dense_tn(ctx, A[:, :k], D, C)
+            B.sat_sync_status(ctx)
+            want = A[:, :k].double().T @ D.double()
+            lost.append(float((1 - C.double() / want).mean()))
+            length.append(rows / -(-2 * sms // (-(-k // 128) * -(-n // 256))))
+    finally:
+        B.sat_destroy(ctx)
+    assert 0 < lost[1] <= 1.2 * lost[0] * length[1] / length[0]

@@ -200,3 +200,54 @@ def test_degenerate_cases_and_argument_errors(B):
         assert all(bool(torch.isfinite(t).all()) for t in g)
     finally:
         ep.close()
+
+
+@pytest.mark.parametrize("tau,d,h", [(2, 64, 20), (8, 64, 20), (10, 300, 32)])
+def test_gradient_sums_over_steps_lose_no_more_than_one_step(B, tau, d, h):
+    """The parameter gradients are sums over nodes and steps; the sum of one step over its nodes truncates, what is added to it does not.
+    With positive weights, snapshots and errors every term is positive, so the relative loss of the sum over all steps is
+    that of one step (window 1) and not more of it the longer the window is.  2^-20: gates in fp32 and the split contractions behind them."""
+    import torch
+    n = 40000                                   # a ring: the two neighbours of every node lie in the other partition
+    ids = np.arange(n)
+    rowptr = 2 * np.arange(n + 1, dtype=np.int64)
+    col = np.sort(np.stack([(ids - 1) % n, (ids + 1) % n], 1), 1).astype(np.int32).ravel()
+    part = (ids % 2).astype(np.int32)
+    perm = np.concatenate([ids[0::2], ids[1::2]])
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d)
+    rand = lambda *s: torch.rand(s, device="cuda", generator=gen)
+    Wx, Uh, b, Wg, bg = rand(d, 4 * h) / d, rand(h, 4 * h) / h, rand(4 * h), rand(h, d) / h, rand(d)
+    snaps = [rand(n, d) for _ in range(tau)]    # rows by node
+    lost = {}
+    for k in (1, tau):
+        ctx = B.sat_create(0, torch.cuda.current_stream().cuda_stream)
+        try:
+            B.sat_graph_load(ctx, rowptr, col)
+            B.sat_partition(ctx, 2, B.SAT_PART_GIVEN, part)
+            B.sat_cache_init(ctx, [d], k)
+            order = torch.from_numpy(perm).cuda()
+            for x in snaps[:k]:
+                B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, x[order])
+                B.sat_cache_commit(ctx)
+            B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, torch.zeros((n, d), device="cuda"))      # the target: errors are positive
+            p = B.make_pred_params(Wx, Uh, b, Wg, bg, h, 0)
+            grads = [torch.empty_like(t) for t in p._keep]
+            B.sat_pred_grad(ctx, 1, p, None, *grads)
+            B.sat_sync_status(ctx)
+        finally:
+            B.sat_destroy(ctx)
+        P64 = [t.double().requires_grad_() for t in (Wx, Uh, b, Wg, bg)]
+        s = c = torch.zeros((n, h), dtype=torch.float64, device="cuda")
+        for x in snaps[:k]:
+            i, f, g, o = (x.double() @ P64[0] + s @ P64[1] + P64[2]).split(h, 1)
+            c = torch.sigmoid(f) * c + torch.sigmoid(i) * torch.tanh(g)
+            s = torch.sigmoid(o) * torch.tanh(c)
+        a = (s + s.roll(1, 0) + s.roll(-1, 0)) / 3
+        out = snaps[k - 1].double() + a @ P64[3] + P64[4]
+        (0.5 * out.square().sum() / n).backward()             # 1 / M sum_m 1 / b_m with two partitions of n / 2 halo rows each
+        # (at the first step there is no state, and the forget gate multiplies a zero)
+        lost[k] = [float((1 - g.double() / w.grad)[w.grad != 0].mean()) for g, w in zip(grads[:2], P64[:2]) if bool((w.grad != 0).any())]
+    assert len(lost[tau]) == 2 and len(lost[1]) == 1
+    for err in lost[tau]:
+        assert abs(err) <= abs(lost[1][0]) + 2.0 ** -20
