@@ -1109,9 +1109,20 @@ k_gemm_tc_mn(const __grid_constant__ MnMaps maps, int32_t seg_splits, int32_t Md
         const bool want_cs = part_cs != nullptr && blockIdx.x == 0;
         // thread t takes 16-byte piece t % 128 of every second 32-column block; row (t % 128) / 8 of each k-block
         const uint32_t off = (uint32_t)(ctid & 127) * 16, half = (uint32_t)(ctid >> 7);
-        float4 cs[4];
+        // column sums in two levels (sixteen k-blocks, then their sums): in one, a long split's sum carried 3.3e-7 instead of 2.2e-7
+        float4 cs[4], cs_sum[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) cs[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < 4; ++i) cs[i] = cs_sum[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto fold = [&]() {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                cs_sum[i].x += cs[i].x;
+                cs_sum[i].y += cs[i].y;
+                cs_sum[i].z += cs[i].z;
+                cs_sum[i].w += cs[i].w;
+                cs[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        };
         bool alive = true;
         for (int32_t kb = 0; kb < nkb && alive; ++kb) {
             const int s = kb % stages;
@@ -1151,7 +1162,9 @@ k_gemm_tc_mn(const __grid_constant__ MnMaps maps, int32_t seg_splits, int32_t Md
             }
             fence_async_smem();
             mbar_arrive(&sh->conv[s]);
+            if ((kb & 15) == 15) fold();
         }
+        fold();
         const int q = warp & 3, e = (warp - 2) >> 2;
         const bool ok = alive && mbar_wait(&sh->accum, 0, dead, status);   // every MMA has completed: the stages are free
         tc_fence_after();
@@ -1186,7 +1199,7 @@ k_gemm_tc_mn(const __grid_constant__ MnMaps maps, int32_t seg_splits, int32_t Md
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int bl = (int)half + 2 * i;
-                if (bl < n_blks_b && ok) *reinterpret_cast<float4 *>(cb + rr * w + bl * 32 + piece * 4) = cs[i];
+                if (bl < n_blks_b && ok) *reinterpret_cast<float4 *>(cb + rr * w + bl * 32 + piece * 4) = cs_sum[i];
             }
             asm volatile("bar.sync 1, 256;" ::: "memory");
             for (int c = ctid; c < w; c += MN_CONV_THREADS) {

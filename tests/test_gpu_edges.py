@@ -410,3 +410,26 @@ def test_weight_gradient_error_with_an_odd_number_of_column_tiles(B, m, n):
     finally:
         B.sat_destroy(ctx)
     assert 0 < lost[1] <= 1.2 * lost[0] * length[1] / length[0]
+
+
+@pytest.mark.parametrize("m,n", [(16, 47), (256, 512)])               # the narrow kernel, and the converters of the tensor-core one
+def test_bias_gradient_of_many_rows(B, m, n):
+    """One large term and many of half its last place, which a plain running sum would lose (2^-25 each, 200 and more behind the large
+    one); levels of at most 16 additions, 64 in all, lose at most 64 units of the sum."""
+    rows = 400000
+    ids = np.arange(rows)
+    col = np.sort(np.stack([(ids - 1) % rows, (ids + 1) % rows], 1), 1).astype(np.int32).ravel()
+    ctx = B.sat_create(0, torch.cuda.current_stream().cuda_stream)
+    try:
+        B.sat_graph_load(ctx, 2 * np.arange(rows + 1, dtype=np.int64), col)
+        B.sat_partition(ctx, 1, B.SAT_PART_CONTIG_BLOCKS)
+        X, D, W = torch.ones((rows, m), device="cuda"), empty2d(rows, n, fill=2.0 ** -25), torch.zeros((m, n), device="cuda")
+        D[0] = 1.0
+        B.sat_layer_fwd(ctx, 0, 1, X, None, W, None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, empty2d(rows, n))
+        gW, gb = torch.empty((m, n), device="cuda"), torch.empty(n, device="cuda")
+        B.sat_layer_bwd(ctx, 0, 1, D, W, gW, gb, 0, None, None)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    want = 1.0 + (rows - 1) * 2.0 ** -25
+    assert float((gb.double() - want).abs().max()) <= 64 * U * want
