@@ -384,8 +384,9 @@ sat_status sat_sgd_steps(sat_ctx *ctx, int32_t n_arrays, const int64_t *counts, 
  * described once.  Per partition (or for all of them at once): for l = 1..L  sat_predict of cached layer l-1 where pred[l-2] is
  * given (SAT_FWD_HALO_CACHED where not), sat_layer_fwd with ReLU and SAT_FWD_PUSH (l < L; layer 1 reads x with
  * SAT_FWD_INPUT_GLOBAL);  sat_loss_grad;  sat_layer_bwd for l = L..1 with the fused ReLU masks.  Results are those of these calls.
- *   order     n_order = 0: all partitions per launch.  Otherwise the partitions to run, one after the other (HOST array): the first
- *             one runs the predictor's recurrence and overwrites the gradients, the others reuse the state table and add to them.
+ *   order     NULL (with n_order = 0): all partitions per launch.  Otherwise the n_order partitions to run, one after the other (HOST
+ *             array): the first one runs the predictor's recurrence and overwrites the gradients, the others reuse the state table and
+ *             add to them.  An empty order runs none: the loss is zero, the gradients stay as they are, commit and step follow as asked.
  *   flags     SAT_EPOCH_GRAD_HISTORY: SAT_BWD_GRAD_HISTORY on layers >= 2;  SAT_EPOCH_COMMIT: sat_cache_commit afterwards;
  *             SAT_EPOCH_STEP: w <- w - lr gw, b <- b - lr gb afterwards;  SAT_EPOCH_CONTINUE: this call goes on with an epoch that an
  *             earlier one began (partitions of `order` that are yet to run): its first partition too reuses the state table and adds to

@@ -269,10 +269,11 @@ def make_epoch_buffers(dims, X, labels, loss_kind: int, H, G, halo, W, b, gW, gb
 
 
 def sat_epoch(ctx, buffers: sat_epoch_buffers, order=None, flags: int = SAT_EPOCH_COMMIT, lr: float = 0.0):
-    """order: partitions to run one after the other, or None for all of them per launch."""
+    """order: partitions to run one after the other (any iterable, an empty one runs none), or None for all of them per launch."""
     if order is None:
         st = _lib.sat_epoch(ctx, C.byref(buffers), None, 0, flags, C.c_float(lr))
     else:
+        order = [int(m) for m in order]
         st = _lib.sat_epoch(ctx, C.byref(buffers), (C.c_int32 * max(len(order), 1))(*order), len(order), flags, C.c_float(lr))
     _check(ctx, st)
 

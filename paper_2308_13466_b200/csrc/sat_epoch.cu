@@ -49,14 +49,16 @@ extern "C" sat_status sat_epoch(sat_ctx *ctx, const sat_epoch_buffers *e, const 
 {
     CHECK_CTX(ctx);
     if (!e || e->n_layers < 1 || e->n_layers > SAT_MAX_LAYERS || !e->dims || !e->x || !e->labels || !e->h || !e->ld_h || !e->g || !e->ld_g || !e->w || !e->b ||
-        !e->gw || !e->gb || (n_order > 0 && !order) || n_order < 0 || (flags & ~(SAT_EPOCH_GRAD_HISTORY | SAT_EPOCH_COMMIT | SAT_EPOCH_STEP | SAT_EPOCH_CONTINUE)))
+        !e->gw || !e->gb || (n_order != 0 && !order) || n_order < 0 || (flags & ~(SAT_EPOCH_GRAD_HISTORY | SAT_EPOCH_COMMIT | SAT_EPOCH_STEP | SAT_EPOCH_CONTINUE)))
         return sat_fail(ctx, SAT_EINVAL, "sat_epoch: incomplete description or unknown flags");
     for (int32_t l = 0; l < e->n_layers; ++l) {
         if (!e->w[l] || !e->gw[l] || !e->h[l] || !e->g[l]) return sat_fail(ctx, SAT_EINVAL, "sat_epoch: null array of layer %d", l + 1);
         if (l > 0 && e->pred && e->pred[l - 1] && !e->halo && ctx->nb > 0) return sat_fail(ctx, SAT_EINVAL, "sat_epoch: no room for the predicted rows");
     }
-    for (int32_t i = 0; i < (n_order > 0 ? n_order : 1); ++i)
-        SAT_TRY(epoch_pass(ctx, e, n_order > 0 ? order[i] : (int32_t)SAT_ALL_PARTS, i == 0 && !(flags & SAT_EPOCH_CONTINUE), flags & SAT_EPOCH_GRAD_HISTORY));
+    const bool begin = !(flags & SAT_EPOCH_CONTINUE);
+    for (int32_t i = 0; i < (order ? n_order : 1); ++i)
+        SAT_TRY(epoch_pass(ctx, e, order ? order[i] : (int32_t)SAT_ALL_PARTS, i == 0 && begin, flags & SAT_EPOCH_GRAD_HISTORY));
+    if (order && n_order == 0 && begin && e->loss_sum) SAT_CUDA(ctx, cudaMemsetAsync(e->loss_sum, 0, sizeof(double), ctx->stream));   // the loss of no partition
     if (flags & SAT_EPOCH_COMMIT) SAT_TRY(sat_cache_commit(ctx));
     if (flags & SAT_EPOCH_STEP) {
         int64_t counts[2 * SAT_MAX_LAYERS];

@@ -320,3 +320,28 @@ def test_odd_shapes_and_degenerate_partitions(B, over, empty_part):
                 B.sat_cache_set_state(ep.ctx, cache.write_idx, cache.n_valid)
     finally:
         ep.close()
+
+
+def test_orders_of_partitions(B):
+    """An order may be any iterable; an empty one runs no partition: loss zero, commit and parameter step on the gradients there are."""
+    import torch
+    wl = make_workload("tiny")
+    ep, P, _, _ = _setup(B, wl)
+    try:
+        preds = pred_to_device(wl.pred, B, 0)
+        W, b = [dev(w) for w in wl.W], [dev(x) for x in wl.b]
+        ep.step_per_partition(W, b, preds, order=[2, 0, 1] + list(range(3, wl.M)))
+        kept = [t.clone() for t in ep.H[1:] + ep.gW + ep.gb]
+        assert float(ep.loss_sum) > 0
+        before, want = B.sat_cache_state(ep.ctx), [w - 0.5 * g for w, g in zip(W + b, ep.gW + ep.gb)]
+        ep.step_per_partition(W, b, preds, order=[], lr=0.5)
+        assert float(ep.loss_sum) == 0.0
+        assert all(torch.equal(x, y) for x, y in zip(ep.H[1:] + ep.gW + ep.gb, kept))
+        assert all(torch.equal(x, y) for x, y in zip(W + b, want))
+        assert B.sat_cache_state(ep.ctx) == ((before[0] + 1) % (wl.tau + 1), min(before[1] + 1, wl.tau))
+        for order in (iter(range(wl.M)), np.arange(wl.M), torch.arange(wl.M)):
+            ep.step_per_partition(W, b, preds, order=order)
+            assert float(ep.loss_sum) > 0
+        B.sat_sync_status(ep.ctx)
+    finally:
+        ep.close()
