@@ -100,16 +100,17 @@ class SatEpoch:
 
     # ---- one epoch ----------------------------------------------------------------
     def _described(self, W, b, pred) -> B.sat_epoch_buffers:
-        """The buffers of an epoch as the library takes them; made anew when any tensor behind them is another one."""
-        key = (self.X, self.labels, *W, *b, *(pred or ()), pred is None)
-        ptrs = [t.data_ptr() for t in W]
-        ptrs += [None if t is None else t.data_ptr() for t in b]
-        old = self._epoch_key
-        if old is None or len(old[0]) != len(key) or any(x is not y for x, y in zip(old[0], key)) or old[1] != ptrs:
+        """The buffers of an epoch as the library takes them; made anew when the place, shape or strides of any of them (this object's own
+        among them) or a predictor is another one."""
+        tensors = (self.X, self.labels, *self.H[1:], *self.G[1:], self.halo, *W, *b, *self.gW, *self.gb, self.loss_sum)
+        key = [t if t is None else (t.data_ptr(), t.shape, t.stride()) for t in tensors]
+        # predictors are read through their own structures at every call: the same structure is all that matters
+        key += [len(W), len(b), self.loss, pred if pred is None else [None if p is None else id(p) for p in pred]]
+        if key != self._epoch_key:
             kind = B.SAT_LOSS_SOFTMAX_CE if self.loss == "ce" else B.SAT_LOSS_SIGMOID_BCE
             self._epoch_buf = B.make_epoch_buffers(self.dims, self.X, self.labels, kind, self.H[1:], self.G[1:], self.halo, W, b, self.gW, self.gb,
                                                    pred, self.loss_sum)
-            self._epoch_key = (key, ptrs)
+            self._epoch_key = key
         return self._epoch_buf
 
     def _forward_backward(self, m: int, W, b, pred, accumulate: int, reuse_state: int, grad_history: bool = False):

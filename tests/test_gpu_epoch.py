@@ -345,3 +345,47 @@ def test_orders_of_partitions(B):
         B.sat_sync_status(ep.ctx)
     finally:
         ep.close()
+
+
+def test_replaced_buffers_are_the_ones_that_count(B):
+    """The public buffers of a SatEpoch and the storage behind the caller's tensors may be others at every step."""
+    import torch
+    wl = make_workload("tiny")
+    ep, P, _, perm = _setup(B, wl)
+    try:
+        preds = pred_to_device(wl.pred, B, 0)
+        W, b = [dev(w) for w in wl.W], [dev(x) for x in wl.b]
+        ep.step(W, b, preds)
+        state = [B.sat_cache_export(ep.ctx, l, wl.tau, ep.n_slots, wl.dims[l]) for l in range(1, wl.L)], B.sat_cache_state(ep.ctx)
+
+        def again():
+            for l in range(1, wl.L):
+                B.sat_cache_import(ep.ctx, l, state[0][l - 1])
+            B.sat_cache_set_state(ep.ctx, *state[1])
+            ep.step(W, b, preds)
+            return [t.clone() for t in ep.H[1:] + ep.gW + ep.gb + [ep.loss_sum]]
+
+        want = again()
+        old = [ep.H[1], ep.G[1], ep.gW[0], ep.gb[0], ep.loss_sum, ep.halo]
+        marks = [torch.full_like(t, 7.0) for t in old]
+        for t, m in zip(old, marks):
+            t.copy_(m)
+        ep.H[1], ep.G[1] = (torch.zeros((t.shape[0], (t.shape[1] + 7) & ~3), device="cuda")[:, :t.shape[1]] for t in old[:2])
+        ep.gW[0], ep.gb[0], ep.loss_sum, ep.halo = torch.zeros_like(old[2]), torch.zeros_like(old[3]), torch.zeros_like(old[4]), torch.zeros_like(old[5])
+        assert all(torch.equal(x, y) for x, y in zip(again(), want))
+        assert all(torch.equal(t, m) for t, m in zip(old, marks))
+        # other storage behind the same tensor objects
+        rng = np.random.default_rng(3)
+        X2 = rng.standard_normal(wl.X.shape).astype(np.float32)
+        ep.X.data = dev2d(X2)
+        got = again()
+        assert not torch.equal(got[0], want[0])
+        ep.set_inputs(dev2d(X2), ep.labels)
+        assert all(torch.equal(x, y) for x, y in zip(again(), got))
+        W[0].resize_(W[0].shape[1], W[0].shape[0])            # the same storage in another shape
+        with pytest.raises(AssertionError):
+            ep.step(W, b, preds)
+        W[0].resize_(W[0].shape[1], W[0].shape[0])
+        assert all(torch.equal(x, y) for x, y in zip(again(), got))
+    finally:
+        ep.close()
