@@ -250,11 +250,14 @@ def sat_layer_bwd(ctx, part: int, layer: int, g_out, W, g_W, g_b, accumulate: in
 
 def make_epoch_buffers(dims, X, labels, loss_kind: int, H, G, halo, W, b, gW, gb, pred, loss_sum) -> sat_epoch_buffers:
     """Description for sat_epoch: H, G the layers' outputs and gradients (row strides multiples of 4), W, b, gW, gb contiguous
-    CUDA fp32 lists, pred a list of sat_pred_params or None per cached layer, or None."""
+    CUDA fp32 lists, pred a list of sat_pred_params or None per cached layer, or None.  dims says how many layers there are: entries of
+    the lists behind them are not looked at, and a list with too few is an IndexError."""
+    n = len(dims) - 1
+    H, G, W, b, gW, gb = ([ts[l] for l in range(n)] for ts in (H, G, W, b, gW, gb))
+    pred = None if pred is None else [pred[l] for l in range(n - 1)]
     for l, (w, gw, bb, gbb) in enumerate(zip(W, gW, b, gb)):
         assert w.is_cuda and w.is_contiguous() and gw.is_contiguous() and tuple(w.shape) == tuple(gw.shape) == (dims[l], dims[l + 1])
         assert bb is None or (bb.is_cuda and bb.is_contiguous() and bb.numel() == gbb.numel() == dims[l + 1])
-    n = len(W)
     ptrs = lambda ts: (C.c_void_p * max(len(ts), 1))(*[None if t is None else t.data_ptr() for t in ts])
     lds = lambda ts: (C.c_int32 * len(ts))(*[_ld(t) for t in ts])
     adr = lambda a: C.cast(a, C.c_void_p).value
@@ -262,7 +265,7 @@ def make_epoch_buffers(dims, X, labels, loss_kind: int, H, G, halo, W, b, gW, gb
     e = sat_epoch_buffers(n_layers=n, x=_dev(X).value, ld_x=_ld(X), loss_kind=loss_kind, labels=_dev(labels).value, halo=_dev(halo).value,
                           ld_halo=_ld(halo), loss_sum=None if loss_sum is None else loss_sum.data_ptr(), **{k: adr(v) for k, v in arr.items()})
     if pred is not None:
-        arr["pred"] = (C.c_void_p * max(n - 1, 1))(*[None if p is None else C.addressof(p) for p in pred[:n - 1]])
+        arr["pred"] = (C.c_void_p * max(n - 1, 1))(*[None if p is None else C.addressof(p) for p in pred])
         e.pred = adr(arr["pred"])
     e._keep = (arr, X, labels, list(H), list(G), halo, list(W), list(b), list(gW), list(gb), None if pred is None else list(pred), loss_sum)
     return e

@@ -113,6 +113,12 @@ class SatEpoch:
             self._epoch_key = key
         return self._epoch_buf
 
+    def _step_flag(self, W, b, lr) -> int:
+        if lr is None:
+            return 0
+        assert len(W) == len(b) == self.L and all(x is not None for x in b), "a parameter step needs a weight and a bias per layer"
+        return B.SAT_EPOCH_STEP
+
     def _forward_backward(self, m: int, W, b, pred, accumulate: int, reuse_state: int, grad_history: bool = False):
         """Forward and backward of one partition (or all) without the commit; accumulate and reuse_state: it is not the first one."""
         assert bool(accumulate) == bool(reuse_state)
@@ -154,8 +160,9 @@ class SatEpoch:
         grad_history: back-propagate with the stale-gradient term (gradient-side history of the previous epoch)."""
         flags = B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0
         if pred_lr is None or pred is None:
-            flags |= B.SAT_EPOCH_COMMIT | (B.SAT_EPOCH_STEP if lr is not None else 0)
-            B.sat_epoch(self.ctx, self._described(W, b, pred), None, flags, lr or 0.0)
+            flags |= B.SAT_EPOCH_COMMIT
+            buffers = self._described(W, b, pred)
+            B.sat_epoch(self.ctx, buffers, None, flags | self._step_flag(W, b, lr), lr or 0.0)
             return
         self._forward_backward(B.SAT_ALL_PARTS, W, b, pred, 0, 0, grad_history)
         self.pred_update(pred, pred_lr)
@@ -165,8 +172,9 @@ class SatEpoch:
 
     def step_per_partition(self, W, b, pred, order=None, lr: float | None = None, grad_history: bool = False):
         """Same epoch, one partition at a time (the LSTM state table is computed by the first call of every layer)."""
-        flags = B.SAT_EPOCH_COMMIT | (B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0) | (B.SAT_EPOCH_STEP if lr is not None else 0)
-        B.sat_epoch(self.ctx, self._described(W, b, pred), order if order is not None else range(self.M), flags, lr or 0.0)
+        buffers = self._described(W, b, pred)
+        flags = B.SAT_EPOCH_COMMIT | (B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0) | self._step_flag(W, b, lr)
+        B.sat_epoch(self.ctx, buffers, order if order is not None else range(self.M), flags, lr or 0.0)
 
     # ---- graph-attention backbone ---------------------------------------------------
     def step_gat(self, params, pred, lr: float | None = None):

@@ -389,3 +389,29 @@ def test_replaced_buffers_are_the_ones_that_count(B):
         assert all(torch.equal(x, y) for x, y in zip(again(), got))
     finally:
         ep.close()
+
+
+def test_lists_of_the_wrong_length(B):
+    """A list without an entry for every layer is refused before anything runs; entries behind the last layer are not looked at."""
+    import torch
+    wl = make_workload("tiny")
+    ep, P, _, _ = _setup(B, wl)
+    try:
+        preds = pred_to_device(wl.pred, B, 0)
+        W, b = [dev(w) for w in wl.W], [dev(x) for x in wl.b]
+        ep.step(W, b, preds)
+        kept, state = [t.clone() for t in ep.H[1:] + ep.gW], B.sat_cache_state(ep.ctx)
+        for args in ((W[:-1], b, preds), (W, b[:-1], preds), (W, b, preds[:-1]), (W[:-1], b[:-1], preds), (W, b, [])):
+            with pytest.raises(IndexError):
+                ep.step(*args)
+            with pytest.raises(IndexError):
+                ep.step_per_partition(*args, lr=0.1)
+        for args in ((W + W[:1], b + b[:1], preds), (W, b[:-1] + [None], preds)):      # a parameter step takes all of what it is given
+            with pytest.raises(AssertionError):
+                ep.step(*args, lr=0.1)
+        assert all(torch.equal(x, y) for x, y in zip(ep.H[1:] + ep.gW, kept)) and B.sat_cache_state(ep.ctx) == state
+        ep.step(W + W[:1], b + b[:1], list(preds) + [None])
+        assert B.sat_cache_state(ep.ctx)[0] == (state[0] + 1) % (wl.tau + 1)
+        B.sat_sync_status(ep.ctx)
+    finally:
+        ep.close()
