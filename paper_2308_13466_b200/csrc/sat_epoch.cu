@@ -45,16 +45,41 @@ static sat_status epoch_pass(sat_ctx *ctx, const sat_epoch_buffers *e, int32_t p
     return SAT_OK;
 }
 
-extern "C" sat_status sat_epoch(sat_ctx *ctx, const sat_epoch_buffers *e, const int32_t *order, int32_t n_order, int flags, float lr)
+// What the calls of a pass would refuse, before the first of them has written anything.
+static sat_status epoch_check(sat_ctx *ctx, const sat_epoch_buffers *e, const int32_t *order, int32_t n_order, int flags)
 {
-    CHECK_CTX(ctx);
     if (!e || e->n_layers < 1 || e->n_layers > SAT_MAX_LAYERS || !e->dims || !e->x || !e->labels || !e->h || !e->ld_h || !e->g || !e->ld_g || !e->w || !e->b ||
         !e->gw || !e->gb || (n_order != 0 && !order) || n_order < 0 || (flags & ~(SAT_EPOCH_GRAD_HISTORY | SAT_EPOCH_COMMIT | SAT_EPOCH_STEP | SAT_EPOCH_CONTINUE)))
         return sat_fail(ctx, SAT_EINVAL, "sat_epoch: incomplete description or unknown flags");
-    for (int32_t l = 0; l < e->n_layers; ++l) {
+    PartView v;
+    for (int32_t i = 0; i < (n_order > 0 ? n_order : 1); ++i) SAT_TRY(sat_part_view(ctx, n_order > 0 ? order[i] : (int32_t)SAT_ALL_PARTS, &v));
+    const int32_t L = e->n_layers;
+    if (e->loss_kind != SAT_LOSS_SOFTMAX_CE && e->loss_kind != SAT_LOSS_SIGMOID_BCE) return sat_fail(ctx, SAT_EINVAL, "sat_epoch: unknown loss");
+    if ((L > 1 || (flags & SAT_EPOCH_COMMIT)) && !ctx->cache_ok) return sat_fail(ctx, SAT_ESTATE, "sat_epoch: call sat_cache_init first");
+    if (e->dims[0] <= 0 || !ok_ld(e->ld_x, e->dims[0]) || !aligned16(e->x)) return sat_fail(ctx, SAT_EINVAL, "sat_epoch: misaligned x or bad leading dimension");
+    for (int32_t l = 0; l < L; ++l) {
+        const int32_t d = e->dims[l + 1];
         if (!e->w[l] || !e->gw[l] || !e->h[l] || !e->g[l]) return sat_fail(ctx, SAT_EINVAL, "sat_epoch: null array of layer %d", l + 1);
-        if (l > 0 && e->pred && e->pred[l - 1] && !e->halo && ctx->nb > 0) return sat_fail(ctx, SAT_EINVAL, "sat_epoch: no room for the predicted rows");
+        if (d <= 0 || !ok_ld(e->ld_h[l], d) || !ok_ld(e->ld_g[l], d) || !aligned16(e->h[l]) || !aligned16(e->g[l]))
+            return sat_fail(ctx, SAT_EINVAL, "sat_epoch: misaligned rows or bad leading dimension of layer %d", l + 1);
+        if (l + 1 == L) break;
+        if (l >= ctx->n_cached || ctx->cache[l].width != d) return sat_fail(ctx, SAT_EINVAL, "sat_epoch: layer %d is not cached at width %d", l + 1, d);
+        const sat_pred_params *p = e->pred ? e->pred[l] : nullptr;
+        if (!p) continue;
+        if (p->h <= 0 || (p->h & 3) || !p->Wx || !p->Uh || !p->b || !p->Wg || !p->bg || (p->cell != SAT_CELL_LSTM && p->cell != SAT_CELL_GRU))
+            return sat_fail(ctx, SAT_EINVAL, "sat_epoch: bad predictor of layer %d", l + 1);
+        if ((flags & SAT_EPOCH_CONTINUE) && !(order && n_order == 0) && (!ctx->cache[l].S_valid || ctx->cache[l].S_h != p->h))
+            return sat_fail(ctx, SAT_ESTATE, "sat_epoch: no state table of layer %d to go on with", l + 1);
+        if (ctx->nb > 0 && (!e->halo || !ok_ld(e->ld_halo, d) || !aligned16(e->halo)))
+            return sat_fail(ctx, SAT_EINVAL, "sat_epoch: no room for the predicted rows of layer %d", l + 1);
     }
+    return SAT_OK;
+}
+
+extern "C" sat_status sat_epoch(sat_ctx *ctx, const sat_epoch_buffers *e, const int32_t *order, int32_t n_order, int flags, float lr)
+{
+    CHECK_CTX(ctx);
+    SAT_TRY(epoch_check(ctx, e, order, n_order, flags));
     const bool begin = !(flags & SAT_EPOCH_CONTINUE);
     for (int32_t i = 0; i < (order ? n_order : 1); ++i)
         SAT_TRY(epoch_pass(ctx, e, order ? order[i] : (int32_t)SAT_ALL_PARTS, i == 0 && begin, flags & SAT_EPOCH_GRAD_HISTORY));

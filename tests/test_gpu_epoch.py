@@ -415,3 +415,85 @@ def test_lists_of_the_wrong_length(B):
         B.sat_sync_status(ep.ctx)
     finally:
         ep.close()
+
+
+def test_epoch_call_refuses_before_it_writes(B):
+    """Bad descriptions, orders and states of sat_epoch: an error, and not an output, a snapshot or a launch."""
+    import ctypes
+    import torch
+    wl = make_workload("tiny")
+    ep, P, _, _ = _setup(B, wl)
+    try:
+        preds = pred_to_device(wl.pred, B, 0)
+        W, b = [dev(w) for w in wl.W], [dev(x) for x in wl.b]
+        ep.step(W, b, preds)
+        outs = ep.H[1:] + ep.G[1:] + ep.gW + ep.gb + [ep.loss_sum, ep.halo]
+        kept, state = [t.clone() for t in outs], (B.sat_cache_state(ep.ctx), B.sat_launch_count(ep.ctx))
+        L = wl.L
+        ints, ptrs = ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_void_p)
+
+        def changed(field, index, value, kind):
+            e = B.make_epoch_buffers(ep.dims, ep.X, ep.labels, B.SAT_LOSS_SOFTMAX_CE, ep.H[1:], ep.G[1:], ep.halo, W, b, ep.gW, ep.gb, preds, ep.loss_sum)
+            if index is None:
+                setattr(e, field, value)
+            else:
+                ctypes.cast(getattr(e, field), kind)[index] = value
+            return e
+
+        wide = B.make_pred_params(*(torch.zeros(s, device="cuda") for s in ((wl.dims[1], 24), (6, 24), (24,), (6, wl.dims[1]), (wl.dims[1],))), 6)   # h = 6
+        good = changed("n_layers", None, L, None)
+        cases = [(changed("n_layers", None, 0, None), None, B.SAT_EINVAL), (changed("n_layers", None, 99, None), None, B.SAT_EINVAL),
+                 (changed("x", None, None, None), None, B.SAT_EINVAL), (changed("x", None, ep.X.data_ptr() + 4, None), None, B.SAT_EINVAL),
+                 (changed("ld_x", None, wl.dims[0] + 1, None), None, B.SAT_EINVAL), (changed("loss_kind", None, 7, None), None, B.SAT_EINVAL),
+                 (changed("labels", None, None, None), None, B.SAT_EINVAL), (changed("halo", None, None, None), None, B.SAT_EINVAL),
+                 (changed("ld_halo", None, 4, None), None, B.SAT_EINVAL), (changed("dims", 1, wl.dims[1] - 4, ints), None, B.SAT_EINVAL),
+                 (changed("pred", L - 2, ctypes.addressof(wide), ptrs), None, B.SAT_EINVAL), (good, [0, wl.M], B.SAT_EINVAL), (good, [0, -2], B.SAT_EINVAL)]
+        cases += [(changed(f, L - 1, None, ptrs), None, B.SAT_EINVAL) for f in ("h", "g", "w", "gw")]
+        cases += [(changed(f, L - 1, getattr(ep, f.upper())[L].data_ptr() + 4, ptrs), None, B.SAT_EINVAL) for f in ("h", "g")]
+        cases += [(changed(f, L - 1, 1, ints), None, B.SAT_EINVAL) for f in ("ld_h", "ld_g")]
+        for e, order, status in cases:
+            with pytest.raises(B.SatError) as ei:
+                B.sat_epoch(ep.ctx, e, order)
+            assert ei.value.status == status
+        for flags, status in ((64, B.SAT_EINVAL), (B.SAT_EPOCH_CONTINUE, B.SAT_ESTATE)):      # after a commit there is no state table
+            with pytest.raises(B.SatError) as ei:
+                B.sat_epoch(ep.ctx, good, [0], flags)
+            assert ei.value.status == status
+        assert all(torch.equal(x, y) for x, y in zip(outs, kept))
+        assert (B.sat_cache_state(ep.ctx), B.sat_launch_count(ep.ctx)) == state
+        fresh = B.sat_create(0, 0)
+        try:
+            with pytest.raises(B.SatError) as ei:
+                B.sat_epoch(fresh, good)
+            assert ei.value.status == B.SAT_ESTATE
+        finally:
+            B.sat_destroy(fresh)
+    finally:
+        ep.close()
+
+
+def test_an_epoch_in_several_calls(B):
+    """SAT_EPOCH_CONTINUE: the partitions of an order spread over calls give the bits of the one call."""
+    import torch
+    wl = make_workload("tiny")
+    got = []
+    for split in (False, True):
+        ep, P, _, _ = _setup(B, wl)
+        try:
+            preds = pred_to_device(wl.pred, B, 0)
+            W, b = [dev(w) for w in wl.W], [dev(x) for x in wl.b]
+            for _ in range(3):
+                if split:
+                    e = ep._described(W, b, preds)
+                    B.sat_epoch(ep.ctx, e, [1, 0], 0)
+                    B.sat_epoch(ep.ctx, e, [], B.SAT_EPOCH_CONTINUE)
+                    for m in range(2, wl.M):
+                        B.sat_epoch(ep.ctx, e, [m], B.SAT_EPOCH_CONTINUE)
+                    B.sat_epoch(ep.ctx, e, [], B.SAT_EPOCH_CONTINUE | B.SAT_EPOCH_COMMIT | B.SAT_EPOCH_STEP, 0.1)
+                else:
+                    ep.step_per_partition(W, b, preds, order=[1, 0] + list(range(2, wl.M)), lr=0.1)
+            B.sat_sync_status(ep.ctx)
+            got.append([t.clone() for t in ep.H[1:] + ep.gW + ep.gb + W + b + [ep.loss_sum]])
+        finally:
+            ep.close()
+    assert all(torch.equal(x, y) for x, y in zip(*got))
