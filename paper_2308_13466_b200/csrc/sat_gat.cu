@@ -173,7 +173,7 @@ k_gat_alpha(const int64_t *__restrict__ lrowptr, const int32_t *__restrict__ len
 // The conversion instruction runs at 16 lanes per clock and SM, 256 of them per entry at d = 256 (392 us at 2.6 M entries).  gat_scaled
 // builds a double from the bits instead: sign, exponent and fraction of x in their places of the double without moving the exponent's
 // bias are exactly 2^-896 x, zeros and subnormals included.  D is scaled by 2^800 (no overflow for any float) and the sum by 2^96,
-// both exact.  (Non-finite z give a finite product here; their softmax weights, which multiply it, are not finite.)
+// both exact.  Non-finite z give a finite product here: k_gat_rows takes care of those (gat_not_finite).
 __device__ __forceinline__ double gat_scaled(float x)
 {
     const int b = __float_as_int(x);
@@ -231,23 +231,38 @@ k_gat_dots(const int4 *__restrict__ items, int32_t n_items, const int32_t *__res
     }
 }
 
+// The dot product of a z row that holds an infinity or a NaN is not a number, whatever D is.  Its score is not finite then, so finite scores
+// settle it; the others are rare and have their row looked at (a score may overflow over a finite row).  This matters where the score is
+// minus infinity, and alpha zero: anything else makes alpha a NaN by itself.
+__device__ __forceinline__ bool gat_not_finite(float score, const float *__restrict__ z, int32_t d)
+{
+    if (isfinite(score)) return false;
+    for (int32_t k = 0; k < d; ++k)
+        if (!isfinite(z[k])) return true;
+    return false;
+}
+
 // per row v: t_v = sum alpha dot / sum alpha and ds_dst[v]; per entry, over the dot product: dpre = alpha slope (dot - t_v)
 // (the sums in double and divided by sum alpha: the fp32 weights sum to 1 + eps, and ds_dst, exactly zero where all slopes agree,
 // would inherit -eps t_v; dpre stays in double until its column is summed, the dpre of a column cancel as well)
 template <int T>
 __device__ __forceinline__ void gat_row(int tid, int64_t e0, int64_t e1, float sd, const int2 *__restrict__ ent, int32_t n,
-                                        const float *__restrict__ s_in, const float *__restrict__ s_halo, double *__restrict__ dots,
+                                        const float *__restrict__ s_in, const float *__restrict__ s_halo, const float *__restrict__ z_in,
+                                        const float *__restrict__ z_halo, int64_t ld_z, int32_t d, double *__restrict__ dots,
                                         float *__restrict__ ds_dst, double *sh)
 {
-    auto slope = [&](int32_t c) { return sd + (c < n ? s_in[c] : s_halo[c - n]) > 0.f ? 1.f : GAT_SLOPE; };
+    auto score = [&](int32_t c) { return c < n ? s_in[c] : s_halo[c - n]; };
+    auto slope = [&](float s) { return sd + s > 0.f ? 1.f : GAT_SLOPE; };
     const int64_t ef = e0 + tid;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, p_first = 0.0;
     float as_first = 0.f;
 #pragma unroll 4
     for (int64_t e = ef; e < e1; e += T) {
         const int2 q = ent[e];
-        const float al = __int_as_float(q.y), sl = slope(q.x);
-        const double p = dots[e], as = (double)al * (double)sl;
+        const float al = __int_as_float(q.y), s = score(q.x), sl = slope(s);
+        const double as = (double)al * (double)sl;
+        double p = dots[e];
+        if (gat_not_finite(s, q.x < n ? z_in + q.x * ld_z : z_halo + (q.x - n) * ld_z, d)) p = __longlong_as_double(0x7ff8000000000000ll);
         a0 += (double)al;
         a1 += (double)al * p;
         a2 += as * p;
@@ -267,20 +282,20 @@ __device__ __forceinline__ void gat_row(int tid, int64_t e0, int64_t e1, float s
 #pragma unroll 4
     for (int64_t e = ef + T; e < e1; e += T) {
         const int2 q = ent[e];
-        dots[e] = (double)(__int_as_float(q.y) * slope(q.x)) * (dots[e] - t);
+        dots[e] = (double)(__int_as_float(q.y) * slope(score(q.x))) * (dots[e] - t);   // (t is a NaN where a product is)
     }
 }
 
 __global__ void __launch_bounds__(256)
 k_gat_rows(const int64_t *__restrict__ lrowptr, const int2 *__restrict__ ent, int32_t n, int32_t row0, int32_t n_rows, const int32_t *__restrict__ long_rows,
-           int32_t n_long, const float *__restrict__ s_in, const float *__restrict__ s_halo, const float *__restrict__ s_dst, double *dots,
-           float *__restrict__ ds_dst)
+           int32_t n_long, const float *__restrict__ s_in, const float *__restrict__ s_halo, const float *__restrict__ s_dst,
+           const float *__restrict__ z_in, const float *__restrict__ z_halo, int64_t ld_z, int32_t d, double *dots, float *__restrict__ ds_dst)
 {
     sat_grid_wait();
     __shared__ double sh[8];
     if ((int32_t)blockIdx.x < n_long) {
         const int32_t row = long_rows[blockIdx.x];
-        gat_row<256>(threadIdx.x, lrowptr[row], lrowptr[row + 1], s_dst[row], ent, n, s_in, s_halo, dots, ds_dst + row, sh);
+        gat_row<256>(threadIdx.x, lrowptr[row], lrowptr[row + 1], s_dst[row], ent, n, s_in, s_halo, z_in, z_halo, ld_z, d, dots, ds_dst + row, sh);
         return;
     }
     const int64_t w = ((int64_t)(blockIdx.x - n_long) * 256 + threadIdx.x) / GAT_TEAM;
@@ -288,7 +303,7 @@ k_gat_rows(const int64_t *__restrict__ lrowptr, const int2 *__restrict__ ent, in
     const int32_t row = row0 + (int32_t)w;
     const int64_t e0 = lrowptr[row], e1 = lrowptr[row + 1];
     if (e1 - e0 > GAT_LONG) return;
-    gat_row<GAT_TEAM>(threadIdx.x & (GAT_TEAM - 1), e0, e1, s_dst[row], ent, n, s_in, s_halo, dots, ds_dst + row, sh);
+    gat_row<GAT_TEAM>(threadIdx.x & (GAT_TEAM - 1), e0, e1, s_dst[row], ent, n, s_in, s_halo, z_in, z_halo, ld_z, d, dots, ds_dst + row, sh);
 }
 
 // column side of node u: its entries are the mirror images map[e] of row entries (v, u); ent_out[e] = {v, alpha_vu}, ds_src[u] = sum dpre_vu
@@ -687,7 +702,7 @@ extern "C" sat_status sat_gat_bwd(sat_ctx *ctx, int32_t part, int32_t layer, con
         const int64_t l0 = ctx->h_gat_long_off[v.p0], n_long = ctx->h_gat_long_off[v.p1] - l0;
         const unsigned grid = (unsigned)(n_long + cdiv64((int64_t)v.n_rows * GAT_TEAM, 256));
         sat_pdl(ctx->stream, k_gat_rows, grid, 256, 0)(ctx->lrowptr, (const int2 *)G.ent.p, ctx->n, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, s_in,
-                                                  s_halo, s_dst, dots_b, ds_dst_b);
+                                                  s_halo, s_dst, z_in, z_halo, ld_z, d_out, dots_b, ds_dst_b);
         SAT_LAUNCHED(ctx);
         sat_pdl(ctx->stream, k_gat_cols, grid, 256, 0)(ctx->lrowptr, ctx->inner_cnt, v.row0, v.n_rows, ctx->gat_long + l0, (int32_t)n_long, ctx->lenc,
                                                   ctx->gat_rev, (const int2 *)G.ent.p, dots_b, ent_in_b, ds_in_b);

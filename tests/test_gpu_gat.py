@@ -224,3 +224,41 @@ def test_score_gradients_of_columns_that_cancel(B, M):
     pairs = (z - np.repeat(z.reshape(-1, 4).mean(1), 4)).reshape(-1, 4, 1) * c * g.reshape(-1, 1, 2, 2).sum(3)   # [block, u, pair]
     terms = (pairs * z.reshape(-1, 4, 1)) if M > 1 else (pairs.sum(2, keepdims=True) * z.reshape(-1, 4, 1))
     assert abs(got - terms.sum()) <= (2 * n + 4) * 2.0 ** -24 * np.abs(terms).sum()
+
+
+@pytest.mark.parametrize("finite", [False, True])
+@pytest.mark.parametrize("M", [1, 2])
+def test_values_that_are_not_finite_reach_the_gradients(B, M, finite):
+    """Complete graphs of four nodes; one node has a score of minus infinity, so its neighbours give it the weight 0.  Where its z is infinite
+    (h overflows in the product), 0 times infinity is a NaN in every row of that block, also behind a ReLU that stopped it in the forward pass;
+    where only the score overflows, all gradients stay finite.  Other blocks are untouched."""
+    import scipy.sparse as sp
+    blocks, d = 4, 4
+    n = 4 * blocks
+    A = sp.kron(sp.identity(blocks), np.ones((4, 4)) - np.eye(4)).tocsr()
+    A.eliminate_zeros()
+    rng = np.random.default_rng(5)
+    X = np.abs(rng.standard_normal((n, d))).astype(np.float32)
+    G = rng.standard_normal((n, d)).astype(np.float32)
+    part = (np.arange(n) // 2 % M).astype(np.int32)
+    perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+    got = []
+    for bad in (False, True):
+        if bad:
+            X[0, 0] = -3e38
+        ctx = B.sat_create(0, 0)
+        try:
+            B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+            B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+            halo = np.concatenate([B.sat_part_lists(ctx, m)["halo_gid"] for m in range(M)])
+            h_in, h_halo, out, g_in = dev2d(X[perm]), dev2d(X[halo]) if M > 1 else None, empty2d(n, d), empty2d(n, d)
+            W, a_src, a_dst = dev(np.diag([1.0 if finite else 2.0, 1, 1, 1]).astype(np.float32)), dev(np.array([2, 0, 0, 0], np.float32)), dev(np.zeros(d, np.float32))
+            gW, gas, gad, gb = dev(np.zeros((d, d), np.float32)), dev(np.zeros(d, np.float32)), dev(np.zeros(d, np.float32)), dev(np.zeros(d, np.float32))
+            B.sat_gat_fwd(ctx, B.SAT_ALL_PARTS, 1, h_in, h_halo, W, a_src, a_dst, None, B.SAT_ACT_RELU, out)
+            B.sat_gat_bwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(G[perm]), out, h_in, h_halo, W, a_src, a_dst, gW, gas, gad, gb, 0, g_in)
+            B.sat_sync_status(ctx)
+            got.append(g_in.cpu().numpy()[np.argsort(perm)])
+        finally:
+            B.sat_destroy(ctx)
+    assert np.isfinite(got[0]).all()
+    assert (np.isfinite if finite else np.isnan)(got[1][:4]).all() and np.array_equal(got[1][4:], got[0][4:])
