@@ -271,7 +271,7 @@ k_codec_decode(const uint8_t *__restrict__ in, int64_t in_bytes, const int64_t *
     uint8_t *win = wins[threadIdx.x >> 5] + 16;
     uint16_t *list = lists[threadIdx.x >> 5];
     float *row = x + r * ld;
-    // windows start at 4-byte aligned addresses; bytes outside the row that share an aligned word with bytes of the row are masked
+    // windows start at 4-byte aligned addresses; a word that lies partly outside the row is put together from the row's own bytes
     const int64_t a0 = b0 - (int64_t)((uintptr_t)(in + b0) & 3u);
     const float inv32 = 1.f / scale32;
     int64_t q_run = 0;
@@ -284,16 +284,19 @@ k_codec_decode(const uint8_t *__restrict__ in, int64_t in_bytes, const int64_t *
 #pragma unroll
         for (int k = 0; k < CODEC_LANE / 4; ++k) {
             const int32_t p = CODEC_LANE * lane + 4 * k;
-            raw[k] = p < n_in ? *reinterpret_cast<const uint32_t *>(src + p) : 0x3f3f3f3fu;
             // bit 7 of each byte: 63 <= byte, byte <= 126, byte < 95 (a terminator).  Bytes above 190 carry into their neighbour, but
             // they are outside the alphabet themselves and flag the row.
             uint32_t inside = 0x80808080u;
-            if (p < head || p + 3 >= n_in) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (p + i < head || p + i >= n_in) inside &= ~(0x80u << (8 * i));
-                const uint32_t m = (inside >> 7) * 0xffu;
-                raw[k] = (raw[k] & m) | (0x3f3f3f3fu & ~m);   // whatever lies outside: no borrow into the row's bytes below
+            if (p >= head && p + 3 < n_in) {
+                raw[k] = *reinterpret_cast<const uint32_t *>(src + p);
+            } else {
+                raw[k] = 0x3f3f3f3fu;   // outside: no borrow into the row's bytes when 63 is subtracted
+                inside = 0;
+#pragma unroll 1
+                for (int i = max(head - p, 0); i < min(n_in - p, 4); ++i) {
+                    raw[k] ^= (0x3fu ^ (uint32_t)src[p + i]) << (8 * i);
+                    inside |= 0x80u << (8 * i);
+                }
             }
             const uint32_t alpha = (raw[k] + 0x41414141u) & ~(raw[k] + 0x01010101u);
             if ((alpha & inside) != inside) bad = true;

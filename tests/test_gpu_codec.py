@@ -167,3 +167,23 @@ def test_requantised_ring_snapshot(B):
             B.sat_cache_requantise(ep.ctx, 1, wl.tau, 3)                # not a committed snapshot
     finally:
         ep.close()
+
+
+@pytest.mark.parametrize("start", [0, 1, 2, 3])
+@pytest.mark.parametrize("rows,d", [(1, 1), (7, 1), (9, 3), (5, 130), (3, 700)])
+def test_decoding_inside_a_larger_buffer(B, ctx, start, rows, d):
+    """Encoded rows at any byte of a buffer, between bytes that are none of theirs (continuation bytes, bytes outside the alphabet): only the
+    rows' own bytes count, whatever word they share."""
+    import torch
+    x = (np.random.default_rng(d + start).standard_normal((rows, d)) * 20).astype(np.float32)
+    data_o, off_o = orc.codec_encode(x, 3)
+    total = int(off_o[-1])
+    want = orc.codec_decode(data_o, off_o, d, 3)
+    for around in (0x00, 0x3e, 0x5f, 0x7e, 0x7f, 0xff):
+        buf = torch.full((16 + total + 16,), around, dtype=torch.uint8, device="cuda")
+        code = buf[16 + start - 4:16 + start - 4 + total]
+        code.copy_(torch.from_numpy(data_o))
+        back = torch.zeros((rows, d), dtype=torch.float32, device="cuda")
+        B.sat_codec_decode(ctx, code, torch.from_numpy(off_o.astype(np.int64)).cuda(), 3, back)
+        B.sat_sync_status(ctx)
+        assert np.array_equal(back.cpu().numpy(), want)
