@@ -149,6 +149,7 @@ k_codec_encode(const float *__restrict__ x, int64_t ld, int64_t rows, int32_t d,
     base -= skip;
     int64_t carry = 0;
     if (lane == 0) buf16[0] = make_uint4(0, 0, 0, 0);
+    __syncwarp();   // a chunk of large values writes its bytes without another wait
     for (int32_t j0 = 0; j0 < d; j0 += CODEC_CHUNK) {
         const int32_t cnt = d - j0 < CODEC_CHUNK ? d - j0 : CODEC_CHUNK, left = cnt - 4 * lane;
         float v[4];
