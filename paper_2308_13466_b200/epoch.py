@@ -50,7 +50,8 @@ class SatEpoch:
         dev = self.device
         self.H = [None] + [_buf(self.n, d, dev) for d in self.dims[1:]]          # H[l], l = 1..L (partition-major rows)
         self.G = [None] + [_buf(self.n, d, dev) for d in self.dims[1:]]          # gradient w.r.t. H[l]
-        self.halo = _buf(self.nb, max(self.dims[1:-1] or [1]), dev)               # predicted halo input of the running layer (layers >= 2)
+        self._halo = _buf(self.nb, max(self.dims[1:-1] or [1]), dev)              # predicted halo input of the running layer (layers >= 2)
+        self._halo_state = None                                                   # ring state whose plain rows `halo` is still to be given
         self.X_in = None                                                          # partition-major copy of the features (made on demand)
         self.gW = [torch.zeros((self.dims[l], self.dims[l + 1]), dtype=torch.float32, device=dev) for l in range(self.L)]
         self.gb = [torch.zeros(self.dims[l + 1], dtype=torch.float32, device=dev) for l in range(self.L)]
@@ -65,7 +66,7 @@ class SatEpoch:
         if self.ctx is not None:
             B.sat_destroy(self.ctx)
             self.ctx = None
-        self.H = self.G = self.halo = self.X_in = self.X = self.labels = self._epoch_key = self._epoch_buf = None
+        self.H = self.G = self._halo = self._halo_state = self.X_in = self.X = self.labels = self._epoch_key = self._epoch_buf = None
         if hasattr(self, "gat_halo"):
             self.gat_halo = None
 
@@ -85,9 +86,27 @@ class SatEpoch:
             B.sat_gather_rows(self.ctx, B.SAT_ALL_PARTS, B.SAT_ROWS_INNER, self.X, self.X_in)
         return self.X_in
 
+    @property
+    def halo(self) -> torch.Tensor:
+        """Out-of-subgraph rows that the last layer of the most recent epoch used.  A layer without a predictor reads the plain
+        historical embeddings from the ring itself; their copy is made here, when it is first asked for, from the snapshot that was
+        the newest one then (it stays in the ring until the next epoch); a view kept from an earlier epoch does not follow."""
+        if self._halo_state is not None:
+            now, used = B.sat_cache_state(self.ctx), self._halo_state
+            B.sat_cache_set_state(self.ctx, *used)
+            try:
+                B.sat_predict(self.ctx, self.L - 1, B.SAT_ALL_PARTS, None, 0, self._halo[:, :self.dims[self.L - 1]])
+            finally:
+                B.sat_cache_set_state(self.ctx, *now)
+            self._halo_state = None
+        return self._halo
+
+    @halo.setter
+    def halo(self, t: torch.Tensor):
+        self._halo, self._halo_state = t, None
+
     def halo_view(self, l: int, m: int = B.SAT_ALL_PARTS):
-        """Halo rows of the input of GNN layer l + 1 (predicted embeddings of cached layer l), all partitions or one.  (Plain
-        historical embeddings are read from the ring by the layer and not copied here.)"""
+        """Halo rows of the input of GNN layer l + 1 (predicted or plain historical embeddings of cached layer l), all partitions or one."""
         d = self.dims[l]
         if m == B.SAT_ALL_PARTS:
             return self.halo[:, :d]
@@ -102,28 +121,37 @@ class SatEpoch:
     def _described(self, W, b, pred) -> B.sat_epoch_buffers:
         """The buffers of an epoch as the library takes them; made anew when the place, shape or strides of any of them (this object's own
         among them) or a predictor is another one."""
-        tensors = (self.X, self.labels, *self.H[1:], *self.G[1:], self.halo, *W, *b, *self.gW, *self.gb, self.loss_sum)
+        tensors = (self.X, self.labels, *self.H[1:], *self.G[1:], self._halo, *W, *b, *self.gW, *self.gb, self.loss_sum)
         key = [t if t is None else (t.data_ptr(), t.shape, t.stride()) for t in tensors]
         # predictors are read through their own structures at every call: the same structure is all that matters
         key += [len(W), len(b), self.loss, pred if pred is None else [None if p is None else id(p) for p in pred]]
         if key != self._epoch_key:
             kind = B.SAT_LOSS_SOFTMAX_CE if self.loss == "ce" else B.SAT_LOSS_SIGMOID_BCE
-            self._epoch_buf = B.make_epoch_buffers(self.dims, self.X, self.labels, kind, self.H[1:], self.G[1:], self.halo, W, b, self.gW, self.gb,
+            self._epoch_buf = B.make_epoch_buffers(self.dims, self.X, self.labels, kind, self.H[1:], self.G[1:], self._halo, W, b, self.gW, self.gb,
                                                    pred, self.loss_sum)
             self._epoch_key = key
         return self._epoch_buf
 
+    def _run(self, W, b, pred, order, flags: int, lr: float = 0.0):
+        buffers = self._described(W, b, pred)
+        plain = self.L > 1 and (pred is None or pred[self.L - 2] is None)
+        state = B.sat_cache_state(self.ctx) if plain else None
+        B.sat_epoch(self.ctx, buffers, order, flags, lr)
+        self._halo_state = state
+
     def _step_flag(self, W, b, lr) -> int:
         if lr is None:
             return 0
-        assert len(W) == len(b) == self.L and all(x is not None for x in b), "a parameter step needs a weight and a bias per layer"
+        if len(W) < self.L or len(b) < self.L:
+            raise IndexError("a weight and a bias per layer")
+        assert len(W) == len(b) == self.L and all(x is not None for x in b), "a parameter step takes one weight and one bias per layer"
         return B.SAT_EPOCH_STEP
 
     def _forward_backward(self, m: int, W, b, pred, accumulate: int, reuse_state: int, grad_history: bool = False):
         """Forward and backward of one partition (or all) without the commit; accumulate and reuse_state: it is not the first one."""
         assert bool(accumulate) == bool(reuse_state)
         flags = (B.SAT_EPOCH_CONTINUE if accumulate else 0) | (B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0)
-        B.sat_epoch(self.ctx, self._described(W, b, pred), None if m == B.SAT_ALL_PARTS else [m], flags)
+        self._run(W, b, pred, None if m == B.SAT_ALL_PARTS else [m], flags)
 
     def pred_update(self, pred, lr: float, max_steps: int = 1, min_gain: float | None = None, row_weight=None):
         """Algorithm 1 "Embedding predictor update", to be called after the pushes of an epoch and before the commit:
@@ -160,9 +188,7 @@ class SatEpoch:
         grad_history: back-propagate with the stale-gradient term (gradient-side history of the previous epoch)."""
         flags = B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0
         if pred_lr is None or pred is None:
-            flags |= B.SAT_EPOCH_COMMIT
-            buffers = self._described(W, b, pred)
-            B.sat_epoch(self.ctx, buffers, None, flags | self._step_flag(W, b, lr), lr or 0.0)
+            self._run(W, b, pred, None, flags | B.SAT_EPOCH_COMMIT | self._step_flag(W, b, lr), lr or 0.0)
             return
         self._forward_backward(B.SAT_ALL_PARTS, W, b, pred, 0, 0, grad_history)
         self.pred_update(pred, pred_lr)
@@ -172,9 +198,8 @@ class SatEpoch:
 
     def step_per_partition(self, W, b, pred, order=None, lr: float | None = None, grad_history: bool = False):
         """Same epoch, one partition at a time (the LSTM state table is computed by the first call of every layer)."""
-        buffers = self._described(W, b, pred)
         flags = B.SAT_EPOCH_COMMIT | (B.SAT_EPOCH_GRAD_HISTORY if grad_history else 0) | self._step_flag(W, b, lr)
-        B.sat_epoch(self.ctx, buffers, order if order is not None else range(self.M), flags, lr or 0.0)
+        self._run(W, b, pred, order if order is not None else range(self.M), flags, lr or 0.0)
 
     # ---- graph-attention backbone ---------------------------------------------------
     def step_gat(self, params, pred, lr: float | None = None):
@@ -186,6 +211,8 @@ class SatEpoch:
         if not hasattr(self, "gat_grads"):
             self.gat_grads = [{k: torch.zeros_like(v) for k, v in p.items()} for p in params]
             self.gat_halo = [_buf(self.nb, self.dims[l], dev) for l in range(L)]       # the pulled embeddings are needed again in the backward
+        if self._halo_state is not None:
+            self.halo       # an earlier epoch's rows, before this one's push may overwrite them
         self.loss_sum.zero_()
         h_in = self.inner_features()
         ins = []

@@ -497,3 +497,38 @@ def test_an_epoch_in_several_calls(B):
         finally:
             ep.close()
     assert all(torch.equal(x, y) for x, y in zip(*got))
+
+
+@pytest.mark.parametrize("tau", [1, 3])
+def test_plain_historical_rows_can_be_looked_at(B, tau):
+    """halo_view after an epoch without a predictor: the rows its last layer used (zeros in the first epoch), also partition by
+    partition and after further calls; sat_staleness takes them as it takes predicted rows; asking changes nothing for the next epoch."""
+    import torch
+    wl = make_workload("odd", tau=tau)
+    got = []
+    for ask in (True, False):
+        ep, P, _, _ = _setup(B, wl)
+        try:
+            L, d = wl.L, wl.dims[wl.L - 1]
+            slots = np.concatenate([B.sat_part_lists(ep.ctx, m)["halo_slot"] for m in range(wl.M)])
+            W, b = [dev(w) for w in wl.W], [dev(x) for x in wl.b]
+            for epoch in range(tau + 3):
+                newest = B.sat_cache_read(ep.ctx, L - 1, 0, ep.n_slots, d) if epoch else np.zeros((ep.n_slots, d), np.float32)
+                ep.halo.fill_(float("nan"))
+                (ep.step if epoch % 2 else ep.step_per_partition)(W, b, None, lr=0.05)
+                if ask:
+                    state = B.sat_cache_state(ep.ctx)
+                    assert np.array_equal(ep.halo_view(L - 1).cpu().numpy(), newest[slots])
+                    assert np.array_equal(ep.halo_view(L - 1, 1).cpu().numpy(), newest[slots[ep.halo_off[1]:ep.halo_off[2]]])
+                    assert B.sat_cache_state(ep.ctx) == state
+                    sq = torch.zeros(1, dtype=torch.float64, device="cuda")
+                    B.sat_staleness(ep.ctx, B.SAT_ALL_PARTS, ep.H[L - 1], ep.halo_view(L - 1), sq)
+                    fresh = np.empty((ep.n_slots, d), np.float32)
+                    fresh[...] = B.sat_cache_read(ep.ctx, L - 1, 0, ep.n_slots, d)
+                    want = ((fresh[slots].astype(np.float64) - newest[slots]) ** 2).sum()
+                    assert abs(float(sq) - want) <= 1e-12 * want
+            B.sat_sync_status(ep.ctx)
+            got.append([t.clone() for t in ep.H[1:] + ep.gW + W])
+        finally:
+            ep.close()
+    assert all(torch.equal(x, y) for x, y in zip(*got))
