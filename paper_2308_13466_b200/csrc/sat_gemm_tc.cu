@@ -248,9 +248,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // A warp's arrival on a barrier that the MMA issuer waits for.  CTAS = 1: every lane arrives.  2: lane 0 does, on the barrier at the same
-// place in CTA 0 of the pair.  What the barrier guards has been performed when the arrive is issued: shared-memory writes by the proxy
-// fence in front of it, TMEM reads by their wait.  (With .release.cluster it also waits for everything else the SM has in flight,
-// 1.4 us: a 179250 x 512 x 512 contraction took 490 us instead of 370.)
+// place in CTA 0 of the pair, without a scope, that is at CTA scope.  An assumption rests on that: that shared-memory writes in front of
+// the proxy fence and TMEM reads in front of their wait are done for the pair's MMAs when the arrival is seen.  The memory model does not
+// say so across two CTAs; it is the form in which CUTLASS's cluster barriers arrive at the other CTA of a pair, and
+// tests/test_gpu_edges.py compares pair launches with single CTAs bit by bit.  (With .release.cluster the arrival also waits for
+// everything else the SM has in flight, 1.4 us: a 179250 x 512 x 512 contraction took 490 us instead of 370.)
 template <int CTAS>
 __device__ __forceinline__ void mbar_arrive_warp(uint64_t *bar, int lane)
 {

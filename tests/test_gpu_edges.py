@@ -433,3 +433,57 @@ def test_bias_gradient_of_many_rows(B, m, n):
         B.sat_destroy(ctx)
     want = 1.0 + (rows - 1) * 2.0 ** -25
     assert float((gb.double() - want).abs().max()) <= 64 * U * want
+
+
+@pytest.mark.parametrize("n,k", [(256, 256), (512, 512), (100, 48), (40, 600)])
+def test_pairs_give_the_bits_of_single_ctas_every_time(B, n, k):
+    """Many tiles per CTA pair, again and again, against the same rows in launches of at most a wave of single CTAs: an order that the pair's
+    barriers fail to keep would show as a tile that differs once in a while."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    step = 128 * (sms // -(-n // 256))
+    m = 6 * step + 77
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    A, W, b = torch.randn((m, k), device="cuda", generator=gen), torch.randn((k, n), device="cuda", generator=gen), torch.randn(n, device="cuda", generator=gen)
+    want, out = empty2d(m, n), empty2d(m, n)
+    ctx = B.sat_create(0, torch.cuda.current_stream().cuda_stream)
+    try:
+        for r in range(0, m, step):
+            B.sat_dense_nn(ctx, A[r:r + step], W, b, want[r:r + step])
+        for _ in range(50):
+            out.fill_(float("nan"))
+            B.sat_dense_nn(ctx, A, W, b, out)
+            assert torch.equal(out, want)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("h", [20, 64])
+def test_lstm_steps_repeat_themselves(B, h):
+    """The state after five steps over cached projections, more than one tile per slot of a CTA pair: the same bits in every run."""
+    n, d, tau = 120000, 32, 5
+    ids = np.arange(n)
+    col = np.sort(np.stack([(ids - 1) % n, (ids + 1) % n], 1), 1).astype(np.int32).ravel()
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(h)
+    rand = lambda *s: torch.randn(s, device="cuda", generator=gen)
+    ctx = B.sat_create(0, torch.cuda.current_stream().cuda_stream)
+    try:
+        B.sat_graph_load(ctx, 2 * np.arange(n + 1, dtype=np.int64), col)
+        B.sat_partition(ctx, 2, B.SAT_PART_GIVEN, (ids % 2).astype(np.int32))       # every node is a boundary node
+        B.sat_cache_init(ctx, [d], tau)
+        out, first = empty2d(n, d), None
+        p = B.make_pred_params(rand(d, 4 * h) / d ** 0.5, rand(h, 4 * h) / h ** 0.5, rand(4 * h), rand(h, d) / h ** 0.5, rand(d), h, 1)
+        for _ in range(tau):
+            B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, rand(n, d))
+            B.sat_cache_commit(ctx)
+            B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, p, 0, out)
+        first = out.clone()
+        for _ in range(50):
+            out.fill_(float("nan"))
+            B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, p, 0, out)
+            assert torch.equal(out, first)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
