@@ -37,7 +37,7 @@ def _propagation(A):
     return sp.diags(dinv) @ (A + sp.identity(A.shape[0])) @ sp.diags(dinv)
 
 
-# degrees around the run lengths (32), the block reduction of many runs (16 x 32) and far above
+# degrees around the run lengths (32; 48 in a list with the longest of these rows) and far above: up to 61 runs, which the last one adds
 HUBS = [29, 30, 31, 32, 33, 62, 64, 100, 500, 510, 520, 1000, 2900]
 
 
@@ -326,7 +326,7 @@ def test_predictor_gradient_over_long_windows(B, tau, h):
 
 
 @pytest.mark.parametrize("parts", [False, True])
-@pytest.mark.parametrize("d_out", [40, 43, 256, 300])                 # one launch per slice of 256 columns; rows of many runs by k_spmm_fixup or their last run
+@pytest.mark.parametrize("d_out", [40, 43, 256, 300])                 # one launch per slice of 256 columns; rows of many runs by their last run
 def test_attention_layer_pushes_its_boundary_rows(B, d_out, parts):
     """SAT_FWD_PUSH of sat_gat_fwd against sat_cache_update: same bits in the ring and in h_out."""
     n, M, d = 3000, 3, 24
@@ -487,3 +487,126 @@ def test_lstm_steps_repeat_themselves(B, h):
         B.sat_sync_status(ctx)
     finally:
         B.sat_destroy(ctx)
+
+
+def _many_runs(kind):
+    """"hub": one row of 9,000 entries in a small list, more runs than the last one adds (64 of at most 128 entries): the block reduction of
+    k_spmm_fixup.  "large": above 2^20 entries, where k_spmm_fixup adds every row of more than one run: ordinary rows of one run of
+    64, rows of 2 to 16 runs by a thread per column, longer ones by a block."""
+    rng = np.random.default_rng(11)
+    if kind == "hub":
+        return _graph([9000, 40, 70], 12000)
+    n = 30000
+    pairs = rng.integers(0, n, (560000, 2))
+    hubs = [np.stack([np.full(deg, i), rng.integers(0, n, deg)], 1) for i, deg in enumerate([20, 30, 90, 200, 500, 900, 1100, 1500, 4000, 25000])]
+    ring = np.stack([np.arange(n), (np.arange(n) + 1) % n], 1)
+    a = np.concatenate([pairs, ring] + hubs)
+    a = a[a[:, 0] != a[:, 1]]
+    m = sp.coo_matrix((np.ones(len(a)), (a[:, 0], a[:, 1])), shape=(n, n))
+    m = ((m + m.T) > 0).astype(np.float64).tocsr()
+    m.sort_indices()
+    return m
+
+
+@pytest.mark.parametrize("kind", ["hub", "large"])
+@pytest.mark.parametrize("d", [40, 43, 260])
+def test_rows_that_the_second_launch_finishes(B, kind, d):
+    """GCN aggregation and the attention layer's forward, push and backward on rows of many runs, against fp64; all partitions at once and
+    one after the other (same bits).  The second launch shows in the launch count: an equal call whose rows are all short has one less."""
+    from tests.gpu_util import assert_close
+    A, k, M = _many_runs(kind), 8, 2
+    n = A.shape[0]
+    if kind == "large":
+        assert A.nnz + n > 2 ** 20
+    rng = np.random.default_rng(d)
+    part = rng.integers(0, M, n).astype(np.int32)
+    perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+    X, G = rng.standard_normal((n, k)).astype(np.float32), rng.standard_normal((n, d)).astype(np.float32)
+    W, a1, a2, b = ((rng.standard_normal(s) * 0.4).astype(np.float32) for s in ((k, d), (d,), (d,), (d,)))
+    Y = rng.standard_normal((n, d)).astype(np.float32)
+    eye = np.eye(d, 4, dtype=np.float32)
+
+    def calls(graph, rows):
+        """Launches of the GCN forward and of the attention layer on the first `rows` nodes of the inputs, and their results."""
+        pt = part[:rows]
+        order = np.concatenate([np.flatnonzero(pt == m) for m in range(M)])
+        ctx = B.sat_create(0, 0)
+        try:
+            B.sat_graph_load(ctx, graph.indptr.astype(np.int64), graph.indices.astype(np.int32))
+            B.sat_partition(ctx, M, B.SAT_PART_GIVEN, pt)
+            B.sat_cache_init(ctx, [d], 2)
+            lists = [B.sat_part_lists(ctx, m) for m in range(M)]
+            halo = np.concatenate([l["halo_gid"] for l in lists])
+            n_in = [len(l["inner_gid"]) for l in lists]
+            n_out = [len(l["halo_gid"]) for l in lists]
+            n_slots = B.sat_slot_map(ctx, rows)[2]
+            agg, h_in, h_halo, g = empty2d(rows, 4), dev2d(X[order]), dev2d(X[halo]), dev2d(G[order])
+            Wd, a1d, a2d, bd = dev(W), dev(a1), dev(a2), dev(b)
+            grads = [torch.empty_like(t) for t in (Wd, a1d, a2d, bd)]
+            out, g_in, got, counts = empty2d(rows, d), empty2d(rows, k), [], []
+            gcn = lambda: B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, dev2d(Y[:rows]), None, dev(eye), None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, agg)
+            fwd = lambda: B.sat_gat_fwd(ctx, B.SAT_ALL_PARTS, 1, h_in, h_halo, Wd, a1d, a2d, bd, B.SAT_ACT_NONE | B.SAT_FWD_PUSH, out)
+            bwd = lambda: B.sat_gat_bwd(ctx, B.SAT_ALL_PARTS, 1, g, None, h_in, h_halo, Wd, a1d, a2d, *grads, 0, g_in)
+            for call in (gcn, fwd, bwd):
+                call()                       # builds the lists
+                at = B.sat_launch_count(ctx)
+                call()
+                counts.append(B.sat_launch_count(ctx) - at)
+            ring = B.sat_cache_read(ctx, 1, -1, n_slots, d)
+            scores = B.sat_gat_scores(ctx, 1, rows, len(halo))
+            got = [t.cpu().numpy() for t in (agg, out, *grads, g_in)]
+            out2, g_in2 = empty2d(rows, d), empty2d(rows, k)
+            r0 = u0 = 0
+            for m in range(M):
+                r1, u1 = r0 + n_in[m], u0 + n_out[m]
+                B.sat_gat_fwd(ctx, m, 1, h_in[r0:r1], h_halo[u0:u1], Wd, a1d, a2d, bd, B.SAT_ACT_NONE | B.SAT_FWD_PUSH, out2[r0:r1])
+                B.sat_gat_bwd(ctx, m, 1, g[r0:r1], None, h_in[r0:r1], h_halo[u0:u1], Wd, a1d, a2d, *grads, 0, g_in2[r0:r1])
+                r0, u0 = r1, u1
+            B.sat_sync_status(ctx)
+            assert np.array_equal(out2.cpu().numpy()[:, :d], got[1][:, :d]) and np.array_equal(g_in2.cpu().numpy()[:, :k], got[6][:, :k])
+            assert np.array_equal(B.sat_cache_read(ctx, 1, -1, n_slots, d), ring)
+            push = np.concatenate([np.stack([l["push_slot"], l["push_local"] + sum(n_in[:m])], 1) for m, l in enumerate(lists)])
+            assert np.array_equal(ring[push[:, 0]], got[1][push[:, 1]][:, :d])
+        finally:
+            B.sat_destroy(ctx)
+        return counts, got, scores, halo
+
+    counts, (agg, out, gW, g1, g2, gb, g_in), (s_src, s_dst, s_halo), halo = calls(A, n)
+    small, *_ = calls(_graph([], 1000), 1000)
+    assert counts[0] == small[0] + 1 and counts[1] == small[1] + 1
+    assert counts[2] >= small[2] + (2 if kind == "large" else 0)     # (the hub's row is half as long in either half of the backward pass)
+    P = _propagation(A)
+    want, mag = (P @ Y.astype(np.float64))[perm][:, :4], (abs(P) @ np.abs(Y.astype(np.float64)))[perm][:, :4]
+    assert (np.abs(agg - want) <= (np.diff(A.indptr).max() + 8) * U * mag).all()
+    # attention in fp64 on the edge list, slopes as the device decided them; a halo copy acts like the node it copies
+    E = (A + sp.identity(n)).tocoo()
+    c = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    v, u = c(E.row.astype(np.int64)), c(E.col.astype(np.int64))
+    by_node = np.empty(n, np.float32), np.empty(n, np.float32)
+    by_node[0][perm], by_node[1][perm] = s_src, s_dst
+    pos = (c(by_node[1])[v] + c(by_node[0])[u]) > 0
+    z, D = c(X).double() @ c(W).double(), c(G).double()
+    pre = (z @ c(a2).double())[v] + (z @ c(a1).double())[u]
+    slope = torch.where(pos, 1.0, float(np.float32(0.2))).double()
+    e = slope * pre
+    zero = lambda *s: torch.zeros(s, dtype=torch.float64, device="cuda")
+    mx = torch.full((n,), -1e300, dtype=torch.float64, device="cuda").scatter_reduce(0, v, e, "amax")
+    x = torch.exp(e - mx[v])
+    al = x / zero(n).index_add(0, v, x)[v]
+    chunks = torch.arange(len(v), device="cuda").split(1 << 18)
+    o, dal, dz, dz_in = zero(n, d), zero(len(v)), zero(n, d), zero(n, d)
+    inner = c(part)[v] == c(part)[u]
+    for i in chunks:
+        o.index_add_(0, v[i], al[i, None] * z[u[i]])
+        dal[i] = (D[v[i]] * z[u[i]]).sum(1)
+        dz.index_add_(0, u[i], al[i, None] * D[v[i]])
+        dz_in.index_add_(0, u[i], (al[i] * inner[i])[:, None] * D[v[i]])
+    t = zero(n).index_add(0, v, al * dal)
+    dpre = al * (dal - t[v]) * slope
+    ds, dd, ds_in = zero(n).index_add(0, u, dpre), zero(n).index_add(0, v, dpre), zero(n).index_add(0, u, dpre * inner)
+    A1, A2 = c(a1).double(), c(a2).double()
+    dz += ds[:, None] * A1 + dd[:, None] * A2
+    dz_in += ds_in[:, None] * A1 + dd[:, None] * A2
+    for what, got, ref in (("out", out[:, :d], (o + c(b).double())[c(perm)]), ("G_W", gW, c(X).double().T @ dz), ("G_a_src", g1, z.T @ ds),
+                           ("G_a_dst", g2, z.T @ dd), ("G_b", gb, D.sum(0)), ("G_in", g_in[:, :k], (dz_in @ c(W).double().T)[c(perm)])):
+        assert_close(got, ref.cpu().numpy(), what)

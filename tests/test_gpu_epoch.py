@@ -487,8 +487,9 @@ def test_an_epoch_in_several_calls(B):
                     e = ep._described(W, b, preds)
                     B.sat_epoch(ep.ctx, e, [1, 0], 0)
                     B.sat_epoch(ep.ctx, e, [], B.SAT_EPOCH_CONTINUE)
-                    for m in range(2, wl.M):
+                    for m in range(2, wl.M - 1):
                         B.sat_epoch(ep.ctx, e, [m], B.SAT_EPOCH_CONTINUE)
+                    ep._forward_backward(wl.M - 1, W, b, preds, 1, 1)
                     B.sat_epoch(ep.ctx, e, [], B.SAT_EPOCH_CONTINUE | B.SAT_EPOCH_COMMIT | B.SAT_EPOCH_STEP, 0.1)
                 else:
                     ep.step_per_partition(W, b, preds, order=[1, 0] + list(range(2, wl.M)), lr=0.1)
