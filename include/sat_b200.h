@@ -320,8 +320,9 @@ sat_status sat_cache_commit(sat_ctx *ctx);
  * The GCN normalisation is not used.  W [d_in x d_out], a_src [d_out], a_dst [d_out], bias [d_out] or NULL: DEVICE, dense.
  * act may carry SAT_FWD_PUSH: the rows of boundary nodes also go to the write buffer of cached layer `layer`, as sat_cache_update
  * with h_out would do (SAT_ESTATE without such a layer, SAT_EINVAL if its width is not d_out).
- * sat_gat_fwd keeps z, the attention scores and the log-sum-exp of every row for sat_gat_bwd (memory: (n + sum_m b_m) *
- * d_out floats per layer, owned by the context).  d_out <= 1024.
+ * sat_gat_fwd keeps z, the attention scores and every entry's column and softmax weight for sat_gat_bwd (memory per layer, owned by the
+ * context: (n + sum_m b_m) * d_out floats, 8 bytes per entry of A + I; and once per partitioning 4 bytes per entry).  sat_gat_bwd
+ * adds scratch of up to 24 bytes per entry and (2 n + sum_m b_m) * d_out floats.  d_out <= 1024.
  * sat_gat_bwd: g_out [n_m x ld_g] gradient w.r.t. h_out; h_out as written by sat_gat_fwd (used for the ReLU mask; may be
  * NULL for SAT_ACT_NONE); h_in / h_halo the same inputs as in the forward call.  The halo embeddings are constants of the
  * epoch, W acts on them as on the inner rows:  g_W [d_in x d_out], g_a_src [d_out], g_a_dst [d_out], g_b [d_out] are

@@ -28,23 +28,6 @@ __device__ __forceinline__ float warp_sum(float x)
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
 }
-__device__ __forceinline__ float warp_max(float x)
-{
-    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
-}
-__device__ __forceinline__ float4 ldz(const float *row, int c4, int d)
-{
-    // the padding columns of the last vector of a row are not data: read them as zero
-    float4 x = *reinterpret_cast<const float4 *>(row + 4 * c4);
-    if (4 * c4 + 3 >= d) {
-        if (4 * c4 + 1 >= d) x.y = 0.f;
-        if (4 * c4 + 2 >= d) x.z = 0.f;
-        x.w = 0.f;
-    }
-    return x;
-}
-__device__ __forceinline__ float dot4(const float4 &a, const float4 &b) { return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w))); }
 __device__ __forceinline__ float lrelu(float x) { return x > 0.f ? x : GAT_SLOPE * x; }
 
 // s_src[r] = a_src . z_r, s_dst[r] = a_dst . z_r (when asked for).  A warp takes four rows: the vectors' elements are loaded once for them and

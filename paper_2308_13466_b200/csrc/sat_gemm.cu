@@ -307,7 +307,7 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
     // Enough row splits for two blocks per SM (one block walking 2,048 rows alone took 168 us, 32 of 64 rows each take 4), and
     // at most TN_ROWS_PER_SPLIT rows in each; a split has at least 4 BK rows, below which its partial sums outweigh its products
     const int64_t r1 = rows > 0 ? rows : 1, tiles = cdiv64(m, BM) * cdiv64(n, BN);
-    int64_t splits = std::max<int64_t>(cdiv64(r1, TN_ROWS_PER_SPLIT), std::min<int64_t>(cdiv64(2 * 148, tiles), cdiv64(r1, 4 * BK)));
+    int64_t splits = std::max<int64_t>(cdiv64(r1, TN_ROWS_PER_SPLIT), std::min<int64_t>(cdiv64(2 * ctx->sms, tiles), cdiv64(r1, 4 * BK)));
     if (splits > 1024) splits = 1024;
     int64_t rows_per_split = cdiv64(cdiv64(r1, splits), BK) * BK;
     splits = cdiv64(r1, rows_per_split);
@@ -469,7 +469,7 @@ static sat_status launch_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_
         attr_set.mark(ctx->device);
     }
     // one wave of row blocks, three per SM; at least four stages each (below that the partial sums outweigh the products)
-    const int64_t yb = cdiv64(m, 64 * TM), want = std::max<int64_t>(1, 3 * 148 / yb);
+    const int64_t yb = cdiv64(m, 64 * TM), want = std::max<int64_t>(1, 3 * ctx->sms / yb);
     const int64_t rpb = std::max<int64_t>(4 * TNN_STAGE, cdiv64(cdiv64(rows > 0 ? rows : 1, want), TNN_STAGE) * TNN_STAGE);
     const int64_t blocks = cdiv64(rows > 0 ? rows : 1, rpb);
     SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)blocks * ((size_t)m * n + n) * sizeof(float)));

@@ -16,6 +16,7 @@
 #include "../../include/sat_b200.h"
 
 #define SAT_MAX_LAYERS 16
+#define SAT_SMS 148           /* multiprocessors of a B200, where no context is at hand to say */
 #define SAT_MAX_PARTS 4096
 #define SAT_HROW_LONG 256  /* rows and halo rows with more entries than this get a thread block in the attention layer */
 
@@ -143,7 +144,7 @@ struct sat_ctx {
     uint64_t prof_mask = ~0ull;  // families that are bracketed while prof_on
     std::vector<ProfRec> prof;
     int device = 0;
-    int sms = 148;           // multiprocessors of the device
+    int sms = SAT_SMS;       // multiprocessors of the device
     cudaStream_t stream = nullptr;
     char err[512] = {0};
     bool cuda_failed = false;
@@ -450,9 +451,10 @@ struct SatPdl {
         cfg.dynamicSmemBytes = smem;
         cfg.stream = stream;
         cfg.attrs = attr;
-        // only grids of at most one wave: the blocks of a longer one that move in early find the SM's shared memory / L1 split as the
-        // running kernel left it and keep it for their whole launch (gathers behind a 200 KB contraction: epochs 3-10 % slower)
-        if ((int64_t)grid.x * grid.y * grid.z * block.x <= 148 * 2048) {
+        // only grids that the SMs' 2,048 threads each could hold at once (up to three waves of kernels with two or three blocks per SM): the
+        // blocks of a longer one that move in early find the SM's shared memory / L1 split as the running kernel left it and keep it for their
+        // whole launch (gathers behind a 200 KB contraction: epochs 3-10 % slower)
+        if ((int64_t)grid.x * grid.y * grid.z * block.x <= SAT_SMS * 2048) {
             attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[n++].val.programmaticStreamSerializationAllowed = 1;
         }

@@ -953,7 +953,7 @@ extern "C" sat_status sat_dense_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_
 // Loss kernels.  The rows go round-robin over the lane groups of at most LOSS_MAX_BLOCKS blocks (one resident wave).  Row losses
 // are summed in double per thread, then per warp, the warps of a block in fixed order, and the last block to finish adds the block
 // partials in fixed order: which rows a thread owns depends on the row count alone, so the total does not depend on scheduling.
-#define LOSS_MAX_BLOCKS (148 * 6)
+#define LOSS_MAX_BLOCKS(ctx) ((ctx)->sms * 6)
 
 __device__ __forceinline__ void loss_finish(double thread_sum, double *__restrict__ block_partial, int *__restrict__ ticket, double *total, int overwrite)
 {
@@ -1124,8 +1124,8 @@ sat_status sat_loss_into(sat_ctx *ctx, int32_t part, int kind, int32_t n_classes
                       (((uintptr_t)labels) & 3u) == 0;
     const int64_t groups = kind == SAT_LOSS_SOFTMAX_CE ? cdiv64(v.n_rows, n_classes <= 128 ? 32 : 8)
                                                        : cdiv64((int64_t)v.n_rows * n_classes, vec4 ? 1024 : 256);
-    const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS ? groups : LOSS_MAX_BLOCKS);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS * sizeof(double)));
+    const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS(ctx) ? groups : LOSS_MAX_BLOCKS(ctx));
+    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS(ctx) * sizeof(double)));
     double *block_partial = (double *)ctx->buf_misc.p;
     int *ticket = ctx->d_flag + 2;
     const float scale = 1.0f / (float)ctx->n;
@@ -1184,8 +1184,8 @@ extern "C" sat_status sat_staleness(sat_ctx *ctx, int32_t part, int32_t d, const
     }
     if (!h_fresh || !h_used_halo || ld < d || ld_halo < d) return sat_fail(ctx, SAT_EINVAL, "sat_staleness: null tensor or bad leading dimension");
     const int64_t groups = cdiv64(v.n_halo, 8);
-    const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS ? groups : LOSS_MAX_BLOCKS);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS * sizeof(double)));
+    const unsigned blocks = (unsigned)(groups < LOSS_MAX_BLOCKS(ctx) ? groups : LOSS_MAX_BLOCKS(ctx));
+    SAT_TRY(sat_ensure(ctx, ctx->buf_misc, (size_t)LOSS_MAX_BLOCKS(ctx) * sizeof(double)));
     sat_pdl(ctx->stream, k_staleness, blocks, 256, 0)(ctx->halo_gid, ctx->pos, v.halo0, v.n_halo, d, h_fresh, ld, h_used_halo, ld_halo,
                                                  (double *)ctx->buf_misc.p, ctx->d_flag + 2, sq_sum, 1);
     SAT_LAUNCHED(ctx);

@@ -290,7 +290,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     }
     // ---- scratch ----
     const int64_t n_tiles = cdiv64(nb, PT_ROWS_PER_BLOCK);
-    const int64_t n_blocks = n_tiles < 8 * 148 ? n_tiles : 8 * 148;   // error kernel: the resident blocks of all SMs, each walking its tiles
+    const int64_t n_blocks = n_tiles < 8 * ctx->sms ? n_tiles : 8 * ctx->sms;   // error kernel: the resident blocks of all SMs, each walking its tiles
     const size_t f_gates = pt_round((size_t)(k > 0 ? k : 1) * R * 4 * h), f_state = pt_round((size_t)(k > 0 ? k : 1) * R * h);
     const size_t f_a = pt_round((size_t)nb * h), f_e = pt_round((size_t)nb * ld_d), f_rh = pt_round((size_t)R * h);
     const size_t f_off = pt_round(2 * (size_t)(M + 1)), f_part = pt_round(2 * (size_t)(n_blocks + 1)), f_nh = pt_round((size_t)ctx->n * h);
@@ -305,7 +305,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     SAT_CUDA(ctx, cudaMemcpyAsync(halo_off, ctx->h_halo_off.data(), (size_t)(M + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, ctx->stream));
     const int64_t plane_g = R * 4 * (int64_t)h, plane_s = R * (int64_t)h;
     const unsigned cell_grid = (unsigned)cdiv64(R, PT_TILE_ROWS);
-    const unsigned bwd_grid = cell_grid < 8 * 148 ? cell_grid : 8 * 148;
+    const unsigned bwd_grid = cell_grid < 8u * ctx->sms ? cell_grid : 8u * ctx->sms;
     const size_t cell_smem = (size_t)(256 / (h / 4)) * 4 * h * sizeof(float);
     // ---- LSTM forward over the snapshots, oldest first, gate values kept ----
     const bool tc_z = sat_use_tc(4 * h, d);
@@ -378,8 +378,8 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
         SAT_TRY(sat_sum_by_slot(ctx, h, g_a, h, 1, 1, dh, h));
         // ---- back-propagation through time ----
         // The parameter gradients are sums over the steps of products of one shape (every step keeps its gate gradients): on the tensor
-        // cores all steps are one launch and one reduction each for Wx (with the bias) and Uh (a launch costs 27 us besides the product; 84671 nodes, four
-        // steps: 18 launches of the epoch, 957 + 236 us).
+        // cores all steps are one launch and one reduction each for Wx (with the bias) and Uh (82,770 cached nodes, 256 -> 64, four steps: the
+        // call takes 1.50 ms; one wave over all steps took 1.40, at three times the error, see sat_gemm_tc_tn).
         const bool merged = sat_use_tc(4 * h, d) && sat_use_tc(4 * h, h) && 4 * h > 64 && R >= 256;
         if (!merged) SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)bwd_grid * 4 * h * sizeof(float)));
         for (int32_t t = k - 1; t >= 0; --t) {

@@ -58,9 +58,10 @@ __device__ __forceinline__ void mask4(float4 &r, const uint32_t *__restrict__ om
 // moved 1.7 ms per epoch into the partial sums and gained 0.4 ms); and not below the mean row (rounded up to a power of two), so that an
 // ordinary row of a dense graph stays in one piece (up to 512: 2 % of an epoch with 490 entries a row against 256).
 //
-// Small lists have no second launch: the run of a row that ends last adds the row's partial sums (epoch of 900 nodes 99 -> 89 us, of
-// 2708 nodes 285 -> 269); their chunk grows until every row has at most LAST_RUN_MAX runs.  Large lists keep k_spmm_fixup: the fence
-// and ticket of every partial run cost more there than a launch (32 M entries: +4 %).
+// Small lists (chunk 32) have no second launch: the run of a row that ends last adds the row's partial sums (epoch of 900 nodes 99 -> 89 us,
+// of 2708 nodes 285 -> 269).  Their chunk grows, up to 128, until the longest row has at most LAST_RUN_MAX runs; where 128 is not
+// enough (a row above 8,192 entries) it stays at 32 and rows of more runs go to k_spmm_fixup.  Large lists keep k_spmm_fixup: the
+// fence and ticket of every partial run cost more there than a launch (32 M entries: +4 %).
 static int32_t list_chunk(int64_t entries, int64_t rows)
 {
     const int64_t M = (int64_t)1 << 20;
@@ -336,7 +337,7 @@ static sat_status list_build(sat_ctx *ctx, const ListKey &want, SpmmList **out)
         // a small launch: runs up to 128 entries where that lets the last run of the longest row do the adding (no second launch)
         int32_t longest = 0;
         SAT_CUDA(ctx, cudaMemsetAsync(ctx->d_flag + 3, 0, sizeof(int32_t), ctx->stream));
-        k_list_max<<<(unsigned)std::min<int64_t>(cdiv64(n_rows, 256), 148), 256, 0, ctx->stream>>>(L, n_rows, ctx->d_flag + 3);
+        k_list_max<<<(unsigned)std::min<int64_t>(cdiv64(n_rows, 256), ctx->sms), 256, 0, ctx->stream>>>(L, n_rows, ctx->d_flag + 3);
         SAT_LAUNCHED(ctx);
         SAT_CUDA(ctx, cudaMemcpyAsync(&longest, ctx->d_flag + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
         SAT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -717,8 +718,10 @@ static sat_status run_list(sat_ctx *ctx, const PartView &v, const SpmmList &l, i
     // the dense one).
     const int4 *items = l.item + item0;
 #define ARGS ctx, l, items, (int32_t)n_items, slot_base, d4, a, partial
-    // A launch that leaves most of the chip idle is as long as its longest run: eight entries in flight per step then
-    const bool small = n_items * 32 <= 148 * 768;
+    // A launch of at most three blocks of eight warps per SM, a warp per item, leaves most of the chip idle and is as long as its longest
+    // run: eight entries in flight per step then, for more registers (epoch of 2,048 nodes 90.6 -> 84.4 us; 6,000 nodes and upward the
+    // same, one drawn graph 515 -> 522)
+    const bool small = n_items * 32 <= ctx->sms * 768;
     if (d4 <= 4) small ? launch_spmm<4, 1, 8, 3>(ARGS) : launch_spmm<4, 1, 4, 6>(ARGS);
     else if (d4 <= 8) small ? launch_spmm<8, 1, 8, 3>(ARGS) : launch_spmm<8, 1, 4, 6>(ARGS);
     else if (d4 <= 16) small ? launch_spmm<16, 1, 8, 3>(ARGS) : launch_spmm<16, 1, 4, 6>(ARGS);
@@ -1199,7 +1202,7 @@ extern "C" sat_status sat_profile_l2_rates(sat_ctx *ctx, int32_t row_floats, dou
         const int64_t n_vec = (int64_t)(bytes / 16);
         for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {  // first pass warms the L2 and the instruction cache
             cudaEventRecord(e0, ctx->stream);
-            k_l2_stream<<<148 * 8, 256, 0, ctx->stream>>>((const float4 *)buf, n_vec, reps, sink);
+            k_l2_stream<<<ctx->sms * 8, 256, 0, ctx->stream>>>((const float4 *)buf, n_vec, reps, sink);
             cudaEventRecord(e1, ctx->stream);
             ctx->launches++;
             e = cudaEventSynchronize(e1);
