@@ -239,7 +239,8 @@ sat_status sat_predict_state(sat_ctx *ctx, int32_t layer, float *S_host, int32_t
  * row_weight  DEVICE [sum_m b_m] (halo rows of all partitions, concatenated in partition order) or NULL
  * g_Wx [d x 4h], g_Uh [h x 4h], g_b [4h], g_Wg [h x d], g_bg [d]   DEVICE, dense row-major, overwritten
  * loss_host   HOST, may be NULL; when given the call synchronises the stream
- * Scratch (owned by the context, kept): about k * |C| * 6h + sum_m b_m * (d + 2h) floats.
+ * Scratch (owned by the context, kept): about k * |C| * 6h + sum_m b_m * (d + 2h) floats, and the partial sums of the weight gradients,
+ * about 150,000 * k * h floats.
  * Errors: SAT_ESTATE without a cache, SAT_EINVAL for null / misaligned arrays or h not a multiple of 4.
  * ------------------------------------------------------------------------------------- */
 sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_params *params, const float *row_weight, float *g_Wx,
