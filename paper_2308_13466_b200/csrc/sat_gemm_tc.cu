@@ -19,6 +19,8 @@
 
 #include "sat_internal.h"
 
+#include <algorithm>
+
 #define TC_BM 128
 #define TC_BK 16          /* fp32 elements per k-block: 64-byte rows */
 #define TC_WAIT_LIMIT (1u << 22)
@@ -1598,7 +1600,7 @@ sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &
 
 // C[m x n] (+)= sum_i A[i]^T B[i] over `rows` rows each: A fp32 [rows x m] (lda), B fp32 [rows x n] (ldb)
 sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *const *A, int32_t lda, const float *const *B, int32_t ldb,
-                          int32_t segments, float *C, int32_t ldc, int accumulate, float *colsum)
+                          int32_t segments, float *C, int32_t ldc, int accumulate, float *colsum, int32_t reserve)
 {
     if (m == 0 || n == 0) return SAT_OK;
     if (segments < 1 || segments > SAT_TN_SEGMENTS) return sat_fail(ctx, SAT_EINVAL, "sat_gemm_tc_tn: 1 to %d segments", SAT_TN_SEGMENTS);
@@ -1615,10 +1617,12 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
     // segments share the launch (one wave over all segments: relative error of the predictor's gradients 8e-6 -> 6e-5 at 512 columns and
     // eight steps; one wave of 256-column tiles over 300 columns 7.2e-5 -> 8.7e-5).  Not less than six k-blocks each: the m x n partial
     // sums of a split, written and read again, cost about as much as that.
-    const int64_t least = cdiv64(2 * ctx->sms, (int64_t)subs * col_tiles), slots = (int64_t)ctx->sms * per_sm, per_split = tiles * segments;
-    const int64_t waves = cdiv64(least * per_split, slots);
-    int64_t splits = per_split < slots * waves ? slots * waves / per_split : 1;
-    if (splits > cdiv64(kblocks, 6)) splits = cdiv64(kblocks, 6);
+    const int64_t least = cdiv64(2 * ctx->sms, (int64_t)subs * col_tiles), slots = (int64_t)ctx->sms * per_sm;
+    auto splits_of = [&](int32_t segs) {
+        const int64_t per_split = tiles * segs, waves = cdiv64(least * per_split, slots);
+        return std::min<int64_t>(per_split < slots * waves ? slots * waves / per_split : 1, cdiv64(kblocks, 6));
+    };
+    int64_t splits = splits_of(segments);
     const int64_t kpb = cdiv64(kblocks, splits), rps = kpb * TC_BK;
     splits = cdiv64(r1, rps);
     int64_t stages = (MN_SMEM_MAX / per_sm - 1024 - (int)sizeof(MnShared) - 1024) / stage_bytes;
@@ -1626,7 +1630,9 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
     if (stages > kpb) stages = kpb;
     const size_t need = (size_t)stages * stage_bytes, turn = MN_TURN_BYTES;
     const size_t smem = (need > turn ? need : turn) + sizeof(MnShared) + 1024;
-    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)(splits * segments) * ((size_t)m * n + n) * sizeof(float)));
+    // room for `reserve` segments at once: a window that fills epoch by epoch would grow it in each of them
+    const int64_t parts = std::max<int64_t>(splits * segments, reserve > segments ? splits_of(reserve) * reserve : 0);
+    SAT_TRY(sat_ensure(ctx, ctx->buf_splitk, (size_t)parts * ((size_t)m * n + n) * sizeof(float)));
     float *part = (float *)ctx->buf_splitk.p;
     float *part_cs = colsum ? part + (size_t)(splits * segments) * m * n : nullptr;
     MnMaps maps;
@@ -1649,5 +1655,5 @@ sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, cons
 sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb, float *C,
                           int32_t ldc, int accumulate, float *colsum)
 {
-    return sat_gemm_tc_tn(ctx, rows, m, n, &A, lda, &B, ldb, 1, C, ldc, accumulate, colsum);
+    return sat_gemm_tc_tn(ctx, rows, m, n, &A, lda, &B, ldb, 1, C, ldc, accumulate, colsum, 0);
 }

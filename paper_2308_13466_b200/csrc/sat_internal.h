@@ -557,9 +557,10 @@ sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &
 // C[m x n] = [A | A2] B^T (+ epilogue)
 sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32_t lda, int32_t k1, const float *A2, int32_t lda2, int32_t k2,
                        const TcWeights &Bw, const TcEpilogueHost &eh, int family);
-// C[m x n] (+)= A^T B over `rows` rows, colsum[n] (+)= 1^T B if non-null
+// C[m x n] (+)= A^T B over `rows` rows, colsum[n] (+)= 1^T B if non-null; the first form sums `segments` such products and makes its
+// workspace large enough for `reserve` of them
 #define SAT_TN_SEGMENTS 8
 sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *const *A, int32_t lda, const float *const *B, int32_t ldb,
-                          int32_t segments, float *C, int32_t ldc, int accumulate, float *colsum = nullptr);
+                          int32_t segments, float *C, int32_t ldc, int accumulate, float *colsum, int32_t reserve);
 sat_status sat_gemm_tc_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B, int32_t ldb, float *C,
                           int32_t ldc, int accumulate, float *colsum = nullptr);

@@ -408,8 +408,9 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
                 ss[i] = t0 + i > 0 ? hs + (t0 + i - 1) * plane_s : nullptr;
                 zs[i] = gates + (t0 + i) * plane_g;
             }
-            SAT_TRY(sat_gemm_tc_tn(ctx, R, d, 4 * h, xs, c->ld, zs, 4 * h, cnt, g_Wx, 4 * h, t0 > 0, g_b));
-            if (cnt > skip) SAT_TRY(sat_gemm_tc_tn(ctx, R, h, 4 * h, ss + skip, h, zs + skip, 4 * h, cnt - skip, g_Uh, 4 * h, t0 > 0));
+            const int32_t window = ctx->tau < SAT_TN_SEGMENTS ? ctx->tau : SAT_TN_SEGMENTS;
+            SAT_TRY(sat_gemm_tc_tn(ctx, R, d, 4 * h, xs, c->ld, zs, 4 * h, cnt, g_Wx, 4 * h, t0 > 0, g_b, window));
+            if (cnt > skip) SAT_TRY(sat_gemm_tc_tn(ctx, R, h, 4 * h, ss + skip, h, zs + skip, 4 * h, cnt - skip, g_Uh, 4 * h, t0 > 0, nullptr, window));
         }
     }
     if (loss_host) {
