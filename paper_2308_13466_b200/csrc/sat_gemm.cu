@@ -123,7 +123,8 @@ sat_status sat_gemm_nn_dual(sat_ctx *ctx, int64_t m, int32_t n, int32_t k1, cons
 
 __global__ void __launch_bounds__(256)
 k_gemm_nt(int64_t m, int32_t n, int32_t k, const float *__restrict__ A, int64_t lda, const uint32_t *__restrict__ mask,
-          int32_t mask_words, const float *__restrict__ B, int64_t ldb, float *__restrict__ C, int64_t ldc)
+          int32_t mask_words, const float *__restrict__ B, int64_t ldb, float *__restrict__ C, int64_t ldc, const uint32_t *__restrict__ omask,
+          int32_t omask_words)
 {
     sat_grid_wait();
     __shared__ float As[BK][BM + 4];
@@ -165,18 +166,18 @@ k_gemm_nt(int64_t m, int32_t n, int32_t k, const float *__restrict__ A, int64_t 
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int32_t gn = col0 + tx * 4 + j;
-            if (gr < m && gn < n) C[gr * ldc + gn] = acc[i][j];
+            if (gr < m && gn < n) C[gr * ldc + gn] = omask && !mask_bit(omask, gr, omask_words, gn) ? 0.f : acc[i][j];
         }
     }
 }
 
 sat_status sat_gemm_nt(sat_ctx *ctx, int64_t m, int32_t n, int32_t k, const float *A, int32_t lda, const uint32_t *mask,
-                       int32_t mask_words, const float *B, int32_t ldb, float *C, int32_t ldc)
+                       int32_t mask_words, const float *B, int32_t ldb, float *C, int32_t ldc, const uint32_t *omask, int32_t omask_words)
 {
     if (m == 0 || n == 0) return SAT_OK;
     ProfScope prof(ctx, SATK_GEMM_NT, 4.0 * ((double)m * (k + n) + (double)k * n), 2.0 * (double)m * n * k);
     dim3 grid((unsigned)cdiv64(m, BM), (unsigned)cdiv64(n, BN));
-    sat_pdl(ctx->stream, k_gemm_nt, grid, 256, 0)(m, n, k, A, lda, mask, mask_words, B, ldb, C, ldc);
+    sat_pdl(ctx->stream, k_gemm_nt, grid, 256, 0)(m, n, k, A, lda, mask, mask_words, B, ldb, C, ldc, omask, omask_words);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }

@@ -286,6 +286,8 @@ struct TcEpilogue {
     int relu;
     uint32_t *mask_out;
     int32_t mask_words;
+    const uint32_t *mask_in;
+    int32_t mask_in_words;
     const float *resid;  // C += resid[resid_idx[row]]  (row gather)
     const int32_t *resid_idx;
     int64_t ld_resid;
@@ -698,6 +700,12 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     if (ep.relu) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(fmaxf(__uint_as_float(r[j]), 0.f));
+                    }
+                    if (EPI == EPI_PLAIN && ep.mask_in) {
+                        const int32_t word = (n0 + c0) >> 5;
+                        const uint32_t keep = word < ep.mask_in_words ? __ldg(ep.mask_in + row * ep.mask_in_words + word) : 0u;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) r[j] = keep >> j & 1u ? r[j] : 0u;
                     }
                 }
                 if (EPI == EPI_PROJ) {   // a warp's store of a unit is 512 contiguous bytes
@@ -1553,6 +1561,9 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.relu = eh.relu;
     ep.mask_out = eh.mask_out;
     ep.mask_words = eh.mask_words;
+    ep.mask_in = eh.mask_in;
+    ep.mask_in_words = eh.mask_in_words;
+    if (eh.mask_in && (eh.lstm_h > 0 || eh.proj_h > 0 || eh.resid_idx || eh.push_dst)) return sat_fail(ctx, SAT_EINVAL, "an input mask needs the plain epilogue");
     ep.resid = eh.resid;
     ep.resid_idx = eh.resid_idx;
     ep.ld_resid = eh.ld_resid;

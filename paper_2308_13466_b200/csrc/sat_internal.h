@@ -337,9 +337,15 @@ enum class SpmmHalo { by_position, by_gid, by_slot };
 // omask (or null): bit mask [rows x omask_words] indexed like out_base; output components whose bit is 0 are written as 0
 // halo_kind: what the halo columns address: the concatenated halo matrix, a matrix over all n nodes in global id order, or one over
 // the cache slots (halo_base = its first row in the last two); in_global: inner and halo columns both address such a matrix (in_base = its first row; halo_base is not used)
+// add: rows added to the results, where given
+struct SpmmAdd {
+    const float *rows = nullptr;         // out[i] += rows[slot[i] * ld ..] where slot[i] >= 0
+    const int32_t *slot = nullptr;       // [rows of out]
+    int64_t ld = 0;
+};
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask = nullptr,
-                    int32_t omask_words = 0, SpmmHalo halo_kind = SpmmHalo::by_position, bool in_global = false);
+                    int32_t omask_words = 0, SpmmHalo halo_kind = SpmmHalo::by_position, bool in_global = false, const SpmmAdd &add = SpmmAdd());
 // the same kernels on weights of the caller's: out[row] = epilogue(sum_e w_e * src(col_e)) with ent[e] = {column, weight} indexed like
 // the entries of the mode (0: local rows; 1: their inner prefix; 3: halo rows, columns = partition-major rows)
 struct SpmmEpilogue {
@@ -347,6 +353,7 @@ struct SpmmEpilogue {
     int relu = 0;
     const float *s1 = nullptr, *v1 = nullptr, *s2 = nullptr, *v2 = nullptr;   // + s1[row] v1[col] + s2[row] v2[col]
     int32_t d = 0;
+    SpmmAdd add;                         // (products with the propagation matrix only) rows added after the scaling
     float *push = nullptr;               // row i goes to row push_slot[i] of this matrix as well where that is >= 0
     const int32_t *push_slot = nullptr;  // [rows]
     int64_t ld_push = 0;
@@ -395,9 +402,9 @@ struct GemmEpilogue {
 };
 sat_status sat_gemm_nn(sat_ctx *ctx, int64_t m, int32_t n, int32_t k, const float *A, int32_t lda, const float *B,
                        int32_t ldb, float *C, int32_t ldc, const GemmEpilogue &ep);
-// C[m x n] = (A o mask)[m x k] B^T, B stored [n x k] row-major (ldb); mask may be null
+// C[m x n] = ((A o mask)[m x k] B^T) o omask, B stored [n x k] row-major (ldb); either mask may be null
 sat_status sat_gemm_nt(sat_ctx *ctx, int64_t m, int32_t n, int32_t k, const float *A, int32_t lda, const uint32_t *mask,
-                       int32_t mask_words, const float *B, int32_t ldb, float *C, int32_t ldc);
+                       int32_t mask_words, const float *B, int32_t ldb, float *C, int32_t ldc, const uint32_t *omask = nullptr, int32_t omask_words = 0);
 // C[m x n] (+)= A^T (B o mask): A [rows x m] (lda), B [rows x n] (ldb); colsum[n] (+)= 1^T (B o mask) if non-null.
 sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const float *A, int32_t lda, const float *B,
                        int32_t ldb, const uint32_t *mask, int32_t mask_words, float *C, int32_t ldc, float *colsum,
@@ -511,6 +518,8 @@ struct TcEpilogueHost {
     int relu = 0;
     uint32_t *mask_out = nullptr;
     int32_t mask_words = 0;
+    const uint32_t *mask_in = nullptr; // [m x mask_in_words] components of C whose bit is 0 are written as 0 (plain epilogue)
+    int32_t mask_in_words = 0;
     const float *resid = nullptr;      // C += resid[resid_idx[i]] (row gather)
     const int32_t *resid_idx = nullptr;
     int32_t ld_resid = 0;

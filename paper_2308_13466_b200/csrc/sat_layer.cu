@@ -854,6 +854,35 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
         }
     }
     if (!want_dx) return SAT_OK;
+    const bool stale_term = hist && GH.has_read && g_in && v.n_push > 0;
+    // G_in = P_in^T (D W^T) = (P_in^T D) W^T.  The second order gathers rows of d_out columns instead of d_in: taken where that is less
+    // (256 -> 40, 169343 nodes, 2.6 M entries: product 152 -> 53 us, epoch 2840 -> 2749; 128 -> 19, 240000 nodes: epoch 1669 -> 1524;
+    // 256 -> 47, 612257 nodes, 31 M entries: product 608 -> 165 us, epoch 16050 -> 15748).  The stale rows then join P_in^T D in the product's
+    // epilogue, which makes their own contraction and the add into G_in unnecessary, so with them the order pays at equal
+    // widths too (84671 nodes, 256 -> 256 -> 40, epoch with the predictor trained: 5342 -> 5087).
+    if (g_in && !g_halo && (!mask || tc_x) && (stale_term ? d_out <= d_in : d_out < d_in)) {
+        const int32_t ld_q = round_up4(d_out);
+        SAT_TRY(sat_ensure(ctx, ctx->buf_gagg, (size_t)v.n_rows * ld_q * sizeof(float)));
+        float *q = (float *)ctx->buf_gagg.p;
+        SpmmAdd add;
+        if (stale_term) {
+            SAT_TRY(sat_row_slots(ctx, &add.slot));
+            add.rows = GH.buf + (size_t)GH.read_idx * ctx->n_slots * GH.ld;
+            add.ld = GH.ld;
+        }
+        SAT_TRY(sat_spmm(ctx, v, 1, d_out, D - (int64_t)v.row0 * ld_d, ld_d, nullptr, 0, q - (int64_t)v.row0 * ld_q, ld_q, nullptr, 0, SpmmHalo::by_position,
+                         false, add));
+        const uint32_t *keep = mask_in ? mask_in + (int64_t)v.row0 * mask_in_words : nullptr;
+        if (!tc_x) return sat_gemm_nt(ctx, v.n_rows, d_in, d_out, q, ld_q, nullptr, 0, W, d_out, g_in, ld_gin, keep, mask_in_words);
+        TcWeights Wp;
+        SAT_TRY(sat_tc_weights(ctx, W, d_out, d_out, nullptr, 0, 0, d_in, 0, ctx->buf_wsplit, &Wp));
+        TcEpilogueHost eh;
+        eh.C = g_in;
+        eh.ldc = ld_gin;
+        eh.mask_in = keep;
+        eh.mask_in_words = mask_in_words;
+        return sat_gemm_tc(ctx, v.n_rows, d_in, q, ld_q, d_out, nullptr, 0, 0, Wp, eh, SATK_GEMM_NT);
+    }
     // G_AGG = D W^T
     const int32_t ld_ga = round_up4(d_in);
     SAT_TRY(sat_ensure(ctx, ctx->buf_gagg, (size_t)v.n_rows * ld_ga * sizeof(float)));
@@ -872,7 +901,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
     // G_in = P_in^T G_AGG: the inner block of P is symmetric, so P_in^T = P_in (inner prefix of every local row)
     if (g_in) SAT_TRY(sat_spmm(ctx, v, 1, d_in, ga_base, ld_ga, nullptr, 0, g_in - (int64_t)v.row0 * ld_gin, ld_gin, mask_in, mask_in_words));
     // gradient-side history, the stale term: G_in[v] += (Q_read[slot(v)] W^T) o mask for the boundary rows v of the selection
-    if (hist && GH.has_read && g_in && v.n_push > 0) {
+    if (stale_term) {
         const size_t plane = (size_t)ctx->n_slots * GH.ld;
         const float *qr = GH.buf + (size_t)GH.read_idx * plane;
         SAT_TRY(sat_ensure(ctx, ctx->buf_ghist_rows, (size_t)v.n_push * GH.ld * sizeof(float)));

@@ -480,6 +480,18 @@ __device__ __forceinline__ float4 spmm_epilogue(const SpmmEpilogue &ep, int64_t 
     return out;
 }
 
+// the row that is added to row `row`, column c
+__device__ __forceinline__ void spmm_add(const SpmmAdd &add, int64_t row, int c, float4 &r)
+{
+    const int32_t slot = __ldg(add.slot + row);
+    if (slot < 0) return;
+    const float4 x = ld4(add.rows + slot * add.ld + 4 * c);
+    r.x += x.x;
+    r.y += x.y;
+    r.z += x.z;
+    r.w += x.w;
+}
+
 // K entries: their columns and weights, their rows (all in flight together), the sums
 template <int G, int NV, int K, typename F>
 __device__ __forceinline__ void spmm_step(const int2 *__restrict__ ents, const F &row_of, int col, int32_t d4, float4 (&acc)[NV])
@@ -592,7 +604,10 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
         if (col + v * G < d4) {
             float4 r = make_float4(s * acc[v].x, s * acc[v].y, s * acc[v].z, s * acc[v].w);
             if (EPI) r = spmm_epilogue(ep, row, col + v * G, r);
-            else if (omask) mask4(r, omask, row * omask_words, col + v * G);
+            else {
+                if (ep.add.rows) spmm_add(ep.add, row, col + v * G, r);
+                if (omask) mask4(r, omask, row * omask_words, col + v * G);
+            }
             o[v * G] = r;
         }
     }
@@ -661,7 +676,10 @@ k_spmm_fixup(const int32_t *__restrict__ hrows, int32_t n_hrows, const int32_t *
     const float s = scale ? scale[row] : 1.f;
     float4 r = make_float4(s * a.x, s * a.y, s * a.z, s * a.w);
     if (!scale) r = spmm_epilogue(ep, row, c, r);
-    else if (omask) mask4(r, omask, row * omask_words, c);
+    else {
+        if (ep.add.rows) spmm_add(ep.add, row, c, r);
+        if (omask) mask4(r, omask, row * omask_words, c);
+    }
     *reinterpret_cast<float4 *>(out_base + row * ld_out + 4 * c) = r;
 }
 
@@ -759,7 +777,7 @@ __global__ void k_ent_all_gid(const int2 *__restrict__ ent, const int32_t *__res
 
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask, int32_t omask_words,
-                    SpmmHalo halo_kind, bool in_global)
+                    SpmmHalo halo_kind, bool in_global, const SpmmAdd &add)
 {
     if (v.n_rows == 0) return SAT_OK;
     const int32_t d4 = (d + 3) / 4;
@@ -803,6 +821,7 @@ sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, 
     SpmmList *l = nullptr;
     SAT_TRY(list_build(ctx, list_key(d4, inner_only), &l));
     a.scale = ctx->dinv_enc;
+    a.ep.add = add;
     a.n = ctx->n;
     a.in_base = in_base;
     a.ld_in = ld_in;

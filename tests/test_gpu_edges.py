@@ -610,3 +610,51 @@ def test_rows_that_the_second_launch_finishes(B, kind, d):
     for what, got, ref in (("out", out[:, :d], (o + c(b).double())[c(perm)]), ("G_W", gW, c(X).double().T @ dz), ("G_a_src", g1, z.T @ ds),
                            ("G_a_dst", g2, z.T @ dd), ("G_b", gb, D.sum(0)), ("G_in", g_in[:, :k], (dz_in @ c(W).double().T)[c(perm)])):
         assert_close(got, ref.cpu().numpy(), what)
+
+
+@pytest.mark.parametrize("hist", [False, True])
+@pytest.mark.parametrize("d_in,d_out", [(16, 15), (33, 5), (40, 40), (72, 17), (256, 40), (260, 256), (300, 299), (24, 40)])
+def test_input_gradient_in_both_orders(B, d_in, d_out, hist):
+    """G_in = (P_in^T D + Q) W^T under the mask of the layer below (Q: stale rows of the boundary nodes, on request) at widths on both sides of the
+    rule that picks the order, all partitions at once = one after the other."""
+    n, M = 2000, 3
+    A = _graph(HUBS[:11], n)
+    Pm = _propagation(A).tocoo()
+    rng = np.random.default_rng(d_in)
+    part = rng.integers(0, M, n).astype(np.int32)
+    perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+    off = np.concatenate([[0], np.cumsum(np.bincount(part, minlength=M))])
+    W1, W2 = (rng.standard_normal(s).astype(np.float32) for s in ((8, d_in), (d_in, d_out)))
+    X, D = rng.standard_normal((n, 8)).astype(np.float32), rng.standard_normal((n, d_out)).astype(np.float32)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        B.sat_cache_init(ctx, [d_in], 2)
+        _, slot, n_slots = B.sat_slot_map(ctx, n)
+        n_halo = B.sat_part_sizes(ctx, B.SAT_ALL_PARTS)[1]
+        H1, H2, g_in, one = empty2d(n, d_in), empty2d(n, d_out), empty2d(n, d_in), empty2d(n, d_in)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(X), None, dev(W1), None, B.SAT_ACT_RELU | B.SAT_FWD_INPUT_GLOBAL, H1)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, H1, dev2d(np.zeros((n_halo, d_in), np.float32)), dev(W2), None, B.SAT_ACT_NONE, H2)
+        Q = np.zeros((n_slots, d_out), np.float32)
+        if hist:
+            Q = rng.standard_normal((n_slots, d_out)).astype(np.float32)
+            B.sat_grad_history_write(ctx, 2, d_out, Q)
+        flags = B.SAT_BWD_MASK_G_IN | (B.SAT_BWD_GRAD_HISTORY if hist else 0)
+        gW, gb = torch.empty((d_in, d_out), device="cuda"), torch.empty(d_out, device="cuda")
+        Dd = dev2d(D[perm])
+        B.sat_layer_bwd(ctx, B.SAT_ALL_PARTS, 2, Dd, dev(W2), gW, gb, flags, g_in, None)
+        for m in range(M):
+            r = slice(off[m], off[m + 1])
+            B.sat_layer_bwd(ctx, m, 2, Dd[r], dev(W2), gW, gb, flags, one[r], None)
+        B.sat_sync_status(ctx)
+        got, keep = g_in.cpu().numpy(), H1.cpu().numpy() > 0
+        assert torch.equal(g_in, one)
+    finally:
+        B.sat_destroy(ctx)
+    same = sp.csr_matrix((Pm.data * (part[Pm.row] == part[Pm.col]), (Pm.row, Pm.col)), shape=Pm.shape)
+    slot = np.asarray(slot)
+    stale = np.where((slot >= 0)[:, None], Q[np.maximum(slot, 0)], 0.0)
+    want, mag = (same @ D.astype(np.float64) + stale) @ W2.T, (abs(same) @ np.abs(D.astype(np.float64)) + np.abs(stale)) @ np.abs(W2.T)
+    terms = np.diff(A.indptr).max() + d_out + 8
+    assert (np.abs(got - want[perm] * keep) <= (terms * U + 2.0 ** -20) * mag[perm]).all()
