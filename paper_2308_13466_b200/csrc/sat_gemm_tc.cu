@@ -16,6 +16,7 @@
 // warps 0 / 1 as above, warps 2..9 convert during the main loop and then run the epilogue.  Every mbarrier wait is
 // bounded; a timeout raises a status word and lets the CTA drain (TMEM is freed, the kernel returns).
 #include <cuda.h>
+#include <cuda_fp16.h>
 
 #include "sat_internal.h"
 
@@ -144,12 +145,12 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar)
 }
 // D (+)= A B.  USE_A: what becomes of the A tile in the tensor core's operand collector -- 1: it stays, 2: it is taken from there for
 // the last time.  (The two products with A hi read it from shared memory once: 1.3 % of a 179250 x 512 x 512 contraction.)
-#define TC_MMA_ASM(G, COLLECTOR)                                                                       \
+#define TC_MMA_ASM(G, KIND, COLLECTOR)                                                                 \
     asm volatile(                                                                                      \
         "{\n\t"                                                                                        \
         ".reg .pred p;\n\t"                                                                            \
         "setp.ne.b32 p, %4, 0;\n\t"                                                                    \
-        "tcgen05.mma.cta_group::" G ".kind::tf32" COLLECTOR " [%0], %1, %2, %3, p;\n\t"                     \
+        "tcgen05.mma.cta_group::" G ".kind::" KIND COLLECTOR " [%0], %1, %2, %3, p;\n\t"                   \
         "}" ::"r"(tmem_d),                                                                             \
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                                            \
         : "memory")
@@ -157,14 +158,22 @@ template <int USE_A, int GROUP>
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
     if (GROUP == 2) {
-        if (USE_A == 1) TC_MMA_ASM("2", ".collector::a::fill");
-        else if (USE_A == 2) TC_MMA_ASM("2", ".collector::a::lastuse");
-        else TC_MMA_ASM("2", "");
+        if (USE_A == 1) TC_MMA_ASM("2", "tf32", ".collector::a::fill");
+        else if (USE_A == 2) TC_MMA_ASM("2", "tf32", ".collector::a::lastuse");
+        else TC_MMA_ASM("2", "tf32", "");
     } else {
-        if (USE_A == 1) TC_MMA_ASM("1", ".collector::a::fill");
-        else if (USE_A == 2) TC_MMA_ASM("1", ".collector::a::lastuse");
-        else TC_MMA_ASM("1", "");
+        if (USE_A == 1) TC_MMA_ASM("1", "tf32", ".collector::a::fill");
+        else if (USE_A == 2) TC_MMA_ASM("1", "tf32", ".collector::a::lastuse");
+        else TC_MMA_ASM("1", "tf32", "");
     }
+}
+// the same with half-precision operands (single CTAs)
+template <int USE_A>
+__device__ __forceinline__ void tc_mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    if (USE_A == 1) TC_MMA_ASM("1", "f16", ".collector::a::fill");
+    else if (USE_A == 2) TC_MMA_ASM("1", "f16", ".collector::a::lastuse");
+    else TC_MMA_ASM("1", "f16", "");
 }
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t *r)
 {
@@ -204,6 +213,29 @@ __host__ __device__ inline uint32_t make_idesc(int m, int n, int a_mn_major, int
     d |= (uint32_t)(n >> 3) << 17;
     d |= (uint32_t)(m >> 4) << 24;
     return d;
+}
+
+// kind::f16 with half-precision operands, both K-major, fp32 accumulation
+__host__ __device__ inline uint32_t make_idesc_f16(int m, int n) { return 1u << 4 | (uint32_t)(n >> 3) << 17 | (uint32_t)(m >> 4) << 24; }
+
+// Two-term split into half precision, x s = hi + lo + e with |e| <= 2^-22 |x s| wherever |x s| is not small: both terms are rounded to nearest,
+// and a power of two s brings the largest element of the operand's row to [2^14, 2^15), so that terms are subnormal (and e
+// is at most 2^-25) only for elements 2^18 times smaller than that one.  Closer than the TF32 split (2^-21 |x|, and hi truncated), on
+// operands of half the size and at twice the rate.  Two elements at a time: the first in the low half.
+__device__ __forceinline__ void split_f16(float x0, float x1, uint32_t &hi, uint32_t &lo)
+{
+    const __half2 h = __floats2half2_rn(x0, x1);
+    const float2 f = __half22float2(h);
+    const __half2 l = __floats2half2_rn(x0 - f.x, x1 - f.y);
+    hi = *reinterpret_cast<const uint32_t *>(&h);
+    lo = *reinterpret_cast<const uint32_t *>(&l);
+}
+// biased exponent of the power of two that brings the elements of a row, the largest of which has this biased exponent, below 2^15; the
+// inverse has 254 minus it.  One for zeros, infinities and NaN.
+__device__ __forceinline__ uint32_t f16_scale_exponent(uint32_t largest)
+{
+    const int e = 268 - (int)largest;
+    return largest == 0 || largest == 255 ? 127u : (uint32_t)(e > 253 ? 253 : e);
 }
 
 // =====================================================================================
@@ -347,7 +379,7 @@ template <> struct TckCfg<EPI_PROJ> : TckCfg<EPI_LSTM> {};
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, bool valid)
 {
     // src-size 0 writes 16 zero bytes without reading the source
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem_dst)), "l"(gsrc), "r"(valid ? 16u : 0u) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem_dst)), "l"(gsrc), "r"(valid ? 16u : 0u) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -807,25 +839,34 @@ done:
 // h = 64, half of it the projection (83 us a step, and 54 for the first one).  Here a row tile stays on the SM for all steps: s as the
 // A operand in shared memory, c in registers, Uh resident; a step reads its projection and nothing else.
 //
-// A CTA pair (cta_group::2) works on two slots of 256 rows (128 per CTA) so that one slot's product runs under the other's cell
-// arithmetic: Uh takes 64 KB per CTA (half of the columns, both planes, h = 64), the two slots 64 KB each, and the accumulators all of
-// TMEM.  Eight warps per slot, two per lane quadrant with alternate quads of four units: one row per thread; the slot's first warp also
-// issues its products.  Projections are stored [row tile of 128][unit][row] float4 (sat_proj_floats), so a warp reads 512 contiguous
-// bytes.  160000 rows, h = 64: 198 us for four steps, 692 MB of projections at 3.5 TB/s.  Bound by latency: sixteen warps of 128 registers are all that fit,
-// and each step of a slot is a chain of product, load, gates and store.  (Without the loads 151 us, without the products 163, without
-// exponentials and reciprocals 209 of 226.  An issuing warp of its own left 96 registers: 213; bulk prefetches into L2: +13.)
+// A CTA works on two slots of 128 rows so that one slot's product runs under the other's cell arithmetic.  The operands are half-precision
+// pairs (split_f16; the state lies in [-1, 1], its scale is 2^14), rows of 128 bytes with 16 hi and 16 lo halves per k-step: 32 KB a slot
+// and 64 KB for Uh at h = 64, half of what TF32 terms take, which leaves 96 KB for the projections.  Those are stored [row tile of 128][unit][row]
+// float4 (sat_proj_floats); a thread copies its own row's 64 bytes of a quad of units by cp.async, SEQ_RING of its quads ahead, so
+// that nobody else has to be waited for.  Eight warps per slot, two per lane quadrant with alternate quads, one row per thread; accumulator
+// columns are fetched a quad ahead.  The slot's first warp also issues its products.
+//
+// 164833 rows, h = 64, four steps (675 MB of projections): 198 -> 158 us; 612257 rows 660 -> 504; 179250 rows and eight steps 393 -> 310.  Before, a
+// CTA pair held TF32 terms and the projections came through registers, two quads ahead; that form was bound by its latencies with every
+// unit below 45 %.  What did it: the copies' depth and their .cg (.ca: 184 us) and the accumulator columns a quad ahead.  (Bulk copies
+// by a warp of their own per slot, which leaves 96 registers: 192 us.)  The errors are what they were (relative 1.6e-6 of the
+// state at K = 256).
 // =====================================================================================
+#define SEQ_BK 32         /* terms of a k-block: 128-byte rows */
 #define SEQ_THREADS 512   /* 128 registers a thread */
+#define SEQ_RING 3        /* quads of projections in flight per thread */
 struct SeqSteps {
     const float *proj[SAT_SEQ_MAX];
 };
 struct SeqShared {
-    uint64_t b_full, b_ready;           // Uh has landed in this CTA; in both
-    uint64_t a_ready[2], acc_full[2];   // per slot: the state is in place; the product is done
+    float unscale[8];                                // per 32 gate columns, of the state and the columns together
+    uint64_t b_full;                                 // Uh has landed
+    uint64_t a_ready[2], acc_full[2];                // per slot: the state is in place; the product is done
     uint32_t tmem_base;
     int dead;
 };
 
+// 16 accumulator columns, to be waited for by tc_wait16 before their use
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t *r)
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -833,77 +874,122 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t *r)
                    "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr)
                  : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tc_wait16(uint32_t *r)   // (the registers are operands so that nothing reads them earlier)
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]),
+                   "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])::"memory");
+}
+// One LSTM cell: gates (i, f, g, o) and the cell state; returns the hidden state.  The quotients share reciprocals, since the transcendental unit
+// (16 lanes per clock, two operations per sigmoid or tanh by themselves) would take as long as the memory:
+//   i g = (e^{2 zg} - 1) / ((1 + e^{-zi}) (1 + e^{2 zg})),  o tanh(c) = (e^{2c} - 1) / ((1 + e^{-zo}) (1 + e^{2c})):
+// eight operations instead of ten.  Exponents are capped at 2^60, where both quotients have reached their limits in fp32, so that the products
+// do not overflow.
+__device__ __forceinline__ float lstm_cell(const float4 &z, float &c)
+{
+    auto capped = [](float x) {   // 2^min(x, 60), NaN for NaN
+        asm("min.NaN.f32 %0, %0, 0f42700000;" : "+f"(x));
+        return ex2_fast(x);
+    };
+    const float L = 1.4426950408889634f;
+    const float ei = capped(-L * z.x), ef = ex2_fast(-L * z.y), eg = capped(2.f * L * z.z), eo = capped(-L * z.w);
+    c = fmaf(rcp_fast(1.f + ef), c, (eg - 1.f) * rcp_fast((1.f + ei) * (1.f + eg)));
+    const float ec = capped(2.f * L * c);
+    return (ec - 1.f) * rcp_fast((1.f + eo) * (1.f + ec));
 }
 
 __global__ void __launch_bounds__(SEQ_THREADS, 1)
-k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo, const __grid_constant__ SeqSteps steps, int32_t n_steps,
-           int first, int64_t rows, int32_t h, int32_t bn, int32_t nkb, float *S, float *cell, int write_cell, int *status)
+k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ unscale, const __grid_constant__ SeqSteps steps, int32_t n_steps, int first,
+           int64_t rows, int32_t h, int32_t bn, int32_t nkb, float *S, float *cell, int write_cell,
+           int *status)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    constexpr uint32_t a_plane = TC_BM * TC_BK * 4;               // one plane of a k-block of the state: 128 rows x 64 B, 64-byte swizzle
-    const uint32_t b_plane = (uint32_t)bn / 2 * TC_BK * 4;
-    const uint32_t slot_bytes = (uint32_t)nkb * 2 * a_plane;      // [k-block][hi | lo]
-    uint8_t *Bs = smem + 2 * slot_bytes;                          // [k-block][hi | lo]
-    SeqShared *sh = (SeqShared *)(Bs + (size_t)nkb * 2 * b_plane);
+    constexpr uint32_t a_block = TC_BM * 128;                     // a k-block: rows of two k-steps of 16 hi and 16 lo halves, 128-byte swizzle
+    const uint32_t b_block = (uint32_t)bn * 128, slot_bytes = (uint32_t)nkb * a_block;
+    uint8_t *Bs = smem + 2 * slot_bytes;
+    uint8_t *Ps = Bs + (uint32_t)nkb * b_block;                   // projections: [SEQ_RING][unit of the quad][thread] float4
+    SeqShared *sh = (SeqShared *)(Ps + SEQ_RING * 4 * SEQ_THREADS * 16);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = blockIdx.x & 1u;
-    const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1, n_pt = (rows + 255) / 256;
-    const int32_t mine = unit < n_pt ? (int32_t)((n_pt - 1 - unit) / units + 1) : 0;   // tiles of the pair, alternately in slot 0 and 1
+    const int64_t n_rt = (rows + TC_BM - 1) / TC_BM;
+    const int32_t mine = blockIdx.x < n_rt ? (int32_t)((n_rt - 1 - blockIdx.x) / gridDim.x + 1) : 0;   // row tiles of the CTA, alternately in slot 0 and 1
+    const int32_t nq = h >> 2;                                    // quads of four units
 
     for (uint32_t o = threadIdx.x * 16; o < 2 * slot_bytes; o += SEQ_THREADS * 16) *reinterpret_cast<float4 *>(smem + o) = make_float4(0.f, 0.f, 0.f, 0.f);
-    fence_async_smem();   // (the columns h .. 16 nkb stay zero)
+    fence_async_smem();   // (the columns from h on stay zero)
     if (threadIdx.x == 0) {
         mbar_init(&sh->b_full, 1);
-        mbar_init(&sh->b_ready, 2);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&sh->a_ready[i], 2 * 8);
+            mbar_init(&sh->a_ready[i], 8);
             mbar_init(&sh->acc_full[i], 1);
         }
         sh->dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tc_alloc<2>(&sh->tmem_base, 512u);
+    if (warp == 0) tc_alloc<1>(&sh->tmem_base, 512u);
     tc_fence_before();
     __syncthreads();
-    cluster_sync();
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
     volatile int *dead = &sh->dead;
     sat_grid_wait();
+    if (threadIdx.x < 8) sh->unscale[threadIdx.x] = 32 * (int)threadIdx.x < bn ? __ldg(unscale + threadIdx.x) * 0x1p-14f : 0.f;
+    __syncthreads();
 
-    if (warp == 0) {
+    if (warp == 0 && mine > 0) {
         if (lane == 0) {
-            mbar_expect_tx(&sh->b_full, (uint32_t)nkb * 2 * b_plane);
-            for (int32_t kb = 0; kb < nkb; ++kb) {
-                tma_load_2d(Bs + (size_t)kb * 2 * b_plane, &mapB, &sh->b_full, kb * TC_BK, (int32_t)rank * (bn / 2));
-                tma_load_2d(Bs + ((size_t)kb * 2 + 1) * b_plane, &mapBlo, &sh->b_full, kb * TC_BK, (int32_t)rank * (bn / 2));
-            }
+            mbar_expect_tx(&sh->b_full, (uint32_t)nkb * b_block);
+            for (int32_t kb = 0; kb < nkb; ++kb) tma_load_2d(Bs + (uint32_t)kb * b_block, &mapB, &sh->b_full, kb * 2 * SEQ_BK, 0);
         }
         if (!mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
-        mbar_arrive_warp<2>(&sh->b_ready, lane);
     }
     {
         const int slot = warp >> 3, q = warp & 3, half = (warp >> 2) & 1;
-        const bool issuer = rank == 0 && (warp & 7) == 0;   // of its slot's products
-        const uint32_t idesc = make_idesc(2 * TC_BM, bn, 0, 0), acc = tmem + (uint32_t)slot * 256u;
-        const uint64_t a0 = make_desc(smem_u32(smem) + (uint32_t)slot * slot_bytes, 16, 512, 4), b0 = make_desc(smem_u32(Bs), 16, 512, 4);
-        const int32_t nq = h >> 2;                       // quads of four units
+        const bool issuer = (warp & 7) == 0;   // of its slot's products
+        const uint32_t idesc = make_idesc_f16(TC_BM, bn), acc = tmem + (uint32_t)slot * 256u;
+        const uint64_t a0 = make_desc(smem_u32(smem) + (uint32_t)slot * slot_bytes, 16, 1024, 2), b0 = make_desc(smem_u32(Bs), 16, 1024, 2);
+        const int32_t nks = (h + 15) / 16;               // k-steps of 16
         const int r_in = q * 32 + lane;                  // this thread's row of the tile
-        uint8_t *A = smem + (uint32_t)slot * slot_bytes + r_in * 64;
-        const uint32_t swz = (uint32_t)(r_in >> 1) & 3u; // 64-byte swizzle: 16-byte piece c of row r sits at c ^ ((r >> 1) & 3)
-        auto put = [&](int qd, const float4 &v) {
-            uint8_t *d = A + (uint32_t)(qd >> 2) * 2 * a_plane + ((((uint32_t)qd & 3u) ^ swz) << 4);
-            *reinterpret_cast<float4 *>(d) = v;
-            *reinterpret_cast<float4 *>(d + a_plane) = residual4(v);
+        uint8_t *A = smem + (uint32_t)slot * slot_bytes + r_in * 128;
+        const uint32_t swz = (uint32_t)r_in & 7u;        // 16-byte piece c of row r sits at c ^ (r & 7)
+        uint8_t *const ring = Ps + threadIdx.x * 16;
+        const uint32_t mine_acc = acc + ((uint32_t)(q * 32) << 16);
+        auto put = [&](int qd, const float4 &v) {   // a quad is half a piece
+            uint2 hi, lo;
+            split_f16(v.x * 0x1p14f, v.y * 0x1p14f, hi.x, lo.x);
+            split_f16(v.z * 0x1p14f, v.w * 0x1p14f, hi.y, lo.y);
+            uint8_t *d = A + ((uint32_t)qd >> 3) * a_block + (((uint32_t)qd & 1u) << 3);
+            const uint32_t piece = ((uint32_t)qd & 4u) | (((uint32_t)qd & 3u) >> 1);
+            *reinterpret_cast<uint2 *>(d + ((piece ^ swz) << 4)) = hi;
+            *reinterpret_cast<uint2 *>(d + (((piece + 2) ^ swz) << 4)) = lo;
         };
-        if (issuer && !mbar_wait_all(&sh->b_ready, 0, dead, status)) goto done;
+        if (issuer && mine > slot && !mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
+        // this thread's quads in the order in which they are taken: (tile, step, quad); the copies run SEQ_RING of them ahead
+        const int32_t my_quads = (nq - half + 1) / 2;
+        int32_t pf_k = slot, pf_t = 0, pf_i = 0;
+        uint32_t pf_at = 0, at = 0;
+        auto copy_next = [&]() {   // a group a call, empty at the end
+            if (pf_k < mine && my_quads > 0) {
+                const float4 *src = reinterpret_cast<const float4 *>(steps.proj[pf_t]) +
+                                    ((blockIdx.x + (int64_t)pf_k * gridDim.x) * h + 4 * (half + 2 * pf_i)) * TC_BM + r_in;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) cp_async16(ring + (pf_at * 4 + u) * (SEQ_THREADS * 16), src + u * TC_BM, true);
+                if (++pf_i == my_quads) {
+                    pf_i = 0;
+                    if (++pf_t == n_steps) pf_t = 0, pf_k += 2;
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            pf_at = pf_at + 1 == SEQ_RING ? 0 : pf_at + 1;
+        };
+#pragma unroll
+        for (int i = 0; i < SEQ_RING; ++i) copy_next();
+        if (issuer && mine > slot && !mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
         uint32_t ph = 0;
         for (int32_t k = slot; k < mine; k += 2) {
-            const int64_t rt = (unit + (int64_t)k * units) * 2 + rank;   // row tile of 128
-            const int64_t row = rt * TC_BM + r_in;
-            const bool row_ok = row < rows, tile_ok = rt * TC_BM < rows;
+            const int64_t row = (blockIdx.x + (int64_t)k * gridDim.x) * TC_BM + r_in;
+            const bool row_ok = row < rows;
             float4 c[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -923,34 +1009,20 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
                 if (product) {
                     fence_async_smem();
                     tc_fence_before();
-                    mbar_arrive_warp<2>(&sh->a_ready[slot], lane);
-                }
-                const float4 *pr = reinterpret_cast<const float4 *>(steps.proj[t]) + rt * h * 128 + r_in;
-                // projections are fetched two quads ahead
-                float4 nx[2][4];
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        nx[i][u] = tile_ok && half + 2 * i < nq ? __ldg(pr + (4 * (half + 2 * i) + u) * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const uint32_t mine_acc = acc + ((uint32_t)(q * 32) << 16);
-                if (product) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sh->a_ready[slot]);
                     if (issuer) {
                         if (!mbar_wait_all(&sh->a_ready[slot], ph, dead, status)) goto done;
                         tc_fence_after();
                         if (elect_one()) {
-                            for (int32_t kb = 0; kb < nkb; ++kb) {
-#pragma unroll
-                                for (int ks = 0; ks < TC_BK / 8; ++ks) {
-                                    const uint64_t a_hi = a0 + (uint64_t)(((uint32_t)kb * 2 * a_plane) >> 4) + (uint64_t)(ks * 2);
-                                    const uint64_t b_hi = b0 + (uint64_t)(((uint32_t)kb * 2 * b_plane) >> 4) + (uint64_t)(ks * 2);
-                                    const uint64_t a_lo = a_hi + (a_plane >> 4), b_lo = b_hi + (b_plane >> 4);
-                                    tc_mma<1, 2>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-                                    tc_mma<2, 2>(acc, a_hi, b_lo, idesc, 1u);
-                                    tc_mma<0, 2>(acc, a_lo, b_hi, idesc, 1u);
-                                }
+                            for (int32_t ks = 0; ks < nks; ++ks) {
+                                const uint64_t a_hi = a0 + (uint64_t)((ks >> 1) * (a_block >> 4) + (ks & 1) * 4), a_lo = a_hi + 2;
+                                const uint64_t b_hi = b0 + (uint64_t)((ks >> 1) * (b_block >> 4) + (ks & 1) * 4), b_lo = b_hi + 2;
+                                tc_mma_f16<1>(acc, a_hi, b_hi, idesc, ks > 0 ? 1u : 0u);
+                                tc_mma_f16<2>(acc, a_hi, b_lo, idesc, 1u);
+                                tc_mma_f16<0>(acc, a_lo, b_hi, idesc, 1u);
                             }
-                            tc_commit<2>(&sh->acc_full[slot]);
+                            tc_commit<1>(&sh->acc_full[slot]);
                         }
                         __syncwarp();
                     }
@@ -958,35 +1030,35 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
                     ph ^= 1u;
                     tc_fence_after();
                 }
+                uint32_t r[2][16];   // accumulator columns of this quad and the next
+                if (product && half < nq) tc_ld16(mine_acc + 16u * (uint32_t)half, r[0]);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int32_t qd = half + 2 * i;
                     if (qd < nq) {
+                        asm volatile("cp.async.wait_group %0;" ::"n"(SEQ_RING - 1) : "memory");   // this thread's own copies
                         float4 z[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            z[u] = nx[i & 1][u];
-                            if (tile_ok && qd + 4 < nq) nx[i & 1][u] = __ldg(pr + (4 * (qd + 4) + u) * 128);
-                        }
+                        for (int u = 0; u < 4; ++u) z[u] = *reinterpret_cast<const float4 *>(ring + (at * 4 + u) * (SEQ_THREADS * 16));
+                        at = at + 1 == SEQ_RING ? 0 : at + 1;
                         if (product) {
-                            uint32_t r[16];
-                            tc_ld16(mine_acc + 16u * (uint32_t)qd, r);
+                            uint32_t(&a)[16] = r[i & 1];
+                            const float us = sh->unscale[qd >> 1];
+                            tc_wait16(a);
+                            if (i < 7 && qd + 2 < nq) tc_ld16(mine_acc + 16u * (uint32_t)(qd + 2), r[(i + 1) & 1]);
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
-                                z[u].x += __uint_as_float(r[4 * u]);
-                                z[u].y += __uint_as_float(r[4 * u + 1]);
-                                z[u].z += __uint_as_float(r[4 * u + 2]);
-                                z[u].w += __uint_as_float(r[4 * u + 3]);
+                                z[u].x = fmaf(__uint_as_float(a[4 * u]), us, z[u].x);
+                                z[u].y = fmaf(__uint_as_float(a[4 * u + 1]), us, z[u].y);
+                                z[u].z = fmaf(__uint_as_float(a[4 * u + 2]), us, z[u].z);
+                                z[u].w = fmaf(__uint_as_float(a[4 * u + 3]), us, z[u].w);
                             }
                         }
+                        copy_next();   // (into the place just read)
                         float4 sv;
                         float *cf = reinterpret_cast<float *>(&c[i]), *sf = reinterpret_cast<float *>(&sv);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {   // (i, f, g, o) of unit 4 qd + u
-                            const float gi = sigmoid_fast(z[u].x), gf = sigmoid_fast(z[u].y), gg = tanh_fast(z[u].z), go = sigmoid_fast(z[u].w);
-                            cf[u] = gf * cf[u] + gi * gg;
-                            sf[u] = go * tanh_fast(cf[u]);
-                        }
+                        for (int u = 0; u < 4; ++u) sf[u] = lstm_cell(z[u], cf[u]);   // unit 4 qd + u
                         if (!last) {
                             put(qd, sv);
                         } else if (row_ok) {
@@ -999,13 +1071,13 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUt
         }
     }
 done:
+    asm volatile("cp.async.wait_all;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
     if (warp == 0) {
         __syncwarp();
         tc_fence_after();
-        tc_dealloc<2>(tmem, 512u);
+        tc_dealloc<1>(tmem, 512u);
     }
 }
 
@@ -1354,6 +1426,37 @@ __global__ void k_split_weights(const float *__restrict__ W, int64_t ldw, int32_
     lo[i] = tf32_residual(x);  // second plane: read by the variants that do not split B in the kernel
 }
 
+// Recurrent weights Uh [h x 4 h] (gate blocks i | f | g | o) as half-precision pairs for k_lstm_seq: packed column 4 j + g is gate g of unit j; per
+// column the k-steps of 16 one after the other, each 16 hi and 16 lo halves (split_f16), zero padded to whole k-blocks, and the inverse of
+// the scale of every 32 columns.  A block takes 32 columns.
+#define PACK_COLS 32
+__global__ void __launch_bounds__(1024)
+k_pack_recurrent(const float *__restrict__ U, int32_t h, int32_t k_all, __half *__restrict__ out, float *__restrict__ unscale)
+{
+    sat_grid_wait();
+    __shared__ uint32_t largest;
+    const int32_t np0 = blockIdx.x * PACK_COLS;
+    auto value = [&](int32_t np, int32_t k) { return np < 4 * h && k < h ? U[(int64_t)k * 4 * h + (np & 3) * h + (np >> 2)] : 0.f; };
+    if (threadIdx.x == 0) largest = 0;
+    __syncthreads();
+    uint32_t m = 0;
+    for (int32_t i = threadIdx.x; i < PACK_COLS * k_all; i += 1024) m = max(m, __float_as_uint(value(np0 + i % PACK_COLS, i / PACK_COLS)) & 0x7fffffffu);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(&largest, m);
+    __syncthreads();
+    const uint32_t e = f16_scale_exponent(largest >> 23);
+    const float s = __uint_as_float(e << 23);
+    for (int32_t i = threadIdx.x; i < PACK_COLS * (k_all / 2); i += 1024) {
+        const int32_t c = i % PACK_COLS, k = 2 * (i / PACK_COLS);
+        uint32_t hi, lo;
+        split_f16(value(np0 + c, k) * s, value(np0 + c, k + 1) * s, hi, lo);
+        uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(np0 + c) * (k_all / 16) + k / 16) * 32 + k % 16);
+        o[0] = hi;
+        o[8] = lo;
+    }
+    if (threadIdx.x == 0) unscale[blockIdx.x] = __uint_as_float((254u - e) << 23);
+}
+
 // =====================================================================================
 // host side
 // =====================================================================================
@@ -1584,27 +1687,54 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     return pair ? launch_tck<EPI_PLAIN, 2>(ctx, L, ep) : launch_tck<EPI_PLAIN, 1>(ctx, L, ep);
 }
 
-sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
+// the recurrent weights of a predictor with h units, packed in `buf` (packed already, with `ready`)
+static size_t recurrent_layout(int32_t h, void *base, SatRecurrent *out)
+{
+    out->n_pad = tile_n_for(4 * h);
+    out->ld = (h + SEQ_BK - 1) / SEQ_BK * 2 * SEQ_BK;
+    const size_t planes = (size_t)out->n_pad * out->ld * sizeof(__half);
+    out->planes = base;
+    out->unscale = (float *)((char *)base + planes);
+    return planes + (size_t)out->n_pad / PACK_COLS * sizeof(float);
+}
+sat_status sat_pack_recurrent(sat_ctx *ctx, const float *Uh, int32_t h, DevBuf &buf, bool ready, SatRecurrent *out)
+{
+    const size_t bytes = recurrent_layout(h, nullptr, out);
+    if (ready && (!buf.p || buf.bytes < bytes)) return SAT_ESTATE;
+    SAT_TRY(sat_ensure(ctx, buf, bytes));
+    recurrent_layout(h, buf.p, out);
+    if (ready) return SAT_OK;
+    sat_pdl(ctx->stream, k_pack_recurrent, (unsigned)(out->n_pad / PACK_COLS), 1024, 0)(Uh, h, out->ld / 2, (__half *)out->planes, out->unscale);
+    SAT_LAUNCHED(ctx);
+    return SAT_OK;
+}
+
+sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const SatRecurrent &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
                         float *cell, int write_cell)
 {
     if (rows == 0 || n_steps == 0) return SAT_OK;
     if (n_steps > SAT_SEQ_MAX || h > 64 || (h & 3)) return sat_fail(ctx, SAT_EINVAL, "sat_lstm_seq: at most %d steps and 64 units", SAT_SEQ_MAX);
     ProfScope prof(ctx, SATK_GEMM_SIDE, 4.0 * (double)rows * h * (4.0 * n_steps + 1.0 + (first ? 0.0 : 2.0)), 8.0 * (double)rows * h * h * (n_steps - (first ? 1 : 0)));
-    const int32_t bn = tile_n_for(4 * h), nkb = (h + TC_BK - 1) / TC_BK;
-    const size_t smem = (size_t)2 * nkb * 2 * TC_BM * TC_BK * 4 + (size_t)nkb * 2 * (bn / 2) * TC_BK * 4 + sizeof(SeqShared) + 1024;
+    const int32_t bn = tile_n_for(4 * h), nkb = (h + SEQ_BK - 1) / SEQ_BK;
+    const size_t smem = (size_t)nkb * (2 * TC_BM + bn) * 128 + (size_t)SEQ_RING * 4 * SEQ_THREADS * 16 + sizeof(SeqShared) + 1024;
     static PerDeviceOnce attr_set;
     if (attr_set.need(ctx->device)) {
         SAT_CUDA(ctx, cudaFuncSetAttribute(k_lstm_seq, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set.mark(ctx->device);
     }
-    CUtensorMap mB, mBlo;
-    SAT_TRY(make_map(ctx, &mB, Uh.hi, Uh.ld, Uh.n_pad, Uh.ld, TC_BK, bn / 2, CU_TENSOR_MAP_SWIZZLE_64B));
-    SAT_TRY(make_map(ctx, &mBlo, Uh.lo, Uh.ld, Uh.n_pad, Uh.ld, TC_BK, bn / 2, CU_TENSOR_MAP_SWIZZLE_64B));
+    CUtensorMap mB;
+    PFN_encodeTiled enc = get_encode();
+    if (!enc) return sat_fail(ctx, SAT_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    const cuuint64_t gdim[2] = {(cuuint64_t)Uh.ld, (cuuint64_t)Uh.n_pad}, gstr[1] = {(cuuint64_t)Uh.ld * 2};
+    const cuuint32_t box[2] = {2 * SEQ_BK, (cuuint32_t)bn}, estr[2] = {1, 1};
+    if (enc(&mB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, Uh.planes, gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return sat_fail(ctx, SAT_EINVAL, "cuTensorMapEncodeTiled failed for the recurrent weights");
     SeqSteps st;
     for (int32_t t = 0; t < SAT_SEQ_MAX; ++t) st.proj[t] = t < n_steps ? proj[t] : nullptr;
-    const int64_t tiles = cdiv64(rows, 2 * TC_BM), units = ctx->sms / 2;
-    sat_pdl(ctx->stream, k_lstm_seq, (unsigned)(tiles < units ? tiles : units) * 2, SEQ_THREADS, smem, 2)(mB, mBlo, st, n_steps, first, rows, h, bn, nkb, S, cell,
-                                                                                                write_cell, ctx->d_flag + 1);
+    const int64_t tiles = cdiv64(rows, TC_BM);
+    sat_pdl(ctx->stream, k_lstm_seq, (unsigned)(tiles < ctx->sms ? tiles : ctx->sms), SEQ_THREADS, smem)(mB, Uh.unscale, st, n_steps, first, rows, h, bn, nkb, S, cell,
+                                                                                              write_cell, ctx->d_flag + 1);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }

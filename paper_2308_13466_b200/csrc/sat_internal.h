@@ -556,12 +556,19 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
                           int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0, int gates = 4, const float *bias = nullptr);
 sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out);
+// Recurrent weights of a predictor as half-precision pairs for sat_lstm_seq
+struct SatRecurrent {
+    void *planes = nullptr;      // __half [n_pad][k-steps][16 hi | 16 lo]
+    float *unscale = nullptr;    // [n_pad / 32] inverse of the scale
+    int32_t ld = 0, n_pad = 0;   // halves of a column; gate columns, padded
+};
+sat_status sat_pack_recurrent(sat_ctx *ctx, const float *Uh, int32_t h, DevBuf &buf, bool ready, SatRecurrent *out);
 // Plane of an input projection x Wx + b of the LSTM, [row tile of 128][unit][row of the tile][i f g o]
 inline int64_t sat_proj_floats(int64_t rows, int32_t h) { return (rows + 127) / 128 * 512 * h; }
 // LSTM steps over `n_steps` projection planes, oldest first, on the state S [rows x h] and the cell state (sat_cell_offset layout; read
-// unless `first`, i.e. both start from zero; written with write_cell).  Uh packed with gate_h; h a multiple of 4 up to 64.
+// unless `first`, i.e. both start from zero; written with write_cell).  h a multiple of 4 up to 64.
 #define SAT_SEQ_MAX 32
-sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
+sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const SatRecurrent &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
                         float *cell, int write_cell);
 // C[m x n] = [A | A2] B^T (+ epilogue)
 sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32_t lda, int32_t k1, const float *A2, int32_t lda2, int32_t k2,

@@ -286,7 +286,8 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
         c->proj_h = h;
         c->proj_tag.assign(ctx->tau + 1, 0);
     }
-    TcWeights Wp, Wxu, Up;   // Wx alone, [Wx ; Uh], Uh alone (all gate-interleaved)
+    TcWeights Wp, Wxu;   // Wx alone, [Wx ; Uh] (gate-interleaved)
+    SatRecurrent Up;     // Uh alone
     bool have_wp = false, have_wxu = false, have_up = false;
     if (c->pk_h != h) {      // another predictor width: nothing packed fits
         c->tag_wx = c->tag_uh = c->tag_wg = c->tag_b = c->tag_bg = 0;
@@ -327,14 +328,8 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
                 planes[n] = c->proj + (int64_t)ring_index(ctx, k - 1 - t - n) * plane;
                 ++n;
             }
-            if (!have_up) {
-                if (c->tag_uh == p->version) {
-                    SAT_TRY(sat_tc_weights_layout(h, 4 * h, c->pk_uh, &Up));
-                } else {
-                    SAT_TRY(sat_tc_weights(ctx, p->Uh, 4 * h, h, nullptr, 0, 0, 4 * h, 1, c->pk_uh, &Up, h));
-                    c->tag_uh = p->version;
-                }
-            }
+            if (!have_up) SAT_TRY(sat_pack_recurrent(ctx, p->Uh, h, c->pk_uh, c->tag_uh == p->version, &Up));
+            c->tag_uh = p->version;
             have_up = true;
             SAT_TRY(sat_lstm_seq(ctx, rows, h, Up, planes, n, t == 0, c->S, cell, t + n < k));
             t += n;

@@ -461,7 +461,7 @@ def test_pairs_give_the_bits_of_single_ctas_every_time(B, n, k):
 
 @pytest.mark.parametrize("h", [20, 64])
 def test_lstm_steps_repeat_themselves(B, h):
-    """The state after five steps over cached projections, more than one tile per slot of a CTA pair: the same bits in every run."""
+    """The state after five steps over cached projections, more than one tile per slot of a CTA: the same bits in every run."""
     n, d, tau = 120000, 32, 5
     ids = np.arange(n)
     col = np.sort(np.stack([(ids - 1) % n, (ids + 1) % n], 1), 1).astype(np.int32).ravel()
@@ -487,6 +487,57 @@ def test_lstm_steps_repeat_themselves(B, h):
         B.sat_sync_status(ctx)
     finally:
         B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("h", [16, 28])
+def test_lstm_cell_at_its_limits(B, h):
+    """Pre-activations far beyond the gates' saturation, and infinite or undefined ones in single rows, over cached projections: the limits of the
+    cell (to 2^-20, the error of a gate), a NaN stays a NaN, and every other row is as it is without them."""
+    n, d, tau = 600, 16, 3
+    ids = np.arange(n)
+    col = np.sort(np.stack([(ids - 1) % n, (ids + 1) % n], 1), 1).astype(np.int32).ravel()
+    rng = np.random.default_rng(h)
+    x = rng.standard_normal((n, d)).astype(np.float32)
+    x[:200] *= np.exp2(rng.integers(0, 40, (200, 1))).astype(np.float32)
+    Wx, b = np.zeros((d, 4 * h), np.float32), rng.standard_normal(4 * h).astype(np.float32) / 4
+    Wx[rng.integers(0, d, 4 * h), np.arange(4 * h)] = 2.0 ** rng.integers(-2, 3, 4 * h)      # one term each: the projections have no rounding but the bias's
+    Uh, Wg, bg = np.zeros((h, 4 * h), np.float32), np.zeros((h, d), np.float32), np.zeros(d, np.float32)
+    bad = {300: np.nan, 417: np.inf, 599: -np.inf}
+    states = []
+    for with_bad in (False, True):
+        xs = x.copy()
+        if with_bad:
+            for r, v in bad.items():
+                xs[r, :] = v
+        ctx = B.sat_create(0, 0)
+        try:
+            B.sat_graph_load(ctx, 2 * np.arange(n + 1, dtype=np.int64), col)
+            B.sat_partition(ctx, 2, B.SAT_PART_GIVEN, (ids % 2).astype(np.int32))
+            B.sat_cache_init(ctx, [d], tau)
+            perm = np.concatenate([np.flatnonzero(ids % 2 == m) for m in range(2)])
+            out = empty2d(n, d)
+            p = B.make_pred_params(*(dev(a) for a in (Wx, Uh, b, Wg, bg)), h, 1)
+            for _ in range(tau):
+                B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, dev2d(xs[perm]))
+                B.sat_cache_commit(ctx)
+                B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, p, 0, out)
+            slot = np.asarray(B.sat_slot_map(ctx, n)[1])
+            states.append(B.sat_predict_state(ctx, 1, n, h)[slot])
+            B.sat_sync_status(ctx)
+        finally:
+            B.sat_destroy(ctx)
+    rest = np.setdiff1d(ids, list(bad))
+    assert np.array_equal(states[0][rest], states[1][rest])
+    assert np.isnan(states[1][list(bad)]).all()
+    z = x.astype(np.float64) @ Wx + b
+    zi, zf, zg, zo = np.split(np.clip(z, -700, 700), 4, axis=1)
+    sig = lambda v: 1 / (1 + np.exp(-v))
+    c, e = 0.0, ((np.abs(x) @ np.abs(Wx) + np.abs(b)) * 2.0 ** -20).reshape(n, 4, h)
+    e = np.minimum(e, 2.0) * np.stack([sig(v) * sig(-v) for v in (zi, zf, 2 * zg, zo)], 1) * 4 + 2.0 ** -20      # slope of the gates at z, four times it for tanh
+    for _ in range(tau):
+        c = sig(zf) * c + sig(zi) * np.tanh(zg)
+    s = sig(zo) * np.tanh(c)
+    assert (np.abs(states[0] - s) <= 3 * tau * e.sum(1)).all()
 
 
 def _many_runs(kind):
