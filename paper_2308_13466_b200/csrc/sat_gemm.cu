@@ -331,8 +331,7 @@ sat_status sat_gemm_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const f
 //   row block, added in block order by k_splitk_reduce.  128 threads: thread t owns the TM columns TM (t % 64) .. of A and one half
 //   (t / 64) of the columns of B, so that a staged row costs it TM / 4 + NT / 8 128-bit shared loads for TM NT / 2 FMAs.  (Two columns
 //   of A against all of B, the first layout, took 1 + NT / 4 loads for the same FMAs.)  NT goes in steps of 8 so that little of it is
-//   padding.  Bound by FMA issue and the shared loads that feed it: 169 k x 256 x 40 115 -> 93 us (48 us of FMAs, 31 us of reads),
-//   2,048 x 16 x 16 9.2 -> 4.5 us.
+//   padding.  Bound by FMA issue and the shared loads that feed it, 73 us of 85 at 169 k x 256 x 40 (44 us for the copies alone).
 // =====================================================================================
 #define TNN_STAGE 16
 __device__ __forceinline__ void tnn_cp16(void *smem_dst, const void *gsrc, bool valid)
@@ -392,7 +391,7 @@ k_gemm_tn_narrow(int64_t rows, int64_t rows_per_block, int32_t m, int32_t n, con
         }
         __syncthreads();
         const float *As = tnn_smem + s * STAGE_FLOATS, *Bs = As + TNN_STAGE * MC;
-#pragma unroll 2
+#pragma unroll 8   // the loads of later rows under the FMAs of earlier ones: 8 rows 85 us where 2 took 118 (169 k x 256 x 40), 21 for 28 at 21 k rows
         for (int rr = 0; rr < TNN_STAGE; ++rr) {
             float av[TM];
             if (TM == 4) {
