@@ -152,6 +152,7 @@ static void free_cache(sat_ctx *ctx)
         dev_free(&ctx->cache[i].buf);
         dev_free(&ctx->cache[i].S);
         dev_free(&ctx->cache[i].proj);
+        dev_free(&ctx->cache[i].row_max);
         sat_free_buf(ctx->cache[i].pk_wx);
         sat_free_buf(ctx->cache[i].pk_uh);
         sat_free_buf(ctx->cache[i].pk_wg);
@@ -167,6 +168,7 @@ static void free_layers(sat_ctx *ctx)
 {
     for (int i = 0; i <= SAT_MAX_LAYERS; ++i) {
         dev_free(&ctx->layers[i].agg);
+        dev_free(&ctx->layers[i].agg_max);
         dev_free(&ctx->layers[i].mask);
         ctx->layers[i] = LayerState();
         dev_free(&ctx->ghist[i].buf);
@@ -216,6 +218,7 @@ extern "C" sat_status sat_destroy(sat_ctx *ctx)
     sat_free_buf(ctx->buf_ghist_out);
     sat_free_buf(ctx->buf_gat);
     sat_free_buf(ctx->buf_gat_items);
+    sat_free_buf(ctx->buf_q_max);
     if (ctx->d_flag) cudaFree(ctx->d_flag);
     if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
     delete ctx;

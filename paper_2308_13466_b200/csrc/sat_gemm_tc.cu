@@ -24,6 +24,7 @@
 
 #define TC_BM 128
 #define TC_BK 16          /* fp32 elements per k-block: 64-byte rows */
+#define TCH_BK 32         /* K-major kernel on half-precision pairs: elements per k-block, 128-byte rows of fp32 and of [hi | lo] halves alike */
 #define TC_WAIT_LIMIT (1u << 22)
 
 // =====================================================================================
@@ -167,13 +168,19 @@ __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t
         else TC_MMA_ASM("1", "tf32", "");
     }
 }
-// the same with half-precision operands (single CTAs)
-template <int USE_A>
+// the same with half-precision operands
+template <int USE_A, int GROUP>
 __device__ __forceinline__ void tc_mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
-    if (USE_A == 1) TC_MMA_ASM("1", "f16", ".collector::a::fill");
-    else if (USE_A == 2) TC_MMA_ASM("1", "f16", ".collector::a::lastuse");
-    else TC_MMA_ASM("1", "f16", "");
+    if (GROUP == 2) {
+        if (USE_A == 1) TC_MMA_ASM("2", "f16", ".collector::a::fill");
+        else if (USE_A == 2) TC_MMA_ASM("2", "f16", ".collector::a::lastuse");
+        else TC_MMA_ASM("2", "f16", "");
+    } else {
+        if (USE_A == 1) TC_MMA_ASM("1", "f16", ".collector::a::fill");
+        else if (USE_A == 2) TC_MMA_ASM("1", "f16", ".collector::a::lastuse");
+        else TC_MMA_ASM("1", "f16", "");
+    }
 }
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t *r)
 {
@@ -305,6 +312,14 @@ __device__ __forceinline__ void mbar_arrive_warp(uint64_t *bar, int lane)
             "}" ::"r"(smem_u32(bar))
             : "memory");
 }
+// lane 0's arrival on the same barriers with single CTAs too
+template <int CTAS>
+__device__ __forceinline__ void mbar_arrive_lane0(uint64_t *bar, int lane)
+{
+    __syncwarp();
+    if (CTAS == 2) mbar_arrive_warp<CTAS>(bar, lane);
+    else if (lane == 0) mbar_arrive(bar);
+}
 // make generic-proxy shared-memory writes visible to the tensor-core (async) proxy
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -312,6 +327,13 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 // K-major kernel
 // =====================================================================================
 struct TcEpilogue {
+    // (half-precision pairs)
+    const uint32_t *row_max; // [row_parts][row_stride] bits of the largest magnitude in each part of a row of A
+    int64_t row_stride;
+    int32_t row_parts;
+    uint32_t row_least;      // what the largest magnitude is taken to be at least (bits)
+    int32_t k1, k2;          // terms of the A operands
+    const float *unscale;    // inverse scale of every eight columns of B
     float *C;
     int64_t ldc;
     const float *bias;
@@ -327,6 +349,7 @@ struct TcEpilogue {
     int lstm_first;
     float *lstm_c;       // cell state in the blocked layout of sat_cell_offset
     int32_t proj_h;      // (EPI_PROJ) hidden units: C is a projection plane, see sat_proj_floats
+    RowMaxOut push_max;  // (EPI_PUSH; or none) largest magnitude of every pushed row: part 2 (column tile) + (half of the epilogue warps), by slot
     float *push_dst;     // (EPI_PUSH) row i is also written to push_dst + push_slot[i] * ld_push when push_slot[i] >= 0
     const int32_t *push_slot;
     int64_t ld_push;
@@ -603,21 +626,10 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             const bool row_ok = row < M;
             float *crow = ep.C + row * ep.ldc;
             float *prow = nullptr;   // (EPI_PUSH) this row's home in the cache ring, if it has one
-            // (EPI_PUSH with the staged store) the push goes out of the staging tile, four rows of 128 bytes per warp
-            // instruction: lane L writes 16-byte piece L & 7 of rows (L >> 3) + 4 i, so it needs those rows' ring rows
-            int32_t ps8[8];
-            if (EPI == EPI_PUSH && !use_tma_store && row_ok) {
-                const int32_t ps = __ldg(ep.push_slot + row);
-                if (ps >= 0) prow = ep.push_dst + (int64_t)ps * ep.ld_push;
-            }
-            if (EPI == EPI_PUSH && use_tma_store) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int64_t rr = m0 + q * 32 + (lane >> 3) + 4 * i;
-                    ps8[i] = rr < M ? __ldg(ep.push_slot + rr) : -1;
-                }
-            }
+            const int32_t push_slot = EPI == EPI_PUSH && row_ok ? __ldg(ep.push_slot + row) : -1;
+            if (EPI == EPI_PUSH && !use_tma_store && push_slot >= 0) prow = ep.push_dst + (int64_t)push_slot * ep.ld_push;
             float4 side[8], cside[2];
+            float largest = 0.f;   // (EPI_PUSH) of this thread's chunks
             // previous cell state (GRU: hidden state) of the next chunk, fetched one chunk ahead (two 128-bit loads per thread)
             auto load_cell = [&](int c0) {
                 if (LSTM) {
@@ -733,6 +745,10 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 #pragma unroll
                         for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(fmaxf(__uint_as_float(r[j]), 0.f));
                     }
+                    if (EPI == EPI_PUSH && ep.push_max.p) {
+#pragma unroll
+                        for (int j = 0; j < 32; j += 2) largest = fmaxf(largest, fmaxf(fabsf(__uint_as_float(r[j])), fabsf(__uint_as_float(r[j + 1]))));
+                    }
                     if (EPI == EPI_PLAIN && ep.mask_in) {
                         const int32_t word = (n0 + c0) >> 5;
                         const uint32_t keep = word < ep.mask_in_words ? __ldg(ep.mask_in + row * ep.mask_in_words + word) : 0u;
@@ -784,9 +800,10 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         const int32_t colb = n0 + c0 + 4 * piece;
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            if (ps8[i] < 0 || colb >= N) continue;
-                            float *pr = ep.push_dst + (int64_t)ps8[i] * ep.ld_push;
                             const int rr = (lane >> 3) + 4 * i;
+                            const int32_t slot = __shfl_sync(0xffffffffu, push_slot, rr);
+                            if (slot < 0 || colb >= N) continue;
+                            float *pr = ep.push_dst + (int64_t)slot * ep.ld_push;
                             const uint4 x = *reinterpret_cast<const uint4 *>(obuf + rr * 128 + ((piece ^ (rr & 7)) << 4));
                             if (colb + 3 < N) {
                                 *reinterpret_cast<uint4 *>(pr + colb) = x;
@@ -817,6 +834,9 @@ k_gemm_tc_k(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             }
             tc_fence_before();
             mbar_arrive_warp<CTAS>(&sh->acc_empty[buf], lane);  // the accumulator buffer may be overwritten by the tile after next
+            if (EPI == EPI_PUSH && ep.push_max.p) {
+                if (push_slot >= 0) ep.push_max.p[(2 * (t % n_tiles_n) + (e >> 2)) * ep.push_max.stride + push_slot] = __float_as_uint(largest);
+            }
         }
         if (use_tma_store && lane == 0) tma_store_wait_all();
         if (RING > 0) cp_async_wait<0>();
@@ -826,6 +846,462 @@ done:
     __syncthreads();
     if (CTAS == 2) cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
     if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tc_dealloc<CTAS>(tmem, 512u);
+    }
+}
+
+// =====================================================================================
+// K-major kernel on half-precision pairs, for contractions of many terms (sat_tc_half)
+// =====================================================================================
+#define TCH_STAGES_MAX 8
+#define TCH_A_BYTES (TC_BM * 128)      /* a k-block of A, raw or split */
+struct TchShared {
+    uint64_t full[TCH_STAGES_MAX];       // TMA bytes of the stage have landed
+    uint64_t conv[TCH_STAGES_MAX];       // the converter threads have split the stage
+    uint64_t empty[TCH_STAGES_MAX];      // the MMAs reading the stage have completed
+    uint64_t acc_full[2];   // accumulator buffer holds a finished tile
+    uint64_t acc_empty[2];  // accumulator buffer has been drained by the epilogue
+    uint64_t b_full, b_ready;   // a resident B has landed in this CTA; in all of them
+    uint32_t tmem_base;
+    int dead;
+};
+
+/* 640 threads.  Warps 0-7 convert, in two groups on alternate k-blocks, 8 is the TMA producer, 9 owns the TMEM and issues the MMAs: 72
+ * registers each (10 and 11 fill their warpgroup).  12-19 are the epilogue, which holds whole chunks of columns: 128. */
+#define TCH_THREADS 640
+#define TCH_EPI_WARPS 8
+
+template <int EPI> struct TchCfg { static constexpr int out_bytes = TCH_EPI_WARPS * 4096; };
+template <> struct TchCfg<EPI_LSTM> { static constexpr int out_bytes = 0; };
+template <> struct TchCfg<EPI_GRU> : TchCfg<EPI_LSTM> {};
+template <> struct TchCfg<EPI_PROJ> : TchCfg<EPI_LSTM> {};
+
+// Persistent: each CTA (CTAS = 1) or pair of CTAs (2) walks tiles unit, unit + units, ... of 128 or 256 rows.  A pair's MMA
+// (cta_group::2) multiplies the 128 rows of either CTA with all columns of B, of which each CTA holds half.  The shared-memory ring of
+// k-block stages and the two TMEM accumulator buffers let the TMA loads, the split, the MMAs and the epilogue of consecutive tiles
+// overlap.
+//
+// A arrives as raw fp32 rows of 128 bytes (32 values).  A converter thread owns a row: it reads 16 of its values, scales and splits them
+// (split_f16) and puts the 16 hi and 16 lo halves in their place, so that a k-step's operands are 32 bytes of every row of a K-major
+// tile.  B was packed like that once (k_pack_half), so a k-block is one TMA load of each.
+//
+// The scale is that of the whole row: the kernel is told the largest element of every row (RowMax) by whoever wrote the matrix, since looking for it
+// here meant fetching A twice.  The epilogue takes the scales back out (powers of two: exact).
+//
+// The TMA unit delivers 34 bytes per clock and SM, whatever it is asked for (four clocks per 128-byte row), which bound the form with TF32 terms
+// (48 KB of A, B and B's second plane per 32 terms); here it is 32 KB, and 16 where B stays in shared memory.
+// 169343 rows, TF32 terms -> pairs, us: 256 -> 256 88 -> 70, 256 -> 40 57 -> 42, projections 256 -> 256 89 -> 72; 179250 rows: 512 -> 512
+// 320 -> 195, projections 512 -> 256 185 -> 119, 512 -> 512 with the push 378 -> 280.  Errors against 64 bits are half of the TF32 form's
+// (embeddings of the first layer of 169343 nodes 1.2e-6 -> 5.7e-7).  (Rows pushed by the two idle warps instead of the epilogue: 120 -> 193.)
+// The epilogue is that of k_gemm_tc_k without the gathered residual, on eight warps.
+template <int EPI, int CTAS>
+__global__ void __launch_bounds__(TCH_THREADS, 1)
+k_gemm_tc_h(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapA2, const __grid_constant__ CUtensorMap mapB,
+            const __grid_constant__ CUtensorMap mapC, int use_tma_store, uint32_t stages, uint32_t out_tiles, int b_resident,
+            int64_t M, int32_t N, int32_t nkb1, int32_t nkb2, int32_t bn, int32_t n_tiles_n, int64_t n_tiles, TcEpilogue ep, int *status)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    constexpr uint32_t a_bytes = TCH_A_BYTES;                // a k-block of A: 128 rows x 128 B, raw or split
+    const uint32_t b_bytes = (uint32_t)bn / CTAS * 128;      // of B: [hi | lo], a CTA of a pair holds half of the columns
+    const uint32_t stage_bytes = a_bytes + (b_resident ? 0 : b_bytes);
+    const uint32_t rank = CTAS == 2 ? blockIdx.x & 1u : 0u;  // in the pair; CTA 0 issues the MMAs of both
+    const int64_t unit = blockIdx.x / CTAS, units = gridDim.x / CTAS;
+    uint8_t *b_all = smem + (size_t)stages * stage_bytes;       // (b_resident) B's k-blocks of this CTA's columns
+    uint8_t *out_stage = b_all + (b_resident ? (nkb1 + nkb2) * b_bytes : 0);   // staging blocks of the epilogue
+    constexpr int CONV_WARPS = 8, TMA_WARP = 8, MMA_WARP = 9, EPI_WARP0 = 12, EPI_WARPS = TCH_EPI_WARPS;
+    constexpr int CHUNK_STEP = 32 * (EPI_WARPS / 4);  // the EPI_WARPS / 4 warps of a TMEM lane quadrant take 32-column chunks in turn
+    TchShared *sh = (TchShared *)(out_stage + TchCfg<EPI>::out_bytes * out_tiles);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int32_t nkb = nkb1 + nkb2;
+    const uint32_t acc_cols = 256;  // column stride between the two accumulator buffers
+
+    if (threadIdx.x == 0) {
+        for (uint32_t s = 0; s < stages; ++s) {
+            mbar_init(&sh->full[s], 1);
+            mbar_init(&sh->conv[s], CTAS * (CONV_WARPS / 2));
+            mbar_init(&sh->empty[s], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sh->acc_full[i], 1);
+            mbar_init(&sh->acc_empty[i], CTAS * EPI_WARPS);
+        }
+        mbar_init(&sh->b_full, 1);
+        mbar_init(&sh->b_ready, CTAS);
+        sh->dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == MMA_WARP) {
+        tc_alloc<CTAS>(&sh->tmem_base, 512u);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (CTAS == 2) cluster_sync();   // the other CTA's barriers are initialised and its TMEM is allocated
+    tc_fence_after();
+    const uint32_t tmem = sh->tmem_base;
+    volatile int *dead = &sh->dead;
+    sat_grid_wait();   // everything above is set-up of this block; no global memory has been touched
+    // exponent of the scale of a row of A (past the matrix: any)
+    auto row_scale = [&](int64_t row) {
+        uint32_t m = ep.row_least;
+        for (int32_t p = 0; p < ep.row_parts; ++p) m = max(m, __ldg(ep.row_max + p * ep.row_stride + (row < M ? row : M - 1)));
+        return f16_scale_exponent(m >> 23);
+    };
+    auto tile_row0 = [&](int64_t t) { return (tck_row_tile(ep, t, n_tiles_n) * CTAS + rank) * TC_BM; };   // first row of this CTA
+
+    if (warp < EPI_WARP0) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");   // 384 x 72 + 256 x 128 of the 640 x 96 registers at launch
+    if (warp == TMA_WARP) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            uint32_t s = 0, ph = 0;
+            if (b_resident) {   // (every tile of the CTA has the same columns)
+                mbar_expect_tx(&sh->b_full, (uint32_t)nkb * b_bytes);
+                for (int32_t kb = 0; kb < nkb; ++kb)
+                    tma_load_2d(b_all + kb * b_bytes, &mapB, &sh->b_full, kb * 2 * TCH_BK, (int32_t)(unit % n_tiles_n) * bn + (int32_t)rank * (bn / CTAS));
+            }
+            for (int64_t t = unit; t < n_tiles; t += units) {
+                const int32_t m0 = (int32_t)tile_row0(t);
+                const int32_t n0 = (int32_t)(t % n_tiles_n) * bn + (int32_t)rank * (bn / CTAS);
+                for (int32_t kb = 0; kb < nkb; ++kb) {
+                    if (!mbar_wait(&sh->empty[s], ph ^ 1u, dead, status)) goto done;
+                    uint8_t *st = smem + (size_t)s * stage_bytes;
+                    mbar_expect_tx(&sh->full[s], stage_bytes);
+                    if (kb < nkb1) tma_load_2d(st, &mapA, &sh->full[s], kb * TCH_BK, m0);
+                    else tma_load_2d(st, &mapA2, &sh->full[s], (kb - nkb1) * TCH_BK, m0);
+                    if (!b_resident) tma_load_2d(st + a_bytes, &mapB, &sh->full[s], kb * 2 * TCH_BK, n0);
+                    if (++s == stages) s = 0, ph ^= 1u;
+                }
+            }
+            // the pair's MMAs have signalled every stage: nothing arrives here any more once both CTAs may exit
+            for (uint32_t i = 0; CTAS == 2 && i < stages; ++i) {
+                if (!mbar_wait(&sh->empty[s], ph ^ 1u, dead, status)) goto done;
+                if (++s == stages) s = 0, ph ^= 1u;
+            }
+        }
+    } else if (warp == MMA_WARP && rank == 0) {
+        // ---------------- MMA issuer ----------------
+        // The whole warp walks the k-blocks and an elected lane issues: the operands of the instructions are then known to be uniform.
+        // (One lane doing all of it took 0.4 us per k-block, which bound the narrow tiles: 169343 x 40, K = 256: 70 -> 62 us.)
+        const uint32_t idesc = make_idesc_f16(TC_BM * CTAS, bn);
+        const uint64_t desc0 = make_desc(smem_u32(smem), 16, 1024, 2);
+        uint32_t s = 0, ph = 0, lt = 0;
+        if (b_resident && !mbar_wait_all(&sh->b_ready, 0, dead, status)) goto done;
+        for (int64_t t = unit; t < n_tiles; t += units, ++lt) {
+            const uint32_t buf = lt & 1u;
+            if (!mbar_wait_all(&sh->acc_empty[buf], ((lt >> 1) & 1u) ^ 1u, dead, status)) goto done;
+            tc_fence_after();
+            const uint32_t acc = tmem + buf * acc_cols;
+            for (int32_t kb = 0; kb < nkb; ++kb) {
+                // the converters arrive on conv[s] only after they have seen full[s] (the TMA bytes) themselves
+                if (!mbar_wait_all(&sh->conv[s], ph, dead, status)) goto done;
+                tc_fence_after();
+                // K-major, 128-byte swizzle: rows 128 B apart, 8-row groups 1024 B; a k-step (16 terms) takes 64 B of the row, its hi halves
+                // and then its lo halves.  Only the 14-bit start-address field (bytes >> 4) differs between the descriptors of a stage.
+                const uint64_t a_hi0 = desc0 + (uint64_t)((s * stage_bytes) >> 4);
+                const uint64_t b_hi0 = b_resident ? desc0 + (uint64_t)((stages * stage_bytes + (uint32_t)kb * b_bytes) >> 4) : a_hi0 + (a_bytes >> 4);
+                const int32_t left = kb < nkb1 ? ep.k1 - kb * TCH_BK : ep.k2 - (kb - nkb1) * TCH_BK;   // terms from here on (the rest of the block is zero)
+                if (elect_one()) {
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks) {
+                        if (ks == 1 && left <= 16) break;
+                        const uint64_t a_hi = a_hi0 + (uint64_t)(ks * 4), a_lo = a_hi + 2;
+                        const uint64_t b_hi = b_hi0 + (uint64_t)(ks * 4), b_lo = b_hi + 2;
+                        tc_mma_f16<1, CTAS>(acc, a_hi, b_hi, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                        tc_mma_f16<2, CTAS>(acc, a_hi, b_lo, idesc, 1u);
+                        tc_mma_f16<0, CTAS>(acc, a_lo, b_hi, idesc, 1u);
+                    }
+                    tc_commit<CTAS>(&sh->empty[s]);  // the stage is free once these MMAs have read it
+                }
+                if (++s == stages) s = 0, ph ^= 1u;
+            }
+            if (elect_one()) tc_commit<CTAS>(&sh->acc_full[buf]);
+        }
+    } else if (warp < CONV_WARPS) {
+        // ---------------- converters: the two-term split of the A tile of every k-block ----------------
+        const uint32_t grp = warp / (CONV_WARPS / 2);
+        const int r = threadIdx.x & (TC_BM - 1), sw = r & 7;   // this thread's row; 16-byte piece c of it sits at c ^ sw
+        if (b_resident && warp == 0) {
+            if (!mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
+            mbar_arrive_lane0<CTAS>(&sh->b_ready, lane);
+        }
+        uint32_t s = grp, ph = 0, odd = 0;    // next own stage; parity of the k-blocks before this tile
+        uint32_t next = unit < n_tiles ? row_scale(tile_row0(unit) + r) : 0;
+        for (int64_t t = unit; t < n_tiles; t += units) {
+            const float scale = __uint_as_float(next << 23);
+            if (t + units < n_tiles) next = row_scale(tile_row0(t + units) + r);   // a tile early
+            for (int32_t kb = (int32_t)(grp ^ odd); kb < nkb; kb += 2) {
+                if (!mbar_wait_all(&sh->full[s], ph, dead, status)) goto done;
+                uint8_t *const row = smem + s * stage_bytes + r * 128;
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {   // 16 values, whose 64 bytes the halves take
+                    float4 x[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) x[c] = *reinterpret_cast<const float4 *>(row + (((4 * ks + c) ^ sw) << 4));
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const float4 u = x[2 * c], v = x[2 * c + 1];
+                        uint4 hi, lo;
+                        split_f16(u.x * scale, u.y * scale, hi.x, lo.x);
+                        split_f16(u.z * scale, u.w * scale, hi.y, lo.y);
+                        split_f16(v.x * scale, v.y * scale, hi.z, lo.z);
+                        split_f16(v.z * scale, v.w * scale, hi.w, lo.w);
+                        *reinterpret_cast<uint4 *>(row + (((4 * ks + c) ^ sw) << 4)) = hi;
+                        *reinterpret_cast<uint4 *>(row + (((4 * ks + c + 2) ^ sw) << 4)) = lo;
+                    }
+                }
+                fence_async_smem();
+                mbar_arrive_lane0<CTAS>(&sh->conv[s], lane);
+                s += 2;
+                if (s >= stages) s -= stages, ph ^= 1u;
+            }
+            odd ^= (uint32_t)nkb & 1u;
+        }
+    }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
+        // ---------------- epilogue ----------------
+        // warp w reads TMEM lanes 32 (w % 4) .. +31 = rows of the tile, one row per thread; the warps of a lane quadrant
+        // take alternate 32-column chunks.
+        constexpr bool LSTM = EPI == EPI_LSTM || EPI == EPI_GRU;   // a recurrent cell
+        const int e = warp - EPI_WARP0;
+        const int q = warp & 3;
+        const int c_first = 32 * (e >> 2);
+        uint32_t staged = 0;   // blocks staged so far
+        const bool vec = ((ep.ldc & 3) == 0) && ((((uintptr_t)ep.C) & 15u) == 0);
+        const bool lstm_full = LSTM && (ep.lstm_h & 3) == 0;
+        const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+
+        uint32_t lt = 0;
+        for (int64_t t = unit; t < n_tiles; t += units, ++lt) {
+            const int64_t m0 = tile_row0(t);
+            const int32_t n0 = (int32_t)(t % n_tiles_n) * bn;
+            const uint32_t buf = lt & 1u;
+            const int64_t row = m0 + q * 32 + lane;
+            const bool row_ok = row < M;
+            float *crow = ep.C + row * ep.ldc;
+            float *prow = nullptr;   // (EPI_PUSH) this row's home in the cache ring, if it has one
+            const int32_t push_slot = EPI == EPI_PUSH && row_ok ? __ldg(ep.push_slot + row) : -1;
+            if (EPI == EPI_PUSH && !use_tma_store && push_slot >= 0) prow = ep.push_dst + (int64_t)push_slot * ep.ld_push;
+            float4 cside[2];
+            float largest = 0.f;   // (EPI_PUSH) of this thread's chunks
+            // previous cell state (GRU: hidden state) of the next chunk, fetched one chunk ahead (two 128-bit loads per thread)
+            auto load_cell = [&](int c0) {
+                if (LSTM) {
+                    cside[0] = cside[1] = zero4;
+                    const int32_t j0 = (n0 + c0) >> 2;
+                    if (row_ok && lstm_full && !ep.lstm_first && j0 + 7 < ep.lstm_h) {
+                        const float *cp = EPI == EPI_GRU ? crow + j0 : ep.lstm_c + sat_cell_offset(row, j0, ep.lstm_h);
+                        cside[0] = *reinterpret_cast<const float4 *>(cp);
+                        cside[1] = *reinterpret_cast<const float4 *>(cp + 4);
+                    }
+                }
+            };
+            if (c_first < bn) load_cell(c_first);
+            const float unscale = __uint_as_float((254u - row_scale(row)) << 23);
+            if (!mbar_wait_warp(&sh->acc_full[buf], (lt >> 1) & 1u, dead, status, lane)) goto done;
+            tc_fence_after();
+            for (int c0 = c_first; c0 < bn; c0 += CHUNK_STEP) {
+                uint32_t r[32];
+                tc_ld32(tmem + buf * acc_cols + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
+                float4 us = __ldg(reinterpret_cast<const float4 *>(ep.unscale + ((n0 + c0) >> 3)));   // takes the scales out, eight columns each
+                us.x *= unscale; us.y *= unscale; us.z *= unscale; us.w *= unscale;
+                const float us4[4] = {us.x, us.y, us.z, us.w};
+                if (LSTM) {
+                    // packed columns 4 j .. 4 j + 3 are the (i, f, g, o) pre-activations of hidden unit j
+                    if (row_ok) {
+                        const int32_t j0 = (n0 + c0) >> 2;
+                        const bool full = lstm_full && j0 + 7 < ep.lstm_h;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            float4 b4 = zero4;
+                            if (ep.bias) {
+                                const float4 bb = __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + c0) + u);
+                                b4.x += bb.x; b4.y += bb.y; b4.z += bb.z; b4.w += bb.w;
+                            }
+                            r[4 * u] = __float_as_uint(fmaf(__uint_as_float(r[4 * u]), us4[u >> 1], b4.x));
+                            r[4 * u + 1] = __float_as_uint(fmaf(__uint_as_float(r[4 * u + 1]), us4[u >> 1], b4.y));
+                            r[4 * u + 2] = __float_as_uint(fmaf(__uint_as_float(r[4 * u + 2]), us4[u >> 1], b4.z));
+                            r[4 * u + 3] = __float_as_uint(fmaf(__uint_as_float(r[4 * u + 3]), us4[u >> 1], b4.w));
+                        }
+                        float cprev[8];
+                        cprev[0] = cside[0].x; cprev[1] = cside[0].y; cprev[2] = cside[0].z; cprev[3] = cside[0].w;
+                        cprev[4] = cside[1].x; cprev[5] = cside[1].y; cprev[6] = cside[1].z; cprev[7] = cside[1].w;
+                        if (!ep.lstm_first && !full) {
+#pragma unroll
+                            for (int u = 0; u < 8; ++u)
+                                if (j0 + u < ep.lstm_h) cprev[u] = EPI == EPI_GRU ? crow[j0 + u] : ep.lstm_c[sat_cell_offset(row, j0 + u, ep.lstm_h)];
+                        }
+                        if (c0 + CHUNK_STEP < bn) load_cell(c0 + CHUNK_STEP);
+                        float sv[8], cv[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            if (EPI == EPI_GRU) {   // (r, z, n from the input, n from the state)
+                                const float gr = 1.f / (1.f + expf(-__uint_as_float(r[4 * u])));
+                                const float gz = 1.f / (1.f + expf(-__uint_as_float(r[4 * u + 1])));
+                                const float gn = tanhf(__uint_as_float(r[4 * u + 2]) + gr * __uint_as_float(r[4 * u + 3]));
+                                sv[u] = (1.f - gz) * gn + gz * cprev[u];
+                                continue;
+                            }
+                            const float gi = sigmoid_fast(__uint_as_float(r[4 * u]));
+                            const float gf = sigmoid_fast(__uint_as_float(r[4 * u + 1]));
+                            const float gg = tanh_fast(__uint_as_float(r[4 * u + 2]));
+                            const float go = sigmoid_fast(__uint_as_float(r[4 * u + 3]));
+                            cv[u] = gf * cprev[u] + gi * gg;
+                            sv[u] = go * tanh_fast(cv[u]);
+                        }
+                        if (full) {
+                            float4 *sd = reinterpret_cast<float4 *>(ep.C + row * ep.ldc + j0);
+                            if (EPI != EPI_GRU) {
+                                float4 *cd = reinterpret_cast<float4 *>(ep.lstm_c + sat_cell_offset(row, j0, ep.lstm_h));
+                                cd[0] = make_float4(cv[0], cv[1], cv[2], cv[3]);
+                                cd[1] = make_float4(cv[4], cv[5], cv[6], cv[7]);
+                            }
+                            sd[0] = make_float4(sv[0], sv[1], sv[2], sv[3]);
+                            sd[1] = make_float4(sv[4], sv[5], sv[6], sv[7]);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 8; ++u)
+                                if (j0 + u < ep.lstm_h) {
+                                    if (EPI != EPI_GRU) ep.lstm_c[sat_cell_offset(row, j0 + u, ep.lstm_h)] = cv[u];
+                                    ep.C[row * ep.ldc + j0 + u] = sv[u];
+                                }
+                        }
+                    }
+                    continue;
+                }
+                uint32_t bits = 0;
+                if (row_ok) {
+                    // bias is padded with zeros to the tile width and the accumulators of padded columns are exactly zero,
+                    // so no column predicate is needed (the stores clip)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        float4 b4 = zero4;
+                        if (ep.bias) {
+                            const float4 bb = __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + c0) + j);
+                            b4.x += bb.x; b4.y += bb.y; b4.z += bb.z; b4.w += bb.w;
+                        }
+                        r[4 * j] = __float_as_uint(fmaf(__uint_as_float(r[4 * j]), us4[j >> 1], b4.x));
+                        r[4 * j + 1] = __float_as_uint(fmaf(__uint_as_float(r[4 * j + 1]), us4[j >> 1], b4.y));
+                        r[4 * j + 2] = __float_as_uint(fmaf(__uint_as_float(r[4 * j + 2]), us4[j >> 1], b4.z));
+                        r[4 * j + 3] = __float_as_uint(fmaf(__uint_as_float(r[4 * j + 3]), us4[j >> 1], b4.w));
+                    }
+                    if ((EPI == EPI_PLAIN || EPI == EPI_PUSH) && ep.mask_out) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) bits |= (__uint_as_float(r[j]) > 0.f ? 1u : 0u) << j;
+                    }
+                    if (ep.relu) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(fmaxf(__uint_as_float(r[j]), 0.f));
+                    }
+                    if (EPI == EPI_PUSH && ep.push_max.p) {
+#pragma unroll
+                        for (int j = 0; j < 32; j += 2) largest = fmaxf(largest, fmaxf(fabsf(__uint_as_float(r[j])), fabsf(__uint_as_float(r[j + 1]))));
+                    }
+                    if (EPI == EPI_PLAIN && ep.mask_in) {
+                        const int32_t word = (n0 + c0) >> 5;
+                        const uint32_t keep = word < ep.mask_in_words ? __ldg(ep.mask_in + row * ep.mask_in_words + word) : 0u;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) r[j] = keep >> j & 1u ? r[j] : 0u;
+                    }
+                }
+                if (EPI == EPI_PROJ) {   // a warp's store of a unit is 512 contiguous bytes
+                    if (row_ok) {
+                        const int32_t j0 = (n0 + c0) >> 2;
+                        float4 *dst = reinterpret_cast<float4 *>(ep.C) + ((row >> 7) * ep.proj_h + j0) * 128 + (row & 127);
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (j0 + u < ep.proj_h)
+                                dst[u * 128] = make_float4(__uint_as_float(r[4 * u]), __uint_as_float(r[4 * u + 1]), __uint_as_float(r[4 * u + 2]),
+                                                           __uint_as_float(r[4 * u + 3]));
+                    }
+                    continue;
+                }
+                if (EPI == EPI_PUSH && prow) {   // one full 128-byte line per thread and chunk
+#pragma unroll
+                    for (int j4 = 0; j4 < 32; j4 += 4) {
+                        const int32_t colb = n0 + c0 + j4;
+                        if (colb + 3 < N) {
+                            *reinterpret_cast<uint4 *>(prow + colb) = make_uint4(r[j4], r[j4 + 1], r[j4 + 2], r[j4 + 3]);
+                        } else {
+#pragma unroll
+                            for (int jj = 0; jj < 4; ++jj)
+                                if (colb + jj < N) prow[colb + jj] = __uint_as_float(r[j4 + jj]);
+                        }
+                    }
+                }
+                if (use_tma_store) {
+                    // stage the 32 x 32 block (128-byte swizzle: 16-byte chunk j of row r sits at chunk j ^ (r & 7)) and
+                    // let the TMA write it as whole 128-byte row segments; rows / columns past the matrix are clipped
+                    // the block before, or the one before that, has left its staging tile
+                    if (lane == 0) {
+                        if (out_tiles == 2) tma_store_wait_read<1>();
+                        else tma_store_wait_read<0>();
+                    }
+                    uint8_t *const obuf = out_stage + (e * out_tiles + (staged++ & (out_tiles - 1))) * 4096;
+                    __syncwarp();
+                    uint8_t *dst = obuf + lane * 128;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        *reinterpret_cast<uint4 *>(dst + ((j ^ (lane & 7)) << 4)) = make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+                    fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) tma_store_2d(&mapC, obuf, n0 + c0, (int32_t)(m0 + q * 32));
+                    if (EPI == EPI_PUSH) {
+                        // the boundary rows also go to the cache ring, read back from the staged block: every instruction
+                        // writes whole 128-byte row segments (the per-thread form touches 32 different lines per instruction)
+                        // (lane L writes 16-byte piece L & 7 of rows (L >> 3) + 4 i)
+                        const int piece = lane & 7;
+                        const int32_t colb = n0 + c0 + 4 * piece;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int rr = (lane >> 3) + 4 * i;
+                            const int32_t slot = __shfl_sync(0xffffffffu, push_slot, rr);
+                            if (slot < 0 || colb >= N) continue;
+                            float *pr = ep.push_dst + (int64_t)slot * ep.ld_push;
+                            const uint4 x = *reinterpret_cast<const uint4 *>(obuf + rr * 128 + ((piece ^ (rr & 7)) << 4));
+                            if (colb + 3 < N) {
+                                *reinterpret_cast<uint4 *>(pr + colb) = x;
+                            } else {
+                                pr[colb] = __uint_as_float(x.x);
+                                if (colb + 1 < N) pr[colb + 1] = __uint_as_float(x.y);
+                                if (colb + 2 < N) pr[colb + 2] = __uint_as_float(x.z);
+                            }
+                        }
+                    }
+                } else if (row_ok) {
+#pragma unroll
+                    for (int j4 = 0; j4 < 32; j4 += 4) {
+                        const int32_t colb = n0 + c0 + j4;
+                        if (vec && colb + 3 < N) {
+                            *reinterpret_cast<uint4 *>(crow + colb) = make_uint4(r[j4], r[j4 + 1], r[j4 + 2], r[j4 + 3]);
+                        } else {
+#pragma unroll
+                            for (int jj = 0; jj < 4; ++jj)
+                                if (colb + jj < N) crow[colb + jj] = __uint_as_float(r[j4 + jj]);
+                        }
+                    }
+                }
+                if ((EPI == EPI_PLAIN || EPI == EPI_PUSH) && ep.mask_out && row_ok) {
+                    const int32_t word = (n0 + c0) >> 5;
+                    if (word < ep.mask_words) ep.mask_out[row * ep.mask_words + word] = bits;
+                }
+            }
+            tc_fence_before();
+            mbar_arrive_lane0<CTAS>(&sh->acc_empty[buf], lane);  // the accumulator buffer may be overwritten by the tile after next
+            if (EPI == EPI_PUSH && ep.push_max.p) {
+                if (push_slot >= 0) ep.push_max.p[(2 * (t % n_tiles_n) + (e >> 2)) * ep.push_max.stride + push_slot] = __float_as_uint(largest);
+            }
+        }
+        if (use_tma_store && lane == 0) tma_store_wait_all();
+    }
+done:
+    tc_fence_before();
+    __syncthreads();
+    if (CTAS == 2) cluster_sync();   // neither CTA's shared memory or TMEM is in use by the other any more
+    if (warp == MMA_WARP) {
         __syncwarp();
         tc_fence_after();
         tc_dealloc<CTAS>(tmem, 512u);
@@ -852,14 +1328,13 @@ done:
 // by a warp of their own per slot, which leaves 96 registers: 192 us.)  The errors are what they were (relative 1.6e-6 of the
 // state at K = 256).
 // =====================================================================================
-#define SEQ_BK 32         /* terms of a k-block: 128-byte rows */
 #define SEQ_THREADS 512   /* 128 registers a thread */
 #define SEQ_RING 3        /* quads of projections in flight per thread */
 struct SeqSteps {
     const float *proj[SAT_SEQ_MAX];
 };
 struct SeqShared {
-    float unscale[8];                                // per 32 gate columns, of the state and the columns together
+    float2 unscale[16];                              // per eight gate columns, of the state and the columns together
     uint64_t b_full;                                 // Uh has landed
     uint64_t a_ready[2], acc_full[2];                // per slot: the state is in place; the product is done
     uint32_t tmem_base;
@@ -934,13 +1409,13 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
     const uint32_t tmem = sh->tmem_base;
     volatile int *dead = &sh->dead;
     sat_grid_wait();
-    if (threadIdx.x < 8) sh->unscale[threadIdx.x] = 32 * (int)threadIdx.x < bn ? __ldg(unscale + threadIdx.x) * 0x1p-14f : 0.f;
+    if (threadIdx.x < 32) reinterpret_cast<float *>(sh->unscale)[threadIdx.x] = 8 * (int)threadIdx.x < bn ? __ldg(unscale + threadIdx.x) * 0x1p-14f : 0.f;
     __syncthreads();
 
     if (warp == 0 && mine > 0) {
         if (lane == 0) {
             mbar_expect_tx(&sh->b_full, (uint32_t)nkb * b_block);
-            for (int32_t kb = 0; kb < nkb; ++kb) tma_load_2d(Bs + (uint32_t)kb * b_block, &mapB, &sh->b_full, kb * 2 * SEQ_BK, 0);
+            for (int32_t kb = 0; kb < nkb; ++kb) tma_load_2d(Bs + (uint32_t)kb * b_block, &mapB, &sh->b_full, kb * 2 * TCH_BK, 0);
         }
         if (!mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
     }
@@ -1018,9 +1493,9 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
                             for (int32_t ks = 0; ks < nks; ++ks) {
                                 const uint64_t a_hi = a0 + (uint64_t)((ks >> 1) * (a_block >> 4) + (ks & 1) * 4), a_lo = a_hi + 2;
                                 const uint64_t b_hi = b0 + (uint64_t)((ks >> 1) * (b_block >> 4) + (ks & 1) * 4), b_lo = b_hi + 2;
-                                tc_mma_f16<1>(acc, a_hi, b_hi, idesc, ks > 0 ? 1u : 0u);
-                                tc_mma_f16<2>(acc, a_hi, b_lo, idesc, 1u);
-                                tc_mma_f16<0>(acc, a_lo, b_hi, idesc, 1u);
+                                tc_mma_f16<1, 1>(acc, a_hi, b_hi, idesc, ks > 0 ? 1u : 0u);
+                                tc_mma_f16<2, 1>(acc, a_hi, b_lo, idesc, 1u);
+                                tc_mma_f16<0, 1>(acc, a_lo, b_hi, idesc, 1u);
                             }
                             tc_commit<1>(&sh->acc_full[slot]);
                         }
@@ -1043,11 +1518,12 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
                         at = at + 1 == SEQ_RING ? 0 : at + 1;
                         if (product) {
                             uint32_t(&a)[16] = r[i & 1];
-                            const float us = sh->unscale[qd >> 1];
+                            const float2 us2 = sh->unscale[qd];
                             tc_wait16(a);
                             if (i < 7 && qd + 2 < nq) tc_ld16(mine_acc + 16u * (uint32_t)(qd + 2), r[(i + 1) & 1]);
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
+                                const float us = u < 2 ? us2.x : us2.y;
                                 z[u].x = fmaf(__uint_as_float(a[4 * u]), us, z[u].x);
                                 z[u].y = fmaf(__uint_as_float(a[4 * u + 1]), us, z[u].y);
                                 z[u].z = fmaf(__uint_as_float(a[4 * u + 2]), us, z[u].z);
@@ -1426,35 +1902,104 @@ __global__ void k_split_weights(const float *__restrict__ W, int64_t ldw, int32_
     lo[i] = tf32_residual(x);  // second plane: read by the variants that do not split B in the kernel
 }
 
-// Recurrent weights Uh [h x 4 h] (gate blocks i | f | g | o) as half-precision pairs for k_lstm_seq: packed column 4 j + g is gate g of unit j; per
-// column the k-steps of 16 one after the other, each 16 hi and 16 lo halves (split_f16), zero padded to whole k-blocks, and the inverse of
-// the scale of every 32 columns.  A block takes 32 columns.
-#define PACK_COLS 32
-__global__ void __launch_bounds__(1024)
-k_pack_recurrent(const float *__restrict__ U, int32_t h, int32_t k_all, __half *__restrict__ out, float *__restrict__ unscale)
+// B operand from fp32 weights: per packed column the k-steps of 16 one after the other, each 16 hi and 16 lo halves (split_f16), zero padded to
+// k-blocks of two k-steps, and the inverse of the column's scale.
+//   transpose = 1: W is [K x N] row-major (ldw) -> B[n][k] = W[k][n]          (C = A W)
+//   transpose = 0: W is [N x K] row-major (ldw) -> B[n][k] = W[n][k]          (C = A W^T)
+// A second source W2 (same orientation, k2 rows) continues along K with a k-block of its own.
+// A bias [n] is packed alike, zero padded (four gates with gates = 3 too).
+// gate_h > 0: packed column 4 j + g is gate g of hidden unit j.  gates = 4: the sources have the columns i | f | g | o.  gates = 3 (GRU,
+// sources r | z | n): the candidate's two parts stay apart, column 4 j + 2 takes n of the first source only and 4 j + 3 n of the second.
+// A block takes eight columns, which share a scale (at most 2^60).  Its threads keep their pairs of terms in registers between the search for the
+// largest and the split, PACK_PAIRS of them (a latency of the memory each time otherwise: 256 x 256 12 us -> 4), and look again at what is beyond.
+#define PACK_COLS 8
+#define PACK_PAIRS 8
+__global__ void __launch_bounds__(256)
+k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, const float *__restrict__ W2, int64_t ldw2, int32_t k2, int32_t nkb,
+                int32_t n, int transpose, int32_t gate_h, int gates, __half *__restrict__ out, float *__restrict__ unscale, const float *__restrict__ bias,
+                float *__restrict__ bias_out)
 {
     sat_grid_wait();
     __shared__ uint32_t largest;
-    const int32_t np0 = blockIdx.x * PACK_COLS;
-    auto value = [&](int32_t np, int32_t k) { return np < 4 * h && k < h ? U[(int64_t)k * 4 * h + (np & 3) * h + (np >> 2)] : 0.f; };
+    const int32_t np0 = blockIdx.x * PACK_COLS, pairs = nkb * (TCH_BK / 2);
+    auto value = [&](int32_t np, int32_t kk) {   // kk: term, the second source's from nkb1 k-blocks on
+        const int32_t g = np & 3, nn = gate_h > 0 ? (gates == 3 && g == 3 ? 2 : g) * gate_h + (np >> 2) : np;   // packed row -> logical column
+        const bool second = kk >= nkb1 * TCH_BK;
+        const int32_t k = second ? kk - nkb1 * TCH_BK : kk;
+        if (np >= n || k >= (second ? k2 : k1) || (gates == 3 && g == (second ? 2 : 3))) return 0.f;
+        const float *w = second ? W2 : W;
+        const int64_t ld = second ? ldw2 : ldw;
+        return __ldg(transpose ? w + k * ld + nn : w + nn * ld + k);
+    };
+    // consecutive threads along the rows of the sources: pair p of column c
+    const int32_t step_c = transpose ? 0 : 256 / pairs, step_p = transpose ? 32 : 256 % pairs;
+    int32_t c = transpose ? threadIdx.x % PACK_COLS : threadIdx.x / pairs, p = transpose ? threadIdx.x / PACK_COLS : threadIdx.x - c * pairs;
+    const int32_t c_first = c, p_first = p;
+    auto advance = [&]() {
+        c += step_c;
+        p += step_p;
+        if (!transpose && p >= pairs) p -= pairs, ++c;
+    };
+    auto inside = [&]() { return c < PACK_COLS && p < pairs; };
     if (threadIdx.x == 0) largest = 0;
-    __syncthreads();
-    uint32_t m = 0;
-    for (int32_t i = threadIdx.x; i < PACK_COLS * k_all; i += 1024) m = max(m, __float_as_uint(value(np0 + i % PACK_COLS, i / PACK_COLS)) & 0x7fffffffu);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(&largest, m);
-    __syncthreads();
-    const uint32_t e = f16_scale_exponent(largest >> 23);
-    const float s = __uint_as_float(e << 23);
-    for (int32_t i = threadIdx.x; i < PACK_COLS * (k_all / 2); i += 1024) {
-        const int32_t c = i % PACK_COLS, k = 2 * (i / PACK_COLS);
-        uint32_t hi, lo;
-        split_f16(value(np0 + c, k) * s, value(np0 + c, k + 1) * s, hi, lo);
-        uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(np0 + c) * (k_all / 16) + k / 16) * 32 + k % 16);
-        o[0] = hi;
-        o[8] = lo;
+    if (threadIdx.x < PACK_COLS) {
+        const int32_t np = np0 + (int32_t)threadIdx.x;
+        if (bias) bias_out[np] = np < n ? bias[gate_h > 0 ? (np & 3) * gate_h + (np >> 2) : np] : 0.f;
     }
+    __syncthreads();
+    float x[PACK_PAIRS][2], m = 0.f;
+#pragma unroll
+    for (int i = 0; i < PACK_PAIRS; ++i) {
+        const bool in = inside();
+        x[i][0] = in ? value(np0 + c, 2 * p) : 0.f;
+        x[i][1] = in ? value(np0 + c, 2 * p + 1) : 0.f;
+        advance();
+    }
+#pragma unroll
+    for (int i = 0; i < PACK_PAIRS; ++i) m = fmaxf(m, fmaxf(fabsf(x[i][0]), fabsf(x[i][1])));
+    for (; inside(); advance()) m = fmaxf(m, fmaxf(fabsf(value(np0 + c, 2 * p)), fabsf(value(np0 + c, 2 * p + 1))));
+    const uint32_t b = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) atomicMax(&largest, b);
+    __syncthreads();
+    const uint32_t e = min(f16_scale_exponent(largest >> 23), 187u);
+    const float s = __uint_as_float(e << 23);
+    auto put = [&](float x0, float x1) {
+        uint32_t h, l;
+        split_f16(x0 * s, x1 * s, h, l);
+        uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(np0 + c) * (pairs / 8) + p / 8) * 32 + 2 * (p % 8));
+        o[0] = h;
+        o[8] = l;
+    };
+    c = c_first;
+    p = p_first;
+#pragma unroll
+    for (int i = 0; i < PACK_PAIRS; ++i) {
+        if (inside()) put(x[i][0], x[i][1]);
+        advance();
+    }
+    for (; inside(); advance()) put(value(np0 + c, 2 * p), value(np0 + c, 2 * p + 1));
     if (threadIdx.x == 0) unscale[blockIdx.x] = __uint_as_float((254u - e) << 23);
+}
+
+// out[r] = bits of the largest magnitude in row r of A: a warp per row (for matrices whose writer did not leave it)
+__global__ void __launch_bounds__(256)
+k_row_max(const float *__restrict__ A, int64_t lda, int32_t d, int64_t rows, uint32_t *__restrict__ out)
+{
+    sat_grid_wait();
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (r >= rows) return;
+    float m = 0.f;
+#pragma unroll 4
+    for (int32_t c = 4 * lane; c < d; c += 128) {   // rows are padded to four floats; what stands there is not part of them
+        const float4 x = __ldg(reinterpret_cast<const float4 *>(A + r * lda + c));
+        m = fmaxf(m, fabsf(x.x));
+        if (c + 1 < d) m = fmaxf(m, fabsf(x.y));
+        if (c + 2 < d) m = fmaxf(m, fabsf(x.z));
+        if (c + 3 < d) m = fmaxf(m, fabsf(x.w));
+    }
+    const uint32_t b = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if (lane == 0) out[r] = b;
 }
 
 // =====================================================================================
@@ -1493,6 +2038,19 @@ static sat_status make_map(sat_ctx *ctx, CUtensorMap *map, const void *base, int
     return SAT_OK;
 }
 
+// packed weights, a k-block of `box_cols` columns at a time
+static sat_status make_map_weights(sat_ctx *ctx, CUtensorMap *map, const TcWeights &B, int box_cols)
+{
+    PFN_encodeTiled enc = get_encode();
+    if (!enc) return sat_fail(ctx, SAT_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    const cuuint64_t gdim[2] = {(cuuint64_t)B.ld, (cuuint64_t)B.n_pad}, gstr[1] = {(cuuint64_t)B.ld * 2};
+    const cuuint32_t box[2] = {2 * TCH_BK, (cuuint32_t)box_cols}, estr[2] = {1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, B.planes, gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return sat_fail(ctx, SAT_EINVAL, "cuTensorMapEncodeTiled failed (%d) for packed weights", (int)r);
+    return SAT_OK;
+}
+
 // output columns per tile: as few tiles of at most 256 as possible, of equal width (a multiple of 32)
 static int tile_n_for(int n)
 {
@@ -1509,6 +2067,14 @@ bool sat_use_tc(int32_t n, int32_t k)
     }
     return !no_tc && k >= 16 && n >= 16;
 }
+
+// The two forms of the K-major kernel.  Pairs pay where the contraction is long and the launch has more than a wave of row tiles; a short launch
+// takes as long either way and its weights take 4 us to pack instead of 2 (epoch of 12,833 nodes, 192-200-200-83 with a GRU of 8 units: 393 us
+// with TF32 terms, 424 with pairs), unless the contraction is very long (2,151 nodes, 21-512-512-35: 688 and 644).  A short
+// contraction is bound by its output, and the epilogue with TF32 terms is the shorter one (169343 x 256, K = 40: 47.5 and 50.7
+// us, K = 128 with the push 92 and 104).  The number of nodes stands for the rows of a launch, so that one partition and all of
+// them in one launch give the same bits.
+bool sat_tc_half(const sat_ctx *ctx, int32_t k) { return (k >= 384 || (k >= 192 && ctx->n >= 32768)) && sat_use_tc(16, k); }
 
 sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t rows, int32_t d, const uint32_t *mask, int32_t mask_words,
                          float *dst, int32_t ld_dst, float *colsum, int accumulate, const float *act, int32_t ld_act)
@@ -1531,9 +2097,32 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
     return SAT_OK;
 }
 
+// where weights packed as half-precision pairs with `nkb` k-blocks and n outputs lie in a buffer, and the bytes they take
+static size_t half_layout(int32_t nkb, int32_t n, void *base, TcWeights *out)
+{
+    const int32_t bn = tile_n_for(n);
+    out->n_pad = (n + bn - 1) / bn * bn;
+    out->ld = nkb * 2 * TCH_BK;
+    const size_t planes = (size_t)out->n_pad * out->ld * sizeof(__half);   // a multiple of 4 KB
+    out->planes = base;
+    out->unscale = (float *)((char *)base + planes);
+    out->bias = out->unscale + out->n_pad / PACK_COLS;   // 16-byte aligned: n_pad is a multiple of 32
+    return planes + ((size_t)out->n_pad + out->n_pad / PACK_COLS) * sizeof(float);
+}
+
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
                           int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h, int gates, const float *bias)
 {
+    if (out->half) {
+        const int32_t nkb1 = (int32_t)cdiv64(k1, TCH_BK), nkb = nkb1 + (W2 ? (int32_t)cdiv64(k2, TCH_BK) : 0);
+        SAT_TRY(sat_ensure(ctx, buf, half_layout(nkb, n, nullptr, out)));
+        half_layout(nkb, n, buf.p, out);
+        if (!bias) out->bias = nullptr;
+        sat_pdl(ctx->stream, k_pack_half, (unsigned)(out->n_pad / PACK_COLS), 256, 0)(W, ldw, k1, nkb1, W2, ldw2, k2, nkb, n, transpose, gate_h, gates,
+                                                                                  (__half *)out->planes, out->unscale, bias, out->bias);
+        SAT_LAUNCHED(ctx);
+        return SAT_OK;
+    }
     const int32_t k1_pad = W2 ? (k1 + TC_BK - 1) / TC_BK * TC_BK : k1;
     const int32_t k_tot = k1_pad + (W2 ? k2 : 0);
     const int32_t k_pad = (k_tot + TC_BK - 1) / TC_BK * TC_BK;
@@ -1555,6 +2144,11 @@ sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1,
 // the description of planes that an earlier sat_tc_weights call (single source, k terms, n outputs) left in `buf`
 sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out)
 {
+    if (out->half) {
+        if (!buf.p || buf.bytes < half_layout((int32_t)cdiv64(k, TCH_BK), n, buf.p, out)) return SAT_ESTATE;
+        out->bias = nullptr;
+        return SAT_OK;
+    }
     const int32_t k_pad = (k + TC_BK - 1) / TC_BK * TC_BK;
     const int32_t bn = tile_n_for(n);
     const int32_t n_pad = (n + bn - 1) / bn * bn;
@@ -1577,7 +2171,7 @@ struct TckLaunch {
     int32_t n, nkb1, nkb2, bn, n_tiles_n;
     int64_t n_tiles;
     unsigned grid;
-    uint32_t stage_bytes;
+    uint32_t stage_bytes, b_resident;   // (half-precision pairs) bytes of a resident B
 };
 
 template <int EPI, int CTAS>
@@ -1602,12 +2196,47 @@ static sat_status launch_tck(sat_ctx *ctx, const TckLaunch &L, const TcEpilogue 
     return SAT_OK;
 }
 
+template <int EPI, int CTAS>
+static sat_status launch_tch(sat_ctx *ctx, const TckLaunch &L, const TcEpilogue &ep)
+{
+    static PerDeviceOnce attr_set;
+    // As many stages as fit, since the bytes in flight bound the narrow contractions, but no more than the longest CTA has k-blocks, so that a
+    // small launch leaves room on the SM for its successor; an even number.
+    const int64_t cta_tiles = cdiv64(L.n_tiles, L.grid / CTAS), blocks = cta_tiles * (L.nkb1 + L.nkb2);
+    size_t fixed = TchCfg<EPI>::out_bytes + L.b_resident + sizeof(TchShared) + 1024;
+    // two staging tiles per epilogue warp where they leave room for six stages 
+    const uint32_t out_tiles = TchCfg<EPI>::out_bytes && cta_tiles > 1 && fixed + TchCfg<EPI>::out_bytes + 6 * L.stage_bytes <= 227 * 1024 ? 2 : 1;
+    fixed += (out_tiles - 1) * TchCfg<EPI>::out_bytes;
+    const int64_t fit = (227 * 1024 - (int64_t)fixed) / L.stage_bytes;
+    uint32_t stages = TCH_STAGES_MAX;
+    while (stages > 2 && (stages > fit || stages - 2 >= blocks)) stages -= 2;
+    const size_t smem = (size_t)stages * L.stage_bytes + fixed;
+    if (smem > 227 * 1024) return sat_fail(ctx, SAT_EINVAL, "tensor-core GEMM: shared-memory layout of %zu bytes does not fit", smem);
+    if (attr_set.need(ctx->device)) {
+        SAT_CUDA(ctx, cudaFuncSetAttribute(k_gemm_tc_h<EPI, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        attr_set.mark(ctx->device);
+    }
+    sat_pdl(ctx->stream, k_gemm_tc_h<EPI, CTAS>, L.grid, TCH_THREADS, smem, CTAS)(L.mA, L.mA2, L.mB, L.mC, L.use_tma_store, stages, out_tiles, L.b_resident > 0, L.m, L.n, L.nkb1, L.nkb2, L.bn, L.n_tiles_n,
+                                                                L.n_tiles, ep, ctx->d_flag + 1);
+    SAT_LAUNCHED(ctx);
+    return SAT_OK;
+}
+
+sat_status sat_row_max(sat_ctx *ctx, const float *A, int32_t lda, int32_t d, int64_t rows, uint32_t *out)
+{
+    if (rows == 0) return SAT_OK;
+    sat_pdl(ctx->stream, k_row_max, (unsigned)cdiv64(rows, 8), 256, 0)(A, lda, d, rows, out);
+    SAT_LAUNCHED(ctx);
+    return SAT_OK;
+}
+
 // C[m x n] = [A | A2] B^T with B = packed weights [n_pad x k_pad]
 sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32_t lda, int32_t k1, const float *A2, int32_t lda2, int32_t k2,
                        const TcWeights &Bw, const TcEpilogueHost &eh, int family)
 {
     if (m == 0 || n == 0) return SAT_OK;
-    const int32_t nkb1 = (k1 + TC_BK - 1) / TC_BK, nkb2 = A2 ? (k2 + TC_BK - 1) / TC_BK : 0;
+    const bool half = Bw.half;
+    const int32_t bk = half ? TCH_BK : TC_BK, nkb1 = (int32_t)cdiv64(k1, bk), nkb2 = A2 ? (int32_t)cdiv64(k2, bk) : 0;
     const int32_t bn = tile_n_for(n);
     // CTA pairs for launches of more than one wave of single CTAs (below, the pair only adds its synchronisation: 6000 x 72, K = 50: 12.0
     // -> 12.9 us), except with a gathered residual: that contracts over the predictor width and is bound by the residual's
@@ -1615,7 +2244,9 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     const int32_t n_tiles_n = (int32_t)cdiv64(n, bn);
     const bool pair = !eh.resid_idx && cdiv64(m, TC_BM) * n_tiles_n > ctx->sms;
     const int ctas = pair ? 2 : 1;
-    const uint32_t stage_bytes = 2 * (TC_BM * TC_BK * 4) + 2 * (uint32_t)bn / ctas * TC_BK * 4;
+    // a B of half-precision pairs of at most 128 KB per CTA stays in shared memory (its CTAs then keep to their columns)
+    const uint32_t b_bytes = (uint32_t)bn / ctas * 128, b_all = b_bytes * (nkb1 + nkb2), b_resident = half && b_all <= 131072u ? b_all : 0;
+    const uint32_t stage_bytes = half ? TCH_A_BYTES + (b_resident ? 0 : b_bytes) : 2 * (TC_BM * TC_BK * 4) + b_bytes;
     // algorithmic bytes: operands once, results once.  Plain: A, B, C.  Gathered residual: + the residual rows.  LSTM cell:
     // the output is the hidden state [m x h] plus the cell state read and written, and the cached projection if it is added.
     double alg_bytes = 4.0 * ((double)m * (k1 + k2) + (double)(k1 + k2) * n);
@@ -1626,12 +2257,27 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     const int use_tma_store = eh.lstm_h == 0 && eh.proj_h == 0 && ((eh.ldc & 3) == 0) && ((((uintptr_t)eh.C) & 15u) == 0);
     if (use_tma_store) SAT_TRY(make_map(ctx, &mC, eh.C, n, m, eh.ldc, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B));
     else memset(&mC, 0, sizeof(mC));
-    SAT_TRY(make_map(ctx, &mA, A, k1, m, lda, TC_BK, TC_BM, CU_TENSOR_MAP_SWIZZLE_64B));
-    if (A2) SAT_TRY(make_map(ctx, &mA2, A2, k2, m, lda2, TC_BK, TC_BM, CU_TENSOR_MAP_SWIZZLE_64B));
+    const CUtensorMapSwizzle swz = half ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    SAT_TRY(make_map(ctx, &mA, A, k1, m, lda, bk, TC_BM, swz));
+    if (A2) SAT_TRY(make_map(ctx, &mA2, A2, k2, m, lda2, bk, TC_BM, swz));
     else mA2 = mA;
-    SAT_TRY(make_map(ctx, &mB, Bw.hi, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / ctas, CU_TENSOR_MAP_SWIZZLE_64B));
-    SAT_TRY(make_map(ctx, &mBlo, Bw.lo, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / ctas, CU_TENSOR_MAP_SWIZZLE_64B));
+    if (half) {
+        SAT_TRY(make_map_weights(ctx, &mB, Bw, bn / ctas));
+        mBlo = mB;
+    } else {
+        SAT_TRY(make_map(ctx, &mB, Bw.hi, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / ctas, swz));
+        SAT_TRY(make_map(ctx, &mBlo, Bw.lo, Bw.ld, Bw.n_pad, Bw.ld, TC_BK, bn / ctas, swz));
+    }
     TcEpilogue ep;
+    if (half && (!eh.rows.p || eh.resid_idx)) return sat_fail(ctx, SAT_EINVAL, "a contraction on half-precision pairs needs the largest magnitudes of its rows and has no residual");
+    ep.row_max = eh.rows.p;
+    ep.row_stride = eh.rows.stride;
+    ep.row_parts = eh.rows.parts;
+    ep.row_least = A2 ? 0x3f800000u : 0u;   // a second operand is a hidden state, which lies in [-1, 1]
+    ep.k1 = k1;
+    ep.k2 = A2 ? k2 : 0;
+    ep.unscale = Bw.unscale;
+    ep.push_max = eh.push_max;
     ep.C = eh.C;
     ep.ldc = eh.ldc;
     ep.bias = nullptr;
@@ -1671,7 +2317,9 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.resid_idx = eh.resid_idx;
     ep.ld_resid = eh.ld_resid;
     ep.tile_order = eh.tile_order;
-    const int64_t n_tiles = cdiv64(m, TC_BM * ctas) * n_tiles_n, units = ctx->sms / ctas;
+    const int64_t n_tiles = cdiv64(m, TC_BM * ctas) * n_tiles_n;
+    int64_t units = ctx->sms / ctas;
+    if (b_resident && units > n_tiles_n) units -= units % n_tiles_n;
     const unsigned grid = (unsigned)(n_tiles < units ? n_tiles : units) * ctas;
     TckLaunch L;
     L.mA = mA; L.mA2 = mA2; L.mB = mB; L.mBlo = mBlo; L.mC = mC;
@@ -1679,6 +2327,14 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     L.m = m; L.n = n; L.nkb1 = nkb1; L.nkb2 = nkb2; L.bn = bn; L.n_tiles_n = n_tiles_n; L.n_tiles = n_tiles;
     L.grid = grid;
     L.stage_bytes = stage_bytes;
+    L.b_resident = b_resident;
+    if (half) {
+        if (eh.gru) return pair ? launch_tch<EPI_GRU, 2>(ctx, L, ep) : launch_tch<EPI_GRU, 1>(ctx, L, ep);
+        if (ep.proj_h > 0) return pair ? launch_tch<EPI_PROJ, 2>(ctx, L, ep) : launch_tch<EPI_PROJ, 1>(ctx, L, ep);
+        if (ep.lstm_h > 0) return pair ? launch_tch<EPI_LSTM, 2>(ctx, L, ep) : launch_tch<EPI_LSTM, 1>(ctx, L, ep);
+        if (ep.push_dst) return pair ? launch_tch<EPI_PUSH, 2>(ctx, L, ep) : launch_tch<EPI_PUSH, 1>(ctx, L, ep);
+        return pair ? launch_tch<EPI_PLAIN, 2>(ctx, L, ep) : launch_tch<EPI_PLAIN, 1>(ctx, L, ep);
+    }
     if (eh.gru) return pair ? launch_tck<EPI_GRU, 2>(ctx, L, ep) : launch_tck<EPI_GRU, 1>(ctx, L, ep);
     if (ep.proj_h > 0) return pair ? launch_tck<EPI_PROJ, 2>(ctx, L, ep) : launch_tck<EPI_PROJ, 1>(ctx, L, ep);
     if (ep.lstm_h > 0) return pair ? launch_tck<EPI_LSTM, 2>(ctx, L, ep) : launch_tck<EPI_LSTM, 1>(ctx, L, ep);
@@ -1687,35 +2343,13 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     return pair ? launch_tck<EPI_PLAIN, 2>(ctx, L, ep) : launch_tck<EPI_PLAIN, 1>(ctx, L, ep);
 }
 
-// the recurrent weights of a predictor with h units, packed in `buf` (packed already, with `ready`)
-static size_t recurrent_layout(int32_t h, void *base, SatRecurrent *out)
-{
-    out->n_pad = tile_n_for(4 * h);
-    out->ld = (h + SEQ_BK - 1) / SEQ_BK * 2 * SEQ_BK;
-    const size_t planes = (size_t)out->n_pad * out->ld * sizeof(__half);
-    out->planes = base;
-    out->unscale = (float *)((char *)base + planes);
-    return planes + (size_t)out->n_pad / PACK_COLS * sizeof(float);
-}
-sat_status sat_pack_recurrent(sat_ctx *ctx, const float *Uh, int32_t h, DevBuf &buf, bool ready, SatRecurrent *out)
-{
-    const size_t bytes = recurrent_layout(h, nullptr, out);
-    if (ready && (!buf.p || buf.bytes < bytes)) return SAT_ESTATE;
-    SAT_TRY(sat_ensure(ctx, buf, bytes));
-    recurrent_layout(h, buf.p, out);
-    if (ready) return SAT_OK;
-    sat_pdl(ctx->stream, k_pack_recurrent, (unsigned)(out->n_pad / PACK_COLS), 1024, 0)(Uh, h, out->ld / 2, (__half *)out->planes, out->unscale);
-    SAT_LAUNCHED(ctx);
-    return SAT_OK;
-}
-
-sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const SatRecurrent &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
+sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
                         float *cell, int write_cell)
 {
     if (rows == 0 || n_steps == 0) return SAT_OK;
     if (n_steps > SAT_SEQ_MAX || h > 64 || (h & 3)) return sat_fail(ctx, SAT_EINVAL, "sat_lstm_seq: at most %d steps and 64 units", SAT_SEQ_MAX);
     ProfScope prof(ctx, SATK_GEMM_SIDE, 4.0 * (double)rows * h * (4.0 * n_steps + 1.0 + (first ? 0.0 : 2.0)), 8.0 * (double)rows * h * h * (n_steps - (first ? 1 : 0)));
-    const int32_t bn = tile_n_for(4 * h), nkb = (h + SEQ_BK - 1) / SEQ_BK;
+    const int32_t bn = tile_n_for(4 * h), nkb = (h + TCH_BK - 1) / TCH_BK;
     const size_t smem = (size_t)nkb * (2 * TC_BM + bn) * 128 + (size_t)SEQ_RING * 4 * SEQ_THREADS * 16 + sizeof(SeqShared) + 1024;
     static PerDeviceOnce attr_set;
     if (attr_set.need(ctx->device)) {
@@ -1723,13 +2357,7 @@ sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const SatRecurren
         attr_set.mark(ctx->device);
     }
     CUtensorMap mB;
-    PFN_encodeTiled enc = get_encode();
-    if (!enc) return sat_fail(ctx, SAT_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    const cuuint64_t gdim[2] = {(cuuint64_t)Uh.ld, (cuuint64_t)Uh.n_pad}, gstr[1] = {(cuuint64_t)Uh.ld * 2};
-    const cuuint32_t box[2] = {2 * SEQ_BK, (cuuint32_t)bn}, estr[2] = {1, 1};
-    if (enc(&mB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, Uh.planes, gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return sat_fail(ctx, SAT_EINVAL, "cuTensorMapEncodeTiled failed for the recurrent weights");
+    SAT_TRY(make_map_weights(ctx, &mB, Uh, bn));
     SeqSteps st;
     for (int32_t t = 0; t < SAT_SEQ_MAX; ++t) st.proj[t] = t < n_steps ? proj[t] : nullptr;
     const int64_t tiles = cdiv64(rows, TC_BM);

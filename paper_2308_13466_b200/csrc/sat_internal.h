@@ -65,6 +65,7 @@ struct DevBuf {
 
 struct LayerState {
     float *agg = nullptr;      // [N x ld_in]  saved aggregation (rows in partition-major order)
+    uint32_t *agg_max = nullptr;   // [sat_spmm_parts(d_in) x N] largest magnitude of its rows, where the transform takes half-precision pairs
     uint32_t *mask = nullptr;  // [N x mask_words] bit j of word w: Z[row][32w + j] > 0
     int32_t d_in = 0, d_out = 0, ld_in = 0, mask_words = 0;
     int act = 0;
@@ -74,6 +75,10 @@ struct LayerState {
 struct CacheLayer {
     float *buf = nullptr;  // [(tau+1) x n_slots x ld]
     int32_t width = 0, ld = 0;
+    // [(tau+1) x parts x n_slots] largest magnitude of the rows of every buffer, where sat_tc_half(width); where row_max_ok[buffer] is 0 it is looked for
+    // before its next use
+    uint32_t *row_max = nullptr;
+    std::vector<uint8_t> row_max_ok;
     float *S = nullptr;  // LSTM state table [n_slots x h]
     int32_t S_h = 0;
     bool S_valid = false;
@@ -216,7 +221,7 @@ struct sat_ctx {
     // ---- scratch ----
     DevBuf buf_codec_sizes, buf_codec_off, buf_codec_bytes;  // embedding codec scratch
     DevBuf buf_ticket, buf_partial, buf_gagg, buf_splitk, buf_lstm_c, buf_lstm_s, buf_lstm_w, buf_pred_a, buf_misc, buf_colsum, buf_dmask,
-        buf_wsplit, buf_wsplit2, buf_wsplit3, buf_bias, buf_pred_train, buf_ghist_halo, buf_ghist_rows, buf_ghist_out, buf_gat, buf_gat_items;
+        buf_wsplit, buf_wsplit2, buf_wsplit3, buf_bias, buf_pred_train, buf_ghist_halo, buf_ghist_rows, buf_ghist_out, buf_gat, buf_gat_items, buf_q_max;
 };
 
 sat_status sat_fail(sat_ctx *ctx, sat_status code, const char *fmt, ...);
@@ -327,7 +332,18 @@ struct PartView {
 };
 sat_status sat_part_view(sat_ctx *ctx, int32_t part, PartView *v);
 
+// Bits of the largest magnitude in every row of a matrix (in each of `parts` parts of the row, `stride` rows of them apart), as left by its writer
+struct RowMax {
+    const uint32_t *p = nullptr;
+    int64_t stride = 0;
+    int32_t parts = 1;
+};
+struct RowMaxOut {
+    uint32_t *p = nullptr;
+    int64_t stride = 0;
+};
 // SpMM family (sat_spmm.cu)
+inline int32_t sat_spmm_parts(int32_t d) { return (d + 255) / 256; }
 enum class SpmmHalo { by_position, by_gid, by_slot };
 //   out[row] = dinv[row] * sum_e dinv[col_e] * src(col_e), over all entries of the row (inner_only = 0)
 //   or over its inner prefix (inner_only = 1), or over its halo suffix (inner_only = 2; in_base is not read, rows without
@@ -337,7 +353,8 @@ enum class SpmmHalo { by_position, by_gid, by_slot };
 // omask (or null): bit mask [rows x omask_words] indexed like out_base; output components whose bit is 0 are written as 0
 // halo_kind: what the halo columns address: the concatenated halo matrix, a matrix over all n nodes in global id order, or one over
 // the cache slots (halo_base = its first row in the last two); in_global: inner and halo columns both address such a matrix (in_base = its first row; halo_base is not used)
-// add: rows added to the results, where given
+// add: rows added to the results, where given; row_max: the largest magnitude of every row of the results goes there (indexed like out_base,
+// in sat_spmm_parts(d) parts)
 struct SpmmAdd {
     const float *rows = nullptr;         // out[i] += rows[slot[i] * ld ..] where slot[i] >= 0
     const int32_t *slot = nullptr;       // [rows of out]
@@ -345,7 +362,8 @@ struct SpmmAdd {
 };
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask = nullptr,
-                    int32_t omask_words = 0, SpmmHalo halo_kind = SpmmHalo::by_position, bool in_global = false, const SpmmAdd &add = SpmmAdd());
+                    int32_t omask_words = 0, SpmmHalo halo_kind = SpmmHalo::by_position, bool in_global = false, const SpmmAdd &add = SpmmAdd(),
+                    const RowMaxOut &row_max = RowMaxOut());
 // the same kernels on weights of the caller's: out[row] = epilogue(sum_e w_e * src(col_e)) with ent[e] = {column, weight} indexed like
 // the entries of the mode (0: local rows; 1: their inner prefix; 3: halo rows, columns = partition-major rows)
 struct SpmmEpilogue {
@@ -353,6 +371,7 @@ struct SpmmEpilogue {
     int relu = 0;
     const float *s1 = nullptr, *v1 = nullptr, *s2 = nullptr, *v2 = nullptr;   // + s1[row] v1[col] + s2[row] v2[col]
     int32_t d = 0;
+    RowMaxOut row_max;
     SpmmAdd add;                         // (products with the propagation matrix only) rows added after the scaling
     float *push = nullptr;               // row i goes to row push_slot[i] of this matrix as well where that is >= 0
     const int32_t *push_slot = nullptr;  // [rows]
@@ -506,12 +525,25 @@ __device__ __forceinline__ float sigmoid_fast(float x) { return rcp_fast(1.f + e
 __device__ __forceinline__ float tanh_fast(float x) { return fmaf(-2.f, rcp_fast(1.f + ex2_fast(2.8853900817779268f * x)), 1.f); }
 #endif
 
-struct TcWeights {         // weight operand as two fp32 planes [n_pad x ld] holding the TF32 hi / lo terms, K-major
-    float *hi = nullptr, *lo = nullptr;
-    float *bias = nullptr;  // [n_pad], where one was packed with them
+// parts in which a contraction with n outputs leaves the largest magnitudes of its rows
+inline int32_t sat_tc_parts(int32_t n) { return 2 * ((n + 255) / 256); }
+// largest magnitudes of the rows of ring buffer idx of a cached layer (none unless sat_tc_half(width))
+sat_status sat_ring_rows(sat_ctx *ctx, int32_t layer, int32_t idx, RowMax *out);
+// out[r] = largest magnitude of row r, looked for (for matrices whose writer did not leave it)
+sat_status sat_row_max(sat_ctx *ctx, const float *A, int32_t lda, int32_t d, int64_t rows, uint32_t *out);
+// contractions of k terms that take half-precision pairs, where the caller has the largest magnitudes of the rows
+bool sat_tc_half(const sat_ctx *ctx, int32_t k);
+struct TcWeights {           // weight operand, K-major
+    bool half;               // which of the two forms it has
+    float *hi = nullptr, *lo = nullptr;   // two fp32 planes [n_pad x ld] holding the TF32 hi / lo terms
+    void *planes = nullptr;     // __half: pairs [n_pad][k-steps][16 hi | 16 lo], scaled per eight columns
+    float *unscale = nullptr;   // [n_pad / 8] inverse of the scale
+    float *bias = nullptr;   // [n_pad], where one was packed with them
     int32_t ld = 0, n_pad = 0;
+    explicit TcWeights(bool half_pairs = false) : half(half_pairs) {}
 };
 struct TcEpilogueHost {
+    RowMax rows;   // of the A operand (half-precision pairs)
     float *C = nullptr;
     int32_t ldc = 0;
     const float *bias = nullptr;
@@ -539,6 +571,7 @@ struct TcEpilogueHost {
     float *push_dst = nullptr;
     const int32_t *push_slot = nullptr;
     int32_t ld_push = 0;
+    RowMaxOut push_max;   // largest magnitude of every pushed row, by slot, in sat_tc_parts(n) parts
     // optional home of the padded bias copy (default: a scratch buffer of the context, repacked by every call); with
     // bias_ready the copy in *bias_home is current and is used as it is
     DevBuf *bias_home = nullptr;
@@ -556,19 +589,12 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
                           int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0, int gates = 4, const float *bias = nullptr);
 sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out);
-// Recurrent weights of a predictor as half-precision pairs for sat_lstm_seq
-struct SatRecurrent {
-    void *planes = nullptr;      // __half [n_pad][k-steps][16 hi | 16 lo]
-    float *unscale = nullptr;    // [n_pad / 32] inverse of the scale
-    int32_t ld = 0, n_pad = 0;   // halves of a column; gate columns, padded
-};
-sat_status sat_pack_recurrent(sat_ctx *ctx, const float *Uh, int32_t h, DevBuf &buf, bool ready, SatRecurrent *out);
 // Plane of an input projection x Wx + b of the LSTM, [row tile of 128][unit][row of the tile][i f g o]
 inline int64_t sat_proj_floats(int64_t rows, int32_t h) { return (rows + 127) / 128 * 512 * h; }
 // LSTM steps over `n_steps` projection planes, oldest first, on the state S [rows x h] and the cell state (sat_cell_offset layout; read
-// unless `first`, i.e. both start from zero; written with write_cell).  h a multiple of 4 up to 64.
+// unless `first`, i.e. both start from zero; written with write_cell).  Uh packed with gate_h; h a multiple of 4 up to 64.
 #define SAT_SEQ_MAX 32
-sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const SatRecurrent &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
+sat_status sat_lstm_seq(sat_ctx *ctx, int64_t rows, int32_t h, const TcWeights &Uh, const float *const *proj, int32_t n_steps, int first, float *S,
                         float *cell, int write_cell);
 // C[m x n] = [A | A2] B^T (+ epilogue)
 sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32_t lda, int32_t k1, const float *A2, int32_t lda2, int32_t k2,

@@ -58,6 +58,7 @@ extern "C" sat_status sat_cache_init(sat_ctx *ctx, int32_t n_cached_layers, cons
         if (ctx->cache[i].buf) cudaFree(ctx->cache[i].buf);
         if (ctx->cache[i].S) cudaFree(ctx->cache[i].S);
         if (ctx->cache[i].proj) cudaFree(ctx->cache[i].proj);
+        if (ctx->cache[i].row_max) cudaFree(ctx->cache[i].row_max);
         ctx->cache[i] = CacheLayer();
     }
     ctx->cache_ok = false;
@@ -65,6 +66,13 @@ extern "C" sat_status sat_cache_init(sat_ctx *ctx, int32_t n_cached_layers, cons
         CacheLayer &c = ctx->cache[i];
         c.width = width[i];
         c.ld = round_up4(width[i]);
+        c.row_max_ok.assign((size_t)tau + 1, 1);   // rows of zeros
+        if (sat_tc_half(ctx, width[i])) {
+            const size_t max_bytes = (size_t)(tau + 1) * sat_tc_parts(width[i]) * (size_t)ctx->n_slots * sizeof(uint32_t);
+            SAT_CUDA(ctx, cudaMalloc((void **)&c.row_max, max_bytes ? max_bytes : 16));
+            SAT_CUDA(ctx, cudaMemsetAsync(c.row_max, 0, max_bytes, ctx->stream));
+        }
+        if (mode == SAT_CACHE_COPY) c.row_max_ok[0] = 0;
         const size_t bytes = (size_t)(tau + 1) * (size_t)ctx->n_slots * c.ld * sizeof(float);
         SAT_CUDA(ctx, cudaMalloc((void **)&c.buf, bytes ? bytes : 16));
         SAT_CUDA(ctx, cudaMemsetAsync(c.buf, 0, bytes, ctx->stream));
@@ -87,7 +95,21 @@ static sat_status cache_layer(sat_ctx *ctx, int32_t layer, CacheLayer **c, const
     return SAT_OK;
 }
 
-// buffer index of the snapshot of a given age (0 = newest committed)
+// largest magnitudes of the rows of ring buffer idx
+static sat_status ring_rows(sat_ctx *ctx, CacheLayer *c, int32_t idx, RowMax *out)
+{
+    if (!c->row_max) return SAT_OK;
+    const int32_t parts = sat_tc_parts(c->width);
+    uint32_t *p = c->row_max + (size_t)idx * parts * ctx->n_slots;
+    if (!c->row_max_ok[idx] && ctx->n_slots > 0) {
+        SAT_TRY(sat_row_max(ctx, ring_buf(ctx, c, idx), c->ld, c->width, ctx->n_slots, p));
+        SAT_CUDA(ctx, cudaMemsetAsync(p + ctx->n_slots, 0, (size_t)(parts - 1) * ctx->n_slots * sizeof(uint32_t), ctx->stream));
+        c->row_max_ok[idx] = 1;
+    }
+    *out = RowMax{p, ctx->n_slots, parts};
+    return SAT_OK;
+}
+sat_status sat_ring_rows(sat_ctx *ctx, int32_t layer, int32_t idx, RowMax *out) { return ring_rows(ctx, &ctx->cache[layer - 1], idx, out); }
 
 extern "C" sat_status sat_cache_update(sat_ctx *ctx, int32_t part, int32_t layer, const float *h_out, int32_t ld)
 {
@@ -99,6 +121,7 @@ extern "C" sat_status sat_cache_update(sat_ctx *ctx, int32_t part, int32_t layer
     if (v.n_push == 0) return SAT_OK;
     if (!h_out || !ok_ld(ld, c->width) || !aligned16(h_out)) return sat_fail(ctx, SAT_EINVAL, "sat_cache_update: null / misaligned h_out or bad ld");
     if (!c->proj_tag.empty()) c->proj_tag[ctx->write_idx] = 0;  // the buffer changes: its cached input projection is stale
+    c->row_max_ok[ctx->write_idx] = 0;
     const float *src_base = h_out - (int64_t)v.row0 * ld;
     return sat_scatter(ctx, ctx->push_row + v.push0, ctx->push_slot + v.push0, v.n_push, c->width, src_base, ld,
                        ring_buf(ctx, c, ctx->write_idx), c->ld, DbgRange{v.row0, (int64_t)v.row0 + v.n_rows}, DbgRange{0, ctx->n_slots});
@@ -172,6 +195,7 @@ extern "C" sat_status sat_cache_requantise(sat_ctx *ctx, int32_t layer, int32_t 
     const int32_t idx = ring_index(ctx, age);
     SAT_TRY(sat_codec_roundtrip(ctx, ring_buf(ctx, c, idx), c->ld, ctx->n_slots, c->width, precision, bytes));
     if (!c->proj_tag.empty()) c->proj_tag[idx] = 0;  // the cached projection was made from the unquantised snapshot
+    c->row_max_ok[idx] = 0;
     c->S_valid = false;
     return SAT_OK;
 }
@@ -236,6 +260,7 @@ extern "C" sat_status sat_cache_import(sat_ctx *ctx, int32_t layer, const float 
     const size_t rows = (size_t)(ctx->tau + 1) * ctx->n_slots;
     c->S_valid = false;
     c->proj_tag.assign(c->proj_tag.size(), 0);
+    c->row_max_ok.assign(c->row_max_ok.size(), 0);
     if (rows == 0) return SAT_OK;
     SAT_CUDA(ctx, cudaMemcpy2DAsync(c->buf, (size_t)c->ld * 4, in_host, (size_t)c->width * 4, (size_t)c->width * 4, rows,
                                     cudaMemcpyHostToDevice, ctx->stream));
@@ -286,8 +311,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
         c->proj_h = h;
         c->proj_tag.assign(ctx->tau + 1, 0);
     }
-    TcWeights Wp, Wxu;   // Wx alone, [Wx ; Uh] (gate-interleaved)
-    SatRecurrent Up;     // Uh alone
+    TcWeights Wp(sat_tc_half(ctx, d)), Wxu(sat_tc_half(ctx, d)), Up(true);   // Wx alone, [Wx ; Uh], Uh alone (all gate-interleaved)
     bool have_wp = false, have_wxu = false, have_up = false;
     if (c->pk_h != h) {      // another predictor width: nothing packed fits
         c->tag_wx = c->tag_uh = c->tag_wg = c->tag_b = c->tag_bg = 0;
@@ -316,6 +340,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
         eh.bias_home = &c->pk_b;
         eh.bias_ready = c->tag_b == p->version;
         c->tag_b = p->version;
+        SAT_TRY(ring_rows(ctx, c, newest, &eh.rows));
         SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, ring_buf(ctx, c, newest), c->ld, d, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
         c->proj_tag[newest] = p->version;
     }
@@ -328,8 +353,14 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
                 planes[n] = c->proj + (int64_t)ring_index(ctx, k - 1 - t - n) * plane;
                 ++n;
             }
-            if (!have_up) SAT_TRY(sat_pack_recurrent(ctx, p->Uh, h, c->pk_uh, c->tag_uh == p->version, &Up));
-            c->tag_uh = p->version;
+            if (!have_up) {
+                if (c->tag_uh == p->version) {
+                    SAT_TRY(sat_tc_weights_layout(h, 4 * h, c->pk_uh, &Up));
+                } else {
+                    SAT_TRY(sat_tc_weights(ctx, p->Uh, 4 * h, h, nullptr, 0, 0, 4 * h, 1, c->pk_uh, &Up, h));
+                    c->tag_uh = p->version;
+                }
+            }
             have_up = true;
             SAT_TRY(sat_lstm_seq(ctx, rows, h, Up, planes, n, t == 0, c->S, cell, t + n < k));
             t += n;
@@ -342,6 +373,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
         eh.lstm_h = h;
         eh.lstm_c = cell;
         eh.bias = p->b;
+        SAT_TRY(ring_rows(ctx, c, ring_index(ctx, k - 1 - t), &eh.rows));
         if (t == 0) {
             SAT_TRY(pack_wx());
             eh.lstm_first = 1;
@@ -406,7 +438,7 @@ static sat_status run_gru(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p)
         return SAT_OK;
     }
     if (sat_use_tc(4 * h, d) && 4 * h <= 256) {
-        TcWeights W1, W2;   // first step: x alone
+        TcWeights W1(sat_tc_half(ctx, d)), W2(sat_tc_half(ctx, d));   // first step: x alone
         SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, h, 3, p->b));
         if (k > 1) SAT_TRY(sat_tc_weights(ctx, p->Wx, 3 * h, d, p->Uh, 3 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, h, 3, p->b));
         for (int32_t t = 0; t < k; ++t) {
@@ -417,6 +449,7 @@ static sat_status run_gru(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p)
             eh.lstm_h = h;
             eh.gru = 1;
             eh.lstm_first = t == 0;
+            SAT_TRY(ring_rows(ctx, c, ring_index(ctx, k - 1 - t), &eh.rows));
             SAT_TRY(sat_gemm_tc(ctx, rows, 4 * h, ring_buf(ctx, c, ring_index(ctx, k - 1 - t)), c->ld, d, t == 0 ? nullptr : c->S, h, t == 0 ? 0 : h,
                                 t == 0 ? W1 : W2, eh, SATK_GEMM_NN));
         }
@@ -491,7 +524,7 @@ static sat_status run_lstm(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p
     // then a tile reads only its own rows of s, and does so before its epilogue overwrites them
     const bool fused = tc && 4 * h <= 256;
     if (fused && p->version != 0 && sat_use_tc(4 * h, h)) return run_lstm_cached(ctx, c, p, k, cell);
-    TcWeights W1, W2;   // packed weights for the first step (x only) and the later steps ([x | s])
+    TcWeights W1(sat_tc_half(ctx, d)), W2(sat_tc_half(ctx, d));   // packed weights for the first step (x only) and the later steps ([x | s])
     if (tc) {
         SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, fused ? h : 0, 4, p->b));
         if (k > 1) SAT_TRY(sat_tc_weights(ctx, p->Wx, 4 * h, d, p->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, fused ? h : 0, 4, p->b));
@@ -501,6 +534,7 @@ static sat_status run_lstm(sat_ctx *ctx, CacheLayer *c, const sat_pred_params *p
         if (tc) {
             TcEpilogueHost eh;
             eh.bias = p->b;
+            SAT_TRY(ring_rows(ctx, c, ring_index(ctx, k - 1 - t), &eh.rows));
             if (fused) {
                 eh.C = c->S;
                 eh.ldc = h;
@@ -708,10 +742,16 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
         return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: null / misaligned h_in / h_out or bad leading dimension");
     if (!in_global && !halo_cached && v.n_halo > 0 && (!h_halo || !ok_ld(ld_halo, d_in) || !aligned16(h_halo)))
         return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: null / misaligned h_halo or bad ld_halo");
+    // The first layer keeps TF32 terms.  Which side of a ReLU a pre-activation near zero takes depends on its rounding, and there, on raw features of a dense
+    // graph, one decision moves an element of the weight gradient by several percent of the matrix's root mean square (58241 nodes, 16 M
+    // entries, 602 -> 256: up to 8 %, against 0.6 % for decisions of later layers), for 0.5 % of an epoch.  A push is bound by its
+    // epilogue up to 256 terms (113 us with TF32 terms, 120 with pairs; 179250 x 512, K = 512: 378 and 280).
+    const bool half_rows = layer > 1 && sat_tc_half(ctx, d_in), half = half_rows && (!push || d_in >= 384);
     LayerState &L = ctx->layers[layer];
     const int32_t ld_agg = round_up4(d_in), words = (d_out + 31) / 32;
     if (!L.agg || L.d_in != d_in || L.d_out != d_out) {
         SAT_TRY(dev_realloc(ctx, &L.agg, (int64_t)ctx->n * ld_agg));
+        SAT_TRY(dev_realloc(ctx, &L.agg_max, half_rows ? (int64_t)ctx->n * sat_spmm_parts(d_in) : 0));
         SAT_TRY(dev_realloc(ctx, &L.mask, (int64_t)ctx->n * words));
         L.d_in = d_in;
         L.d_out = d_out;
@@ -732,11 +772,12 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
         ld_halo = hc->ld;
     }
     // (no snapshot yet: the halo terms are zero, the inner entries of the rows are all there is)
-    SAT_TRY(sat_spmm(ctx, v, halo_cached && !halo_base ? 1 : 0, d_in, in_base, ld_in, halo_base, ld_halo, L.agg, ld_agg, nullptr, 0, halo_kind, in_global));
+    SAT_TRY(sat_spmm(ctx, v, halo_cached && !halo_base ? 1 : 0, d_in, in_base, ld_in, halo_base, ld_halo, L.agg, ld_agg, nullptr, 0, halo_kind, in_global,
+                     SpmmAdd(), half ? RowMaxOut{L.agg_max, ctx->n} : RowMaxOut()));
     uint32_t *mask_out = act == SAT_ACT_RELU ? L.mask + (int64_t)v.row0 * words : nullptr;
     const float *agg = L.agg + (int64_t)v.row0 * ld_agg;
     if (sat_use_tc(d_out, d_in)) {
-        TcWeights Wp;
+        TcWeights Wp(half);
         SAT_TRY(sat_tc_weights(ctx, W, d_out, d_in, nullptr, 0, 0, d_out, 1, ctx->buf_wsplit, &Wp, 0, 4, bias));
         TcEpilogueHost eh;
         eh.C = h_out;
@@ -745,12 +786,16 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
         eh.relu = act == SAT_ACT_RELU;
         eh.mask_out = mask_out;
         eh.mask_words = words;
+        if (Wp.half) eh.rows = RowMax{L.agg_max + v.row0, ctx->n, sat_spmm_parts(d_in)};
         if (push && ctx->n_slots > 0) {   // the boundary rows go to the ring's write buffer from the epilogue
             SAT_TRY(sat_row_slots(ctx, &eh.push_slot));
             eh.push_slot += v.row0;
             eh.push_dst = ring_buf(ctx, pc, ctx->write_idx);
             eh.ld_push = pc->ld;
             if (!pc->proj_tag.empty()) pc->proj_tag[ctx->write_idx] = 0;
+            // the rows' maxima stay in step with the rows: all of them from now on, or those of this partition where all of them were
+            if (pc->row_max) eh.push_max = RowMaxOut{pc->row_max + (size_t)ctx->write_idx * sat_tc_parts(d_out) * ctx->n_slots, ctx->n_slots};
+            if (part == SAT_ALL_PARTS) pc->row_max_ok[ctx->write_idx] = 1;
         }
         SAT_TRY(sat_gemm_tc(ctx, v.n_rows, d_out, agg, ld_agg, d_in, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
     } else {
@@ -849,13 +894,15 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
         }
     }
     if (!want_dx) return SAT_OK;
+    const bool half_x = tc_x && sat_tc_half(ctx, d_out);
     const bool stale_term = hist && GH.has_read && g_in && v.n_push > 0;
     // G_in = P_in^T (D W^T) = (P_in^T D) W^T.  The second order gathers rows of d_out columns instead of d_in: taken where that is less
     // (256 -> 40, 169343 nodes, 2.6 M entries: product 152 -> 53 us, epoch 2840 -> 2749; 128 -> 19, 240000 nodes: epoch 1669 -> 1524;
     // 256 -> 47, 612257 nodes, 31 M entries: product 608 -> 165 us, epoch 16050 -> 15748).  The stale rows then join P_in^T D in the product's
     // epilogue, which makes their own contraction and the add into G_in unnecessary, so with them the order pays at equal
-    // widths too (84671 nodes, 256 -> 256 -> 40, epoch with the predictor trained: 5342 -> 5087).
-    if (g_in && !g_halo && (!mask || tc_x) && (stale_term ? d_out <= d_in : d_out < d_in)) {
+    // widths too (84671 nodes, 256 -> 256 -> 40, epoch with the predictor trained: 5342 -> 5087).  So it does where the contraction takes
+    // half-precision pairs: the product leaves the largest magnitudes of its rows.
+    if (g_in && !g_halo && (!mask || tc_x) && (stale_term || half_x ? d_out <= d_in : d_out < d_in)) {
         const int32_t ld_q = round_up4(d_out);
         SAT_TRY(sat_ensure(ctx, ctx->buf_gagg, (size_t)v.n_rows * ld_q * sizeof(float)));
         float *q = (float *)ctx->buf_gagg.p;
@@ -865,17 +912,23 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
             add.rows = GH.buf + (size_t)GH.read_idx * ctx->n_slots * GH.ld;
             add.ld = GH.ld;
         }
+        RowMaxOut q_max;
+        if (half_x) {
+            SAT_TRY(sat_ensure(ctx, ctx->buf_q_max, (size_t)v.n_rows * sat_spmm_parts(d_out) * sizeof(uint32_t)));
+            q_max = RowMaxOut{(uint32_t *)ctx->buf_q_max.p - v.row0, v.n_rows};
+        }
         SAT_TRY(sat_spmm(ctx, v, 1, d_out, D - (int64_t)v.row0 * ld_d, ld_d, nullptr, 0, q - (int64_t)v.row0 * ld_q, ld_q, nullptr, 0, SpmmHalo::by_position,
-                         false, add));
+                         false, add, q_max));
         const uint32_t *keep = mask_in ? mask_in + (int64_t)v.row0 * mask_in_words : nullptr;
         if (!tc_x) return sat_gemm_nt(ctx, v.n_rows, d_in, d_out, q, ld_q, nullptr, 0, W, d_out, g_in, ld_gin, keep, mask_in_words);
-        TcWeights Wp;
+        TcWeights Wp(half_x);
         SAT_TRY(sat_tc_weights(ctx, W, d_out, d_out, nullptr, 0, 0, d_in, 0, ctx->buf_wsplit, &Wp));
         TcEpilogueHost eh;
         eh.C = g_in;
         eh.ldc = ld_gin;
         eh.mask_in = keep;
         eh.mask_in_words = mask_in_words;
+        if (half_x) eh.rows = RowMax{(const uint32_t *)ctx->buf_q_max.p, v.n_rows, sat_spmm_parts(d_out)};
         return sat_gemm_tc(ctx, v.n_rows, d_in, q, ld_q, d_out, nullptr, 0, 0, Wp, eh, SATK_GEMM_NT);
     }
     // G_AGG = D W^T

@@ -5,6 +5,8 @@
 // GEMM kernels as the layer steps; this file holds the element-wise and sparse kernels around them.
 #include "sat_internal.h"
 
+#include <algorithm>
+
 
 // -------------------------------------------------------------------------------------
 // LSTM cell kernels.  A thread owns four consecutive hidden units of a row (one 16-byte access per gate block and state
@@ -58,10 +60,11 @@ k_pt_cell_fwd(float *__restrict__ z, int64_t rows, int32_t h, const float *__res
 // to the gate pre-activations; dc carries the gradient of the cell state from the later steps (null at the last step) and
 // leaves as the gradient with respect to the previous cell state.  The column sums of the written gradients (the bias
 // gradient of the step) are accumulated on the way: per thread over its rows, then over the row groups of the block in
-// fixed order into colsum_part [gridDim.x x 4h] (null: the weight gradient takes them along).
+// fixed order into colsum_part [gridDim.x x 4h] (null: the weight gradient takes them along).  row_max (or null): the largest magnitude of every
+// written row, for the contraction that reads it next; needs h / 4 a power of two up to 32.
 __global__ void __launch_bounds__(256)
 k_pt_cell_bwd(float *__restrict__ gz, int64_t rows, int32_t h, const float *__restrict__ c_prev, const float *__restrict__ c_cur,
-              const float *__restrict__ dh, const float *dc_in, float *dc_out, float *__restrict__ colsum_part)
+              const float *__restrict__ dh, const float *dc_in, float *dc_out, float *__restrict__ colsum_part, uint32_t *__restrict__ row_max)
 {
     sat_grid_wait();
     extern __shared__ float red[];   // [rpp][4h]
@@ -92,6 +95,14 @@ k_pt_cell_bwd(float *__restrict__ gz, int64_t rows, int32_t h, const float *__re
             st4s(a + 2 * h, dg);
             st4s(a + 3 * h, dd);
             st4s(dc_out + o, dcp);
+            if (row_max) {   // h4 is a power of two: the lanes of a row are an aligned group
+                float m = 0.f;
+                PT_MAP4(tc, fmaxf(fmaxf(fabsf(el(di, e)), fabsf(el(df, e))), fmaxf(fabsf(el(dg, e)), fabsf(el(dd, e)))));
+                m = fmaxf(fmaxf(tc.x, tc.y), fmaxf(tc.z, tc.w));
+                const unsigned mask = h4 >= 32 ? 0xffffffffu : ((1u << h4) - 1u) << (threadIdx.x & 31 & ~(h4 - 1));
+                const uint32_t b = __reduce_max_sync(mask, __float_as_uint(m));
+                if (q == 0) row_max[r] = b;
+            }
             PT_MAP4(si, el(si, e) + el(di, e));
             PT_MAP4(sf, el(sf, e) + el(df, e));
             PT_MAP4(sg, el(sg, e) + el(dg, e));
@@ -126,7 +137,7 @@ k_pt_cell_bwd(float *__restrict__ gz, int64_t rows, int32_t h, const float *__re
 __global__ void __launch_bounds__(256)
 k_pt_error(float *__restrict__ pred, int64_t ld, int64_t n_halo, int32_t d, const float *__restrict__ target, int64_t ld_t,
            const int32_t *__restrict__ halo_slot, const float *__restrict__ row_weight, const int64_t *__restrict__ halo_off, int32_t M,
-           double *__restrict__ block_partial, float *__restrict__ colsum_part)
+           double *__restrict__ block_partial, float *__restrict__ colsum_part, uint32_t *__restrict__ row_max)
 {
     sat_grid_wait();
     extern __shared__ float4 cs4[];   // [8 warps][d rounded up to 4]
@@ -158,7 +169,7 @@ k_pt_error(float *__restrict__ pred, int64_t ld, int64_t n_halo, int32_t d, cons
         float4 *p4 = reinterpret_cast<float4 *>(pred + u * ld);
         const float4 *t4 = reinterpret_cast<const float4 *>(target + (int64_t)halo_slot[u] * ld_t);
         float4 *m4 = reinterpret_cast<float4 *>(mine);
-        float acc = 0.f;
+        float acc = 0.f, largest = 0.f;
 #pragma unroll 2
         for (int c4 = lane; c4 < d4; c4 += 32) {
             const float4 pv = p4[c4], tv = __ldg(t4 + c4);
@@ -171,6 +182,7 @@ k_pt_error(float *__restrict__ pred, int64_t ld, int64_t n_halo, int32_t d, cons
             acc = fmaf(df.x, df.x, fmaf(df.y, df.y, fmaf(df.z, df.z, fmaf(df.w, df.w, acc))));
             const float4 ev = make_float4(w * df.x, w * df.y, w * df.z, w * df.w);
             p4[c4] = ev;
+            largest = fmaxf(fmaxf(largest, fmaxf(fabsf(ev.x), fabsf(ev.y))), fmaxf(fabsf(ev.z), fabsf(ev.w)));
             float4 mv = m4[c4];
             mv.x += ev.x;
             mv.y += ev.y;
@@ -179,6 +191,10 @@ k_pt_error(float *__restrict__ pred, int64_t ld, int64_t n_halo, int32_t d, cons
             m4[c4] = mv;
         }
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (row_max) {
+            const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(largest));
+            if (lane == 0) row_max[u] = m;
+        }
         sum += 0.5 * (double)w * (double)acc;
     }
     if (lane == 0) red[warp] = sum;
@@ -242,14 +258,15 @@ static sat_status pt_tn(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, const 
 }
 
 // C[m x n] = A[m x k] W^T, W stored [n x k] row-major
-static sat_status pt_nt(sat_ctx *ctx, int64_t m, int32_t n, int32_t k, const float *A, int32_t lda, const float *W, float *C, int32_t ldc)
+static sat_status pt_nt(sat_ctx *ctx, int64_t m, int32_t n, int32_t k, const float *A, int32_t lda, const RowMax &rows, const float *W, float *C, int32_t ldc)
 {
     if (sat_use_tc(n, k)) {
-        TcWeights Wp;
+        TcWeights Wp(rows.p && sat_tc_half(ctx, k));
         SAT_TRY(sat_tc_weights(ctx, W, k, k, nullptr, 0, 0, n, 0, ctx->buf_wsplit, &Wp));
         TcEpilogueHost eh;
         eh.C = C;
         eh.ldc = ldc;
+        eh.rows = rows;
         return sat_gemm_tc(ctx, m, n, A, lda, k, nullptr, 0, 0, Wp, eh, SATK_GEMM_NT);
     }
     return sat_gemm_nt(ctx, m, n, k, A, lda, nullptr, 0, W, k, C, ldc);
@@ -275,7 +292,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     const int32_t h = params->h, d = c->width, M = ctx->M;
     const int64_t R = ctx->n_slots, nb = v.n_halo;
     const int32_t k = ctx->n_valid < ctx->tau ? ctx->n_valid : ctx->tau;
-    const int32_t ld_d = round_up4(d);
+    const int32_t ld_d = round_up4(d), h4 = h >> 2;
     SAT_CUDA(ctx, cudaMemsetAsync(g_Wx, 0, (size_t)d * 4 * h * sizeof(float), ctx->stream));
     SAT_CUDA(ctx, cudaMemsetAsync(g_Uh, 0, (size_t)h * 4 * h * sizeof(float), ctx->stream));
     SAT_CUDA(ctx, cudaMemsetAsync(g_b, 0, (size_t)4 * h * sizeof(float), ctx->stream));
@@ -293,8 +310,8 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     const int64_t n_blocks = n_tiles < 8 * ctx->sms ? n_tiles : 8 * ctx->sms;   // error kernel: the resident blocks of all SMs, each walking its tiles
     const size_t f_gates = pt_round((size_t)(k > 0 ? k : 1) * R * 4 * h), f_state = pt_round((size_t)(k > 0 ? k : 1) * R * h);
     const size_t f_a = pt_round((size_t)nb * h), f_e = pt_round((size_t)nb * ld_d), f_rh = pt_round((size_t)R * h);
-    const size_t f_off = pt_round(2 * (size_t)(M + 1)), f_part = pt_round(2 * (size_t)(n_blocks + 1)), f_nh = pt_round((size_t)ctx->n * h);
-    SAT_TRY(sat_ensure(ctx, ctx->buf_pred_train, (f_gates + 2 * f_state + 2 * f_a + f_e + 2 * f_rh + f_off + f_part + f_nh) * sizeof(float)));
+    const size_t f_max = pt_round((size_t)std::max(nb, R)), f_off = pt_round(2 * (size_t)(M + 1)), f_part = pt_round(2 * (size_t)(n_blocks + 1)), f_nh = pt_round((size_t)ctx->n * h);
+    SAT_TRY(sat_ensure(ctx, ctx->buf_pred_train, (f_gates + 2 * f_state + 2 * f_a + f_e + 2 * f_rh + f_off + f_part + f_nh + f_max) * sizeof(float)));
     float *gates = (float *)ctx->buf_pred_train.p;
     float *hs = gates + f_gates, *cs = hs + f_state;
     float *a = cs + f_state, *g_a = a + f_a, *E = g_a + f_a;
@@ -302,6 +319,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     int64_t *halo_off = (int64_t *)(dc + f_rh);
     double *partial = (double *)((float *)halo_off + f_off);
     float *g_rows = (float *)partial + f_part;   // [n x h] neighbour terms of the transposed convolution by inner row
+    uint32_t *row_max = (uint32_t *)(g_rows + f_nh);   // largest magnitudes of the rows of a contraction's operand: E, then the steps' gradients
     SAT_CUDA(ctx, cudaMemcpyAsync(halo_off, ctx->h_halo_off.data(), (size_t)(M + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, ctx->stream));
     const int64_t plane_g = R * 4 * (int64_t)h, plane_s = R * (int64_t)h;
     const unsigned cell_grid = (unsigned)cdiv64(R, PT_TILE_ROWS);
@@ -309,7 +327,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     const size_t cell_smem = (size_t)(256 / (h / 4)) * 4 * h * sizeof(float);
     // ---- LSTM forward over the snapshots, oldest first, gate values kept ----
     const bool tc_z = sat_use_tc(4 * h, d);
-    TcWeights W1, W2;
+    TcWeights W1(sat_tc_half(ctx, d)), W2(sat_tc_half(ctx, d));
     if (tc_z && k > 0) SAT_TRY(sat_tc_weights(ctx, params->Wx, 4 * h, d, nullptr, 0, 0, 4 * h, 1, ctx->buf_wsplit, &W1, 0, 4, params->b));
     if (tc_z && k > 1) SAT_TRY(sat_tc_weights(ctx, params->Wx, 4 * h, d, params->Uh, 4 * h, h, 4 * h, 1, ctx->buf_wsplit2, &W2, 0, 4, params->b));
     for (int32_t t = 0; t < k; ++t) {
@@ -321,6 +339,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
             eh.C = z;
             eh.ldc = 4 * h;
             eh.bias = params->b;
+            SAT_TRY(sat_ring_rows(ctx, layer, ring_index(ctx, k - 1 - t), &eh.rows));
             SAT_TRY(sat_gemm_tc(ctx, R, 4 * h, x, c->ld, d, h_prev, h, t ? h : 0, t ? W2 : W1, eh, SATK_GEMM_NN));
         } else {
             SAT_TRY(sat_gemm_nn_dual(ctx, R, 4 * h, d, x, c->ld, params->Wx, 4 * h, t ? h : 0, h_prev, h, params->Uh, 4 * h, params->b, z, 4 * h));
@@ -362,7 +381,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
         SAT_TRY(sat_ensure(ctx, ctx->buf_colsum, (size_t)n_blocks * d * sizeof(float)));
         sat_pdl(ctx->stream, k_pt_error, (unsigned)n_blocks, 256, (size_t)8 * ld_d * sizeof(float))(E, ld_d, nb, d, ring_buf(ctx, c, ctx->write_idx), c->ld,
                                                                                            ctx->halo_slot, row_weight, halo_off, M, partial,
-                                                                                           (float *)ctx->buf_colsum.p);
+                                                                                           (float *)ctx->buf_colsum.p, sat_tc_half(ctx, d) ? row_max : nullptr);
         SAT_LAUNCHED(ctx);
         sat_pdl(ctx->stream, k_pt_sum, 1, 256, 0)(partial, n_blocks, partial + n_blocks);
         SAT_LAUNCHED(ctx);
@@ -371,7 +390,8 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
     // ---- output layer: G_Wg = a^T E, G_bg = 1^T E, G_a = E Wg^T ----
     SAT_TRY(pt_tn(ctx, nb, h, d, a, h, E, ld_d, g_Wg, nullptr, 0));
     if (k > 0) {
-        SAT_TRY(pt_nt(ctx, nb, h, d, E, ld_d, params->Wg, g_a, h));
+        SAT_TRY(pt_nt(ctx, nb, h, d, E, ld_d, RowMax{sat_tc_half(ctx, d) ? row_max : nullptr, nb, 1}, params->Wg, g_a, h));
+        uint32_t *const dz_max = sat_tc_half(ctx, 4 * h) && (h4 & (h4 - 1)) == 0 && h4 <= 32 ? row_max : nullptr;
         // ---- transposed graph convolution: gradient of the final hidden state ----
         SAT_TRY(sat_spmm(ctx, v, 2, h, nullptr, 0, g_a, h, g_rows, h));
         SAT_TRY(sat_scatter(ctx, ctx->push_row, ctx->push_slot, R, h, g_rows, h, dh, h));
@@ -389,7 +409,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
                 ProfScope prof(ctx, SATK_PRED_TRAIN, 4.0 * (double)plane_s * 13.0, 0.0);
                 sat_pdl(ctx->stream, k_pt_cell_bwd, bwd_grid, 256, cell_smem)(z, R, h, t ? cs + (t - 1) * plane_s : nullptr, cs + t * plane_s, dh,
                                                                           t == k - 1 ? nullptr : dc, dc,
-                                                                          merged ? nullptr : (float *)ctx->buf_colsum.p);
+                                                                          merged ? nullptr : (float *)ctx->buf_colsum.p, dz_max);
                 SAT_LAUNCHED(ctx);
             }
             const int acc = t != k - 1;
@@ -397,7 +417,7 @@ extern "C" sat_status sat_pred_grad(sat_ctx *ctx, int32_t layer, const sat_pred_
             if (!merged) SAT_TRY(pt_tn(ctx, R, d, 4 * h, x, c->ld, z, 4 * h, g_Wx, nullptr, acc));
             if (t > 0) {
                 if (!merged) SAT_TRY(pt_tn(ctx, R, h, 4 * h, hs + (t - 1) * plane_s, h, z, 4 * h, g_Uh, nullptr, acc));
-                SAT_TRY(pt_nt(ctx, R, h, 4 * h, z, 4 * h, params->Uh, dh, h));
+                SAT_TRY(pt_nt(ctx, R, h, 4 * h, z, 4 * h, RowMax{dz_max, R, 1}, params->Uh, dh, h));
             }
         }
         for (int32_t t0 = 0; merged && t0 < k; t0 += SAT_TN_SEGMENTS) {

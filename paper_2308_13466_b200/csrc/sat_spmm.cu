@@ -492,6 +492,16 @@ __device__ __forceinline__ void spmm_add(const SpmmAdd &add, int64_t row, int c,
     r.w += x.w;
 }
 
+// largest magnitude of the columns 4 c .. 4 c + 3 that a row of d columns has
+__device__ __forceinline__ float spmm_largest(float m, const float4 &r, int c, int32_t d)
+{
+    if (4 * c + 3 < d) return fmaxf(fmaxf(m, fmaxf(fabsf(r.x), fabsf(r.y))), fmaxf(fabsf(r.z), fabsf(r.w)));
+    if (4 * c < d) m = fmaxf(m, fabsf(r.x));
+    if (4 * c + 1 < d) m = fmaxf(m, fabsf(r.y));
+    if (4 * c + 2 < d) m = fmaxf(m, fabsf(r.z));
+    return m;
+}
+
 // K entries: their columns and weights, their rows (all in flight together), the sums
 template <int G, int NV, int K, typename F>
 __device__ __forceinline__ void spmm_step(const int2 *__restrict__ ents, const F &row_of, int col, int32_t d4, float4 (&acc)[NV])
@@ -512,7 +522,7 @@ __device__ __forceinline__ void spmm_step(const int2 *__restrict__ ents, const F
         for (int v = 0; v < NV; ++v) fma4(acc[v], __int_as_float(q[u].y), x[u][v]);
 }
 
-template <int G, int NV, int U, int MINB, bool EPI>
+template <int G, int NV, int U, int MINB, bool EPI, bool MAX>
 __global__ void __launch_bounds__(256, MINB)
 k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const int2 *__restrict__ ent, const float *__restrict__ scale, int32_t n,
        int32_t d4, const float *__restrict__ in_base, int64_t ld_in, const float *__restrict__ halo_base, int64_t ld_halo, float *__restrict__ out_base,
@@ -560,9 +570,13 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
 #pragma unroll
         for (int v = 0; v < NV; ++v)
             if (col + v * G < d4) pr[v * G] = acc[v];
-        if (last_max == 0) return;
-        const int32_t first = __ldg(slot0 + it.x), cnt = __ldg(tot + it.x);
-        if (cnt > last_max) return;   // k_spmm_fixup
+        if (!MAX && last_max == 0) return;
+        const bool last = !MAX || last_max > 0;
+        const int32_t first = last ? __ldg(slot0 + it.x) : 0, cnt = last ? __ldg(tot + it.x) : 0;
+        if (cnt > last_max || !last) {   // k_spmm_fixup, which raises the row's maximum from zero
+            if (MAX && lane == 0) ep.row_max.p[blockIdx.y * ep.row_max.stride + it.x] = 0u;
+            return;
+        }
         const unsigned mask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
         __threadfence();
         __syncwarp(mask);
@@ -599,6 +613,7 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
     const int64_t row = SAT_IDX((int64_t)it.x, dbg.out_lo, dbg.out_hi, dbg.status);
     const float s = EPI ? 1.f : __ldg(scale + row);
     float4 *o = reinterpret_cast<float4 *>(out_base + row * ld_out) + col;
+    float largest = 0.f;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         if (col + v * G < d4) {
@@ -609,7 +624,14 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
                 if (omask) mask4(r, omask, row * omask_words, col + v * G);
             }
             o[v * G] = r;
+            if (MAX) largest = spmm_largest(largest, r, col + v * G, ep.d);
         }
+    }
+    if (MAX) {
+        unsigned lane_id;
+        asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane_id));   // (not kept through the loops)
+        const uint32_t m = __reduce_max_sync(G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (lane_id & ~(unsigned)(G - 1)), __float_as_uint(largest));
+        if ((lane_id & (G - 1)) == 0) ep.row_max.p[blockIdx.y * ep.row_max.stride + row] = m;
     }
 }
 
@@ -635,6 +657,7 @@ __device__ __forceinline__ float4 fixup_range(const float4 *__restrict__ p, int3
     return a;
 }
 
+template <bool MAX>
 __global__ void __launch_bounds__(256)
 k_spmm_fixup(const int32_t *__restrict__ hrows, int32_t n_hrows, const int32_t *__restrict__ mrows, int32_t n_mrows, const int32_t *__restrict__ slot0,
              const int32_t *__restrict__ tot, int64_t slot_base, const float *__restrict__ scale, int32_t d4, const float *__restrict__ partial,
@@ -681,6 +704,11 @@ k_spmm_fixup(const int32_t *__restrict__ hrows, int32_t n_hrows, const int32_t *
         if (omask) mask4(r, omask, row * omask_words, c);
     }
     *reinterpret_cast<float4 *>(out_base + row * ld_out + 4 * c) = r;
+    if (MAX) {   // the lanes of a warp that hold columns of the same row raise it together
+        const unsigned same = __match_any_sync(__activemask(), (int32_t)row);
+        const uint32_t m = __reduce_max_sync(same, __float_as_uint(spmm_largest(0.f, r, c, ep.d)));
+        if ((threadIdx.x & 31) == __ffs((int)same) - 1) atomicMax(ep.row_max.p + row, m);
+    }
 }
 
 struct SpmmArgs {
@@ -697,16 +725,16 @@ struct SpmmArgs {
     DbgRange src, halo, out;
 };
 
-template <int G, int NV, int U, int MINB>
+template <int G, int NV, int U, int MINB, bool MAX = false>
 static void launch_spmm(sat_ctx *ctx, const SpmmList &l, const int4 *items, int32_t n_items, int64_t slot_base, int32_t d4, const SpmmArgs &a, float *partial)
 {
     dim3 grid((unsigned)cdiv64((int64_t)n_items * G, 256), (unsigned)cdiv64(d4, G * NV));
     const DbgLimits dbg = dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1);
     if (a.scale)
-        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, false>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
+        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, false, MAX>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
                                                                      a.out_base, a.ld_out, partial, l.slot0, l.tot, (int32_t *)ctx->buf_ticket.p, l.last_max, a.omask, a.omask_words, a.ep, dbg);
     else
-        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, true>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
+        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, true, false>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
                                                                     a.out_base, a.ld_out, partial, l.slot0, l.tot, (int32_t *)ctx->buf_ticket.p, l.last_max, a.omask, a.omask_words, a.ep, dbg);
 }
 
@@ -740,7 +768,8 @@ static sat_status run_list(sat_ctx *ctx, const PartView &v, const SpmmList &l, i
     // run: eight entries in flight per step then, for more registers (epoch of 2,048 nodes 90.6 -> 84.4 us; 6,000 nodes and upward the
     // same, one drawn graph 515 -> 522)
     const bool small = n_items * 32 <= ctx->sms * 768;
-    if (d4 <= 4) small ? launch_spmm<4, 1, 8, 3>(ARGS) : launch_spmm<4, 1, 4, 6>(ARGS);
+    if (a.ep.row_max.p) small ? launch_spmm<32, 2, 8, 3, true>(ARGS) : launch_spmm<32, 2, 4, 5, true>(ARGS);   // (sat_tc_half: wide rows)
+    else if (d4 <= 4) small ? launch_spmm<4, 1, 8, 3>(ARGS) : launch_spmm<4, 1, 4, 6>(ARGS);
     else if (d4 <= 8) small ? launch_spmm<8, 1, 8, 3>(ARGS) : launch_spmm<8, 1, 4, 6>(ARGS);
     else if (d4 <= 16) small ? launch_spmm<16, 1, 8, 3>(ARGS) : launch_spmm<16, 1, 4, 6>(ARGS);
     else if (d4 <= 32) small ? launch_spmm<16, 2, 8, 3>(ARGS) : launch_spmm<16, 2, 4, 5>(ARGS);
@@ -748,7 +777,7 @@ static sat_status run_list(sat_ctx *ctx, const PartView &v, const SpmmList &l, i
 #undef ARGS
     SAT_LAUNCHED(ctx);
     if (n_hrows + n_mrows > 0) {
-        sat_pdl(ctx->stream, k_spmm_fixup, (unsigned)(n_hrows * cdiv64(d4, 32) + cdiv64(n_mrows * d4, 256)), 256, 0)(
+        sat_pdl(ctx->stream, a.ep.row_max.p ? k_spmm_fixup<true> : k_spmm_fixup<false>, (unsigned)(n_hrows * cdiv64(d4, 32) + cdiv64(n_mrows * d4, 256)), 256, 0)(
             l.hrows + hrow0, (int32_t)n_hrows, l.mrows + mrow0, (int32_t)n_mrows, l.slot0, l.tot, slot_base, a.scale, d4, partial, a.out_base, a.ld_out, a.omask,
             a.omask_words, a.ep, dbg_limits(a.src, a.halo, a.out, ctx->d_flag + 1));
         SAT_LAUNCHED(ctx);
@@ -777,7 +806,7 @@ __global__ void k_ent_all_gid(const int2 *__restrict__ ent, const int32_t *__res
 
 sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, const float *in_base, int32_t ld_in,
                     const float *halo_base, int32_t ld_halo, float *out_base, int32_t ld_out, const uint32_t *omask, int32_t omask_words,
-                    SpmmHalo halo_kind, bool in_global, const SpmmAdd &add)
+                    SpmmHalo halo_kind, bool in_global, const SpmmAdd &add, const RowMaxOut &row_max)
 {
     if (v.n_rows == 0) return SAT_OK;
     const int32_t d4 = (d + 3) / 4;
@@ -822,6 +851,8 @@ sat_status sat_spmm(sat_ctx *ctx, const PartView &v, int inner_only, int32_t d, 
     SAT_TRY(list_build(ctx, list_key(d4, inner_only), &l));
     a.scale = ctx->dinv_enc;
     a.ep.add = add;
+    a.ep.row_max = row_max;
+    a.ep.d = d;
     a.n = ctx->n;
     a.in_base = in_base;
     a.ld_in = ld_in;

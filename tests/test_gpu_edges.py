@@ -709,3 +709,124 @@ def test_input_gradient_in_both_orders(B, d_in, d_out, hist):
     want, mag = (same @ D.astype(np.float64) + stale) @ W2.T, (abs(same) @ np.abs(D.astype(np.float64)) + np.abs(stale)) @ np.abs(W2.T)
     terms = np.diff(A.indptr).max() + d_out + 8
     assert (np.abs(got - want[perm] * keep) <= (terms * U + 2.0 ** -20) * mag[perm]).all()
+
+
+# halves from 192 terms on in large graphs, from 384 on in all; B resident and not, one and two tiles of columns
+@pytest.mark.parametrize("m,n,k", [(m, n, k) for m in (1, 130) for n, k in ((16, 384), (40, 401), (256, 400), (512, 512), (300, 602))] +
+                         [(40000, 16, 192), (40000, 256, 256), (40000, 100, 320), (40000, 300, 602), (32767, 64, 383), (32768, 64, 192)])
+def test_contraction_of_rows_of_any_size(B, m, n, k):
+    """Long contractions split their operands into halves with a scale per row and per eight columns of W: rows and columns of very different sizes, rows of
+    zeros, and rows that are not finite and stay by themselves.  |x s - hi - lo| <= 2^-22 |x s| + 2^-25 with the largest |x s| at 2^14 or more.
+    In a graph without edges the product with P is the row itself."""
+    rng = np.random.default_rng(n + k)
+    A = (rng.standard_normal((m, k)) * np.exp2(rng.integers(-60, 60, (m, 1)))).astype(np.float32)
+    A[::7] *= np.exp2(rng.integers(-12, 1, (len(A[::7]), k))).astype(np.float32)       # a spread inside the row, too
+    A[5:6] = 0.0
+    W = (rng.standard_normal((k, n)) * np.exp2(rng.integers(-6, 6, (1, n)))).astype(np.float32)
+    out, bad = empty2d(m, n), empty2d(m, n)
+    A2 = A.copy()
+    not_finite = [r for r in (3, 64, 129) if r < m]
+    for r, v in zip(not_finite, (np.nan, np.inf, -np.inf)):
+        A2[r, rng.integers(0, k)] = v
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, np.zeros(m + 1, np.int64), np.zeros(0, np.int32))
+        B.sat_partition(ctx, 1, B.SAT_PART_CONTIG_BLOCKS)
+        for x, y in ((A, out), (A2, bad)):
+            B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, dev2d(x), None, dev(W), None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, y)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    out, bad = out.cpu().numpy(), bad.cpu().numpy()
+    sel = np.unique(np.concatenate([np.arange(min(m, 130)), rng.integers(0, m, 500)]))
+    a = A[sel].astype(np.float64)
+    mag = np.abs(a) @ np.abs(W)
+    floor = np.abs(a).max(1, keepdims=True) * 2.0 ** -39 * np.abs(W).sum(0)       # what a term loses below the smallest half
+    assert (np.abs(out[sel] - a @ W) <= ((k + 2) * U + 2.0 ** -20) * mag + 2 * floor).all()
+    assert (out[5:6] == 0).all()
+    ok = np.ones(m, bool)
+    ok[not_finite] = False
+    assert np.array_equal(out[ok], bad[ok]) and not np.isfinite(bad[~ok]).any()
+
+
+@pytest.mark.parametrize("kind", ["small", "hub", "large"])
+@pytest.mark.parametrize("d,n_out", [(383, 16), (384, 16), (512, 64), (602, 300)])     # the last without and the first with halves, several slices of columns
+def test_aggregated_rows_of_any_size(B, kind, d, n_out):
+    """The transform takes the size of every aggregated row from the product that wrote it: rows of one run, rows added by their last run and rows of the
+    second launch, one slice of columns and several.  A size that is too small would overflow a half, one that is too large lose the terms."""
+    A = _graph(HUBS, 3000) if kind == "small" else _many_runs(kind)
+    n, P = A.shape[0], _propagation(A)
+    rng = np.random.default_rng(d)
+    X = (rng.standard_normal((n, d)) * np.exp2(rng.integers(-30, 30, (n, 1)))).astype(np.float32)
+    W = rng.standard_normal((d, n_out)).astype(np.float32)
+    out = empty2d(n, n_out)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, 2, B.SAT_PART_CONTIG_BLOCKS)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, dev2d(X), None, dev(W), None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, out)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    agg, mag = P @ X.astype(np.float64), abs(P) @ np.abs(X.astype(np.float64))
+    terms = np.diff(A.indptr).max() + d + 8
+    floor = mag.max(1, keepdims=True) * 2.0 ** -39 * np.abs(W).sum(0)
+    assert (np.abs(out.cpu().numpy() - agg @ W) <= (terms * U + 2.0 ** -20) * (mag @ np.abs(W)) + 2 * floor).all()
+
+
+@pytest.mark.parametrize("d0,layer", [(24, 1), (400, 2)])      # pushed by either form of the contraction
+def test_pushed_rows_and_imported_rows_predict_alike(B, d0, layer):
+    """Snapshots that the layer pushed bring their rows' sizes along; imported ones have them looked for: the same prediction, bit for bit, also after a
+    single partition has pushed over imported rows."""
+    n, M, d, h = 1500, 3, 400, 32
+    A = _graph(HUBS[:8], n)
+    rng = np.random.default_rng(4)
+    part = rng.integers(0, M, n).astype(np.int32)
+    rand = lambda *s: dev(rng.standard_normal(s).astype(np.float32) / 8)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        B.sat_cache_init(ctx, [d] * layer, 2)
+        n_halo, n_slots = B.sat_part_sizes(ctx, B.SAT_ALL_PARTS)[1], B.sat_slot_map(ctx, n)[2]
+        off = np.concatenate([[0], np.cumsum(np.bincount(part, minlength=M))])
+        W, out = rand(d0, d), empty2d(n, d)
+        weights = [rand(d, 4 * h), rand(h, 4 * h), rand(4 * h), rand(h, d), rand(d)]
+        push = B.SAT_ACT_RELU | B.SAT_FWD_PUSH | B.SAT_FWD_INPUT_GLOBAL
+        for epoch in range(3):
+            X = dev2d((rng.standard_normal((n, d0)) * np.exp2(rng.integers(-9, 9, (n, 1)))).astype(np.float32))
+            B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, layer, X, None, W, None, push, out)
+            B.sat_cache_commit(ctx)
+        got = [empty2d(n_halo, d) for _ in range(4)]
+        for i, version in ((0, 0), (1, 1)):
+            p = B.make_pred_params(*weights, h, version, B.SAT_CELL_LSTM)
+            B.sat_predict(ctx, layer, B.SAT_ALL_PARTS, p, 0, got[i])
+        state = B.sat_cache_state(ctx)
+        ring = B.sat_cache_export(ctx, layer, 2, n_slots, d)
+        for i, version in ((2, 0), (3, 2)):
+            B.sat_cache_import(ctx, layer, ring)
+            B.sat_cache_set_state(ctx, *state)
+            # the next snapshot: one partition's rows over imported ones
+            B.sat_layer_fwd(ctx, 1, layer, X, None, W, None, push, out[off[1]:off[2]])
+            p = B.make_pred_params(*weights, h, version, B.SAT_CELL_LSTM)
+            B.sat_predict(ctx, layer, B.SAT_ALL_PARTS, p, 0, got[i])
+        assert torch.equal(got[0], got[2]) and torch.equal(got[1], got[3])
+        B.sat_cache_commit(ctx)                  # the mixed snapshot is the newest one
+        B.sat_predict(ctx, layer, B.SAT_ALL_PARTS, B.make_pred_params(*weights, h, 0, B.SAT_CELL_LSTM), 0, got[0])
+        state, ring = B.sat_cache_state(ctx), B.sat_cache_export(ctx, layer, 2, n_slots, d)
+        B.sat_cache_import(ctx, layer, ring)
+        B.sat_predict(ctx, layer, B.SAT_ALL_PARTS, B.make_pred_params(*weights, h, 0, B.SAT_CELL_LSTM), 0, got[2])
+        assert torch.equal(got[0], got[2])
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+
+
+@pytest.mark.parametrize("h", [4, 20, 64])
+@pytest.mark.parametrize("d", [384, 401])
+def test_recurrent_cells_on_halves(B, d, h):
+    """The cells' contractions over [x | s] and over projections where the input is wide enough for halves: the state's part has the scale of the input's
+    rows or of one, whichever is larger."""
+    test_gru_state(B, d, h, 3)
+    for versions in ([0, 0, 0], [1, 2, 1, 1], [1, 1, 1]):
+        test_lstm_state_over_cached_projections(B, 700, h, d, versions)
