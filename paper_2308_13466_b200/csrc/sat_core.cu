@@ -170,6 +170,8 @@ static void free_layers(sat_ctx *ctx)
         dev_free(&ctx->layers[i].agg);
         dev_free(&ctx->layers[i].agg_max);
         dev_free(&ctx->layers[i].mask);
+        sat_free_buf(ctx->layers[i].packed[0]);
+        sat_free_buf(ctx->layers[i].packed[1]);
         ctx->layers[i] = LayerState();
         dev_free(&ctx->ghist[i].buf);
         ctx->ghist[i] = GradHist();

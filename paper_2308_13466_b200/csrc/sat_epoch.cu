@@ -81,8 +81,13 @@ extern "C" sat_status sat_epoch(sat_ctx *ctx, const sat_epoch_buffers *e, const 
     CHECK_CTX(ctx);
     SAT_TRY(epoch_check(ctx, e, order, n_order, flags));
     const bool begin = !(flags & SAT_EPOCH_CONTINUE);
-    for (int32_t i = 0; i < (order ? n_order : 1); ++i)
-        SAT_TRY(epoch_pass(ctx, e, order ? order[i] : (int32_t)SAT_ALL_PARTS, i == 0 && begin, flags & SAT_EPOCH_GRAD_HISTORY));
+    for (int32_t l = 0; l <= SAT_MAX_LAYERS; ++l) ctx->layers[l].packed_as[0] = ctx->layers[l].packed_as[1] = 0;
+    ctx->keep_packed = order && n_order > 1;   // the parameter step comes after the passes
+    sat_status st = SAT_OK;
+    for (int32_t i = 0; i < (order ? n_order : 1) && st == SAT_OK; ++i)
+        st = epoch_pass(ctx, e, order ? order[i] : (int32_t)SAT_ALL_PARTS, i == 0 && begin, flags & SAT_EPOCH_GRAD_HISTORY);
+    ctx->keep_packed = false;
+    SAT_TRY(st);
     if (order && n_order == 0 && begin && e->loss_sum) SAT_CUDA(ctx, cudaMemsetAsync(e->loss_sum, 0, sizeof(double), ctx->stream));   // the loss of no partition
     if (flags & SAT_EPOCH_COMMIT) SAT_TRY(sat_cache_commit(ctx));
     if (flags & SAT_EPOCH_STEP) {

@@ -2141,24 +2141,24 @@ sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1,
     return SAT_OK;
 }
 
-// the description of planes that an earlier sat_tc_weights call (single source, k terms, n outputs) left in `buf`
-sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out)
+// the description of planes that an earlier sat_tc_weights call (single source, k terms, n outputs, `bias`: with one) left in `buf`
+sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out, bool bias)
 {
     if (out->half) {
         if (!buf.p || buf.bytes < half_layout((int32_t)cdiv64(k, TCH_BK), n, buf.p, out)) return SAT_ESTATE;
-        out->bias = nullptr;
+        if (!bias) out->bias = nullptr;
         return SAT_OK;
     }
     const int32_t k_pad = (k + TC_BK - 1) / TC_BK * TC_BK;
     const int32_t bn = tile_n_for(n);
     const int32_t n_pad = (n + bn - 1) / bn * bn;
     const size_t plane = ((size_t)n_pad * k_pad * sizeof(float) + 255) & ~(size_t)255;
-    if (!buf.p || buf.bytes < 2 * plane) return SAT_ESTATE;
+    if (!buf.p || buf.bytes < 2 * plane + (bias ? (size_t)n_pad * sizeof(float) : 0)) return SAT_ESTATE;
     out->hi = (float *)buf.p;
     out->lo = (float *)((char *)buf.p + plane);
     out->ld = k_pad;
     out->n_pad = n_pad;
-    out->bias = nullptr;
+    out->bias = bias ? (float *)((char *)buf.p + 2 * plane) : nullptr;
     return SAT_OK;
 }
 

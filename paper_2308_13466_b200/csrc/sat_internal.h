@@ -70,6 +70,8 @@ struct LayerState {
     int32_t d_in = 0, d_out = 0, ld_in = 0, mask_words = 0;
     int act = 0;
     std::vector<uint8_t> valid;  // per partition: forward state present
+    DevBuf packed[2];            // weights as the forward and the backward contraction take them, kept while sat_ctx::keep_packed
+    uint8_t packed_as[2] = {0, 0};   // 0: not there, 1: TF32 planes, 2: half-precision pairs
 };
 
 struct CacheLayer {
@@ -218,6 +220,7 @@ struct sat_ctx {
     GradHist ghist[SAT_MAX_LAYERS + 1];
     GatState gat[SAT_MAX_LAYERS + 1];
 
+    bool keep_packed = false;   // inside sat_epoch over several partitions: the parameters of the layers stay as they are until its end
     // ---- scratch ----
     DevBuf buf_codec_sizes, buf_codec_off, buf_codec_bytes;  // embedding codec scratch
     DevBuf buf_ticket, buf_partial, buf_gagg, buf_splitk, buf_lstm_c, buf_lstm_s, buf_lstm_w, buf_pred_a, buf_misc, buf_colsum, buf_dmask,
@@ -588,7 +591,7 @@ sat_status sat_mask_rows(sat_ctx *ctx, const float *src, int32_t ld, int64_t row
 // of hidden unit j (what the fused LSTM epilogue expects); gates = 3: the GRU's, see k_split_weights
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
                           int transpose, DevBuf &buf, TcWeights *out, int32_t gate_h = 0, int gates = 4, const float *bias = nullptr);
-sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out);
+sat_status sat_tc_weights_layout(int32_t k, int32_t n, const DevBuf &buf, TcWeights *out, bool bias = false);
 // Plane of an input projection x Wx + b of the LSTM, [row tile of 128][unit][row of the tile][i f g o]
 inline int64_t sat_proj_floats(int64_t rows, int32_t h) { return (rows + 127) / 128 * 512 * h; }
 // LSTM steps over `n_steps` projection planes, oldest first, on the state S [rows x h] and the cell state (sat_cell_offset layout; read

@@ -713,6 +713,20 @@ sat_status sat_row_slots(sat_ctx *ctx, const int32_t **out)
     return SAT_OK;
 }
 
+// Weights of a layer for its forward (transpose = 1) or backward contraction.  The calls of an epoch partition by partition take them from the first one's
+// packing (169343 nodes in eight partitions: epoch 4195 -> 4139 us).
+static sat_status layer_weights(sat_ctx *ctx, LayerState &L, const float *W, int32_t ldw, int32_t k, int32_t n, int transpose, const float *bias, TcWeights *out)
+{
+    if (!ctx->keep_packed) return sat_tc_weights(ctx, W, ldw, k, nullptr, 0, 0, n, transpose, ctx->buf_wsplit, out, 0, 4, bias);
+    const int i = transpose ? 0 : 1;
+    const uint8_t as = out->half ? 2 : 1;
+    if (L.packed_as[i] == as) return sat_tc_weights_layout(k, n, L.packed[i], out, bias != nullptr);
+    L.packed_as[i] = 0;
+    SAT_TRY(sat_tc_weights(ctx, W, ldw, k, nullptr, 0, 0, n, transpose, L.packed[i], out, 0, 4, bias));
+    L.packed_as[i] = as;
+    return SAT_OK;
+}
+
 extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int32_t d_in, int32_t d_out, const float *h_in,
                                     int32_t ld_in, const float *h_halo, int32_t ld_halo, const float *W, const float *bias, int act,
                                     float *h_out, int32_t ld_out)
@@ -778,7 +792,7 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
     const float *agg = L.agg + (int64_t)v.row0 * ld_agg;
     if (sat_use_tc(d_out, d_in)) {
         TcWeights Wp(half);
-        SAT_TRY(sat_tc_weights(ctx, W, d_out, d_in, nullptr, 0, 0, d_out, 1, ctx->buf_wsplit, &Wp, 0, 4, bias));
+        SAT_TRY(layer_weights(ctx, L, W, d_out, d_in, d_out, 1, bias, &Wp));
         TcEpilogueHost eh;
         eh.C = h_out;
         eh.ldc = ld_out;
@@ -896,13 +910,14 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
     if (!want_dx) return SAT_OK;
     const bool half_x = tc_x && sat_tc_half(ctx, d_out);
     const bool stale_term = hist && GH.has_read && g_in && v.n_push > 0;
-    // G_in = P_in^T (D W^T) = (P_in^T D) W^T.  The second order gathers rows of d_out columns instead of d_in: taken where that is less
+    // G_in = P_in^T (D W^T) = (P_in^T D) W^T.  The second order gathers rows of d_out columns instead of d_in: taken where that is less and not
+    // the same four lanes a row either way (2,048 nodes, 16 -> 4: 84.7 us with the first order, 85.2 with the second)
     // (256 -> 40, 169343 nodes, 2.6 M entries: product 152 -> 53 us, epoch 2840 -> 2749; 128 -> 19, 240000 nodes: epoch 1669 -> 1524;
     // 256 -> 47, 612257 nodes, 31 M entries: product 608 -> 165 us, epoch 16050 -> 15748).  The stale rows then join P_in^T D in the product's
     // epilogue, which makes their own contraction and the add into G_in unnecessary, so with them the order pays at equal
     // widths too (84671 nodes, 256 -> 256 -> 40, epoch with the predictor trained: 5342 -> 5087).  So it does where the contraction takes
     // half-precision pairs: the product leaves the largest magnitudes of its rows.
-    if (g_in && !g_halo && (!mask || tc_x) && (stale_term || half_x ? d_out <= d_in : d_out < d_in)) {
+    if (g_in && !g_halo && (!mask || tc_x) && (stale_term || half_x ? d_out <= d_in : d_out < d_in && d_in > 16)) {
         const int32_t ld_q = round_up4(d_out);
         SAT_TRY(sat_ensure(ctx, ctx->buf_gagg, (size_t)v.n_rows * ld_q * sizeof(float)));
         float *q = (float *)ctx->buf_gagg.p;
@@ -922,7 +937,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
         const uint32_t *keep = mask_in ? mask_in + (int64_t)v.row0 * mask_in_words : nullptr;
         if (!tc_x) return sat_gemm_nt(ctx, v.n_rows, d_in, d_out, q, ld_q, nullptr, 0, W, d_out, g_in, ld_gin, keep, mask_in_words);
         TcWeights Wp(half_x);
-        SAT_TRY(sat_tc_weights(ctx, W, d_out, d_out, nullptr, 0, 0, d_in, 0, ctx->buf_wsplit, &Wp));
+        SAT_TRY(layer_weights(ctx, L, W, d_out, d_out, d_in, 0, nullptr, &Wp));
         TcEpilogueHost eh;
         eh.C = g_in;
         eh.ldc = ld_gin;
@@ -937,7 +952,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
     float *gagg = (float *)ctx->buf_gagg.p;
     if (tc_x) {
         TcWeights Wp;
-        SAT_TRY(sat_tc_weights(ctx, W, d_out, d_out, nullptr, 0, 0, d_in, 0, ctx->buf_wsplit, &Wp));
+        SAT_TRY(layer_weights(ctx, L, W, d_out, d_out, d_in, 0, nullptr, &Wp));
         TcEpilogueHost eh;
         eh.C = gagg;
         eh.ldc = ld_ga;
@@ -958,7 +973,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
         SAT_TRY(sat_gather(ctx, ctx->push_slot + v.push0, v.n_push, d_out, qr, GH.ld, rows, GH.ld, DbgRange{0, ctx->n_slots}));
         if (sat_use_tc(d_in, d_out)) {
             TcWeights Wp;
-            SAT_TRY(sat_tc_weights(ctx, W, d_out, d_out, nullptr, 0, 0, d_in, 0, ctx->buf_wsplit, &Wp));
+            SAT_TRY(layer_weights(ctx, L, W, d_out, d_out, d_in, 0, nullptr, &Wp));
             TcEpilogueHost eh;
             eh.C = stale;
             eh.ldc = ld_ga;

@@ -830,3 +830,31 @@ def test_recurrent_cells_on_halves(B, d, h):
     test_gru_state(B, d, h, 3)
     for versions in ([0, 0, 0], [1, 2, 1, 1], [1, 1, 1]):
         test_lstm_state_over_cached_projections(B, 700, h, d, versions)
+
+
+@pytest.mark.parametrize("dims", [(24, 20, 12, 5), (24, 400, 400, 24)])      # TF32 terms, half-precision pairs
+def test_partitions_of_an_epoch_share_packed_weights(B, dims):
+    """The passes of an epoch partition by partition take the weights that the first one packed; the next epoch packs its own, whatever happened to the
+    parameters in between (here: a write to the same tensors).  Same bits as all partitions in one launch."""
+    from paper_2308_13466_b200.epoch import SatEpoch
+    n, M = 900, 3
+    A = _graph([300, 40], n)
+    rng = np.random.default_rng(dims[1])
+    rand = lambda *s: dev(rng.standard_normal(s).astype(np.float32) / s[0] ** 0.5)
+    X, labels = dev2d(rng.standard_normal((n, dims[0])).astype(np.float32)), dev(rng.integers(0, dims[-1], n).astype(np.int32))
+    eps = [SatEpoch(A.indptr.astype(np.int64), A.indices.astype(np.int32), M, list(dims), 2, "ce") for _ in range(2)]
+    try:
+        W, b = [rand(x, y) for x, y in zip(dims, dims[1:])], [rand(y) for y in dims[1:]]
+        for ep in eps:
+            ep.set_inputs(X, labels)
+        for epoch in range(3):
+            eps[0].step_per_partition(W, b, None)
+            eps[1].step(W, b, None)
+            for l in range(1, len(dims)):
+                assert torch.equal(eps[0].H[l], eps[1].H[l]), (epoch, l)
+                assert torch.equal(eps[0].G[l], eps[1].G[l]), (epoch, l)
+            for w in W + b:
+                w.copy_(rand(*w.shape))
+    finally:
+        for ep in eps:
+            ep.close()
