@@ -910,14 +910,15 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
     if (!want_dx) return SAT_OK;
     const bool half_x = tc_x && sat_tc_half(ctx, d_out);
     const bool stale_term = hist && GH.has_read && g_in && v.n_push > 0;
-    // G_in = P_in^T (D W^T) = (P_in^T D) W^T.  The second order gathers rows of d_out columns instead of d_in: taken where that is less and not
-    // the same four lanes a row either way (2,048 nodes, 16 -> 4: 84.7 us with the first order, 85.2 with the second)
+    // G_in = P_in^T (D W^T) = (P_in^T D) W^T.  The second order gathers rows of d_out columns instead of d_in: taken where that is less and the
+    // graph is not small (by nodes, so that one partition and all of them add up alike; 6,000 nodes, 72 -> 40 -> 7: 254.8 and 253.5
+    // us, 8,292 nodes and 597 k entries, 64 -> 20: 260.8 and 266.1; 2,048 nodes, 16 -> 4: 84.7 and 85.2)
     // (256 -> 40, 169343 nodes, 2.6 M entries: product 152 -> 53 us, epoch 2840 -> 2749; 128 -> 19, 240000 nodes: epoch 1669 -> 1524;
     // 256 -> 47, 612257 nodes, 31 M entries: product 608 -> 165 us, epoch 16050 -> 15748).  The stale rows then join P_in^T D in the product's
     // epilogue, which makes their own contraction and the add into G_in unnecessary, so with them the order pays at equal
     // widths too (84671 nodes, 256 -> 256 -> 40, epoch with the predictor trained: 5342 -> 5087).  So it does where the contraction takes
     // half-precision pairs: the product leaves the largest magnitudes of its rows.
-    if (g_in && !g_halo && (!mask || tc_x) && (stale_term || half_x ? d_out <= d_in : d_out < d_in && d_in > 16)) {
+    if (g_in && !g_halo && (!mask || tc_x) && (stale_term || half_x ? d_out <= d_in : d_out < d_in && ctx->n >= 32768)) {
         const int32_t ld_q = round_up4(d_out);
         SAT_TRY(sat_ensure(ctx, ctx->buf_gagg, (size_t)v.n_rows * ld_q * sizeof(float)));
         float *q = (float *)ctx->buf_gagg.p;
