@@ -492,6 +492,7 @@ sat_status sat_gemm_tn_narrow(sat_ctx *ctx, int64_t rows, int32_t m, int32_t n, 
     (m <= 64 ? launch_tn_narrow<NT, 1>(ctx, rows, m, n, A, lda, B, ldb, accumulate, C, ldc, colsum)                      \
              : m <= 128 ? launch_tn_narrow<NT, 2>(ctx, rows, m, n, A, lda, B, ldb, accumulate, C, ldc, colsum)           \
                         : launch_tn_narrow<NT, 4>(ctx, rows, m, n, A, lda, B, ldb, accumulate, C, ldc, colsum))
+    if (n <= 8) return CALL(8);
     if (n <= 16) return CALL(16);
     if (n <= 24) return CALL(24);
     if (n <= 32) return CALL(32);

@@ -858,3 +858,9 @@ def test_partitions_of_an_epoch_share_packed_weights(B, dims):
     finally:
         for ep in eps:
             ep.close()
+
+
+@pytest.mark.parametrize("rows", [255, 256, 257, 21000])        # the general kernel below 256 rows
+@pytest.mark.parametrize("m,n", [(16, 1), (17, 4), (64, 7), (65, 8), (130, 9), (300, 15)])
+def test_weight_gradient_of_few_columns(B, rows, m, n):
+    test_weight_and_bias_gradient(B, rows, m, n)
