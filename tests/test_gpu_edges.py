@@ -864,3 +864,41 @@ def test_partitions_of_an_epoch_share_packed_weights(B, dims):
 @pytest.mark.parametrize("m,n", [(16, 1), (17, 4), (64, 7), (65, 8), (130, 9), (300, 15)])
 def test_weight_gradient_of_few_columns(B, rows, m, n):
     test_weight_and_bias_gradient(B, rows, m, n)
+
+
+@pytest.mark.parametrize("parts", [False, True])
+def test_prediction_from_rows_that_an_attention_layer_pushed(B, parts):
+    """The ring's rows change under sat_gat_fwd as under sat_cache_update: the same prediction, from rows whose size a half does not hold without their own scale."""
+    n, M, d, d_out, h = 1500, 3, 24, 400, 32
+    A = _graph(HUBS[:8], n)
+    rng = np.random.default_rng(7)
+    part = rng.integers(0, M, n).astype(np.int32)
+    rand = lambda *s: dev(rng.standard_normal(s).astype(np.float32) / 8)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        sizes = [B.sat_part_sizes(ctx, m) for m in range(M)]
+        n_halo = sum(s[1] for s in sizes)
+        H, halo = dev2d(1e6 * rng.standard_normal((n, d)).astype(np.float32)), dev2d(1e6 * rng.standard_normal((n_halo, d)).astype(np.float32))
+        W, a1, a2, b = rand(d, d_out), 1e-6 * rand(d_out), 1e-6 * rand(d_out), rand(d_out)
+        p = B.make_pred_params(1e-6 * rand(d_out, 4 * h), rand(h, 4 * h), rand(4 * h), rand(h, d_out), rand(d_out), h, 0, B.SAT_CELL_LSTM)
+        got = []
+        for push in (0, B.SAT_FWD_PUSH):
+            B.sat_cache_init(ctx, [d_out], 2)
+            out, pred = empty2d(n, d_out), empty2d(n_halo, d_out)
+            r0 = u0 = 0
+            for m in range(M) if parts else [B.SAT_ALL_PARTS]:
+                r1, u1 = (r0 + sizes[m][0], u0 + sizes[m][1]) if parts else (n, n_halo)
+                B.sat_gat_fwd(ctx, m, 1, H[r0:r1], halo[u0:u1], W, a1, a2, b, B.SAT_ACT_RELU | push, out[r0:r1])
+                if not push:
+                    B.sat_cache_update(ctx, m, 1, out[r0:r1])
+                r0, u0 = r1, u1
+            B.sat_cache_commit(ctx)
+            B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, p, 0, pred)
+            got.append((out.clone(), pred.clone(), B.sat_predict_state(ctx, 1, B.sat_slot_map(ctx, n)[2], h)))
+        assert float(got[0][0].abs().max()) > 65504 and np.isfinite(got[1][2]).all()
+        assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1]) and np.array_equal(got[0][2], got[1][2])
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
