@@ -2244,8 +2244,13 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     const int32_t n_tiles_n = (int32_t)cdiv64(n, bn);
     const bool pair = !eh.resid_idx && cdiv64(m, TC_BM) * n_tiles_n > ctx->sms;
     const int ctas = pair ? 2 : 1;
-    // a B of half-precision pairs of at most 128 KB per CTA stays in shared memory (its CTAs then keep to their columns)
-    const uint32_t b_bytes = (uint32_t)bn / ctas * 128, b_all = b_bytes * (nkb1 + nkb2), b_resident = half && b_all <= 131072u ? b_all : 0;
+    // a B of half-precision pairs of at most 128 KB per CTA stays in shared memory, where there are as many CTAs (or pairs) as column tiles: it is
+    // loaded once, for the columns of the CTA's first tile, so the number of CTAs has to be a multiple of the number of column tiles
+    int64_t units = ctx->sms / ctas;
+    const uint32_t b_bytes = (uint32_t)bn / ctas * 128;
+    const int64_t b_all = (int64_t)b_bytes * (nkb1 + nkb2);
+    const uint32_t b_resident = half && b_all <= 131072 && n_tiles_n <= units ? (uint32_t)b_all : 0;
+    if (b_resident) units -= units % n_tiles_n;
     const uint32_t stage_bytes = half ? TCH_A_BYTES + (b_resident ? 0 : b_bytes) : 2 * (TC_BM * TC_BK * 4) + b_bytes;
     // algorithmic bytes: operands once, results once.  Plain: A, B, C.  Gathered residual: + the residual rows.  LSTM cell:
     // the output is the hidden state [m x h] plus the cell state read and written, and the cached projection if it is added.
@@ -2318,8 +2323,6 @@ sat_status sat_gemm_tc(sat_ctx *ctx, int64_t m, int32_t n, const float *A, int32
     ep.ld_resid = eh.ld_resid;
     ep.tile_order = eh.tile_order;
     const int64_t n_tiles = cdiv64(m, TC_BM * ctas) * n_tiles_n;
-    int64_t units = ctx->sms / ctas;
-    if (b_resident && units > n_tiles_n) units -= units % n_tiles_n;
     const unsigned grid = (unsigned)(n_tiles < units ? n_tiles : units) * ctas;
     TckLaunch L;
     L.mA = mA; L.mA2 = mA2; L.mB = mB; L.mBlo = mBlo; L.mC = mC;

@@ -902,3 +902,32 @@ def test_prediction_from_rows_that_an_attention_layer_pushed(B, parts):
         B.sat_sync_status(ctx)
     finally:
         B.sat_destroy(ctx)
+
+
+def _rows_times(B, A, W, bias=None):
+    """A W + bias by the transform of layer 2 of a graph without edges, where the product with P is the row itself."""
+    m, n = len(A), W.shape[1]
+    out = empty2d(m, n)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, np.zeros(m + 1, np.int64), np.zeros(0, np.int32))
+        B.sat_partition(ctx, 1, B.SAT_PART_CONTIG_BLOCKS)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, dev2d(A), None, dev(W), None if bias is None else dev(bias), B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, out)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    return out
+
+
+# one column tile to three with B resident; one tile more than there are pairs of SMs, where it is not (18,944 columns are 74 tiles)
+@pytest.mark.parametrize("m,n,k", [(33000, 300, 256), (33000, 700, 256), (33000, 770, 192), (33000, 18944, 192), (33000, 18945, 192), (257, 38000, 384)])
+def test_contraction_with_many_column_tiles(B, m, n, k):
+    rng = np.random.default_rng(n)
+    A, W, bias = (rng.standard_normal(s).astype(np.float32) for s in ((m, k), (k, n), (n,)))
+    out = _rows_times(B, A, W, bias)
+    tiles = -(-n // 256)
+    width = -(-(-(-n // tiles)) // 32) * 32
+    cols = np.unique(np.concatenate([np.arange(0, n, width), np.arange(width - 1, n, width), rng.integers(0, n, 60), [n - 1]]))
+    got = out[:, dev(cols.astype(np.int64))].cpu().numpy()
+    a, w = A.astype(np.float64), W[:, cols].astype(np.float64)
+    assert (np.abs(got - (a @ w + bias[cols])) <= ((k + 3) * U + 2.0 ** -20) * (np.abs(a) @ np.abs(w) + np.abs(bias[cols]))).all()
