@@ -245,6 +245,15 @@ __device__ __forceinline__ uint32_t f16_scale_exponent(uint32_t largest)
     return largest == 0 || largest == 255 ? 127u : (uint32_t)(e > 253 ? 253 : e);
 }
 
+// (x s) s2 + y by packed operations (each component rounded as by itself)
+__device__ __forceinline__ float4 scaled_add(const uint32_t *x, const float4 &s, const float4 &y, const float2 &s2)
+{
+    const float2 lo = __fmul2_rn(make_float2(__uint_as_float(x[0]), __uint_as_float(x[1])), make_float2(s.x, s.y));
+    const float2 hi = __fmul2_rn(make_float2(__uint_as_float(x[2]), __uint_as_float(x[3])), make_float2(s.z, s.w));
+    const float2 a = __ffma2_rn(lo, s2, make_float2(y.x, y.y)), b = __ffma2_rn(hi, s2, make_float2(y.z, y.w));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
 // =====================================================================================
 // TF32 split of a shared-memory tile, element-wise (the swizzled layout never has to be decoded).
 //
@@ -333,7 +342,7 @@ struct TcEpilogue {
     int32_t row_parts;
     uint32_t row_least;      // what the largest magnitude is taken to be at least (bits)
     int32_t k1, k2;          // terms of the A operands
-    const float *unscale;    // inverse scale of every eight columns of B
+    const float *unscale;    // inverse scale of every column of B
     float *C;
     int64_t ldc;
     const float *bias;
@@ -1106,26 +1115,23 @@ k_gemm_tc_h(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             for (int c0 = c_first; c0 < bn; c0 += CHUNK_STEP) {
                 uint32_t r[32];
                 tc_ld32(tmem + buf * acc_cols + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-                float4 us = __ldg(reinterpret_cast<const float4 *>(ep.unscale + ((n0 + c0) >> 3)));   // takes the scales out, eight columns each
-                us.x *= unscale; us.y *= unscale; us.z *= unscale; us.w *= unscale;
-                const float us4[4] = {us.x, us.y, us.z, us.w};
+                // takes the scales out and adds the bias to four columns: the column's scale first, since the product of the two may lie outside of fp32
+                auto finish = [&](uint32_t *x, int u) {
+                    const float4 us = __ldg(reinterpret_cast<const float4 *>(ep.unscale + n0 + c0) + u);
+                    const float4 b4 = ep.bias ? __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + c0) + u) : zero4;
+                    const float4 y = scaled_add(x, us, b4, make_float2(unscale, unscale));
+                    x[0] = __float_as_uint(y.x);
+                    x[1] = __float_as_uint(y.y);
+                    x[2] = __float_as_uint(y.z);
+                    x[3] = __float_as_uint(y.w);
+                };
                 if (LSTM) {
                     // packed columns 4 j .. 4 j + 3 are the (i, f, g, o) pre-activations of hidden unit j
                     if (row_ok) {
                         const int32_t j0 = (n0 + c0) >> 2;
                         const bool full = lstm_full && j0 + 7 < ep.lstm_h;
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            float4 b4 = zero4;
-                            if (ep.bias) {
-                                const float4 bb = __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + c0) + u);
-                                b4.x += bb.x; b4.y += bb.y; b4.z += bb.z; b4.w += bb.w;
-                            }
-                            r[4 * u] = __float_as_uint(fmaf(__uint_as_float(r[4 * u]), us4[u >> 1], b4.x));
-                            r[4 * u + 1] = __float_as_uint(fmaf(__uint_as_float(r[4 * u + 1]), us4[u >> 1], b4.y));
-                            r[4 * u + 2] = __float_as_uint(fmaf(__uint_as_float(r[4 * u + 2]), us4[u >> 1], b4.z));
-                            r[4 * u + 3] = __float_as_uint(fmaf(__uint_as_float(r[4 * u + 3]), us4[u >> 1], b4.w));
-                        }
+                        for (int u = 0; u < 8; ++u) finish(r + 4 * u, u);
                         float cprev[8];
                         cprev[0] = cside[0].x; cprev[1] = cside[0].y; cprev[2] = cside[0].z; cprev[3] = cside[0].w;
                         cprev[4] = cside[1].x; cprev[5] = cside[1].y; cprev[6] = cside[1].z; cprev[7] = cside[1].w;
@@ -1177,17 +1183,7 @@ k_gemm_tc_h(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     // bias is padded with zeros to the tile width and the accumulators of padded columns are exactly zero,
                     // so no column predicate is needed (the stores clip)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        float4 b4 = zero4;
-                        if (ep.bias) {
-                            const float4 bb = __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + c0) + j);
-                            b4.x += bb.x; b4.y += bb.y; b4.z += bb.z; b4.w += bb.w;
-                        }
-                        r[4 * j] = __float_as_uint(fmaf(__uint_as_float(r[4 * j]), us4[j >> 1], b4.x));
-                        r[4 * j + 1] = __float_as_uint(fmaf(__uint_as_float(r[4 * j + 1]), us4[j >> 1], b4.y));
-                        r[4 * j + 2] = __float_as_uint(fmaf(__uint_as_float(r[4 * j + 2]), us4[j >> 1], b4.z));
-                        r[4 * j + 3] = __float_as_uint(fmaf(__uint_as_float(r[4 * j + 3]), us4[j >> 1], b4.w));
-                    }
+                    for (int j = 0; j < 8; ++j) finish(r + 4 * j, j);
                     if ((EPI == EPI_PLAIN || EPI == EPI_PUSH) && ep.mask_out) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j) bits |= (__uint_as_float(r[j]) > 0.f ? 1u : 0u) << j;
@@ -1326,7 +1322,9 @@ done:
 // CTA pair held TF32 terms and the projections came through registers, two quads ahead; that form was bound by its latencies with every
 // unit below 45 %.  What did it: the copies' depth and their .cg (.ca: 184 us) and the accumulator columns a quad ahead.  (Bulk copies
 // by a warp of their own per slot, which leaves 96 registers: 192 us.)  The errors are what they were (relative 1.6e-6 of the
-// state at K = 256).
+// state at K = 256).  The inverse scales of a quad's sixteen columns come out of shared memory too, next to projections and state: 164833 rows 161 -> 180 us with
+// one for every column, so eight neighbours (a pair of units) share theirs where they are of a size (k_pack_half), and only a matrix where they are not
+// takes that form.
 // =====================================================================================
 #define SEQ_THREADS 512   /* 128 registers a thread */
 #define SEQ_RING 3        /* quads of projections in flight per thread */
@@ -1334,7 +1332,9 @@ struct SeqSteps {
     const float *proj[SAT_SEQ_MAX];
 };
 struct SeqShared {
-    float2 unscale[16];                              // per eight gate columns, of the state and the columns together
+    float4 unscale[64];                              // inverse scales of a unit's gate columns, the state's taken along
+    float2 pair_unscale[16];                         // of the pairs of units of a quad, whose columns share them unless
+    int own_scales;                                  // ... somewhere the columns of a pair have scales of their own
     uint64_t b_full;                                 // Uh has landed
     uint64_t a_ready[2], acc_full[2];                // per slot: the state is in place; the product is done
     uint32_t tmem_base;
@@ -1374,6 +1374,153 @@ __device__ __forceinline__ float lstm_cell(const float4 &z, float &c)
     return (ec - 1.f) * rcp_fast((1.f + eo) * (1.f + ec));
 }
 
+// The row tiles of a slot.  SHARED: the columns of a pair of units have one scale.
+template <bool SHARED>
+__device__ __forceinline__ void
+lstm_tiles(uint8_t *smem, uint8_t *Bs, uint8_t *Ps, SeqShared *sh, uint32_t tmem, const SeqSteps &steps, int32_t n_steps, int first, int64_t rows, int32_t h,
+           int32_t bn, int32_t nkb, int32_t mine, float *S, float *cell, int write_cell, int *status)
+{
+    constexpr uint32_t a_block = TC_BM * 128;
+    const uint32_t b_block = (uint32_t)bn * 128, slot_bytes = (uint32_t)nkb * a_block;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int32_t nq = h >> 2;                       // quads of four units
+    volatile int *dead = &sh->dead;
+    const int slot = warp >> 3, q = warp & 3, half = (warp >> 2) & 1;
+    const bool issuer = (warp & 7) == 0;   // of its slot's products
+    const uint32_t idesc = make_idesc_f16(TC_BM, bn), acc = tmem + (uint32_t)slot * 256u;
+    const uint64_t a0 = make_desc(smem_u32(smem) + (uint32_t)slot * slot_bytes, 16, 1024, 2), b0 = make_desc(smem_u32(Bs), 16, 1024, 2);
+    const int32_t nks = (h + 15) / 16;               // k-steps of 16
+    const int r_in = q * 32 + lane;                  // this thread's row of the tile
+    uint8_t *A = smem + (uint32_t)slot * slot_bytes + r_in * 128;
+    const uint32_t swz = (uint32_t)r_in & 7u;        // 16-byte piece c of row r sits at c ^ (r & 7)
+    uint8_t *const ring = Ps + threadIdx.x * 16;
+    const uint32_t mine_acc = acc + ((uint32_t)(q * 32) << 16);
+    auto put = [&](int qd, const float4 &v) {   // a quad is half a piece
+        uint2 hi, lo;
+        split_f16(v.x * 0x1p14f, v.y * 0x1p14f, hi.x, lo.x);
+        split_f16(v.z * 0x1p14f, v.w * 0x1p14f, hi.y, lo.y);
+        uint8_t *d = A + ((uint32_t)qd >> 3) * a_block + (((uint32_t)qd & 1u) << 3);
+        const uint32_t piece = ((uint32_t)qd & 4u) | (((uint32_t)qd & 3u) >> 1);
+        *reinterpret_cast<uint2 *>(d + ((piece ^ swz) << 4)) = hi;
+        *reinterpret_cast<uint2 *>(d + (((piece + 2) ^ swz) << 4)) = lo;
+    };
+    if (issuer && mine > slot && !mbar_wait_all(&sh->b_full, 0, dead, status)) return;
+    // this thread's quads in the order in which they are taken: (tile, step, quad); the copies run SEQ_RING of them ahead
+    const int32_t my_quads = (nq - half + 1) / 2;
+    int32_t pf_k = slot, pf_t = 0, pf_i = 0;
+    uint32_t pf_at = 0, at = 0;
+    auto copy_next = [&]() {   // a group a call, empty at the end
+        if (pf_k < mine && my_quads > 0) {
+            const float4 *src = reinterpret_cast<const float4 *>(steps.proj[pf_t]) +
+                                ((blockIdx.x + (int64_t)pf_k * gridDim.x) * h + 4 * (half + 2 * pf_i)) * TC_BM + r_in;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) cp_async16(ring + (pf_at * 4 + u) * (SEQ_THREADS * 16), src + u * TC_BM, true);
+            if (++pf_i == my_quads) {
+                pf_i = 0;
+                if (++pf_t == n_steps) pf_t = 0, pf_k += 2;
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        pf_at = pf_at + 1 == SEQ_RING ? 0 : pf_at + 1;
+    };
+#pragma unroll
+    for (int i = 0; i < SEQ_RING; ++i) copy_next();
+    if (issuer && mine > slot && !mbar_wait_all(&sh->b_full, 0, dead, status)) return;
+    uint32_t ph = 0;
+    for (int32_t k = slot; k < mine; k += 2) {
+        const int64_t row = (blockIdx.x + (int64_t)k * gridDim.x) * TC_BM + r_in;
+        const bool row_ok = row < rows;
+        float4 c[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int32_t qd = half + 2 * i;
+            c[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!first && qd < nq) {
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (row_ok) {
+                    v = *reinterpret_cast<const float4 *>(S + row * h + 4 * qd);
+                    c[i] = *reinterpret_cast<const float4 *>(cell + sat_cell_offset(row, 4 * qd, h));
+                }
+                put(qd, v);
+            }
+        }
+        for (int32_t t = 0; t < n_steps; ++t) {
+            const bool product = t > 0 || !first, last = t + 1 == n_steps;
+            if (product) {
+                fence_async_smem();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh->a_ready[slot]);
+                if (issuer) {
+                    if (!mbar_wait_all(&sh->a_ready[slot], ph, dead, status)) return;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        for (int32_t ks = 0; ks < nks; ++ks) {
+                            const uint64_t a_hi = a0 + (uint64_t)((ks >> 1) * (a_block >> 4) + (ks & 1) * 4), a_lo = a_hi + 2;
+                            const uint64_t b_hi = b0 + (uint64_t)((ks >> 1) * (b_block >> 4) + (ks & 1) * 4), b_lo = b_hi + 2;
+                            tc_mma_f16<1, 1>(acc, a_hi, b_hi, idesc, ks > 0 ? 1u : 0u);
+                            tc_mma_f16<2, 1>(acc, a_hi, b_lo, idesc, 1u);
+                            tc_mma_f16<0, 1>(acc, a_lo, b_hi, idesc, 1u);
+                        }
+                        tc_commit<1>(&sh->acc_full[slot]);
+                    }
+                    __syncwarp();
+                }
+                if (!mbar_wait_all(&sh->acc_full[slot], ph, dead, status)) return;
+                ph ^= 1u;
+                tc_fence_after();
+            }
+            uint32_t r[2][16];   // accumulator columns of this quad and the next
+            if (product && half < nq) tc_ld16(mine_acc + 16u * (uint32_t)half, r[0]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int32_t qd = half + 2 * i;
+                if (qd < nq) {
+                    asm volatile("cp.async.wait_group %0;" ::"n"(SEQ_RING - 1) : "memory");   // this thread's own copies
+                    float4 z[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) z[u] = *reinterpret_cast<const float4 *>(ring + (at * 4 + u) * (SEQ_THREADS * 16));
+                    at = at + 1 == SEQ_RING ? 0 : at + 1;
+                    if (product) {
+                        uint32_t(&a)[16] = r[i & 1];
+                        const float2 us2 = SHARED ? sh->pair_unscale[qd] : make_float2(0.f, 0.f);
+                        tc_wait16(a);
+                        if (i < 7 && qd + 2 < nq) tc_ld16(mine_acc + 16u * (uint32_t)(qd + 2), r[(i + 1) & 1]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            float4 us = make_float4(u < 2 ? us2.x : us2.y, 0.f, 0.f, 0.f);
+                            if (SHARED) us.y = us.z = us.w = us.x;
+                            else us = sh->unscale[4 * qd + u];
+                            z[u].x = fmaf(__uint_as_float(a[4 * u]), us.x, z[u].x);
+                            z[u].y = fmaf(__uint_as_float(a[4 * u + 1]), us.y, z[u].y);
+                            z[u].z = fmaf(__uint_as_float(a[4 * u + 2]), us.z, z[u].z);
+                            z[u].w = fmaf(__uint_as_float(a[4 * u + 3]), us.w, z[u].w);
+                        }
+                    }
+                    copy_next();   // (into the place just read)
+                    float4 sv;
+                    float *cf = reinterpret_cast<float *>(&c[i]), *sf = reinterpret_cast<float *>(&sv);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) sf[u] = lstm_cell(z[u], cf[u]);   // unit 4 qd + u
+                    if (!last) {
+                        put(qd, sv);
+                    } else if (row_ok) {
+                        *reinterpret_cast<float4 *>(S + row * h + 4 * qd) = sv;
+                        if (write_cell) *reinterpret_cast<float4 *>(cell + sat_cell_offset(row, 4 * qd, h)) = c[i];
+                    }
+                }
+            }
+        }
+    }
+}
+// (with registers of its own: in line with the other form it made that one spill, 161 -> 178 us)
+__device__ __noinline__ void
+lstm_tiles_own_scales(uint8_t *smem, uint8_t *Bs, uint8_t *Ps, SeqShared *sh, uint32_t tmem, const SeqSteps &steps, int32_t n_steps, int first, int64_t rows, int32_t h,
+                      int32_t bn, int32_t nkb, int32_t mine, float *S, float *cell, int write_cell, int *status)
+{
+    lstm_tiles<false>(smem, Bs, Ps, sh, tmem, steps, n_steps, first, rows, h, bn, nkb, mine, S, cell, write_cell, status);
+}
+
 __global__ void __launch_bounds__(SEQ_THREADS, 1)
 k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ unscale, const __grid_constant__ SeqSteps steps, int32_t n_steps, int first,
            int64_t rows, int32_t h, int32_t bn, int32_t nkb, float *S, float *cell, int write_cell,
@@ -1389,7 +1536,6 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n_rt = (rows + TC_BM - 1) / TC_BM;
     const int32_t mine = blockIdx.x < n_rt ? (int32_t)((n_rt - 1 - blockIdx.x) / gridDim.x + 1) : 0;   // row tiles of the CTA, alternately in slot 0 and 1
-    const int32_t nq = h >> 2;                                    // quads of four units
 
     for (uint32_t o = threadIdx.x * 16; o < 2 * slot_bytes; o += SEQ_THREADS * 16) *reinterpret_cast<float4 *>(smem + o) = make_float4(0.f, 0.f, 0.f, 0.f);
     fence_async_smem();   // (the columns from h on stay zero)
@@ -1399,7 +1545,7 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
             mbar_init(&sh->a_ready[i], 8);
             mbar_init(&sh->acc_full[i], 1);
         }
-        sh->dead = 0;
+        sh->dead = sh->own_scales = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tc_alloc<1>(&sh->tmem_base, 512u);
@@ -1409,7 +1555,12 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
     const uint32_t tmem = sh->tmem_base;
     volatile int *dead = &sh->dead;
     sat_grid_wait();
-    if (threadIdx.x < 32) reinterpret_cast<float *>(sh->unscale)[threadIdx.x] = 8 * (int)threadIdx.x < bn ? __ldg(unscale + threadIdx.x) * 0x1p-14f : 0.f;
+    if ((int)threadIdx.x < bn) {
+        const float us = __ldg(unscale + threadIdx.x) * 0x1p-14f;
+        reinterpret_cast<float *>(sh->unscale)[threadIdx.x] = us;
+        if (us != __shfl_sync(0xffffffffu, us, lane & 24)) sh->own_scales = 1;   // (whole warps: bn is a multiple of 32)
+        if ((lane & 7) == 0) reinterpret_cast<float *>(sh->pair_unscale)[threadIdx.x >> 3] = us;
+    }
     __syncthreads();
 
     if (warp == 0 && mine > 0) {
@@ -1419,133 +1570,8 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
         }
         if (!mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
     }
-    {
-        const int slot = warp >> 3, q = warp & 3, half = (warp >> 2) & 1;
-        const bool issuer = (warp & 7) == 0;   // of its slot's products
-        const uint32_t idesc = make_idesc_f16(TC_BM, bn), acc = tmem + (uint32_t)slot * 256u;
-        const uint64_t a0 = make_desc(smem_u32(smem) + (uint32_t)slot * slot_bytes, 16, 1024, 2), b0 = make_desc(smem_u32(Bs), 16, 1024, 2);
-        const int32_t nks = (h + 15) / 16;               // k-steps of 16
-        const int r_in = q * 32 + lane;                  // this thread's row of the tile
-        uint8_t *A = smem + (uint32_t)slot * slot_bytes + r_in * 128;
-        const uint32_t swz = (uint32_t)r_in & 7u;        // 16-byte piece c of row r sits at c ^ (r & 7)
-        uint8_t *const ring = Ps + threadIdx.x * 16;
-        const uint32_t mine_acc = acc + ((uint32_t)(q * 32) << 16);
-        auto put = [&](int qd, const float4 &v) {   // a quad is half a piece
-            uint2 hi, lo;
-            split_f16(v.x * 0x1p14f, v.y * 0x1p14f, hi.x, lo.x);
-            split_f16(v.z * 0x1p14f, v.w * 0x1p14f, hi.y, lo.y);
-            uint8_t *d = A + ((uint32_t)qd >> 3) * a_block + (((uint32_t)qd & 1u) << 3);
-            const uint32_t piece = ((uint32_t)qd & 4u) | (((uint32_t)qd & 3u) >> 1);
-            *reinterpret_cast<uint2 *>(d + ((piece ^ swz) << 4)) = hi;
-            *reinterpret_cast<uint2 *>(d + (((piece + 2) ^ swz) << 4)) = lo;
-        };
-        if (issuer && mine > slot && !mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
-        // this thread's quads in the order in which they are taken: (tile, step, quad); the copies run SEQ_RING of them ahead
-        const int32_t my_quads = (nq - half + 1) / 2;
-        int32_t pf_k = slot, pf_t = 0, pf_i = 0;
-        uint32_t pf_at = 0, at = 0;
-        auto copy_next = [&]() {   // a group a call, empty at the end
-            if (pf_k < mine && my_quads > 0) {
-                const float4 *src = reinterpret_cast<const float4 *>(steps.proj[pf_t]) +
-                                    ((blockIdx.x + (int64_t)pf_k * gridDim.x) * h + 4 * (half + 2 * pf_i)) * TC_BM + r_in;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) cp_async16(ring + (pf_at * 4 + u) * (SEQ_THREADS * 16), src + u * TC_BM, true);
-                if (++pf_i == my_quads) {
-                    pf_i = 0;
-                    if (++pf_t == n_steps) pf_t = 0, pf_k += 2;
-                }
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            pf_at = pf_at + 1 == SEQ_RING ? 0 : pf_at + 1;
-        };
-#pragma unroll
-        for (int i = 0; i < SEQ_RING; ++i) copy_next();
-        if (issuer && mine > slot && !mbar_wait_all(&sh->b_full, 0, dead, status)) goto done;
-        uint32_t ph = 0;
-        for (int32_t k = slot; k < mine; k += 2) {
-            const int64_t row = (blockIdx.x + (int64_t)k * gridDim.x) * TC_BM + r_in;
-            const bool row_ok = row < rows;
-            float4 c[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int32_t qd = half + 2 * i;
-                c[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (!first && qd < nq) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (row_ok) {
-                        v = *reinterpret_cast<const float4 *>(S + row * h + 4 * qd);
-                        c[i] = *reinterpret_cast<const float4 *>(cell + sat_cell_offset(row, 4 * qd, h));
-                    }
-                    put(qd, v);
-                }
-            }
-            for (int32_t t = 0; t < n_steps; ++t) {
-                const bool product = t > 0 || !first, last = t + 1 == n_steps;
-                if (product) {
-                    fence_async_smem();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sh->a_ready[slot]);
-                    if (issuer) {
-                        if (!mbar_wait_all(&sh->a_ready[slot], ph, dead, status)) goto done;
-                        tc_fence_after();
-                        if (elect_one()) {
-                            for (int32_t ks = 0; ks < nks; ++ks) {
-                                const uint64_t a_hi = a0 + (uint64_t)((ks >> 1) * (a_block >> 4) + (ks & 1) * 4), a_lo = a_hi + 2;
-                                const uint64_t b_hi = b0 + (uint64_t)((ks >> 1) * (b_block >> 4) + (ks & 1) * 4), b_lo = b_hi + 2;
-                                tc_mma_f16<1, 1>(acc, a_hi, b_hi, idesc, ks > 0 ? 1u : 0u);
-                                tc_mma_f16<2, 1>(acc, a_hi, b_lo, idesc, 1u);
-                                tc_mma_f16<0, 1>(acc, a_lo, b_hi, idesc, 1u);
-                            }
-                            tc_commit<1>(&sh->acc_full[slot]);
-                        }
-                        __syncwarp();
-                    }
-                    if (!mbar_wait_all(&sh->acc_full[slot], ph, dead, status)) goto done;
-                    ph ^= 1u;
-                    tc_fence_after();
-                }
-                uint32_t r[2][16];   // accumulator columns of this quad and the next
-                if (product && half < nq) tc_ld16(mine_acc + 16u * (uint32_t)half, r[0]);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int32_t qd = half + 2 * i;
-                    if (qd < nq) {
-                        asm volatile("cp.async.wait_group %0;" ::"n"(SEQ_RING - 1) : "memory");   // this thread's own copies
-                        float4 z[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) z[u] = *reinterpret_cast<const float4 *>(ring + (at * 4 + u) * (SEQ_THREADS * 16));
-                        at = at + 1 == SEQ_RING ? 0 : at + 1;
-                        if (product) {
-                            uint32_t(&a)[16] = r[i & 1];
-                            const float2 us2 = sh->unscale[qd];
-                            tc_wait16(a);
-                            if (i < 7 && qd + 2 < nq) tc_ld16(mine_acc + 16u * (uint32_t)(qd + 2), r[(i + 1) & 1]);
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const float us = u < 2 ? us2.x : us2.y;
-                                z[u].x = fmaf(__uint_as_float(a[4 * u]), us, z[u].x);
-                                z[u].y = fmaf(__uint_as_float(a[4 * u + 1]), us, z[u].y);
-                                z[u].z = fmaf(__uint_as_float(a[4 * u + 2]), us, z[u].z);
-                                z[u].w = fmaf(__uint_as_float(a[4 * u + 3]), us, z[u].w);
-                            }
-                        }
-                        copy_next();   // (into the place just read)
-                        float4 sv;
-                        float *cf = reinterpret_cast<float *>(&c[i]), *sf = reinterpret_cast<float *>(&sv);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) sf[u] = lstm_cell(z[u], cf[u]);   // unit 4 qd + u
-                        if (!last) {
-                            put(qd, sv);
-                        } else if (row_ok) {
-                            *reinterpret_cast<float4 *>(S + row * h + 4 * qd) = sv;
-                            if (write_cell) *reinterpret_cast<float4 *>(cell + sat_cell_offset(row, 4 * qd, h)) = c[i];
-                        }
-                    }
-                }
-            }
-        }
-    }
+    if (sh->own_scales) lstm_tiles_own_scales(smem, Bs, Ps, sh, tmem, steps, n_steps, first, rows, h, bn, nkb, mine, S, cell, write_cell, status);
+    else lstm_tiles<true>(smem, Bs, Ps, sh, tmem, steps, n_steps, first, rows, h, bn, nkb, mine, S, cell, write_cell, status);
 done:
     asm volatile("cp.async.wait_all;" ::: "memory");
     tc_fence_before();
@@ -1910,17 +1936,20 @@ __global__ void k_split_weights(const float *__restrict__ W, int64_t ldw, int32_
 // A bias [n] is packed alike, zero padded (four gates with gates = 3 too).
 // gate_h > 0: packed column 4 j + g is gate g of hidden unit j.  gates = 4: the sources have the columns i | f | g | o.  gates = 3 (GRU,
 // sources r | z | n): the candidate's two parts stay apart, column 4 j + 2 takes n of the first source only and 4 j + 3 n of the second.
-// A block takes eight columns, which share a scale (at most 2^60).  Its threads keep their pairs of terms in registers between the search for the
-// largest and the split, PACK_PAIRS of them (a latency of the memory each time otherwise: 256 x 256 12 us -> 4), and look again at what is beyond.
+// Every column has its own scale, so that none loses bits to (or is overrun by) a larger neighbour; it is at most 2^100, so that an accumulator times its
+// inverse stays normal.  share: the eight columns of a block have one where their largest elements lie within 2^PACK_SHARE of each other
+// (k_lstm_seq).  A block takes eight columns.  Its threads keep their pairs of terms in registers between the search for the largest and the
+// split, PACK_PAIRS of them (a latency of the memory each time otherwise: 256 x 256 12 us -> 4), and look again at what is beyond.
 #define PACK_COLS 8
+#define PACK_SHARE 2
 #define PACK_PAIRS 8
 __global__ void __launch_bounds__(256)
 k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, const float *__restrict__ W2, int64_t ldw2, int32_t k2, int32_t nkb,
-                int32_t n, int transpose, int32_t gate_h, int gates, __half *__restrict__ out, float *__restrict__ unscale, const float *__restrict__ bias,
+                int32_t n, int transpose, int32_t gate_h, int gates, int share, __half *__restrict__ out, float *__restrict__ unscale, const float *__restrict__ bias,
                 float *__restrict__ bias_out)
 {
     sat_grid_wait();
-    __shared__ uint32_t largest;
+    __shared__ uint32_t largest[PACK_COLS];
     const int32_t np0 = blockIdx.x * PACK_COLS, pairs = nkb * (TCH_BK / 2);
     auto value = [&](int32_t np, int32_t kk) {   // kk: term, the second source's from nkb1 k-blocks on
         const int32_t g = np & 3, nn = gate_h > 0 ? (gates == 3 && g == 3 ? 2 : g) * gate_h + (np >> 2) : np;   // packed row -> logical column
@@ -1941,13 +1970,13 @@ k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, 
         if (!transpose && p >= pairs) p -= pairs, ++c;
     };
     auto inside = [&]() { return c < PACK_COLS && p < pairs; };
-    if (threadIdx.x == 0) largest = 0;
     if (threadIdx.x < PACK_COLS) {
+        largest[threadIdx.x] = 0;
         const int32_t np = np0 + (int32_t)threadIdx.x;
         if (bias) bias_out[np] = np < n ? bias[gate_h > 0 ? (np & 3) * gate_h + (np >> 2) : np] : 0.f;
     }
     __syncthreads();
-    float x[PACK_PAIRS][2], m = 0.f;
+    float x[PACK_PAIRS][2];
 #pragma unroll
     for (int i = 0; i < PACK_PAIRS; ++i) {
         const bool in = inside();
@@ -1955,16 +1984,44 @@ k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, 
         x[i][1] = in ? value(np0 + c, 2 * p + 1) : 0.f;
         advance();
     }
+    const int lane = threadIdx.x & 31;
+    if (transpose) {   // a thread keeps to its column, and lanes eight apart share one
+        float m = 0.f;
 #pragma unroll
-    for (int i = 0; i < PACK_PAIRS; ++i) m = fmaxf(m, fmaxf(fabsf(x[i][0]), fabsf(x[i][1])));
-    for (; inside(); advance()) m = fmaxf(m, fmaxf(fabsf(value(np0 + c, 2 * p)), fabsf(value(np0 + c, 2 * p + 1))));
-    const uint32_t b = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-    if ((threadIdx.x & 31) == 0) atomicMax(&largest, b);
+        for (int i = 0; i < PACK_PAIRS; ++i) m = fmaxf(m, fmaxf(fabsf(x[i][0]), fabsf(x[i][1])));
+        for (; inside(); advance()) m = fmaxf(m, fmaxf(fabsf(value(np0 + c, 2 * p)), fabsf(value(np0 + c, 2 * p + 1))));
+        uint32_t b = __float_as_uint(m);
+        b = max(b, __shfl_xor_sync(0xffffffffu, b, 8));
+        b = max(b, __shfl_xor_sync(0xffffffffu, b, 16));
+        if (lane < PACK_COLS) atomicMax(&largest[lane], b);
+    } else {   // half a warp has pairs of one column: their number is a multiple of 16
+        for (; inside(); advance()) atomicMax(&largest[c], __float_as_uint(fmaxf(fabsf(value(np0 + c, 2 * p)), fabsf(value(np0 + c, 2 * p + 1)))));
+        c = c_first;
+        p = p_first;
+#pragma unroll
+        for (int i = 0; i < PACK_PAIRS; ++i) {
+            uint32_t b = __float_as_uint(fmaxf(fabsf(x[i][0]), fabsf(x[i][1])));
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+            if ((lane & 15) == 0 && inside()) atomicMax(&largest[c], b);
+            advance();
+        }
+    }
     __syncthreads();
-    const uint32_t e = min(f16_scale_exponent(largest >> 23), 187u);
-    const float s = __uint_as_float(e << 23);
+    uint32_t common = 0;
+    if (share) {
+        uint32_t least = 255, most = 0;
+#pragma unroll
+        for (int i = 0; i < PACK_COLS; ++i) {
+            const uint32_t l = largest[i] >> 23;
+            if (l > 0) least = min(least, l), most = max(most, l);
+        }
+        if (most < 255 && most <= least + PACK_SHARE) common = min(f16_scale_exponent(most), 227u);
+    }
+    auto exponent = [&](int32_t column) { return common ? common : min(f16_scale_exponent(largest[column] >> 23), 227u); };
     auto put = [&](float x0, float x1) {
         uint32_t h, l;
+        const float s = __uint_as_float(exponent(c) << 23);
         split_f16(x0 * s, x1 * s, h, l);
         uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(np0 + c) * (pairs / 8) + p / 8) * 32 + 2 * (p % 8));
         o[0] = h;
@@ -1978,7 +2035,7 @@ k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, 
         advance();
     }
     for (; inside(); advance()) put(value(np0 + c, 2 * p), value(np0 + c, 2 * p + 1));
-    if (threadIdx.x == 0) unscale[blockIdx.x] = __uint_as_float((254u - e) << 23);
+    if (threadIdx.x < PACK_COLS) unscale[np0 + threadIdx.x] = __uint_as_float((254u - exponent(threadIdx.x)) << 23);
 }
 
 // out[r] = bits of the largest magnitude in row r of A: a warp per row (for matrices whose writer did not leave it)
@@ -2106,8 +2163,8 @@ static size_t half_layout(int32_t nkb, int32_t n, void *base, TcWeights *out)
     const size_t planes = (size_t)out->n_pad * out->ld * sizeof(__half);   // a multiple of 4 KB
     out->planes = base;
     out->unscale = (float *)((char *)base + planes);
-    out->bias = out->unscale + out->n_pad / PACK_COLS;   // 16-byte aligned: n_pad is a multiple of 32
-    return planes + ((size_t)out->n_pad + out->n_pad / PACK_COLS) * sizeof(float);
+    out->bias = out->unscale + out->n_pad;   // 16-byte aligned: n_pad is a multiple of 32
+    return planes + 2 * (size_t)out->n_pad * sizeof(float);
 }
 
 sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1, const float *W2, int32_t ldw2, int32_t k2, int32_t n,
@@ -2119,7 +2176,7 @@ sat_status sat_tc_weights(sat_ctx *ctx, const float *W, int32_t ldw, int32_t k1,
         half_layout(nkb, n, buf.p, out);
         if (!bias) out->bias = nullptr;
         sat_pdl(ctx->stream, k_pack_half, (unsigned)(out->n_pad / PACK_COLS), 256, 0)(W, ldw, k1, nkb1, W2, ldw2, k2, nkb, n, transpose, gate_h, gates,
-                                                                                  (__half *)out->planes, out->unscale, bias, out->bias);
+                                                                                  out->share, (__half *)out->planes, out->unscale, bias, out->bias);
         SAT_LAUNCHED(ctx);
         return SAT_OK;
     }

@@ -538,9 +538,10 @@ sat_status sat_row_max(sat_ctx *ctx, const float *A, int32_t lda, int32_t d, int
 bool sat_tc_half(const sat_ctx *ctx, int32_t k);
 struct TcWeights {           // weight operand, K-major
     bool half;               // which of the two forms it has
+    bool share = false;      // (half-precision pairs) eight neighbouring columns may have one scale
     float *hi = nullptr, *lo = nullptr;   // two fp32 planes [n_pad x ld] holding the TF32 hi / lo terms
-    void *planes = nullptr;     // __half: pairs [n_pad][k-steps][16 hi | 16 lo], scaled per eight columns
-    float *unscale = nullptr;   // [n_pad / 8] inverse of the scale
+    void *planes = nullptr;     // __half: pairs [n_pad][k-steps][16 hi | 16 lo], scaled per column of the result
+    float *unscale = nullptr;   // [n_pad] inverse of the scale
     float *bias = nullptr;   // [n_pad], where one was packed with them
     int32_t ld = 0, n_pad = 0;
     explicit TcWeights(bool half_pairs = false) : half(half_pairs) {}

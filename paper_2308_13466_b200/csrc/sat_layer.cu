@@ -312,6 +312,7 @@ static sat_status run_lstm_cached(sat_ctx *ctx, CacheLayer *c, const sat_pred_pa
         c->proj_tag.assign(ctx->tau + 1, 0);
     }
     TcWeights Wp(sat_tc_half(ctx, d)), Wxu(sat_tc_half(ctx, d)), Up(true);   // Wx alone, [Wx ; Uh], Uh alone (all gate-interleaved)
+    Up.share = true;
     bool have_wp = false, have_wxu = false, have_up = false;
     if (c->pk_h != h) {      // another predictor width: nothing packed fits
         c->tag_wx = c->tag_uh = c->tag_wg = c->tag_b = c->tag_bg = 0;

@@ -931,3 +931,102 @@ def test_contraction_with_many_column_tiles(B, m, n, k):
     got = out[:, dev(cols.astype(np.int64))].cpu().numpy()
     a, w = A.astype(np.float64), W[:, cols].astype(np.float64)
     assert (np.abs(got - (a @ w + bias[cols])) <= ((k + 3) * U + 2.0 ** -20) * (np.abs(a) @ np.abs(w) + np.abs(bias[cols]))).all()
+
+
+def _sizes_bound(a, w):
+    """Of |result - a w| for operands split into halves, every row of a and every column of w with a scale of its own: |x s - hi - lo| <= 2^-22 |x s| + 2^-25 with
+    the largest |x s| of the row (column) at 2^14 or more."""
+    a, w = np.abs(a), np.abs(w)
+    return ((a.shape[1] + 3) * U + 2.0 ** -20) * (a @ w) + 2.0 ** -38 * (a.max(1, keepdims=True) * w.sum(0) + a.sum(1, keepdims=True) * w.max(0))
+
+
+# halves; TF32 terms; halves in a large graph; terms beyond those that the packing keeps in registers
+@pytest.mark.parametrize("m,n,k", [(200, 61, 384), (200, 61, 383), (33000, 40, 200), (130, 256, 1030)])
+def test_columns_of_very_different_sizes(B, m, n, k):
+    """A column of W next to ones that are 2^60 times larger is as precise as by itself, and one that is not finite stays by itself."""
+    rng = np.random.default_rng(k)
+    A = rng.standard_normal((m, k)).astype(np.float32)
+    W = (rng.standard_normal((k, n)) * np.exp2(rng.integers(-30, 31, (1, n)))).astype(np.float32)
+    bad = W.copy()
+    for j, x in ((2, np.inf), (11, -np.inf), (n - 1, np.nan)):
+        bad[rng.integers(0, k), j] = x
+    out, with_bad = _rows_times(B, A, W).cpu().numpy()[:, :n], _rows_times(B, A, bad).cpu().numpy()[:, :n]
+    sel = np.unique(np.concatenate([np.arange(130), rng.integers(0, m, 200)]))
+    a, w = A[sel].astype(np.float64), W.astype(np.float64)
+    assert (np.abs(out[sel] - a @ w) <= _sizes_bound(a, w)).all()
+    ok = np.setdiff1d(np.arange(n), [2, 11, n - 1])
+    assert np.array_equal(out[:, ok], with_bad[:, ok]) and not np.isfinite(with_bad[:, [2, 11, n - 1]]).any()
+
+
+@pytest.mark.parametrize("m,d_in,d_out", [(200, 400, 390), (300, 1030, 1030), (33000, 200, 200)])
+def test_input_gradient_with_features_of_very_different_sizes(B, m, d_in, d_out):
+    """The same for the rows of W, one of which makes a column of the input gradient.  In a graph without edges P is the identity."""
+    rng = np.random.default_rng(d_out)
+    X, D = rng.standard_normal((m, d_in)).astype(np.float32), rng.standard_normal((m, d_out)).astype(np.float32)
+    W = (rng.standard_normal((d_in, d_out)) * np.exp2(rng.integers(-30, 31, (d_in, 1)))).astype(np.float32)
+    out, g_in, gW, gb = empty2d(m, d_out), empty2d(m, d_in), torch.empty((d_in, d_out), device="cuda"), torch.empty(d_out, device="cuda")
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, np.zeros(m + 1, np.int64), np.zeros(0, np.int32))
+        B.sat_partition(ctx, 1, B.SAT_PART_CONTIG_BLOCKS)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, dev2d(X), None, dev(W), None, B.SAT_ACT_NONE | B.SAT_FWD_INPUT_GLOBAL, out)
+        B.sat_layer_bwd(ctx, B.SAT_ALL_PARTS, 2, dev2d(D), dev(W), gW, gb, 0, g_in, None)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    sel = np.unique(np.concatenate([np.arange(130), rng.integers(0, m, 200)]))
+    a, w = D[sel].astype(np.float64), W.T.astype(np.float64)
+    assert (np.abs(g_in.cpu().numpy()[sel][:, :d_in] - a @ w) <= _sizes_bound(a, w)).all()
+
+
+@pytest.mark.parametrize("h", [8, 64])
+def test_lstm_gates_of_very_different_sizes(B, h):
+    """Forget gates that saturate through a weight of 2^30 leave the other gates' columns of Uh as precise as they are by themselves (bound of
+    test_lstm_state_over_cached_projections; a saturated gate has no error)."""
+    n, d, tau = 600, 16, 3
+    ids = np.arange(n)
+    col = np.sort(np.stack([(ids - 1) % n, (ids + 1) % n], 1), 1).astype(np.int32).ravel()
+    rng = np.random.default_rng(h)
+    W, Uh, b = rng.standard_normal((d, 4, h)) / d ** 0.5, rng.standard_normal((h, 4, h)) / h ** 0.5, rng.standard_normal((4, h)) / 4
+    W[:, :, 0], Uh[:, :, 0], b[:, 0] = 0, 0, 2           # unit 0: a positive state
+    Uh[:, 1, :] = 0
+    Uh[0, 1, :] = 2.0 ** 30
+    W, Uh, b = (x.reshape(-1, 4 * h).astype(np.float32) for x in (W, Uh, b))
+    snaps = rng.standard_normal((tau, n, d)).astype(np.float32)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, 2 * np.arange(n + 1, dtype=np.int64), col)
+        B.sat_partition(ctx, 2, B.SAT_PART_GIVEN, (ids % 2).astype(np.int32))
+        B.sat_cache_init(ctx, [d], tau)
+        perm = np.concatenate([np.flatnonzero(ids % 2 == m) for m in range(2)])
+        out = empty2d(n, d)
+        p = B.make_pred_params(dev(W), dev(Uh), dev(b.ravel()), dev(np.zeros((h, d), np.float32)), dev(np.zeros(d, np.float32)), h, 1)
+        for x in snaps:
+            B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 1, dev2d(x[perm]))
+            B.sat_cache_commit(ctx)
+            B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, p, 0, out)
+        got = B.sat_predict_state(ctx, 1, n, h)[np.asarray(B.sat_slot_map(ctx, n)[1])]
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    s, c, ds, dc = (np.zeros((n, h)) for _ in range(4))
+    U64, eta = Uh.astype(np.float64), 2.0 ** -20
+    for x in snaps.astype(np.float64):
+        z = x @ W + s @ U64 + b
+        e = ((d + h + 2) * U + 2.0 ** -20) * (np.abs(x) @ np.abs(W) + np.abs(s) @ np.abs(U64) + np.abs(b)) + ds @ np.abs(U64)
+        (zi, zf, zg, zo), (ei, ef, eg, eo) = (np.split(v, 4, axis=1) for v in (z, e))
+        ef = np.where(zf > 2.0 ** 20, 0.0, ef)
+        sig = lambda v: 1 / (1 + np.exp(-np.minimum(v, 700)))
+        g = np.tanh(zg)
+        dc = np.abs(c) * (ef / 4 + eta) + dc + np.abs(g) * (ei / 4 + eta) + eg + eta
+        c = sig(zf) * c + sig(zi) * g
+        s = sig(zo) * np.tanh(c)
+        ds = eo / 4 + eta + dc + eta
+    assert (np.abs(got - s) <= ds).all()
+
+
+def test_scales_whose_product_is_no_float(B):
+    """Large elements that meet zeros on either side: the sum is zero although the product of the two scales overflows."""
+    A, W = np.zeros((130, 384), np.float32), np.zeros((384, 40), np.float32)
+    A[:, 0], W[1] = 2.0 ** 100, 2.0 ** 80
+    assert (_rows_times(B, A, W).cpu().numpy()[:, :40] == 0.0).all()
