@@ -17,11 +17,11 @@
  *   - All floating tensors are fp32, row-major.
  *   - Dense contractions run on the tensor cores with every fp32 operand split into two terms, fp32 accumulation.  Short ones keep
  *     2^-21 of each operand element.  Long ones (384 terms and more; 192 and more in graphs of at least 32,768 nodes; not the
- *     transform of layer 1) and the LSTM's steps over cached projections keep 2^-22 of each element down to 2^-18 of the largest
- *     one it shares a scale with, and 2^-39 of that largest one below.  A scale is shared by the elements of one row of the
- *     left operand ([x | state] of a recurrent step is one row) and by those of one column of the weights (input gradients: of
- *     one row), as they meet in one element of the result; by several of these only in the LSTM's steps, where the gate columns of two
- *     units share one if their largest elements are within a factor of eight.
+ *     transform of layer 1 nor, up to 383 terms, one to more than 128 columns) and the LSTM's steps over cached projections keep
+ *     2^-22 of each element down to 2^-18 of the largest one it shares a scale with, and 2^-39 of that largest one below.  A scale
+ *     is shared by the elements of one row of the left operand ([x | state] of a recurrent step is one row) and by those of one
+ *     column of the weights (input gradients: of one row), as they meet in one element of the result; by several of these only in
+ *     the LSTM's steps, where the gate columns of two units share one if their largest elements are within a factor of eight.
  *   - All work is enqueued on the stream given to sat_create (borrowed, not owned) and
  *     is asynchronous; argument and state errors are reported synchronously and leave
  *     the outputs untouched.

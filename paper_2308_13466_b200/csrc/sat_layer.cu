@@ -759,14 +759,16 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
         return sat_fail(ctx, SAT_EINVAL, "sat_layer_fwd: null / misaligned h_halo or bad ld_halo");
     // The first layer keeps TF32 terms.  Which side of a ReLU a pre-activation near zero takes depends on its rounding, and there, on raw features of a dense
     // graph, one decision moves an element of the weight gradient by several percent of the matrix's root mean square (58241 nodes, 16 M
-    // entries, 602 -> 256: up to 8 %, against 0.6 % for decisions of later layers), for 0.5 % of an epoch.  A push is bound by its
-    // epilogue up to 256 terms (113 us with TF32 terms, 120 with pairs; 179250 x 512, K = 512: 378 and 280).
-    const bool half_rows = layer > 1 && sat_tc_half(ctx, d_in), half = half_rows && (!push || d_in >= 384);
+    // entries, 602 -> 256: up to 8 %, against 0.6 % for decisions of later layers), for 0.5 % of an epoch.  Below 384 terms
+    // wide outputs keep them too: those are hidden layers, whose push is bound by its epilogue (169343 rows, K -> n with the push, us with TF32 terms and with
+    // pairs: 192 -> 256 111 and 118, 256 -> 256 121 and 121, 256 -> 128 78 and 79, 256 -> 40 65 and 57; without it 94 and 75, 68 and 56, 63 and 48;
+    // 179250 rows, 512 -> 512 with it 378 and 280).  The push itself does not decide, so that h_out is the same with it and without.
+    const bool half = layer > 1 && sat_tc_half(ctx, d_in) && (d_in >= 384 || d_out <= 128);
     LayerState &L = ctx->layers[layer];
     const int32_t ld_agg = round_up4(d_in), words = (d_out + 31) / 32;
     if (!L.agg || L.d_in != d_in || L.d_out != d_out) {
         SAT_TRY(dev_realloc(ctx, &L.agg, (int64_t)ctx->n * ld_agg));
-        SAT_TRY(dev_realloc(ctx, &L.agg_max, half_rows ? (int64_t)ctx->n * sat_spmm_parts(d_in) : 0));
+        SAT_TRY(dev_realloc(ctx, &L.agg_max, half ? (int64_t)ctx->n * sat_spmm_parts(d_in) : 0));
         SAT_TRY(dev_realloc(ctx, &L.mask, (int64_t)ctx->n * words));
         L.d_in = d_in;
         L.d_out = d_out;

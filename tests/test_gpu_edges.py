@@ -1030,3 +1030,30 @@ def test_scales_whose_product_is_no_float(B):
     A, W = np.zeros((130, 384), np.float32), np.zeros((384, 40), np.float32)
     A[:, 0], W[1] = 2.0 ** 100, 2.0 ** 80
     assert (_rows_times(B, A, W).cpu().numpy()[:, :40] == 0.0).all()
+
+
+# halves in a large graph (one column tile, two; a narrow layer) and in a small one, TF32 terms
+@pytest.mark.parametrize("n,k,m", [(33000, 200, 200), (33000, 256, 300), (33000, 383, 20), (600, 384, 64), (600, 200, 200)])
+def test_the_push_does_not_change_the_layer(B, n, k, m):
+    """sat_layer_fwd with SAT_FWD_PUSH = without, then sat_cache_update: output and ring, bit for bit, behind the first layer too."""
+    ids = np.arange(n)
+    col = np.sort(np.stack([(ids - 1) % n, (ids + 1) % n], 1), 1).astype(np.int32).ravel()
+    rng = np.random.default_rng(k)
+    X, W, b = dev2d(rng.standard_normal((n, k)).astype(np.float32)), dev(rng.standard_normal((k, m)).astype(np.float32)), dev(rng.standard_normal(m).astype(np.float32))
+    act, rows = B.SAT_ACT_RELU | B.SAT_FWD_INPUT_GLOBAL, []
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, 2 * np.arange(n + 1, dtype=np.int64), col)
+        B.sat_partition(ctx, 2, B.SAT_PART_GIVEN, (ids % 2).astype(np.int32))       # every node is a boundary node
+        B.sat_cache_init(ctx, [8, m], 1)
+        outs = [empty2d(n, m) for _ in range(2)]
+        for push, out in zip((0, B.SAT_FWD_PUSH), outs):
+            B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, X, None, W, b, act | push, out)
+            if not push:
+                B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 2, out)
+            rows.append(B.sat_cache_read(ctx, 2, -1, n, m))
+            B.sat_cache_update(ctx, B.SAT_ALL_PARTS, 2, dev2d(np.zeros((n, m), np.float32)))
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    assert torch.equal(outs[0], outs[1]) and np.array_equal(rows[0], rows[1]) and rows[0].any()
