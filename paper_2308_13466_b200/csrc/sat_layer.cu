@@ -763,7 +763,7 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
     // wide outputs keep them too: those are hidden layers, whose push is bound by its epilogue (169343 rows, K -> n with the push, us with TF32 terms and with
     // pairs: 192 -> 256 111 and 118, 256 -> 256 121 and 121, 256 -> 128 78 and 79, 256 -> 40 65 and 57; without it 94 and 75, 68 and 56, 63 and 48;
     // 179250 rows, 512 -> 512 with it 378 and 280).  The push itself does not decide, so that h_out is the same with it and without.
-    const bool half = layer > 1 && sat_tc_half(ctx, d_in) && (d_in >= 384 || d_out <= 128);
+    const bool half = layer > 1 && sat_tc_half(ctx, d_in) && sat_use_tc(d_out, d_in) && (d_in >= 384 || d_out <= 128);
     LayerState &L = ctx->layers[layer];
     const int32_t ld_agg = round_up4(d_in), words = (d_out + 31) / 32;
     if (!L.agg || L.d_in != d_in || L.d_out != d_out) {
