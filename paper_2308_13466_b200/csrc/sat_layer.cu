@@ -914,7 +914,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
     }
     if (!want_dx) return SAT_OK;
     const bool half_x = tc_x && sat_tc_half(ctx, d_out);
-    const bool stale_term = hist && GH.has_read && g_in && v.n_push > 0;
+    const bool stale_term = hist && GH.has_read && g_in, stale_rows = stale_term && v.n_push > 0;   // (the order below is the same for a partition without such rows)
     // G_in = P_in^T (D W^T) = (P_in^T D) W^T.  The second order gathers rows of d_out columns instead of d_in: taken where that is less and the
     // graph is not small (by nodes, so that one partition and all of them add up alike; 6,000 nodes, 72 -> 40 -> 7: 254.8 and 253.5
     // us, 8,292 nodes and 597 k entries, 64 -> 20: 260.8 and 266.1; 2,048 nodes, 16 -> 4: 84.7 and 85.2)
@@ -928,7 +928,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
         SAT_TRY(sat_ensure(ctx, ctx->buf_gagg, (size_t)v.n_rows * ld_q * sizeof(float)));
         float *q = (float *)ctx->buf_gagg.p;
         SpmmAdd add;
-        if (stale_term) {
+        if (stale_rows) {
             SAT_TRY(sat_row_slots(ctx, &add.slot));
             add.rows = GH.buf + (size_t)GH.read_idx * ctx->n_slots * GH.ld;
             add.ld = GH.ld;
@@ -970,7 +970,7 @@ extern "C" sat_status sat_layer_bwd(sat_ctx *ctx, int32_t part, int32_t layer, c
     // G_in = P_in^T G_AGG: the inner block of P is symmetric, so P_in^T = P_in (inner prefix of every local row)
     if (g_in) SAT_TRY(sat_spmm(ctx, v, 1, d_in, ga_base, ld_ga, nullptr, 0, g_in - (int64_t)v.row0 * ld_gin, ld_gin, mask_in, mask_in_words));
     // gradient-side history, the stale term: G_in[v] += (Q_read[slot(v)] W^T) o mask for the boundary rows v of the selection
-    if (stale_term) {
+    if (stale_rows) {
         const size_t plane = (size_t)ctx->n_slots * GH.ld;
         const float *qr = GH.buf + (size_t)GH.read_idx * plane;
         SAT_TRY(sat_ensure(ctx, ctx->buf_ghist_rows, (size_t)v.n_push * GH.ld * sizeof(float)));

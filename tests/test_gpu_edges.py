@@ -1057,3 +1057,57 @@ def test_the_push_does_not_change_the_layer(B, n, k, m):
     finally:
         B.sat_destroy(ctx)
     assert torch.equal(outs[0], outs[1]) and np.array_equal(rows[0], rows[1]) and rows[0].any()
+
+
+def _input_gradients(B, A, part, d_in, d_out, hist, seed):
+    """G_in of layer 2 under the mask of layer 1 with (hist) and without stale rows: all partitions at once, one after the other, the value in fp64 and
+    a bound of the error (that of test_input_gradient_in_both_orders, and what halves lose)."""
+    n, M = A.shape[0], int(part.max()) + 1
+    Pm = _propagation(A).tocoo()
+    rng = np.random.default_rng(seed)
+    perm = np.concatenate([np.flatnonzero(part == m) for m in range(M)])
+    off = np.concatenate([[0], np.cumsum(np.bincount(part, minlength=M))])
+    W1, W2 = (rng.standard_normal(s).astype(np.float32) for s in ((8, d_in), (d_in, d_out)))
+    X, D = rng.standard_normal((n, 8)).astype(np.float32), rng.standard_normal((n, d_out)).astype(np.float32)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        B.sat_cache_init(ctx, [d_in], 2)
+        _, slot, n_slots = B.sat_slot_map(ctx, n)
+        n_halo = B.sat_part_sizes(ctx, B.SAT_ALL_PARTS)[1]
+        H1, H2, g_in, one = empty2d(n, d_in), empty2d(n, d_out), empty2d(n, d_in), empty2d(n, d_in)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 1, dev2d(X), None, dev(W1), None, B.SAT_ACT_RELU | B.SAT_FWD_INPUT_GLOBAL, H1)
+        B.sat_layer_fwd(ctx, B.SAT_ALL_PARTS, 2, H1, dev2d(np.zeros((n_halo, d_in), np.float32)), dev(W2), None, B.SAT_ACT_NONE, H2)
+        Q = np.zeros((n_slots, d_out), np.float32)
+        if hist:
+            Q = (4 * rng.standard_normal((n_slots, d_out))).astype(np.float32)       # larger than the rows that they are added to
+            B.sat_grad_history_write(ctx, 2, d_out, Q)
+        flags = B.SAT_BWD_MASK_G_IN | (B.SAT_BWD_GRAD_HISTORY if hist else 0)
+        gW, gb, Dd = torch.empty((d_in, d_out), device="cuda"), torch.empty(d_out, device="cuda"), dev2d(D[perm])
+        B.sat_layer_bwd(ctx, B.SAT_ALL_PARTS, 2, Dd, dev(W2), gW, gb, flags, g_in, None)
+        for m in range(M):
+            r = slice(off[m], off[m + 1])
+            B.sat_layer_bwd(ctx, m, 2, Dd[r], dev(W2), gW, gb, flags, one[r], None)
+        B.sat_sync_status(ctx)
+        keep = H1.cpu().numpy()[:, :d_in] > 0
+    finally:
+        B.sat_destroy(ctx)
+    same = sp.csr_matrix((Pm.data * (part[Pm.row] == part[Pm.col]), (Pm.row, Pm.col)), shape=Pm.shape)
+    slot = np.asarray(slot)
+    stale = np.where((slot >= 0)[:, None], Q[np.maximum(slot, 0)], 0.0)
+    rows, mag, w = (same @ D.astype(np.float64) + stale)[perm], (abs(same) @ np.abs(D.astype(np.float64)) + np.abs(stale))[perm], np.abs(W2.T).astype(np.float64)
+    terms = np.diff(A.indptr).max() + d_out + 8
+    bound = (terms * U + 2.0 ** -20) * (mag @ w) + 2.0 ** -38 * (mag.max(1, keepdims=True) * w.sum(0) + mag.sum(1, keepdims=True) * w.max(0))
+    return g_in, one, (rows @ W2.T.astype(np.float64)) * keep, bound
+
+
+@pytest.mark.parametrize("d_in,d_out", [(40, 40), (72, 17), (400, 384)])
+def test_input_gradient_of_a_partition_without_cut_edges(B, d_in, d_out):
+    """A partition that has no boundary rows, and so no stale ones, adds up as in the call on all partitions, where others have them."""
+    n = 1500
+    A = sp.block_diag([_graph(HUBS[:8], n), _graph([30, 200], 600)]).tocsr()
+    part = np.concatenate([np.random.default_rng(3).integers(0, 2, n), np.full(600, 2)]).astype(np.int32)
+    g_in, one, want, bound = _input_gradients(B, A, part, d_in, d_out, True, d_out)
+    assert torch.equal(g_in, one)
+    assert (np.abs(g_in.cpu().numpy()[:, :d_in] - want) <= bound).all()
