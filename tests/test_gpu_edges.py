@@ -1111,3 +1111,27 @@ def test_input_gradient_of_a_partition_without_cut_edges(B, d_in, d_out):
     g_in, one, want, bound = _input_gradients(B, A, part, d_in, d_out, True, d_out)
     assert torch.equal(g_in, one)
     assert (np.abs(g_in.cpu().numpy()[:, :d_in] - want) <= bound).all()
+
+
+# halves behind the product, whose rows' sizes come from one launch or two, one slice of columns or several, stale rows among them
+@pytest.mark.parametrize("hist", [False, True])
+@pytest.mark.parametrize("kind", ["hub", "large"])
+@pytest.mark.parametrize("d_in,d_out", [(400, 384), (520, 512), (602, 401)])
+def test_wide_input_gradient(B, kind, d_in, d_out, hist):
+    A = _many_runs(kind)
+    part = np.random.default_rng(5).integers(0, 2, A.shape[0]).astype(np.int32)
+    g_in, one, want, bound = _input_gradients(B, A, part, d_in, d_out, hist, d_in)
+    assert torch.equal(g_in, one)
+    assert (np.abs(g_in.cpu().numpy()[:, :d_in] - want) <= bound).all()
+
+
+# graphs of at least 32,768 nodes take the product first at any width below d_in: on CUDA cores (with the mask) below 16 columns, TF32 terms, halves
+@pytest.mark.parametrize("d_in,d_out", [(200, 5), (33, 15), (200, 17), (200, 192), (192, 192)])
+def test_input_gradient_in_a_large_graph(B, d_in, d_out):
+    n = 33000
+    rng = np.random.default_rng(d_out)
+    A = _graph([9000, 300, 40], n)
+    part = rng.integers(0, 3, n).astype(np.int32)
+    g_in, one, want, bound = _input_gradients(B, A, part, d_in, d_out, False, d_out)
+    assert torch.equal(g_in, one)
+    assert (np.abs(g_in.cpu().numpy()[:, :d_in] - want) <= bound).all()
