@@ -812,9 +812,9 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
             if (!pc->proj_tag.empty()) pc->proj_tag[ctx->write_idx] = 0;
             // the rows' maxima stay in step with the rows: all of them from now on, or those of this partition where all of them were
             if (pc->row_max) eh.push_max = RowMaxOut{pc->row_max + (size_t)ctx->write_idx * sat_tc_parts(d_out) * ctx->n_slots, ctx->n_slots};
-            if (part == SAT_ALL_PARTS) pc->row_max_ok[ctx->write_idx] = 1;
         }
         SAT_TRY(sat_gemm_tc(ctx, v.n_rows, d_out, agg, ld_agg, d_in, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
+        if (eh.push_max.p && part == SAT_ALL_PARTS) pc->row_max_ok[ctx->write_idx] = 1;   // (not before: a call that fails writes neither)
     } else {
         GemmEpilogue ep;
         ep.bias = bias;
