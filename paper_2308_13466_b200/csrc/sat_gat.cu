@@ -598,9 +598,10 @@ extern "C" sat_status sat_gat_fwd(sat_ctx *ctx, int32_t part, int32_t layer, int
             ep.push = ring_buf(ctx, pc, ctx->write_idx);
             ep.ld_push = pc->ld;
             if (!pc->proj_tag.empty()) pc->proj_tag[ctx->write_idx] = 0;   // the buffer changes: its cached input projection is stale
-            pc->row_max_ok[ctx->write_idx] = 0;                            // and so are its rows' largest magnitudes
+            ep.row_max = sat_ring_max(ctx, pc, ctx->write_idx);
         }
         SAT_TRY(sat_spmm_entries(ctx, v, 0, d_out, (const int2 *)G.ent.p, z_in, ld_z, z_halo, ld_z, h_out - (int64_t)v.row0 * ld_out, ld_out, ep));
+        if (ep.row_max.p && part == SAT_ALL_PARTS) pc->row_max_ok[ctx->write_idx] = 1;
     }
     for (int m = (part == SAT_ALL_PARTS ? 0 : part); m < (part == SAT_ALL_PARTS ? ctx->M : part + 1); ++m) G.valid[m] = 1;
     return SAT_OK;

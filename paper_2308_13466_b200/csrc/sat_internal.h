@@ -77,8 +77,8 @@ struct LayerState {
 struct CacheLayer {
     float *buf = nullptr;  // [(tau+1) x n_slots x ld]
     int32_t width = 0, ld = 0;
-    // [(tau+1) x parts x n_slots] largest magnitude of the rows of every buffer, where sat_tc_half(width); where row_max_ok[buffer] is 0 it is looked for
-    // before its next use
+    // [(tau+1) x parts x n_slots] largest magnitude of the rows of every buffer, where sat_tc_half(width), as every push leaves it; where
+    // row_max_ok[buffer] is 0 (imported, requantised) it is looked for before its next use
     uint32_t *row_max = nullptr;
     std::vector<uint8_t> row_max_ok;
     float *S = nullptr;  // LSTM state table [n_slots x h]
@@ -374,7 +374,7 @@ struct SpmmEpilogue {
     int relu = 0;
     const float *s1 = nullptr, *v1 = nullptr, *s2 = nullptr, *v2 = nullptr;   // + s1[row] v1[col] + s2[row] v2[col]
     int32_t d = 0;
-    RowMaxOut row_max;
+    RowMaxOut row_max;                   // of the rows, indexed like the results (products with the propagation matrix) or by push_slot, in sat_tc_parts(d) parts
     SpmmAdd add;                         // (products with the propagation matrix only) rows added after the scaling
     float *push = nullptr;               // row i goes to row push_slot[i] of this matrix as well where that is >= 0
     const int32_t *push_slot = nullptr;  // [rows]
@@ -397,7 +397,7 @@ sat_status sat_gather(sat_ctx *ctx, const int32_t *idx, int64_t count, int32_t d
                       float *out, int32_t ld_out, DbgRange src_rows = SAT_ANY_ROW);
 sat_status sat_scatter(sat_ctx *ctx, const int32_t *src_row, const int32_t *dst_row, int64_t count, int32_t d,
                        const float *src_base, int32_t ld_src, float *dst, int32_t ld_dst, DbgRange src_rows = SAT_ANY_ROW,
-                       DbgRange dst_rows = SAT_ANY_ROW);
+                       DbgRange dst_rows = SAT_ANY_ROW, const RowMaxOut &row_max = RowMaxOut(), int32_t parts = 1);   // row_max: of the written rows, by dst_row
 // out[s] (+)= scale_s * sum over the halo positions p of cache slot s, in ascending partition order, of src[p]; scale_s = p_ss
 // (the self-loop weight of the node behind the slot) when self_scale, else 1.  One writer per slot: no atomics, fixed order.
 sat_status sat_sum_by_slot(sat_ctx *ctx, int32_t d, const float *src, int32_t ld_src, int self_scale, int add, float *out, int32_t ld_out);
@@ -530,6 +530,11 @@ __device__ __forceinline__ float tanh_fast(float x) { return fmaf(-2.f, rcp_fast
 
 // parts in which a contraction with n outputs leaves the largest magnitudes of its rows
 inline int32_t sat_tc_parts(int32_t n) { return 2 * ((n + 255) / 256); }
+// where the writers of ring buffer idx leave the largest magnitudes of its rows (nowhere unless sat_tc_half(width))
+inline RowMaxOut sat_ring_max(const sat_ctx *ctx, const CacheLayer *c, int32_t idx)
+{
+    return c->row_max ? RowMaxOut{c->row_max + (size_t)idx * sat_tc_parts(c->width) * ctx->n_slots, ctx->n_slots} : RowMaxOut();
+}
 // largest magnitudes of the rows of ring buffer idx of a cached layer (none unless sat_tc_half(width))
 sat_status sat_ring_rows(sat_ctx *ctx, int32_t layer, int32_t idx, RowMax *out);
 // out[r] = largest magnitude of row r, looked for (for matrices whose writer did not leave it)

@@ -121,10 +121,11 @@ extern "C" sat_status sat_cache_update(sat_ctx *ctx, int32_t part, int32_t layer
     if (v.n_push == 0) return SAT_OK;
     if (!h_out || !ok_ld(ld, c->width) || !aligned16(h_out)) return sat_fail(ctx, SAT_EINVAL, "sat_cache_update: null / misaligned h_out or bad ld");
     if (!c->proj_tag.empty()) c->proj_tag[ctx->write_idx] = 0;  // the buffer changes: its cached input projection is stale
-    c->row_max_ok[ctx->write_idx] = 0;
     const float *src_base = h_out - (int64_t)v.row0 * ld;
-    return sat_scatter(ctx, ctx->push_row + v.push0, ctx->push_slot + v.push0, v.n_push, c->width, src_base, ld,
-                       ring_buf(ctx, c, ctx->write_idx), c->ld, DbgRange{v.row0, (int64_t)v.row0 + v.n_rows}, DbgRange{0, ctx->n_slots});
+    SAT_TRY(sat_scatter(ctx, ctx->push_row + v.push0, ctx->push_slot + v.push0, v.n_push, c->width, src_base, ld, ring_buf(ctx, c, ctx->write_idx), c->ld,
+                        DbgRange{v.row0, (int64_t)v.row0 + v.n_rows}, DbgRange{0, ctx->n_slots}, sat_ring_max(ctx, c, ctx->write_idx), sat_tc_parts(c->width)));
+    if (part == SAT_ALL_PARTS) c->row_max_ok[ctx->write_idx] = 1;
+    return SAT_OK;
 }
 
 extern "C" sat_status sat_cache_commit(sat_ctx *ctx)
@@ -811,7 +812,7 @@ extern "C" sat_status sat_layer_fwd(sat_ctx *ctx, int32_t part, int32_t layer, i
             eh.ld_push = pc->ld;
             if (!pc->proj_tag.empty()) pc->proj_tag[ctx->write_idx] = 0;
             // the rows' maxima stay in step with the rows: all of them from now on, or those of this partition where all of them were
-            if (pc->row_max) eh.push_max = RowMaxOut{pc->row_max + (size_t)ctx->write_idx * sat_tc_parts(d_out) * ctx->n_slots, ctx->n_slots};
+            eh.push_max = sat_ring_max(ctx, pc, ctx->write_idx);
         }
         SAT_TRY(sat_gemm_tc(ctx, v.n_rows, d_out, agg, ld_agg, d_in, nullptr, 0, 0, Wp, eh, SATK_GEMM_NN));
         if (eh.push_max.p && part == SAT_ALL_PARTS) pc->row_max_ok[ctx->write_idx] = 1;   // (not before: a call that fails writes neither)

@@ -502,6 +502,21 @@ __device__ __forceinline__ float spmm_largest(float m, const float4 &r, int c, i
     return m;
 }
 
+// Leaves the largest magnitude of a slice of row `row`: by row, or (attention layer) by the row's ring slot, where it has one, in the first of the two parts that
+// stand for 256 columns there.
+template <bool EPI>
+__device__ __forceinline__ void spmm_put_max(const SpmmEpilogue &ep, int64_t row, unsigned slice, uint32_t m)
+{
+    if (EPI) {
+        const int32_t slot = __ldg(ep.push_slot + row);
+        if (slot < 0) return;
+        ep.row_max.p[2 * slice * ep.row_max.stride + slot] = m;
+        ep.row_max.p[(2 * slice + 1) * ep.row_max.stride + slot] = 0u;
+    } else {
+        ep.row_max.p[slice * ep.row_max.stride + row] = m;
+    }
+}
+
 // K entries: their columns and weights, their rows (all in flight together), the sums
 template <int G, int NV, int K, typename F>
 __device__ __forceinline__ void spmm_step(const int2 *__restrict__ ents, const F &row_of, int col, int32_t d4, float4 (&acc)[NV])
@@ -574,7 +589,7 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
         const bool last = !MAX || last_max > 0;
         const int32_t first = last ? __ldg(slot0 + it.x) : 0, cnt = last ? __ldg(tot + it.x) : 0;
         if (cnt > last_max || !last) {   // k_spmm_fixup, which raises the row's maximum from zero
-            if (MAX && lane == 0) ep.row_max.p[blockIdx.y * ep.row_max.stride + it.x] = 0u;
+            if (MAX && lane == 0) spmm_put_max<EPI>(ep, it.x, blockIdx.y, 0u);
             return;
         }
         const unsigned mask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
@@ -631,7 +646,7 @@ k_spmm(const int4 *__restrict__ items, int32_t n_items, int64_t slot_base, const
         unsigned lane_id;
         asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane_id));   // (not kept through the loops)
         const uint32_t m = __reduce_max_sync(G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (lane_id & ~(unsigned)(G - 1)), __float_as_uint(largest));
-        if ((lane_id & (G - 1)) == 0) ep.row_max.p[blockIdx.y * ep.row_max.stride + row] = m;
+        if ((lane_id & (G - 1)) == 0) spmm_put_max<EPI>(ep, row, blockIdx.y, m);
     }
 }
 
@@ -707,7 +722,10 @@ k_spmm_fixup(const int32_t *__restrict__ hrows, int32_t n_hrows, const int32_t *
     if (MAX) {   // the lanes of a warp that hold columns of the same row raise it together
         const unsigned same = __match_any_sync(__activemask(), (int32_t)row);
         const uint32_t m = __reduce_max_sync(same, __float_as_uint(spmm_largest(0.f, r, c, ep.d)));
-        if ((threadIdx.x & 31) == __ffs((int)same) - 1) atomicMax(ep.row_max.p + row, m);
+        if ((threadIdx.x & 31) == __ffs((int)same) - 1) {
+            const int64_t at = scale ? row : __ldg(ep.push_slot + row);
+            if (at >= 0) atomicMax(ep.row_max.p + at, m);
+        }
     }
 }
 
@@ -734,7 +752,7 @@ static void launch_spmm(sat_ctx *ctx, const SpmmList &l, const int4 *items, int3
         sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, false, MAX>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
                                                                      a.out_base, a.ld_out, partial, l.slot0, l.tot, (int32_t *)ctx->buf_ticket.p, l.last_max, a.omask, a.omask_words, a.ep, dbg);
     else
-        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, true, false>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
+        sat_pdl(ctx->stream, k_spmm<G, NV, U, MINB, true, MAX>, grid, 256, 0)(items, n_items, slot_base, a.ent, a.scale, a.n, d4, a.in_base, a.ld_in, a.halo_base, a.ld_halo,
                                                                     a.out_base, a.ld_out, partial, l.slot0, l.tot, (int32_t *)ctx->buf_ticket.p, l.last_max, a.omask, a.omask_words, a.ep, dbg);
 }
 
@@ -1011,14 +1029,37 @@ __global__ void k_scatter_rows(const int32_t *__restrict__ src_row, const int32_
     *reinterpret_cast<float4 *>(dst + SAT_IDX((int64_t)dst_row[i], dbg.out_lo, dbg.out_hi, dbg.status) * ld_dst + 4 * c) = x;
 }
 
+// the same, a warp per row, leaving the largest magnitude of every row by its destination (the first of `parts` parts; the others hold zeros)
+__global__ void __launch_bounds__(256)
+k_scatter_rows_max(const int32_t *__restrict__ src_row, const int32_t *__restrict__ dst_row, int64_t count, int32_t d, const float *__restrict__ src_base,
+                   int64_t ld_src, float *__restrict__ dst, int64_t ld_dst, RowMaxOut row_max, int32_t parts, DbgLimits dbg)
+{
+    sat_grid_wait();
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= count) return;
+    const float *src = src_base + SAT_IDX((int64_t)src_row[i], dbg.src_lo, dbg.src_hi, dbg.status) * ld_src;
+    const int64_t slot = SAT_IDX((int64_t)dst_row[i], dbg.out_lo, dbg.out_hi, dbg.status);
+    float largest = 0.f;
+#pragma unroll 4
+    for (int c = lane; 4 * c < d; c += 32) {
+        const float4 x = ld4(src + 4 * c);
+        reinterpret_cast<float4 *>(dst + slot * ld_dst)[c] = x;
+        largest = spmm_largest(largest, x, c, d);
+    }
+    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(largest));
+    for (int32_t p = lane; p < parts; p += 32) row_max.p[p * row_max.stride + slot] = p == 0 ? m : 0u;
+}
+
 sat_status sat_scatter(sat_ctx *ctx, const int32_t *src_row, const int32_t *dst_row, int64_t count, int32_t d, const float *src_base,
-                       int32_t ld_src, float *dst, int32_t ld_dst, DbgRange src_rows, DbgRange dst_rows)
+                       int32_t ld_src, float *dst, int32_t ld_dst, DbgRange src_rows, DbgRange dst_rows, const RowMaxOut &row_max, int32_t parts)
 {
     if (count == 0) return SAT_OK;
     const int32_t d4 = (d + 3) / 4;
+    const DbgLimits dbg = dbg_limits(src_rows, DbgRange{0, 0}, dst_rows, ctx->d_flag + 1);
     ProfScope prof(ctx, SATK_SCATTER, (8.0 * d + 8.0) * (double)count, 0.0);
-    sat_pdl(ctx->stream, k_scatter_rows, (unsigned)cdiv64(count * d4, 256), 256, 0)(src_row, dst_row, count, d4, src_base, ld_src, dst, ld_dst,
-                                                                               dbg_limits(src_rows, DbgRange{0, 0}, dst_rows, ctx->d_flag + 1));
+    if (row_max.p) sat_pdl(ctx->stream, k_scatter_rows_max, (unsigned)cdiv64(count * 32, 256), 256, 0)(src_row, dst_row, count, d, src_base, ld_src, dst, ld_dst, row_max, parts, dbg);
+    else sat_pdl(ctx->stream, k_scatter_rows, (unsigned)cdiv64(count * d4, 256), 256, 0)(src_row, dst_row, count, d4, src_base, ld_src, dst, ld_dst, dbg);
     SAT_LAUNCHED(ctx);
     return SAT_OK;
 }

@@ -1135,3 +1135,70 @@ def test_input_gradient_in_a_large_graph(B, d_in, d_out):
     g_in, one, want, bound = _input_gradients(B, A, part, d_in, d_out, False, d_out)
     assert torch.equal(g_in, one)
     assert (np.abs(g_in.cpu().numpy()[:, :d_in] - want) <= bound).all()
+
+
+@pytest.mark.parametrize("parts", [False, True])
+@pytest.mark.parametrize("route", ["layer", "update", "attention"])
+@pytest.mark.parametrize("kind,d", [("hub", 400), ("hub", 1000), ("large", 400), ("ring", 200)])     # rows of one launch and of two, one to four slices of columns
+def test_every_push_leaves_the_sizes_of_its_rows(B, kind, d, route, parts):
+    """A prediction from pushed rows does not look for their sizes again (as many launches as the next one) and is the one from the same rows when they have
+    been imported, whose sizes are looked for, bit for bit."""
+    if kind == "ring":
+        n = 33000
+        ids = np.arange(n)
+        col = np.sort(np.stack([(ids - 1) % n, (ids + 1) % n], 1), 1).astype(np.int32).ravel()
+        A = sp.csr_matrix((np.ones(2 * n), col, 2 * np.arange(n + 1)), shape=(n, n))
+    else:
+        A = _many_runs(kind)
+        n = A.shape[0]
+    rng, M, h, k = np.random.default_rng(d), 2, 32, 8
+    part = rng.integers(0, M, n).astype(np.int32)
+    rand = lambda *s: dev(rng.standard_normal(s).astype(np.float32) / 8)
+    ctx = B.sat_create(0, 0)
+    try:
+        B.sat_graph_load(ctx, A.indptr.astype(np.int64), A.indices.astype(np.int32))
+        B.sat_partition(ctx, M, B.SAT_PART_GIVEN, part)
+        B.sat_cache_init(ctx, [d], 1)
+        sizes, n_slots = [B.sat_part_sizes(ctx, m) for m in range(M)], B.sat_slot_map(ctx, n)[2]
+        n_halo = sum(s[1] for s in sizes)
+        spread = np.exp2(rng.integers(-9, 9, (n, 1)))
+        X, halo, Y = dev2d((rng.standard_normal((n, k)) * spread).astype(np.float32)), dev2d(rng.standard_normal((n_halo, k)).astype(np.float32)), empty2d(n, d)
+        W, a1, a2, b = rand(k, d), 1e-3 * rand(d), 1e-3 * rand(d), rand(d)
+        W1 = dev(rng.standard_normal((16, d)).astype(np.float32) * np.exp2(rng.integers(0, 9, (16, 1))).astype(np.float32))
+        X1 = dev2d((rng.standard_normal((n, 16)) * spread).astype(np.float32))
+        p = B.make_pred_params(rand(d, 4 * h) / 64, rand(h, 4 * h), rand(4 * h), rand(h, d), rand(d), h, 0, B.SAT_CELL_LSTM)
+        out, counts = [empty2d(n_halo, d) for _ in range(4)], []
+
+        def predict(i):
+            at = B.sat_launch_count(ctx)
+            B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, p, 0, out[i])
+            counts.append(B.sat_launch_count(ctx) - at)
+
+        B.sat_cache_commit(ctx)          # a snapshot of zeros, and the lists that a first prediction makes
+        B.sat_predict(ctx, 1, B.SAT_ALL_PARTS, p, 0, out[0])
+        push = B.SAT_ACT_RELU | B.SAT_FWD_PUSH
+        r0 = u0 = 0
+        for m in range(M) if parts else [B.SAT_ALL_PARTS]:
+            r1, u1 = (r0 + sizes[m][0], u0 + sizes[m][1]) if parts else (n, n_halo)
+            if route == "layer":
+                B.sat_layer_fwd(ctx, m, 1, X1, None, W1, b, push | B.SAT_FWD_INPUT_GLOBAL, Y[r0:r1])
+            elif route == "attention":
+                B.sat_gat_fwd(ctx, m, 1, X[r0:r1], halo[u0:u1], W, a1, a2, b, push, Y[r0:r1])
+            else:
+                Y[r0:r1] = dev((rng.standard_normal((r1 - r0, d)) * spread[:r1 - r0]).astype(np.float32))
+                B.sat_cache_update(ctx, m, 1, Y[r0:r1])
+            r0, u0 = r1, u1
+        B.sat_cache_commit(ctx)
+        predict(0)
+        predict(1)
+        state, ring = B.sat_cache_state(ctx), B.sat_cache_export(ctx, 1, 1, n_slots, d)
+        B.sat_cache_import(ctx, 1, ring)
+        B.sat_cache_set_state(ctx, *state)
+        predict(2)
+        predict(3)
+        S = B.sat_predict_state(ctx, 1, n_slots, h)
+        B.sat_sync_status(ctx)
+    finally:
+        B.sat_destroy(ctx)
+    assert counts[0] == counts[1] == counts[3] == counts[2] - 1
+    assert all(torch.equal(out[0], o) for o in out[1:]) and np.isfinite(S).all() and S.any()
