@@ -1404,7 +1404,6 @@ lstm_tiles(uint8_t *smem, uint8_t *Bs, uint8_t *Ps, SeqShared *sh, uint32_t tmem
         *reinterpret_cast<uint2 *>(d + ((piece ^ swz) << 4)) = hi;
         *reinterpret_cast<uint2 *>(d + (((piece + 2) ^ swz) << 4)) = lo;
     };
-    if (issuer && mine > slot && !mbar_wait_all(&sh->b_full, 0, dead, status)) return;
     // this thread's quads in the order in which they are taken: (tile, step, quad); the copies run SEQ_RING of them ahead
     const int32_t my_quads = (nq - half + 1) / 2;
     int32_t pf_k = slot, pf_t = 0, pf_i = 0;
