@@ -1,14 +1,17 @@
-// Dense contractions on the 5th-generation tensor cores (tcgen05.mma kind::tf32, accumulators in TMEM,
-// operands staged in shared memory by TMA) with fp32-level accuracy from a two-term TF32 split:
-//     x = hi + lo                                               (|x - hi - lo| <= 2^-21 |x|)
+// Dense contractions on the 5th-generation tensor cores (tcgen05.mma, accumulators in TMEM, operands staged in shared
+// memory by TMA) with fp32-level accuracy from a split of either operand into two terms:
+//     x = hi + lo                                               (kind::tf32: |x - hi - lo| <= 2^-21 |x|; kind::f16, scaled by powers of two: see split_f16)
 //     A B ~= Ah Bh + Ah Bl + Al Bh                              (three MMAs per k-step, fp32 accumulate)
-// Activations and weights stay plain fp32 in global memory: TMA brings the fp32 tiles into shared memory and the
-// converter warps write the residual tiles next to them, element-wise, so the swizzled layout never has to be decoded
-// (see "TF32 split of a shared-memory tile" below for the two variants).  Weights are repacked once per call into the
-// K-major operand layout.
+// Activations and weights stay plain fp32 in global memory: TMA brings the fp32 tiles into shared memory.  For TF32 terms
+// the converter warps write the residual tiles next to them, element-wise, so the swizzled layout never has to be decoded
+// (see "TF32 split of a shared-memory tile" below for the two variants); halves take the place of the raw values.  Weights
+// are repacked into the K-major operand layout: once per call, for the layers of an epoch over several partitions once per
+// epoch, for a predictor with a version once per version.
 //
 //   k_gemm_tc_k   C[M x N] = A[M x K] B[N x K]^T   both operands K-major, 64-byte swizzle, BLOCK_K = 16, persistent CTA pairs
 //                 (layer transform, recurrent gates with two A operands, input projections, predictor output, input gradient)
+//   k_gemm_tc_h   the same on half-precision pairs, 128-byte swizzle, BLOCK_K = 32, for long contractions (sat_tc_half)
+//   k_lstm_seq    LSTM steps over cached input projections, half-precision pairs
 //   k_gemm_tc_mn  C[M x N] = A[R x M]^T B[R x N]   both operands MN-major, 128-byte swizzle with 32-byte atoms, split over R
 //                 (weight gradient)
 // Warp roles of k_gemm_tc_k (512 threads): warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, then 6 converter and
@@ -227,8 +230,9 @@ __host__ __device__ inline uint32_t make_idesc_f16(int m, int n) { return 1u << 
 
 // Two-term split into half precision, x s = hi + lo + e with |e| <= 2^-22 |x s| wherever |x s| is not small: both terms are rounded to nearest,
 // and a power of two s brings the largest element of the operand's row to [2^14, 2^15), so that terms are subnormal (and e
-// is at most 2^-25) only for elements 2^18 times smaller than that one.  Closer than the TF32 split (2^-21 |x|, and hi truncated), on
-// operands of half the size and at twice the rate.  Two elements at a time: the first in the low half.
+// is at most 2^-25) only for elements 2^18 times smaller than that one.  Closer than the TF32 split (2^-21 |x|, and hi truncated) down to there, on
+// operands of half the size and at twice the rate; below 2^-19 of its row's largest element the TF32 split keeps more of an element, which shows
+// only in sums where that largest one meets a near-zero element of the other operand.  Two elements at a time: the first in the low half.
 __device__ __forceinline__ void split_f16(float x0, float x1, uint32_t &hi, uint32_t &lo)
 {
     const __half2 h = __floats2half2_rn(x0, x1);
@@ -899,8 +903,9 @@ template <> struct TchCfg<EPI_PROJ> : TchCfg<EPI_LSTM> {};
 // The scale is that of the whole row: the kernel is told the largest element of every row (RowMax) by whoever wrote the matrix, since looking for it
 // here meant fetching A twice.  The epilogue takes the scales back out (powers of two: exact).
 //
-// The TMA unit delivers 34 bytes per clock and SM, whatever it is asked for (four clocks per 128-byte row), which bound the form with TF32 terms
-// (48 KB of A, B and B's second plane per 32 terms); here it is 32 KB, and 16 where B stays in shared memory.
+// The form with TF32 terms takes in 48 KB of A, B and B's second plane per 32 terms; here it is 32 KB, and 16 where B stays in shared memory.  At
+// 164833 x 512, K = 512 (208 us) that is 29 bytes per clock and SM with the tensor pipe active for 75 % of the time; with B resident (256 -> 128,
+// 55 us) 13 bytes, tensor pipe 32 %, DRAM 4 TB/s: bound by the chain of a k-block (arrival, split, product) there.
 // 169343 rows, TF32 terms -> pairs, us: 256 -> 256 88 -> 70, 256 -> 40 57 -> 42, projections 256 -> 256 89 -> 72; 179250 rows: 512 -> 512
 // 320 -> 195, projections 512 -> 256 185 -> 119, 512 -> 512 with the push 378 -> 280.  Errors against 64 bits are half of the TF32 form's
 // (embeddings of the first layer of 169343 nodes 1.2e-6 -> 5.7e-7).  (Rows pushed by the two idle warps instead of the epilogue: 120 -> 193.)
