@@ -1954,6 +1954,7 @@ k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, 
 {
     sat_grid_wait();
     __shared__ uint32_t largest[PACK_COLS];
+    __shared__ float scale[PACK_COLS];
     const int32_t np0 = blockIdx.x * PACK_COLS, pairs = nkb * (TCH_BK / 2);
     auto value = [&](int32_t np, int32_t kk) {   // kk: term, the second source's from nkb1 k-blocks on
         const int32_t g = np & 3, nn = gate_h > 0 ? (gates == 3 && g == 3 ? 2 : g) * gate_h + (np >> 2) : np;   // packed row -> logical column
@@ -2012,21 +2013,25 @@ k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, 
         }
     }
     __syncthreads();
-    uint32_t common = 0;
-    if (share) {
-        uint32_t least = 255, most = 0;
+    if (threadIdx.x < PACK_COLS) {
+        uint32_t l = largest[threadIdx.x] >> 23;
+        if (share) {
+            uint32_t least = 255, most = 0;
 #pragma unroll
-        for (int i = 0; i < PACK_COLS; ++i) {
-            const uint32_t l = largest[i] >> 23;
-            if (l > 0) least = min(least, l), most = max(most, l);
+            for (int i = 0; i < PACK_COLS; ++i) {
+                const uint32_t li = largest[i] >> 23;
+                if (li > 0) least = min(least, li), most = max(most, li);
+            }
+            if (most < 255 && most <= least + PACK_SHARE) l = most;
         }
-        if (most < 255 && most <= least + PACK_SHARE) common = min(f16_scale_exponent(most), 227u);
+        const uint32_t e = min(f16_scale_exponent(l), 227u);
+        scale[threadIdx.x] = __uint_as_float(e << 23);
+        unscale[np0 + threadIdx.x] = __uint_as_float((254u - e) << 23);
     }
-    auto exponent = [&](int32_t column) { return common ? common : min(f16_scale_exponent(largest[column] >> 23), 227u); };
+    __syncthreads();
     auto put = [&](float x0, float x1) {
         uint32_t h, l;
-        const float s = __uint_as_float(exponent(c) << 23);
-        split_f16(x0 * s, x1 * s, h, l);
+        split_f16(x0 * scale[c], x1 * scale[c], h, l);
         uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(np0 + c) * (pairs / 8) + p / 8) * 32 + 2 * (p % 8));
         o[0] = h;
         o[8] = l;
@@ -2039,7 +2044,6 @@ k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, 
         advance();
     }
     for (; inside(); advance()) put(value(np0 + c, 2 * p), value(np0 + c, 2 * p + 1));
-    if (threadIdx.x < PACK_COLS) unscale[np0 + threadIdx.x] = __uint_as_float((254u - exponent(threadIdx.x)) << 23);
 }
 
 // out[r] = bits of the largest magnitude in row r of A: a warp per row (for matrices whose writer did not leave it)
