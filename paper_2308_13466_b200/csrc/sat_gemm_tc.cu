@@ -241,6 +241,9 @@ __device__ __forceinline__ void split_f16(float x0, float x1, uint32_t &hi, uint
     hi = *reinterpret_cast<const uint32_t *>(&h);
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
+// An accumulator is multiplied by the inverse scales of its column and of its row, one after the other: their product may lie outside of fp32.  2^SCALE_SHIFT goes
+// over from the column's to the row's, so that the first product stays inside for columns up to 2^118.
+#define SCALE_SHIFT 14
 // biased exponent of the power of two that brings the elements of a row, the largest of which has this biased exponent, below 2^15; the
 // inverse has 254 minus it.  One for zeros, infinities and NaN.
 __device__ __forceinline__ uint32_t f16_scale_exponent(uint32_t largest)
@@ -346,7 +349,7 @@ struct TcEpilogue {
     int32_t row_parts;
     uint32_t row_least;      // what the largest magnitude is taken to be at least (bits)
     int32_t k1, k2;          // terms of the A operands
-    const float *unscale;    // inverse scale of every column of B
+    const float *unscale;    // inverse scale of every column of B, see TcWeights
     float *C;
     int64_t ldc;
     const float *bias;
@@ -1114,13 +1117,13 @@ k_gemm_tc_h(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 }
             };
             if (c_first < bn) load_cell(c_first);
-            const float unscale = __uint_as_float((254u - row_scale(row)) << 23);
+            const float unscale = __uint_as_float((254u + SCALE_SHIFT - row_scale(row)) << 23);
             if (!mbar_wait_warp(&sh->acc_full[buf], (lt >> 1) & 1u, dead, status, lane)) goto done;
             tc_fence_after();
             for (int c0 = c_first; c0 < bn; c0 += CHUNK_STEP) {
                 uint32_t r[32];
                 tc_ld32(tmem + buf * acc_cols + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-                // takes the scales out and adds the bias to four columns: the column's scale first, since the product of the two may lie outside of fp32
+                // takes the scales out and adds the bias to four columns
                 auto finish = [&](uint32_t *x, int u) {
                     const float4 us = __ldg(reinterpret_cast<const float4 *>(ep.unscale + n0 + c0) + u);
                     const float4 b4 = ep.bias ? __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + c0) + u) : zero4;
@@ -1560,7 +1563,7 @@ k_lstm_seq(const __grid_constant__ CUtensorMap mapB, const float *__restrict__ u
     volatile int *dead = &sh->dead;
     sat_grid_wait();
     if ((int)threadIdx.x < bn) {
-        const float us = __ldg(unscale + threadIdx.x) * 0x1p-14f;
+        const float us = __ldg(unscale + threadIdx.x);   // (with the inverse of the state's scale, 2^-SCALE_SHIFT, in it)
         reinterpret_cast<float *>(sh->unscale)[threadIdx.x] = us;
         if (us != __shfl_sync(0xffffffffu, us, lane & 24)) sh->own_scales = 1;   // (whole warps: bn is a multiple of 32)
         if ((lane & 7) == 0) reinterpret_cast<float *>(sh->pair_unscale)[threadIdx.x >> 3] = us;
@@ -1941,7 +1944,7 @@ __global__ void k_split_weights(const float *__restrict__ W, int64_t ldw, int32_
 // gate_h > 0: packed column 4 j + g is gate g of hidden unit j.  gates = 4: the sources have the columns i | f | g | o.  gates = 3 (GRU,
 // sources r | z | n): the candidate's two parts stay apart, column 4 j + 2 takes n of the first source only and 4 j + 3 n of the second.
 // Every column has its own scale, so that none loses bits to (or is overrun by) a larger neighbour; it is at most 2^100, so that an accumulator times its
-// inverse stays normal.  share: the eight columns of a block have one where their largest elements lie within 2^PACK_SHARE of each other
+// inverse (and 2^-SCALE_SHIFT) stays normal.  share: the eight columns of a block have one where their largest elements lie within 2^PACK_SHARE of each other
 // (k_lstm_seq).  A block takes eight columns.  Its threads keep their pairs of terms in registers between the search for the largest and the
 // split, PACK_PAIRS of them (a latency of the memory each time otherwise: 256 x 256 12 us -> 4), and look again at what is beyond.
 #define PACK_COLS 8
@@ -2026,7 +2029,7 @@ k_pack_half(const float *__restrict__ W, int64_t ldw, int32_t k1, int32_t nkb1, 
         }
         const uint32_t e = min(f16_scale_exponent(l), 227u);
         scale[threadIdx.x] = __uint_as_float(e << 23);
-        unscale[np0 + threadIdx.x] = __uint_as_float((254u - e) << 23);
+        unscale[np0 + threadIdx.x] = __uint_as_float((254u - SCALE_SHIFT - e) << 23);
     }
     __syncthreads();
     auto put = [&](float x0, float x1) {

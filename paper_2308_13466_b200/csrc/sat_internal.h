@@ -546,7 +546,7 @@ struct TcWeights {           // weight operand, K-major
     bool share = false;      // (half-precision pairs) eight neighbouring columns may have one scale
     float *hi = nullptr, *lo = nullptr;   // two fp32 planes [n_pad x ld] holding the TF32 hi / lo terms
     void *planes = nullptr;     // __half: pairs [n_pad][k-steps][16 hi | 16 lo], scaled per column of the result
-    float *unscale = nullptr;   // [n_pad] inverse of the scale
+    float *unscale = nullptr;   // [n_pad] inverse of the scale times 2^-14 (the row's has 2^14 in it)
     float *bias = nullptr;   // [n_pad], where one was packed with them
     int32_t ld = 0, n_pad = 0;
     explicit TcWeights(bool half_pairs = false) : half(half_pairs) {}

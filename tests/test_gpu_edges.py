@@ -1202,3 +1202,14 @@ def test_every_push_leaves_the_sizes_of_its_rows(B, kind, d, route, parts):
         B.sat_destroy(ctx)
     assert counts[0] == counts[1] == counts[3] == counts[2] - 1
     assert all(torch.equal(out[0], o) for o in out[1:]) and np.isfinite(S).all() and S.any()
+
+
+@pytest.mark.parametrize("row,column", [(-60, 115), (60, -100), (60, 60), (-60, -58), (100, 0), (-110, 100), (110, -95)])
+def test_rows_and_columns_far_from_one(B, row, column):
+    """Rows of A near 2^row, columns of W near 2^column: the result is a float, and so is what the scales of either leave on the way."""
+    rng = np.random.default_rng(7)
+    A, W = (rng.uniform(0.25, 1, s) * rng.choice([-1, 1], s) for s in ((130, 384), (384, 40)))
+    A, W = (A * 2.0 ** row).astype(np.float32), (W * 2.0 ** column).astype(np.float32)
+    out = _rows_times(B, A, W).cpu().numpy()[:, :40]
+    a, w = A.astype(np.float64), W.astype(np.float64)
+    assert (np.abs(out - a @ w) <= _sizes_bound(a, w)).all()
