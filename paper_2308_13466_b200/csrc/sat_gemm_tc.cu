@@ -1338,7 +1338,7 @@ done:
 // by a warp of their own per slot, which leaves 96 registers: 192 us.)  The errors are what they were (relative 1.6e-6 of the
 // state at K = 256).  The inverse scales of a quad's sixteen columns come out of shared memory too, next to projections and state: 164833 rows 161 -> 180 us with
 // one for every column, so eight neighbours (a pair of units) share theirs where they are of a size (k_pack_half), and only a matrix where they are not
-// takes that form.
+// takes that form, which costs the other 6 us by its call.
 // =====================================================================================
 #define SEQ_THREADS 512   /* 128 registers a thread */
 #define SEQ_RING 3        /* quads of projections in flight per thread */
